@@ -122,21 +122,23 @@ void layout_compress(asi_plan* pl) {
       pl->fiber_grid[m] = fiber2_grid(pl->mv[m].O, pl->mv[m].a, pl->mv[m].I, pl->r[m], pl->bf16,
                                       (pl->d.flags & ASI_FLAG_SHARE_SM) != 0);
     }
-  int64_t vmax = 0;
-  if (!pl->fast_compress)
-    for (int m = 0; m < pl->nd; ++m) vmax = std::max<int64_t>(vmax, pl->mv[m].Q * pl->r[m]);
-  pl->fork = pl->d.kind == ASI_LINEAR && pl->nd == 3 && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY);
-  pl->off_V = off;
-  pl->v_stride = pl->fork ? align_up((size_t)vmax * 4, 256) : 0;
-  off = align_up(off + (size_t)vmax * 4, 256) + (pl->fork ? (size_t)(pl->nd - 1) * pl->v_stride : 0);
+  // V_m of the modes without a one-pass kernel, one region each (their products share launches); at least the
+  // largest V of the layer
+  if (!pl->fast_compress) {
+    size_t used = 0, vmax = 0;
+    for (int m = 0; m < pl->nd; ++m) {
+      const size_t bytes = align_up((size_t)pl->mv[m].Q * pl->r[m] * 4, 256);
+      pl->v_off[m] = off + used;
+      vmax = std::max(vmax, bytes);
+      if (!pl->fiber[m] && !(pl->plane && m >= 2)) used += bytes;
+    }
+    off += std::max(used, vmax);
+  }
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
-    const int64_t kchunks = (v.a + kExpandKC - 1) / kExpandKC;
-    // about two waves of CTAs, at least four 64-column tiles per split
-    int64_t ns = std::max<int64_t>(1, 296 / kchunks);
-    ns = std::min<int64_t>(ns, std::max<int64_t>(1, v.Q / 256));
+    int64_t ns = gemm_expand_splits(v.a, v.Q);
     int64_t qps = (v.Q + ns - 1) / ns;
-    qps = (qps + 63) / 64 * 64;
+    qps = (qps + 127) / 128 * 128;
     ns = (v.Q + qps - 1) / qps;
     if (pl->fast_compress) {                                             // one partial per tile; the cold-start
       ns = (m == 1) ? sm_pass1_role_c_ctas(pl->fast_S, (int)pl->dims[0]) : pl->n_tiles_b;   // expansion splits the
@@ -148,8 +150,8 @@ void layout_compress(asi_plan* pl) {
     }                                                                    // write 0)
     pl->nsplit[m] = (int)ns;
     pl->q_per_split[m] = qps;
-    const int qr_rows = (pl->fast_compress || pl->small_rank) ? kRedRows : kQRRows;
-    pl->nchunk[m] = (int)((v.a + qr_rows - 1) / qr_rows);
+    pl->qr_rows[m] = (pl->fast_compress || pl->small_rank) ? kRedRows : orth_rows(v.a, v.r, ns);
+    pl->nchunk[m] = (int)((v.a + pl->qr_rows[m] - 1) / pl->qr_rows[m]);
     pl->off_Pp[m] = off;
     size_t pp_elems = (size_t)ns * v.a * v.r;
     if (pl->fast_compress && (pl->fast_S == 7 || pl->fast_S == 14) && m >= 2) pp_elems = std::max(pp_elems, (size_t)ns * v.a * v.a);
@@ -157,7 +159,7 @@ void layout_compress(asi_plan* pl) {
     pl->off_Pred[m] = off;
     off = align_up(off + (size_t)v.a * std::max<int64_t>(v.r, (pl->fast_compress && m >= 2) ? v.a : 0) * 8, 256);
     pl->off_Gp[m] = off;
-    off = align_up(off + (size_t)pl->nchunk[m] * v.r * v.r * 8, 256);
+    off = align_up(off + orth_gp_elems(pl->nchunk[m], v.r) * 8, 256);
   }
   // bf16 operand of the tensor-core kernels: products of bf16 tensors with a wide factor (16..64 columns, a
   // multiple of 16) over the last mode (a_m a multiple of 64, >= 128 fibers) or over a mode whose inner
@@ -175,6 +177,7 @@ void layout_compress(asi_plan* pl) {
       pl->tc_mode[m] = last ? 1 : 2;
       pl->tc_bytes = std::max(pl->tc_bytes, tc_scratch_bytes(std::max(v.a, v.Q), pl->r[m]));
     }
+  pl->fork = pl->d.kind == ASI_LINEAR && pl->nd == 3 && pl->tc_bytes > 0 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY);
   pl->tc_stride = pl->fork ? align_up(pl->tc_bytes, 256) : 0;
   off = align_up(off + pl->tc_bytes, 256) + (pl->fork ? (size_t)(pl->nd - 1) * pl->tc_stride : 0);
   pl->off_Rf = off;                                   // Cholesky factors of the fused path
@@ -191,6 +194,8 @@ void layout_compress(asi_plan* pl) {
   int best = 0;
   for (int m = 1; m < pl->nd; ++m)
     if ((double)pl->dims[m] / pl->r[m] > (double)pl->dims[best] / pl->r[best]) best = m;
+  // linear layers: the feature mode first where that shrinks the tensor by four at least (k_core_tok does the rest)
+  if (pl->d.kind == ASI_LINEAR && (pl->nd == 2 || pl->dims[pl->nd - 1] >= 4 * pl->r[pl->nd - 1])) best = pl->nd - 1;
   std::swap(order[0], order[best]);
   std::sort(order + 1, order + pl->nd);
   std::memcpy(pl->core_order, order, sizeof(order));
@@ -213,7 +218,7 @@ void layout_compress(asi_plan* pl) {
     pl->off_T[t] = off;
     off = align_up(off + (size_t)tmax[t] * 4, 256);
   }
-  pl->core_tail = false;
+  pl->core_tail = pl->core_tok = false;
   pl->off_ctp = off;
   if (pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
       order[0] == 0 && order[1] == 1 && order[2] == 2 && order[3] == 3 &&
@@ -225,18 +230,24 @@ void layout_compress(asi_plan* pl) {
   pl->compress_ws = off;
   pl->launches_compress = 3;
   if (!pl->fast_compress) {
-    pl->launches_compress = 2 + (pl->core_tail ? 2 : pl->nd) + (pl->small_rank ? 0 : 1);   // reduction/QR kernels, core chain
-    for (int m = 0; m < pl->nd; ++m)
-      pl->launches_compress += (pl->plane && m >= 2) ? (m == 2 ? 1 : 0) : pl->fiber[m] ? 1 : 2;
-    // a tensor-core product is two launches (operand split + GEMM): V_m, the expansion when it fits too,
-    // and the first core product when it contracts such a mode of the bf16 activation
+    pl->core_tok = pl->d.kind == ASI_LINEAR && (pl->nd == 2 || order[0] == 2);
+    // the two kernels of Orthogonalize, the core chain, one launch per one-pass mode (one for both spatial modes),
+    // one projection and one expansion launch for all SIMT modes together
+    pl->launches_compress = 2 + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
+    bool simt = false;
     for (int m = 0; m < pl->nd; ++m) {
-      if (!pl->tc_mode[m]) continue;
-      const ModeView& v = pl->mv[m];
-      pl->launches_compress += 1;
-      if (pl->tc_mode[m] == 2 || (v.a % 8 == 0 && v.a >= 128 && v.Q % 8 == 0)) pl->launches_compress += 1;
-      if (pl->core_order[0] == m) pl->launches_compress += 1;
+      if (pl->plane && m >= 2) pl->launches_compress += (m == 2);
+      else if (pl->fiber[m]) pl->launches_compress += 1;
+      else if (pl->tc_mode[m]) {
+        // a tensor-core product is two launches (operand split + GEMM): V_m, the expansion when it fits too
+        const ModeView& v = pl->mv[m];
+        pl->launches_compress += 3;
+        if (pl->tc_mode[m] == 2 || (v.a % 8 == 0 && v.a >= 128 && v.Q % 8 == 0)) pl->launches_compress += 1;
+      } else simt = true;
+      // .. and the first core product when it contracts such a mode of the bf16 activation
+      if (pl->tc_mode[m] && pl->core_order[0] == m) pl->launches_compress += 1;
     }
+    if (simt) pl->launches_compress += 2;
   }
 }
 
@@ -245,28 +256,15 @@ void layout_wgrad(asi_plan* pl) {
   int64_t z[3] = {0, 0, 0};
   if (pl->d.kind == ASI_CONV2D) {
     z[0] = (int64_t)pl->r[0] * pl->d.cout * pl->Ho * pl->Wo;          // Z1
-    z[1] = (int64_t)pl->r[0] * pl->r[1] * pl->dims[2] * pl->r[3];     // core x_3 U_3
-    z[2] = (int64_t)pl->r[0] * pl->r[1] * pl->dims[2] * pl->dims[3];  // Z3
-    pl->launches_wgrad = pl->fast_wgrad ? 1 : 4;
+    z[1] = (int64_t)pl->r[0] * pl->r[1] * pl->dims[2] * pl->dims[3];  // Z3
+    pl->launches_wgrad = pl->fast_wgrad ? 1 : 3;
   } else {
-    const int nlead = pl->nd - 1;
-    int64_t rest = pl->d.cout;
-    for (int m = 1; m < nlead; ++m) rest *= pl->dims[m];
-    z[0] = (int64_t)pl->r[0] * rest;                                   // dY x_1 U_1^T
-    z[1] = (nlead > 1) ? (int64_t)pl->r[0] * pl->r[1] * pl->d.cout : 0;  // .. x_2 U_2^T
-    pl->lin_nsplit = lin_tail_nsplit(pl->r[0] * (nlead > 1 ? pl->r[1] : 1), pl->d.cout);
-    z[2] = (int64_t)pl->lin_nsplit * pl->r[pl->nd - 1] * pl->d.cout;   // Z4 (its shares)
-    pl->launches_wgrad = nlead + 2;
-    // bf16 token layers whose token-mode factor fits the tensor-core kernel: contract the token mode of dY
-    // first (dY is then read once, by tcgen05, and no [r1 x N x Dout] intermediate exists)
-    pl->lin_reorder = pl->nd == 3 && pl->bf16 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && pl->r[0] <= 8 &&
-                      pl->r[1] % 4 == 0 && pl->r[1] >= 16 && pl->r[1] <= 64 && pl->d.cout % 64 == 0 &&
-                      pl->dims[0] < 65536;
-    if (pl->lin_reorder) {
-      z[0] = pl->dims[0] * pl->d.cout * pl->r[1];                      // dY x_2 U_2^T  [B][Dout][r2]
-      z[1] = (int64_t)pl->r[0] * pl->d.cout * pl->r[1];                // .. x_1 U_1^T  [r1][Dout][r2]
-      pl->launches_wgrad = 5;
-    }
+    // dY x_2 U_2^T [B][Dout][r2] (two modes: dY x_1 U_1^T [Dout][r1]), then Z4 [Dout][r_last]
+    z[0] = pl->nd == 3 ? pl->dims[0] * pl->d.cout * pl->r[1] : (int64_t)pl->d.cout * pl->r[0];
+    z[1] = (int64_t)pl->r[pl->nd - 1] * pl->d.cout;
+    pl->lin_tc = pl->nd == 3 && pl->bf16 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && pl->r[1] % 4 == 0 &&
+                 pl->r[1] >= 16 && pl->r[1] <= 64 && pl->d.cout % 64 == 0 && pl->dims[0] < 65536;
+    pl->launches_wgrad = pl->lin_tc ? 4 : 3;
   }
   for (int t = 0; t < 3; ++t) {
     pl->off_Z[t] = off;
@@ -274,21 +272,18 @@ void layout_wgrad(asi_plan* pl) {
   }
   pl->off_wtc = off;
   pl->wtc_bytes = 0;
-  if (pl->d.kind == ASI_LINEAR && pl->lin_reorder) {
+  if (pl->d.kind == ASI_LINEAR && pl->lin_tc) {
     pl->wtc_bytes = tc_scratch_bytes(pl->dims[1], pl->r[1]);
     off = align_up(off + pl->wtc_bytes, 256);
   }
   pl->conv_nsp = 1;
   pl->off_Z4p = off;
-  pl->conv_z3 = pl->d.kind == ASI_CONV2D && !pl->fast_wgrad && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
-                pl->r[2] <= 8 && pl->r[3] <= 8;
-  if (pl->conv_z3) pl->launches_wgrad = 3;
   if (pl->d.kind == ASI_CONV2D && !pl->fast_wgrad && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
       (int64_t)pl->r[0] * pl->Ho * pl->Wo >= 1024 && pl->d.cout < 296) {
     pl->conv_nsp = (int)std::min<int64_t>(16, std::max<int64_t>(2, 592 / pl->d.cout));
     pl->conv_nsp = (int)std::min<int64_t>(pl->conv_nsp, (int64_t)pl->r[0] * pl->Ho);
     off = align_up(off + (size_t)pl->conv_nsp * pl->d.cout * pl->r[1] * pl->d.kh * pl->d.kw * 4, 256);
-    pl->launches_wgrad = pl->conv_z3 ? 4 : 5;
+    pl->launches_wgrad = 4;
   }
   pl->wgrad_ws = off;
 }
@@ -405,7 +400,6 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
 asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const float* gram_U_prev,
                                cudaStream_t st) {
   int max_chunks = 1;
-  for (int m = 0; m < pl->nd; ++m) max_chunks = std::max(max_chunks, pl->nchunk[m]);
   if (pl->fast_compress) {
     SmReduceArgs ra;
     max_chunks = build_fused_reduce(pl, w, gram_U_prev, &ra);
@@ -414,17 +408,21 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
   }
   if (pl->small_rank) {
     SmReduceArgs ra;
-    std::memset(&ra, 0, sizeof(ra));
-    for (int m = 0; m < pl->nd; ++m) {
-      ra.m[m].Pp = reinterpret_cast<const float*>(w + pl->off_Pp[m]);
-      ra.m[m].Pred = reinterpret_cast<double*>(w + pl->off_Pred[m]);
-      ra.m[m].Gp = reinterpret_cast<double*>(w + pl->off_Gp[m]);
-      ra.m[m].a = (int)pl->dims[m];
-      ra.m[m].r = pl->r[m];
-      ra.m[m].nsplit = pl->nsplit[m];
-      ra.m[m].nchunk = pl->nchunk[m];
-    }
+    max_chunks = build_fused_reduce(pl, w, nullptr, &ra);
     ASI_CUDA(launch_sm_reduce(ra, pl->nd, max_chunks, st));
+    RowSolveArgs rs;
+    std::memset(&rs, 0, sizeof(rs));
+    rs.Rf = ra.Rf;
+    rs.nd = pl->nd;
+    for (int m = 0; m < pl->nd; ++m) {
+      rs.Pred[m] = ra.m[m].Pred;
+      rs.U[m] = U_new + pl->u_off[m];
+      rs.a[m] = (int)pl->dims[m];
+      rs.r[m] = pl->r[m];
+      rs.total += rs.a[m];
+    }
+    ASI_CUDA(launch_row_solve(rs, st));
+    return ASI_OK;
   }
   QRArgs qa;
   std::memset(&qa, 0, sizeof(qa));
@@ -437,38 +435,48 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
     qa.m[m].r = pl->r[m];
     qa.m[m].nsplit = pl->nsplit[m];
     qa.m[m].nchunk = pl->nchunk[m];
+    qa.m[m].rows = pl->qr_rows[m];
+    qa.m[m].gs = orth_group(pl->nchunk[m]);
+    qa.m[m].count = reinterpret_cast<int*>(w) + 20 + m;
+    qa.m[m].gcount = reinterpret_cast<int*>(w) + 64 + kOrthGroups * m;
   }
   qa.status = reinterpret_cast<int*>(w);
-  if (pl->small_rank) ASI_CUDA(launch_qr_solve(qa, pl->nd, max_chunks, st));
-  else ASI_CUDA(launch_qr(qa, pl->nd, max_chunks, st));
+  ASI_CUDA(launch_orth(qa, pl->nd, st));
   return ASI_OK;
 }
 
-// A mode product that streams a large tensor once: the register-tiled kernel when the shape fits it
-// (strided fibers, a <= 128, at most four outputs, contiguous outputs per (o, j)), else the general one.
-cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, cudaStream_t st) {
-  const bool fits = !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && a.si == 1 && a.ldb_j == 1 && a.sj == a.I &&
+// A mode product: the register-tiled streaming kernel when a large tensor fits it (strided fibers, contiguous outputs
+// per (o, j)), the tensor cores for a wide factor on a bf16 tensor, else the grouped SIMT product.
+// dep: launched as a programmatic dependent (never the first kernel of a call: the kernels behind it may start
+// before it does, and must find everything older finished).
+cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, bool dep, cudaStream_t st) {
+  const bool fits = !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && a.si == 1 && a.sj == a.I &&
                     a.so == (int64_t)a.n_out * a.I && a.Q * a.a >= (1 << 20) &&
                     fiber2_supported(a.O, a.a, a.I, a.n_out, x_bf16) &&
                     (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0;
   if (!fits) {
-    int ichunk = 0;
-    size_t smem = 0;
-    if (!x_bf16 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && modeprod_stage_fits(a, &ichunk, &smem))
-      return launch_modeprod_stage(a, ichunk, smem, st);      // few columns, long mode
-    return launch_modeprod(a, x_bf16, st);
+    if (x_bf16 && a.tc_scratch) {
+      const cudaError_t e = launch_tc_lastmode(a, a.tc_scratch, a.tc_scratch_bytes, st);
+      if (e != cudaErrorNotSupported) return e;
+    }
+    GemmGroup g;
+    g.np = 0;
+    g.clear = nullptr;
+    gemm_add(&g, gemm_project(a.X, a.B, a.Y, a.O, a.a, a.I, a.n_out, a.so, a.sj, a.si, x_bf16));
+    return launch_gemm_group(g, x_bf16, dep, st);
   }
   Fiber2Args f;
   std::memset(&f, 0, sizeof(f));
   f.X = a.X;
   f.U = a.B;
-  f.ldu = (int)a.ldb_k;
+  f.ldu = a.n_out;
   f.Y = a.Y;
   f.y_so = a.so;
   f.y_sj = a.sj;
   f.O = a.O; f.I = a.I; f.a = (int)a.a; f.r = a.n_out;
   f.n_tiles = fiber2_tiles(a.O, a.I);
   f.project_only = 1;
+  f.plain = !dep;
   return launch_fiber2(f, fiber2_grid(a.O, a.a, a.I, a.n_out, x_bf16, (pl->d.flags & ASI_FLAG_SHARE_SM) != 0),
                        x_bf16, st);
 }
@@ -500,17 +508,30 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     a.a = cd[m];
     a.Q = a.O * a.I;
     a.n_out = pl->r[m];
-    a.ldb_k = pl->r[m];
-    a.ldb_j = 1;
     a.so = (int64_t)pl->r[m] * a.I;
     a.sj = a.I;
     a.si = 1;
     float* dst = (s == pl->nd - 1) ? core : reinterpret_cast<float*>(w + pl->off_T[s & 1]);
     a.Y = dst;
-    a.tc_scratch = w + pl->off_tc;
+    a.tc_scratch = pl->tc_bytes ? w + pl->off_tc : nullptr;
     a.tc_scratch_bytes = pl->tc_bytes;
     a.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(stream_modeprod(pl, a, src_bf16, st));
+    ASI_CUDA(stream_modeprod(pl, a, src_bf16, true, st));
+    if (s == 0 && pl->core_tok) {
+      CoreTokArgs t;
+      t.T = dst;
+      t.core = core;
+      t.r3 = pl->r[pl->nd - 1];
+      if (pl->nd == 3) {
+        t.U1 = U_new + pl->u_off[0]; t.U2 = U_new + pl->u_off[1];
+        t.B = (int)pl->dims[0]; t.N = (int)pl->dims[1]; t.r1 = pl->r[0]; t.r2 = pl->r[1];
+      } else {
+        t.U1 = nullptr; t.U2 = U_new + pl->u_off[0];
+        t.B = 1; t.N = (int)pl->dims[0]; t.r1 = 1; t.r2 = pl->r[0];
+      }
+      ASI_CUDA(launch_core_tok(t, st));
+      break;
+    }
     cd[m] = pl->r[m];
     src = dst;
     src_bf16 = false;
@@ -557,24 +578,42 @@ bool fork_ready(const asi_plan* pl) {
   return true;
 }
 
-asi_status_t expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w,
-                         cudaStream_t st, int slot = 0) {
+// P_m = A_m V: the tensor cores where the plan says so and the pointers allow it, else one product of a grouped launch
+cudaError_t tc_expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, int slot, cudaStream_t st) {
   const ModeView& v = pl->mv[m];
+  if (!pl->tc_mode[m]) return cudaErrorNotSupported;
   ExpandArgs e;
   e.X = act;
   e.V = V;
   e.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
-  e.O = v.O;
-  e.a = v.a;
-  e.I = v.I;
-  e.Q = v.Q;
+  e.O = v.O; e.a = v.a; e.I = v.I; e.Q = v.Q;
   e.r = v.r;
   e.nsplit = pl->nsplit[m];
   e.q_per_split = pl->q_per_split[m];
   e.tc_scratch = w + pl->off_tc + (size_t)slot * pl->tc_stride;
   e.tc_scratch_bytes = pl->tc_bytes;
   e.status = reinterpret_cast<int*>(w);
-  ASI_CUDA(launch_expand(e, pl->bf16, st));
+  return launch_tc_expand(e, e.tc_scratch, e.tc_scratch_bytes, st);
+}
+
+GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V, char* w) {
+  const ModeView& v = pl->mv[m];
+  return gemm_expand(act, V, reinterpret_cast<float*>(w + pl->off_Pp[m]), v.O, v.a, v.I, v.r, pl->nsplit[m],
+                     pl->q_per_split[m], pl->bf16);
+}
+
+// cold start: P_m = A_m Omega_m for one mode
+asi_status_t expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, cudaStream_t st) {
+  const cudaError_t e = tc_expand_mode(pl, m, act, V, w, 0, st);
+  if (e != cudaErrorNotSupported) {
+    ASI_CUDA(e);
+    return ASI_OK;
+  }
+  GemmGroup g;
+  g.np = 0;
+  g.clear = nullptr;
+  gemm_add(&g, simt_expand(pl, m, act, V, w));
+  ASI_CUDA(launch_gemm_group(g, pl->bf16, false, st));
   return ASI_OK;
 }
 
@@ -747,14 +786,37 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
     ASI_CUDA(launch_sm_pass1(a, pl->fast_S, pl->fast_R, pl->bf16, st));
     return finish_compress(pl, act, U_new, core, w, U_prev, st);
   }
-  ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
-  float* V = reinterpret_cast<float*>(w + pl->off_V);
+  for (int m = 0; m < pl->nd; ++m)                   // bulk and 16-byte copies; errors before anything is enqueued
+    if ((pl->fiber2[m] || pl->plane2) && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
+  // The first kernel on the caller's stream clears the status block and starts only when the stream's earlier work
+  // is done; the mode passes behind it do not depend on one another and are launched as programmatic dependents
+  // (each waits for its predecessor before it ends, so that what follows the last one sees all of them).
+  int* const status = reinterpret_cast<int*>(w);
+  bool first = true;
+  auto take_clear = [&]() {
+    int* c = first ? status : nullptr;
+    first = false;
+    return c;
+  };
+  GemmGroup gp, ge;
+  gp.np = ge.np = 0;
+  gp.clear = ge.clear = nullptr;
+  bool tc[ASI_MAX_MODES] = {false, false, false, false};
+  for (int m = 0; m < pl->nd; ++m) {
+    const ModeView& v = pl->mv[m];
+    if (pl->fiber[m] || (pl->plane && m >= 2)) continue;
+    float* V = reinterpret_cast<float*>(w + pl->v_off[m]);
+    tc[m] = pl->tc_mode[m] != 0 && (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+    if (tc[m]) continue;
+    gemm_add(&gp, gemm_project(act, U_prev + pl->u_off[m], V, v.O, v.a, v.I, v.r, v.I * v.r, 1, v.r, pl->bf16));
+    gemm_add(&ge, simt_expand(pl, m, act, V, w));
+  }
   const bool forked = allow_fork && fork_ready(pl);
   if (forked) {
     ASI_CUDA(cudaEventRecord(pl->fr.fork, st));
-    for (int i = 0; i < pl->nd - 1; ++i) ASI_CUDA(cudaStreamWaitEvent(pl->fr.side[i], pl->fr.fork, 0));
+    for (int i = 0; i < pl->nd - 1; ++i)
+      if (tc[i + 1]) ASI_CUDA(cudaStreamWaitEvent(pl->fr.side[i], pl->fr.fork, 0));
   }
-  const cudaStream_t st0 = st;
   if (pl->plane) {
     PlaneArgs g;
     g.X = act;
@@ -767,24 +829,14 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
     g.r3 = pl->r[2];
     g.r4 = pl->r[3];
     g.vec4 = (!pl->bf16 && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) ? 1 : 0;
-    g.status = reinterpret_cast<int*>(w);
-    if (pl->plane2) {
-      if (reinterpret_cast<uintptr_t>(act) & 15u) return ASI_ERR_INVALID_ARG;   // bulk copies need 16-byte alignment
-      ASI_CUDA(launch_plane2(g, pl->plane_grid, pl->bf16, st));
-    } else {
-      ASI_CUDA(launch_plane(g, pl->plane_grid, pl->bf16, st));
-    }
+    g.status = status;
+    g.clear = take_clear();
+    ASI_CUDA(pl->plane2 ? launch_plane2(g, pl->plane_grid, pl->bf16, st) : launch_plane(g, pl->plane_grid, pl->bf16, st));
   }
-  for (int m = 0; m < pl->nd; ++m)                   // argument errors before anything is forked
-    if (pl->fiber2[m] && !(pl->plane && m >= 2) && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
-    if (pl->plane && m >= 2) continue;
-    const int slot = forked ? m : 0;                 // scratch and stream of this mode's pass
-    st = (forked && m > 0) ? pl->fr.side[m - 1] : st0;
-    V = reinterpret_cast<float*>(w + pl->off_V + (size_t)slot * pl->v_stride);
+    if (!pl->fiber[m] || (pl->plane && m >= 2)) continue;
     if (pl->fiber2[m]) {
-      if (reinterpret_cast<uintptr_t>(act) & 15u) return ASI_ERR_INVALID_ARG;
       Fiber2Args f;
       std::memset(&f, 0, sizeof(f));
       f.X = act;
@@ -793,11 +845,10 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
       f.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
       f.O = v.O; f.I = v.I; f.a = (int)v.a; f.r = v.r;
       f.n_tiles = fiber2_tiles(v.O, v.I);
+      f.plain = first;
+      f.clear = take_clear();
       ASI_CUDA(launch_fiber2(f, pl->fiber_grid[m], pl->bf16, st));
-      continue;
-    }
-    if (pl->fiber[m]) {
-      // both products of the mode in one pass; V stays on chip
+    } else {
       FiberArgs f;
       f.X = act;
       f.U = U_prev + pl->u_off[m];
@@ -806,38 +857,58 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
       f.n_tiles = fiber_tiles(v.O, v.a, v.I);
       f.r = v.r;
       f.vec4 = (!pl->bf16 && v.I % 4 == 0 && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) ? 1 : 0;
+      f.clear = take_clear();
       ASI_CUDA(launch_fiber(f, pl->fiber_grid[m], pl->bf16, st));
-      continue;
     }
-    // V = A_m^T U_m^{prev}, stored [b_m x r_m]
+  }
+  if (gp.np) {
+    const bool dep = !first;
+    gp.clear = take_clear();
+    ASI_CUDA(launch_gemm_group(gp, pl->bf16, dep, st));
+    ASI_CUDA(launch_gemm_group(ge, pl->bf16, true, st));
+  }
+  const cudaStream_t st0 = st;
+  for (int m = 0; m < pl->nd; ++m) {
+    if (!tc[m]) continue;
+    const ModeView& v = pl->mv[m];
+    const int slot = forked ? m : 0;                 // scratch and stream of this mode's products
+    st = (forked && m > 0) ? pl->fr.side[m - 1] : st0;
+    if (st == st0 && first) {
+      ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
+      first = false;
+    }
+    // V = A_m^T U_m^{prev}, stored [b_m x r_m]; P = A_m V
     ModeProdArgs a;
     a.X = act;
     a.B = U_prev + pl->u_off[m];
-    a.Y = V;
-    a.O = v.O;
-    a.a = v.a;
-    a.I = v.I;
-    a.Q = v.Q;
+    a.Y = reinterpret_cast<float*>(w + pl->v_off[m]);
+    a.O = v.O; a.a = v.a; a.I = v.I; a.Q = v.Q;
     a.n_out = v.r;
-    a.ldb_k = v.r;
-    a.ldb_j = 1;
     a.so = v.I * v.r;
     a.sj = 1;
     a.si = v.r;
     a.tc_scratch = w + pl->off_tc + (size_t)slot * pl->tc_stride;
     a.tc_scratch_bytes = pl->tc_bytes;
-    a.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(launch_modeprod(a, pl->bf16, st));
-    // P = A_m V
-    s = expand_mode(pl, m, act, V, w, st, slot);
-    if (s != ASI_OK) return s;
+    a.status = status;
+    ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
+    const cudaError_t e = tc_expand_mode(pl, m, act, a.Y, w, slot, st);
+    if (e == cudaErrorNotSupported) {
+      GemmGroup g;
+      g.np = 0;
+      g.clear = nullptr;
+      gemm_add(&g, simt_expand(pl, m, act, a.Y, w));
+      ASI_CUDA(launch_gemm_group(g, pl->bf16, true, st));
+    } else {
+      ASI_CUDA(e);
+    }
   }
   st = st0;
   if (forked)
-    for (int i = 0; i < pl->nd - 1; ++i) {
-      ASI_CUDA(cudaEventRecord(pl->fr.join[i], pl->fr.side[i]));
-      ASI_CUDA(cudaStreamWaitEvent(st, pl->fr.join[i], 0));
-    }
+    for (int i = 0; i < pl->nd - 1; ++i)
+      if (tc[i + 1]) {
+        ASI_CUDA(cudaEventRecord(pl->fr.join[i], pl->fr.side[i]));
+        ASI_CUDA(cudaStreamWaitEvent(st, pl->fr.join[i], 0));
+      }
   return finish_compress(pl, act, U_new, core, w, nullptr, st);
 }
 
@@ -1065,8 +1136,7 @@ asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float
     return ASI_OK;
   }
   float* Z1 = reinterpret_cast<float*>(w + pl->off_Z[0]);
-  float* Z3a = reinterpret_cast<float*>(w + pl->off_Z[1]);
-  float* Z3 = reinterpret_cast<float*>(w + pl->off_Z[2]);
+  float* Z3 = reinterpret_cast<float*>(w + pl->off_Z[1]);
   const int64_t B = pl->dims[0], H = pl->dims[2], W = pl->dims[3];
   const int r1 = pl->r[0], r2 = pl->r[1], r3 = pl->r[2], r4 = pl->r[3];
   const int64_t per_sample = (int64_t)pl->d.cout * pl->Ho * pl->Wo;
@@ -1075,26 +1145,11 @@ asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float
   // term 1: Z1 = dY x_1 U_1^T
   a.X = dY; a.B = U + pl->u_off[0]; a.Y = Z1;
   a.O = 1; a.a = B; a.I = per_sample; a.Q = per_sample;
-  a.n_out = r1; a.ldb_k = r1; a.ldb_j = 1;
+  a.n_out = r1;
   a.so = (int64_t)r1 * per_sample; a.sj = per_sample; a.si = 1;
-  ASI_CUDA(stream_modeprod(pl, a, pl->bf16, st));
-  if (pl->conv_z3) {
-    // terms 2-3 in one launch
-    ASI_CUDA(launch_z3(core, U + pl->u_off[2], U + pl->u_off[3], Z3, r1 * r2, r3, r4, (int)H, (int)W, st));
-  } else {
-  // term 2: core x_3 U_3  -> [r1 r2, H, r4]
-  a.X = core; a.B = U + pl->u_off[2]; a.Y = Z3a;
-  a.O = (int64_t)r1 * r2; a.a = r3; a.I = r4; a.Q = a.O * a.I;
-  a.n_out = (int)H; a.ldb_k = 1; a.ldb_j = r3;
-  a.so = H * r4; a.sj = r4; a.si = 1;
-  ASI_CUDA(launch_modeprod(a, false, st));
-  // term 3: .. x_4 U_4 -> Z3 [r1 r2 H, W]
-  a.X = Z3a; a.B = U + pl->u_off[3]; a.Y = Z3;
-  a.O = (int64_t)r1 * r2 * H; a.a = r4; a.I = 1; a.Q = a.O;
-  a.n_out = (int)W; a.ldb_k = 1; a.ldb_j = r4;
-  a.so = W; a.sj = 1; a.si = 1;
-  ASI_CUDA(launch_modeprod(a, false, st));
-  }
+  ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
+  // terms 2-3 in one launch
+  ASI_CUDA(launch_z3(core, U + pl->u_off[2], U + pl->u_off[3], Z3, r1 * r2, r3, r4, (int)H, (int)W, st));
   // terms 4 and 5
   ConvTailArgs t;
   t.Z1 = Z1; t.Z3 = Z3; t.U2 = U + pl->u_off[1]; t.dW = dW;
@@ -1118,86 +1173,39 @@ asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const flo
   if (s != ASI_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
-  const int nd = pl->nd, nlead = nd - 1;
-  const int64_t Dout = pl->d.cout, Din = pl->dims[nd - 1];
-  const int rl = pl->r[nd - 1];
-
+  const int64_t B = pl->nd == 3 ? pl->dims[0] : 1, N = pl->nd == 3 ? pl->dims[1] : pl->dims[0], Dout = pl->d.cout;
+  const int m2 = pl->nd - 2;                         // the mode contracted first: tokens (two modes: the rows)
+  float* Y1 = reinterpret_cast<float*>(w + pl->off_Z[0]);
+  float* Z4 = reinterpret_cast<float*>(w + pl->off_Z[1]);
+  // Y1[b][o][j] = sum_n dY[b][n][o] U_2[n][j]
   ModeProdArgs a;
-  if (pl->lin_reorder) {
-    // dY x_2 U_2^T on the tensor cores -> [B][Dout][r2], then x_1 U_1^T -> [r1][Dout][r2]
-    const int64_t B = pl->dims[0], N = pl->dims[1];
-    const int r1 = pl->r[0], r2 = pl->r[1];
-    float* Y1 = reinterpret_cast<float*>(w + pl->off_Z[0]);
-    float* Y2 = reinterpret_cast<float*>(w + pl->off_Z[1]);
-    a.X = dY; a.B = U + pl->u_off[1]; a.Y = Y1;
-    a.O = B; a.a = N; a.I = Dout; a.Q = B * Dout;
-    a.n_out = r2; a.ldb_k = r2; a.ldb_j = 1;
-    a.so = Dout * r2; a.sj = 1; a.si = r2;
-    a.tc_scratch = w + pl->off_wtc; a.tc_scratch_bytes = pl->wtc_bytes;
-    a.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(launch_modeprod(a, true, st));
-    ModeProdArgs b;
-    b.X = Y1; b.B = U + pl->u_off[0]; b.Y = Y2;
-    b.O = 1; b.a = B; b.I = Dout * r2; b.Q = b.I;
-    b.n_out = r1; b.ldb_k = r1; b.ldb_j = 1;
-    b.so = (int64_t)r1 * b.I; b.sj = b.I; b.si = 1;
-    b.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(stream_modeprod(pl, b, false, st));
-    LinTailArgs t;
-    t.Z = Y2; t.core = core; t.U = U + pl->u_off[2]; t.dW = dW;
-    t.s1 = Dout * r2; t.s2 = 1; t.so = r2;
-    t.L1 = r1; t.L2 = r2; t.Dout = (int)Dout; t.Din = (int)Din; t.r = rl; t.lead_fastest = 1;
-    t.Z4p = reinterpret_cast<float*>(w + pl->off_Z[2]); t.nsplit = pl->lin_nsplit;
-    ASI_CUDA(launch_lin_tail(t, st));
-    return ASI_OK;
+  a.X = dY; a.B = U + pl->u_off[m2]; a.Y = Y1;
+  a.O = B; a.a = N; a.I = Dout; a.Q = B * Dout;
+  a.n_out = pl->r[m2];
+  a.so = Dout * a.n_out; a.sj = 1; a.si = a.n_out;
+  a.tc_scratch = pl->lin_tc ? w + pl->off_wtc : nullptr;
+  a.tc_scratch_bytes = pl->wtc_bytes;
+  a.status = reinterpret_cast<int*>(w);
+  if (pl->lin_tc) {
+    ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
+  } else {
+    GemmGroup g;
+    g.np = 0;
+    g.clear = nullptr;
+    gemm_add(&g, gemm_project(a.X, a.B, a.Y, a.O, a.a, a.I, a.n_out, a.so, a.sj, a.si, pl->bf16));
+    ASI_CUDA(launch_gemm_group(g, pl->bf16, false, st));
   }
-  // Z = dY x_1 U_1^T (x_2 U_2^T): leading modes one by one
-  int64_t cd[ASI_MAX_MODES];
-  for (int m = 0; m < nlead; ++m) cd[m] = pl->dims[m];
-  cd[nlead] = Dout;
-  const void* src = dY;
-  bool src_bf16 = pl->bf16;
-  int64_t lead_r = 1;
-  for (int m = 0; m < nlead; ++m) {
-    a.X = src; a.B = U + pl->u_off[m];
-    a.Y = reinterpret_cast<float*>(w + pl->off_Z[m]);
-    a.O = 1; a.I = 1;
-    for (int j = 0; j < m; ++j) a.O *= cd[j];
-    for (int j = m + 1; j <= nlead; ++j) a.I *= cd[j];
-    a.a = cd[m]; a.Q = a.O * a.I;
-    a.n_out = pl->r[m]; a.ldb_k = pl->r[m]; a.ldb_j = 1;
-    a.so = (int64_t)pl->r[m] * a.I; a.sj = a.I; a.si = 1;
-    a.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(stream_modeprod(pl, a, src_bf16, st));
-    cd[m] = pl->r[m];
-    lead_r *= pl->r[m];
-    src = a.Y;
-    src_bf16 = false;
-  }
-  if (!(pl->d.flags & ASI_FLAG_GENERIC_ONLY)) {
-    // Z4 = Z . core over the leading ranks and dW = Z4 U_last^T in one launch; Z is [r1 (r2)][Dout]
-    LinTailArgs t;
-    t.Z = static_cast<const float*>(src); t.core = core; t.U = U + pl->u_off[nd - 1]; t.dW = dW;
-    t.L1 = pl->r[0]; t.L2 = (nlead > 1) ? pl->r[1] : 1;
-    t.s1 = (int64_t)t.L2 * Dout; t.s2 = Dout; t.so = 1;
-    t.Dout = (int)Dout; t.Din = (int)Din; t.r = rl; t.lead_fastest = 0;
-    t.Z4p = reinterpret_cast<float*>(w + pl->off_Z[2]); t.nsplit = pl->lin_nsplit;
-    ASI_CUDA(launch_lin_tail(t, st));
-    return ASI_OK;
-  }
-  // Z4^T[k, o] = sum_{lead} Z[lead, o] core[lead, k]
-  float* Z4t = reinterpret_cast<float*>(w + pl->off_Z[2]);
-  a.X = src; a.B = core; a.Y = Z4t;
-  a.O = 1; a.a = lead_r; a.I = Dout; a.Q = Dout;
-  a.n_out = rl; a.ldb_k = rl; a.ldb_j = 1;
-  a.so = 0; a.sj = Dout; a.si = 1;
-  ASI_CUDA(launch_modeprod(a, false, st));
-  // dW[o, d] = sum_k Z4^T[k, o] U_last[d, k]
-  a.X = Z4t; a.B = U + pl->u_off[nd - 1]; a.Y = dW;
-  a.O = 1; a.a = rl; a.I = Dout; a.Q = Dout;
-  a.n_out = (int)Din; a.ldb_k = 1; a.ldb_j = rl;
-  a.so = 0; a.sj = 1; a.si = Din;
-  ASI_CUDA(launch_modeprod(a, false, st));
+  LinMidArgs mid;
+  mid.Y1 = Y1; mid.core = core; mid.Z4 = Z4;
+  mid.U1 = pl->nd == 3 ? U + pl->u_off[0] : nullptr;
+  mid.B = (int)B; mid.Dout = (int)Dout;
+  mid.r1 = pl->nd == 3 ? pl->r[0] : 1;
+  mid.r2 = pl->r[m2]; mid.r3 = pl->r[pl->nd - 1];
+  ASI_CUDA(launch_lin_mid(mid, st));
+  LinTailArgs t;
+  t.Z4 = Z4; t.U = U + pl->u_off[pl->nd - 1]; t.dW = dW;
+  t.Dout = (int)Dout; t.Din = (int)pl->dims[pl->nd - 1]; t.r = pl->r[pl->nd - 1];
+  ASI_CUDA(launch_lin_tail(t, st));
   return ASI_OK;
 }
 

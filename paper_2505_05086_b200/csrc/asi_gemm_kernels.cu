@@ -1,0 +1,405 @@
+// Grouped fp32 products of a tensor with a narrow factor (1..64 columns), any sizes, strides and ranks: the
+// projections V_m = A_m^T U_m, the expansions P_m = A_m V_m (Algorithm 1), the core products and the first
+// contraction of the linear backward wherever no shape-specialised kernel applies.  One launch runs several
+// products (the modes of a layer), a CTA finds its product in a table.
+//
+//   C[m][j] = sum_k A(m, k) B[k][j]      m: 32 rows per CTA, j < n <= BN, k in chunks of 128
+//     m-major A (a projection of a strided mode, the expansion of the last mode): A(m, k) = X[o sxo + k ld + m]
+//     k-major A (a projection of the last mode, the expansion of a strided mode): A(m, k) = X[(k / kin) sxo + m ld + k % kin]
+//
+// What bounds it: the factor is so narrow that a product is a stream over X; with 32 x n outputs per CTA there are
+// few CTAs and a long contraction, so the eight warps of a CTA split every chunk of 128 along k (16 each, all 32
+// rows and all columns in registers) and meet once, at the end, in warp order.  fp32 tensors with 16-byte rows
+// arrive by cp.async two or three chunks ahead; bf16 and ragged tensors pass through registers one chunk ahead.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "asi_internal.h"
+
+namespace asi {
+
+namespace {
+
+constexpr int kGT = 256, kGW = 8, kGM = 32, kGK = 128;
+constexpr int kPK = kGK + 4;             // pitch of a k-major tile: rows four banks apart
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void cp16(float* dst, const void* src, bool on) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp4(float* dst, const void* src, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ float as_f(float v) { return v; }
+__device__ __forceinline__ float as_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+// What passes through registers between global and shared memory: four 8-byte groups of bf16 or 16 single values
+template <typename TX, bool VEC> struct Regs { TX v[16]; };
+template <> struct Regs<__nv_bfloat16, true> { uint2 v[4]; };
+
+template <typename TX, bool KM, bool VEC, int BN>
+struct GemmTile {
+  static constexpr bool kAsync = VEC && sizeof(TX) == 4;
+  static constexpr int kTileA = KM ? kGM * kPK : kGK * kGM;      // floats
+  static constexpr int kTileB = kGK * BN;
+
+  // A chunk [k0, k0 + 128) x rows [m0, m0 + 32): position of element / vector t of this thread
+  static __device__ __forceinline__ void issue_async(float* As, const TX* X, const GemmProb& p, int m0, int k0, int kend) {
+    const int tid = threadIdx.x;
+    if constexpr (KM) {
+      const int v = tid & 31, k = k0 + 4 * v;
+      const bool kon = k < kend;
+      const int o = (kon && p.kin < p.K) ? k / p.kin : 0;
+      const TX* src = X + (kon ? (int64_t)o * p.sxo + (k - o * p.kin) : 0);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int m = (tid >> 5) + 8 * t;
+        const bool on = kon && m0 + m < p.M;
+        cp16(As + m * kPK + 4 * v, src + (on ? (int64_t)(m0 + m) * p.ld : 0), on);
+      }
+    } else {
+      const int v = tid & 7, m = m0 + 4 * v;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int k = (tid >> 3) + 32 * t;
+        const bool on = k0 + k < kend && m < p.M;
+        cp16(As + k * kGM + 4 * v, X + (on ? (int64_t)(k0 + k) * p.ld + m : 0), on);
+      }
+    }
+  }
+  static __device__ __forceinline__ void load_regs(Regs<TX, VEC>& rg, const TX* X, const GemmProb& p, int m0, int k0, int kend) {
+    const int tid = threadIdx.x;
+    if constexpr (VEC) {
+      static_assert(sizeof(TX) == 2, "fp32 vectors go through cp.async");
+      if constexpr (KM) {
+        const int k = k0 + 4 * (tid & 31);
+        const bool kon = k < kend;
+        const int o = (kon && p.kin < p.K) ? k / p.kin : 0;
+        const TX* src = X + (kon ? (int64_t)o * p.sxo + (k - o * p.kin) : 0);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int m = m0 + (tid >> 5) + 8 * t;
+          rg.v[t] = __ldg(reinterpret_cast<const uint2*>(src + ((kon && m < p.M) ? (int64_t)m * p.ld : 0)));
+        }
+      } else {
+        const int m = m0 + 4 * (tid & 7);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int k = k0 + (tid >> 3) + 32 * t;
+          rg.v[t] = __ldg(reinterpret_cast<const uint2*>(X + ((k < kend && m < p.M) ? (int64_t)k * p.ld + m : 0)));
+        }
+      }
+    } else if constexpr (KM) {
+      const int k = k0 + (tid & 127);
+      const bool kon = k < kend;
+      const int o = (kon && p.kin < p.K) ? k / p.kin : 0;
+      const TX* src = X + (kon ? (int64_t)o * p.sxo + (k - o * p.kin) : 0);
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        const int m = m0 + (tid >> 7) + 2 * t;
+        rg.v[t] = src[(kon && m < p.M) ? (int64_t)m * p.ld : 0];
+      }
+    } else {
+      const int m = m0 + (tid & 31);
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        const int k = k0 + (tid >> 5) + 8 * t;
+        rg.v[t] = X[(k < kend && m < p.M) ? (int64_t)k * p.ld + m : 0];
+      }
+    }
+  }
+  static __device__ __forceinline__ void store_regs(const Regs<TX, VEC>& rg, float* As, const GemmProb& p, int m0, int k0, int kend) {
+    const int tid = threadIdx.x;
+    if constexpr (VEC) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        int m, k;
+        float* dst;
+        if constexpr (KM) { m = (tid >> 5) + 8 * t; k = 4 * (tid & 31); dst = As + m * kPK + k; }
+        else { m = 4 * (tid & 7); k = (tid >> 3) + 32 * t; dst = As + k * kGM + m; }
+        const bool on = m0 + m < p.M && k0 + k < kend;
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (on)
+          f = make_float4(__uint_as_float(rg.v[t].x << 16), __uint_as_float(rg.v[t].x & 0xffff0000u),
+                          __uint_as_float(rg.v[t].y << 16), __uint_as_float(rg.v[t].y & 0xffff0000u));
+        *reinterpret_cast<float4*>(dst) = f;
+      }
+    } else {
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        int m, k;
+        if constexpr (KM) { m = (tid >> 7) + 2 * t; k = tid & 127; }
+        else { m = tid & 31; k = (tid >> 5) + 8 * t; }
+        As[KM ? m * kPK + k : k * kGM + m] = (m0 + m < p.M && k0 + k < kend) ? as_f(rg.v[t]) : 0.f;
+      }
+    }
+  }
+  static __device__ __forceinline__ void issue_b(float* Bs, const float* B, const GemmProb& p, int k0, int kend) {
+    const int tid = threadIdx.x;
+    if (p.bvec) {
+      constexpr int VPR = BN / 4;
+#pragma unroll
+      for (int t = 0; t < (kGK * VPR + kGT - 1) / kGT; ++t) {
+        const int e = tid + t * kGT, k = e / VPR, v = e - k * VPR;
+        if (kGK * VPR % kGT && e >= kGK * VPR) break;
+        const bool on = k0 + k < kend && 4 * v < p.n;
+        cp16(Bs + k * BN + 4 * v, B + (on ? (int64_t)(k0 + k) * p.ldb + 4 * v : 0), on);
+      }
+    } else {
+#pragma unroll 4
+      for (int t = 0; t < kGK * BN / kGT; ++t) {
+        const int e = tid + t * kGT, k = e / BN, j = e - k * BN;
+        const bool on = k0 + k < kend && j < p.n;
+        cp4(Bs + e, B + (on ? (int64_t)(k0 + k) * p.ldb + j : 0), on);
+      }
+    }
+  }
+
+  static __device__ void run(const GemmProb& p, int cta, int nst, float* smem) {
+    constexpr int TN = BN / 4;                         // columns per lane
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lm = lane & 7, ln = lane >> 3;
+    const int mt = cta % p.tiles_m, rest = cta / p.tiles_m, o = rest % p.O, split = rest / p.O;
+    const int m0 = mt * kGM;
+    const int kbeg = split * p.kps, kend = min(p.K, kbeg + p.kps);
+    const int nit = kend > kbeg ? (kend - kbeg + kGK - 1) / kGK : 0;
+    const TX* X = reinterpret_cast<const TX*>(p.X) + (KM ? 0 : (int64_t)o * p.sxo);
+    const float* B = p.B;
+    float* stage = smem;
+    constexpr int kStage = kTileA + kTileB;
+    float acc[4][TN];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+    Regs<TX, VEC> rg;
+    for (int s = 0; s < nst - 1; ++s) {
+      if (s < nit) {
+        if constexpr (kAsync) issue_async(stage + s * kStage, X, p, m0, kbeg + s * kGK, kend);
+        issue_b(stage + s * kStage + kTileA, B, p, kbeg + s * kGK, kend);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if constexpr (!kAsync) {
+      if (nit > 0) {
+        load_regs(rg, X, p, m0, kbeg, kend);
+        store_regs(rg, stage, p, m0, kbeg, kend);
+      }
+    }
+    int st = 0;
+#pragma unroll 1
+    for (int it = 0; it < nit; ++it) {
+      if (nst == 2) asm volatile("cp.async.wait_group 0;" ::: "memory");
+      else asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncthreads();
+      {
+        int sf = st + nst - 1;
+        if (sf >= nst) sf -= nst;
+        if (it + nst - 1 < nit) {
+          const int k0 = kbeg + (it + nst - 1) * kGK;
+          if constexpr (kAsync) issue_async(stage + sf * kStage, X, p, m0, k0, kend);
+          issue_b(stage + sf * kStage + kTileA, B, p, k0, kend);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+      const int k1 = kbeg + (it + 1) * kGK;
+      if constexpr (!kAsync) {
+        if (it + 1 < nit) load_regs(rg, X, p, m0, k1, kend);
+      }
+      const float* As = stage + st * kStage;
+      const float* Bs = As + kTileA + warp * 16 * BN;
+      if (kbeg + it * kGK + warp * 16 < kend) {
+#pragma unroll
+        for (int k4 = 0; k4 < 16; k4 += 4) {
+          float a[4][4];                               // [k][row] (m-major) or [row][k] (k-major)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 v = KM ? *reinterpret_cast<const float4*>(As + (lm + 8 * i) * kPK + warp * 16 + k4)
+                                : *reinterpret_cast<const float4*>(As + (warp * 16 + k4 + i) * kGM + 4 * lm);
+            a[i][0] = v.x; a[i][1] = v.y; a[i][2] = v.z; a[i][3] = v.w;
+          }
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const float* b = Bs + (k4 + kk) * BN;
+            if constexpr (BN == 8) {
+              const float2 v = *reinterpret_cast<const float2*>(b + 2 * ln);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float x = KM ? a[i][kk] : a[kk][i];
+                acc[i][0] = fmaf(x, v.x, acc[i][0]);
+                acc[i][1] = fmaf(x, v.y, acc[i][1]);
+              }
+            } else {
+#pragma unroll
+              for (int q = 0; q < TN / 4; ++q) {
+                const float4 v = *reinterpret_cast<const float4*>(b + 4 * ln + 16 * q);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const float x = KM ? a[i][kk] : a[kk][i];
+                  acc[i][4 * q] = fmaf(x, v.x, acc[i][4 * q]);
+                  acc[i][4 * q + 1] = fmaf(x, v.y, acc[i][4 * q + 1]);
+                  acc[i][4 * q + 2] = fmaf(x, v.z, acc[i][4 * q + 2]);
+                  acc[i][4 * q + 3] = fmaf(x, v.w, acc[i][4 * q + 3]);
+                }
+              }
+            }
+          }
+        }
+      }
+      st = (st + 1 == nst) ? 0 : st + 1;
+      if constexpr (!kAsync) {
+        if (it + 1 < nit) store_regs(rg, stage + st * kStage, p, m0, k1, kend);
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    // the warps' shares meet in warp order
+    float* red = smem;                                 // [8][32][BN]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float* dst = red + (warp * kGM + (KM ? lm + 8 * i : 4 * lm + i)) * BN;
+      if constexpr (BN == 8) {
+        *reinterpret_cast<float2*>(dst + 2 * ln) = make_float2(acc[i][0], acc[i][1]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < TN / 4; ++q)
+          *reinterpret_cast<float4*>(dst + 4 * ln + 16 * q) =
+              make_float4(acc[i][4 * q], acc[i][4 * q + 1], acc[i][4 * q + 2], acc[i][4 * q + 3]);
+      }
+    }
+    __syncthreads();
+    float* Y = p.Y + (int64_t)split * p.ysplit + (int64_t)o * p.so;
+#pragma unroll
+    for (int t = 0; t < kGM * BN / kGT; ++t) {
+      const int e = tid + t * kGT;
+      int m, j;
+      if (p.si == 1) { j = e / kGM; m = e - j * kGM; } else { m = e / BN; j = e - m * BN; }
+      float v = red[m * BN + j];
+#pragma unroll
+      for (int w = 1; w < kGW; ++w) v += red[(w * kGM + m) * BN + j];
+      if (m0 + m < p.M && j < p.n) Y[(int64_t)j * p.sj + (int64_t)(m0 + m) * p.si] = v;
+    }
+  }
+};
+
+template <typename TX, bool KM, bool VEC>
+__device__ __forceinline__ void gemm_dispatch(const GemmProb& p, int cta, int nst, float* smem) {
+  if (p.n <= 8) GemmTile<TX, KM, VEC, 8>::run(p, cta, nst, smem);
+  else if (p.n <= 16) GemmTile<TX, KM, VEC, 16>::run(p, cta, nst, smem);
+  else if (p.n <= 32) GemmTile<TX, KM, VEC, 32>::run(p, cta, nst, smem);
+  else GemmTile<TX, KM, VEC, 64>::run(p, cta, nst, smem);
+}
+
+int bn_of(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : (n <= 32 ? 32 : 64)); }
+
+}  // namespace
+
+template <typename TX>
+__global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ GemmGroup g) {
+  extern __shared__ __align__(16) float gemm_smem[];
+  pdl_launch_dependents();
+  int q = 0;
+  while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
+  const GemmProb& p = g.p[q];
+  const int cta = (int)blockIdx.x - p.first;
+  pdl_wait();
+  if (blockIdx.x == 0 && g.clear) g.clear[threadIdx.x] = 0;   // status block of the workspace (256 ints)
+  if (p.km) {
+    if (p.vec) gemm_dispatch<TX, true, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<TX, true, false>(p, cta, g.nst, gemm_smem);
+  } else {
+    if (p.vec) gemm_dispatch<TX, false, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<TX, false, false>(p, cta, g.nst, gemm_smem);
+  }
+}
+
+// CTAs the projection of a mode launches, and column splits of an expansion: enough for two CTAs per SM, at least
+// two chunks of 128 each, so that a partial of P is worth its reduction
+int gemm_expand_splits(int64_t a, int64_t Q) {
+  const int64_t tiles = (a + kGM - 1) / kGM;
+  int64_t ns = std::max<int64_t>(1, 296 / tiles);
+  ns = std::min<int64_t>(ns, std::max<int64_t>(1, Q / (2 * kGK)));
+  return (int)std::min<int64_t>(ns, 296);
+}
+
+GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_t a, int64_t I, int n, int64_t so, int64_t sj,
+                      int64_t si, bool bf16) {
+  GemmProb p;
+  std::memset(&p, 0, sizeof(p));
+  p.X = X; p.B = B; p.Y = Y; p.n = n; p.ldb = n;
+  p.km = I == 1;
+  p.nsplit = 1;
+  p.K = (int)a; p.kps = p.K;
+  p.sj = sj;
+  if (I == 1) {
+    p.M = (int)O; p.O = 1; p.ld = a; p.kin = p.K; p.si = so;
+  } else {
+    p.M = (int)I; p.O = (int)O; p.ld = I; p.sxo = a * I; p.kin = p.K; p.so = so; p.si = si;
+  }
+  const int64_t al = I == 1 ? a : I;
+  p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
+  p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15u) == 0;
+  p.tiles_m = (p.M + kGM - 1) / kGM;
+  return p;
+}
+
+GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_t a, int64_t I, int n, int nsplit, int64_t kps,
+                     bool bf16) {
+  GemmProb p;
+  std::memset(&p, 0, sizeof(p));
+  p.X = X; p.B = V; p.Y = Pp; p.n = n; p.ldb = n;
+  p.km = I != 1;
+  p.M = (int)a; p.O = 1; p.K = (int)(O * I);
+  p.nsplit = nsplit; p.kps = (int)kps;
+  p.ysplit = a * n; p.si = n; p.sj = 1;
+  if (I == 1) { p.ld = a; p.kin = p.K; }
+  else { p.ld = I; p.kin = (int)I; p.sxo = a * I; }
+  const int64_t al = I == 1 ? a : I;
+  p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
+  p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(V) & 15u) == 0;
+  p.tiles_m = (p.M + kGM - 1) / kGM;
+  return p;
+}
+
+// adds a product; more than 64 columns go as several products over the same X
+void gemm_add(GemmGroup* g, const GemmProb& p) {
+  for (int j = 0; j < p.n; j += 64) {
+    GemmProb q = p;
+    q.n = std::min(64, p.n - j);
+    q.B = p.B + j;
+    q.Y = p.Y + (int64_t)j * p.sj;
+    g->p[g->np++] = q;
+  }
+}
+
+bool gemm_fits(int64_t O, int64_t a, int64_t I, int n) {
+  return n >= 1 && n <= ASI_MAX_RANK && O * I < (1ll << 30) && a < (1ll << 30) && ((I + kGM - 1) / kGM) * O < (1ll << 30);
+}
+
+cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st) {
+  if (g.np < 1) return cudaSuccess;
+  int first = 0, bn = 8;
+  double bytes = 0.0;
+  for (int q = 0; q < g.np; ++q) {
+    GemmProb& p = g.p[q];
+    p.first = first;
+    first += p.tiles_m * p.O * p.nsplit;
+    bn = std::max(bn, bn_of(p.n));
+    bytes += (double)p.M * p.O * p.K * (bf16 ? 2 : 4);
+  }
+  g.nst = bn == 64 ? 2 : 3;
+  const size_t stage = (size_t)(kGM * kPK + kGK * bn) * 4;
+  const size_t smem = std::max<size_t>(stage * g.nst, (size_t)kGW * kGM * bn * 4);
+  ProfScope prof(ASI_K_MODEPROD, st, bytes);
+  auto kernel = bf16 ? k_gemm_group<__nv_bfloat16> : k_gemm_group<float>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
+  if (e != cudaSuccess) return e;
+  if (pdl) return launch_pdl(kernel, dim3((unsigned)first), dim3(kGT), smem, st, g);
+  kernel<<<(unsigned)first, kGT, smem, st>>>(g);
+  return cudaGetLastError();
+}
+
+}  // namespace asi

@@ -2,10 +2,8 @@
 // They are the correctness baseline every layer shape can fall back on; shape-specialised
 // kernels live in their own files.
 //
-//   k_modeprod : Y = X x_m B^T-like small contraction over one mode (Sec. 3.2, m-mode product)
-//   k_expand   : P_m = A_m V_m, split over the columns of the unfolding (Algorithm 1)
-//   k_qr_gram / k_qr_gsum / k_qr_solve : Orthogonalize(P) as Cholesky-QR with the Gram matrix and the
-//                triangular solve in fp64 -- in exact arithmetic the Gram-Schmidt basis
+//   k_fiber, k_plane : both products of a mode (of the two spatial modes) in one pass, ranks <= 8
+//   k_qrb_*    : Orthogonalize(P) for ranks 65..128 as Cholesky-QR in fp64 (up to 64: asi_orth_kernels.cu)
 //   k_conv_tail: terms 4 and 5 of C_ASI (appendix "Speedup")
 #include <cuda_bf16.h>
 
@@ -37,455 +35,6 @@ cudaError_t opt_in_smem(const void* kernel, size_t need) {
 
 __device__ __forceinline__ float ld_as_float(const float* p) { return *p; }
 __device__ __forceinline__ float ld_as_float(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-// four neighbouring values read once (streaming hint), as fp32
-template <typename TX>
-__device__ __forceinline__ float4 ld4_stream(const TX* p);
-template <>
-__device__ __forceinline__ float4 ld4_stream<float>(const float* p) {
-  return __ldcs(reinterpret_cast<const float4*>(p));
-}
-template <>
-__device__ __forceinline__ float4 ld4_stream<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 raw = __ldcs(reinterpret_cast<const uint2*>(p));
-  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
-  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
-  return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
-}
-
-// ---------------------------------------------------------------------------------------------
-// Tile loader: Xs[kl][ql] = X(k0 + kl, q0 + ql), zero outside [0,a) x [q0, q_end).
-// Fibers strided by I > 1 (or short fibers) are read column-wise: consecutive threads take
-// consecutive columns.  Contiguous long fibers (I == 1, a >= 32) are read along k.
-// ---------------------------------------------------------------------------------------------
-template <int KC, int TQ, int NT, typename TX>
-__device__ __forceinline__ void load_x_tile(float (*Xs)[TQ + 1], const TX* __restrict__ X, int64_t a,
-                                            int64_t I, int64_t k0, int64_t q0, int64_t q_end) {
-  const int tid = threadIdx.x;
-  // All the loads of a thread are issued first, from clamped addresses where the tile hangs over
-  // the edge, and selected when they are stored: a load under a condition, or next to the store of
-  // the one before, waits for its predecessor, and a chunk then costs KC * TQ / NT round trips.
-  static_assert((KC * TQ) % NT == 0 && NT % TQ == 0, "threads must tile the chunk");
-  constexpr int PER = KC * TQ / NT;
-  float v[PER];
-  if (I == 1 && a >= 32) {
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int idx = tid + t * NT;
-      const int64_t k = k0 + idx % KC, q = q0 + idx / KC;
-      const bool on = k < a && q < q_end;
-      v[t] = ld_as_float(X + (on ? q * a + k : 0));
-    }
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int idx = tid + t * NT;
-      const int kl = idx % KC, ql = idx / KC;
-      Xs[kl][ql] = (k0 + kl < a && q0 + ql < q_end) ? v[t] : 0.f;
-    }
-  } else {
-    const int ql = tid % TQ;
-    const int64_t q = q0 + ql;
-    const bool qok = q < q_end;
-    int64_t base = 0;
-    if (qok) {
-      const int64_t o = q / I, i = q - o * I;
-      base = o * a * I + i;
-    }
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int64_t k = k0 + tid / TQ + t * (NT / TQ);
-      v[t] = ld_as_float(X + ((qok && k < a) ? base + k * I : 0));
-    }
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int kl = tid / TQ + t * (NT / TQ);
-      Xs[kl][ql] = (qok && k0 + kl < a) ? v[t] : 0.f;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_modeprod: one thread per column q, R outputs per thread.
-// ---------------------------------------------------------------------------------------------
-template <int R, typename TX>
-__global__ void __launch_bounds__(128) k_modeprod(ModeProdArgs p) {
-  constexpr int KC = 32, TQ = 128, NT = 128;
-  __shared__ float Xs[KC][TQ + 1];
-  __shared__ __align__(16) float Bs[KC][R];
-  const int tid = threadIdx.x;
-  const int64_t q0 = (int64_t)blockIdx.x * TQ;
-  const int j0 = blockIdx.y * R;
-  const TX* X = reinterpret_cast<const TX*>(p.X);
-
-  float acc[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) acc[j] = 0.f;
-
-  for (int64_t k0 = 0; k0 < p.a; k0 += KC) {
-    load_x_tile<KC, TQ, NT, TX>(Xs, X, p.a, p.I, k0, q0, p.Q);
-    {
-      // the factor's chunk, its loads issued together like the tile's
-      static_assert((KC * R) % NT == 0, "threads must tile the factor chunk");
-      constexpr int PB = KC * R / NT;
-      float b[PB];
-#pragma unroll
-      for (int t = 0; t < PB; ++t) {
-        const int idx = tid + t * NT;
-        const int64_t k = k0 + idx / R;
-        const int jj = j0 + idx % R;
-        b[t] = p.B[(k < p.a && jj < p.n_out) ? k * p.ldb_k + jj * p.ldb_j : 0];
-      }
-#pragma unroll
-      for (int t = 0; t < PB; ++t) {
-        const int idx = tid + t * NT;
-        const int kl = idx / R, j = idx % R;
-        Bs[kl][j] = (k0 + kl < p.a && j0 + j < p.n_out) ? b[t] : 0.f;
-      }
-    }
-    __syncthreads();
-    const int kmax = (int)((p.a - k0 < KC) ? (p.a - k0) : KC);
-    for (int kl = 0; kl < kmax; ++kl) {
-      const float x = Xs[kl][tid];
-#pragma unroll
-      for (int j = 0; j < R; j += 4) {
-        const float4 b = *reinterpret_cast<const float4*>(&Bs[kl][j]);
-        acc[j + 0] = fmaf(x, b.x, acc[j + 0]);
-        acc[j + 1] = fmaf(x, b.y, acc[j + 1]);
-        acc[j + 2] = fmaf(x, b.z, acc[j + 2]);
-        acc[j + 3] = fmaf(x, b.w, acc[j + 3]);
-      }
-    }
-    __syncthreads();
-  }
-  const int64_t q = q0 + tid;
-  if (q < p.Q) {
-    const int64_t o = q / p.I, i = q - o * p.I;
-    float* y = p.Y + o * p.so + i * p.si;
-#pragma unroll
-    for (int j = 0; j < R; ++j)
-      if (j0 + j < p.n_out) y[(int64_t)(j0 + j) * p.sj] = acc[j];
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_gemm: register-tiled fp32 GEMM C = op(A) B for the last mode of a tensor (contiguous fibers) at
-// ranks >= 16, where the thread-per-column kernels above run out of parallelism:
-//   AKMAJOR  : C[M x N] = A[M x K] B[K x N], A stored [M][lda]      (V = A_m^T U, core product)
-//   !AKMAJOR : C[M x N] = A^T B,            A stored [K][lda]      (P = A_m V), K split over grid.y
-// CTA tile 64 x BN, K chunks of 32, thread tile 4 x BN/16; B and C are row-major with N columns.
-// ---------------------------------------------------------------------------------------------
-struct GemmArgs {
-  const void* A;
-  const float* B;
-  float* C;            // [nsplit][M][N]
-  int M, N, K;
-  int64_t lda;
-  int k_per_split;
-  int vec8;            // bf16 A rows may be read 16 bytes at a time (aligned base, lda % 8 == 0)
-};
-
-template <bool AKMAJOR, int BM, int BN, typename TX>
-__global__ void __launch_bounds__(BM * 4) k_gemm(GemmArgs p) {
-  constexpr int BK = 32, TN = BN / 16, NT = BM * 4;
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * BM;
-  const int kb = blockIdx.y * p.k_per_split;
-  const int ke = (kb + p.k_per_split < p.K) ? kb + p.k_per_split : p.K;
-  const TX* __restrict__ A = reinterpret_cast<const TX*>(p.A);
-  float acc[4][TN];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  for (int k0 = kb; k0 < ke; k0 += BK) {
-    if (AKMAJOR) {
-      if (sizeof(TX) == 2 && p.vec8 && k0 + BK <= ke) {
-        // 8 bf16 (16 bytes) per load: thread -> row r, k-octet o
-        for (int idx = tid; idx < BM * (BK / 8); idx += NT) {
-          const int r = idx / (BK / 8), o = idx % (BK / 8);
-          const int m = m0 + r;
-          uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-          if (m < p.M) raw = *reinterpret_cast<const uint4*>(A + (int64_t)m * p.lda + k0 + 8 * o);
-          const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            As[8 * o + 2 * e][r] = __uint_as_float(w[e] << 16);
-            As[8 * o + 2 * e + 1][r] = __uint_as_float(w[e] & 0xffff0000u);
-          }
-        }
-      } else {
-        for (int idx = tid; idx < BM * BK; idx += NT) {
-          const int r = idx / BK, kk = idx % BK;
-          const int m = m0 + r, k = k0 + kk;
-          As[kk][r] = (m < p.M && k < ke) ? ld_as_float(A + (int64_t)m * p.lda + k) : 0.f;
-        }
-      }
-    } else {
-      for (int idx = tid; idx < BM * BK; idx += NT) {
-        const int kk = idx / BM, r = idx % BM;
-        const int m = m0 + r, k = k0 + kk;
-        As[kk][r] = (m < p.M && k < ke) ? ld_as_float(A + (int64_t)k * p.lda + m) : 0.f;
-      }
-    }
-    for (int idx = tid; idx < BK * BN; idx += NT) {
-      const int kk = idx / BN, n = idx % BN;
-      const int k = k0 + kk;
-      Bs[kk][n] = (k < ke && n < p.N) ? p.B[(int64_t)k * p.N + n] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w};
-      float bv[TN];
-      if constexpr (TN == 4) {
-        const float4 b = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-        bv[0] = b.x; bv[1] = b.y; bv[2] = b.z; bv[3] = b.w;
-      } else {
-        const float2 b = *reinterpret_cast<const float2*>(&Bs[kk][tx * 2]);
-        bv[0] = b.x; bv[1] = b.y;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  float* C = p.C + (int64_t)blockIdx.y * p.M * p.N;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= p.M) continue;
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int n = tx * TN + j;
-      if (n < p.N) C[(int64_t)m * p.N + n] = acc[i][j];
-    }
-  }
-}
-
-template <bool AKMAJOR, typename TX>
-static cudaError_t launch_gemm_t(const GemmArgs& g, int nsplit, cudaStream_t st) {
-  GemmArgs a = g;
-  a.vec8 = (sizeof(TX) == 2 && g.lda % 8 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15u) == 0 &&
-            g.k_per_split % 8 == 0) ? 1 : 0;
-  if ((int64_t)((g.M + 63) / 64) * nsplit >= 148) {     // enough 64-row tiles to fill the machine
-    dim3 grid((unsigned)((g.M + 63) / 64), (unsigned)nsplit);
-    if (g.N <= 32) k_gemm<AKMAJOR, 64, 32, TX><<<grid, 256, 0, st>>>(a);
-    else k_gemm<AKMAJOR, 64, 64, TX><<<grid, 256, 0, st>>>(a);
-  } else {
-    dim3 grid((unsigned)((g.M + 31) / 32), (unsigned)nsplit);
-    if (g.N <= 32) k_gemm<AKMAJOR, 32, 32, TX><<<grid, 128, 0, st>>>(a);
-    else k_gemm<AKMAJOR, 32, 64, TX><<<grid, 128, 0, st>>>(a);
-  }
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_rowstream: the first-mode product Y[j][q] = sum_k B(k, j) X[k][q] (O = 1: row k of X is one
-// contiguous slab of Q values) with n_out <= R <= 8.  Pure streaming: a thread owns four neighbouring
-// columns and one of KS slices of the rows, and walks down its rows with UNR 16-byte loads in flight
-// (a single thread walking all rows is bound by the latency of its own loads); the KS partial sums
-// meet in shared memory in slice order.  The factor sits in shared memory.  X is read exactly once,
-// coalesced; nothing else of size moves.
-// ---------------------------------------------------------------------------------------------
-template <int R, typename TX>
-__global__ void __launch_bounds__(256) k_rowstream(ModeProdArgs p) {
-  constexpr int NT = 256, CG = 64, KS = NT / CG, UNR = 8;
-  extern __shared__ __align__(16) float rs_smem[];
-  float* Bsm = rs_smem;                              // [a][R], zero-padded
-  float* part = rs_smem + (((int)p.a * R + 3) & ~3); // [KS - 1][CG][4 R]
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < (int)p.a * R; idx += NT) {
-    const int k = idx / R, j = idx % R;
-    Bsm[idx] = (j < p.n_out) ? p.B[k * p.ldb_k + j * p.ldb_j] : 0.f;
-  }
-  __syncthreads();
-  const int cg = tid & (CG - 1), ks = tid / CG;
-  const int64_t q = ((int64_t)blockIdx.x * CG + cg) * 4;
-  const bool live = q < p.Q;
-  float acc[4][R];
-#pragma unroll
-  for (int c = 0; c < 4; ++c)
-#pragma unroll
-    for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
-  const int a = (int)p.a;
-  const int kper = (a + KS - 1) / KS;
-  int k0 = ks * kper;
-  const int k1 = (k0 + kper < a) ? k0 + kper : a;
-  if (live) {
-    const TX* X = reinterpret_cast<const TX*>(p.X) + q;
-    // batches of UNR rows, all loads of a batch issued before any is used; rows past the end of the
-    // slice are read from the slice's last row and contribute zero
-    for (; k0 < k1; k0 += UNR) {
-      float4 x[UNR];
-#pragma unroll
-      for (int u = 0; u < UNR; ++u) x[u] = ld4_stream<TX>(X + (int64_t)((k0 + u < k1) ? (k0 + u) : (k1 - 1)) * p.Q);
-#pragma unroll
-      for (int u = 0; u < UNR; ++u) {
-        const bool on = k0 + u < k1;
-        const float xs[4] = {on ? x[u].x : 0.f, on ? x[u].y : 0.f, on ? x[u].z : 0.f, on ? x[u].w : 0.f};
-        const int kr = on ? (k0 + u) : (k1 - 1);
-#pragma unroll
-        for (int j = 0; j < R; j += 4) {
-          const float4 b = *reinterpret_cast<const float4*>(Bsm + kr * R + j);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            acc[c][j] = fmaf(xs[c], b.x, acc[c][j]);
-            acc[c][j + 1] = fmaf(xs[c], b.y, acc[c][j + 1]);
-            acc[c][j + 2] = fmaf(xs[c], b.z, acc[c][j + 2]);
-            acc[c][j + 3] = fmaf(xs[c], b.w, acc[c][j + 3]);
-          }
-        }
-      }
-    }
-  }
-  if (ks > 0) {
-    float* dst = part + ((ks - 1) * CG + cg) * 4 * R;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int j = 0; j < R; j += 4)
-        *reinterpret_cast<float4*>(dst + c * R + j) = make_float4(acc[c][j], acc[c][j + 1], acc[c][j + 2], acc[c][j + 3]);
-  }
-  __syncthreads();
-  if (ks == 0 && live) {
-#pragma unroll 1
-    for (int s = 1; s < KS; ++s) {
-      const float* src = part + ((s - 1) * CG + cg) * 4 * R;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int j = 0; j < R; ++j) acc[c][j] += src[c * R + j];
-    }
-#pragma unroll
-    for (int j = 0; j < R; ++j)
-      if (j < p.n_out)
-        *reinterpret_cast<float4*>(p.Y + (int64_t)j * p.sj + q) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
-  }
-}
-
-template <typename TX>
-static cudaError_t launch_modeprod_t(const ModeProdArgs& p, cudaStream_t st) {
-  if (p.Q <= 0 || p.n_out <= 0) return cudaSuccess;
-  ProfScope prof(ASI_K_MODEPROD, st,
-                 (double)p.Q * p.a * sizeof(TX) + 4.0 * ((double)p.a * p.n_out + (double)p.Q * p.n_out));
-  if constexpr (std::is_same<TX, __nv_bfloat16>::value) {
-    // a dense contraction with a wide factor: tensor cores (tcgen05), when the shape fits
-    const cudaError_t e = launch_tc_lastmode(p, p.tc_scratch, p.tc_scratch_bytes, st);
-    if (e != cudaErrorNotSupported) return e;
-  }
-  if (p.O == 1 && p.n_out <= 8 && p.si == 1 && p.Q % 4 == 0 && p.sj % 4 == 0 && p.Q >= (1 << 16) &&
-      p.a <= 512 && p.a >= 8 && (reinterpret_cast<uintptr_t>(p.X) & 15u) == 0 &&
-      (reinterpret_cast<uintptr_t>(p.Y) & 15u) == 0) {
-    const unsigned grid = (unsigned)((p.Q / 4 + 63) / 64);
-    const auto smem = [&](int R) { return (size_t)((((int)p.a * R + 3) & ~3) + 3 * 64 * 4 * R) * 4; };
-    if (p.n_out <= 4) k_rowstream<4, TX><<<grid, 256, smem(4), st>>>(p);
-    else k_rowstream<8, TX><<<grid, 256, smem(8), st>>>(p);
-    return cudaGetLastError();
-  }
-  if (p.I == 1 && p.n_out >= 16 && p.n_out <= 64 && p.a >= 64 && p.Q >= 64 && p.sj == 1 && p.so == p.n_out &&
-      p.ldb_k == p.n_out && p.ldb_j == 1 && p.Q < (1 << 30) && p.a < (1 << 30)) {
-    GemmArgs g = {p.X, p.B, p.Y, (int)p.Q, p.n_out, (int)p.a, p.a, (int)p.a, 0};
-    return launch_gemm_t<true, TX>(g, 1, st);
-  }
-  int R = 4;
-  while (R < p.n_out && R < 64) R *= 2;
-  dim3 grid((unsigned)((p.Q + 127) / 128), (unsigned)((p.n_out + R - 1) / R));
-  switch (R) {
-    case 4: k_modeprod<4, TX><<<grid, 128, 0, st>>>(p); break;
-    case 8: k_modeprod<8, TX><<<grid, 128, 0, st>>>(p); break;
-    case 16: k_modeprod<16, TX><<<grid, 128, 0, st>>>(p); break;
-    case 32: k_modeprod<32, TX><<<grid, 128, 0, st>>>(p); break;
-    default: k_modeprod<64, TX><<<grid, 128, 0, st>>>(p); break;
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_modeprod(const ModeProdArgs& p, bool x_bf16, cudaStream_t st) {
-  return x_bf16 ? launch_modeprod_t<__nv_bfloat16>(p, st) : launch_modeprod_t<float>(p, st);
-}
-
-// ---------------------------------------------------------------------------------------------
-// k_expand: CTA (kc, s) owns rows [32 kc, 32 kc + 32) of P and the column split s.
-// Thread (kl, jg) accumulates R/8 entries of its row.  Partials are summed later in a fixed
-// order, so the result does not depend on scheduling.
-// ---------------------------------------------------------------------------------------------
-template <int R, typename TX>
-__global__ void __launch_bounds__(256) k_expand(ExpandArgs p) {
-  constexpr int KC = kExpandKC, TQ = 64, NT = 256, RJ = R / 8;
-  __shared__ float Xs[KC][TQ + 1];
-  __shared__ __align__(16) float Vs[TQ][R];
-  const int tid = threadIdx.x;
-  const int kl = tid / 8, jg = tid % 8;
-  const int64_t k0 = (int64_t)blockIdx.x * KC;
-  const int s = blockIdx.y;
-  const int64_t qb = (int64_t)s * p.q_per_split;
-  int64_t qe = qb + p.q_per_split;
-  if (qe > p.Q) qe = p.Q;
-  const TX* X = reinterpret_cast<const TX*>(p.X);
-
-  float acc[RJ];
-#pragma unroll
-  for (int j = 0; j < RJ; ++j) acc[j] = 0.f;
-
-  for (int64_t q0 = qb; q0 < qe; q0 += TQ) {
-    load_x_tile<KC, TQ, NT, TX>(Xs, X, p.a, p.I, k0, q0, qe);
-    for (int idx = tid; idx < TQ * R; idx += NT) {
-      const int ql = idx / R, j = idx % R;
-      const int64_t q = q0 + ql;
-      Vs[ql][j] = (q < qe && j < p.r) ? p.V[q * p.r + j] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int ql = 0; ql < TQ; ++ql) {
-      const float x = Xs[kl][ql];
-#pragma unroll
-      for (int j = 0; j < RJ; ++j) acc[j] = fmaf(x, Vs[ql][jg * RJ + j], acc[j]);
-    }
-    __syncthreads();
-  }
-  const int64_t k = k0 + kl;
-  if (k < p.a) {
-#pragma unroll
-    for (int j = 0; j < RJ; ++j) {
-      const int jj = jg * RJ + j;
-      if (jj < p.r) p.Pp[((int64_t)s * p.a + k) * p.r + jj] = acc[j];
-    }
-  }
-}
-
-template <typename TX>
-static cudaError_t launch_expand_t(const ExpandArgs& p, cudaStream_t st) {
-  ProfScope prof(ASI_K_EXPAND, st,
-                 (double)p.Q * p.a * sizeof(TX) + 4.0 * ((double)p.Q * p.r + (double)p.nsplit * p.a * p.r));
-  if constexpr (std::is_same<TX, __nv_bfloat16>::value) {
-    const cudaError_t e = launch_tc_expand(p, p.tc_scratch, p.tc_scratch_bytes, st);   // tensor cores when it fits
-    if (e != cudaErrorNotSupported) return e;
-  }
-  if (p.I == 1 && p.r >= 16 && p.r <= 64 && p.a >= 64 && p.Q < (1 << 30) && p.a < (1 << 30)) {
-    GemmArgs g = {p.X, p.V, p.Pp, (int)p.a, p.r, (int)p.Q, p.a, (int)p.q_per_split, 0};
-    return launch_gemm_t<false, TX>(g, p.nsplit, st);
-  }
-  int R = 8;
-  while (R < p.r) R *= 2;
-  dim3 grid((unsigned)((p.a + kExpandKC - 1) / kExpandKC), (unsigned)p.nsplit);
-  switch (R) {
-    case 8: k_expand<8, TX><<<grid, 256, 0, st>>>(p); break;
-    case 16: k_expand<16, TX><<<grid, 256, 0, st>>>(p); break;
-    case 32: k_expand<32, TX><<<grid, 256, 0, st>>>(p); break;
-    case 64: k_expand<64, TX><<<grid, 256, 0, st>>>(p); break;
-    default: k_expand<128, TX><<<grid, 256, 0, st>>>(p); break;
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_expand(const ExpandArgs& p, bool x_bf16, cudaStream_t st) {
-  return x_bf16 ? launch_expand_t<__nv_bfloat16>(p, st) : launch_expand_t<float>(p, st);
-}
-
 // ---------------------------------------------------------------------------------------------
 // k_fiber: P_m = A_m (A_m^T U_m) for one mode in ONE pass over the activation (Algorithm 1, both
 // products of a mode).  A tile is TQ whole fibers of the mode: a rows of TQ contiguous values when the
@@ -504,6 +53,7 @@ template <int R, typename TX>
 __global__ void __launch_bounds__(256) k_fiber(FiberArgs p) {
   constexpr int TQ = kFiberTQ, NT = 256, KS = NT / TQ;
   extern __shared__ __align__(16) float fsm[];
+  pass_begin(p.clear);
   const int tid = threadIdx.x, lane = tid & 31;
   const int a = (int)p.a, r = p.r;
   const bool last = p.I == 1;                       // fibers are contiguous
@@ -644,6 +194,7 @@ __global__ void __launch_bounds__(256) k_fiber(FiberArgs p) {
   for (int j = 0; j < R; ++j)
     for (int off = 1; off < QS; off <<= 1) acc2[j] += __shfl_xor_sync(0xffffffffu, acc2[j], off);
   (void)lane;
+  if (tid == 0) pdl_wait();
   if (ek < a && eqs == 0) {
     float* dst = p.Pp + ((int64_t)blockIdx.x * a + ek) * r;
 #pragma unroll
@@ -664,6 +215,7 @@ template <int R, typename TX>
 __global__ void __launch_bounds__(256) k_plane(PlaneArgs p) {
   constexpr int NT = 256;
   extern __shared__ __align__(16) float fsm[];
+  pass_begin(p.clear);
   const int tid = threadIdx.x;
   const int S = p.S, SS = S * S, NP = NT / S;
   float* Xs0 = fsm;
@@ -778,6 +330,7 @@ __global__ void __launch_bounds__(256) k_plane(PlaneArgs p) {
     n_cur = n_next;
     buf ^= 1;
   }
+  if (tid == 0) pdl_wait();
   // the NP planes of the CTA meet in shared memory in plane order: one partial of P3 and P4 per CTA
   if (pl < NP) {
 #pragma unroll
@@ -809,8 +362,7 @@ static cudaError_t launch_plane_t(const PlaneArgs& p, int grid, cudaStream_t st)
   const size_t smem = plane_smem(p.S);   // the default limit counts static shared memory too: always opt in
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_plane<R, TX>), smem);
   if (e != cudaSuccess) return e;
-  k_plane<R, TX><<<grid, 256, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_maybe_pdl(!p.clear, k_plane<R, TX>, dim3(grid), dim3(256), smem, st, p);
 }
 
 cudaError_t launch_plane(const PlaneArgs& p, int grid, bool x_bf16, cudaStream_t st) {
@@ -837,8 +389,7 @@ static cudaError_t launch_fiber_t(const FiberArgs& p, int grid, cudaStream_t st)
   const size_t smem = fiber_smem((int)p.a);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_fiber<R, TX>), smem);
   if (e != cudaSuccess) return e;
-  k_fiber<R, TX><<<grid, 256, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_maybe_pdl(!p.clear, k_fiber<R, TX>, dim3(grid), dim3(256), smem, st, p);
 }
 
 cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t st) {
@@ -846,270 +397,6 @@ cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t
                  (double)p.O * p.a * p.I * (x_bf16 ? 2 : 4) + 4.0 * ((double)p.a * p.r * (grid + 1)));
   if (p.r <= 4) return x_bf16 ? launch_fiber_t<4, __nv_bfloat16>(p, grid, st) : launch_fiber_t<4, float>(p, grid, st);
   return x_bf16 ? launch_fiber_t<8, __nv_bfloat16>(p, grid, st) : launch_fiber_t<8, float>(p, grid, st);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Orthogonalize.  Stage 1 (k_qr_gram): sum the column-split partials of P in fp64 in a fixed
-// order, keep P in fp64, and form this row chunk's share of G = P^T P.  Stage 2 (k_qr_solve):
-// G = R^T R by Cholesky (R upper, positive diagonal), U = P R^{-1} row by row.  That U is the
-// Gram-Schmidt basis of the columns of P.  A pivot d_j with d_j <= 1e-12 * trace(G), i.e. a
-// Gram-Schmidt residual below 1e-6 * ||P||_F, raises ASI_ERR_RANK_DEFICIENT in the status word.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_qr_gram(QRArgs args) {
-  const QRMode M = args.m[blockIdx.y];
-  const int c = blockIdx.x;
-  if (c >= M.nchunk || M.r > kQRMaxRank) return;   // ranks above 64 take the k_qrb_* kernels
-  __shared__ double Ps[kQRRows * kQRMaxRank];      // this chunk's rows of P, pitch r
-  constexpr int kPer = 16;
-  static_assert(kQRRows * kQRMaxRank == kPer * 256, "one thread holds 16 elements of a full chunk");
-  const int tid = threadIdx.x;
-  const int r = M.r;
-  const int row0 = c * kQRRows;
-  const int nrows = min(kQRRows, M.a - row0);
-  const int nval = nrows * r;                        // the chunk is one contiguous run of P
-  const int64_t base = (int64_t)row0 * r;
-  // A thread has 16 accumulators: `ethr` elements (a power of two) times 16 / ethr lanes that take
-  // every (16 / ethr)-th split, so 16 loads are in flight whatever the chunk's size; the lanes of
-  // an element then fold pairwise.  The order of the sum is fixed by (nval, nsplit) alone.
-  int ethr = 1, lg = 0;
-  while (ethr * 256 < nval) { ethr <<= 1; ++lg; }
-  const int ssub = 16 >> lg;
-  const int64_t sstride = (int64_t)M.a * r;
-  double acc[kPer];
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) acc[q] = 0.0;
-  // four batches of 16 loads are issued before the first is used: with many splits and a full chunk (one
-  // split per batch) the loop is otherwise one memory round trip per split
-  constexpr int kBatch = 4;
-  for (int s0 = 0; s0 < M.nsplit; s0 += kBatch * ssub) {
-    float t[kBatch][kPer];
-#pragma unroll
-    for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const int idx = tid + (q & (ethr - 1)) * 256;
-        const int s = s0 + b * ssub + (q >> lg);
-        const bool on = idx < nval && s < M.nsplit;
-        // Every load is issued, from a clamped address when off, and nothing here touches its
-        // result: a use or a condition next to a load makes the following loads wait for it.
-        t[b][q] = __ldcg(M.Pp + (on ? s * sstride + base + idx : 0));
-      }
-#pragma unroll
-    for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        const bool on = tid + (q & (ethr - 1)) * 256 < nval && s0 + b * ssub + (q >> lg) < M.nsplit;
-        acc[q] += on ? (double)t[b][q] : 0.0;
-      }
-  }
-#pragma unroll
-  for (int h = kPer / 2; h >= 1; h >>= 1)
-    if (h >= ethr) {
-#pragma unroll
-      for (int q = 0; q < h; ++q) acc[q] += acc[q + h];
-    }
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int idx = tid + q * 256;
-    if (q < ethr && idx < nval) {
-      M.Pred[base + idx] = acc[q];
-      Ps[idx] = acc[q];
-    }
-  }
-  __syncthreads();
-  // Thread (ti, tj) owns G[ti + 16x][tj + 16y]: per row of P it reads 4 + 4 values for 16 products.
-  const int ti = tid >> 4, tj = tid & 15;
-  double g[4][4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) g[x][y] = 0.0;
-  for (int rl = 0; rl < nrows; ++rl) {
-    const double* prow = Ps + rl * r;
-    double pi[4], pj[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      pi[t] = (ti + 16 * t < r) ? prow[ti + 16 * t] : 0.0;
-      pj[t] = (tj + 16 * t < r) ? prow[tj + 16 * t] : 0.0;
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) g[x][y] = fma(pi[x], pj[y], g[x][y]);
-  }
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int i = ti + 16 * x, j = tj + 16 * y;
-      if (i < r && j < r && j >= i) M.Gp[((int64_t)c * r + i) * r + j] = g[x][y];
-    }
-}
-
-// k_qr_gsum: G = sum of the row chunks' shares, chunk by chunk in order, left in the place of
-// share 0, so that the solve kernel's CTAs read r*r numbers each instead of every share.  One
-// thread per element of the upper triangle, eight loads in flight.
-__global__ void __launch_bounds__(256) k_qr_gsum(QRArgs args) {
-  const QRMode M = args.m[blockIdx.y];
-  const int rr = M.r * M.r;
-  const int e = blockIdx.x * 256 + threadIdx.x;
-  if (M.r > kQRMaxRank || e >= rr || (e % M.r) < (e / M.r)) return;
-  const double* G = M.Gp + e;
-  double acc = 0.0;
-#pragma unroll 16
-  for (int cc = 0; cc < M.nchunk; ++cc) acc += __ldcg(G + (int64_t)cc * rr);
-  M.Gp[e] = acc;
-}
-
-// k_qr_solve keeps the running Schur complement of the Cholesky factorisation and the rows it
-// solves in registers; shared memory carries only what one step hands to the next (the pivot
-// row, the next unknown of each row) and R^T for the row solve.
-constexpr int kQRPitch = kQRMaxRank + 1;
-
-__global__ void __launch_bounds__(256) k_qr_solve(QRArgs args) {
-  static_assert(kQRMaxRank == 64 && kQRRows == 64, "4 x 4 slots of stride 16; four threads per row");
-  const QRMode M = args.m[blockIdx.y];
-  const int c = blockIdx.x;
-  const int row0 = c * kQRRows;
-  if (c >= M.nchunk || row0 >= M.a || M.r > kQRMaxRank) return;
-  __shared__ double Rt[kQRMaxRank * kQRPitch];      // Rt[k][j] = R[j][k], k > j
-  __shared__ double rowbuf[2][kQRMaxRank];          // pivot row of step j in rowbuf[j & 1]
-  __shared__ double pub[2][kQRRows];                  // v_j of each row in pub[j & 1]
-  __shared__ double Rinv[kQRMaxRank];               // 1 / R[j][j]
-  __shared__ double s_trace;
-  const int tid = threadIdx.x;
-  const int r = M.r;
-  const int ti = tid >> 4, tj = tid & 15;             // slot (x, y) of a thread is G[ti + 16x][tj + 16y]
-
-  // The rows of P this CTA solves: four threads per row, thread ql holds columns ql, ql + 4, ...
-  const int rowl = tid >> 2, ql = tid & 3;
-  const int row = row0 + rowl;
-  const bool live = row < M.a;                        // rows past the end are solved as zeros, unstored
-  double v[kQRMaxRank / 4];
-  {
-    const double* prow = M.Pred + (int64_t)(live ? row : 0) * r;
-#pragma unroll
-    for (int t = 0; t < kQRMaxRank / 4; ++t) {
-      const int k = ql + 4 * t;
-      v[t] = __ldcg(prow + (k < r ? k : 0));         // unconditional, selected afterwards
-    }
-#pragma unroll
-    for (int t = 0; t < kQRMaxRank / 4; ++t)
-      if (!(live && ql + 4 * t < r)) v[t] = 0.0;
-  }
-  // G = sum of the row chunks' shares, chunk by chunk in order (upper triangle).
-  double g[4][4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) g[x][y] = 0.0;
-  const int nsum = args.gsum ? 1 : M.nchunk;          // share 0 already holds the total
-  for (int cc = 0; cc < nsum; cc += 2) {              // two chunks' loads in flight, added in order
-    const double* Gc = M.Gp + (int64_t)cc * r * r;
-    const bool two = cc + 1 < nsum;
-    double t0[4][4], t1[4][4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const int i = ti + 16 * x, k = tj + 16 * y;
-        const bool on = k < r && k >= i;
-        const int o = on ? i * r + k : 0;
-        t0[x][y] = __ldcg(Gc + o);                   // unconditional loads, selected afterwards
-        t1[x][y] = __ldcg(Gc + (two ? r * r : 0) + o);
-      }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const int i = ti + 16 * x, k = tj + 16 * y;
-        const bool on = k < r && k >= i;
-        g[x][y] = (g[x][y] + (on ? t0[x][y] : 0.0)) + ((on && two) ? t1[x][y] : 0.0);
-      }
-  }
-  // Diagonal -> trace; row 0 -> the first pivot row.
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-    if (ti == tj && ti + 16 * x < r) Rinv[ti + 16 * x] = g[x][x];
-  if (ti == 0) {
-#pragma unroll
-    for (int y = 0; y < 4; ++y)
-      if (tj + 16 * y < r) rowbuf[0][tj + 16 * y] = g[0][y];
-  }
-  if (ql == 0) pub[0][rowl] = v[0];
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0.0;
-    for (int i = 0; i < r; ++i) t += Rinv[i];
-    s_trace = t;
-  }
-  __syncthreads();
-  const double floor_d = 1e-12 * s_trace;
-  // Right-looking Cholesky, one barrier per column.  Step j reads the pivot row (row j of the
-  // Schur complement), updates the rows below it in registers, hands row j + 1 to the next step
-  // and leaves R[j][k] = G[j][k] / R[j][j] in Rt.
-  for (int j = 0; j < r; ++j) {
-    const double* rb = rowbuf[j & 1];
-    double* nb = rowbuf[(j + 1) & 1];
-    double d = rb[j];
-    if (!(d > floor_d)) {
-      if (tid == 0 && c == 0) atomicMax(args.status, (int)ASI_ERR_RANK_DEFICIENT);
-      d = (floor_d > 0.0) ? floor_d : 1.0;
-    }
-    const double inv = rsqrt(d);
-    double ai[4], bk[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int i = ti + 16 * t, k = tj + 16 * t;
-      ai[t] = (i > j && i < r) ? rb[i] * inv : 0.0;
-      bk[t] = (k > j && k < r) ? rb[k] * inv : 0.0;
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const int i = ti + 16 * x, k = tj + 16 * y;
-        g[x][y] = fma(-ai[x], bk[y], g[x][y]);       // ai, bk are 0 outside the trailing block
-        if (i == j + 1 && k >= i && k < r) nb[k] = g[x][y];
-      }
-    if (tid > j && tid < r) Rt[tid * kQRPitch + j] = rb[tid] * inv;
-    if (tid == 0) Rinv[j] = inv;
-    __syncthreads();
-  }
-  // U = P R^{-1}, row by row: q_j = v_j / R[j][j], then v_k -= q_j R[j][k] for k > j.  The four
-  // threads of a row sit in one warp; every lane takes every step (the warp barriers are
-  // unconditional), and the thread that owns column j + 1 hands v_{j+1} to the next step.
-  for (int j = 0; j < r; ++j) {
-    double rt[kQRMaxRank / 4];
-#pragma unroll
-    for (int t = 0; t < kQRMaxRank / 4; ++t) {
-      const int k = ql + 4 * t;
-      rt[t] = (k > j && k < r) ? Rt[k * kQRPitch + j] : 0.0;
-    }
-    const double q = pub[j & 1][rowl] * Rinv[j];
-    double* np = pub[(j + 1) & 1];
-#pragma unroll
-    for (int t = 0; t < kQRMaxRank / 4; ++t) {
-      const int k = ql + 4 * t;
-      v[t] = (k == j) ? q : fma(-q, rt[t], v[t]);     // rt = 0 leaves the solved and the unused columns alone
-      if (k == j + 1 && k < r) np[rowl] = v[t];
-    }
-    __syncwarp();
-  }
-  if (live) {
-    float* urow = M.Uout + (int64_t)row * r;
-#pragma unroll
-    for (int t = 0; t < kQRMaxRank / 4; ++t) {
-      const int k = ql + 4 * t;
-      if (k < r) urow[k] = (float)v[t];
-    }
-  }
-}
-
-cudaError_t launch_qr_solve(const QRArgs& p, int nd, int max_chunks, cudaStream_t st) {
-  dim3 grid((unsigned)max_chunks, (unsigned)nd);
-  k_qr_solve<<<grid, 256, 0, st>>>(p);
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1210,7 +497,7 @@ __global__ void __launch_bounds__(128) k_qrb_solve(QRArgs args) {
   for (int j = 0; j < r; ++j) urow[j] = (float)u[j];
 }
 
-static cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st) {
+cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st) {
   int amax = 1, rmax = 1;
   for (int m = 0; m < nd; ++m)
     if (p.m[m].r > kQRMaxRank) {
@@ -1228,28 +515,6 @@ static cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_qr(const QRArgs& p, int nd, int max_chunks, cudaStream_t st) {
-  double qr_bytes = 0.0;
-  for (int m = 0; m < nd; ++m)
-    qr_bytes += 4.0 * p.m[m].a * p.m[m].r * (p.m[m].nsplit + 1);
-  ProfScope prof(ASI_K_QR, st, qr_bytes);
-  dim3 grid((unsigned)max_chunks, (unsigned)nd);
-  k_qr_gram<<<grid, 256, 0, st>>>(p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_qr_gsum<<<dim3(kQRMaxRank * kQRMaxRank / 256, (unsigned)nd), 256, 0, st>>>(p);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  QRArgs q = p;
-  q.gsum = 1;
-  k_qr_solve<<<grid, 256, 0, st>>>(q);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  for (int m = 0; m < nd; ++m)
-    if (p.m[m].r > kQRMaxRank) return launch_qr_big(p, nd, st);
-  return cudaSuccess;
-}
-
 // ---------------------------------------------------------------------------------------------
 // k_conv_tail: one CTA per output channel c'.  Thread (o, s): output o = (j, kh, kw) of Z4 and
 // split s of the reduction over (i, h'); partial sums meet in shared memory in a fixed order.
@@ -1257,6 +522,8 @@ cudaError_t launch_qr(const QRArgs& p, int nd, int max_chunks, cudaStream_t st) 
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_conv_tail(ConvTailArgs p) {
   extern __shared__ float sm[];
+  pdl_launch_dependents();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int co = blockIdx.x;
   const int kk = p.kh * p.kw;
@@ -1332,6 +599,8 @@ __global__ void __launch_bounds__(256) k_conv_tail(ConvTailArgs p) {
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_conv_z4(ConvTailArgs p, float* __restrict__ Z4p, int nsp) {
   extern __shared__ float sm[];
+  pdl_launch_dependents();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int co = blockIdx.x, sp = blockIdx.y;
   const int kk = p.kh * p.kw;
@@ -1370,8 +639,10 @@ __global__ void __launch_bounds__(256) k_conv_z4(ConvTailArgs p, float* __restri
   }
 }
 
-__global__ void __launch_bounds__(256) k_conv_dw(ConvTailArgs p, const float* __restrict__ Z4p, int nsp) {
+__global__ void __launch_bounds__(256) k_conv_dw(ConvTailArgs p, const float* Z4p, int nsp) {
   extern __shared__ float sm[];
+  pdl_launch_dependents();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int co = blockIdx.x;
   const int kk = p.kh * p.kw;
@@ -1408,11 +679,9 @@ cudaError_t launch_conv_tail_split(const ConvTailArgs& p, float* Z4p, int nsp, c
     if (e == cudaSuccess) e = opt_in_smem(reinterpret_cast<const void*>(k_conv_dw), smem);
     if (e != cudaSuccess) return e;
   }
-  k_conv_z4<<<dim3(p.Cout, nsp), 256, smem, st>>>(p, Z4p, nsp);
-  e = cudaGetLastError();
+  e = launch_pdl(k_conv_z4, dim3(p.Cout, nsp), dim3(256), smem, st, p, Z4p, nsp);
   if (e != cudaSuccess) return e;
-  k_conv_dw<<<p.Cout, 256, (size_t)n_out * sizeof(float), st>>>(p, Z4p, nsp);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_dw, dim3(p.Cout), dim3(256), (size_t)n_out * sizeof(float), st, p, (const float*)Z4p, nsp);
 }
 
 size_t conv_tail_smem(int r2, int kh, int kw) {
@@ -1433,8 +702,7 @@ cudaError_t launch_conv_tail(const ConvTailArgs& p, cudaStream_t st) {
     cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_conv_tail), smem);
     if (e != cudaSuccess) return e;
   }
-  k_conv_tail<<<p.Cout, 256, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(k_conv_tail, dim3(p.Cout), dim3(256), smem, st, p);
 }
 
 }  // namespace asi

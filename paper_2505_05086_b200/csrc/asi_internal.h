@@ -21,19 +21,17 @@ struct ModeView {
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr int kStatusBytes = 1024;    // status word (int 0), completion counters (ints 16..255)
-constexpr int kQRRows = 64;          // rows per CTA in the orthonormalisation kernels
-constexpr int kQRMaxRank = 64;       // ranks the register-resident Cholesky-QR kernels cover (above: k_qrb_*)
-constexpr int kExpandKC = 32;        // rows of P per CTA in the expand kernel
+constexpr int kQRMaxRank = 64;       // ranks k_orth_* cover (above: k_qrb_*)
+constexpr int kOrthGroups = 48;      // groups of Gram shares per mode (one counter each in the status block)
 
 // Y(o, j, i) = sum_k X(o, k, i) * B(k, j): the small-mode contraction that serves the
 // projection V = A_m^T U, the core products, Z1, Z3, and the final expansions.
 struct ModeProdArgs {
   const void* X;
-  const float* B;
+  const float* B;          // [a][n_out]
   float* Y;
   int64_t O, a, I, Q;
   int n_out;
-  int64_t ldb_k, ldb_j;    // B(k, j) = B[k*ldb_k + j*ldb_j]
   int64_t so, sj, si;      // Y(o, j, i) = Y[o*so + j*sj + i*si]
   void* tc_scratch = nullptr;      // device scratch for the tensor-core kernel's bf16 operand (optional)
   size_t tc_scratch_bytes = 0;
@@ -60,6 +58,7 @@ struct FiberArgs {
   float* Pp;
   int64_t O, a, I, n_tiles;
   int r, vec4;
+  int* clear;          // as in PlaneArgs
 };
 
 // Modes 3 and 4 of a conv activation in one pass over whole planes (k_plane).
@@ -71,6 +70,7 @@ struct PlaneArgs {
   float* Pp4;          // [grid][S][r4]
   int64_t n_planes;
   int S, r3, r4, vec4;
+  int* clear = nullptr;    // not null: CTA 0 zeroes the 256 ints of the workspace's status block
   int* status = nullptr;   // status word of the workspace (k_plane2: an expired wait on the bulk copy)
 };
 
@@ -84,19 +84,31 @@ struct Fiber2Args {
   int64_t y_so, y_sj;
   int64_t O, I, n_tiles;
   int ldu, a, r, project_only, nstage;
+  int plain;           // launched after all earlier work of the stream (the first kernel of a call)
+  int* clear;          // as in PlaneArgs (plain launches only)
 };
 
 struct QRMode {
   const float* Pp;     // [nsplit][a][r]
   double* Pred;        // [a][r]
-  double* Gp;          // [nchunk][r][r]
+  double* Gp;          // [nchunk][r][r] shares of G, then their group sums, then R^{-T} (orth_gp_elems doubles)
   float* Uout;         // [a][r]
+  int* gcount;         // one counter per group of shares, zero on entry and on exit
+  int* count;          // one counter, same convention
   int a, r, nsplit, nchunk;
+  int rows, gs;        // rows of P per share, shares per group
 };
 struct QRArgs {
   QRMode m[ASI_MAX_MODES];
   int* status;
-  int gsum;            // set by launch_qr: share 0 of Gp holds the whole of G (else k_qr_solve sums the shares)
+};
+// U_m = P_m R_m^{-1} for ranks <= 8, one row per thread, from what k_sm_reduce left (P_m and the Cholesky factor)
+struct RowSolveArgs {
+  const double* Pred[ASI_MAX_MODES];   // [a][r]
+  const double* Rf;                    // [modes][kRfStride]
+  float* U[ASI_MAX_MODES];
+  int a[ASI_MAX_MODES], r[ASI_MAX_MODES];
+  int nd, total;                       // total = sum of a
 };
 
 // Z4[c', j, kh, kw] = sum_{i,h',w'} Z1[i,c',h',w'] Z3pad[i,j,h's+kh-p,w's+kw-p], then
@@ -218,14 +230,89 @@ struct ProfScope {
   }
 };
 
+#ifdef __CUDACC__
+// Programmatic dependent launch.  A kernel launched with launch_pdl may start (and do whatever does not depend on
+// its predecessor in the stream) once every CTA of the predecessor has passed pdl_launch_dependents() or has
+// exited; pdl_wait() then blocks until the predecessor has finished and its writes are visible.  Without the
+// launch attribute both are no-ops.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A mode pass of Algorithm 1 depends on nothing the passes before it on the stream write.  The first one (clear not
+// null) is launched normally and zeroes the workspace's status block; the others are programmatic dependents that
+// run beside their predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass
+// sees all of them finished.
+__device__ __forceinline__ void pass_begin(int* clear) {
+  pdl_launch_dependents();
+  if (clear && blockIdx.x == 0)
+    for (int e = threadIdx.x; e < 256; e += blockDim.x) clear[e] = 0;
+}
+
+template <typename... Params, typename... Args>
+static inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                     const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+// a programmatic dependent when `dep`, else an ordinary launch
+template <typename... Params, typename... Args>
+static inline cudaError_t launch_maybe_pdl(bool dep, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                                           cudaStream_t st, const Args&... args) {
+  if (dep) return launch_pdl(kernel, grid, block, smem, st, args...);
+  kernel<<<grid, block, smem, st>>>(static_cast<Params>(args)...);
+  return cudaGetLastError();
+}
+#endif
+
 // Opt-in to more than 48 KB of dynamic shared memory.  The attribute belongs to a (device, kernel) pair,
 // so the sizes already granted are remembered per device.
 cudaError_t opt_in_smem(const void* kernel, size_t need);
 
-cudaError_t launch_modeprod(const ModeProdArgs& p, bool x_bf16, cudaStream_t st);
-cudaError_t launch_expand(const ExpandArgs& p, bool x_bf16, cudaStream_t st);
-cudaError_t launch_qr(const QRArgs& p, int nd, int max_chunks, cudaStream_t st);
-cudaError_t launch_qr_solve(const QRArgs& p, int nd, int max_chunks, cudaStream_t st);
+// One product of a grouped launch (asi_gemm_kernels.cu): C[m][j] = sum_k A(m, k) B[k][j] per outer index o
+struct GemmProb {
+  const void* X;
+  const float* B;          // [K][ldb], columns 0 .. n - 1
+  float* Y;                // C(o, m, j) of split s at s * ysplit + o * so + m * si + j * sj
+  int64_t sxo, ld, ysplit, so, sj, si;
+  int ldb;                 // row pitch of B
+  int kin;                 // k-major A: k per outer slab of X (K when there is one)
+  int M, K, O, n;
+  int nsplit, kps;         // K in nsplit parts of kps (a multiple of 128 unless nsplit == 1)
+  int tiles_m, first;      // 32-row tiles; first CTA of the product in the launch
+  int km, vec, bvec;       // k-major A; rows of A / of B readable four values at a time
+};
+constexpr int kMaxGroup = 8;
+struct GemmGroup {
+  GemmProb p[kMaxGroup];
+  int np, nst;
+  int* clear;              // not null: the first CTA zeroes the 256 ints of the workspace's status block
+};
+int gemm_expand_splits(int64_t a, int64_t Q);
+bool gemm_fits(int64_t O, int64_t a, int64_t I, int n);
+// Y(o, j, i) = sum_k X[o][k][i] B[k][j] at Y + o * so + j * sj + i * si
+void gemm_add(GemmGroup* g, const GemmProb& p);
+GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_t a, int64_t I, int n, int64_t so, int64_t sj,
+                      int64_t si, bool bf16);
+// Pp[s][k][j] = sum over the columns (o, i) of split s of X[o][k][i] V[(o, i)][j]
+GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_t a, int64_t I, int n, int nsplit, int64_t kps,
+                     bool bf16);
+cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st);
+
+int orth_rows(int64_t a, int r, int64_t nsplit);
+int orth_group(int64_t nchunk);
+size_t orth_gp_elems(int64_t nchunk, int r);
+cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st);
+cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st);
+cudaError_t launch_row_solve(const RowSolveArgs& p, cudaStream_t st);
 cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t st);
 size_t fiber_smem(int a);
 size_t conv_tail_smem(int r2, int kh, int kw);
@@ -253,23 +340,29 @@ cudaError_t launch_core_tail(const CoreTailArgs& p, cudaStream_t st);
 cudaError_t launch_z3(const float* core, const float* U3, const float* U4, float* Z3, int r12, int r3, int r4,
                       int H, int W, cudaStream_t st);
 // token path (asi_token_kernels.cu)
+struct CoreTokArgs {
+  const float* T;      // [B][N][r3]
+  const float* U1;     // [B][r1], or null: B = r1 = 1 with coefficient one
+  const float* U2;     // [N][r2]
+  float* core;         // [r1][r2][r3]
+  int B, N, r1, r2, r3;
+};
+cudaError_t launch_core_tok(const CoreTokArgs& p, cudaStream_t st);
+struct LinMidArgs {
+  const float* Y1;     // [B][Dout][r2]
+  const float* U1;     // [B][r1], or null: B = r1 = 1 with coefficient one
+  const float* core;   // [r1 r2][r3]
+  float* Z4;           // [Dout][r3]
+  int B, Dout, r1, r2, r3;
+};
+cudaError_t launch_lin_mid(const LinMidArgs& p, cudaStream_t st);
 struct LinTailArgs {
-  const float* Z;      // Z(l1, l2, o) = Z[l1 * s1 + l2 * s2 + o * so]
-  const float* core;   // [L1 L2][r]
+  const float* Z4;     // [Dout][r]
   const float* U;      // [Din][r]
   float* dW;           // [Dout][Din]
-  float* Z4p;          // [nsplit][Dout][r] shares of Z4 (scratch)
-  int nsplit;
-  int64_t s1, s2, so;
-  int L1, L2, Dout, Din, r;
-  int lead_fastest;    // 1: the lead index is the contiguous one in memory (s2 == 1), else o is
+  int Dout, Din, r, vec;
 };
-bool lin_tail_supported(int r);
-int lin_tail_nsplit(int nlead, int64_t Dout);
 cudaError_t launch_lin_tail(const LinTailArgs& p, cudaStream_t st);
-bool modeprod_stage_fits(const ModeProdArgs& p, int* ichunk, size_t* smem);
-int modeprod_stage_ksp(int64_t a);
-cudaError_t launch_modeprod_stage(const ModeProdArgs& p, int ichunk, size_t smem, cudaStream_t st);
 bool plane2_supported(int S, int64_t n_planes, int r3, int r4);
 int plane2_grid(int S, int64_t n_planes, int max_ctas);
 cudaError_t launch_plane2(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st);
@@ -305,14 +398,14 @@ struct asi_plan {
   bool bf16;
 
   // compress workspace (byte offsets)
-  size_t off_V, off_Pp[ASI_MAX_MODES], off_Pred[ASI_MAX_MODES], off_Gp[ASI_MAX_MODES], off_T[2];
+  size_t off_Pp[ASI_MAX_MODES], off_Pred[ASI_MAX_MODES], off_Gp[ASI_MAX_MODES], off_T[2];
   size_t off_Rf, off_Pg[ASI_MAX_MODES];
   size_t off_tc, tc_bytes;         // bf16 operand of the tensor-core products (0 bytes: not used)
-  // Token layers run the passes of their modes side by side (they read the same activation and write disjoint
-  // scratch): mode m > 0 is enqueued on a stream of the plan's own that forks from and joins the caller's
-  // stream by events.  Each mode then has its own V and operand scratch (strides below; 0 when not forked).
+  // Token layers with tensor-core modes run the passes of their modes side by side (they read the same activation
+  // and write disjoint scratch): such a mode m > 0 is enqueued on a stream of the plan's own that forks from and
+  // joins the caller's stream by events.  Each mode has its own V and operand scratch.
   bool fork;
-  size_t v_stride, tc_stride;
+  size_t v_off[ASI_MAX_MODES], tc_stride;
   struct ForkRes {
     cudaStream_t side[ASI_MAX_MODES - 1];
     cudaEvent_t fork, join[ASI_MAX_MODES - 1];
@@ -321,7 +414,7 @@ struct asi_plan {
   };
   mutable ForkRes fr;              // created at the first forked call (under a library-wide lock)
   int tc_mode[ASI_MAX_MODES];      // 0: SIMT, 1: last-mode tensor-core kernels, 2: inner-extent (token) kernels
-  int nsplit[ASI_MAX_MODES], nchunk[ASI_MAX_MODES];
+  int nsplit[ASI_MAX_MODES], nchunk[ASI_MAX_MODES], qr_rows[ASI_MAX_MODES];
   int64_t q_per_split[ASI_MAX_MODES];
   int core_order[ASI_MAX_MODES];
   size_t compress_ws;
@@ -329,10 +422,9 @@ struct asi_plan {
   // wgrad workspace (byte offsets)
   size_t off_Z[3], off_Z4p;
   int conv_nsp;                    // > 1: terms 4-5 in two launches with conv_nsp partial Z4 per channel
-  bool conv_z3;                    // terms 2-3 in one launch (k_z3)
-  int lin_nsplit;                  // shares of the leading indices in the Z4 kernel of the linear backward
-  bool lin_reorder;                // linear backward of a bf16 token layer: dY x_2 U_2^T first (tensor cores)
+  bool lin_tc;                     // linear backward: dY x_2 U_2^T on the tensor cores
   size_t off_wtc, wtc_bytes;       // bf16 operand scratch of that product
+  bool core_tok;                   // token layer whose first core product contracts the last mode: the rest in one launch
   bool core_tail;                  // the core products after the first in one launch
   size_t off_ctp;                  // partial cores of that launch
   size_t wgrad_ws;

@@ -95,6 +95,8 @@ __global__ void __launch_bounds__(kF2Threads, (RW <= 4 && NJ == 4) ? 3 : 2) k_fi
   constexpr int EPU = 16 / (int)sizeof(TX);          // elements per 16-byte unit
   constexpr int UPR = TQ / EPU;                      // units per staged row
   extern __shared__ __align__(128) unsigned char f2_smem[];
+  pass_begin(p.clear);
+  if (p.project_only) pdl_wait();                    // its factor comes from the kernel before
   const int tid = threadIdx.x, grp = tid >> 4, lane = tid & 15;
   const int a = p.a, r = p.r, nst = p.nstage;
   constexpr int AR = NG * RW;                        // staged rows: rows a..AR-1 stay zero, so no loop tests k < a
@@ -254,6 +256,7 @@ __global__ void __launch_bounds__(kF2Threads, (RW <= 4 && NJ == 4) ? 3 : 2) k_fi
   }
   cp_wait<0>();
   if (p.project_only) return;
+  if (tid == 0) pdl_wait();
   // the 16 lanes of a row group meet by shuffles in a fixed order; one partial of P per CTA
 #pragma unroll
   for (int i = 0; i < RW; ++i) {
@@ -314,8 +317,7 @@ template <int RW, int NJ, typename TX>
 static cudaError_t launch_fiber2_t(const Fiber2Args& p, int grid, size_t smem, cudaStream_t st) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_fiber2<RW, NJ, TX>), smem);
   if (e != cudaSuccess) return e;
-  k_fiber2<RW, NJ, TX><<<grid, kF2Threads, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_maybe_pdl(!p.plain, k_fiber2<RW, NJ, TX>, dim3(grid), dim3(kF2Threads), smem, st, p);
 }
 
 cudaError_t launch_fiber2(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
   extern __shared__ __align__(128) unsigned char p2_smem[];
   __shared__ __align__(8) uint64_t bars[NST];
   __shared__ int s_fail;
+  pass_begin(p.clear);
   TX* stages = reinterpret_cast<TX*>(p2_smem);                                   // [NST][G][S][S]
   f2* U3d = reinterpret_cast<f2*>(p2_smem + (size_t)NST * kTileBytes);           // [S][4]: (u, u)
   float* U4t = reinterpret_cast<float*>(U3d + S * 4);                            // [4][S]
@@ -564,6 +567,7 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
     }
     st = (st + 1 == NST) ? 0 : st + 1;
   }
+  if (tid == 0) pdl_wait();
   // ---- one partial of P3 and P4 per CTA: the threads' sums meet in shared memory in thread order
   __syncthreads();
   float* red3 = V3p;                 // [NT][4]
@@ -616,8 +620,7 @@ static cudaError_t launch_plane2_t(const PlaneArgs& p, int grid, cudaStream_t st
   const size_t smem = plane2_smem(S, sizeof(TX) == 2);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_plane2<S, TX>), smem);
   if (e != cudaSuccess) return e;
-  k_plane2<S, TX><<<grid, kP2Threads, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_maybe_pdl(!p.clear, k_plane2<S, TX>, dim3(grid), dim3(kP2Threads), smem, st, p);
 }
 
 cudaError_t launch_plane2(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st) {
@@ -641,6 +644,8 @@ int plane2_grid(int S, int64_t n_planes, int max_ctas) {
 __global__ void __launch_bounds__(256) k_core_tail(CoreTailArgs p) {
   extern __shared__ __align__(16) float ct_smem[];
   __shared__ int s_last;
+  pdl_launch_dependents();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int chunk = blockIdx.x, i = blockIdx.y, cs = blockIdx.z;
   const int r2 = p.r2, r3 = p.r3, r4 = p.r4, W = p.W, RH = p.RH;
@@ -739,8 +744,7 @@ cudaError_t launch_core_tail(const CoreTailArgs& p0, cudaStream_t st) {
   const size_t smem = 4 * ((size_t)p.r2 * p.RH * p.W + (size_t)p.r2 * p.RH * p.r4 + (size_t)p.cper * p.r2 +
                            (size_t)p.RH * p.r3 + (size_t)p.W * p.r4);
   ProfScope prof(ASI_K_MODEPROD, st, 4.0 * p.r1 * p.C * p.H * p.W);
-  k_core_tail<<<dim3(nchunk, p.r1, csplit), 256, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(k_core_tail, dim3(nchunk, p.r1, csplit), dim3(256), smem, st, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -750,6 +754,7 @@ __global__ void __launch_bounds__(256) k_z3(const float* __restrict__ core, cons
                                             const float* __restrict__ U4, float* __restrict__ Z3, int r12, int r3,
                                             int r4, int H, int W) {
   extern __shared__ float z3_smem[];
+  pdl_launch_dependents();
   float* Ss = z3_smem;                 // [r3][r4] of this (i, j)
   float* U3s = Ss + r3 * r4;           // [H][r3]
   float* U4s = U3s + H * r3;           // [W][r4]
@@ -768,6 +773,7 @@ __global__ void __launch_bounds__(256) k_z3(const float* __restrict__ core, cons
     }
     Z3[(int64_t)ij * H * W + pos] = s;
   }
+  if (tid == 0) pdl_wait();                          // Z1 (the kernel before) must be complete for what follows
 }
 
 cudaError_t launch_z3(const float* core, const float* U3, const float* U4, float* Z3, int r12, int r3, int r4,
@@ -776,8 +782,11 @@ cudaError_t launch_z3(const float* core, const float* U3, const float* U4, float
   int gx = (H * W + 255) / 256;
   if (gx > 16) gx = 16;
   const size_t smem = 4 * ((size_t)r3 * r4 + (size_t)H * r3 + (size_t)W * r4);
-  k_z3<<<dim3(gx, r12), 256, smem, st>>>(core, U3, U4, Z3, r12, r3, r4, H, W);
-  return cudaGetLastError();
+  if (smem > 40 * 1024) {
+    const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_z3), smem);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(k_z3, dim3(gx, r12), dim3(256), smem, st, core, U3, U4, Z3, r12, r3, r4, H, W);
 }
 
 }  // namespace asi

@@ -190,14 +190,6 @@ __device__ __forceinline__ void fma_row(float (&acc)[R], float x, const float* _
   }
 }
 
-// Programmatic dependent launch: the reduce and core kernels are launched with the
-// programmatic-stream-serialization attribute, so their CTAs may start (and do whatever does not
-// depend on the previous kernel, e.g. stage their activation tile) once every CTA of the previous
-// kernel has passed pdl_launch_dependents(); pdl_wait() then blocks until that kernel has finished
-// and its writes are visible.  Without the attribute both are no-ops.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Division of a small index (n < 2^21) by a run-time divisor through one reciprocal: the integer
 // division sequence costs ~150 cycles of latency, which dominates the short index loops below.
 struct FDiv {
@@ -877,30 +869,13 @@ __global__ void __launch_bounds__(kRedNT) k_sm_reduce_b(const __grid_constant__ 
   sm_reduce_cta(b.a[l], (int)blockIdx.x - b.first[l], (int)blockIdx.y);
 }
 
-// <<<>>> with the programmatic-stream-serialization attribute
-template <typename Arg>
-static cudaError_t launch_dependent(void (*kernel)(Arg), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                    const Arg& arg) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, arg);
-}
-
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st) {
   double bytes = 0.0;
   for (int m = 0; m < nd; ++m)
     bytes += 4.0 * p.m[m].nsplit * p.m[m].a * (p.m[m].gram ? p.m[m].a : p.m[m].r) + 8.0 * p.m[m].a * p.m[m].r;
   ProfScope prof(ASI_K_QR, st, bytes);
   dim3 grid((unsigned)max_chunks, (unsigned)nd);
-  return launch_dependent(k_sm_reduce, grid, dim3(kRedNT), 0, st, p);
+  return launch_pdl(k_sm_reduce, grid, dim3(kRedNT), 0, st, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1399,7 +1374,7 @@ static cudaError_t launch_core_t(const SmCoreArgs& p, cudaStream_t st) {
   const size_t smem = sm_core_smem(S, R, p.B);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core<S, R, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_dependent(k_sm_core<S, R, TX>, dim3(p.n_tiles), dim3(kNT), smem, st, p);
+  return launch_pdl(k_sm_core<S, R, TX>, dim3(p.n_tiles), dim3(kNT), smem, st, p);
 }
 
 template <int R, typename TX>
@@ -1465,7 +1440,7 @@ template <int S, int R, typename TX>
 static cudaError_t launch_core_bt(const SmBatch<SmCoreArgs>& b, size_t smem, cudaStream_t st) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core_b<S, R, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_dependent(k_sm_core_b<S, R, TX>, dim3(b.first[b.n]), dim3(kNT), smem, st, b);
+  return launch_pdl(k_sm_core_b<S, R, TX>, dim3(b.first[b.n]), dim3(kNT), smem, st, b);
 }
 template <int R, typename TX>
 static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, cudaStream_t st) {
@@ -1517,7 +1492,7 @@ cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunk
     b.first[l + 1] = b.first[l] + max_chunks[l];
   }
   ProfScope prof(ASI_K_QR, st, 0.0);
-  return launch_dependent(k_sm_reduce_b, dim3((unsigned)b.first[n], 4), dim3(kRedNT), 0, st, b);
+  return launch_pdl(k_sm_reduce_b, dim3((unsigned)b.first[n], 4), dim3(kRedNT), 0, st, b);
 }
 
 cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int S, int R, bool bf16, cudaStream_t st) {

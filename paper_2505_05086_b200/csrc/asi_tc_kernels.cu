@@ -356,7 +356,7 @@ cudaError_t launch_tc_token(const ModeProdArgs& p, void* scratch, size_t scratch
   const int nv = p.n_out, N = (nv + 15) / 16 * 16;       // the factor is zero-padded to a multiple of 16 columns
   const int64_t Kp = (p.a + 63) / 64 * 64;
   if (p.I < 64 || p.I % 64 != 0 || p.O < 1 || p.O >= 65536 || nv % 4 != 0 || nv < 16 || N > kTcNMax || p.a < 1 ||
-      p.a >= (1ll << 31) || p.I >= (1ll << 31) || p.sj != 1 || p.si != nv || p.so != p.I * nv || p.ldb_j != 1 ||
+      p.a >= (1ll << 31) || p.I >= (1ll << 31) || p.sj != 1 || p.si != nv || p.so != p.I * nv ||
       !scratch || scratch_bytes < tc_scratch_bytes(p.a, N) || (reinterpret_cast<uintptr_t>(scratch) & 15u) ||
       (reinterpret_cast<uintptr_t>(p.X) & 15u) || (reinterpret_cast<uintptr_t>(p.Y) & 15u))
     return cudaErrorNotSupported;
@@ -376,7 +376,7 @@ cudaError_t launch_tc_token(const ModeProdArgs& p, void* scratch, size_t scratch
   const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_token), kTcSmem);
   if (attr_err != cudaSuccess) return attr_err;
   k_tc_split<<<dim3((unsigned)((p.a + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      p.B, (int)p.ldb_k, (int)p.a, N, nv, static_cast<__nv_bfloat16*>(scratch), Kp);
+      p.B, nv, (int)p.a, N, nv, static_cast<__nv_bfloat16*>(scratch), Kp);
   TcArgs a = {p.Y, (int)p.I, N, (int)p.a, nv, (int)Kp, p.so, 0, p.status, nv};
   dim3 grid((unsigned)((p.I + kTcM - 1) / kTcM), (unsigned)p.O);
   k_tc_token<<<grid, kTcThreads, kTcSmem, st>>>(mapX, mapB, a);
@@ -426,7 +426,7 @@ cudaError_t launch_tc_lastmode(const ModeProdArgs& p, void* scratch, size_t scra
   const int64_t M = p.Q, K = p.a;
   const int nv = p.n_out, N = (nv + 15) / 16 * 16;
   if (p.I != 1 || nv % 4 != 0 || nv < 16 || N > kTcNMax || K % kTcKC != 0 || K < kTcKC || M < kTcM ||
-      M >= (1ll << 31) || K >= (1ll << 31) || p.sj != 1 || p.so % 4 != 0 || p.ldb_j != 1 || !scratch ||
+      M >= (1ll << 31) || K >= (1ll << 31) || p.sj != 1 || p.so % 4 != 0 || !scratch ||
       scratch_bytes < tc_scratch_bytes(K, N) || (reinterpret_cast<uintptr_t>(scratch) & 15u) ||
       (reinterpret_cast<uintptr_t>(p.X) & 15u) || (reinterpret_cast<uintptr_t>(p.Y) & 15u))
     return cudaErrorNotSupported;
@@ -456,7 +456,7 @@ cudaError_t launch_tc_lastmode(const ModeProdArgs& p, void* scratch, size_t scra
   const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_lastmode), smem);
   if (attr_err != cudaSuccess) return attr_err;
   k_tc_split<<<dim3((unsigned)((K + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      p.B, (int)p.ldb_k, (int)K, N, nv, static_cast<__nv_bfloat16*>(scratch), K);
+      p.B, nv, (int)K, N, nv, static_cast<__nv_bfloat16*>(scratch), K);
   TcArgs a = {p.Y, (int)M, N, (int)K, (int)p.so, (int)K, 0, 0, p.status, nv};
   const unsigned grid = (unsigned)((M + kTcM - 1) / kTcM);
   k_tc_lastmode<<<grid, kTcThreads, smem, st>>>(mapX, mapB, a);
