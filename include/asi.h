@@ -158,8 +158,9 @@ asi_status_t asi_philox_words(uint64_t seed, uint32_t stream_id, int64_t n_group
  * every layer has its own workspace (distinct pointers).  Results are bit-identical to n separate
  * calls.  Layers on the fused small-map path that share a kernel variant (map size, rank bucket, input
  * type) share one launch per kernel stage -- a step of L such layers is 3 + 1 launches instead of
- * 3L + L --, the others are enqueued one after another on `stream`.  Host-detectable errors are checked
- * for all layers before anything is enqueued. */
+ * 3L + L --; such a group and every other layer run side by side on streams the library keeps (at most eight sets
+ * of eight, destroyed with the last plan), forked from and joined to `stream` by events, or one after another when
+ * `stream` is being captured.  Host-detectable errors are checked for all layers before anything is enqueued. */
 asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* const* acts,
                                   const float* const* U_prev, float* const* U_new, float* const* cores,
                                   void* const* ws, const size_t* ws_bytes, int32_t n, void* stream);

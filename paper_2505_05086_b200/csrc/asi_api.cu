@@ -578,6 +578,88 @@ bool fork_ready(const asi_plan* pl) {
   return true;
 }
 
+// Side streams of the batched entry points: the layers of a step are independent, so their kernel chains run beside
+// one another on up to kLanes streams that fork from and join the caller's stream by events.  A call borrows a set
+// for the time it enqueues and hands it back (a set may serve the next call while its kernels still run: a stream
+// only orders work).  At most kMaxSets sets exist; they are destroyed with the last plan.  No set -- or a caller that
+// is capturing a graph, whose capture would otherwise keep the streams -- means one chain after another.
+constexpr int kLanes = 8, kMaxSets = 8;
+struct LaneSet {
+  int device;
+  cudaStream_t s[kLanes];
+  cudaEvent_t fork, join[kLanes];
+};
+std::mutex g_lane_mu;
+std::vector<LaneSet*> g_lane_idle;
+int g_lane_sets = 0;                                 // idle and borrowed
+long g_plans = 0;                                    // live plans (under g_lane_mu)
+
+void destroy_lanes(LaneSet* l) {
+  for (int i = 0; i < kLanes; ++i) {
+    if (l->s[i]) cudaStreamDestroy(l->s[i]);
+    if (l->join[i]) cudaEventDestroy(l->join[i]);
+  }
+  if (l->fork) cudaEventDestroy(l->fork);
+  delete l;
+}
+
+LaneSet* borrow_lanes(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  int dev = -1;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+      cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  std::lock_guard<std::mutex> lock(g_lane_mu);
+  for (size_t i = 0; i < g_lane_idle.size(); ++i)
+    if (g_lane_idle[i]->device == dev) {
+      LaneSet* l = g_lane_idle[i];
+      g_lane_idle.erase(g_lane_idle.begin() + i);
+      return l;
+    }
+  if (g_lane_sets >= kMaxSets) return nullptr;
+  LaneSet* l = new (std::nothrow) LaneSet;
+  if (!l) return nullptr;
+  std::memset(l, 0, sizeof(*l));
+  l->device = dev;
+  bool ok = cudaEventCreateWithFlags(&l->fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; ok && i < kLanes; ++i)
+    ok = cudaStreamCreateWithFlags(&l->s[i], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&l->join[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    (void)cudaGetLastError();
+    destroy_lanes(l);
+    return nullptr;
+  }
+  ++g_lane_sets;
+  return l;
+}
+
+// Runs n_chains independent pieces of work, chain c on the caller's stream (c == 0) or on a lane.
+template <typename F>
+asi_status_t run_chains(int n_chains, cudaStream_t st, F&& chain) {
+  LaneSet* l = n_chains > 1 ? borrow_lanes(st) : nullptr;
+  asi_status_t rc = ASI_OK;
+  cudaError_t e = cudaSuccess;
+  const int used = l ? std::min(n_chains - 1, kLanes) : 0;
+  if (l) e = cudaEventRecord(l->fork, st);
+  for (int i = 0; i < used && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(l->s[i], l->fork, 0);
+  for (int c = 0; c < n_chains && rc == ASI_OK && e == cudaSuccess; ++c)
+    rc = chain(c, (l && c > 0) ? l->s[(c - 1) % kLanes] : st);
+  for (int i = 0; i < used; ++i) {                   // joined whatever happened: nothing of this call stays behind
+    const cudaError_t e1 = cudaEventRecord(l->join[i], l->s[i]), e2 = cudaStreamWaitEvent(st, l->join[i], 0);
+    if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
+  }
+  if (l) {
+    std::lock_guard<std::mutex> lock(g_lane_mu);
+    g_lane_idle.push_back(l);
+  }
+  if (rc != ASI_OK) return rc;
+  ASI_CUDA(e);
+  return ASI_OK;
+}
+
 // P_m = A_m V: the tensor cores where the plan says so and the pointers allow it, else one product of a grouped launch
 cudaError_t tc_expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, int slot, cudaStream_t st) {
   const ModeView& v = pl->mv[m];
@@ -699,6 +781,10 @@ asi_status_t asi_plan_create(const asi_layer_desc_t* desc, asi_plan_t** out) {
   choose_kernels(pl);
   layout_compress(pl);
   layout_wgrad(pl);
+  {
+    std::lock_guard<std::mutex> lock(g_lane_mu);
+    ++g_plans;
+  }
   *out = pl;
   return ASI_OK;
 }
@@ -713,6 +799,12 @@ asi_status_t asi_plan_destroy(asi_plan_t* plan) {
     cudaEventDestroy(plan->fr.fork);
   }
   delete plan;
+  std::lock_guard<std::mutex> lock(g_lane_mu);
+  if (--g_plans == 0) {                              // the last plan takes the side streams with it
+    for (LaneSet* l : g_lane_idle) destroy_lanes(l);
+    g_lane_sets -= (int)g_lane_idle.size();
+    g_lane_idle.clear();
+  }
   return ASI_OK;
 }
 
@@ -946,18 +1038,29 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     for (int j = 0; j < i; ++j)
       if (ws[j] == ws[i]) return ASI_ERR_INVALID_ARG;            // every layer needs a workspace of its own
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  // chains: one per group of fused layers of a variant, one per other layer
   std::vector<char> done(n, 0);
+  std::vector<std::vector<int>> chains;
   const int maxb = sm_max_batch();
   for (int i = 0; i < n; ++i) {
-    if (done[i] || !plans[i]->fast_compress) continue;
-    const Variant v = {plans[i]->fast_S, plans[i]->fast_R, plans[i]->bf16 ? 1 : 0};
-    std::vector<int> grp;
-    for (int j = i; j < n && (int)grp.size() < maxb; ++j) {
-      const asi_plan* q = plans[j];
-      if (!done[j] && q->fast_compress && v == Variant{q->fast_S, q->fast_R, q->bf16 ? 1 : 0}) grp.push_back(j);
+    if (done[i]) continue;
+    std::vector<int> grp(1, i);
+    if (plans[i]->fast_compress) {
+      const Variant v = {plans[i]->fast_S, plans[i]->fast_R, plans[i]->bf16 ? 1 : 0};
+      for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j) {
+        const asi_plan* q = plans[j];
+        if (!done[j] && q->fast_compress && v == Variant{q->fast_S, q->fast_R, q->bf16 ? 1 : 0}) grp.push_back(j);
+      }
     }
-    const int g = (int)grp.size();
+    for (int j : grp) done[j] = 1;
+    chains.push_back(std::move(grp));
+  }
+  return run_chains((int)chains.size(), static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
+    const std::vector<int>& grp = chains[c];
+    const int g = (int)grp.size(), i0 = grp[0];
+    if (g == 1)
+      return asi_compress(plans[i0], acts[i0], U_prev[i0], U_new[i0], cores[i0], ws[i0], ws_bytes[i0], st);
+    const asi_plan* p0 = plans[i0];
     std::vector<SmPass1Args> pa(g);
     std::vector<SmReduceArgs> ra(g);
     std::vector<SmCoreArgs> ca(g);
@@ -968,18 +1071,12 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
       build_fused_pass1(plans[j], acts[j], U_prev[j], w, &pa[k]);
       mc[k] = build_fused_reduce(plans[j], w, U_prev[j], &ra[k]);
       build_fused_core(plans[j], acts[j], U_new[j], cores[j], w, true, &ca[k]);
-      done[j] = 1;
     }
-    ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, v.S, v.R, v.bf16 != 0, st));
+    ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_S, p0->fast_R, p0->bf16, st));
     ASI_CUDA(launch_sm_reduce_batched(ra.data(), mc.data(), g, st));
-    ASI_CUDA(launch_sm_core_batched(ca.data(), g, v.S, v.R, v.bf16 != 0, st));
-  }
-  for (int i = 0; i < n; ++i) {
-    if (done[i]) continue;
-    const asi_status_t s = asi_compress(plans[i], acts[i], U_prev[i], U_new[i], cores[i], ws[i], ws_bytes[i], stream);
-    if (s != ASI_OK) return s;
-  }
-  return ASI_OK;
+    ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_S, p0->fast_R, p0->bf16, st));
+    return ASI_OK;
+  });
 }
 
 asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* const* cores, const float* const* U,
@@ -994,33 +1091,35 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     if (s != ASI_OK) return s;
     if (pl->fast_wgrad && pl->wgrad_bulk && (reinterpret_cast<uintptr_t>(dY[i]) & 15u)) return ASI_ERR_INVALID_ARG;
   }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<char> done(n, 0);
+  std::vector<std::vector<int>> chains;
   const int maxb = sm_max_batch();
   for (int i = 0; i < n; ++i) {
-    if (done[i] || !plans[i]->fast_wgrad) continue;
-    const int R = plans[i]->fast_R, bf = plans[i]->bf16 ? 1 : 0;
-    std::vector<SmWgradArgs> wa;
-    for (int j = i; j < n && (int)wa.size() < maxb; ++j) {
-      const asi_plan* q = plans[j];
-      if (done[j] || !q->fast_wgrad || q->fast_R != R || (q->bf16 ? 1 : 0) != bf) continue;
-      SmWgradArgs g;
-      if (!build_fused_wgrad(q, cores[j], U[j], dY[j], dW[j], static_cast<char*>(ws[j]), &g))
-        return ASI_ERR_INVALID_ARG;
-      wa.push_back(g);
-      done[j] = 1;
-    }
-    ASI_CUDA(launch_sm_wgrad_batched(wa.data(), (int)wa.size(), R, bf != 0, st));
-  }
-  for (int i = 0; i < n; ++i) {
     if (done[i]) continue;
-    const asi_plan* pl = plans[i];
-    const asi_status_t s = pl->d.kind == ASI_CONV2D
-        ? asi_conv_wgrad(pl, cores[i], U[i], dY[i], dW[i], ws[i], ws_bytes[i], stream)
-        : asi_linear_wgrad(pl, cores[i], U[i], dY[i], dW[i], ws[i], ws_bytes[i], stream);
-    if (s != ASI_OK) return s;
+    std::vector<int> grp(1, i);
+    if (plans[i]->fast_wgrad)
+      for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j)
+        if (!done[j] && plans[j]->fast_wgrad && plans[j]->fast_R == plans[i]->fast_R && plans[j]->bf16 == plans[i]->bf16)
+          grp.push_back(j);
+    for (int j : grp) done[j] = 1;
+    chains.push_back(std::move(grp));
   }
-  return ASI_OK;
+  return run_chains((int)chains.size(), static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
+    const std::vector<int>& grp = chains[c];
+    const int g = (int)grp.size(), i0 = grp[0];
+    const asi_plan* p0 = plans[i0];
+    if (g == 1)
+      return p0->d.kind == ASI_CONV2D ? asi_conv_wgrad(p0, cores[i0], U[i0], dY[i0], dW[i0], ws[i0], ws_bytes[i0], st)
+                                      : asi_linear_wgrad(p0, cores[i0], U[i0], dY[i0], dW[i0], ws[i0], ws_bytes[i0], st);
+    std::vector<SmWgradArgs> wa(g);
+    for (int k = 0; k < g; ++k) {
+      const int j = grp[k];
+      if (!build_fused_wgrad(plans[j], cores[j], U[j], dY[j], dW[j], static_cast<char*>(ws[j]), &wa[k]))
+        return ASI_ERR_INVALID_ARG;                  // alignment: refused above, before anything was enqueued
+    }
+    ASI_CUDA(launch_sm_wgrad_batched(wa.data(), g, p0->fast_R, p0->bf16, st));
+    return ASI_OK;
+  });
 }
 
 // ---------------------------------------------------------------------------------------------
