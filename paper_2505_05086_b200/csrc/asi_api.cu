@@ -161,25 +161,19 @@ void layout_compress(asi_plan* pl) {
     pl->off_Gp[m] = off;
     off = align_up(off + orth_gp_elems(pl->nchunk[m], v.r) * 8, 256);
   }
-  // bf16 operand of the tensor-core kernels: products of bf16 tensors with a wide factor (16..64 columns, a
-  // multiple of 16) over the last mode (a_m a multiple of 64, >= 128 fibers) or over a mode whose inner
-  // extent I is a multiple of 64; the same scratch then serves the mode's expansion (operand = V_m)
-  pl->off_tc = off;
-  pl->tc_bytes = 0;
-  for (int m = 0; m < pl->nd; ++m) pl->tc_mode[m] = 0;
-  if (pl->bf16 && !pl->fast_compress)
-    for (int m = 0; m < pl->nd; ++m) {
-      const ModeView& v = pl->mv[m];
-      if (pl->r[m] % 4 != 0 || pl->r[m] < 16 || pl->r[m] > 64) continue;   // factor zero-padded to 16 x
-      const bool last = v.I == 1 && v.a % 64 == 0 && v.Q >= 128;
-      const bool inner = v.I >= 64 && v.I % 64 == 0 && v.O < 65536;
-      if (!last && !inner) continue;
-      pl->tc_mode[m] = last ? 1 : 2;
-      pl->tc_bytes = std::max(pl->tc_bytes, tc_scratch_bytes(std::max(v.a, v.Q), pl->r[m]));
-    }
-  pl->fork = pl->d.kind == ASI_LINEAR && pl->nd == 3 && pl->tc_bytes > 0 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY);
-  pl->tc_stride = pl->fork ? align_up(pl->tc_bytes, 256) : 0;
-  off = align_up(off + pl->tc_bytes, 256) + (pl->fork ? (size_t)(pl->nd - 1) * pl->tc_stride : 0);
+  // Tensor-core products of bf16 tensors: a factor of 16..64 columns (a multiple of 4) over the last mode (a_m a
+  // multiple of 64, at least 128 fibers) or over a mode whose inner extent is a multiple of 64
+  for (int m = 0; m < pl->nd; ++m) {
+    const ModeView& v = pl->mv[m];
+    pl->tc_mode[m] = 0;
+    if (pl->bf16 && pl->d.kind == ASI_LINEAR && !pl->fiber[m] && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY))
+      pl->tc_mode[m] = tc_kind(v.O, v.a, v.I, v.r);
+    if (!pl->tc_mode[m]) continue;
+    pl->tcu_off[m] = off;
+    off = align_up(off + tc_operand_bytes(v.a, v.r), 256);
+    pl->tcv_off[m] = off;
+    off = align_up(off + tc_operand_bytes(v.Q, v.r), 256);
+  }
   pl->off_Rf = off;                                   // Cholesky factors of the fused path
   off = align_up(off + (size_t)ASI_MAX_MODES * kRfStride * 8, 256);
   for (int m = 0; m < ASI_MAX_MODES; ++m) pl->off_Pg[m] = 0;
@@ -234,19 +228,14 @@ void layout_compress(asi_plan* pl) {
     // the two kernels of Orthogonalize, the core chain, one launch per one-pass mode (one for both spatial modes),
     // one projection and one expansion launch for all SIMT modes together
     pl->launches_compress = 2 + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
-    bool simt = false;
+    bool simt = false, tc = false;
     for (int m = 0; m < pl->nd; ++m) {
       if (pl->plane && m >= 2) pl->launches_compress += (m == 2);
       else if (pl->fiber[m]) pl->launches_compress += 1;
-      else if (pl->tc_mode[m]) {
-        // a tensor-core product is two launches (operand split + GEMM): V_m, the expansion when it fits too
-        const ModeView& v = pl->mv[m];
-        pl->launches_compress += 3;
-        if (pl->tc_mode[m] == 2 || (v.a % 8 == 0 && v.a >= 128 && v.Q % 8 == 0)) pl->launches_compress += 1;
-      } else simt = true;
-      // .. and the first core product when it contracts such a mode of the bf16 activation
-      if (pl->tc_mode[m] && pl->core_order[0] == m) pl->launches_compress += 1;
+      else if (pl->tc_mode[m]) tc = true;
+      else simt = true;
     }
+    if (tc) pl->launches_compress += 3;              // operand split, projections, expansions
     if (simt) pl->launches_compress += 2;
   }
 }
@@ -262,8 +251,8 @@ void layout_wgrad(asi_plan* pl) {
     // dY x_2 U_2^T [B][Dout][r2] (two modes: dY x_1 U_1^T [Dout][r1]), then Z4 [Dout][r_last]
     z[0] = pl->nd == 3 ? pl->dims[0] * pl->d.cout * pl->r[1] : (int64_t)pl->d.cout * pl->r[0];
     z[1] = (int64_t)pl->r[pl->nd - 1] * pl->d.cout;
-    pl->lin_tc = pl->nd == 3 && pl->bf16 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && pl->r[1] % 4 == 0 &&
-                 pl->r[1] >= 16 && pl->r[1] <= 64 && pl->d.cout % 64 == 0 && pl->dims[0] < 65536;
+    pl->lin_tc = pl->nd == 3 && pl->bf16 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
+                 tc_kind(pl->dims[0], pl->dims[1], pl->d.cout, pl->r[1]) == 2;
     pl->launches_wgrad = pl->lin_tc ? 4 : 3;
   }
   for (int t = 0; t < 3; ++t) {
@@ -271,11 +260,7 @@ void layout_wgrad(asi_plan* pl) {
     off = align_up(off + (size_t)z[t] * 4, 256);
   }
   pl->off_wtc = off;
-  pl->wtc_bytes = 0;
-  if (pl->d.kind == ASI_LINEAR && pl->lin_tc) {
-    pl->wtc_bytes = tc_scratch_bytes(pl->dims[1], pl->r[1]);
-    off = align_up(off + pl->wtc_bytes, 256);
-  }
+  if (pl->d.kind == ASI_LINEAR && pl->lin_tc) off = align_up(off + tc_operand_bytes(pl->dims[1], pl->r[1]), 256);
   pl->conv_nsp = 1;
   pl->off_Z4p = off;
   if (pl->d.kind == ASI_CONV2D && !pl->fast_wgrad && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
@@ -398,7 +383,7 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
 // gram_U_prev != nullptr: the partials of modes 3 and 4 of a 7x7 or 14x14 map are Gram matrices A_m A_m^T
 // (written by the fused first pass) and P_m = G_m U_m^prev is formed during the reduction.
 asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const float* gram_U_prev,
-                               cudaStream_t st) {
+                               bool first_core_tc, cudaStream_t st) {
   int max_chunks = 1;
   if (pl->fast_compress) {
     SmReduceArgs ra;
@@ -439,6 +424,11 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
     qa.m[m].gs = orth_group(pl->nchunk[m]);
     qa.m[m].count = reinterpret_cast<int*>(w) + 20 + m;
     qa.m[m].gcount = reinterpret_cast<int*>(w) + 64 + kOrthGroups * m;
+    if (first_core_tc && m == pl->core_order[0]) {   // the first core product reads U_m as a stacked operand
+      qa.m[m].bt = reinterpret_cast<__nv_bfloat16*>(w + pl->tcu_off[m]);
+      qa.m[m].bt_n = tc_operand_n(pl->r[m]);
+      qa.m[m].bt_ld = tc_operand_ld(pl->dims[m]);
+    }
   }
   qa.status = reinterpret_cast<int*>(w);
   ASI_CUDA(launch_orth(qa, pl->nd, st));
@@ -446,7 +436,7 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
 }
 
 // A mode product: the register-tiled streaming kernel when a large tensor fits it (strided fibers, contiguous outputs
-// per (o, j)), the tensor cores for a wide factor on a bf16 tensor, else the grouped SIMT product.
+// per (o, j)), else the grouped SIMT product.
 // dep: launched as a programmatic dependent (never the first kernel of a call: the kernels behind it may start
 // before it does, and must find everything older finished).
 cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, bool dep, cudaStream_t st) {
@@ -455,10 +445,6 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
                     fiber2_supported(a.O, a.a, a.I, a.n_out, x_bf16) &&
                     (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0;
   if (!fits) {
-    if (x_bf16 && a.tc_scratch) {
-      const cudaError_t e = launch_tc_lastmode(a, a.tc_scratch, a.tc_scratch_bytes, st);
-      if (e != cudaErrorNotSupported) return e;
-    }
     GemmGroup g;
     g.np = 0;
     g.clear = nullptr;
@@ -483,9 +469,20 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
 
 // Orthogonalize, then core = A x_1 U_1^T ... x_n U_n^T (Algorithm 1, core update with U^T).
 asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, float* core,
-                             char* w, const float* gram_U_prev, cudaStream_t st) {
-  asi_status_t qs = orthogonalize_all(pl, U_new, w, gram_U_prev, st);
+                             char* w, const float* gram_U_prev, bool tc_ready, cudaStream_t st) {
+  // the first core product runs on the tensor cores when its mode does: after a warm step the operand's zero columns
+  // are there from the split of U_prev and Orthogonalize fills in the rest, a cold start splits U_new here
+  const int m0 = pl->core_order[0];
+  const bool tc_core = pl->tc_mode[m0] == 1 && (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+  asi_status_t qs = orthogonalize_all(pl, U_new, w, gram_U_prev, tc_core && tc_ready, st);
   if (qs != ASI_OK) return qs;
+  if (tc_core && !tc_ready) {
+    TcSplitArgs sp;
+    sp.n = 0;
+    sp.clear = nullptr;
+    tc_add_split(&sp, U_new + pl->u_off[m0], pl->mv[m0].a, pl->r[m0], w + pl->tcu_off[m0]);
+    ASI_CUDA(launch_tc_split(sp, true, st));
+  }
   if (pl->fast_compress) {
     SmCoreArgs c;
     build_fused_core(pl, act, U_new, core, w, gram_U_prev != nullptr, &c);
@@ -513,10 +510,13 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     a.si = 1;
     float* dst = (s == pl->nd - 1) ? core : reinterpret_cast<float*>(w + pl->off_T[s & 1]);
     a.Y = dst;
-    a.tc_scratch = pl->tc_bytes ? w + pl->off_tc : nullptr;
-    a.tc_scratch_bytes = pl->tc_bytes;
-    a.status = reinterpret_cast<int*>(w);
-    ASI_CUDA(stream_modeprod(pl, a, src_bf16, true, st));
+    if (s == 0 && tc_core) {
+      const ModeView& v = pl->mv[m];
+      const TcCall t = {act, w + pl->tcu_off[m], dst, nullptr, 0, v.O, v.a, v.I, 0, v.r, 1, 0};
+      ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
+    } else {
+      ASI_CUDA(stream_modeprod(pl, a, src_bf16, true, st));
+    }
     if (s == 0 && pl->core_tok) {
       CoreTokArgs t;
       t.T = dst;
@@ -550,32 +550,6 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     }
   }
   return ASI_OK;
-}
-
-std::mutex g_fork_mu;
-
-// The plan's side streams and events, created on first use for the current device.  false: run the modes one
-// after another on the caller's stream (creation failed once, or the plan was first used on another device).
-bool fork_ready(const asi_plan* pl) {
-  if (!pl->fork) return false;
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  std::lock_guard<std::mutex> lock(g_fork_mu);
-  asi_plan::ForkRes& f = pl->fr;
-  if (f.failed) return false;
-  if (f.ready) return f.device == dev;
-  bool ok = cudaEventCreateWithFlags(&f.fork, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; ok && i < pl->nd - 1; ++i)
-    ok = cudaStreamCreateWithFlags(&f.side[i], cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&f.join[i], cudaEventDisableTiming) == cudaSuccess;
-  if (!ok) {
-    (void)cudaGetLastError();
-    f.failed = true;
-    return false;
-  }
-  f.device = dev;
-  f.ready = true;
-  return true;
 }
 
 // Side streams of the batched entry points: the layers of a step are independent, so their kernel chains run beside
@@ -660,24 +634,6 @@ asi_status_t run_chains(int n_chains, cudaStream_t st, F&& chain) {
   return ASI_OK;
 }
 
-// P_m = A_m V: the tensor cores where the plan says so and the pointers allow it, else one product of a grouped launch
-cudaError_t tc_expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, int slot, cudaStream_t st) {
-  const ModeView& v = pl->mv[m];
-  if (!pl->tc_mode[m]) return cudaErrorNotSupported;
-  ExpandArgs e;
-  e.X = act;
-  e.V = V;
-  e.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
-  e.O = v.O; e.a = v.a; e.I = v.I; e.Q = v.Q;
-  e.r = v.r;
-  e.nsplit = pl->nsplit[m];
-  e.q_per_split = pl->q_per_split[m];
-  e.tc_scratch = w + pl->off_tc + (size_t)slot * pl->tc_stride;
-  e.tc_scratch_bytes = pl->tc_bytes;
-  e.status = reinterpret_cast<int*>(w);
-  return launch_tc_expand(e, e.tc_scratch, e.tc_scratch_bytes, st);
-}
-
 GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V, char* w) {
   const ModeView& v = pl->mv[m];
   return gemm_expand(act, V, reinterpret_cast<float*>(w + pl->off_Pp[m]), v.O, v.a, v.I, v.r, pl->nsplit[m],
@@ -686,9 +642,16 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
 
 // cold start: P_m = A_m Omega_m for one mode
 asi_status_t expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, cudaStream_t st) {
-  const cudaError_t e = tc_expand_mode(pl, m, act, V, w, 0, st);
-  if (e != cudaErrorNotSupported) {
-    ASI_CUDA(e);
+  if (pl->tc_mode[m] && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) {
+    const ModeView& v = pl->mv[m];
+    TcSplitArgs sp;
+    sp.n = 0;
+    sp.clear = nullptr;
+    tc_add_split(&sp, V, v.Q, v.r, w + pl->tcv_off[m]);
+    ASI_CUDA(launch_tc_split(sp, false, st));
+    const TcCall t = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
+                      pl->q_per_split[m], v.r, pl->nsplit[m], 1};
+    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
     return ASI_OK;
   }
   GemmGroup g;
@@ -791,13 +754,6 @@ asi_status_t asi_plan_create(const asi_layer_desc_t* desc, asi_plan_t** out) {
 
 asi_status_t asi_plan_destroy(asi_plan_t* plan) {
   if (!plan) return ASI_ERR_INVALID_ARG;
-  if (plan->fr.ready) {
-    for (int i = 0; i < plan->nd - 1; ++i) {
-      cudaStreamDestroy(plan->fr.side[i]);
-      cudaEventDestroy(plan->fr.join[i]);
-    }
-    cudaEventDestroy(plan->fr.fork);
-  }
   delete plan;
   std::lock_guard<std::mutex> lock(g_lane_mu);
   if (--g_plans == 0) {                              // the last plan takes the side streams with it
@@ -860,9 +816,8 @@ int32_t asi_launch_count(const asi_plan_t* pl, int32_t which) {
   return which == 0 ? pl->launches_compress : pl->launches_wgrad;
 }
 
-// allow_fork: the passes of a token layer's modes may run side by side on the plan's own streams
-static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const float* U_prev, float* U_new,
-                                  float* core, void* ws, size_t ws_bytes, void* stream, bool allow_fork) {
+asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_prev, float* U_new,
+                          float* core, void* ws, size_t ws_bytes, void* stream) {
   if (!pl || !valid_ptr(act) || !valid_ptr(U_prev) || !valid_ptr(U_new) || !valid_ptr(core))
     return ASI_ERR_INVALID_ARG;
   if (U_prev == U_new) return ASI_ERR_INVALID_ARG;
@@ -876,7 +831,7 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
     SmPass1Args a;
     build_fused_pass1(pl, act, U_prev, w, &a);
     ASI_CUDA(launch_sm_pass1(a, pl->fast_S, pl->fast_R, pl->bf16, st));
-    return finish_compress(pl, act, U_new, core, w, U_prev, st);
+    return finish_compress(pl, act, U_new, core, w, U_prev, false, st);
   }
   for (int m = 0; m < pl->nd; ++m)                   // bulk and 16-byte copies; errors before anything is enqueued
     if ((pl->fiber2[m] || pl->plane2) && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
@@ -903,11 +858,23 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
     gemm_add(&gp, gemm_project(act, U_prev + pl->u_off[m], V, v.O, v.a, v.I, v.r, v.I * v.r, 1, v.r, pl->bf16));
     gemm_add(&ge, simt_expand(pl, m, act, V, w));
   }
-  const bool forked = allow_fork && fork_ready(pl);
-  if (forked) {
-    ASI_CUDA(cudaEventRecord(pl->fr.fork, st));
-    for (int i = 0; i < pl->nd - 1; ++i)
-      if (tc[i + 1]) ASI_CUDA(cudaStreamWaitEvent(pl->fr.side[i], pl->fr.fork, 0));
+  // tensor-core modes: split U_m^{prev}, then V_m = A_m^T U_m (left as the stacked operand), then P_m = A_m V_m
+  TcSplitArgs sp;
+  sp.n = 0;
+  TcCall proj[3], expd[3];
+  for (int m = 0; m < pl->nd; ++m) {
+    if (!tc[m]) continue;
+    const ModeView& v = pl->mv[m];
+    char* bu = w + pl->tcu_off[m];
+    char* bv = w + pl->tcv_off[m];
+    proj[sp.n] = {act, bu, nullptr, bv, tc_operand_ld(v.Q), v.O, v.a, v.I, 0, v.r, 1, 0};
+    expd[sp.n] = {act, bv, reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I, pl->q_per_split[m],
+                  v.r, pl->nsplit[m], 1};
+    tc_add_split(&sp, U_prev + pl->u_off[m], v.a, v.r, bu);
+  }
+  if (sp.n) {
+    sp.clear = take_clear();
+    ASI_CUDA(launch_tc_split(sp, false, st));
   }
   if (pl->plane) {
     PlaneArgs g;
@@ -959,54 +926,11 @@ static asi_status_t compress_impl(const asi_plan_t* pl, const void* act, const f
     ASI_CUDA(launch_gemm_group(gp, pl->bf16, dep, st));
     ASI_CUDA(launch_gemm_group(ge, pl->bf16, true, st));
   }
-  const cudaStream_t st0 = st;
-  for (int m = 0; m < pl->nd; ++m) {
-    if (!tc[m]) continue;
-    const ModeView& v = pl->mv[m];
-    const int slot = forked ? m : 0;                 // scratch and stream of this mode's products
-    st = (forked && m > 0) ? pl->fr.side[m - 1] : st0;
-    if (st == st0 && first) {
-      ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
-      first = false;
-    }
-    // V = A_m^T U_m^{prev}, stored [b_m x r_m]; P = A_m V
-    ModeProdArgs a;
-    a.X = act;
-    a.B = U_prev + pl->u_off[m];
-    a.Y = reinterpret_cast<float*>(w + pl->v_off[m]);
-    a.O = v.O; a.a = v.a; a.I = v.I; a.Q = v.Q;
-    a.n_out = v.r;
-    a.so = v.I * v.r;
-    a.sj = 1;
-    a.si = v.r;
-    a.tc_scratch = w + pl->off_tc + (size_t)slot * pl->tc_stride;
-    a.tc_scratch_bytes = pl->tc_bytes;
-    a.status = status;
-    ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
-    const cudaError_t e = tc_expand_mode(pl, m, act, a.Y, w, slot, st);
-    if (e == cudaErrorNotSupported) {
-      GemmGroup g;
-      g.np = 0;
-      g.clear = nullptr;
-      gemm_add(&g, simt_expand(pl, m, act, a.Y, w));
-      ASI_CUDA(launch_gemm_group(g, pl->bf16, true, st));
-    } else {
-      ASI_CUDA(e);
-    }
+  if (sp.n) {
+    ASI_CUDA(launch_tc_group(proj, sp.n, status, true, st));
+    ASI_CUDA(launch_tc_group(expd, sp.n, status, true, st));
   }
-  st = st0;
-  if (forked)
-    for (int i = 0; i < pl->nd - 1; ++i)
-      if (tc[i + 1]) {
-        ASI_CUDA(cudaEventRecord(pl->fr.join[i], pl->fr.side[i]));
-        ASI_CUDA(cudaStreamWaitEvent(st, pl->fr.join[i], 0));
-      }
-  return finish_compress(pl, act, U_new, core, w, nullptr, st);
-}
-
-asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_prev, float* U_new,
-                          float* core, void* ws, size_t ws_bytes, void* stream) {
-  return compress_impl(pl, act, U_prev, U_new, core, ws, ws_bytes, stream, true);
+  return finish_compress(pl, act, U_new, core, w, nullptr, sp.n > 0, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1156,7 +1080,7 @@ asi_status_t asi_compress_static_ws(const asi_plan_t* pl, const void* act, const
   }
   // asi_compress clears the status word and the completion counters itself; everything else in the
   // array is written before it is read.
-  return compress_impl(pl, act, U_prev, U_new, core, ws, (size_t)ASI_STATIC_WS_MAX_BYTES, stream, false);
+  return asi_compress(pl, act, U_prev, U_new, core, ws, (size_t)ASI_STATIC_WS_MAX_BYTES, stream);
 }
 
 asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float* omega, float* U_new,
@@ -1175,7 +1099,7 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
     if (s != ASI_OK) return s;
     off += pl->mv[m].Q * pl->r[m];
   }
-  return finish_compress(pl, act, U_new, core, w, nullptr, st);
+  return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
 }
 
 static size_t omega_scratch_bytes(const asi_plan* pl) {
@@ -1203,7 +1127,7 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
     s = expand_mode(pl, m, act, omega, w, st);
     if (s != ASI_OK) return s;
   }
-  return finish_compress(pl, act, U_new, core, w, nullptr, st);
+  return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
 }
 
 asi_status_t asi_gaussian_stream(uint64_t seed, uint32_t stream_id, int64_t n, float* out, void* stream) {
@@ -1282,11 +1206,14 @@ asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const flo
   a.O = B; a.a = N; a.I = Dout; a.Q = B * Dout;
   a.n_out = pl->r[m2];
   a.so = Dout * a.n_out; a.sj = 1; a.si = a.n_out;
-  a.tc_scratch = pl->lin_tc ? w + pl->off_wtc : nullptr;
-  a.tc_scratch_bytes = pl->wtc_bytes;
-  a.status = reinterpret_cast<int*>(w);
-  if (pl->lin_tc) {
-    ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
+  if (pl->lin_tc && (reinterpret_cast<uintptr_t>(dY) & 15u) == 0) {
+    TcSplitArgs sp;
+    sp.n = 0;
+    sp.clear = reinterpret_cast<int*>(w);
+    tc_add_split(&sp, a.B, N, a.n_out, w + pl->off_wtc);
+    ASI_CUDA(launch_tc_split(sp, false, st));
+    const TcCall t = {dY, w + pl->off_wtc, Y1, nullptr, 0, B, N, Dout, 0, a.n_out, 1, 0};
+    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
   } else {
     GemmGroup g;
     g.np = 0;

@@ -256,6 +256,7 @@ struct GemmTile {
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    pdl_launch_dependents();
     // the warps' shares meet in warp order
     float* red = smem;                                 // [8][32][BN]
 #pragma unroll
@@ -300,7 +301,6 @@ int bn_of(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : (n <= 32 ? 32 : 64)); }
 template <typename TX>
 __global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ GemmGroup g) {
   extern __shared__ __align__(16) float gemm_smem[];
-  pdl_launch_dependents();
   int q = 0;
   while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
   const GemmProb& p = g.p[q];

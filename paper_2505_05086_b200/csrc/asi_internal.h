@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of the ASI library.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -33,22 +34,6 @@ struct ModeProdArgs {
   int64_t O, a, I, Q;
   int n_out;
   int64_t so, sj, si;      // Y(o, j, i) = Y[o*so + j*sj + i*si]
-  void* tc_scratch = nullptr;      // device scratch for the tensor-core kernel's bf16 operand (optional)
-  size_t tc_scratch_bytes = 0;
-  int* status = nullptr;           // status word of the caller's workspace (a tensor-core wait that expires lands there)
-};
-
-// Pp[s](k, j) = sum_{q in split s} X(k, q) * V[q*r + j]
-struct ExpandArgs {
-  const void* X;
-  const float* V;
-  float* Pp;
-  int64_t O, a, I, Q;
-  int r, nsplit;
-  int64_t q_per_split;
-  void* tc_scratch = nullptr;      // device scratch for the tensor-core kernel's bf16 operand (optional)
-  size_t tc_scratch_bytes = 0;
-  int* status = nullptr;           // status word of the caller's workspace
 };
 
 // One mode's P = A_m (A_m^T U) in a single pass (k_fiber); Pp: [grid][a][r] partials.
@@ -97,6 +82,9 @@ struct QRMode {
   int* count;          // one counter, same convention
   int a, r, nsplit, nchunk;
   int rows, gs;        // rows of P per share, shares per group
+  __nv_bfloat16* bt;   // not null: U_m also as the stacked operand [3 bt_n][bt_ld] of the tensor-core products
+  int64_t bt_ld;
+  int bt_n;
 };
 struct QRArgs {
   QRMode m[ASI_MAX_MODES];
@@ -190,10 +178,34 @@ int sm_core_max_rows();
 size_t sm_wgrad_smem(const SmWgradArgs& p, int R);
 int sm_wgrad_pitch(int J);
 cudaError_t launch_sm_pass1(const SmPass1Args& p, int S, int R, bool bf16, cudaStream_t st);
-// Tensor-core last-mode product of a bf16 tensor (tcgen05); cudaErrorNotSupported when the shape does not fit.
-cudaError_t launch_tc_lastmode(const ModeProdArgs& p, void* scratch, size_t scratch_bytes, cudaStream_t st);
-size_t tc_scratch_bytes(int64_t K, int N);
-cudaError_t launch_tc_expand(const ExpandArgs& e, void* scratch, size_t scratch_bytes, cudaStream_t st);
+// Tensor-core products of bf16 tensors (asi_tc_kernels.cu).  A factor enters as its stacked operand (three bf16 terms).
+size_t tc_operand_bytes(int64_t K, int n);
+int64_t tc_operand_ld(int64_t K);
+int tc_operand_n(int n);
+int tc_kind(int64_t O, int64_t a, int64_t I, int n);
+struct TcSplitMat {
+  const float* U;          // [K][nv]
+  __nv_bfloat16* Bt;       // [3 N][ldb]
+  int64_t ldb;
+  int K, nv, N, first;
+};
+struct TcSplitArgs {
+  TcSplitMat m[3];
+  int* clear;              // not null: the first CTA zeroes the workspace's status block
+  int n;
+};
+void tc_add_split(TcSplitArgs* p, const float* U, int64_t K, int n, void* Bt);
+cudaError_t launch_tc_split(TcSplitArgs& p, bool dep, cudaStream_t st);
+struct TcCall {
+  const void* X;           // bf16 [O][a][I]
+  const void* bt;          // stacked operand of U [a][n] (projection) or of V [O I][n] (expansion)
+  float* Y;                // projection: [O][I][n]; expansion: [nsplit][a][n]
+  void* out_bt;            // projection with Y == null: the result as the stacked operand of an [O I][n] factor
+  int64_t out_ld;
+  int64_t O, a, I, q_per_split;
+  int n, nsplit, expand;
+};
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st);
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st);
 cudaError_t launch_sm_core(const SmCoreArgs& p, int S, int R, bool bf16, cudaStream_t st);
 cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t st);
@@ -242,6 +254,16 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // null) is launched normally and zeroes the workspace's status block; the others are programmatic dependents that
 // run beside their predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass
 // sees all of them finished.
+// Bt[(t N + j) ldb + k] = t-th bf16 term of v (hi, mid, lo: v = hi + mid + lo to 24 bits)
+__device__ __forceinline__ void tc_store_terms(__nv_bfloat16* Bt, int N, int64_t ldb, int j, int64_t k, float v) {
+  const __nv_bfloat16 h = __float2bfloat16_rn(v);
+  const float r1 = v - __bfloat162float(h);
+  const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+  Bt[(int64_t)j * ldb + k] = h;
+  Bt[(int64_t)(N + j) * ldb + k] = m;
+  Bt[(int64_t)(2 * N + j) * ldb + k] = __float2bfloat16_rn(r1 - __bfloat162float(m));
+}
+
 __device__ __forceinline__ void pass_begin(int* clear) {
   pdl_launch_dependents();
   if (clear && blockIdx.x == 0)
@@ -400,20 +422,9 @@ struct asi_plan {
   // compress workspace (byte offsets)
   size_t off_Pp[ASI_MAX_MODES], off_Pred[ASI_MAX_MODES], off_Gp[ASI_MAX_MODES], off_T[2];
   size_t off_Rf, off_Pg[ASI_MAX_MODES];
-  size_t off_tc, tc_bytes;         // bf16 operand of the tensor-core products (0 bytes: not used)
-  // Token layers with tensor-core modes run the passes of their modes side by side (they read the same activation
-  // and write disjoint scratch): such a mode m > 0 is enqueued on a stream of the plan's own that forks from and
-  // joins the caller's stream by events.  Each mode has its own V and operand scratch.
-  bool fork;
-  size_t v_off[ASI_MAX_MODES], tc_stride;
-  struct ForkRes {
-    cudaStream_t side[ASI_MAX_MODES - 1];
-    cudaEvent_t fork, join[ASI_MAX_MODES - 1];
-    int device;
-    bool ready, failed;
-  };
-  mutable ForkRes fr;              // created at the first forked call (under a library-wide lock)
-  int tc_mode[ASI_MAX_MODES];      // 0: SIMT, 1: last-mode tensor-core kernels, 2: inner-extent (token) kernels
+  size_t v_off[ASI_MAX_MODES];     // V_m of the modes without a one-pass kernel
+  int tc_mode[ASI_MAX_MODES];      // 0: SIMT, 1: last-mode tensor-core products, 2: inner-extent (token) products
+  size_t tcu_off[ASI_MAX_MODES], tcv_off[ASI_MAX_MODES];   // their stacked operands of U_m and V_m
   int nsplit[ASI_MAX_MODES], nchunk[ASI_MAX_MODES], qr_rows[ASI_MAX_MODES];
   int64_t q_per_split[ASI_MAX_MODES];
   int core_order[ASI_MAX_MODES];
@@ -423,7 +434,7 @@ struct asi_plan {
   size_t off_Z[3], off_Z4p;
   int conv_nsp;                    // > 1: terms 4-5 in two launches with conv_nsp partial Z4 per channel
   bool lin_tc;                     // linear backward: dY x_2 U_2^T on the tensor cores
-  size_t off_wtc, wtc_bytes;       // bf16 operand scratch of that product
+  size_t off_wtc;                  // bf16 operand scratch of that product
   bool core_tok;                   // token layer whose first core product contracts the last mode: the rest in one launch
   bool core_tail;                  // the core products after the first in one launch
   size_t off_ctp;                  // partial cores of that launch

@@ -156,7 +156,6 @@ __device__ void factor_packed(const double* Gq, double* Prow, double* W, double 
 
 __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRArgs args) {
   const QRMode M = args.m[blockIdx.y];
-  pdl_launch_dependents();
   const int c = blockIdx.x;
   if (c >= M.nchunk || M.r > kQRMaxRank) return;     // ranks above 64 take the k_qrb_* kernels
   pdl_wait();
@@ -176,28 +175,36 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
   {
     const int e0 = tid % lanes, sg = tid / lanes;
     double* part = Ps + nval;                        // [SG][nval] (SG > 1 only: nval <= 128)
-    for (int e = e0; e < nval; e += lanes) {
-      const float* src = M.Pp + base + e;
-      double acc = 0.0;
-      int s = sg;
-      for (; s + 7 * SG < M.nsplit; s += 8 * SG) {
-        float t[8];
+    constexpr int EB = 8, SB = 4;                    // elements x splits in flight per thread
+    for (int eb = e0; eb < nval; eb += EB * lanes) {
+      const float* src = M.Pp + base;
+      double acc[EB];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) t[q] = __ldcg(src + (int64_t)(s + q * SG) * sstride);
+      for (int q = 0; q < EB; ++q) acc[q] = 0.0;
+      for (int s = sg; s < M.nsplit; s += SB * SG) {
+        float t[EB][SB];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) acc += (double)t[q];
+        for (int q = 0; q < EB; ++q)
+#pragma unroll
+          for (int u = 0; u < SB; ++u) {
+            const int e = eb + q * lanes, ss = s + u * SG;
+            // always a load, from a clamped address when off: a condition next to a load makes the others wait
+            t[q][u] = __ldcg(src + (int64_t)(ss < M.nsplit ? ss : s) * sstride + (e < nval ? e : 0));
+          }
+#pragma unroll
+        for (int q = 0; q < EB; ++q)
+#pragma unroll
+          for (int u = 0; u < SB; ++u) acc[q] += (s + u * SG < M.nsplit) ? (double)t[q][u] : 0.0;
       }
-      if (s < M.nsplit) {
-        float t[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) t[q] = __ldcg(src + (int64_t)(s + q * SG < M.nsplit ? s + q * SG : s) * sstride);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) acc += (s + q * SG < M.nsplit) ? (double)t[q] : 0.0;
-      }
-      if (SG > 1) part[sg * nval + e] = acc;
-      else {
-        Ps[e] = acc;
-        M.Pred[base + e] = acc;
+      for (int q = 0; q < EB; ++q) {
+        const int e = eb + q * lanes;
+        if (e >= nval) break;
+        if (SG > 1) part[sg * nval + e] = acc[q];
+        else {
+          Ps[e] = acc[q];
+          M.Pred[base + e] = acc[q];
+        }
       }
     }
     if (SG > 1) {
@@ -271,7 +278,7 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  constexpr int EB = 3;
+  constexpr int EB = 5;
   double v[EB];
   if (ngroups > 1) {
     for (int e0 = tid; e0 < len; e0 += EB * kOT) {
@@ -319,7 +326,6 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
 // CTA (c, m): 32 rows of U_m; thread (ti, tj) owns rows ti, ti + 16 and columns tj, tj + 16, ..
 __global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRArgs args) {
   const QRMode M = args.m[blockIdx.y];
-  pdl_launch_dependents();
   const int row0 = blockIdx.x * 32;
   if (row0 >= M.a || M.r > kQRMaxRank) return;
   pdl_wait();
@@ -331,13 +337,23 @@ __global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRAr
   const int nrows = min(32, M.a - row0);
   const int nb = (r + 3) >> 2;
   const double* Yg = M.Gp + (int64_t)(M.nchunk + (M.nchunk + M.gs - 1) / M.gs) * (nb * (nb + 1) * 8);
-#pragma unroll 4
-  for (int e = tid; e < rr; e += kOT) {
-    const int j = e / r, i = e - j * r;
-    Ys[j * PY + i] = __ldcg(Yg + e);
+  // eight loads of P and eight of Y in flight per round
+  for (int e0 = tid; e0 < rr; e0 += 8 * kOT) {
+    double t[8], q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + u * kOT;
+      t[u] = __ldcg(Yg + (e < rr ? e : 0));
+      q[u] = __ldcg(M.Pred + (int64_t)row0 * r + (e < nrows * r ? e : 0));
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + u * kOT;
+      if (e < rr) Ys[e / r * PY + e % r] = t[u];
+      if (e < 32 * r) Ps[e] = (e < nrows * r) ? q[u] : 0.0;
+    }
   }
-#pragma unroll 4
-  for (int e = tid; e < 32 * r; e += kOT) Ps[e] = (e < nrows * r) ? __ldcg(M.Pred + (int64_t)row0 * r + e) : 0.0;
+  for (int e = rr + tid; e < 32 * r; e += kOT) Ps[e] = (e < nrows * r) ? __ldcg(M.Pred + (int64_t)row0 * r + e) : 0.0;
   __syncthreads();
   const int ti = tid >> 4, tj = tid & 15;
 #pragma unroll 1
@@ -345,6 +361,7 @@ __global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRAr
     const double* y = Ys + j * PY;
     double s0 = 0.0, s1 = 0.0, t0 = 0.0, t1 = 0.0;
     int i = 0;
+#pragma unroll 4
     for (; i + 1 <= j; i += 2) {
       s0 = fma(Ps[ti * r + i], y[i], s0);
       t0 = fma(Ps[ti * r + i + 1], y[i + 1], t0);
@@ -355,8 +372,15 @@ __global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRAr
       s0 = fma(Ps[ti * r + i], y[i], s0);
       s1 = fma(Ps[(ti + 16) * r + i], y[i], s1);
     }
-    if (row0 + ti < M.a) M.Uout[(int64_t)(row0 + ti) * r + j] = (float)(s0 + t0);
-    if (row0 + ti + 16 < M.a) M.Uout[(int64_t)(row0 + ti + 16) * r + j] = (float)(s1 + t1);
+    const float u0 = (float)(s0 + t0), u1 = (float)(s1 + t1);
+    if (row0 + ti < M.a) {
+      M.Uout[(int64_t)(row0 + ti) * r + j] = u0;
+      if (M.bt) tc_store_terms(M.bt, M.bt_n, M.bt_ld, j, row0 + ti, u0);
+    }
+    if (row0 + ti + 16 < M.a) {
+      M.Uout[(int64_t)(row0 + ti + 16) * r + j] = u1;
+      if (M.bt) tc_store_terms(M.bt, M.bt_n, M.bt_ld, j, row0 + ti + 16, u1);
+    }
   }
 }
 
@@ -400,9 +424,9 @@ int orth_rows(int64_t a, int r, int64_t nsplit) {
   while (rows < kOrthMaxRows && (a + rows - 1) / rows > 1024) rows *= 2;
   return rows;
 }
-// shares per group: at least 8, at most kOrthGroups groups per mode (their counters sit in the status block)
+// shares per group: one group up to 16 shares, else 8 each, at most kOrthGroups groups per mode (their counters sit in the status block)
 int orth_group(int64_t nchunk) {
-  int gs = 8;
+  int gs = nchunk <= 16 ? 16 : 8;
   while ((nchunk + gs - 1) / gs > kOrthGroups) gs *= 2;
   return gs;
 }

@@ -1,29 +1,36 @@
 // Tensor-core kernels (sm_100a: tcgen05.mma, TMEM accumulator, TMA operand staging) for the steps of the
 // path that are plain dense contractions: products of a bf16 tensor with a wide fp32 factor (16..64
 // columns) in Algorithm 1 on token layers (B x N x D activations),
-//   k_tc_lastmode      Y[q][j]     = sum_k X[q][k] U[k][j]          V_3 = A_(3)^T U_3, first core product
-//   k_tc_expand        P[k][j]     = sum_q X[q][k] V[q][j]          P_3 = A_(3) V_3 (split-K partials)
-//   k_tc_token         V[o][i][j]  = sum_k X[o][k][i] U[k][j]       V_2 = A_(2)^T U_2, one sample o per CTA row
-//   k_tc_token_expand  P[k][j]     = sum_{o,i} X[o][k][i] V[o][i][j]  P_2 = A_(2) V_2 (split-K partials)
+//   kTcLast         Y[q][j]     = sum_k X[q][k] U[k][j]          V_3 = A_(3)^T U_3, first core product
+//   kTcLastExpand   P[k][j]     = sum_q X[q][k] V[q][j]          P_3 = A_(3) V_3 (split-K partials)
+//   kTcToken        V[o][i][j]  = sum_k X[o][k][i] U[k][j]       V_2 = A_(2)^T U_2, dY x_2 U_2^T
+//   kTcTokenExpand  P[k][j]     = sum_{o,i} X[o][k][i] V[o][i][j]  P_2 = A_(2) V_2 (split-K partials)
 // X is exact in bf16; the fp32 factor (U or V) is split into three bf16 terms (24 mantissa bits), so one
 // MMA of width 3 n per k-step (the three terms stacked as operand rows) yields three partial products in
 // TMEM whose sum reproduces the fp32 product to fp32 rounding.
 //
-// k_tc_split writes the stacked operand [3 n][K] (bf16, K contiguous: hi rows, then mid, then lo) to
-// scratch memory once per product; the GEMM kernel then streams both operands by TMA.  One CTA owns a
-// 128-row tile of Y and walks K in chunks of 64, its warps in three roles that meet only through mbarriers:
-//   * a producer thread keeps four stages in flight, each the X tile [128 x 64] and the operand tile
+// The stacked operand [3 n][K] (bf16, K contiguous: hi rows, then mid, then lo) of a factor U is written by
+// k_tc_split (one launch for all factors of a call; k_orth_apply writes that of a new factor itself); that of
+// V_m is written by the projection's own epilogue, so V_m exists only in the form its expansion reads.
+//
+// k_tc_group runs up to three products in one launch (a CTA finds its product in a table).  One CTA owns a
+// 128-row tile of Y and a share of K in chunks of 64, its warps in three roles that meet only through mbarriers:
+//   * a producer thread keeps the stages full, each the X tile [128 x 64] and the operand tile
 //     [3 n x 64] (cp.async.bulk.tensor, 128-byte swizzle);
 //   * an issuer thread launches 4 k-steps of tcgen05.mma (M = 128, N = 3 n, K = 16) per chunk and commits
 //     them to the mbarrier that frees the stage;
-//   * eight warps then read the three accumulator groups with tcgen05.ld (lane = row), add them and store
-//     fp32 rows.
+//   * eight warps then read the three accumulator groups with tcgen05.ld (lane = row) and add them.
+// A launch uses clusters of 1, 2 or 4 CTAs: the CTAs of a cluster share one tile of a product whose contraction
+// is long (each takes a quarter of K, the partial tiles meet in distributed shared memory in rank order) or own
+// different tiles.  Stage count and TMEM columns follow n so that two CTAs share an SM: what bounds these products
+// is latency -- few tiles, a prologue and an epilogue per tile, bytes in flight -- not the tensor pipe.
 // Every wait has a time limit; on expiry the kernel records ASI_ERR_TIMEOUT in the workspace's status word,
 // frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -37,10 +44,9 @@ constexpr int kTcWorkers = 8;       // epilogue warps
 constexpr int kTcThreads = (kTcWorkers + 2) * 32;   // + the MMA issuer warp and the TMA producer warp
 constexpr int kTcM = 128;          // rows of Y per CTA (= TMEM lanes)
 constexpr int kTcKC = 64;          // k per chunk: 64 bf16 = one 128-byte swizzle row
-constexpr int kTcStages = 4;       // X stages in flight
+constexpr int kTcMaxStages = 4;
 constexpr int kTcNMax = 64;
 constexpr uint32_t kTileA = kTcM * kTcKC * 2;       // 16 KB
-constexpr uint32_t kTileB = 3 * kTcNMax * kTcKC * 2;   // 24 KB: the three terms stacked
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -129,39 +135,35 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {   /
                : "r"(taddr)
                : "memory");
 }
-struct TcArgs {
-  float* Y;            // [M][ldy]; CTA (., s) writes Y + s * y_split
-  int M, N, K, ldy;    // K: total extent of the contraction
-  int k_per_split;     // multiple of 64; CTA (., s) contracts [s * k_per_split, min(K, (s + 1) * k_per_split))
-  int64_t y_split;
-  int inner;           // kTcTokenExpand: K enumerates (o, i) with i < inner (a multiple of 64)
-  int* status;         // status word of the caller's workspace (may be null): ASI_ERR_TIMEOUT when a wait expires
-  int nv;              // columns of Y that exist (a multiple of 4, N - 15 <= nv <= N): the factor is zero-padded to N
-};
-
-// Bt[(t*n + j) * ldb + k] = t-th bf16 term of U[k][j] (hi, mid, lo: U = hi + mid + lo to 24 bits)
-__global__ void __launch_bounds__(256) k_tc_split(const float* __restrict__ U, int ldu, int K, int N, int nv,
-                                                  __nv_bfloat16* __restrict__ Bt, int64_t ldb) {
+// Bt[(t*n + j) * ldb + k] = t-th bf16 term of U[k][j] (hi, mid, lo: U = hi + mid + lo to 24 bits), for every factor
+// of the call in one launch
+__global__ void __launch_bounds__(256) k_tc_split(const __grid_constant__ TcSplitArgs p) {
   __shared__ float tile[32][33];
-  const int k0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (p.clear && blockIdx.x == 0) p.clear[threadIdx.x] = 0;
+  int q = 0;
+  while (q + 1 < p.n && (int)blockIdx.x >= p.m[q + 1].first) ++q;
+  const TcSplitMat& m = p.m[q];
+  const int t = (int)blockIdx.x - m.first, nk = (m.K + 31) / 32;
+  const int k0 = (t % nk) * 32, j0 = (t / nk) * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8) {
-    const int k = k0 + r, j = j0 + tx;
-    tile[r][tx] = (k < K && j < nv) ? U[(int64_t)k * ldu + j] : 0.f;     // columns nv..N-1 of the operand are zero
+  float v[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int k = k0 + ty + 8 * r, j = j0 + tx;
+    v[r] = __ldg(m.U + ((k < m.K && j < m.nv) ? (int64_t)k * m.nv + j : 0));
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int k = k0 + ty + 8 * r, j = j0 + tx;
+    tile[ty + 8 * r][tx] = (k < m.K && j < m.nv) ? v[r] : 0.f;           // columns nv..N-1 of the operand are zero
   }
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int j = j0 + r, k = k0 + tx;
-    if (j < N && k < K) {
-      const float u = tile[tx][r];
-      const __nv_bfloat16 h = __float2bfloat16_rn(u);
-      const float r1 = u - __bfloat162float(h);
-      const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-      const __nv_bfloat16 l = __float2bfloat16_rn(r1 - __bfloat162float(m));
-      Bt[(int64_t)j * ldb + k] = h;
-      Bt[(int64_t)(N + j) * ldb + k] = m;
-      Bt[(int64_t)(2 * N + j) * ldb + k] = l;
-    }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int j = j0 + ty + 8 * r, k = k0 + tx;
+    if (j < m.N && k < m.K) tc_store_terms(m.Bt, m.N, m.ldb, j, k, tile[tx][ty + 8 * r]);
   }
 }
 
@@ -173,35 +175,98 @@ __global__ void __launch_bounds__(256) k_tc_split(const float* __restrict__ U, i
 // Rows of a box that fall outside the tensor are zero-filled by TMA.
 enum TcMode { kTcLast = 0, kTcLastExpand = 1, kTcToken = 2, kTcTokenExpand = 3 };
 
-template <int MODE>
-__device__ __forceinline__ void tc_gemm_body(const CUtensorMap& mapX, const CUtensorMap& mapB, const TcArgs& p) {
+struct TcProb {
+  CUtensorMap mapX, mapB;
+  float* Y;            // fp32 result [M][ldy] of outer index / split s at Y + s * y_split (null: Bt instead)
+  __nv_bfloat16* Bt;   // the result as a stacked operand: row m of outer index o is k = o * M + m
+  int64_t y_split, ldb;
+  int mode, M, N, nv, K, ldy;
+  int k_per_split;     // multiple of 64; second tile index s contracts [s * k_per_split, min(K, (s + 1) * k_per_split))
+  int inner;           // kTcTokenExpand: K enumerates (o, i) with i < inner (a multiple of 64)
+  int mt;              // 128-row tiles
+  int ksp;             // CTAs that share a tile (1 or the cluster size)
+  int first;           // first CTA of the product in the launch (a multiple of the cluster size)
+  int n_cta;
+};
+struct TcGroup {
+  TcProb p[3];
+  int* status;         // status word of the caller's workspace (may be null): ASI_ERR_TIMEOUT when a wait expires
+  int np, nst, tmem_cols, cs;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t local_addr, uint32_t rank) {
+  uint32_t ra;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(ra)
+               : "memory");
+  return v;
+}
+
+// four columns col.. of result row m (outer index or split s)
+__device__ __forceinline__ void tc_store4(const TcProb& p, int s, int m, int col, float4 v) {
+  if (m >= p.M || col >= p.N) return;
+  if (p.Y) {
+    if (col < p.nv) *reinterpret_cast<float4*>(p.Y + (int64_t)s * p.y_split + (int64_t)m * p.ldy + col) = v;
+  } else {
+    const int64_t k = (int64_t)s * p.M + m;          // columns nv.. are exact zeros (their factor columns are)
+    tc_store_terms(p.Bt, p.N, p.ldb, col, k, v.x);
+    tc_store_terms(p.Bt, p.N, p.ldb, col + 1, k, v.y);
+    tc_store_terms(p.Bt, p.N, p.ldb, col + 2, k, v.z);
+    tc_store_terms(p.Bt, p.N, p.ldb, col + 3, k, v.w);
+  }
+}
+
+__global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constant__ TcGroup g) {
   extern __shared__ __align__(1024) uint8_t tc_smem[];
-  // carve-up: per stage the X tile and the operand tile, then barriers
+  int q = 0;
+  while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
+  const TcProb& p = g.p[q];
+  const int nst = g.nst, N = p.N;
+  const uint32_t tile_b = (uint32_t)(3 * N) * 128u;     // operand tile: 3 N rows of 64 bf16
+  const uint32_t stage = kTileA + tile_b;               // 1024-byte multiples: N is a multiple of 16
+  // carve-up: stages, then barriers
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem) + 1023) & ~(uintptr_t)1023);
-  uint8_t* As = base;                                   // [stages][16 KB]
-  uint8_t* Bs = As + kTcStages * kTileA;                // [stages][24 KB]
-  uint64_t* full = reinterpret_cast<uint64_t*>(Bs + kTcStages * kTileB);   // [stages] both tiles landed
-  uint64_t* s_free = full + kTcStages;                  // [stages] the MMAs that read the stage are done
-  uint64_t* done = s_free + kTcStages;                  // all MMAs of the tile are done
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[1];
+  __shared__ uint32_t tmem_slot[1];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr bool A_MN = (MODE == kTcLastExpand || MODE == kTcToken);
-  const int row0 = blockIdx.x * kTcM;
-  const int k_begin = (MODE == kTcToken) ? 0 : blockIdx.y * p.k_per_split;
-  const int k_end = (MODE == kTcToken || p.K - k_begin < p.k_per_split) ? p.K : k_begin + p.k_per_split;
-  const int nchunk = (k_end - k_begin + kTcKC - 1) / kTcKC;   // a ragged last chunk is zero-filled by TMA
-  const int N = p.N;
-  float* Yout = p.Y + (int64_t)blockIdx.y * p.y_split;
+  const bool a_mn = p.mode == kTcLastExpand || p.mode == kTcToken;
+  const int cta = (int)blockIdx.x - p.first;
+  const bool live = cta < p.n_cta;                      // padding CTAs of the last cluster only take the barriers
+  const int rank = p.ksp > 1 ? (int)cluster_rank() : 0;
+  const int tile = live ? cta / p.ksp : 0;
+  const int row0 = (tile % p.mt) * kTcM, s = tile / p.mt;   // s: outer index (kTcToken) or split of K
+  int k_begin = p.mode == kTcToken ? 0 : s * p.k_per_split;
+  int k_end = (p.mode == kTcToken || p.K - k_begin < p.k_per_split) ? p.K : k_begin + p.k_per_split;
+  if (k_end < k_begin) k_end = k_begin;
+  int nchunk = (k_end - k_begin + kTcKC - 1) / kTcKC;   // a ragged last chunk is zero-filled by TMA
+  if (p.ksp > 1) {
+    const int per = (nchunk + p.ksp - 1) / p.ksp;
+    k_begin += rank * per * kTcKC;
+    nchunk = nchunk - rank * per < per ? nchunk - rank * per : per;
+    if (nchunk < 0) nchunk = 0;
+  }
+  if (!live) nchunk = 0;
 
   if (tid == 0) {
-    for (int s = 0; s < kTcStages; ++s) { mbar_init(full + s, 1); mbar_init(s_free + s, 1); }
+    for (int i = 0; i < nst; ++i) { mbar_init(full + i, 1); mbar_init(s_free + i, 1); }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {                                      // TMEM: 256 fp32 columns x 128 lanes (3 N are used)
+  if (warp == 0) {                                      // TMEM: fp32 columns x 128 lanes (3 N are used)
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(256)
+                 "r"(g.tmem_cols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -209,112 +274,130 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& mapX, const CUte
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_d = *tmem_slot;
+  pdl_wait();
 
   // The three bf16 terms of the factor are stacked along the operand's rows: one MMA of width 3 N per
   // k-step reads the X tile once and leaves the three partial products in three column groups of TMEM.
-  const uint32_t idesc = instr_desc_bf16(kTcM, 3 * N, A_MN);
-  const uint32_t b_bytes = (uint32_t)(3 * N) * 128u;    // operand tile: 3 N rows of 64 bf16
   bool ok = true;                                       // this thread's waits so far
-  if (warp == kTcWorkers) {
-    // ---- MMA issuer (one thread): 4 k-steps per chunk, then the commit that frees the stage
-    if (lane == 0) {
-      const uint32_t a_base = smem_u32(As), b_base = smem_u32(Bs);
+  if (nchunk > 0) {
+    if (warp == kTcWorkers) {
+      // ---- MMA issuer (one thread): 4 k-steps per chunk, then the commit that frees the stage
+      if (lane == 0) {
+        const uint32_t idesc = instr_desc_bf16(kTcM, 3 * N, a_mn);
+        const uint32_t a_base = smem_u32(base);
+        const uint64_t a_step = a_mn ? 128 : 2;         // a k-step is 16 bf16: 32 bytes inside the swizzle row of a
+        int st = 0;                                     // K-major tile, 16 rows (2048 bytes) of an MN-major tile
+        uint32_t ph = 0;                                // (start-address field in 16-byte units)
 #pragma unroll 1
-      for (int c = 0; c < nchunk && ok; ++c) {
-        const int s = c % kTcStages;
-        ok = mbar_wait(full + s, (c / kTcStages) & 1);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // a k-step is 16 bf16: 32 bytes inside the swizzle row of a K-major tile, 16 rows (2048 bytes) of
-        // an MN-major tile (start-address field in 16-byte units)
-        const uint64_t da0 = smem_desc_sw128(a_base + s * kTileA, A_MN ? kTileA / 2 : 16);
-        const uint64_t db0 = smem_desc_sw128(b_base + s * kTileB);
+        for (int c = 0; c < nchunk && ok; ++c) {
+          ok = mbar_wait(full + st, ph);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da0 = smem_desc_sw128(a_base + st * stage, a_mn ? kTileA / 2 : 16);
+          const uint64_t db0 = smem_desc_sw128(a_base + st * stage + kTileA);
 #pragma unroll
-        for (int ks = 0; ks < kTcKC / 16; ++ks)
-          umma_bf16(tmem_d, da0 + (uint64_t)(ks * (A_MN ? 128 : 2)), db0 + (uint64_t)(ks * 2), idesc,
-                    (c | ks) ? 1u : 0u);
-        umma_commit(s_free + s);
-      }
-      umma_commit(done);
-    }
-  } else if (warp == kTcWorkers + 1) {
-    // ---- TMA producer (one thread): keeps kTcStages stages in flight
-    if (lane == 0) {
-#pragma unroll 1
-      for (int c = 0; c < nchunk && ok; ++c) {
-        const int s = c % kTcStages;
-        if (c >= kTcStages) ok = mbar_wait(s_free + s, ((c / kTcStages) - 1) & 1);
-        if (!ok) break;
-        mbar_expect_tx(full + s, kTileA + b_bytes);
-        const int kc = k_begin + c * kTcKC;
-        if (MODE == kTcLastExpand) {
-          tma_load_2d(As + s * kTileA, &mapX, row0, kc, full + s);
-          tma_load_2d(As + s * kTileA + kTileA / 2, &mapX, row0 + 64, kc, full + s);
-        } else if (MODE == kTcToken) {
-          tma_load_3d(As + s * kTileA, &mapX, row0, kc, blockIdx.y, full + s);
-          tma_load_3d(As + s * kTileA + kTileA / 2, &mapX, row0 + 64, kc, blockIdx.y, full + s);
-        } else if (MODE == kTcTokenExpand) {
-          const int o = kc / p.inner;
-          tma_load_3d(As + s * kTileA, &mapX, kc - o * p.inner, row0, o, full + s);
-        } else {
-          tma_load_2d(As + s * kTileA, &mapX, kc, row0, full + s);
+          for (int ks = 0; ks < kTcKC / 16; ++ks)
+            umma_bf16(tmem_d, da0 + (uint64_t)ks * a_step, db0 + (uint64_t)(ks * 2), idesc, (c | ks) ? 1u : 0u);
+          umma_commit(s_free + st);
+          if (++st == nst) { st = 0; ph ^= 1u; }
         }
-        tma_load_2d(Bs + s * kTileB, &mapB, kc, 0, full + s);
+        umma_commit(done);
       }
+    } else if (warp == kTcWorkers + 1) {
+      // ---- TMA producer (one thread): keeps the stages full
+      if (lane == 0) {
+        int st = 0;
+        uint32_t ph = 1;
+#pragma unroll 1
+        for (int c = 0; c < nchunk && ok; ++c) {
+          if (c >= nst) ok = mbar_wait(s_free + st, ph);
+          if (!ok) break;
+          uint8_t* As = base + st * stage;
+          mbar_expect_tx(full + st, stage);
+          const int kc = k_begin + c * kTcKC;
+          if (p.mode == kTcLastExpand) {
+            tma_load_2d(As, &p.mapX, row0, kc, full + st);
+            tma_load_2d(As + kTileA / 2, &p.mapX, row0 + 64, kc, full + st);
+          } else if (p.mode == kTcToken) {
+            tma_load_3d(As, &p.mapX, row0, kc, s, full + st);
+            tma_load_3d(As + kTileA / 2, &p.mapX, row0 + 64, kc, s, full + st);
+          } else if (p.mode == kTcTokenExpand) {
+            const int o = kc / p.inner;
+            tma_load_3d(As, &p.mapX, kc - o * p.inner, row0, o, full + st);
+          } else {
+            tma_load_2d(As, &p.mapX, kc, row0, full + st);
+          }
+          tma_load_2d(As + kTileA, &p.mapB, kc, 0, full + st);
+          if (++st == nst) { st = 0; ph ^= 1u; }
+        }
+      }
+    } else {
+      ok = mbar_wait(done, 0);                          // every reader of TMEM observes the completed phase
     }
-  } else {
-    ok = mbar_wait(done, 0);                            // every reader of TMEM observes the completed phase
   }
   const bool fail = __syncthreads_or(ok ? 0 : 1) != 0;
-  if (!fail) {
-    if (warp < kTcWorkers) {
-      // thread = row: warp w reads lanes 32 (w % 4) ..., warps 0-3 the columns [0, N/2), warps 4-7 the rest
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int half = N >> 1;                          // 8, 16, 24 or 32 columns per warp
-      const int col0 = (warp >> 2) * half;
-      const int row = row0 + (warp & 3) * 32 + lane;
-      const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-      for (int cc = 0; cc < half; cc += 8) {
+  pdl_launch_dependents();
+  const int PN = N + 4;                                 // pitch of the exchanged tile: rows four banks apart
+  float* xch = reinterpret_cast<float*>(base);          // [128][PN] (the stages are free now)
+  if (!fail && warp < kTcWorkers && live) {
+    // thread = row: warp w reads lanes 32 (w % 4) ..., warps 0-3 the columns [0, N/2), warps 4-7 the rest
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int half = N >> 1;                            // 8, 16, 24 or 32 columns per warp
+    const int col0 = (warp >> 2) * half;
+    const int r = (warp & 3) * 32 + lane;
+    const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
+    for (int cc = 0; cc < half; cc += 8) {
+      float o[8];
+      if (nchunk > 0) {
         uint32_t h[8], m[8], l[8];
         tmem_ld8(taddr + (uint32_t)cc, h);
         tmem_ld8(taddr + (uint32_t)(N + cc), m);
         tmem_ld8(taddr + (uint32_t)(2 * N + cc), l);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (row < p.M) {
-          float o[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i)                   // small terms first
-            o[i] = (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
-          float* y = Yout + (int64_t)row * p.ldy + col0 + cc;
-          if (col0 + cc < p.nv) *reinterpret_cast<float4*>(y) = make_float4(o[0], o[1], o[2], o[3]);
-          if (col0 + cc + 4 < p.nv) *reinterpret_cast<float4*>(y + 4) = make_float4(o[4], o[5], o[6], o[7]);
-        }
+        for (int i = 0; i < 8; ++i)                     // small terms first
+          o[i] = (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i] = 0.f;         // an empty share of K
+      }
+      const float4 v0 = make_float4(o[0], o[1], o[2], o[3]), v1 = make_float4(o[4], o[5], o[6], o[7]);
+      if (p.ksp > 1) {
+        *reinterpret_cast<float4*>(xch + r * PN + col0 + cc) = v0;
+        *reinterpret_cast<float4*>(xch + r * PN + col0 + cc + 4) = v1;
+      } else {
+        tc_store4(p, s, row0 + r, col0 + cc, v0);
+        tc_store4(p, s, row0 + r, col0 + cc + 4, v1);
       }
     }
-  } else if (tid == 0 && p.status) {
-    atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
   }
+  if (fail && tid == 0 && g.status) atomicMax(g.status, (int)ASI_ERR_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(256) : "memory");
-}
-
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_lastmode(const __grid_constant__ CUtensorMap mapX,
-                                                                const __grid_constant__ CUtensorMap mapB, TcArgs p) {
-  tc_gemm_body<kTcLast>(mapX, mapB, p);
-}
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_expand(const __grid_constant__ CUtensorMap mapX,
-                                                              const __grid_constant__ CUtensorMap mapB, TcArgs p) {
-  tc_gemm_body<kTcLastExpand>(mapX, mapB, p);
-}
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_token(const __grid_constant__ CUtensorMap mapX,
-                                                             const __grid_constant__ CUtensorMap mapB, TcArgs p) {
-  tc_gemm_body<kTcToken>(mapX, mapB, p);
-}
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_token_expand(const __grid_constant__ CUtensorMap mapX,
-                                                                    const __grid_constant__ CUtensorMap mapB, TcArgs p) {
-  tc_gemm_body<kTcTokenExpand>(mapX, mapB, p);
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(g.tmem_cols) : "memory");
+  if (g.cs > 1) {
+    // the shares of a tile meet: CTA `rank` adds the rows [rank * 128 / ksp, ..) in rank order
+    cluster_sync_all();
+    if (p.ksp > 1 && live && !fail) {
+      const int rows = kTcM / p.ksp, r0 = rank * rows;
+      const int items = rows * (N / 4);
+      const uint32_t xa = smem_u32(xch);
+      for (int e = tid; e < items; e += kTcThreads) {
+        const int r = r0 + e % rows, c4 = e / rows;     // lanes = neighbouring rows: coalesced operand stores
+        const uint32_t a = xa + (uint32_t)(r * PN + 4 * c4) * 4u;
+        float4 v[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[t] = ld_cluster4(a, (uint32_t)(t < p.ksp ? t : 0));
+        float4 sum = v[0];
+#pragma unroll
+        for (int t = 1; t < 4; ++t)
+          if (t < p.ksp) { sum.x += v[t].x; sum.y += v[t].y; sum.z += v[t].z; sum.w += v[t].w; }
+        tc_store4(p, s, row0 + r, 4 * c4, sum);
+      }
+    }
+    cluster_sync_all();                                 // no CTA leaves while its tile is being read
+  }
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -334,12 +417,6 @@ EncodeFn encode_fn() {
   return fn;
 }
 
-}  // namespace
-
-size_t tc_scratch_bytes(int64_t K, int N) { return (size_t)3 * ((N + 15) / 16 * 16) * ((K + 63) / 64 * 64) * 2; }
-
-namespace {
-constexpr size_t kTcSmem = 1024 + kTcStages * (kTileA + kTileB) + (2 * kTcStages + 1) * 8 + 16;
 
 bool encode_bf16_map(CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                      const cuuint32_t* box) {
@@ -351,161 +428,153 @@ bool encode_bf16_map(CUtensorMap* map, const void* base, int rank, const cuuint6
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// V[o][i][j] = sum_k X[o][k][i] U[k][j]: a middle mode of a bf16 token tensor (I = inner extent, a multiple of 64)
-cudaError_t launch_tc_token(const ModeProdArgs& p, void* scratch, size_t scratch_bytes, cudaStream_t st) {
-  const int nv = p.n_out, N = (nv + 15) / 16 * 16;       // the factor is zero-padded to a multiple of 16 columns
-  const int64_t Kp = (p.a + 63) / 64 * 64;
-  if (p.I < 64 || p.I % 64 != 0 || p.O < 1 || p.O >= 65536 || nv % 4 != 0 || nv < 16 || N > kTcNMax || p.a < 1 ||
-      p.a >= (1ll << 31) || p.I >= (1ll << 31) || p.sj != 1 || p.si != nv || p.so != p.I * nv ||
-      !scratch || scratch_bytes < tc_scratch_bytes(p.a, N) || (reinterpret_cast<uintptr_t>(scratch) & 15u) ||
-      (reinterpret_cast<uintptr_t>(p.X) & 15u) || (reinterpret_cast<uintptr_t>(p.Y) & 15u))
-    return cudaErrorNotSupported;
-  CUtensorMap mapX, mapB;
-  {
-    const cuuint64_t dims[3] = {(cuuint64_t)p.I, (cuuint64_t)p.a, (cuuint64_t)p.O};
-    const cuuint64_t strides[2] = {(cuuint64_t)p.I * 2, (cuuint64_t)p.a * p.I * 2};
-    const cuuint32_t box[3] = {64, 64, 1};
-    if (!encode_bf16_map(&mapX, p.X, 3, dims, strides, box)) return cudaErrorNotSupported;
-  }
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)p.a, (cuuint64_t)(3 * N)};
-    const cuuint64_t strides[1] = {(cuuint64_t)Kp * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)(3 * N)};
-    if (!encode_bf16_map(&mapB, scratch, 2, dims, strides, box)) return cudaErrorNotSupported;
-  }
-  const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_token), kTcSmem);
-  if (attr_err != cudaSuccess) return attr_err;
-  k_tc_split<<<dim3((unsigned)((p.a + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      p.B, nv, (int)p.a, N, nv, static_cast<__nv_bfloat16*>(scratch), Kp);
-  TcArgs a = {p.Y, (int)p.I, N, (int)p.a, nv, (int)Kp, p.so, 0, p.status, nv};
-  dim3 grid((unsigned)((p.I + kTcM - 1) / kTcM), (unsigned)p.O);
-  k_tc_token<<<grid, kTcThreads, kTcSmem, st>>>(mapX, mapB, a);
-  return cudaGetLastError();
-}
+int pad16(int n) { return (n + 15) / 16 * 16; }
+int64_t pad64(int64_t k) { return (k + 63) / 64 * 64; }
 
-// Pp[s][k][j] = sum_{(o,i) in split s} X[o][k][i] V[o][i][j]: the expansion of a middle mode
-cudaError_t launch_tc_token_expand(const ExpandArgs& e, void* scratch, size_t scratch_bytes, cudaStream_t st) {
-  const int nv = e.r, N = (nv + 15) / 16 * 16;
-  const int64_t Q = e.Q;
-  if (e.I < 64 || e.I % 64 != 0 || e.O < 1 || e.O >= 65536 || nv % 4 != 0 || nv < 16 || N > kTcNMax || e.a < 1 ||
-      e.a >= (1ll << 31) || Q >= (1ll << 31) || e.q_per_split % kTcKC != 0 || e.q_per_split >= (1ll << 31) ||
-      e.nsplit < 1 || !scratch || scratch_bytes < tc_scratch_bytes(Q, N) ||
-      (reinterpret_cast<uintptr_t>(scratch) & 15u) || (reinterpret_cast<uintptr_t>(e.X) & 15u) ||
-      (reinterpret_cast<uintptr_t>(e.Pp) & 15u))
-    return cudaErrorNotSupported;
-  CUtensorMap mapX, mapB;
-  {
-    const cuuint64_t dims[3] = {(cuuint64_t)e.I, (cuuint64_t)e.a, (cuuint64_t)e.O};
-    const cuuint64_t strides[2] = {(cuuint64_t)e.I * 2, (cuuint64_t)e.a * e.I * 2};
-    const cuuint32_t box[3] = {64, (cuuint32_t)kTcM, 1};
-    if (!encode_bf16_map(&mapX, e.X, 3, dims, strides, box)) return cudaErrorNotSupported;
-  }
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)Q, (cuuint64_t)(3 * N)};
-    const cuuint64_t strides[1] = {(cuuint64_t)Q * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)(3 * N)};
-    if (!encode_bf16_map(&mapB, scratch, 2, dims, strides, box)) return cudaErrorNotSupported;
-  }
-  const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_token_expand), kTcSmem);
-  if (attr_err != cudaSuccess) return attr_err;
-  k_tc_split<<<dim3((unsigned)((Q + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      e.V, nv, (int)Q, N, nv, static_cast<__nv_bfloat16*>(scratch), Q);
-  TcArgs a = {e.Pp, (int)e.a, N, (int)Q, nv, (int)e.q_per_split, e.a * nv, (int)e.I, e.status, nv};
-  dim3 grid((unsigned)((e.a + kTcM - 1) / kTcM), (unsigned)e.nsplit);
-  k_tc_token_expand<<<grid, kTcThreads, kTcSmem, st>>>(mapX, mapB, a);
-  return cudaGetLastError();
+bool operand_map(CUtensorMap* map, const __nv_bfloat16* Bt, int64_t K, int N) {
+  const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)(3 * N)};
+  const cuuint64_t strides[1] = {(cuuint64_t)pad64(K) * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)(3 * N)};
+  return encode_bf16_map(map, Bt, 2, dims, strides, box);
 }
 }  // namespace
 
+// bytes of the stacked operand of a [K x n] factor
+size_t tc_operand_bytes(int64_t K, int n) { return (size_t)3 * pad16(n) * pad64(K) * 2; }
+int64_t tc_operand_ld(int64_t K) { return pad64(K); }
+int tc_operand_n(int n) { return pad16(n); }
 
-// Y[q][j] = sum_k X[q][k] U[k][j] on the tensor cores.  `scratch` (device, 16-byte aligned, at least
-// tc_scratch_bytes(K, N)) receives the bf16 operand.  Returns cudaErrorNotSupported when the shape or the
-// alignment does not fit (the caller then takes the SIMT kernel).
-cudaError_t launch_tc_lastmode(const ModeProdArgs& p, void* scratch, size_t scratch_bytes, cudaStream_t st) {
-  if (p.I != 1) return launch_tc_token(p, scratch, scratch_bytes, st);
-  const int64_t M = p.Q, K = p.a;
-  const int nv = p.n_out, N = (nv + 15) / 16 * 16;
-  if (p.I != 1 || nv % 4 != 0 || nv < 16 || N > kTcNMax || K % kTcKC != 0 || K < kTcKC || M < kTcM ||
-      M >= (1ll << 31) || K >= (1ll << 31) || p.sj != 1 || p.so % 4 != 0 || !scratch ||
-      scratch_bytes < tc_scratch_bytes(K, N) || (reinterpret_cast<uintptr_t>(scratch) & 15u) ||
-      (reinterpret_cast<uintptr_t>(p.X) & 15u) || (reinterpret_cast<uintptr_t>(p.Y) & 15u))
-    return cudaErrorNotSupported;
-  EncodeFn enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
-  CUtensorMap mapX, mapB;
-  const cuuint32_t estr[2] = {1, 1};
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)kTcM};
-    if (enc(&mapX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p.X), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorNotSupported;
-  }
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)(3 * N)};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)(3 * N)};
-    if (enc(&mapB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, scratch, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorNotSupported;
-  }
-  const size_t smem = kTcSmem;
-  const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_lastmode), smem);
-  if (attr_err != cudaSuccess) return attr_err;
-  k_tc_split<<<dim3((unsigned)((K + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      p.B, nv, (int)K, N, nv, static_cast<__nv_bfloat16*>(scratch), K);
-  TcArgs a = {p.Y, (int)M, N, (int)K, (int)p.so, (int)K, 0, 0, p.status, nv};
-  const unsigned grid = (unsigned)((M + kTcM - 1) / kTcM);
-  k_tc_lastmode<<<grid, kTcThreads, smem, st>>>(mapX, mapB, a);
-  return cudaGetLastError();
+// Which products of mode (O, a, I) with n columns run here: 0 none, 1 the last mode, 2 a mode with inner extent
+int tc_kind(int64_t O, int64_t a, int64_t I, int n) {
+  if (n % 4 != 0 || n < 16 || n > kTcNMax || a >= (1ll << 31) || O * I >= (1ll << 31)) return 0;
+  if (I == 1) return a % 64 == 0 && O >= kTcM ? 1 : 0;
+  return I % 64 == 0 && O < 65536 ? 2 : 0;
 }
 
-// Pp[s][k][j] = sum_{q in split s} X[q][k] V[q][j] on the tensor cores (the expansion P = A_m V of the last
-// mode, X bf16 [Q x a], V fp32 [Q x r]).  `scratch` as above, at least tc_scratch_bytes(Q, r).
-cudaError_t launch_tc_expand(const ExpandArgs& e, void* scratch, size_t scratch_bytes, cudaStream_t st) {
-  if (e.I != 1) return launch_tc_token_expand(e, scratch, scratch_bytes, st);
-  const int64_t Q = e.Q, A = e.a;
-  const int nv = e.r, N = (nv + 15) / 16 * 16;
-  if (e.I != 1 || nv % 4 != 0 || nv < 16 || N > kTcNMax || A % 8 != 0 || A < kTcM || Q % 8 != 0 || Q < kTcKC ||
-      Q >= (1ll << 31) || A >= (1ll << 31) || e.q_per_split % kTcKC != 0 || e.q_per_split >= (1ll << 31) ||
-      e.nsplit < 1 || !scratch || scratch_bytes < tc_scratch_bytes(Q, N) ||
-      (reinterpret_cast<uintptr_t>(scratch) & 15u) || (reinterpret_cast<uintptr_t>(e.X) & 15u) ||
-      (reinterpret_cast<uintptr_t>(e.Pp) & 15u))
-    return cudaErrorNotSupported;
-  EncodeFn enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
-  CUtensorMap mapX, mapB;
-  const cuuint32_t estr[2] = {1, 1};
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)A, (cuuint64_t)Q};
-    const cuuint64_t strides[1] = {(cuuint64_t)A * 2};
-    const cuuint32_t box[2] = {64, 64};
-    if (enc(&mapX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(e.X), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorNotSupported;
+void tc_add_split(TcSplitArgs* p, const float* U, int64_t K, int n, void* Bt) {
+  TcSplitMat& m = p->m[p->n++];
+  m.U = U;
+  m.Bt = static_cast<__nv_bfloat16*>(Bt);
+  m.K = (int)K;
+  m.nv = n;
+  m.N = pad16(n);
+  m.ldb = pad64(K);
+}
+
+cudaError_t launch_tc_split(TcSplitArgs& p, bool dep, cudaStream_t st) {
+  int first = 0;
+  for (int q = 0; q < p.n; ++q) {
+    p.m[q].first = first;
+    first += ((p.m[q].K + 31) / 32) * ((p.m[q].N + 31) / 32);
   }
-  {
-    const cuuint64_t dims[2] = {(cuuint64_t)Q, (cuuint64_t)(3 * N)};
-    const cuuint64_t strides[1] = {(cuuint64_t)Q * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTcKC, (cuuint32_t)(3 * N)};
-    if (enc(&mapB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, scratch, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorNotSupported;
+  return launch_maybe_pdl(dep, k_tc_split, dim3((unsigned)first), dim3(256), 0, st, p);
+}
+
+// One launch over the products of `c` (all with operands already split).  cudaErrorNotSupported: a tensor map could
+// not be made (nothing was launched).
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st) {
+  if (n < 1 || n > 3) return cudaErrorInvalidValue;
+  TcGroup g;
+  g.np = n;
+  g.status = status;
+  int nmax = 16;
+  double bytes = 0.0;
+  int64_t tiles[3];
+  int chunks[3];
+  for (int q = 0; q < n; ++q) {
+    const TcCall& k = c[q];
+    TcProb& p = g.p[q];
+    p.N = pad16(k.n);
+    p.nv = k.n;
+    p.inner = (int)k.I;
+    p.ldb = k.out_ld;
+    p.Bt = static_cast<__nv_bfloat16*>(k.out_bt);
+    p.Y = k.Y;
+    p.ldy = k.n;
+    nmax = p.N > nmax ? p.N : nmax;
+    const int64_t Q = k.O * k.I;
+    bool ok;
+    int64_t second = 1;
+    if (k.expand) {
+      p.mode = k.I == 1 ? kTcLastExpand : kTcTokenExpand;
+      p.M = (int)k.a;
+      p.K = (int)Q;
+      p.k_per_split = (int)k.q_per_split;
+      p.y_split = k.a * k.n;
+      second = k.nsplit;
+      chunks[q] = (int)((std::min<int64_t>(k.q_per_split, Q) + kTcKC - 1) / kTcKC);
+    } else {
+      p.mode = k.I == 1 ? kTcLast : kTcToken;
+      p.M = (int)(k.I == 1 ? Q : k.I);
+      p.K = (int)k.a;
+      p.k_per_split = (int)pad64(k.a);
+      p.y_split = k.I * k.n;
+      second = k.I == 1 ? 1 : k.O;
+      chunks[q] = (int)((k.a + kTcKC - 1) / kTcKC);
+    }
+    if (k.I == 1) {
+      const cuuint64_t dims[2] = {(cuuint64_t)k.a, (cuuint64_t)Q};
+      const cuuint64_t strides[1] = {(cuuint64_t)k.a * 2};
+      const cuuint32_t box[2] = {64, (cuuint32_t)(k.expand ? 64 : kTcM)};
+      ok = encode_bf16_map(&p.mapX, k.X, 2, dims, strides, box);
+    } else {
+      const cuuint64_t dims[3] = {(cuuint64_t)k.I, (cuuint64_t)k.a, (cuuint64_t)k.O};
+      const cuuint64_t strides[2] = {(cuuint64_t)k.I * 2, (cuuint64_t)k.a * k.I * 2};
+      const cuuint32_t box[3] = {64, (cuuint32_t)(k.expand ? kTcM : 64), 1};
+      ok = encode_bf16_map(&p.mapX, k.X, 3, dims, strides, box);
+    }
+    ok = ok && operand_map(&p.mapB, static_cast<const __nv_bfloat16*>(k.bt), p.K, p.N);
+    if (!ok) return cudaErrorNotSupported;
+    p.mt = (p.M + kTcM - 1) / kTcM;
+    tiles[q] = p.mt * second;
+    bytes += 2.0 * (double)k.a * Q;
   }
-  const size_t smem = kTcSmem;
-  const cudaError_t attr_err = opt_in_smem(reinterpret_cast<const void*>(k_tc_expand), smem);
-  if (attr_err != cudaSuccess) return attr_err;
-  k_tc_split<<<dim3((unsigned)((Q + 31) / 32), (unsigned)((N + 31) / 32)), 256, 0, st>>>(
-      e.V, nv, (int)Q, N, nv, static_cast<__nv_bfloat16*>(scratch), Q);
-  TcArgs a = {e.Pp, (int)A, N, (int)Q, nv, (int)e.q_per_split, A * nv, 0, e.status, nv};
-  dim3 grid((unsigned)((A + kTcM - 1) / kTcM), (unsigned)e.nsplit);
-  k_tc_expand<<<grid, kTcThreads, smem, st>>>(mapX, mapB, a);
-  return cudaGetLastError();
+  // a product with few tiles and a long contraction shares each tile between the CTAs of a cluster
+  int64_t total = 0;
+  for (int q = 0; q < n; ++q) total += tiles[q];
+  int cs = 1;
+  for (int q = 0; q < n; ++q)
+    while (cs < 4 && tiles[q] * cs < 200 && chunks[q] >= 8 * cs) cs *= 2;
+  int first = 0;
+  for (int q = 0; q < n; ++q) {
+    TcProb& p = g.p[q];
+    p.ksp = (cs > 1 && tiles[q] < 200 && chunks[q] >= 4 * cs) ? cs : 1;
+    p.first = first;
+    p.n_cta = (int)tiles[q] * p.ksp;
+    first += (p.n_cta + cs - 1) / cs * cs;
+  }
+  g.cs = cs;
+  g.tmem_cols = 3 * nmax <= 64 ? 64 : (3 * nmax <= 128 ? 128 : 256);
+  const int stage = (int)kTileA + 3 * nmax * 128;
+  g.nst = nmax <= 16 ? 4 : (nmax <= 48 ? 3 : 2);
+  size_t smem = 1024 + (size_t)g.nst * stage;
+  const size_t xch = 1024 + (size_t)kTcM * (nmax + 4) * 4;
+  if (xch > smem) smem = xch;
+  const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_tc_group), smem);
+  if (e != cudaSuccess) return e;
+  ProfScope prof(c[0].expand ? ASI_K_EXPAND : ASI_K_MODEPROD, st, bytes);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)first);
+  cfg.blockDim = dim3(kTcThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (cs > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)cs;
+    at[na].val.clusterDim.y = 1;
+    at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  if (dep) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, k_tc_group, g);
 }
 
 }  // namespace asi
