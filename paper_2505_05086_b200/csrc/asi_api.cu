@@ -159,7 +159,8 @@ void layout_compress(asi_plan* pl) {
     pl->off_Pred[m] = off;
     off = align_up(off + (size_t)v.a * std::max<int64_t>(v.r, (pl->fast_compress && m >= 2) ? v.a : 0) * 8, 256);
     pl->off_Gp[m] = off;
-    off = align_up(off + orth_gp_elems(pl->nchunk[m], v.r) * 8, 256);
+    const size_t shares = (pl->fast_compress || pl->small_rank) ? (size_t)pl->nchunk[m] * v.r * v.r : 0;   // k_sm_reduce's
+    off = align_up(off + std::max(shares, orth_gp_elems(pl->nchunk[m], v.r)) * 8, 256);
   }
   // Tensor-core products of bf16 tensors: a factor of 16..64 columns (a multiple of 4) over the last mode (a_m a
   // multiple of 64, at least 128 fibers) or over a mode whose inner extent is a multiple of 64
@@ -421,9 +422,7 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
     qa.m[m].nsplit = pl->nsplit[m];
     qa.m[m].nchunk = pl->nchunk[m];
     qa.m[m].rows = pl->qr_rows[m];
-    qa.m[m].gs = orth_group(pl->nchunk[m]);
     qa.m[m].count = reinterpret_cast<int*>(w) + 20 + m;
-    qa.m[m].gcount = reinterpret_cast<int*>(w) + 64 + kOrthGroups * m;
     if (first_core_tc && m == pl->core_order[0]) {   // the first core product reads U_m as a stacked operand
       qa.m[m].bt = reinterpret_cast<__nv_bfloat16*>(w + pl->tcu_off[m]);
       qa.m[m].bt_n = tc_operand_n(pl->r[m]);

@@ -212,8 +212,9 @@ struct GemmTile {
       const float* As = stage + st * kStage;
       const float* Bs = As + kTileA + warp * 16 * BN;
       if (kbeg + it * kGK + warp * 16 < kend) {
-#pragma unroll
-        for (int k4 = 0; k4 < 16; k4 += 4) {
+#pragma unroll 1
+        for (int k4 = 0; k4 < 16; k4 += 4) {           // not unrolled: the loop runs a few dozen times per CTA, and
+                                                       // straight-line code stalled on instruction fetch
           float a[4][4];                               // [k][row] (m-major) or [row][k] (k-major)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -273,7 +274,21 @@ struct GemmTile {
     }
     __syncthreads();
     float* Y = p.Y + (int64_t)split * p.ysplit + (int64_t)o * p.so;
+    if (BN >= 16 && p.sj == 1 && p.yvec) {              // rows of C are contiguous: four columns at a time
+#pragma unroll 1
+      for (int e = tid; e < kGM * BN / 4; e += kGT) {
+        const int m = e / (BN / 4), j = 4 * (e - m * (BN / 4));
+        float4 v = *reinterpret_cast<const float4*>(red + m * BN + j);
 #pragma unroll
+        for (int w = 1; w < kGW; ++w) {
+          const float4 t = *reinterpret_cast<const float4*>(red + (w * kGM + m) * BN + j);
+          v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+        }
+        if (m0 + m < p.M && j < p.n) *reinterpret_cast<float4*>(Y + (int64_t)(m0 + m) * p.si + j) = v;
+      }
+      return;
+    }
+#pragma unroll 1
     for (int t = 0; t < kGM * BN / kGT; ++t) {
       const int e = tid + t * kGT;
       int m, j;
@@ -343,6 +358,8 @@ GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_
   p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
   p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15u) == 0;
   p.tiles_m = (p.M + kGM - 1) / kGM;
+  p.yvec = p.sj == 1 && n % 4 == 0 && p.si % 4 == 0 && p.so % 4 == 0 && p.ysplit % 4 == 0 &&
+           (reinterpret_cast<uintptr_t>(p.Y) & 15u) == 0;
   return p;
 }
 
@@ -361,6 +378,8 @@ GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_
   p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
   p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(V) & 15u) == 0;
   p.tiles_m = (p.M + kGM - 1) / kGM;
+  p.yvec = p.sj == 1 && n % 4 == 0 && p.si % 4 == 0 && p.so % 4 == 0 && p.ysplit % 4 == 0 &&
+           (reinterpret_cast<uintptr_t>(p.Y) & 15u) == 0;
   return p;
 }
 
@@ -381,6 +400,10 @@ bool gemm_fits(int64_t O, int64_t a, int64_t I, int n) {
 
 cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st) {
   if (g.np < 1) return cudaSuccess;
+  // the longest contractions first: their CTAs would otherwise start last and run alone
+  std::sort(g.p, g.p + g.np, [](const GemmProb& a, const GemmProb& b) {
+    return (int64_t)std::min(a.K, a.kps) * bn_of(a.n) > (int64_t)std::min(b.K, b.kps) * bn_of(b.n);
+  });
   int first = 0, bn = 8;
   double bytes = 0.0;
   for (int q = 0; q < g.np; ++q) {

@@ -23,7 +23,6 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 constexpr int kStatusBytes = 1024;    // status word (int 0), completion counters (ints 16..255)
 constexpr int kQRMaxRank = 64;       // ranks k_orth_* cover (above: k_qrb_*)
-constexpr int kOrthGroups = 48;      // groups of Gram shares per mode (one counter each in the status block)
 
 // Y(o, j, i) = sum_k X(o, k, i) * B(k, j): the small-mode contraction that serves the
 // projection V = A_m^T U, the core products, Z1, Z3, and the final expansions.
@@ -76,12 +75,11 @@ struct Fiber2Args {
 struct QRMode {
   const float* Pp;     // [nsplit][a][r]
   double* Pred;        // [a][r]
-  double* Gp;          // [nchunk][r][r] shares of G, then their group sums, then R^{-T} (orth_gp_elems doubles)
+  double* Gp;          // packed shares of G, one per eight chunks, then R^{-T} (orth_gp_elems doubles)
   float* Uout;         // [a][r]
-  int* gcount;         // one counter per group of shares, zero on entry and on exit
-  int* count;          // one counter, same convention
+  int* count;          // one counter, zero on entry and on exit
   int a, r, nsplit, nchunk;
-  int rows, gs;        // rows of P per share, shares per group
+  int rows;            // rows of P per chunk
   __nv_bfloat16* bt;   // not null: U_m also as the stacked operand [3 bt_n][bt_ld] of the tensor-core products
   int64_t bt_ld;
   int bt_n;
@@ -310,7 +308,7 @@ struct GemmProb {
   int M, K, O, n;
   int nsplit, kps;         // K in nsplit parts of kps (a multiple of 128 unless nsplit == 1)
   int tiles_m, first;      // 32-row tiles; first CTA of the product in the launch
-  int km, vec, bvec;       // k-major A; rows of A / of B readable four values at a time
+  int km, vec, bvec, yvec; // k-major A; rows of A / of B readable, rows of C writable four values at a time
 };
 constexpr int kMaxGroup = 8;
 struct GemmGroup {
@@ -330,7 +328,6 @@ GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_
 cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st);
 
 int orth_rows(int64_t a, int r, int64_t nsplit);
-int orth_group(int64_t nchunk);
 size_t orth_gp_elems(int64_t nchunk, int r);
 cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st);
 cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st);

@@ -2,16 +2,22 @@
 // products in fp64 (in exact arithmetic the Gram-Schmidt basis of the columns of P).  Two launches for all modes:
 //
 //   k_orth_factor : CTA (c, m) sums the split partials of its rows of P_m in fp64 in split order and forms its
-//                   share of G = P^T P; the last CTA of a group of shares adds the group, the last group adds the
-//                   groups (both in index order) and factors G = R^T R once per mode, carrying the identity along
-//                   so that Y = R^{-T} falls out of the same elimination.
+//                   share of G = P^T P; the eight CTAs of a cluster add their shares through distributed shared
+//                   memory, the last cluster of a mode adds the clusters' shares (both in index order) and factors
+//                   G = R^T R once per mode, carrying the identity along so that Y = R^{-T} falls out of the same
+//                   elimination.
 //   k_orth_apply  : U = P R^{-1}, i.e. U[k][j] = sum_{i <= j} P[k][i] Y[j][i]: a plain product without a chain.
 //
-// What bounds it: the elimination is a serial chain of r pivots.  Four columns share one step (every thread
-// factors the 4 x 4 pivot block for itself, so a step has two barriers and no broadcast), and only one CTA per
-// mode walks the chain; the row solve that every CTA used to repeat is now the parallel second launch.
+// What bounds it: latency.  The elimination is a serial chain of r pivots (a reciprocal square root and two dependent
+// multiply-adds each, ~90 cycles); around it every step is a round trip to L2 (~1000 cycles under load).  So four
+// columns share one step, the two pivot warps work on step p + 1 while the other eight still update the rows behind
+// step p, shares meet inside a cluster instead of through memory, and the loads of a sum are issued in batches that
+// fit the chunk's shape.  The code is kept small: most of it runs once per launch, and straight-line code costs an
+// instruction fetch per 128 bytes.
 // A pivot d_j with d_j <= 1e-12 * trace(G), i.e. a Gram-Schmidt residual below 1e-6 * ||P||_F, raises
 // ASI_ERR_RANK_DEFICIENT in the status word.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "asi_internal.h"
@@ -20,50 +26,57 @@ namespace asi {
 
 namespace {
 
-constexpr int kOT = 256;                 // threads per CTA
+constexpr int kOT = 320;                 // threads per CTA: two pivot warps and eight update warps
+constexpr int kPivot = 64;               // threads of the pivot warps
+constexpr int kAT = 256;                 // threads of k_orth_apply
 constexpr int kOrthMaxRows = 64;         // rows of P per share, at most
-constexpr int kMaxPacked = 136 * 16;     // packed upper triangle of a 64 x 64 matrix
+constexpr int kOrthCluster = 8;          // chunks whose shares meet in distributed shared memory
+constexpr int kMaxPacked = 136 * 16;     // packed upper triangle of a 64 x 64 matrix, in 4 x 4 blocks
 
-// G = R^T R and Y = R^{-T} by one elimination on the r x r array T (ranks up to 16 NX): entries k >= i start as G,
-// the rest as zero; row i of Y takes the place of the entries k <= i.  Thread (ti, tj) keeps T[ti + 16 x][tj + 16 y]
-// in registers; shared memory carries what one step of four columns hands to the next: the four pivot rows
-// (Prow [4][64]) and the finished rows of R and Y (W [64][4]).  Y goes to Yg (row-major, zero above the diagonal).
+__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void named_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// element (i, k), k >= i, of the packed 4 x 4 blocks of an upper triangle with nb block rows
+__device__ __forceinline__ int packed_at(int i, int k, int nb) {
+  const int bi = i >> 2, bk = k >> 2;
+  return (bi * nb - bi * (bi - 1) / 2 + bk - bi) * 16 + (i & 3) * 4 + (k & 3);
+}
+
+// G = R^T R and Y = R^{-T} by one elimination on an r x r array T (ranks up to 16 NX): entries k >= i start as G,
+// the rest as zero; row i of Y takes the place of the entries k <= i.  Update thread (ti, tj) keeps
+// T[ti + 16 x][tj + 16 y] in registers and hands the four pivot rows of the next step over in Prow [4][64]; pivot
+// thread k solves column k of them and hands rows of R and Y back in W[step & 1] [64][4].  Y goes to Yg (row-major,
+// zero above the diagonal).
 template <int NX>
-__device__ void chol_with_inverse(double (&T)[NX][NX], double* Prow, double* W, double trace, int r,
-                                  double* __restrict__ Yg, int* status) {
-  const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
-  const double floor_d = 1e-12 * trace;
-  if (ti < 4) {
-#pragma unroll
-    for (int y = 0; y < NX; ++y) Prow[ti * kQRMaxRank + tj + 16 * y] = T[0][y];
-  }
-  __syncthreads();
+__device__ __forceinline__ void eliminate(const double* Gq, double* Prow, double* W, double floor_d, int r,
+                                          double* __restrict__ Yg, int* status) {
+  const int tid = threadIdx.x, nb = (r + 3) >> 2;
+  if (tid < kPivot) {
+    bool bad = false;
 #pragma unroll 1
-  for (int p0 = 0; p0 < r; p0 += 4) {
-    // column k of the four pivot rows; the pivot block itself is factored by every thread that needs it
-    if (tid < r) {
-      double D[4][4], inv[4], w[4];
+    for (int p0 = 0; p0 < r; p0 += 4) {
+      named_sync(1, kOT);                            // Prow holds the rows p0 .. p0 + 3
+      double D[4][4], w[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int k = i; k < 4; ++k)
-          D[i][k] = (p0 + k < r) ? Prow[i * kQRMaxRank + p0 + k] : (i == k ? 1.0 : 0.0);
+        for (int k = i; k < 4; ++k) D[i][k] = Prow[i * kQRMaxRank + p0 + k];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         w[c] = Prow[c * kQRMaxRank + tid];
         if (tid >= p0 && tid < p0 + 4) w[c] = (tid == p0 + c) ? 1.0 : 0.0;     // the identity's columns p0 .. p0 + 3
+        if (p0 + c >= r) D[c][c] = 1.0;              // rows past the end: identity
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         double d = D[c][c];
-        if (p0 + c < r && !(d > floor_d)) {
-          if (tid == 0) atomicMax(status, (int)ASI_ERR_RANK_DEFICIENT);
-          d = (floor_d > 0.0) ? floor_d : 1.0;
-        }
-        inv[c] = rsqrt(d);
-        w[c] *= inv[c];
+        const bool low = p0 + c < r && !(d > floor_d);
+        bad |= low;
+        if (low) d = floor_d > 0.0 ? floor_d : 1.0;
+        const double inv = rsqrt(d);
+        w[c] *= inv;
 #pragma unroll
-        for (int k = c + 1; k < 4; ++k) D[c][k] *= inv[c];
+        for (int k = c + 1; k < 4; ++k) D[c][k] *= inv;
 #pragma unroll
         for (int i = c + 1; i < 4; ++i) {
           w[i] = fma(-D[c][i], w[c], w[i]);
@@ -71,188 +84,178 @@ __device__ void chol_with_inverse(double (&T)[NX][NX], double* Prow, double* W, 
           for (int k = i; k < 4; ++k) D[i][k] = fma(-D[c][i], D[c][k], D[i][k]);
         }
       }
-      *reinterpret_cast<double2*>(W + tid * 4) = make_double2(w[0], w[1]);
-      *reinterpret_cast<double2*>(W + tid * 4 + 2) = make_double2(w[2], w[3]);
-      // rows p0 .. p0 + 3 of Y are final
+      double* Wp = W + ((p0 >> 2) & 1) * (4 * kQRMaxRank) + tid * 4;
+      *reinterpret_cast<double2*>(Wp) = make_double2(w[0], w[1]);
+      *reinterpret_cast<double2*>(Wp + 2) = make_double2(w[2], w[3]);
+      named_arrive(2, kOT);                          // W of this step is there
+      if (tid < r) {                                 // rows p0 .. p0 + 3 of Y are final
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (p0 + c < r) Yg[(int64_t)(p0 + c) * r + tid] = (tid <= p0 + c) ? w[c] : 0.0;
-    }
-    __syncthreads();
-    // rows i >= b: T[i][k] -= sum_c W[i][c] W[k][c] for the columns of Y done so far (k < b) and of G (k >= i)
-    const int b = p0 + 4;
-    if (b >= r) break;
-    double wk[NX][4];
-#pragma unroll
-    for (int y = 0; y < NX; ++y) {
-      const double2 c0 = *reinterpret_cast<const double2*>(W + (tj + 16 * y) * 4);
-      const double2 c1 = *reinterpret_cast<const double2*>(W + (tj + 16 * y) * 4 + 2);
-      wk[y][0] = c0.x; wk[y][1] = c0.y; wk[y][2] = c1.x; wk[y][3] = c1.y;
-    }
-#pragma unroll
-    for (int x = 0; x < NX; ++x) {
-      const int i = ti + 16 * x;
-      if (i >= b) {
-        const double2 a0 = *reinterpret_cast<const double2*>(W + i * 4);
-        const double2 a1 = *reinterpret_cast<const double2*>(W + i * 4 + 2);
-#pragma unroll
-        for (int y = 0; y < NX; ++y) {
-          const int k = tj + 16 * y;
-          double v = fma(-a0.x, wk[y][0], T[x][y]);
-          v = fma(-a0.y, wk[y][1], v);
-          v = fma(-a1.x, wk[y][2], v);
-          v = fma(-a1.y, wk[y][3], v);
-          T[x][y] = (k < b || k >= i) ? v : 0.0;
-        }
-        if (i < b + 4) {
-#pragma unroll
-          for (int y = 0; y < NX; ++y) Prow[(i - b) * kQRMaxRank + tj + 16 * y] = T[x][y];
-        }
+        for (int c = 0; c < 4; ++c)
+          if (p0 + c < r) Yg[(int64_t)(p0 + c) * r + tid] = (tid <= p0 + c) ? w[c] : 0.0;
       }
     }
-    __syncthreads();
+    if (bad && tid == 0) atomicMax(status, (int)ASI_ERR_RANK_DEFICIENT);
+  } else {
+    const int ut = tid - kPivot, ti = ut >> 4, tj = ut & 15;
+    double T[NX][NX];
+#pragma unroll
+    for (int x = 0; x < NX; ++x)
+#pragma unroll
+      for (int y = 0; y < NX; ++y) {
+        const int i = ti + 16 * x, k = tj + 16 * y;
+        T[x][y] = (k >= i && k < r) ? Gq[packed_at(i, k, nb)] : 0.0;
+      }
+    if (ti < 4) {
+#pragma unroll
+      for (int y = 0; y < NX; ++y) Prow[ti * kQRMaxRank + tj + 16 * y] = T[0][y];
+    }
+    named_arrive(1, kOT);
+#pragma unroll 1
+    for (int p0 = 0; p0 < r; p0 += 4) {
+      named_sync(2, kOT);
+      const int b = p0 + 4;
+      if (b >= r) break;
+      // rows i >= b: T[i][k] -= sum_c W[i][c] W[k][c] for the columns of Y done so far (k < b) and of G (k >= i);
+      // the four rows of the next step first
+      const double* Ws = W + ((p0 >> 2) & 1) * (4 * kQRMaxRank);
+      const bool mine = ((b ^ ti) & 12) == 0;        // this thread owns one of the rows b .. b + 3
+      const int bx = b >> 4;
+#pragma unroll
+      for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1 || mine) {
+#pragma unroll
+          for (int x = 0; x < NX; ++x) {
+            const int i = ti + 16 * x;
+            const bool next = mine && x == bx;
+            if (i >= b && (pass == 0) == next) {
+              const double2 a0 = *reinterpret_cast<const double2*>(Ws + i * 4);
+              const double2 a1 = *reinterpret_cast<const double2*>(Ws + i * 4 + 2);
+#pragma unroll
+              for (int y = 0; y < NX; ++y) {
+                const int k = tj + 16 * y;
+                const double2 c0 = *reinterpret_cast<const double2*>(Ws + k * 4);
+                const double2 c1 = *reinterpret_cast<const double2*>(Ws + k * 4 + 2);
+                double v = fma(-a0.x, c0.x, T[x][y]);
+                v = fma(-a0.y, c0.y, v);
+                v = fma(-a1.x, c1.x, v);
+                v = fma(-a1.y, c1.y, v);
+                T[x][y] = (k < b || k >= i) ? v : 0.0;
+                if (pass == 0) Prow[(i - b) * kQRMaxRank + k] = T[x][y];
+              }
+            }
+          }
+        }
+        if (pass == 0) named_arrive(1, kOT);
+      }
+    }
   }
 }
 
-// Sum of n shares (each `len` doubles) at element e, for up to EB elements at once so that EB * 8 loads are in
-// flight; the shares are added in index order.
-template <int EB>
-__device__ __forceinline__ void fold_shares(const double* __restrict__ src, int n, int len, int e0, double (&v)[EB]) {
+// dst[e] = sum over n of src[s * step + e] in order of s, e < len, with EB x SB loads in flight per thread.  Every
+// load is issued from a clamped address: a condition next to a load makes the others wait for it.
+template <int EB, int SB, typename TS, typename F>
+__device__ __forceinline__ void sum_strided(const TS* __restrict__ src, int n, int64_t step, int len, int e0, int estep, int s0,
+                                            int sstep, F&& put) {
+#pragma unroll 1
+  for (int eb = e0; eb < len; eb += EB * estep) {
+    double acc[EB];
 #pragma unroll
-  for (int q = 0; q < EB; ++q) v[q] = 0.0;
-  for (int s = 0; s < n; s += 8) {
-    double t[EB][8];
+    for (int q = 0; q < EB; ++q) acc[q] = 0.0;
+#pragma unroll 1
+    for (int s = s0; s < n; s += SB * sstep) {
+      TS t[EB][SB];
 #pragma unroll
-    for (int q = 0; q < EB; ++q)
+      for (int q = 0; q < EB; ++q)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + q * kOT;
-        t[q][u] = __ldcg(src + (int64_t)(s + u < n ? s + u : s) * len + (e < len ? e : 0));
-      }
+        for (int u = 0; u < SB; ++u) {
+          const int e = eb + q * estep, ss = s + u * sstep;
+          t[q][u] = __ldcg(src + (int64_t)(ss < n ? ss : s) * step + (e < len ? e : eb));
+        }
 #pragma unroll
-    for (int q = 0; q < EB; ++q)
+      for (int q = 0; q < EB; ++q)
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[q] += (s + u < n) ? t[q][u] : 0.0;
-  }
-}
-
-// the r x r matrix from packed 4 x 4 blocks of its upper triangle (shared memory), then the elimination
-template <int NX>
-__device__ void factor_packed(const double* Gq, double* Prow, double* W, double trace, int r, double* Yg, int* status) {
-  const int nb = (r + 3) >> 2, ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
-  double T[NX][NX];
-#pragma unroll
-  for (int x = 0; x < NX; ++x)
-#pragma unroll
-    for (int y = 0; y < NX; ++y) {
-      const int i = ti + 16 * x, k = tj + 16 * y;
-      const int bi = i >> 2, bk = k >> 2;
-      T[x][y] = (k >= i && k < r) ? Gq[(bi * nb - bi * (bi - 1) / 2 + bk - bi) * 16 + (i & 3) * 4 + (k & 3)] : 0.0;
+        for (int u = 0; u < SB; ++u) acc[q] += (s + u * sstep < n) ? (double)t[q][u] : 0.0;
     }
-  chol_with_inverse<NX>(T, Prow, W, trace, r, Yg, status);
+#pragma unroll
+    for (int q = 0; q < EB; ++q)
+      if (eb + q * estep < len) put(eb + q * estep, acc[q]);
+  }
 }
 
 }  // namespace
 
 __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRArgs args) {
   const QRMode M = args.m[blockIdx.y];
-  const int c = blockIdx.x;
-  if (c >= M.nchunk || M.r > kQRMaxRank) return;     // ranks above 64 take the k_qrb_* kernels
+  const int c = blockIdx.x, c8 = c & ~(kOrthCluster - 1), rank = c - c8;
+  if (c8 >= M.nchunk || M.r > kQRMaxRank) return;    // the whole cluster; ranks above 64 take the k_qrb_* kernels
   pdl_wait();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) double orth_smem[];
   __shared__ int s_last;
-  double* Ps = orth_smem;                            // this chunk's rows of P, pitch r
   const int tid = threadIdx.x, r = M.r;
+  const int nb = (r + 3) >> 2, nblk = nb * (nb + 1) / 2, len = nblk * 16, RP = 4 * nb;
+  double* Ps = orth_smem;                            // this chunk's rows of P, [rows][2][nb][2]: pairs (4 b, 4 b + 1), then (4 b + 2, 4 b + 3)
+  double* share = Ps + kOrthMaxRows * kQRMaxRank;    // [len]: this CTA's share of G
+  double* red = share + kMaxPacked;                  // scratch: partial sums over splits / over row groups
   const int row0 = c * M.rows;
-  const int nrows = min(M.rows, M.a - row0);
+  const int nrows = c < M.nchunk ? min(M.rows, M.a - row0) : 0;
   const int nval = nrows * r;                        // the chunk is one contiguous run of P
   const int64_t base = (int64_t)row0 * r, sstride = (int64_t)M.a * r;
-  // ---- sum of the split partials, in split order per lane group; eight loads in flight per element.  A short
-  // chunk leaves threads over: they take every SG-th split and the SG sums meet in order.
-  int SG = 1;
-  while (SG < 8 && nval * SG * 2 <= kOT) SG *= 2;
-  const int lanes = kOT / SG;
-  {
-    const int e0 = tid % lanes, sg = tid / lanes;
-    double* part = Ps + nval;                        // [SG][nval] (SG > 1 only: nval <= 128)
-    constexpr int EB = 8, SB = 4;                    // elements x splits in flight per thread
-    for (int eb = e0; eb < nval; eb += EB * lanes) {
-      const float* src = M.Pp + base;
-      double acc[EB];
-#pragma unroll
-      for (int q = 0; q < EB; ++q) acc[q] = 0.0;
-      for (int s = sg; s < M.nsplit; s += SB * SG) {
-        float t[EB][SB];
-#pragma unroll
-        for (int q = 0; q < EB; ++q)
-#pragma unroll
-          for (int u = 0; u < SB; ++u) {
-            const int e = eb + q * lanes, ss = s + u * SG;
-            // always a load, from a clamped address when off: a condition next to a load makes the others wait
-            t[q][u] = __ldcg(src + (int64_t)(ss < M.nsplit ? ss : s) * sstride + (e < nval ? e : 0));
-          }
-#pragma unroll
-        for (int q = 0; q < EB; ++q)
-#pragma unroll
-          for (int u = 0; u < SB; ++u) acc[q] += (s + u * SG < M.nsplit) ? (double)t[q][u] : 0.0;
-      }
-#pragma unroll
-      for (int q = 0; q < EB; ++q) {
-        const int e = eb + q * lanes;
-        if (e >= nval) break;
-        if (SG > 1) part[sg * nval + e] = acc[q];
-        else {
-          Ps[e] = acc[q];
-          M.Pred[base + e] = acc[q];
-        }
-      }
-    }
+  // ---- sum of the split partials: a short chunk leaves threads over, which take every SG-th split
+  auto place = [&](int e, double v) {
+    const int k = e / r, j = e - k * r;
+    Ps[k * RP + ((j & 2) ? RP / 2 : 0) + (j >> 2) * 2 + (j & 1)] = v;
+    M.Pred[base + e] = v;
+  };
+  if (nrows > 0) {
+    if (RP != r)
+      for (int e = tid; e < nrows * RP; e += kOT) Ps[e] = 0.0;   // columns past r
+    const int SG = nval >= kOT ? 1 : min(kOT / nval, min(M.nsplit, 8));
+    if (RP != r) __syncthreads();
     if (SG > 1) {
+      const int sg = tid / nval;
+      if (sg < SG)
+        sum_strided<1, 16>(M.Pp + base, M.nsplit, sstride, nval, tid - sg * nval, nval, sg, SG,
+                           [&](int e, double v) { red[sg * nval + e] = v; });
       __syncthreads();
       for (int e = tid; e < nval; e += kOT) {
-        double v = 0.0;
-        for (int q = 0; q < SG; ++q) v += part[q * nval + e];
-        Ps[e] = v;
-        M.Pred[base + e] = v;
+        double v = red[e];
+        for (int q = 1; q < SG; ++q) v += red[q * nval + e];
+        place(e, v);
       }
+    } else if (nval <= 4 * kOT) {
+      sum_strided<4, 8>(M.Pp + base, M.nsplit, sstride, nval, tid, kOT, 0, 1, place);
+    } else {
+      sum_strided<7, 4>(M.Pp + base, M.nsplit, sstride, nval, tid, kOT, 0, 1, place);
     }
   }
   __syncthreads();
-  // ---- share of G in packed 4 x 4 blocks of the upper triangle: thread (block, row group); the row groups of a
-  // block (rows == rg mod RG) meet in order
-  const int nb = (r + 3) >> 2, nblk = nb * (nb + 1) / 2, len = nblk * 16;
-  double* Gc = M.Gp + (int64_t)c * len;
+  // ---- share of G in packed 4 x 4 blocks of the upper triangle: thread (block, row group), row groups in order
   {
-    int RG = kOT / nblk;
-    if (RG > 8) RG = 8;
-    if (RG < 1) RG = 1;
-    double* red = Ps + kOrthMaxRows * kQRMaxRank;    // [RG][len]
+    const int RG = min(kOT / nblk, 8);
     const int rg = tid / nblk, t = tid - rg * nblk;
     if (rg < RG) {
       int bi = 0, left = t;
       while (left >= nb - bi) { left -= nb - bi; ++bi; }
-      const int i0 = 4 * bi, j0 = 4 * (bi + left);
+      const int bj = bi + left;
       double g[4][4];
-      int ii[4], jj[4];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        ii[x] = i0 + x < r ? i0 + x : r - 1;
-        jj[x] = j0 + x < r ? j0 + x : r - 1;
+      for (int x = 0; x < 4; ++x)
 #pragma unroll
         for (int y = 0; y < 4; ++y) g[x][y] = 0.0;
-      }
-#pragma unroll 2
+#pragma unroll 1
       for (int rl = rg; rl < nrows; rl += RG) {
-        const double* prow = Ps + rl * r;
-        double a[4], b[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) { a[x] = prow[ii[x]]; b[x] = prow[jj[x]]; }
+        const double* prow = Ps + rl * RP;
+        const double2 a0 = *reinterpret_cast<const double2*>(prow + 2 * bi), a1 = *reinterpret_cast<const double2*>(prow + RP / 2 + 2 * bi);
+        const double2 b0 = *reinterpret_cast<const double2*>(prow + 2 * bj), b1 = *reinterpret_cast<const double2*>(prow + RP / 2 + 2 * bj);
+        const double a[4] = {a0.x, a0.y, a1.x, a1.y}, b[4] = {b0.x, b0.y, b1.x, b1.y};
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
           for (int y = 0; y < 4; ++y) g[x][y] = fma(a[x], b[y], g[x][y]);
       }
-      double* dst = (RG > 1 ? red + rg * len : Gc) + t * 16;
+      double* dst = (RG > 1 ? red + rg * len : share) + t * 16;
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -263,68 +266,53 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
       for (int e = tid; e < len; e += kOT) {
         double v = red[e];
         for (int q = 1; q < RG; ++q) v += red[q * len + e];
-        Gc[e] = v;
+        share[e] = v;
       }
     }
   }
-  // ---- shares -> groups -> G, each level by its last CTA, in index order
-  const int grp = c / M.gs, ngroups = (M.nchunk + M.gs - 1) / M.gs;
-  const int gfirst = grp * M.gs, gsize = min(M.gs, M.nchunk - gfirst);
-  double* Gg = M.Gp + (int64_t)M.nchunk * len;       // [ngroups][len]
-  double* Yg = Gg + (int64_t)ngroups * len;          // R^{-T}, row-major
+  // ---- the cluster's shares meet: CTA `rank` adds the elements [rank * per, ..) of all of them, in chunk order
+  cluster.sync();
+  const int live = min(kOrthCluster, M.nchunk - c8), nclu = (M.nchunk + kOrthCluster - 1) / kOrthCluster;
+  double* Gc = M.Gp + (int64_t)(c8 / kOrthCluster) * len;
+  {
+    const int per = (len + kOrthCluster - 1) / kOrthCluster, e1 = min(len, (rank + 1) * per);
+    for (int e = rank * per + tid; e < e1; e += kOT) {
+      double t[kOrthCluster], v = 0.0;
+#pragma unroll
+      for (int q = 0; q < kOrthCluster; ++q) t[q] = cluster.map_shared_rank(share, q < live ? q : 0)[e];
+#pragma unroll
+      for (int q = 0; q < kOrthCluster; ++q) v += q < live ? t[q] : 0.0;
+      Gc[e] = v;
+    }
+  }
   __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(M.gcount + grp, 1) == gsize - 1);
+  cluster.sync();                                    // every share has been read and every part of Gc written
+  if (rank != 0) return;
+  if (tid == 0) {
+    __threadfence();
+    s_last = (atomicAdd(M.count, 1) == nclu - 1);
+    if (s_last) *M.count = 0;
+  }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  constexpr int EB = 5;
-  double v[EB];
-  if (ngroups > 1) {
-    for (int e0 = tid; e0 < len; e0 += EB * kOT) {
-      fold_shares<EB>(M.Gp + (int64_t)gfirst * len, gsize, len, e0, v);
-#pragma unroll
-      for (int q = 0; q < EB; ++q)
-        if (e0 + q * kOT < len) Gg[(int64_t)grp * len + e0 + q * kOT] = v[q];
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-      M.gcount[grp] = 0;
-      s_last = (atomicAdd(M.count, 1) == ngroups - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (tid == 0) *M.count = 0;
-  } else if (tid == 0) {
-    M.gcount[grp] = 0;
-  }
-  const double* src = ngroups > 1 ? Gg : M.Gp;
-  const int nsum = ngroups > 1 ? ngroups : gsize;
-  double* Gq = orth_smem;                            // [len]
+  double* Gq = Ps;                                   // [len]
   double* Prow = Gq + kMaxPacked;                    // [4][64]
-  double* W = Prow + 4 * kQRMaxRank;                 // [64][4]
-  for (int e0 = tid; e0 < len; e0 += EB * kOT) {
-    fold_shares<EB>(src, nsum, len, e0, v);
-#pragma unroll
-    for (int q = 0; q < EB; ++q)
-      if (e0 + q * kOT < len) Gq[e0 + q * kOT] = v[q];
-  }
-  W[tid] = 0.0;                                      // columns past r multiply zeros
+  double* W = Prow + 4 * kQRMaxRank;                 // [2][64][4]
+  sum_strided<3, 8>(M.Gp, nclu, len, len, tid, kOT, 0, 1, [&](int e, double v) { Gq[e] = v; });
+  for (int e = tid; e < 2 * 4 * kQRMaxRank; e += kOT) W[e] = 0.0;
+  for (int e = tid; e < 4 * kQRMaxRank; e += kOT) Prow[e] = 0.0;
   __syncthreads();
   double trace = 0.0;
-  for (int b = 0, o = 0; b < nb; o += nb - b, ++b)
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-      if (4 * b + x < r) trace += Gq[o * 16 + x * 5];
-  if (r <= 16) factor_packed<1>(Gq, Prow, W, trace, r, Yg, args.status);
-  else if (r <= 32) factor_packed<2>(Gq, Prow, W, trace, r, Yg, args.status);
-  else factor_packed<4>(Gq, Prow, W, trace, r, Yg, args.status);
+  for (int b = 0, o = 0; b < nb; o += nb - b, ++b)   // entries past r are zero
+    trace += (Gq[o * 16] + Gq[o * 16 + 5]) + (Gq[o * 16 + 10] + Gq[o * 16 + 15]);
+  double* Yg = M.Gp + (int64_t)nclu * len;           // R^{-T}, row-major
+  if (r <= 32) eliminate<2>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
+  else eliminate<4>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
 }
 
 // CTA (c, m): 32 rows of U_m; thread (ti, tj) owns rows ti, ti + 16 and columns tj, tj + 16, ..
-__global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRArgs args) {
+__global__ void __launch_bounds__(kAT) k_orth_apply(const __grid_constant__ QRArgs args) {
   const QRMode M = args.m[blockIdx.y];
   const int row0 = blockIdx.x * 32;
   if (row0 >= M.a || M.r > kQRMaxRank) return;
@@ -336,24 +324,24 @@ __global__ void __launch_bounds__(kOT) k_orth_apply(const __grid_constant__ QRAr
   double* Ps = Ys + r * PY;                          // [32][r]
   const int nrows = min(32, M.a - row0);
   const int nb = (r + 3) >> 2;
-  const double* Yg = M.Gp + (int64_t)(M.nchunk + (M.nchunk + M.gs - 1) / M.gs) * (nb * (nb + 1) * 8);
+  const double* Yg = M.Gp + (int64_t)((M.nchunk + kOrthCluster - 1) / kOrthCluster) * (nb * (nb + 1) * 8);
   // eight loads of P and eight of Y in flight per round
-  for (int e0 = tid; e0 < rr; e0 += 8 * kOT) {
+  for (int e0 = tid; e0 < rr; e0 += 8 * kAT) {
     double t[8], q[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int e = e0 + u * kOT;
+      const int e = e0 + u * kAT;
       t[u] = __ldcg(Yg + (e < rr ? e : 0));
       q[u] = __ldcg(M.Pred + (int64_t)row0 * r + (e < nrows * r ? e : 0));
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int e = e0 + u * kOT;
+      const int e = e0 + u * kAT;
       if (e < rr) Ys[e / r * PY + e % r] = t[u];
       if (e < 32 * r) Ps[e] = (e < nrows * r) ? q[u] : 0.0;
     }
   }
-  for (int e = rr + tid; e < 32 * r; e += kOT) Ps[e] = (e < nrows * r) ? __ldcg(M.Pred + (int64_t)row0 * r + e) : 0.0;
+  for (int e = rr + tid; e < 32 * r; e += kAT) Ps[e] = (e < nrows * r) ? __ldcg(M.Pred + (int64_t)row0 * r + e) : 0.0;
   __syncthreads();
   const int ti = tid >> 4, tj = tid & 15;
 #pragma unroll 1
@@ -424,16 +412,9 @@ int orth_rows(int64_t a, int r, int64_t nsplit) {
   while (rows < kOrthMaxRows && (a + rows - 1) / rows > 1024) rows *= 2;
   return rows;
 }
-// shares per group: one group up to 16 shares, else 8 each, at most kOrthGroups groups per mode (their counters sit in the status block)
-int orth_group(int64_t nchunk) {
-  int gs = nchunk <= 16 ? 16 : 8;
-  while ((nchunk + gs - 1) / gs > kOrthGroups) gs *= 2;
-  return gs;
-}
 size_t orth_gp_elems(int64_t nchunk, int r) {
-  const int gs = orth_group(nchunk);
   const size_t nb = (r + 3) / 4;
-  return (size_t)(nchunk + (nchunk + gs - 1) / gs) * nb * (nb + 1) * 8 + (size_t)r * r;   // packed shares and groups, R^{-T}
+  return (size_t)((nchunk + kOrthCluster - 1) / kOrthCluster) * nb * (nb + 1) * 8 + (size_t)r * r;   // clusters' shares, R^{-T}
 }
 
 cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st) {
@@ -450,13 +431,27 @@ cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st) {
   }
   ProfScope prof(ASI_K_QR, st, bytes);
   if (any) {
-    const size_t s1 = (size_t)2 * kOrthMaxRows * kQRMaxRank * 8, s2 = ((size_t)rmax * (rmax | 1) + 32 * rmax) * 8;
+    const size_t s1 = (size_t)(kOrthMaxRows * kQRMaxRank + kMaxPacked + kOT * 16) * 8, s2 = ((size_t)rmax * (rmax | 1) + 32 * rmax) * 8;
     cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_orth_factor), s1);
     if (e == cudaSuccess) e = opt_in_smem(reinterpret_cast<const void*>(k_orth_apply), s2);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_orth_factor, dim3((unsigned)chunks, (unsigned)nd), dim3(kOT), s1, st, p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((chunks + kOrthCluster - 1) / kOrthCluster * kOrthCluster), (unsigned)nd);
+    cfg.blockDim = dim3(kOT);
+    cfg.dynamicSmemBytes = s1;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kOrthCluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, k_orth_factor, p);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_orth_apply, dim3((unsigned)((amax + 31) / 32), (unsigned)nd), dim3(kOT), s2, st, p);
+    e = launch_pdl(k_orth_apply, dim3((unsigned)((amax + 31) / 32), (unsigned)nd), dim3(kAT), s2, st, p);
     if (e != cudaSuccess) return e;
   }
   return big ? launch_qr_big(p, nd, st) : cudaSuccess;
