@@ -28,10 +28,13 @@ void set_mode_views(asi_plan* pl) {
 // dynamic shared memory a fused kernel may ask for: 227 KB per CTA minus up to ~17 KB of static arrays
 constexpr size_t kSmemLimit = 208 * 1024;
 
+void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev, char* w, SmPass1Args* a);
+void build_fused_core(const asi_plan* pl, const void* act, float* U_new, float* core, char* w, bool gram_modes, SmCoreArgs* c);
+
 // Which fused kernels cover this layer (decided once, at plan creation).
 void choose_kernels(asi_plan* pl) {
   pl->fast_compress = pl->fast_wgrad = false;
-  pl->fast_S = pl->fast_R = pl->n_tiles_b = pl->cpb = 0;
+  pl->fast_kind = pl->fast_R = pl->n_tiles_b = pl->cpb = 0;
   if (pl->d.kind != ASI_CONV2D || (pl->d.flags & ASI_FLAG_GENERIC_ONLY)) return;
   int rmax = 0;
   for (int m = 0; m < 4; ++m) rmax = std::max(rmax, pl->r[m]);
@@ -39,34 +42,37 @@ void choose_kernels(asi_plan* pl) {
   const int R = rmax <= 4 ? 4 : 8;
   pl->fast_R = R;
   const int64_t B = pl->dims[0], C = pl->dims[1], H = pl->dims[2], W = pl->dims[3];
-  if (H == W && (H == 7 || H == 14 || H == 16) && B % 8 == 0 && B <= 1024 && C <= 4096 &&
-      (H != 7 || C % 4 == 0)) {
-    const int S = (int)H;
-    if (sm_pass1_smem(S, R, (int)B, (int)C) <= kSmemLimit && sm_core_smem(S, R, (int)B) <= kSmemLimit &&
-        B + 4 + 2 * S <= sm_core_max_rows()) {
-      pl->fast_compress = true;
-      pl->fast_S = S;
-      pl->n_tiles_b = (int)((S == 7) ? C / 4 : C);
-    }
+  // whole planes of at most 256 positions (a CTA's threads), rows and columns of at most 32 (a warp's lanes)
+  if (H * W <= 256 && H <= 32 && W <= 32 && B <= 1024 && C <= 4096) {
+    pl->fast_kind = (H == W && (H == 7 || H == 14)) ? (int)H : 0;
+    pl->fast_vec4 = (C * H * W) % 4 == 0;
+    sm_pass1_split((int)(H * W), (int)C, &pl->fast_cs, &pl->fast_cc);
+    pl->core_tile_c = sm_core_tile_c((int)(H * W), (int)C);
+    pl->n_tiles_core = (int)((C + pl->core_tile_c - 1) / pl->core_tile_c);
+    pl->n_tiles_b = sm_pass1_tiles_b(C * H * W, pl->fast_vec4);
+    pl->fold_gs = 8;                                 // tiles per group of the core's two-level sum
+    while ((pl->n_tiles_core + pl->fold_gs - 1) / pl->fold_gs > 192) pl->fold_gs *= 2;
+    SmPass1Args a;
+    SmCoreArgs c;
+    build_fused_pass1(pl, nullptr, nullptr, nullptr, &a);
+    build_fused_core(pl, nullptr, nullptr, nullptr, nullptr, true, &c);
+    pl->fast_compress = sm_pass1_smem(a, pl->fast_kind, R) <= kSmemLimit && sm_core_smem(c, R) <= kSmemLimit;
   }
   if (B <= 4096 && H <= 64 && W <= 64) {
     const int Cout = pl->d.cout;
     const int64_t HoWo = pl->Ho * pl->Wo;
-    // channels per CTA: the smallest count that makes a staged row a multiple of 16 bytes (rows can
-    // then be staged by 16-byte asynchronous copies); failing that, the smallest that makes it even
-    int cpb = 0;
-    bool rows_ok = false;
-    for (int c = 1; c <= 4 && !cpb; c *= 2)
-      if (Cout % c == 0 && (c * HoWo * 4) % 16 == 0) { cpb = c; rows_ok = true; }
-    for (int c = 1; c <= 2 && !cpb; c *= 2)
-      if (Cout % c == 0 && (c * HoWo) % 2 == 0) cpb = c;
-    if (!cpb) return;
+    // channels per CTA: the smallest count of one, two, four that makes a row of the tile a multiple of four values
+    int cpb = 1;
+    for (int c = 1; c <= 4; c *= 2)
+      if (Cout % c == 0 && (c * HoWo) % 4 == 0) { cpb = c; break; }
+    pl->wgrad_vec4 = (cpb * HoWo) % 4 == 0 && (Cout * HoWo) % 4 == 0;
     SmWgradArgs a;
     std::memset(&a, 0, sizeof(a));
     for (int m = 0; m < 4; ++m) a.r[m] = pl->r[m];
     a.B = (int)B; a.C = (int)C; a.Cout = Cout; a.H = (int)H; a.W = (int)W;
     a.Ho = (int)pl->Ho; a.Wo = (int)pl->Wo; a.kh = pl->d.kh; a.kw = pl->d.kw; a.cpb = cpb;
     a.ph = pl->d.pad_h; a.pw = pl->d.pad_w; a.groups = pl->d.groups;
+    a.vec4 = pl->wgrad_vec4 ? 1 : 0;
     // term 5 expands the channels in two rounds when the staging blocks fit, else one at a time
     a.ncl = cpb >= 2 ? cpb / 2 : 1;
     if (sm_wgrad_smem(a, R) > kSmemLimit) a.ncl = 1;
@@ -74,7 +80,6 @@ void choose_kernels(asi_plan* pl) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
       pl->wgrad_ncl = a.ncl;
-      pl->wgrad_bulk = rows_ok && !pl->bf16;
     }
   }
 }
@@ -140,9 +145,9 @@ void layout_compress(asi_plan* pl) {
     int64_t qps = (v.Q + ns - 1) / ns;
     qps = (qps + 127) / 128 * 128;
     ns = (v.Q + qps - 1) / qps;
-    if (pl->fast_compress) {                                             // one partial per tile; the cold-start
-      ns = (m == 1) ? sm_pass1_role_c_ctas(pl->fast_S, (int)pl->dims[0]) : pl->n_tiles_b;   // expansion splits the
-      qps = ((v.Q + ns - 1) / ns + 63) / 64 * 64;                        // columns over the same count
+    if (pl->fast_compress) {                                             // one partial per column tile, per sample,
+      ns = m == 0 ? pl->n_tiles_b : (m == 1 ? pl->dims[0] : pl->dims[0] * pl->fast_cs);   // per role-C CTA; the cold-start
+      qps = ((v.Q + ns - 1) / ns + 127) / 128 * 128;                     // expansion splits the columns over at most as many
     }
     if (pl->fiber[m] || (pl->plane && m >= 2)) {                         // one partial per CTA of k_fiber /
       ns = pl->fiber[m] ? pl->fiber_grid[m] : pl->plane_grid;            // k_plane; the cold-start expansion
@@ -154,7 +159,7 @@ void layout_compress(asi_plan* pl) {
     pl->nchunk[m] = (int)((v.a + pl->qr_rows[m] - 1) / pl->qr_rows[m]);
     pl->off_Pp[m] = off;
     size_t pp_elems = (size_t)ns * v.a * v.r;
-    if (pl->fast_compress && (pl->fast_S == 7 || pl->fast_S == 14) && m >= 2) pp_elems = std::max(pp_elems, (size_t)ns * v.a * v.a);
+    if (pl->fast_compress && pl->fast_kind && m >= 2) pp_elems = std::max(pp_elems, (size_t)ns * v.a * v.a);
     off = align_up(off + pp_elems * 4, 256);
     pl->off_Pred[m] = off;
     off = align_up(off + (size_t)v.a * std::max<int64_t>(v.r, (pl->fast_compress && m >= 2) ? v.a : 0) * 8, 256);
@@ -204,10 +209,8 @@ void layout_compress(asi_plan* pl) {
     tmax[s & 1] = std::max(tmax[s & 1], n);
   }
   if (pl->fast_compress) {
-    tmax[0] = (int64_t)pl->n_tiles_b * pl->core_elems;          // per-tile partial cores
-    pl->fold_gs = 8;                                             // tiles per group of the two-level sum
-    while ((pl->n_tiles_b + pl->fold_gs - 1) / pl->fold_gs > 192) pl->fold_gs *= 2;
-    tmax[1] = (int64_t)((pl->n_tiles_b + pl->fold_gs - 1) / pl->fold_gs) * pl->core_elems;
+    tmax[0] = pl->dims[1] * (pl->core_elems / pl->r[1]);        // per-channel shares
+    tmax[1] = (int64_t)((pl->n_tiles_core + pl->fold_gs - 1) / pl->fold_gs) * pl->core_elems;
   }
   for (int t = 0; t < 2; ++t) {
     pl->off_T[t] = off;
@@ -274,6 +277,11 @@ void layout_wgrad(asi_plan* pl) {
   pl->wgrad_ws = off;
 }
 
+// the fused kernels read the activation four values at a time where its columns allow it
+bool fused_misaligned(const asi_plan* pl, const void* act) {
+  return pl->fast_vec4 && (reinterpret_cast<uintptr_t>(act) & (pl->bf16 ? 7u : 15u)) != 0;
+}
+
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
   if (!valid_ptr(ws)) return ASI_ERR_INVALID_ARG;
   if (have < need || (reinterpret_cast<uintptr_t>(ws) & 255u)) return ASI_ERR_WORKSPACE;
@@ -304,7 +312,15 @@ void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev,
   a->status = reinterpret_cast<int*>(w);     // cleared by the kernel itself
   a->B = (int)pl->dims[0];
   a->C = (int)pl->dims[1];
+  a->H = (int)pl->dims[2];
+  a->W = (int)pl->dims[3];
   a->n_tiles_b = pl->n_tiles_b;
+  a->cs = pl->fast_cs;
+  a->cc = pl->fast_cc;
+  a->pitch = sm_pass1_pitch(a->H * a->W);
+  a->off_u2 = sm_pass1_off_u2(pl->fast_R, a->cc, a->pitch);
+  a->vec4 = pl->fast_vec4 ? 1 : 0;
+  a->bulk = (!pl->bf16 && pl->fast_vec4) ? 1 : 0;
   a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;      // 1 ms under the test hook, else 1 s
 }
@@ -320,7 +336,7 @@ int build_fused_reduce(const asi_plan* pl, char* w, const float* gram_U_prev, Sm
     ra->m[m].r = pl->r[m];
     ra->m[m].nsplit = pl->nsplit[m];
     ra->m[m].nchunk = pl->nchunk[m];
-    if (gram_U_prev && (pl->fast_S == 7 || pl->fast_S == 14) && m >= 2) {
+    if (gram_U_prev && pl->fast_kind && m >= 2) {
       ra->m[m].gram = 1;
       ra->m[m].nchunk = (int)((pl->dims[m] * pl->dims[m] + 24) / 25);   // ~25 Gram elements per CTA
       ra->m[m].Pg = reinterpret_cast<double*>(w + pl->off_Pg[m]);
@@ -348,14 +364,18 @@ void build_fused_core(const asi_plan* pl, const void* act, float* U_new, float* 
   c->gs = pl->fold_gs;
   c->Tg = reinterpret_cast<float*>(w + pl->off_T[1]);
   for (int m = 0; m < 4; ++m) {
-    const bool gram = gram_modes && (pl->fast_S == 7 || pl->fast_S == 14) && m >= 2;
+    const bool gram = gram_modes && pl->fast_kind && m >= 2;
     c->Pred[m] = reinterpret_cast<const double*>(w + (gram ? pl->off_Pg[m] : pl->off_Pred[m]));
     c->u_off[m] = pl->u_off[m];
     c->r[m] = pl->r[m];
   }
   c->B = (int)pl->dims[0];
   c->C = (int)pl->dims[1];
-  c->n_tiles = pl->n_tiles_b;
+  c->H = (int)pl->dims[2];
+  c->W = (int)pl->dims[3];
+  c->tile_c = pl->core_tile_c;
+  c->n_tiles = pl->n_tiles_core;
+  c->vec4 = (pl->fast_vec4 && (pl->core_tile_c * c->H * c->W) % 4 == 0) ? 1 : 0;
 }
 
 // false: dY is not aligned as the staged copies of this plan need
@@ -371,9 +391,8 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
   g->kh = pl->d.kh; g->kw = pl->d.kw; g->sh = pl->d.stride_h; g->sw = pl->d.stride_w;
   g->ph = pl->d.pad_h; g->pw = pl->d.pad_w; g->groups = pl->d.groups; g->cpb = pl->cpb;
   g->ncl = pl->wgrad_ncl;
-  g->pj = sm_wgrad_pitch(pl->cpb * (int)(pl->Ho * pl->Wo));
-  g->bulk = pl->wgrad_bulk ? 1 : 0;
-  if (g->bulk && (reinterpret_cast<uintptr_t>(dY) & 15u)) return false;
+  g->vec4 = pl->wgrad_vec4 ? 1 : 0;
+  if (g->vec4 && (reinterpret_cast<uintptr_t>(dY) & (pl->bf16 ? 7u : 15u))) return false;
   g->status = reinterpret_cast<int*>(w);
   g->bulk_store = (((pl->dims[1] / pl->d.groups) * pl->d.kh * pl->d.kw) % 4 == 0 &&
                    (reinterpret_cast<uintptr_t>(dW) & 15u) == 0) ? 1 : 0;
@@ -485,7 +504,7 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
   if (pl->fast_compress) {
     SmCoreArgs c;
     build_fused_core(pl, act, U_new, core, w, gram_U_prev != nullptr, &c);
-    ASI_CUDA(launch_sm_core(c, pl->fast_S, pl->fast_R, pl->bf16, st));
+    ASI_CUDA(launch_sm_core(c, pl->fast_R, pl->bf16, st));
     return ASI_OK;
   }
   int64_t cd[ASI_MAX_MODES];
@@ -825,11 +844,10 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   if (pl->fast_compress) {
-    // fp32 tiles are staged by 16-byte asynchronous copies, which need 16-byte aligned sources
-    if (!pl->bf16 && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
+    if (fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
     SmPass1Args a;
     build_fused_pass1(pl, act, U_prev, w, &a);
-    ASI_CUDA(launch_sm_pass1(a, pl->fast_S, pl->fast_R, pl->bf16, st));
+    ASI_CUDA(launch_sm_pass1(a, pl->fast_kind, pl->fast_R, pl->bf16, st));
     return finish_compress(pl, act, U_new, core, w, U_prev, false, st);
   }
   for (int m = 0; m < pl->nd; ++m)                   // bulk and 16-byte copies; errors before anything is enqueued
@@ -939,9 +957,11 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
 // table the CTAs index; the remaining layers are enqueued one after another on the same stream.
 // ---------------------------------------------------------------------------------------------
 namespace {
+// layers that share launches: one kernel variant, one cluster size
 struct Variant {
-  int S, R, bf16;
-  bool operator==(const Variant& o) const { return S == o.S && R == o.R && bf16 == o.bf16; }
+  int kind, R, cs, bf16;
+  explicit Variant(const asi_plan* p) : kind(p->fast_kind), R(p->fast_R), cs(p->fast_cs), bf16(p->bf16 ? 1 : 0) {}
+  bool operator==(const Variant& o) const { return kind == o.kind && R == o.R && cs == o.cs && bf16 == o.bf16; }
 };
 }  // namespace
 
@@ -957,7 +977,7 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (U_prev[i] == U_new[i]) return ASI_ERR_INVALID_ARG;
     const asi_status_t s = check_ws(ws[i], ws_bytes[i], pl->compress_ws);
     if (s != ASI_OK) return s;
-    if (pl->fast_compress && !pl->bf16 && (reinterpret_cast<uintptr_t>(acts[i]) & 15u)) return ASI_ERR_INVALID_ARG;
+    if (pl->fast_compress && fused_misaligned(pl, acts[i])) return ASI_ERR_INVALID_ARG;
     for (int j = 0; j < i; ++j)
       if (ws[j] == ws[i]) return ASI_ERR_INVALID_ARG;            // every layer needs a workspace of its own
   }
@@ -969,10 +989,10 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (done[i]) continue;
     std::vector<int> grp(1, i);
     if (plans[i]->fast_compress) {
-      const Variant v = {plans[i]->fast_S, plans[i]->fast_R, plans[i]->bf16 ? 1 : 0};
+      const Variant v(plans[i]);
       for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j) {
         const asi_plan* q = plans[j];
-        if (!done[j] && q->fast_compress && v == Variant{q->fast_S, q->fast_R, q->bf16 ? 1 : 0}) grp.push_back(j);
+        if (!done[j] && q->fast_compress && v == Variant(q)) grp.push_back(j);
       }
     }
     for (int j : grp) done[j] = 1;
@@ -995,9 +1015,9 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
       mc[k] = build_fused_reduce(plans[j], w, U_prev[j], &ra[k]);
       build_fused_core(plans[j], acts[j], U_new[j], cores[j], w, true, &ca[k]);
     }
-    ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_S, p0->fast_R, p0->bf16, st));
+    ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_kind, p0->fast_R, p0->bf16, st));
     ASI_CUDA(launch_sm_reduce_batched(ra.data(), mc.data(), g, st));
-    ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_S, p0->fast_R, p0->bf16, st));
+    ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_R, p0->bf16, st));
     return ASI_OK;
   });
 }
@@ -1012,7 +1032,7 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
       return ASI_ERR_INVALID_ARG;
     const asi_status_t s = check_ws(ws[i], ws_bytes[i], pl->wgrad_ws);
     if (s != ASI_OK) return s;
-    if (pl->fast_wgrad && pl->wgrad_bulk && (reinterpret_cast<uintptr_t>(dY[i]) & 15u)) return ASI_ERR_INVALID_ARG;
+    if (pl->fast_wgrad && pl->wgrad_vec4 && (reinterpret_cast<uintptr_t>(dY[i]) & (pl->bf16 ? 7u : 15u))) return ASI_ERR_INVALID_ARG;
   }
   std::vector<char> done(n, 0);
   std::vector<std::vector<int>> chains;
@@ -1090,7 +1110,7 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
   if (s != ASI_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
-  if (pl->fast_compress && !pl->bf16 && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
+  if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
   ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
   int64_t off = 0;
   for (int m = 0; m < pl->nd; ++m) {
@@ -1119,7 +1139,7 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   float* omega = reinterpret_cast<float*>(w + align_up(pl->compress_ws, 256));
-  if (pl->fast_compress && !pl->bf16 && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
+  if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
   ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
   for (int m = 0; m < pl->nd; ++m) {               // one mode's Omega at a time, in the same scratch
     ASI_CUDA(launch_fill_gaussian(seed, (uint32_t)m, pl->mv[m].Q * pl->r[m], omega, st));

@@ -29,11 +29,6 @@ template <> struct RawCols<float, 4> {
   __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float4*>(p)); }
   __device__ __forceinline__ void get(float (&x)[4]) const { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
 };
-template <> struct RawCols<float, 2> {
-  float2 v;
-  __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float2*>(p)); }
-  __device__ __forceinline__ void get(float (&x)[2]) const { x[0] = v.x; x[1] = v.y; }
-};
 template <> struct RawCols<__nv_bfloat16, 4> {
   uint2 v;
   __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint2*>(p)); }
@@ -46,9 +41,6 @@ template <> struct RawCols<__nv_bfloat16, 4> {
 template <int CW> __device__ __forceinline__ void store_cols(float* dst, const float (&v)[CW]);
 template <> __device__ __forceinline__ void store_cols<4>(float* dst, const float (&v)[4]) {
   *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-}
-template <> __device__ __forceinline__ void store_cols<2>(float* dst, const float (&v)[2]) {
-  *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
 }
 
 }  // namespace

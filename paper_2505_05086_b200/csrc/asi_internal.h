@@ -116,7 +116,10 @@ struct SmPass1Args {
   int* status;                  // status word (int 0) and completion counters (ints 16..255) of the workspace
   int64_t u_off[ASI_MAX_MODES];
   int r[ASI_MAX_MODES];
-  int B, C, n_tiles_b;
+  int B, C, H, W, n_tiles_b;    // n_tiles_b: role-B CTAs (column tiles of all samples)
+  int cs, cc, pitch, off_u2;    // role C: CTAs per sample, channels per CTA, floats per channel, start of U_2 in shared memory
+  int vec4;                     // columns may be read four at a time (C H W % 4 == 0, 16-byte aligned base)
+  int bulk;                     // role C's tile comes by bulk copies (fp32, vec4)
   unsigned long long wait_ns;   // limit of the bounded wait on the bulk-copy barrier
   int stall_copy;               // test hook: the producer arms the barrier but issues no copy (the wait must expire)
 };
@@ -144,7 +147,7 @@ struct SmCoreArgs {
   const double* Pred[ASI_MAX_MODES];   // P_m [a][r] in fp64
   const double* Rf;                    // [4][kRfStride]: the Cholesky factors written by the reduction kernel
   float* U_new;
-  float* Tp;                    // [n_tiles][core_elems] per-tile partial cores
+  float* Tp;                    // [C][r1 r3 r4]: the activation contracted over all modes but the channels
   float* Tg;                    // [ceil(n_tiles / gs)][core_elems] per-group partial cores
   float* core;
   int* status;
@@ -153,7 +156,8 @@ struct SmCoreArgs {
   int gs;
   int64_t u_off[ASI_MAX_MODES];
   int r[ASI_MAX_MODES];
-  int B, C, n_tiles;
+  int B, C, H, W, tile_c, n_tiles;   // tile_c: channels per tile
+  int vec4;                     // as in SmPass1Args
 };
 struct SmWgradArgs {
   const float* core;
@@ -164,18 +168,19 @@ struct SmWgradArgs {
   int64_t u_off[ASI_MAX_MODES];
   int r[ASI_MAX_MODES];
   int B, C, Cout, H, W, Ho, Wo, kh, kw, sh, sw, ph, pw, groups, cpb;
-  int pj;                       // row pitch (floats) of the staged dY tile
-  int bulk;                     // 1: rows staged by 16-byte asynchronous copies (fp32, 16-byte aligned rows)
+  int vec4;                     // columns of dY may be read four at a time
   int ncl;                      // output channels expanded per round of term 5 (divides cpb)
   int bulk_store;               // 1: dW row blocks leave through the bulk-copy engine (16-byte sized and aligned)
 };
-size_t sm_pass1_smem(int S, int R, int B, int C);
-int sm_pass1_role_c_ctas(int S, int B);
-size_t sm_core_smem(int S, int R, int B);
-int sm_core_max_rows();
+size_t sm_pass1_smem(const SmPass1Args& p, int kind, int R);
+int sm_pass1_pitch(int HW);
+void sm_pass1_split(int HW, int C, int* cs, int* cc);
+int sm_pass1_off_u2(int R, int cc, int pitch);
+int sm_pass1_tiles_b(int64_t chw, bool vec4);
+int sm_core_tile_c(int HW, int C);
+size_t sm_core_smem(const SmCoreArgs& p, int R);
 size_t sm_wgrad_smem(const SmWgradArgs& p, int R);
-int sm_wgrad_pitch(int J);
-cudaError_t launch_sm_pass1(const SmPass1Args& p, int S, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_pass1(const SmPass1Args& p, int kind, int R, bool bf16, cudaStream_t st);
 // Tensor-core products of bf16 tensors (asi_tc_kernels.cu).  A factor enters as its stacked operand (three bf16 terms).
 size_t tc_operand_bytes(int64_t K, int n);
 int64_t tc_operand_ld(int64_t K);
@@ -205,13 +210,13 @@ struct TcCall {
 };
 cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st);
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st);
-cudaError_t launch_sm_core(const SmCoreArgs& p, int S, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, cudaStream_t st);
 cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t st);
 // the same kernels over several layers of one variant in one launch each (n <= sm_max_batch())
 int sm_max_batch();
-cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int S, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int kind, int R, bool bf16, cudaStream_t st);
 cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunks, int n, cudaStream_t st);
-cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int S, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, cudaStream_t st);
 cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, cudaStream_t st);
 
 // Benchmark timing aid (asi_profile_begin / asi_profile_end).
@@ -440,7 +445,8 @@ struct asi_plan {
   int launches_compress, launches_wgrad;
 
   // fused small-map path
-  bool fast_compress, fast_wgrad, wgrad_bulk;
+  bool fast_compress, fast_wgrad;
+  bool fast_vec4, wgrad_vec4;      // columns of the activation / of dY come in whole groups of four
   bool small_rank;                 // every rank <= 8: partials are reduced by the parallel fp64 kernel
   bool fiber[ASI_MAX_MODES];       // mode handled by the single-pass fiber kernel
   int fiber_grid[ASI_MAX_MODES];
@@ -448,5 +454,6 @@ struct asi_plan {
   int plane_grid;
   bool fiber2[ASI_MAX_MODES];      // ... by its register-tiled successor (ranks <= 4, 16-byte aligned rows)
   bool plane2;                     // 28 x 28 and 56 x 56 planes, ranks <= 4
-  int fast_S, fast_R, n_tiles_b, cpb, wgrad_ncl, fold_gs;
+  int fast_kind;                   // 7, 14: modes 3 and 4 as Gram matrices of such square maps; 0: any map of at most 256 positions
+  int fast_R, n_tiles_b, fast_cs, fast_cc, core_tile_c, n_tiles_core, cpb, wgrad_ncl, fold_gs;
 };

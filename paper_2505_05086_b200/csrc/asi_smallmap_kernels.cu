@@ -1,22 +1,18 @@
-// Fused kernels for conv layers with small square feature maps (S x S, S in {7, 14, 16}) and
-// ranks <= 8 -- the shapes of the ResNet / MobileNet tails.  One compress call is three launches:
+// Fused kernels for conv layers with small feature maps (H W <= 256, ranks <= 8) -- the shapes of the ResNet /
+// MobileNet tails.  One compress call is three launches:
 //
-//   k_sm_pass1  : forms every P_m = A_m (A_m^T U_m^prev) (Algorithm 1) tile-locally, so no V_m ever
-//                 reaches global memory.  CTAs of role B hold a tile [all B x J contiguous (c,h,w)]
-//                 that contains whole mode-1/3/4 fibers (one half of the CTA iterates mode 1 while the
-//                 other half does modes 3 and 4); CTAs of role C hold one sample [all C x HW] that
-//                 contains whole mode-2 fibers.  fp32 tiles are staged in shared memory by the
-//                 bulk-copy engine (cp.async.bulk + mbarrier), one row or chunk per copy; the
-//                 activation comes from HBM once, the other role's traversal is served by L2.
+//   k_sm_pass1  : forms every P_m = A_m (A_m^T U_m^prev) (Algorithm 1) tile-locally, so no V_m ever reaches global
+//                 memory; the activation is read once from HBM and once more from L2 (mode 1 needs whole batches,
+//                 modes 2-4 whole samples);
 //   k_sm_reduce : fixed-order fp64 reduction of the per-tile partials of every P_m and per-chunk
-//                 shares of the Gram matrices G_m = P_m^T P_m;
-//   k_sm_core   : every CTA finishes Orthogonalize for the factor rows it needs while its tile is in
-//                 flight (Cholesky G_m = R^T R, U_m = P_m R^{-1}: the Gram-Schmidt basis), then
-//                 contracts its tile [all B x J] with U_1..U_4; the last CTA sums the per-tile cores.
+//                 shares of the Gram matrices G_m = P_m^T P_m, factored once per mode;
+//   k_sm_core   : every CTA finishes Orthogonalize for the factor rows it needs (U_m = P_m R^{-1}: the Gram-Schmidt
+//                 basis), then contracts its channels with U_1, U_3, U_4; the last CTAs contract the channels.
 //
 // and the whole compressed weight gradient is one kernel, k_sm_wgrad (terms 1-5 of C_ASI).
 // Every wait on an mbarrier is bounded (about one second); on expiry the CTA records
 // ASI_ERR_TIMEOUT in the status word and returns.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -27,32 +23,9 @@ namespace asi {
 
 namespace {
 
-constexpr int kNT = 512;             // threads per CTA of the tile kernels
-constexpr int kNG = 256;             // threads of one half (warp-specialised phases)
+constexpr int kNT = 512;             // threads per CTA of k_sm_wgrad
 constexpr int kRedNT = 256;          // threads per CTA of the partial-reduction kernel
 
-__host__ __device__ constexpr int pitch4(int J) {      // >= J, multiple of 4, == 4 (mod 32)
-  int p = (J + 3) / 4 * 4;
-  while (p % 32 != 4) p += 4;
-  return p;
-}
-
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-template <typename TX>
-__device__ __forceinline__ float4 ld4(const TX* p);
-template <>
-__device__ __forceinline__ float4 ld4<float>(const float* p) {
-  return *reinterpret_cast<const float4*>(p);
-}
-template <>
-__device__ __forceinline__ float4 ld4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 raw = *reinterpret_cast<const uint2*>(p);
-  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
-  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
-  return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
-}
 
 // ---- bulk-copy engine (TMA, untiled form) and mbarrier ------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -152,32 +125,9 @@ __device__ __forceinline__ void fac_issue_padded(const float* __restrict__ src, 
     cp_async4(dst + idx, src + (j < r ? k * r + j : 0), j < r ? 4 : 0);
   }
 }
-__device__ __forceinline__ void fac_issue_flat(const float* __restrict__ src, float* dst, int n) {
-#pragma unroll 1
-  for (int idx = threadIdx.x; idx < n; idx += kNT) cp_async4(dst + idx, src + idx, 4);
-}
 __device__ __forceinline__ void fac_wait() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// waits until at most N of this thread's committed groups are still in flight
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-// Starts the copy of `rows` fp32 rows of J values (J a multiple of 4, both sides 16-byte aligned): row i
-// from src + i*src_stride to dst + i*PJ, 16 bytes per cp.async, one row per warp at a time.  (One bulk
-// copy per row would leave the issuing warp busy for ~60 cycles per row: the tile of a 64-sample
-// batch would arrive ~2 us later.)
-__device__ __forceinline__ void stage_rows_async(float* dst, const float* __restrict__ src, int rows, int J,
-                                                 int64_t src_stride, int PJ) {
-  const int lane = threadIdx.x & 31, nv = J >> 2;
-  for (int i = threadIdx.x >> 5; i < rows; i += kNT / 32) {
-    const float* s = src + i * src_stride;
-    float* d = dst + i * PJ;
-    for (int v = lane; v < nv; v += 32)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(d + 4 * v)), "l"(s + 4 * v) : "memory");
-  }
-}
-
 template <int R>
 __device__ __forceinline__ void fma_row(float (&acc)[R], float x, const float* __restrict__ u) {
 #pragma unroll
@@ -202,10 +152,6 @@ struct FDiv {
     r = n - q * d;
   }
 };
-
-__device__ __forceinline__ void bar_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 // Sum of N per-lane values over the 32 lanes of a warp by recursive halving: every step each lane
 // hands half of its values to its partner, so the whole reduction costs N-N/32 shuffles.  On return
@@ -236,114 +182,6 @@ __device__ __forceinline__ int scatter_base(int lane) {
          ((lane >> 1) & 1) * (N / 16) + (lane & 1) * (N / 32);
 }
 
-// Number of interleaved sample groups project_batch uses for a tile of J columns on nthr threads.
-__host__ __device__ constexpr int batch_groups(int nthr, int J) {
-  const int items = J / 2;
-  int nh = nthr / items;
-  return nh < 1 ? 1 : (nh > 4 ? 4 : nh);
-}
-
-// out[j][0..R) = sum_b Xs[b*PJ + j] * Us[b*R + ..] for j < J: the mode-1 contraction of a staged tile
-// [B x J].  Runs on `nthr` threads (t = 0..nthr-1) that synchronise on named barrier `bar`.  A thread
-// owns two neighbouring columns (one 8-byte shared load per sample) and the samples b == h (mod NH);
-// the NH partial sums meet in `part` ([NH][J][R]) in a fixed order.
-template <int R>
-__device__ __forceinline__ void project_batch(const float* __restrict__ Xs, int PJ,
-                                              const float* __restrict__ Us, int B, int J,
-                                              float* __restrict__ part, float* __restrict__ out, int t,
-                                              int nthr, int bar) {
-  const int NH = batch_groups(nthr, J);
-  const int J2 = J >> 1;                             // J is even
-  const FDiv dJ2(J2);
-#pragma unroll 1
-  for (int it = t; it < NH * J2; it += nthr) {
-    int h, jp;
-    dJ2.divmod(it, h, jp);
-    float a0[R], a1[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) a0[q] = a1[q] = 0.f;
-#pragma unroll 4
-    for (int b = h; b < B; b += NH) {
-      const float2 x = *reinterpret_cast<const float2*>(Xs + b * PJ + 2 * jp);
-      fma_row<R>(a0, x.x, Us + b * R);
-      fma_row<R>(a1, x.y, Us + b * R);
-    }
-    float* dst = (NH > 1 ? part + h * J * R : out) + 2 * jp * R;
-#pragma unroll
-    for (int q = 0; q < R; q += 4) {
-      *reinterpret_cast<float4*>(dst + q) = make_float4(a0[q], a0[q + 1], a0[q + 2], a0[q + 3]);
-      *reinterpret_cast<float4*>(dst + R + q) = make_float4(a1[q], a1[q + 1], a1[q + 2], a1[q + 3]);
-    }
-  }
-  if (NH > 1) {
-    bar_sync(bar, nthr);
-#pragma unroll 1
-    for (int idx = t; idx < J * R; idx += nthr) {
-      float s = 0.f;
-      for (int h = 0; h < NH; ++h) s += part[h * J * R + idx];
-      out[idx] = s;
-    }
-  }
-  bar_sync(bar, nthr);
-}
-
-// V[hw][:] = sum_c Xs[c*PC + hw] * Us[c][:] for a staged block Xs [C][HWC] of one sample (the mode-2
-// projection of HWC positions).  Thread (g, hw) sums the channels c = g (mod G); group 0 writes V
-// itself, groups 1..G-1 write Vp ([G-1][HWC][R]; may alias Us: it is written only after every thread
-// has finished reading Us) and the sums meet in a fixed order.  All kNT threads call it.
-template <int HWC, int PC, int R>
-__device__ __forceinline__ void project_channels(const float* __restrict__ Xs, const float* Us, float* Vp,
-                                                 float* V, int C) {
-  constexpr int G = kNT / HWC;
-  const int tid = threadIdx.x;
-  float acc[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) acc[j] = 0.f;
-  const int g = tid / HWC, hw = tid - g * HWC;
-  if (g < G) {
-#pragma unroll 4
-    for (int c = g; c < C; c += G) fma_row<R>(acc, Xs[c * PC + hw], Us + c * R);
-  }
-  if (G > 1) __syncthreads();
-  if (g < G) {
-    float* dst = (g == 0 ? V : Vp + (g - 1) * HWC * R) + hw * R;
-#pragma unroll
-    for (int j = 0; j < R; j += 4)
-      *reinterpret_cast<float4*>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
-  }
-  __syncthreads();
-  if (G > 1) {
-    for (int idx = tid; idx < HWC * R; idx += kNT) {
-      float s = V[idx];
-#pragma unroll
-      for (int gg = 0; gg < G - 1; ++gg) s += Vp[gg * HWC * R + idx];
-      V[idx] = s;
-    }
-    __syncthreads();
-  }
-}
-
-// Stages one tile [B x J] (row b at src + b*sample_stride) as fp32 rows of pitch PJ.
-template <typename TX>
-__device__ __forceinline__ void stage_tile_begin(const TX* __restrict__ src, int64_t sample_stride, float* Xs,
-                                                 int B, int J, int PJ) {
-  if constexpr (std::is_same<TX, float>::value) {
-    stage_rows_async(Xs, src, B, J, sample_stride, PJ);
-  } else {
-    const int J4 = J / 4;
-    for (int idx = threadIdx.x; idx < B * J4; idx += kNT) {
-      const int b = idx / J4, v = idx - b * J4;
-      *reinterpret_cast<float4*>(Xs + b * PJ + 4 * v) = ld4<TX>(src + b * sample_stride + 4 * v);
-    }
-  }
-}
-
-// Role C of the first pass takes the positions of a sample in NQ parts.  S = 7: the whole map.  Larger
-// maps: four parts that start on 16-byte boundaries -- 14 x 14 splits its 49 float4 per channel as
-// 13 + 12 + 12 + 12 (parts 1..3 carry four zero columns), 16 x 16 as 4 x 16.
-__host__ __device__ constexpr int role_c_hwc(int S) { return S == 7 ? 49 : (S == 14 ? 52 : S * S / 4); }
-__host__ __device__ constexpr int role_c_pitch(int S) { return S == 7 ? 49 : pitch4(role_c_hwc(S)); }
-
 __host__ __device__ constexpr int tri_index(int S, int k, int k2) {   // k <= k2 < S, row-major upper triangle
   return k * S - k * (k - 1) / 2 + (k2 - k);
 }
@@ -354,8 +192,7 @@ __host__ __device__ constexpr int tri_index(int S, int k, int k2) {   // k <= k2
 // A unit is a quarter of a plane (fibers == part mod 4), so the lanes of a warp hit 32 banks; this
 // thread takes units u0, u0 + ustride, ...  es = step between the elements of a fiber, cs = step
 // between neighbouring fibers (mode 3: 14, 1; mode 4: 1, 14).
-template <int PJ>
-__device__ __forceinline__ void gram14_accumulate(const float* __restrict__ Xs, int nunits, int u0, int ustride,
+__device__ __forceinline__ void gram14_accumulate(const float* __restrict__ Xs, int PJ, int nunits, int u0, int ustride,
                                                   int role, int es, int cs, float (&acc)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) acc[i] = 0.f;
@@ -410,271 +247,473 @@ __device__ __forceinline__ void gram14_slot(int o, int& rl, int& e) {
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
-// k_sm_pass1
+// k_sm_pass1: every P_m = A_m (A_m^T U_m^prev) in one launch, 256 threads per CTA.
+//
+// Role B (mode 1), one CTA per 128 neighbouring columns (c, h, w): lane = four columns, warp w = the samples b == w
+// (mod 8).  The activation goes straight from memory to registers -- a warp reads 512 contiguous bytes per sample --
+// V_1 of the columns meets in shared memory, and at ranks <= 4 the same registers feed the expansion (no tile is
+// staged, so nothing but the registers limits how many CTAs share an SM).
+//
+// Role C (modes 2, 3, 4), a cluster of `cs` CTAs per sample, each with cc channels of it in shared memory (one bulk
+// copy): V_2 is the sum of the CTAs' shares through distributed shared memory, P_2 of the CTA's own channels follows
+// from its tile; modes 3 and 4 come from the same planes -- as Gram matrices A_m A_m^T on 7 x 7 and 14 x 14 maps
+// (S + 1 multiply-adds per element against 4 r; P_m = G_m U_m^prev is formed in k_sm_reduce), on other maps as the
+// two products with a lane per row and per column of a plane.
+// The split of a sample over a cluster is what lets two to four CTAs share an SM: with the whole sample and the whole
+// batch of a tile in shared memory (up to 204 KB) one CTA per SM waited for its own copy.
 // ---------------------------------------------------------------------------------------------
-template <int S, int R, typename TX>
-__device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid) {
-  constexpr bool kBulk = std::is_same<TX, float>::value;
-  constexpr bool kGram = (S == 7);                   // modes 3, 4 as Gram matrices A_m A_m^T (7 x 7)
-  constexpr bool kGram14 = (S == 14);                // ... as 14 x 14 Gram matrices in four 7 x 7 blocks
-  constexpr int HW = S * S;
-  constexpr int CC = (S == 7) ? 4 : 1;               // channels per role-B tile
-  constexpr int J = CC * HW;                         // contiguous elements per sample in a tile
-  constexpr int PJ = pitch4(J);                      // row pitch == 4 (mod 32): conflict-free (b, j) reads
-  constexpr int NH1 = batch_groups(kNG, J);
-  extern __shared__ __align__(128) float smem[];
+constexpr int kPT = 256;             // threads per CTA of k_sm_pass1 and k_sm_core
+
+template <typename TX, int VW> struct RawCol;                 // VW neighbouring values as they lie in memory
+template <> struct RawCol<float, 4> {
+  float4 v;
+  __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float4*>(p)); }
+  __device__ __forceinline__ void get(float (&x)[4]) const { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
+};
+template <> struct RawCol<float, 1> {
+  float v;
+  __device__ __forceinline__ void load(const float* p) { v = __ldg(p); }
+  __device__ __forceinline__ void get(float (&x)[1]) const { x[0] = v; }
+};
+template <> struct RawCol<__nv_bfloat16, 4> {
+  uint2 v;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint2*>(p)); }
+  __device__ __forceinline__ void get(float (&x)[4]) const {
+    x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xffff0000u);
+    x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xffff0000u);
+  }
+};
+template <> struct RawCol<__nv_bfloat16, 1> {
+  __nv_bfloat16 v;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = *p; }
+  __device__ __forceinline__ void get(float (&x)[1]) const { x[0] = __bfloat162float(v); }
+};
+
+template <int R, int VW, typename TX>
+__device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, float* smem) {
+  constexpr int JT = 32 * VW, NBH = 16, BPG = 32 / R;         // samples per thread and chunk; samples per reduction
+  constexpr bool kHold = (R == 4);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int B = p.B, r1 = p.r[0];
+  const int64_t chw = (int64_t)p.C * p.H * p.W;
+  float* U1s = smem;                                 // [B][R]
+  float* part = U1s + ((B * R + 3) & ~3);            // [8][JT][R]
+  float* V1s = part + 8 * JT * R;                    // [JT][R]
+  for (int idx = tid; idx < B * R; idx += kPT) {
+    const int k = idx / R, j = idx % R;
+    cp_async4(U1s + idx, p.U_prev + p.u_off[0] + (j < r1 ? k * r1 + j : 0), j < r1 ? 4 : 0);
+  }
+  const int64_t col = (int64_t)tile * JT + VW * lane;
+  const bool con = col < chw;
+  const TX* A = reinterpret_cast<const TX*>(p.act) + (con ? col : 0);
+  RawCol<TX, VW> x[NBH];
+  float v[VW][R];
+#pragma unroll
+  for (int c = 0; c < VW; ++c)
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[c][j] = 0.f;
+  bool waited = false;
+  for (int bb = 0; bb < B; bb += 8 * NBH) {
+#pragma unroll
+    for (int t = 0; t < NBH; ++t) {
+      const int b = bb + warp + 8 * t;
+      x[t].load(A + (int64_t)(b < B ? b : B - 1) * chw);
+    }
+    if (!waited) {
+      fac_wait();
+      __syncthreads();
+      waited = true;
+    }
+#pragma unroll
+    for (int t = 0; t < NBH; ++t) {
+      const int b = bb + warp + 8 * t;
+      if (b < B) {                                   // warp-uniform
+        float xs[VW];
+        x[t].get(xs);
+#pragma unroll
+        for (int c = 0; c < VW; ++c) fma_row<R>(v[c], xs[c], U1s + b * R);
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < VW; ++c)
+#pragma unroll
+    for (int j = 0; j < R; j += 4)
+      *reinterpret_cast<float4*>(part + (warp * JT + VW * lane + c) * R + j) = make_float4(v[c][j], v[c][j + 1], v[c][j + 2], v[c][j + 3]);
+  __syncthreads();
+  for (int idx = tid; idx < JT * R; idx += kPT) {
+    float s = part[idx];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w * JT * R + idx];
+    V1s[idx] = s;
+  }
+  __syncthreads();
+  pdl_launch_dependents();
+#pragma unroll
+  for (int c = 0; c < VW; ++c)
+#pragma unroll
+    for (int j = 0; j < R; j += 4) {
+      const float4 s = con ? *reinterpret_cast<const float4*>(V1s + (VW * lane + c) * R + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[c][j] = s.x; v[c][j + 1] = s.y; v[c][j + 2] = s.z; v[c][j + 3] = s.w;
+    }
+  // P1[b,:] = sum over the tile's columns of X[b][col] V1[col,:]: BPG samples meet in one butterfly of 32 values
+  float* P1 = p.Pp[0] + (int64_t)tile * B * r1;
+  const bool held = kHold && B <= 8 * NBH;
+#pragma unroll 1
+  for (int bb = 0; bb < B; bb += 8 * NBH) {
+    if (!held) {
+#pragma unroll
+      for (int t = 0; t < NBH; ++t) {
+        const int b = bb + warp + 8 * t;
+        x[t].load(A + (int64_t)(b < B ? b : B - 1) * chw);
+      }
+    }
+#pragma unroll
+    for (int t0 = 0; t0 < NBH; t0 += BPG) {
+      if (bb + warp + 8 * t0 < B) {                  // warp-uniform
+        float val[32];
+#pragma unroll
+        for (int q = 0; q < BPG; ++q) {
+          float xs[VW];
+          x[t0 + q].get(xs);
+#pragma unroll
+          for (int j = 0; j < R; ++j) {
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < VW; ++c) s = fmaf(xs[c], v[c][j], s);
+            val[q * R + j] = s;
+          }
+        }
+        warp_reduce_scatter<32>(val, lane);
+        const int e = scatter_base<32>(lane), b = bb + warp + 8 * (t0 + e / R), j = e % R;
+        if (b < B && j < r1) P1[b * r1 + j] = val[0];
+      }
+    }
+  }
+}
+
+// modes 3 and 4 of nc planes [H][W] in shared memory (pitch P): P_m = A_m (A_m^T U_m), lane = (plane of the warp's
+// group, row or column).  Rows are read rotated by the lane so that an even width does not fold them onto a few banks.
+template <int R>
+__device__ __forceinline__ void planes_modes34(const float* Xs, int P, int nc, int H, int W, const float* U3s, const float* U4s,
+                                               float* Vw, float* red, float* P3, float* P4, int r3, int r4) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int L = H > W ? H : W, G = 32 / L;
+  const int g = lane / L, x = lane - g * L;
+  float* V = Vw + warp * 32 * R;                     // [32 lanes][R] of this warp
+  float a3[R], a4[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) a3[j] = a4[j] = 0.f;
+#pragma unroll 1
+  for (int p0 = warp * G; p0 < nc; p0 += 8 * G) {
+    const bool on = g < G && p0 + g < nc;
+    const float* Xp = Xs + (on ? p0 + g : 0) * P;
+    float v[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[j] = 0.f;
+    if (on && x < W) {
+#pragma unroll 4
+      for (int h = 0; h < H; ++h) fma_row<R>(v, Xp[h * W + x], U3s + h * R);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < R; j += 4) *reinterpret_cast<float4*>(V + lane * R + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[j] = 0.f;
+    if (on && x < H) {
+      int w = x < W ? x : 0;
+#pragma unroll 4
+      for (int k = 0; k < W; ++k) {
+        const float xv = Xp[x * W + w];
+        fma_row<R>(a3, xv, V + (g * L + w) * R);
+        fma_row<R>(v, xv, U4s + w * R);
+        if (++w == W) w = 0;
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < R; j += 4) *reinterpret_cast<float4*>(V + lane * R + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    __syncwarp();
+    if (on && x < W) {
+#pragma unroll 4
+      for (int h = 0; h < H; ++h) fma_row<R>(a4, Xp[h * W + x], V + (g * L + h) * R);
+    }
+  }
+  // [8 warps][32 lanes][2 R]: the planes' shares meet in (warp, group) order
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    red[(warp * 32 + lane) * 2 * R + j] = a3[j];
+    red[(warp * 32 + lane) * 2 * R + R + j] = a4[j];
+  }
+  __syncthreads();
+  for (int idx = tid; idx < (H + W) * R; idx += kPT) {
+    const bool m4 = idx >= H * R;
+    const int e = m4 ? idx - H * R : idx, k = e / R, j = e % R;
+    float s = 0.f;
+    for (int w = 0; w < 8; ++w)
+      for (int q = 0; q < G; ++q) s += red[(w * 32 + q * L + k) * 2 * R + (m4 ? R : 0) + j];
+    if (!m4 && j < r3) P3[k * r3 + j] = s;
+    if (m4 && j < r4) P4[k * r4 + j] = s;
+  }
+}
+
+template <int KIND, int R, typename TX>
+__device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, float* smem) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ int s_flag;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const TX* __restrict__ A = reinterpret_cast<const TX*>(p.act);
-  const int B = p.B, C = p.C;
-
-  if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
-  pdl_launch_dependents();
-
-  constexpr int kNQ = (S == 7) ? 1 : 4;             // role-C CTAs per sample
-  if (bid >= B * kNQ) {
-    // ---------------- role B: modes 1, 3, 4 on tile [B x J] ----------------
-    const int tile = bid - B * kNQ;
-    float* Xs = smem;                                // [B][PJ]
-    float* U1s = Xs + B * PJ;                        // [B][R]
-    float* U3s = U1s + B * R;                        // [S][R]
-    float* U4s = U3s + S * R;                        // [S][R]
-    float* V1s = U4s + S * R;                        // [J][R]
-    float* part = V1s + J * R;                       // [NH1][J][R] (NH1 > 1 only)
-    float* red = part + (NH1 > 1 ? NH1 : 0) * J * R; // [8][32], S = 14: [8 + 16][32]
-    fac_issue_padded<R>(p.U_prev + p.u_off[0], U1s, B, p.r[0]);
-    if constexpr (!kGram && !kGram14) {
-      fac_issue_padded<R>(p.U_prev + p.u_off[2], U3s, S, p.r[2]);
-      fac_issue_padded<R>(p.U_prev + p.u_off[3], U4s, S, p.r[3]);
+  namespace cg = cooperative_groups;
+  const int C = p.C, H = KIND ? KIND : p.H, W = KIND ? KIND : p.W, HW = H * W, P = p.pitch, cs = p.cs;
+  const int b = bid / cs, rank = bid - b * cs;
+  const int c0 = rank * p.cc, nc = (C - c0 < p.cc) ? (C > c0 ? C - c0 : 0) : p.cc;
+  const int r2 = p.r[1];
+  float* Xs = smem;                                  // [cc][P]
+  float* U2s = smem + p.off_u2;                      // [cc][R]
+  float* V2l = U2s + p.cc * R;                       // [HW][R]: this CTA's share of V_2
+  float* V2s = V2l + HW * R;                         // [HW][R]
+  float* Vp = V2s + HW * R;                          // [G][HW][R], G = 256 / HW
+  float* U3s = Vp + (kPT / HW) * HW * R;             // KIND 0: [H][R], [W][R], [8][32][R]
+  float* red = Xs;                                   // free once every thread is done with the tile
+  const TX* A = reinterpret_cast<const TX*>(p.act) + ((int64_t)b * C + c0) * HW;
+  const bool bulk = std::is_same<TX, float>::value && p.bulk;
+  if (bulk) {
+    const char* src = reinterpret_cast<const char*>(A);
+    if (P == HW) {
+      stage_block(&s_bar, reinterpret_cast<char*>(Xs), src, (uint32_t)(nc * HW) * 4u, p.stall_copy != 0);
+    } else if (warp == 0) {                          // one row per channel, padded pitch
+      if (lane == 0) {
+        mbar_init(&s_bar, 1);
+        mbar_expect_tx(&s_bar, (uint32_t)(nc * HW) * 4u);
+      }
+      __syncwarp();
+      for (int c = lane; c < nc && !p.stall_copy; c += 32) bulk_g2s(Xs + c * P, src + (int64_t)c * HW * 4, (uint32_t)HW * 4u, &s_bar);
     }
-    stage_tile_begin<TX>(A + (int64_t)tile * J, (int64_t)C * HW, Xs, B, J, PJ);
-    fac_wait();
-    __syncthreads();
-    const int t = tid & (kNG - 1), wg = t >> 5;
-    if (tid < kNG) {
-      // ---- half 0: mode 1.  V[j,:] = sum_b X[b,j] U1[b,:], then P1[b,:] = sum_j X[b,j] V[j,:]
-      project_batch<R>(Xs, PJ, U1s, B, J, part, V1s, t, kNG, 1);
-      float* P1 = p.Pp[0] + (int64_t)tile * B * p.r[0];
-      const int bl = lane >> 2, jl = lane & 3;       // a warp covers 8 samples x 4 column phases
-      for (int b0 = wg * 8; b0 < B; b0 += 64) {
-        const int b = b0 + bl;
-        float acc[R];
-#pragma unroll
-        for (int q = 0; q < R; ++q) acc[q] = 0.f;
-#pragma unroll 7
-        for (int jj = jl; jj < J; jj += 4) fma_row<R>(acc, Xs[b * PJ + jj], V1s + jj * R);
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-          acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
-          acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 2);
-        }
-        if (jl == 0) {
-#pragma unroll
-          for (int q = 0; q < R; ++q)
-            if (q < p.r[0]) P1[b * p.r[0] + q] = acc[q];
-        }
+  }
+  for (int idx = tid; idx < nc * R; idx += kPT) {
+    const int k = idx / R, j = idx % R;
+    cp_async4(U2s + idx, p.U_prev + p.u_off[1] + (j < r2 ? (c0 + k) * r2 + j : 0), j < r2 ? 4 : 0);
+  }
+  if (KIND == 0)
+    for (int idx = tid; idx < (H + W) * R; idx += kPT) {
+      const int k = idx / R, j = idx % R, m = k < H ? 2 : 3, kk = k < H ? k : k - H;
+      cp_async4(U3s + idx, p.U_prev + p.u_off[m] + (j < p.r[m] ? kk * p.r[m] + j : 0), j < p.r[m] ? 4 : 0);
+    }
+  if (!bulk) {
+    if constexpr (std::is_same<TX, float>::value) {
+      const FDiv dHW(HW);
+      for (int idx = tid; idx < nc * HW; idx += kPT) {
+        int c, q;
+        dHW.divmod(idx, c, q);
+        cp_async4(Xs + c * P + q, reinterpret_cast<const float*>(A) + idx, 4);
       }
-    } else if constexpr (kGram) {
-      // ---- half 1, S = 7: G_m = A_m A_m^T for m = 3, 4, one plane (b, c) per thread at a time; the
-      // 32 lanes of a warp touch 32 different banks.  P_m = G_m U_m^prev follows in k_sm_reduce.
-      constexpr int NACC = 32;
-      static_assert(S * (S + 1) / 2 <= NACC, "upper triangle of the Gram matrix");
-      const int nplanes = B * CC;
-#pragma unroll 1
-      for (int mode = 2; mode <= 3; ++mode) {
-        const int es = (mode == 2) ? S : 1;          // step between the elements of a fiber
-        const int cs = (mode == 2) ? 1 : S;          // step between neighbouring fibers
-        float* Gm = p.Pp[mode] + (int64_t)tile * HW;
-        float acc[NACC];
+    } else if (p.vec4) {
+      const FDiv dV(HW % 4 == 0 ? HW / 4 : 1 << 20);
+      for (int i0 = tid; i0 < nc * HW / 4; i0 += 4 * kPT) {
+        uint2 raw[4];
 #pragma unroll
-        for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
-        for (int pl = t; pl < nplanes; pl += kNG) {
-          const int b = pl / CC, cl = pl % CC;
-          const float* base = Xs + b * PJ + cl * HW;
-#pragma unroll 1
-          for (int col = 0; col < S; ++col) {
-            const float* colp = base + col * cs;
-            float x[S];
+        for (int u = 0; u < 4; ++u) raw[u] = __ldg(reinterpret_cast<const uint2*>(A) + (i0 + u * kPT < nc * HW / 4 ? i0 + u * kPT : 0));
 #pragma unroll
-            for (int k = 0; k < S; ++k) x[k] = colp[k * es];
-#pragma unroll
-            for (int k = 0; k < S; ++k)
-#pragma unroll
-              for (int k2 = k; k2 < S; ++k2) acc[tri_index(S, k, k2)] = fmaf(x[k], x[k2], acc[tri_index(S, k, k2)]);
-          }
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * kPT;
+          if (i >= nc * HW / 4) break;
+          int c = 0, q = i;
+          if (P != HW) dV.divmod(i, c, q);
+          *reinterpret_cast<float4*>(Xs + c * P + 4 * q) =
+              make_float4(__uint_as_float(raw[u].x << 16), __uint_as_float(raw[u].x & 0xffff0000u),
+                          __uint_as_float(raw[u].y << 16), __uint_as_float(raw[u].y & 0xffff0000u));
         }
-        warp_reduce_scatter<NACC>(acc, lane);
-        red[wg * 32 + scatter_base<NACC>(lane)] = acc[0];
-        bar_sync(2, kNG);
-        for (int o = t; o < HW; o += kNG) {
-          const int k = o / S, k2 = o % S;
-          const int e = (k <= k2) ? tri_index(S, k, k2) : tri_index(S, k2, k);
-          float s = 0.f;
-#pragma unroll
-          for (int w = 0; w < 8; ++w) s += red[w * 32 + e];
-          Gm[o] = s;
-        }
-        bar_sync(2, kNG);
-      }
-    } else if constexpr (kGram14) {
-      // ---- half 1, S = 14: G_3 = A_3 A_3^T (see gram14_accumulate); G_4 follows on all sixteen warps
-      const int role = wg & 3;
-      float* Gm = p.Pp[2] + (int64_t)tile * HW;
-      float acc[32];
-      gram14_accumulate<PJ>(Xs, B * 4, (wg >> 2) * 32 + lane, 64, role, S, 1, acc);
-      warp_reduce_scatter<32>(acc, lane);
-      red[wg * 32 + scatter_base<32>(lane)] = acc[0];
-      bar_sync(2, kNG);
-      for (int o = t; o < HW; o += kNG) {
-        int rl, e;
-        gram14_slot(o, rl, e);
-        Gm[o] = red[rl * 32 + e] + red[(rl + 4) * 32 + e];
       }
     } else {
-      // ---- half 1, other sizes: P_m = A_m (A_m^T U_m^prev) for m = 3, 4.  A unit is a quarter of a plane
-      // (columns == part mod 4); unit -> thread so that the 32 lanes of a warp touch 32 different
-      // banks.  Each thread owns 2 columns of the factor; warp w serves column pair w mod JH.
-      constexpr int TPP = 4, JT = 2, JH = R / JT, NACC = 32;
-      static_assert(S * JT <= NACC, "accumulators of one thread");
-      const int jh = wg % JH;
-      const int u0 = (wg / JH) * 32 + lane;
-      const int nunits = B * CC * TPP;
-#pragma unroll 1
-      for (int mode = 2; mode <= 3; ++mode) {
-        const float* Us = ((mode == 2) ? U3s : U4s) + jh * JT;
-        const int es = (mode == 2) ? S : 1;
-        const int cs = (mode == 2) ? 1 : S;
-        const int rm = p.r[mode];
-        float* Pm = p.Pp[mode] + (int64_t)tile * S * rm;
-        float acc[NACC];
-#pragma unroll
-        for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
-        for (int un = u0; un < nunits; un += kNG / JH) {
-          const int pl = un / TPP, part_ = un % TPP;
-          const int b = pl / CC, cl = pl % CC;
-          const float* base = Xs + b * PJ + cl * HW;
-#pragma unroll 1
-          for (int col = part_; col < S; col += TPP) {
-            const float* colp = base + col * cs;
-            float x[S], v0 = 0.f, v1 = 0.f;
-#pragma unroll
-            for (int k = 0; k < S; ++k) {
-              x[k] = colp[k * es];
-              const float2 u = *reinterpret_cast<const float2*>(Us + k * R);
-              v0 = fmaf(x[k], u.x, v0);
-              v1 = fmaf(x[k], u.y, v1);
-            }
-#pragma unroll
-            for (int k = 0; k < S; ++k) {
-              acc[2 * k] = fmaf(x[k], v0, acc[2 * k]);
-              acc[2 * k + 1] = fmaf(x[k], v1, acc[2 * k + 1]);
-            }
-          }
-        }
-        warp_reduce_scatter<NACC>(acc, lane);
-        red[wg * 32 + scatter_base<NACC>(lane)] = acc[0];
-        bar_sync(2, kNG);
-        for (int o = t; o < S * R; o += kNG) {
-          const int k = o / R, j = o % R;
-          const int e = k * JT + (j % JT);
-          float s = 0.f;
-          for (int w = j / JT; w < 8; w += JH) s += red[w * 32 + e];
-          if (j < rm) Pm[k * rm + j] = s;
-        }
-        bar_sync(2, kNG);
+      const FDiv dHW(HW);
+      for (int idx = tid; idx < nc * HW; idx += kPT) {
+        int c, q;
+        dHW.divmod(idx, c, q);
+        Xs[c * P + q] = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(A)[idx]);
       }
     }
-    if constexpr (kGram14) {
-      // ---- S = 14, G_4 = A_4 A_4^T: each half joins as it finishes its first job (mode 1 or G_3)
-      const int gw = tid >> 5, role = gw & 3;
-      float* red4 = red + 8 * 32;                    // [16][32]
-      float acc[32];
-      gram14_accumulate<PJ>(Xs, B * 4, (gw >> 2) * 32 + lane, 128, role, 1, S, acc);
-      warp_reduce_scatter<32>(acc, lane);
-      red4[gw * 32 + scatter_base<32>(lane)] = acc[0];
-      __syncthreads();
-      float* Gm = p.Pp[3] + (int64_t)tile * HW;
-      for (int o = tid; o < HW; o += kNT) {
-        int rl, e;
-        gram14_slot(o, rl, e);
-        Gm[o] = ((red4[rl * 32 + e] + red4[(rl + 4) * 32 + e]) + red4[(rl + 8) * 32 + e]) + red4[(rl + 12) * 32 + e];
-      }
-    }
-  } else {
-    // ---------------- role C: mode 2 on block [C x HWC] of one sample ----------------
-    // S = 7: the whole sample (contiguous, staged by the bulk-copy engine, odd row pitch for the
-    // row-per-thread reads below); larger maps: one part of the positions, rows staged by 16-byte
-    // cp.async at a pitch == 4 (mod 32), read back as float4.
-    constexpr int NQ = (S == 7) ? 1 : 4;
-    constexpr int HWC = role_c_hwc(S);
-    constexpr int PC = role_c_pitch(S);
-    constexpr int G = kNT / HWC;
-    constexpr bool kBulkC = kBulk && NQ == 1;
-    const int b = bid / NQ, q = bid % NQ;
-    const int hw0 = (S == 14) ? (q == 0 ? 0 : 4 + 48 * q) : q * HWC;     // first position of this part
-    const int nval = (S == 14 && q > 0) ? 48 : HWC;                      // positions it holds
-    float* Xs = smem;                                // [C][PC]
-    float* U2s = Xs + ((C * PC + 3) & ~3);           // [C][R]
-    float* V2s = U2s + C * R;                        // [HWC][R]
-    float* Vp = (C >= (G - 1) * HWC) ? U2s : V2s + HWC * R;   // [G-1][HWC][R]: on top of U2s when it fits
-    const TX* Xb = A + (int64_t)b * C * HW + hw0;
-    if constexpr (kBulkC)
-      stage_block(&s_bar, reinterpret_cast<char*>(Xs), reinterpret_cast<const char*>(Xb), (uint32_t)C * HW * 4u,
-                  p.stall_copy != 0);
-    fac_issue_padded<R>(p.U_prev + p.u_off[1], U2s, C, p.r[1]);
-    if constexpr (kBulkC) {
-    } else if constexpr (NQ == 1) {
-      const int n4 = C * HW / 4;
-      for (int idx = tid; idx < n4; idx += kNT) *reinterpret_cast<float4*>(Xs + 4 * idx) = ld4<TX>(Xb + 4 * idx);
-    } else {
-      constexpr int NV = HWC / 4;
-      const int n = C * NV;
-#pragma unroll 1
-      for (int idx = tid; idx < n; idx += kNT) {
-        const int c = idx / NV, v = idx - c * NV;
-        float* dst = Xs + c * PC + 4 * v;
-        const TX* src = Xb + (int64_t)c * HW + 4 * v;
-        if (4 * v >= nval) {
-          *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else if constexpr (kBulk) {
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-        } else {
-          *reinterpret_cast<float4*>(dst) = ld4<TX>(src);
-        }
-      }
-    }
-    fac_wait();
-    if constexpr (kBulkC) {
-      if (!cta_wait_tile(&s_bar, &s_flag, p.status, p.wait_ns)) return;
-    } else {
-      __syncthreads();
-    }
-    project_channels<HWC, PC, R>(Xs, U2s, Vp, V2s, C);
-    // expansion: P2[c,:] = sum_hw X[c,hw] V2[hw,:], one channel row per thread
-    float* P2 = p.Pp[1] + (int64_t)bid * C * p.r[1];
-    for (int c = tid; c < C; c += kNT) {
-      const float* row = Xs + c * PC;
+  }
+  fac_wait();
+  bool ok = true;
+  if (bulk && nc > 0) ok = cta_wait_tile(&s_bar, &s_flag, p.status, p.wait_ns);
+  else __syncthreads();
+  // ---- this CTA's share of V_2: thread (g, hw) sums the channels c == g (mod G)
+  const int G = kPT / HW;                            // HW <= 256
+  {
+    const FDiv dHW(HW);
+    int g, hw;
+    dHW.divmod(tid, g, hw);
+    if (g < G && ok) {
       float acc[R];
 #pragma unroll
       for (int j = 0; j < R; ++j) acc[j] = 0.f;
-      if constexpr (NQ == 1) {
-#pragma unroll 7
-        for (int hw = 0; hw < HWC; ++hw) fma_row<R>(acc, row[hw], V2s + hw * R);
+#pragma unroll 4
+      for (int c = g; c < nc; c += G) fma_row<R>(acc, Xs[c * P + hw], U2s + c * R);
+      float* dst = (G == 1 ? V2l : Vp) + (g * HW + hw) * R;
+#pragma unroll
+      for (int j = 0; j < R; j += 4) *reinterpret_cast<float4*>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+    }
+    if (G > 1) {
+      __syncthreads();
+      for (int idx = tid; idx < HW * R; idx += kPT) {
+        float s = Vp[idx];
+        for (int q = 1; q < G; ++q) s += Vp[q * HW * R + idx];
+        V2l[idx] = s;
+      }
+    }
+  }
+  if (cs > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  else __syncthreads();
+  // ---- modes 3 and 4 while the other CTAs of the cluster finish their shares
+  if (KIND == 7 || KIND == 14) {
+    const int mode = 2 + (warp >> 2), wq = warp & 3;  // warps 0-3: mode 3, warps 4-7: mode 4
+    const int es = mode == 2 ? W : 1, st = mode == 2 ? 1 : W;
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+    if (KIND == 7) {
+      // upper triangle of G, one plane per thread at a time (odd pitch: 32 lanes, 32 banks)
+      if (ok)
+        for (int pl = wq * 32 + lane; pl < nc; pl += 128) {
+          const float* base = Xs + pl * P;
+#pragma unroll 1
+          for (int col = 0; col < 7; ++col) {
+            float xv[7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) xv[k] = base[col * st + k * es];
+#pragma unroll
+            for (int k = 0; k < 7; ++k)
+#pragma unroll
+              for (int k2 = k; k2 < 7; ++k2) acc[tri_index(7, k, k2)] = fmaf(xv[k], xv[k2], acc[tri_index(7, k, k2)]);
+          }
+        }
+    } else if (ok) {
+      gram14_accumulate(Xs, P, nc * 4, lane, 32, wq, es, st, acc);
+    }
+    warp_reduce_scatter<32>(acc, lane);
+    float* gr = Vp;                                  // [8][32] (Vp is at least that large; its sums are in V2l)
+    __syncthreads();
+    gr[warp * 32 + scatter_base<32>(lane)] = acc[0];
+    __syncthreads();
+    for (int o = tid; o < 2 * HW; o += kPT) {
+      const int m = o >= HW, q = m ? o - HW : o;
+      float s;
+      if (KIND == 7) {
+        const int k = q / 7, k2 = q % 7;
+        const int e = (k <= k2) ? tri_index(7, k, k2) : tri_index(7, k2, k);
+        s = ((gr[(4 * m) * 32 + e] + gr[(4 * m + 1) * 32 + e]) + gr[(4 * m + 2) * 32 + e]) + gr[(4 * m + 3) * 32 + e];
       } else {
+        int rl, e;
+        gram14_slot(q, rl, e);
+        s = gr[(4 * m + rl) * 32 + e];
+      }
+      p.Pp[2 + m][(int64_t)bid * HW + q] = s;
+    }
+  } else {
+    float* Vw = U3s + (H + W) * R;
+    float* rd = Vw + 8 * 32 * R;
+    planes_modes34<R>(Xs, P, ok ? nc : 0, H, W, U3s, U3s + H * R, Vw, rd, p.Pp[2] + (int64_t)bid * H * p.r[2],
+                      p.Pp[3] + (int64_t)bid * W * p.r[3], p.r[2], p.r[3]);
+  }
+  pdl_launch_dependents();
+  // ---- V_2 = the shares of the cluster, in rank order
+  if (cs > 1) {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    cg::cluster_group cluster = cg::this_cluster();
+    for (int idx = tid; idx < HW * R; idx += kPT) {
+      float s = cluster.map_shared_rank(V2l, 0)[idx];
+      for (int q = 1; q < cs; ++q) s += cluster.map_shared_rank(V2l, q)[idx];
+      V2s[idx] = s;
+    }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // the shares have been read
+    __syncthreads();
+  } else {
+    V2s = V2l;
+  }
+  // ---- P_2 of the CTA's channels: thread = four channels q, q + Q, .. and a share of the positions
+  const int Q = (nc + 3) >> 2;
+  if (ok && nc > 0) {
+    float* P2 = p.Pp[1] + ((int64_t)b * C + c0) * r2;
+    const int parts = Q < kPT ? (kPT / Q < 16 ? kPT / Q : 16) : 1;
+    const FDiv dQ(Q);
+    const int rounds = (Q * parts + kPT - 1) / kPT;  // > 1 only when parts == 1
+#pragma unroll 1
+    for (int rd = 0; rd < rounds; ++rd) {
+      const int it = tid + rd * kPT;
+      int part, q;
+      dQ.divmod(it, part, q);
+      const bool on = part < parts;
+      float acc[4][R];
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[m][j] = 0.f;
+      if (on) {
+        const float* row[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) row[m] = Xs + (q + m * Q < nc ? q + m * Q : q) * P;
+        if ((HW & 3) == 0) {
+#pragma unroll 1
+          for (int hw = 4 * part; hw < HW; hw += 4 * parts) {
+            float4 xv[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) xv[m] = *reinterpret_cast<const float4*>(row[m] + hw);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              fma_row<R>(acc[m], xv[m].x, V2s + hw * R);
+              fma_row<R>(acc[m], xv[m].y, V2s + (hw + 1) * R);
+              fma_row<R>(acc[m], xv[m].z, V2s + (hw + 2) * R);
+              fma_row<R>(acc[m], xv[m].w, V2s + (hw + 3) * R);
+            }
+          }
+        } else {
 #pragma unroll 2
-        for (int hw = 0; hw < HWC; hw += 4) {
-          const float4 x = *reinterpret_cast<const float4*>(row + hw);
-          fma_row<R>(acc, x.x, V2s + hw * R);
-          fma_row<R>(acc, x.y, V2s + (hw + 1) * R);
-          fma_row<R>(acc, x.z, V2s + (hw + 2) * R);
-          fma_row<R>(acc, x.w, V2s + (hw + 3) * R);
+          for (int hw = part; hw < HW; hw += parts) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) fma_row<R>(acc[m], row[m][hw], V2s + hw * R);
+          }
         }
       }
+      if (parts > 1) {
+        __syncthreads();                             // the tile is free
+        if (on) {
 #pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (j < p.r[1]) P2[c * p.r[1] + j] = acc[j];
+          for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int j = 0; j < R; j += 4)
+              *reinterpret_cast<float4*>(red + ((part * 4 + m) * Q + q) * R + j) = make_float4(acc[m][j], acc[m][j + 1], acc[m][j + 2], acc[m][j + 3]);
+        }
+        __syncthreads();
+        for (int idx = tid; idx < nc * R; idx += kPT) {
+          const int c = idx / R, j = idx % R;        // channel c = m Q + q
+          float s = red[idx];
+          for (int k = 1; k < parts; ++k) s += red[k * 4 * Q * R + idx];
+          if (j < r2) P2[c * r2 + j] = s;
+        }
+      } else if (on) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+          for (int j = 0; j < R; ++j)
+            if (q + m * Q < nc && j < r2) P2[(q + m * Q) * r2 + j] = acc[m][j];
+      }
     }
+  }
+  if (cs > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int KIND, int R, typename TX>
+__device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid) {
+  extern __shared__ __align__(128) float smem[];
+  const int tid = threadIdx.x;
+  if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
+  if (bid >= p.B * p.cs) {
+    const int tile = bid - p.B * p.cs;
+    if (tile >= p.n_tiles_b) return;                 // padding to whole clusters
+    if (p.vec4) pass1_role_b<R, 4, TX>(p, tile, smem);
+    else pass1_role_b<R, 1, TX>(p, tile, smem);
+  } else {
+    pass1_role_c<KIND, R, TX>(p, bid, smem);
   }
 }
 
@@ -693,14 +732,14 @@ __device__ __forceinline__ int batch_layer(const SmBatch<Args>& b, int bid) {
   return l;
 }
 
-template <int S, int R, typename TX>
-__global__ void __launch_bounds__(kNT, 2) k_sm_pass1(const __grid_constant__ SmPass1Args p) {
-  sm_pass1_cta<S, R, TX>(p, (int)blockIdx.x);
+template <int KIND, int R, typename TX>
+__global__ void __launch_bounds__(kPT, 2) k_sm_pass1(const __grid_constant__ SmPass1Args p) {
+  sm_pass1_cta<KIND, R, TX>(p, (int)blockIdx.x);
 }
-template <int S, int R, typename TX>
-__global__ void __launch_bounds__(kNT, 2) k_sm_pass1_b(const __grid_constant__ SmBatch<SmPass1Args> b) {
+template <int KIND, int R, typename TX>
+__global__ void __launch_bounds__(kPT, 2) k_sm_pass1_b(const __grid_constant__ SmBatch<SmPass1Args> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_pass1_cta<S, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_pass1_cta<KIND, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -879,63 +918,111 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
 }
 
 // ---------------------------------------------------------------------------------------------
-// k_sm_core.  Tile t = [all B x J] as in role B of the first pass.
-//   prologue (while the tile is in flight): one thread per needed factor row fetches the fp64 row of
-//     P_m and solves u = p R_m^{-1} with the Cholesky factor the reduction kernel left -- all of U_1,
-//     the tile's own rows of U_2, all of U_3 and U_4 -- and the owners write them to U_new;
-//   W[i][c,h,w] = sum_b U1[b,i] X[b][c,h,w];  Y[i,j][h,w] = sum_c U2[c,j] W[i][c,h,w];
-//   T[i,j,k,l] = Y x_3 U3^T x_4 U4^T  -> per-tile partial core, summed in two ordered levels.
+// k_sm_core.  Tile = CC whole channels (at most 256 columns (c, h, w)) of all samples:
+//   prologue: one thread per needed factor row fetches the fp64 row of P_m and solves u = p R_m^{-1} with the
+//     Cholesky factor the reduction kernel left -- all of U_1, the tile's own rows of U_2, all of U_3 and U_4 -- and
+//     the owners write them to U_new; the first samples of the tile are already on their way;
+//   W[c,h,w][i] = sum_b U1[b,i] X[b][c,h,w] straight from memory in registers (the activation is in L2 or streams
+//     from HBM; nothing is staged, so several CTAs share an SM);
+//   M[c][i,k,l] = W x_3 U3^T x_4 U4^T per channel -- the spatial modes before the channel mode: r1 r3 (W + r4) short
+//     sums per channel instead of r1 r2 HW, and r1 r3 r4 numbers leave a channel instead of a whole core;
+//   core[i,j,k,l] = sum_c U2[c,j] M[c][i,k,l] by the last CTA of every group of tiles, then over the groups by the last
+//     group, both in index order.
 // ---------------------------------------------------------------------------------------------
-template <int S, int R, typename TX>
+template <int R, int VW, typename TX>
+__device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t chw, int B, int J, int jvalid,
+                                             const float* __restrict__ U1s, float* __restrict__ part, float* __restrict__ Ws,
+                                             bool wait_rows) {
+  constexpr int U = 8;
+  const int tid = threadIdx.x;
+  const int JV = (J + VW - 1) / VW, NH = kPT / JV;
+  const FDiv dJ(JV);
+  int h, jq;
+  dJ.divmod(tid, h, jq);
+  const bool on = h < NH && jq * VW < jvalid;
+  const TX* src = A + (on ? jq * VW : 0);
+  float acc[VW][R];
+#pragma unroll
+  for (int c = 0; c < VW; ++c)
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
+  if (h >= NH) h = 0;
+  for (int b0 = h; (on && b0 < B) || wait_rows; b0 += U * NH) {
+    RawCol<TX, VW> x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u].load(src + (int64_t)(b0 + u * NH < B ? b0 + u * NH : B - 1) * chw);
+    if (wait_rows) {                                 // uniform: every thread's first batch
+      __syncthreads();                               // the factor rows are there
+      wait_rows = false;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int b = b0 + u * NH;
+      if (b < B) {
+        float xs[VW];
+        x[u].get(xs);
+#pragma unroll
+        for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], U1s + b * R);
+      }
+    }
+  }
+  if (on) {
+    float* dst = part + (h * J + jq * VW) * R;
+#pragma unroll
+    for (int c = 0; c < VW; ++c)
+#pragma unroll
+      for (int j = 0; j < R; j += 4)
+        *reinterpret_cast<float4*>(dst + c * R + j) = make_float4(acc[c][j], acc[c][j + 1], acc[c][j + 2], acc[c][j + 3]);
+  }
+  __syncthreads();
+  for (int idx = tid; idx < jvalid * R; idx += kPT) {
+    float s = part[idx];
+    for (int q = 1; q < NH; ++q) s += part[q * J * R + idx];
+    Ws[idx] = s;
+  }
+  __syncthreads();
+}
+
+template <int R, typename TX>
 __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) {
-  constexpr int HW = S * S;
-  constexpr int CC = (S == 7) ? 4 : 1;
-  constexpr int J = CC * HW;
-  constexpr int PJ = pitch4(J);
-  constexpr int NH = batch_groups(kNT, J);
   extern __shared__ __align__(128) float smem[];
   __shared__ int s_last;
   __shared__ double Rs[4][kRfStride];   // per mode: rows of R_m (pitch 8), then 1 / diag(R_m) at [64..]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int B = p.B, C = p.C, tile = bid;
+  const int tid = threadIdx.x;
+  const int B = p.B, C = p.C, H = p.H, W = p.W, HW = H * W, CC = p.tile_c, J = CC * HW, tile = bid;
   const int r1 = p.r[0], r2 = p.r[1], r3 = p.r[2], r4 = p.r[3];
-  float* Xs = smem;                     // [B][PJ]
-  float* U1s = Xs + B * PJ;             // [B][R]
-  float* U2s = U1s + B * R;             // [CC][R]
-  float* U3s = U2s + CC * R;            // [S][R]
-  float* U4s = U3s + S * R;             // [S][R]
-  float* Ws = U4s + S * R;              // [J][R]
-  float* part = Ws + J * R;             // [NH][J][R]
-  float* Ysm = part + NH * J * R;       // [R R][HW]
-  float* T3s = Ysm + R * R * HW;        // [R R][R][S]
-  stage_tile_begin<TX>(reinterpret_cast<const TX*>(p.act) + (int64_t)tile * J, (int64_t)C * HW, Xs, B, J, PJ);
-  cp_async_commit();
-  pdl_wait();                           // P_m and the Gram shares come from the reduction kernel
-  // ---- the factor row this thread will solve for: [U1: B rows][U2: CC rows][U3: S][U4: S]
-  const int nrows = B + CC + 2 * S;     // <= kNT (checked when the plan picks this kernel)
-  int rm = 0, rk = 0, rr = 0;
-  float* rdst = nullptr;
-  bool rowner = false;
-  double prow[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) prow[j] = 0.0;
-  if (tid < nrows) {
-    if (tid < B) { rm = 0; rk = tid; rdst = U1s + rk * R; rowner = tile == 0; }
-    else if (tid < B + CC) { rm = 1; rk = tile * CC + (tid - B); rdst = U2s + (tid - B) * R; rowner = true; }
-    else if (tid < B + CC + S) { rm = 2; rk = tid - B - CC; rdst = U3s + rk * R; rowner = tile == 0; }
-    else { rm = 3; rk = tid - B - CC - S; rdst = U4s + rk * R; rowner = tile == 0; }
-    rr = p.r[rm];
-    const double* src = p.Pred[rm] + (int64_t)rk * rr;
-#pragma unroll
-    for (int j = 0; j < R; ++j)
-      if (j < rr) prow[j] = __ldcg(src + j);
-  }
+  const int c0 = tile * CC, ncl = (C - c0 < CC) ? C - c0 : CC, jvalid = ncl * HW;
+  float* U1s = smem;                    // [B][R]
+  float* U3s = U1s + ((B * R + 3) & ~3);   // [H][R]
+  float* U4s = U3s + H * R;             // [W][R]
+  float* Ws = U4s + W * R;              // [J][R]
+  float* part = Ws + J * R;             // [NH][J][R], at most 256 * 4 R
+  float* T1 = part;                     // [ncl r1][r3][W] after part is free
+  pdl_wait();                           // P_m and the Cholesky factors come from the reduction kernel
   // ---- the Cholesky factors of the four modes (computed once, by the reduction kernel)
-  for (int e = tid; e < 4 * kRfStride; e += kNT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
-  __syncthreads();
-  if (tid < nrows) {
-    float* gdst = p.U_new + p.u_off[rm] + (int64_t)rk * rr;
-    double q[R];
+  for (int e = tid; e < 4 * kRfStride; e += kPT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
+  // ---- factor rows: [U1: B rows][the tile's rows of U2][U3: H][U4: W]
+  const int nrows = B + ncl + H + W;
+  double prow[R];
+  bool synced = false;
+#pragma unroll 1
+  for (int row = tid; row < nrows || !synced; row += kPT) {
+    int m = 0, k = row;
+    float* rdst = U1s + k * R;
+    bool owner = tile == 0;
+    if (row >= B + ncl + H) { m = 3; k = row - B - ncl - H; rdst = U4s + k * R; }
+    else if (row >= B + ncl) { m = 2; k = row - B - ncl; rdst = U3s + k * R; }
+    else if (row >= B) { m = 1; k = c0 + row - B; rdst = nullptr; owner = true; }
+    const int rr = p.r[m];
+    const bool on = row < nrows;
+#pragma unroll
+    for (int j = 0; j < R; ++j) prow[j] = (on && j < rr) ? __ldcg(p.Pred[m] + (int64_t)k * rr + j) : 0.0;
+    if (!synced) {
+      __syncthreads();
+      synced = true;
+    }
+    if (!on) break;
+    float* gdst = p.U_new + p.u_off[m] + (int64_t)k * rr;
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       float out = 0.f;
@@ -943,75 +1030,77 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
         double v = prow[j];
 #pragma unroll
         for (int i = 0; i < R; ++i)
-          if (i < j) v -= q[i] * Rs[rm][i * 8 + j];
-        v *= Rs[rm][64 + j];
-        q[j] = v;
+          if (i < j) v = fma(-prow[i], Rs[m][i * 8 + j], v);
+        v *= Rs[m][64 + j];
+        prow[j] = v;
         out = (float)v;
-        if (rowner) gdst[j] = out;
+        if (owner) gdst[j] = out;
       }
-      rdst[j] = out;
+      if (rdst) rdst[j] = out;
     }
   }
-  cp_async_wait<0>();
-  __syncthreads();
-  project_batch<R>(Xs, PJ, U1s, B, J, part, Ws, tid, kNT, 0);
-  // Y[(i,j)][hw] = sum_cl U2[cl][j] W[cl*HW + hw][i]
-  const int r12 = r1 * r2;
-  const FDiv d_r2(r2), d_r3(r3), d_r4(r4);
-  for (int idx = tid; idx < r12 * HW; idx += kNT) {
-    const int hw = idx % HW, ij = idx / HW;
-    int i, j;
-    d_r2.divmod(ij, i, j);
+  const TX* A = reinterpret_cast<const TX*>(p.act) + (int64_t)c0 * HW;
+  const int64_t chw = (int64_t)C * HW;
+  if (p.vec4) core_project<R, 4, TX>(A, chw, B, J, jvalid, U1s, part, Ws, true);
+  else core_project<R, 1, TX>(A, chw, B, J, jvalid, U1s, part, Ws, true);
+  // T1[cl,i][k][w] = sum_h W[cl,h,w][i] U3[h][k]
+  const FDiv dW(W), d_r1(r1), d_r3(r3), d_r4(r4);
+  for (int idx = tid; idx < ncl * r1 * r3 * W; idx += kPT) {
+    int t, w, ci, k, cl, i;
+    dW.divmod(idx, t, w);
+    d_r3.divmod(t, ci, k);
+    d_r1.divmod(ci, cl, i);
+    const float* ws = Ws + (cl * HW + w) * R + i;
     float s = 0.f;
-#pragma unroll
-    for (int cl = 0; cl < CC; ++cl) s = fmaf(U2s[cl * R + j], Ws[(cl * HW + hw) * R + i], s);
-    Ysm[ij * HW + hw] = s;
+#pragma unroll 4
+    for (int h = 0; h < H; ++h) s = fmaf(ws[h * W * R], U3s[h * R + k], s);
+    T1[idx] = s;
   }
   __syncthreads();
-  // T3[(i,j)][k][w] = sum_h Y[(i,j)][h,w] U3[h][k]
-  for (int idx = tid; idx < r12 * r3 * S; idx += kNT) {
-    const int w = idx % S;
-    int ij, k;
-    d_r3.divmod(idx / S, ij, k);
+  // M[c][i,k,l] = sum_w T1[cl,i][k][w] U4[w][l]
+  const int ce3 = r1 * r3 * r4;
+  for (int idx = tid; idx < ncl * ce3; idx += kPT) {
+    int t, l;
+    d_r4.divmod(idx, t, l);
+    const float* ts = T1 + t * W;
     float s = 0.f;
-#pragma unroll
-    for (int h = 0; h < S; ++h) s = fmaf(Ysm[ij * HW + h * S + w], U3s[h * R + k], s);
-    T3s[(ij * R + k) * S + w] = s;
+#pragma unroll 4
+    for (int w = 0; w < W; ++w) s = fmaf(ts[w], U4s[w * R + l], s);
+    p.Tp[(int64_t)c0 * ce3 + idx] = s;
   }
-  __syncthreads();
-  // T[(i,j)][k][l] = sum_w T3[(i,j)][k][w] U4[w][l]
-  const int ce = r12 * r3 * r4;
-  for (int idx = tid; idx < ce; idx += kNT) {
-    int t34, l, ij, k;
-    d_r4.divmod(idx, t34, l);
-    d_r3.divmod(t34, ij, k);
-    float s = 0.f;
-#pragma unroll
-    for (int w = 0; w < S; ++w) s = fmaf(T3s[(ij * R + k) * S + w], U4s[w * R + l], s);
-    p.Tp[(int64_t)tile * ce + idx] = s;
-  }
-  // Two-level sum of the per-tile cores, both levels in index order: the last CTA of every group of
-  // p.gs tiles sums that group, the last group to finish sums the groups.
+  // ---- groups of gs tiles, then the groups, both by the last CTA and in index order
   __threadfence();
   __syncthreads();
-  const int grp = tile / p.gs, gfirst = grp * p.gs;
+  const int grp = tile / p.gs, gfirst = grp * p.gs, ce = ce3 * r2;
   const int gsize = (p.n_tiles - gfirst < p.gs) ? p.n_tiles - gfirst : p.gs;
   const int ngroups = (p.n_tiles + p.gs - 1) / p.gs;
   if (tid == 0) s_last = (atomicAdd(p.gcount + grp, 1) == gsize - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int idx = tid; idx < ce; idx += kNT) {
-    const float* src = p.Tp + (int64_t)gfirst * ce + idx;
-    float s = 0.f;
-    for (int t0 = 0; t0 < gsize; t0 += 8) {
-      float v[8];
+  {
+    const int ch0 = gfirst * CC, nch = ((gfirst + gsize) * CC < C ? (gfirst + gsize) * CC : C) - ch0;
+    float* u2 = part;                   // [nch][r2] (gs CC r2 floats: fits, checked by the host)
+    for (int e = tid; e < nch * r2; e += kPT) u2[e] = __ldcg(p.U_new + p.u_off[1] + (int64_t)ch0 * r2 + e);
+    __syncthreads();
+    const FDiv d34(r3 * r4), d_r2(r2);
+    for (int idx = tid; idx < ce; idx += kPT) {
+      int ij, kl, i, j;
+      d34.divmod(idx, ij, kl);
+      d_r2.divmod(ij, i, j);
+      const float* src = p.Tp + (int64_t)ch0 * ce3 + i * r3 * r4 + kl;
+      float s = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < nch; c += 16) {
+        float v[16];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = (t0 + k < gsize) ? __ldcg(src + (int64_t)(t0 + k) * ce) : 0.f;
+        for (int q = 0; q < 16; ++q) v[q] = __ldcg(src + (int64_t)(c + q < nch ? c + q : c) * ce3);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) s += v[k];
+        for (int q = 0; q < 16; ++q)
+          if (c + q < nch) s = fmaf(v[q], u2[(c + q) * r2 + j], s);
+      }
+      p.Tg[(int64_t)grp * ce + idx] = s;
     }
-    p.Tg[(int64_t)grp * ce + idx] = s;
   }
   __threadfence();
   __syncthreads();
@@ -1022,63 +1111,52 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (ce * 2 <= kNT) {
-    // few core elements: thread (e, q) sums the groups == q (mod nq) of element e, the nq sums meet
-    // in index order (shared memory: the tile is no longer needed)
-    int nq = kNT / ce;
-    nq = nq > 8 ? 8 : nq;
-    float* fold = smem;                              // [nq][ce]
-    if (tid < nq * ce) {
-      const int q = tid / ce, e = tid - q * ce;
-      const float* src = p.Tg + e;
-      float s = 0.f;
-      for (int g0 = q; g0 < ngroups; g0 += 8 * nq) {
-        float v[8];
+  // few core elements: thread (e, q) sums the groups == q (mod nq) of element e, the nq sums meet in index order
+  int nq = kPT / ce;
+  nq = nq > 8 ? 8 : (nq < 1 ? 1 : nq);
+  float* fold = part;                   // [nq][ce]
+  for (int it = tid; it < nq * ce; it += kPT) {
+    const int q = it / ce, e = it - q * ce;
+    const float* src = p.Tg + e;
+    float s = 0.f;
+#pragma unroll 1
+    for (int g0 = q; g0 < ngroups; g0 += 16 * nq) {
+      float v[16];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = (g0 + k * nq < ngroups) ? __ldcg(src + (int64_t)(g0 + k * nq) * ce) : 0.f;
+      for (int k = 0; k < 16; ++k) v[k] = __ldcg(src + (int64_t)(g0 + k * nq < ngroups ? g0 + k * nq : g0) * ce);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) s += v[k];
-      }
-      fold[tid] = s;
+      for (int k = 0; k < 16; ++k) s += (g0 + k * nq < ngroups) ? v[k] : 0.f;
     }
+    if (nq > 1) fold[it] = s;
+    else p.core[e] = s;
+  }
+  if (nq > 1) {
     __syncthreads();
     if (tid < ce) {
       float s = fold[tid];
       for (int q = 1; q < nq; ++q) s += fold[q * ce + tid];
       p.core[tid] = s;
     }
-  } else {
-    for (int idx = tid; idx < ce; idx += kNT) {
-      const float* src = p.Tg + idx;
-      float s = 0.f;
-      for (int g0 = 0; g0 < ngroups; g0 += 16) {
-        float v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = (g0 + k < ngroups) ? __ldcg(src + (int64_t)(g0 + k) * ce) : 0.f;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) s += v[k];
-      }
-      p.core[idx] = s;
-    }
   }
   if (tid == 0) *p.counter = 0;
 }
 
-template <int S, int R, typename TX>
-__global__ void __launch_bounds__(kNT) k_sm_core(const __grid_constant__ SmCoreArgs p) {
-  sm_core_cta<S, R, TX>(p, (int)blockIdx.x);
+template <int R, typename TX>
+__global__ void __launch_bounds__(kPT, 3) k_sm_core(const __grid_constant__ SmCoreArgs p) {
+  sm_core_cta<R, TX>(p, (int)blockIdx.x);
 }
-template <int S, int R, typename TX>
-__global__ void __launch_bounds__(kNT) k_sm_core_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
+template <int R, typename TX>
+__global__ void __launch_bounds__(kPT, 3) k_sm_core_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_core_cta<S, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_core_cta<R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
 // k_sm_wgrad: CTA owns cpb consecutive output channels, i.e. the dY tile [B x J], J = cpb*Ho*Wo
-// contiguous values per sample (staged by 16-byte cp.async when fp32 and 16-byte aligned).
-//   Z3 = core x_3 U3 x_4 U4 (recomputed per CTA while the tile is in flight);
-//   Z1 = dY x_1 U1^T on the CTA's channels;
+// contiguous values per sample.
+//   Z1 = dY x_1 U1^T on the CTA's channels, straight from memory in registers (no staged tile: 100 KB less shared
+//     memory, so two CTAs share an SM and the set-up of one hides behind the stream of the other);
+//   Z3 = core x_3 U3 x_4 U4 (recomputed per CTA);
 //   Z4[c',j,kh,kw] = sum_{i,h',w'} Z1[i,c',h',w'] Z3pad[i,j,h's+kh-p,w's+kw-p];  dW = Z4 x_2 U2.
 // ---------------------------------------------------------------------------------------------
 // Term 5: dW[c0+cl, c, t] = sum_j Z4[cl][t][j] U2[(g cg + c), j].  The rows of Z4 are the same for every
@@ -1169,25 +1247,86 @@ __device__ __forceinline__ void wgrad_expand_rows(const SmWgradArgs& p, const fl
   if (p.bulk_store && tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
+// groups of samples a CTA of k_sm_wgrad splits the batch over (JV column items)
+__host__ __device__ inline int wgrad_groups(int JV) {
+  const int n = kNT / (JV < kNT ? JV : kNT);
+  return n > 8 ? 8 : n;
+}
+// Z1[j][:] = sum_b dY[b][j] U1[b][:] for the CTA's J columns; thread = VW neighbouring columns and the samples
+// b == h (mod NH), eight of them in flight; the NH shares meet in order.  The factors' asynchronous copies of this
+// thread are waited for behind the first loads.
+template <int R, int VW, typename TX>
+__device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t sstride, int B, int J, int NH,
+                                              const float* __restrict__ U1s, float* __restrict__ part, float* __restrict__ Z1s) {
+  constexpr int U = R == 4 ? 8 : 4;                  // 64 registers a thread: two CTAs of 512
+  const int tid = threadIdx.x, JV = (J + VW - 1) / VW;
+  const FDiv dJ(JV);
+  bool waited = false;
+  for (int it = tid; it < NH * JV || !waited; it += kNT) {      // one round unless there are more columns than threads
+    int h, jq;
+    dJ.divmod(it, h, jq);
+    const bool on = h < NH;
+    const TX* src = dY + (on ? jq * VW : 0);
+    if (!on) h = 0;
+    float acc[VW][R];
+#pragma unroll
+    for (int c = 0; c < VW; ++c)
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
+    for (int b0 = h; (on && b0 < B) || !waited; b0 += U * NH) {
+      RawCol<TX, VW> x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u].load(src + (int64_t)(b0 + u * NH < B ? b0 + u * NH : B - 1) * sstride);
+      if (!waited) {
+        fac_wait();
+        __syncthreads();
+        waited = true;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int b = b0 + u * NH;
+        if (b < B) {
+          float xs[VW];
+          x[u].get(xs);
+#pragma unroll
+          for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], U1s + b * R);
+        }
+      }
+    }
+    if (on) {
+      float* dst = part + (h * J + jq * VW) * R;
+#pragma unroll
+      for (int c = 0; c < VW; ++c)
+#pragma unroll
+        for (int j = 0; j < R; j += 4)
+          *reinterpret_cast<float4*>(dst + c * R + j) = make_float4(acc[c][j], acc[c][j + 1], acc[c][j + 2], acc[c][j + 3]);
+    }
+  }
+  __syncthreads();
+  for (int idx = tid; idx < J * R; idx += kNT) {
+    float s = part[idx];
+    for (int q = 1; q < NH; ++q) s += part[q * J * R + idx];
+    Z1s[idx] = s;
+  }
+}
+
 template <int R, typename TX>
 __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
   const int r1 = p.r[0], r2 = p.r[1], r3 = p.r[2], r4 = p.r[3];
-  const int H = p.H, W = p.W, HW = H * W, HoWo = p.Ho * p.Wo, kk = p.kh * p.kw;
+  const int H = p.H, W = p.W, HoWo = p.Ho * p.Wo, kk = p.kh * p.kw;
   const int J = p.cpb * HoWo;                        // dY columns of this CTA, contiguous per sample
-  const int PJ = p.pj;
-  const int NH = batch_groups(kNT, J);
   const int c0 = bid * p.cpb;
-  const int n_out = p.cpb * r2 * kk;
   // staging blocks of term 5 reuse the tile's space: ncl channels per round, doubled when rounds follow
   const int n_stage = (p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
-  float* Ys = smem;                                  // [B][PJ]
-  float* U1s = Ys + ((p.B * PJ > n_stage ? p.B * PJ : n_stage) + 3) / 4 * 4;   // [B][R]
+  const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV);
+  float* stage = smem;                               // term 5's blocks; before that the shares of Z1 [NH][J][R]
+  float* part = smem;
+  float* U1s = smem + ((NH * J * R > n_stage ? NH * J * R : n_stage) + 3) / 4 * 4;   // [B][R]
   float* U2s = U1s + p.B * R;                        // [C][R]
   float* Z1s = U2s + p.C * R;                        // [J][R]
-  float* part = Z1s + J * R;                         // [NH][J][R] (NH > 1 only)
-  float* Ss = part + (NH > 1 ? NH : 0) * J * R;      // [r1 r2][R (l)][R (k)]: core, modes 3 and 4 swapped, zero-padded
+  float* Ss = Z1s + J * R;                           // [r1 r2][R (l)][R (k)]: core, modes 3 and 4 swapped, zero-padded
   float* U3s = Ss + r1 * r2 * R * R;                 // [H][R]
   float* U4s = U3s + H * R;                          // [W][R]
   float* Tm = U4s + W * R;                           // [r1 r2][H][R]
@@ -1198,7 +1337,6 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
 
   const TX* dY = reinterpret_cast<const TX*>(p.dY) + (int64_t)c0 * HoWo;
   const int64_t sstride = (int64_t)p.Cout * HoWo;
-  const bool bulk = std::is_same<TX, float>::value && p.bulk;
   {
 #pragma unroll 1
     for (int idx = tid; idx < r1 * r2 * R * R; idx += kNT) {      // Ss[ij][l][k] = core[ij][k][l]
@@ -1210,20 +1348,9 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
     fac_issue_padded<R>(p.U + p.u_off[3], U4s, W, r4);
     fac_issue_padded<R>(p.U + p.u_off[0], U1s, p.B, r1);
     fac_issue_padded<R>(p.U + p.u_off[1], U2s, p.C, r2);
-    cp_async_commit();                               // group 1: factors and core; group 0 (younger): the tile
-    if constexpr (std::is_same<TX, float>::value) {
-      if (bulk) stage_rows_async(Ys, reinterpret_cast<const float*>(dY), p.B, J, sstride, PJ);
-    }
-    if (!bulk) {
-      for (int idx = tid; idx < p.B * J; idx += kNT) {
-        const int b = idx / J, j = idx - b * J;
-        Ys[b * PJ + j] = to_f(dY[b * sstride + j]);
-      }
-    }
-    cp_async_commit();
-    cp_async_wait<1>();
+    if (p.vec4) wgrad_project<R, 4, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
+    else wgrad_project<R, 1, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
   }
-  __syncthreads();
   // terms 2-3: Tm[ij][h][l] = sum_k S[ij][k][l] U3[h][k];  Z3[ij][h][w] = sum_l Tm[ij][h][l] U4[w][l]
   // (rank indices padded to R with zeros: every sum is a fixed-length dot product of 16-byte reads)
   const FDiv d_H(H), d_Wp(Wp), d_Hp(Hp), d_kk(kk), d_kw(p.kw);
@@ -1259,10 +1386,7 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
     }
     Z3s[idx] = s;
   }
-  cp_async_wait<0>();
   __syncthreads();
-  // term 1: Z1[j,:] = sum_b dY[b, c0*HoWo + j] U1[b,:]
-  project_batch<R>(Ys, PJ, U1s, p.B, J, part, Z1s, tid, kNT, 0);
   // term 4: thread (n, g): outputs n = (j, kh, kw) of all cpb channels and every G-th pair (i, h') of
   // the reduction; one Z3 operand feeds cpb FMAs.  The G partial sums meet in order.
   const int N4 = r2 * kk;
@@ -1305,15 +1429,15 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
   }
   __syncthreads();
   // term 5: dW[c0+cl, c, t] = sum_j Z4[cl][j][t] U2[(g cg + c), j]
-  wgrad_expand_rows<R>(p, Z4s, U2s, Ys, c0);
+  wgrad_expand_rows<R>(p, Z4s, U2s, stage, c0);
 }
 
 template <int R, typename TX>
-__global__ void __launch_bounds__(kNT) k_sm_wgrad(const __grid_constant__ SmWgradArgs p) {
+__global__ void __launch_bounds__(kNT, 2) k_sm_wgrad(const __grid_constant__ SmWgradArgs p) {
   sm_wgrad_cta<R, TX>(p, (int)blockIdx.x);
 }
 template <int R, typename TX>
-__global__ void __launch_bounds__(kNT) k_sm_wgrad_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
+__global__ void __launch_bounds__(kNT, 2) k_sm_wgrad_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
   sm_wgrad_cta<R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
@@ -1321,60 +1445,91 @@ __global__ void __launch_bounds__(kNT) k_sm_wgrad_b(const __grid_constant__ SmBa
 // ---------------------------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------------------------
-int sm_pass1_role_c_ctas(int S, int B) { return (S == 7) ? B : 4 * B; }
+int sm_pass1_pitch(int HW) { return HW % 4 == 0 && (HW / 4) % 2 == 0 ? HW + 4 : HW; }
 
-size_t sm_pass1_smem(int S, int R, int B, int C) {
-  const int HW = S * S, CC = (S == 7) ? 4 : 1, J = CC * HW, PJ = pitch4(J);
-  const int NH1 = batch_groups(kNG, J);
-  const size_t role_b = (size_t)B * PJ + (size_t)B * R + 2 * S * R + (size_t)J * R +
-                        (NH1 > 1 ? (size_t)NH1 * J * R : 0) + 24 * 32;
-  const int HWC = role_c_hwc(S), PC = role_c_pitch(S);
-  const int G = kNT / HWC;
-  const size_t vp = (C >= (G - 1) * HWC) ? 0 : (size_t)(G - 1) * HWC * R;
-  const size_t role_c = (size_t)((C * PC + 3) & ~3) + (size_t)C * R + (size_t)HWC * R + vp;
+// CTAs per sample (a cluster) and channels per CTA: a sample of 32 or more channels goes to four CTAs, to eight where
+// four would hold more than 56 KB each
+void sm_pass1_split(int HW, int C, int* cs, int* cc) {
+  int n = C >= 32 ? 4 : 1;
+  auto per = [&](int k) { return ((C + k - 1) / k + 3) / 4 * 4; };
+  while (n < 8 && (size_t)per(n) * sm_pass1_pitch(HW) * 4 > 56 * 1024) n *= 2;
+  *cs = n;
+  *cc = per(n);
+}
+int sm_pass1_off_u2(int R, int cc, int pitch) {
+  const int tile = (cc * pitch + 3) & ~3, red = 4 * kPT * R;
+  return tile > red ? tile : red;
+}
+
+size_t sm_pass1_smem(const SmPass1Args& p, int kind, int R) {
+  const int HW = p.H * p.W, JT = p.vec4 ? 128 : 32;
+  const size_t role_b = (size_t)((p.B * R + 3) & ~3) + (size_t)9 * JT * R;
+  const size_t role_c = (size_t)p.off_u2 + (size_t)p.cc * R + (size_t)2 * HW * R + (size_t)(kPT / HW) * HW * R +
+                        (kind == 0 ? (size_t)(p.H + p.W + 3 * 8 * 32) * R : 0);
   return 4 * (role_b > role_c ? role_b : role_c);
 }
+int sm_pass1_tiles_b(int64_t chw, bool vec4) { return (int)((chw + (vec4 ? 127 : 31)) / (vec4 ? 128 : 32)); }
 
-size_t sm_core_smem(int S, int R, int B) {
-  const int HW = S * S, CC = (S == 7) ? 4 : 1, J = CC * HW, PJ = pitch4(J);
-  const int NH = batch_groups(kNT, J);
-  return 4 * ((size_t)B * PJ + (size_t)B * R + (size_t)CC * R + 2 * S * R + (size_t)J * R + (size_t)NH * J * R +
-              (size_t)R * R * HW + (size_t)R * R * R * S);
+// channels per tile of k_sm_core: as many as 256 columns hold, a multiple of four where that makes the tile's base
+// 16-byte aligned
+int sm_core_tile_c(int HW, int C) {
+  int cc = 256 / HW;
+  if (HW % 4 != 0 && cc >= 4) cc = cc / 4 * 4;
+  return cc < C ? cc : C;
 }
-
-int sm_core_max_rows() { return kNT; }
-
-int sm_wgrad_pitch(int J) { return pitch4(J); }
+size_t sm_core_smem(const SmCoreArgs& p, int R) {
+  const int HW = p.H * p.W, J = p.tile_c * HW, VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW;
+  size_t part = (size_t)(kPT / JV) * J * R;
+  const size_t t1 = (size_t)p.tile_c * p.r[0] * p.r[2] * p.W, u2 = (size_t)p.gs * p.tile_c * p.r[1];
+  if (t1 > part) part = t1;
+  if (u2 > part) part = u2;
+  if (part < 8 * kPT) part = 8 * kPT;                // the final fold
+  return 4 * ((size_t)((p.B * R + 3) & ~3) + (size_t)(p.H + p.W) * R + (size_t)J * R + part);
+}
 
 size_t sm_wgrad_smem(const SmWgradArgs& p, int R) {
   const int r1 = p.r[0], r2 = p.r[1];
-  const int J = p.cpb * p.Ho * p.Wo, kk = p.kh * p.kw;
+  const int J = p.cpb * p.Ho * p.Wo, kk = p.kh * p.kw, JV = p.vec4 ? J / 4 : J;
   const int N4 = r2 * kk;
-  const int NH = batch_groups(kNT, J);
-  const size_t tile = (size_t)p.B * pitch4(J),
+  const size_t part = (size_t)wgrad_groups(JV) * J * R,
                stage = (size_t)(p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
-  size_t n = ((tile > stage ? tile : stage) + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
-             (NH > 1 ? (size_t)NH * J * R : 0) + (size_t)r1 * r2 * R * R + (size_t)p.H * R + (size_t)p.W * R +
+  size_t n = ((part > stage ? part : stage) + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
+             (size_t)r1 * r2 * R * R + (size_t)p.H * R + (size_t)p.W * R +
              (size_t)r1 * r2 * p.H * R + ((size_t)r1 * r2 * (p.H + 2 * p.ph) * (p.W + 2 * p.pw) + 3) / 4 * 4 +
              (size_t)p.cpb * kk * R + (size_t)p.cpb * (N4 > kNT ? N4 : kNT);
   return 4 * n + 64;
 }
 
-template <int S, int R, typename TX>
-static cudaError_t launch_pass1_t(const SmPass1Args& p, cudaStream_t st) {
-  const size_t smem = sm_pass1_smem(S, R, p.B, p.C);   // the default limit counts static shared memory too: always opt in
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_pass1<S, R, TX>), smem);
+// an ordinary launch, in clusters of cs CTAs
+template <typename Arg>
+static cudaError_t launch_clustered(void (*kernel)(Arg), int grid, int cs, size_t smem, cudaStream_t st, const Arg& arg) {
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  k_sm_pass1<S, R, TX><<<p.n_tiles_b + sm_pass1_role_c_ctas(S, p.B), kNT, smem, st>>>(p);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kPT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cs > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
+static int pass1_grid(const SmPass1Args& p) { return p.B * p.cs + (p.n_tiles_b + p.cs - 1) / p.cs * p.cs; }
 
-template <int S, int R, typename TX>
-static cudaError_t launch_core_t(const SmCoreArgs& p, cudaStream_t st) {
-  const size_t smem = sm_core_smem(S, R, p.B);
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core<S, R, TX>), smem);
+template <int KIND, int R, typename TX>
+static cudaError_t launch_pass1_t(const SmPass1Args& p, size_t smem, cudaStream_t st) {
+  return launch_clustered(k_sm_pass1<KIND, R, TX>, pass1_grid(p), p.cs, smem, st, p);
+}
+template <int R, typename TX>
+static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t st) {
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core<R, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_sm_core<S, R, TX>, dim3(p.n_tiles), dim3(kNT), smem, st, p);
+  return launch_pdl(k_sm_core<R, TX>, dim3(p.n_tiles), dim3(kPT), smem, st, p);
 }
 
 template <int R, typename TX>
@@ -1386,31 +1541,37 @@ static cudaError_t launch_wgrad_t(const SmWgradArgs& p, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-#define ASI_DISPATCH_SR(FN, ARGS)                                              \
-  do {                                                                         \
-    if (S == 7) {                                                              \
-      if (R == 4) return bf16 ? FN<7, 4, __nv_bfloat16>(ARGS, st) : FN<7, 4, float>(ARGS, st);   \
-      return bf16 ? FN<7, 8, __nv_bfloat16>(ARGS, st) : FN<7, 8, float>(ARGS, st);               \
-    }                                                                          \
-    if (S == 14) {                                                             \
-      if (R == 4) return bf16 ? FN<14, 4, __nv_bfloat16>(ARGS, st) : FN<14, 4, float>(ARGS, st); \
-      return bf16 ? FN<14, 8, __nv_bfloat16>(ARGS, st) : FN<14, 8, float>(ARGS, st);             \
-    }                                                                          \
-    if (R == 4) return bf16 ? FN<16, 4, __nv_bfloat16>(ARGS, st) : FN<16, 4, float>(ARGS, st);   \
-    return bf16 ? FN<16, 8, __nv_bfloat16>(ARGS, st) : FN<16, 8, float>(ARGS, st);               \
+// FN<kind, R, TX> and FN<R, TX> for the plan's variant
+#define ASI_DISPATCH_KR(FN, ...)                                                                         \
+  do {                                                                                                   \
+    if (kind == 7) {                                                                                     \
+      if (R == 4) return bf16 ? FN<7, 4, __nv_bfloat16>(__VA_ARGS__) : FN<7, 4, float>(__VA_ARGS__);     \
+      return bf16 ? FN<7, 8, __nv_bfloat16>(__VA_ARGS__) : FN<7, 8, float>(__VA_ARGS__);                 \
+    }                                                                                                    \
+    if (kind == 14) {                                                                                    \
+      if (R == 4) return bf16 ? FN<14, 4, __nv_bfloat16>(__VA_ARGS__) : FN<14, 4, float>(__VA_ARGS__);   \
+      return bf16 ? FN<14, 8, __nv_bfloat16>(__VA_ARGS__) : FN<14, 8, float>(__VA_ARGS__);               \
+    }                                                                                                    \
+    if (R == 4) return bf16 ? FN<0, 4, __nv_bfloat16>(__VA_ARGS__) : FN<0, 4, float>(__VA_ARGS__);       \
+    return bf16 ? FN<0, 8, __nv_bfloat16>(__VA_ARGS__) : FN<0, 8, float>(__VA_ARGS__);                   \
+  } while (0)
+#define ASI_DISPATCH_R(FN, ...)                                                                          \
+  do {                                                                                                   \
+    if (R == 4) return bf16 ? FN<4, __nv_bfloat16>(__VA_ARGS__) : FN<4, float>(__VA_ARGS__);             \
+    return bf16 ? FN<8, __nv_bfloat16>(__VA_ARGS__) : FN<8, float>(__VA_ARGS__);                         \
   } while (0)
 
-cudaError_t launch_sm_pass1(const SmPass1Args& p, int S, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_pass1(const SmPass1Args& p, int kind, int R, bool bf16, cudaStream_t st) {
   const size_t eb = bf16 ? 2 : 4;
-  const double bytes = (double)p.B * p.C * S * S * eb;      // the activation, read once
+  const double bytes = (double)p.B * p.C * p.H * p.W * eb;      // the activation, read once
   ProfScope prof(ASI_K_SM_PASS1, st, bytes);
-  ASI_DISPATCH_SR(launch_pass1_t, p);
+  ASI_DISPATCH_KR(launch_pass1_t, p, sm_pass1_smem(p, kind, R), st);
 }
 
-cudaError_t launch_sm_core(const SmCoreArgs& p, int S, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, cudaStream_t st) {
   const size_t eb = bf16 ? 2 : 4;
-  ProfScope prof(ASI_K_SM_CORE, st, (double)p.B * p.C * S * S * eb);
-  ASI_DISPATCH_SR(launch_core_t, p);
+  ProfScope prof(ASI_K_SM_CORE, st, (double)p.B * p.C * p.H * p.W * eb);
+  ASI_DISPATCH_R(launch_core_t, p, sm_core_smem(p, R), st);
 }
 
 cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t st) {
@@ -1429,18 +1590,15 @@ cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t
 // ---------------------------------------------------------------------------------------------
 int sm_max_batch() { return kMaxBatch; }
 
-template <int S, int R, typename TX>
+template <int KIND, int R, typename TX>
 static cudaError_t launch_pass1_bt(const SmBatch<SmPass1Args>& b, size_t smem, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_pass1_b<S, R, TX>), smem);
-  if (e != cudaSuccess) return e;
-  k_sm_pass1_b<S, R, TX><<<b.first[b.n], kNT, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_clustered(k_sm_pass1_b<KIND, R, TX>, b.first[b.n], b.a[0].cs, smem, st, b);
 }
-template <int S, int R, typename TX>
+template <int R, typename TX>
 static cudaError_t launch_core_bt(const SmBatch<SmCoreArgs>& b, size_t smem, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core_b<S, R, TX>), smem);
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core_b<R, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_sm_core_b<S, R, TX>, dim3(b.first[b.n]), dim3(kNT), smem, st, b);
+  return launch_pdl(k_sm_core_b<R, TX>, dim3(b.first[b.n]), dim3(kPT), smem, st, b);
 }
 template <int R, typename TX>
 static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, cudaStream_t st) {
@@ -1450,21 +1608,7 @@ static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, c
   return cudaGetLastError();
 }
 
-#define ASI_DISPATCH_SRB(FN, ARGS, SMEM)                                       \
-  do {                                                                         \
-    if (S == 7) {                                                              \
-      if (R == 4) return bf16 ? FN<7, 4, __nv_bfloat16>(ARGS, SMEM, st) : FN<7, 4, float>(ARGS, SMEM, st);   \
-      return bf16 ? FN<7, 8, __nv_bfloat16>(ARGS, SMEM, st) : FN<7, 8, float>(ARGS, SMEM, st);               \
-    }                                                                          \
-    if (S == 14) {                                                             \
-      if (R == 4) return bf16 ? FN<14, 4, __nv_bfloat16>(ARGS, SMEM, st) : FN<14, 4, float>(ARGS, SMEM, st); \
-      return bf16 ? FN<14, 8, __nv_bfloat16>(ARGS, SMEM, st) : FN<14, 8, float>(ARGS, SMEM, st);             \
-    }                                                                          \
-    if (R == 4) return bf16 ? FN<16, 4, __nv_bfloat16>(ARGS, SMEM, st) : FN<16, 4, float>(ARGS, SMEM, st);   \
-    return bf16 ? FN<16, 8, __nv_bfloat16>(ARGS, SMEM, st) : FN<16, 8, float>(ARGS, SMEM, st);               \
-  } while (0)
-
-cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int S, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int kind, int R, bool bf16, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
   SmBatch<SmPass1Args> b;
   size_t smem = 0;
@@ -1473,13 +1617,13 @@ cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int S, int R, b
   b.first[0] = 0;
   for (int l = 0; l < n; ++l) {
     b.a[l] = a[l];
-    b.first[l + 1] = b.first[l] + a[l].n_tiles_b + sm_pass1_role_c_ctas(S, a[l].B);
-    const size_t need = sm_pass1_smem(S, R, a[l].B, a[l].C);
+    b.first[l + 1] = b.first[l] + pass1_grid(a[l]);
+    const size_t need = sm_pass1_smem(a[l], kind, R);
     if (need > smem) smem = need;
-    bytes += (double)a[l].B * a[l].C * S * S * (bf16 ? 2 : 4);
+    bytes += (double)a[l].B * a[l].C * a[l].H * a[l].W * (bf16 ? 2 : 4);
   }
   ProfScope prof(ASI_K_SM_PASS1, st, bytes);
-  ASI_DISPATCH_SRB(launch_pass1_bt, b, smem);
+  ASI_DISPATCH_KR(launch_pass1_bt, b, smem, st);
 }
 
 cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunks, int n, cudaStream_t st) {
@@ -1495,7 +1639,7 @@ cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunk
   return launch_pdl(k_sm_reduce_b, dim3((unsigned)b.first[n], 4), dim3(kRedNT), 0, st, b);
 }
 
-cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int S, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
   SmBatch<SmCoreArgs> b;
   size_t smem = 0;
@@ -1505,12 +1649,12 @@ cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int S, int R, boo
   for (int l = 0; l < n; ++l) {
     b.a[l] = a[l];
     b.first[l + 1] = b.first[l] + a[l].n_tiles;
-    const size_t need = sm_core_smem(S, R, a[l].B);
+    const size_t need = sm_core_smem(a[l], R);
     if (need > smem) smem = need;
-    bytes += (double)a[l].B * a[l].C * S * S * (bf16 ? 2 : 4);
+    bytes += (double)a[l].B * a[l].C * a[l].H * a[l].W * (bf16 ? 2 : 4);
   }
   ProfScope prof(ASI_K_SM_CORE, st, bytes);
-  ASI_DISPATCH_SRB(launch_core_bt, b, smem);
+  ASI_DISPATCH_R(launch_core_bt, b, smem, st);
 }
 
 cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, cudaStream_t st) {
