@@ -46,10 +46,18 @@ void choose_kernels(asi_plan* pl) {
   if (H * W <= 256 && H <= 32 && W <= 32 && B <= 1024 && C <= 4096) {
     pl->fast_kind = (H == W && (H == 7 || H == 14)) ? (int)H : 0;
     pl->fast_vec4 = (C * H * W) % 4 == 0;
-    sm_pass1_split((int)(H * W), (int)C, &pl->fast_cs, &pl->fast_cc);
+    sm_pass1_split((int)(H * W), (int)C, (int)B, &pl->fast_cs, &pl->fast_cc);
     pl->core_tile_c = sm_core_tile_c((int)(H * W), (int)C);
     pl->n_tiles_core = (int)((C + pl->core_tile_c - 1) / pl->core_tile_c);
     pl->n_tiles_b = sm_pass1_tiles_b(C * H * W, pl->fast_vec4);
+    // whole batches and whole samples as tiles of 512 threads where two such CTAs share an SM (7 x 7 maps: batches up
+    // to 64; at 128 the two kernels are level and the other one keeps all layers of a network in one launch)
+    pl->tile_S = 0;
+    if (H == W && (H == 7 || H == 14 || H == 16) && B % 8 == 0 && (H != 7 || (C % 4 == 0 && B <= 64)) &&
+        sm_tile1_smem((int)H, R, (int)B, (int)C) <= 113 * 1024) {
+      pl->tile_S = (int)H;
+      pl->n_tiles_b = (int)(H == 7 ? C / 4 : C);
+    }
     pl->fold_gs = 8;                                 // tiles per group of the core's two-level sum
     while ((pl->n_tiles_core + pl->fold_gs - 1) / pl->fold_gs > 192) pl->fold_gs *= 2;
     SmPass1Args a;
@@ -73,13 +81,21 @@ void choose_kernels(asi_plan* pl) {
     a.Ho = (int)pl->Ho; a.Wo = (int)pl->Wo; a.kh = pl->d.kh; a.kw = pl->d.kw; a.cpb = cpb;
     a.ph = pl->d.pad_h; a.pw = pl->d.pad_w; a.groups = pl->d.groups;
     a.vec4 = pl->wgrad_vec4 ? 1 : 0;
+    a.nt = 256;
     // term 5 expands the channels in two rounds when the staging blocks fit, else one at a time
+    // (one at a time, too, where two would keep the CTA from sharing its SM with three others)
     a.ncl = cpb >= 2 ? cpb / 2 : 1;
-    if (sm_wgrad_smem(a, R) > kSmemLimit) a.ncl = 1;
-    if (sm_wgrad_smem(a, R) <= kSmemLimit) {
+    if (sm_wgrad_smem(a, R) > 56 * 1024) a.ncl = 1;
+    // 256 threads where three such CTAs share an SM, else 512 where two do.  A CTA that needs an SM for itself pays on
+    // small maps only: larger ones recompute Z3 in every CTA, and four launches are faster (28 x 28, B = 128, seven
+    // layers: 118 us here against 28 us a layer beside other work)
+    const size_t need = sm_wgrad_smem(a, R);
+    if (need > 75 * 1024) a.nt = 512;
+    if (need <= 113 * 1024 || (need <= kSmemLimit && H * W <= 256)) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
       pl->wgrad_ncl = a.ncl;
+      pl->wgrad_nt = a.nt;
     }
   }
 }
@@ -146,7 +162,8 @@ void layout_compress(asi_plan* pl) {
     qps = (qps + 127) / 128 * 128;
     ns = (v.Q + qps - 1) / qps;
     if (pl->fast_compress) {                                             // one partial per column tile, per sample,
-      ns = m == 0 ? pl->n_tiles_b : (m == 1 ? pl->dims[0] : pl->dims[0] * pl->fast_cs);   // per role-C CTA; the cold-start
+      ns = m == 0 ? pl->n_tiles_b : (m == 1 ? pl->dims[0] : pl->dims[0] * pl->fast_cs);   // per role-C CTA (k_sm_tile1: per
+      if (pl->tile_S) ns = m == 1 ? sm_tile1_role_c_ctas(pl->tile_S, (int)pl->dims[0]) : pl->n_tiles_b;   // tile); the cold-start
       qps = ((v.Q + ns - 1) / ns + 127) / 128 * 128;                     // expansion splits the columns over at most as many
     }
     if (pl->fiber[m] || (pl->plane && m >= 2)) {                         // one partial per CTA of k_fiber /
@@ -279,7 +296,7 @@ void layout_wgrad(asi_plan* pl) {
 
 // the fused kernels read the activation four values at a time where its columns allow it
 bool fused_misaligned(const asi_plan* pl, const void* act) {
-  return pl->fast_vec4 && (reinterpret_cast<uintptr_t>(act) & (pl->bf16 ? 7u : 15u)) != 0;
+  return (pl->fast_vec4 || pl->tile_S) && (reinterpret_cast<uintptr_t>(act) & (pl->bf16 ? 7u : 15u)) != 0;
 }
 
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
@@ -316,6 +333,7 @@ void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev,
   a->W = (int)pl->dims[3];
   a->n_tiles_b = pl->n_tiles_b;
   a->cs = pl->fast_cs;
+  a->cl = pl->fast_cs;
   a->cc = pl->fast_cc;
   a->pitch = sm_pass1_pitch(a->H * a->W);
   a->off_u2 = sm_pass1_off_u2(pl->fast_R, a->cc, a->pitch);
@@ -323,6 +341,22 @@ void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev,
   a->bulk = (!pl->bf16 && pl->fast_vec4) ? 1 : 0;
   a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;      // 1 ms under the test hook, else 1 s
+}
+
+void build_tile1(const asi_plan* pl, const void* act, const float* U_prev, char* w, SmTile1Args* a) {
+  a->act = act;
+  a->U_prev = U_prev;
+  for (int m = 0; m < 4; ++m) {
+    a->Pp[m] = reinterpret_cast<float*>(w + pl->off_Pp[m]);
+    a->u_off[m] = pl->u_off[m];
+    a->r[m] = pl->r[m];
+  }
+  a->status = reinterpret_cast<int*>(w);
+  a->B = (int)pl->dims[0];
+  a->C = (int)pl->dims[1];
+  a->n_tiles_b = pl->n_tiles_b;
+  a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
+  a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;
 }
 
 int build_fused_reduce(const asi_plan* pl, char* w, const float* gram_U_prev, SmReduceArgs* ra) {
@@ -392,6 +426,7 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
   g->ph = pl->d.pad_h; g->pw = pl->d.pad_w; g->groups = pl->d.groups; g->cpb = pl->cpb;
   g->ncl = pl->wgrad_ncl;
   g->vec4 = pl->wgrad_vec4 ? 1 : 0;
+  g->nt = pl->wgrad_nt;
   if (g->vec4 && (reinterpret_cast<uintptr_t>(dY) & (pl->bf16 ? 7u : 15u))) return false;
   g->status = reinterpret_cast<int*>(w);
   g->bulk_store = (((pl->dims[1] / pl->d.groups) * pl->d.kh * pl->d.kw) % 4 == 0 &&
@@ -845,9 +880,15 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
   char* w = static_cast<char*>(ws);
   if (pl->fast_compress) {
     if (fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
-    SmPass1Args a;
-    build_fused_pass1(pl, act, U_prev, w, &a);
-    ASI_CUDA(launch_sm_pass1(a, pl->fast_kind, pl->fast_R, pl->bf16, st));
+    if (pl->tile_S) {
+      SmTile1Args a;
+      build_tile1(pl, act, U_prev, w, &a);
+      ASI_CUDA(launch_sm_tile1(a, pl->tile_S, pl->fast_R, pl->bf16, st));
+    } else {
+      SmPass1Args a;
+      build_fused_pass1(pl, act, U_prev, w, &a);
+      ASI_CUDA(launch_sm_pass1(a, pl->fast_kind, pl->fast_R, pl->bf16, st));
+    }
     return finish_compress(pl, act, U_new, core, w, U_prev, false, st);
   }
   for (int m = 0; m < pl->nd; ++m)                   // bulk and 16-byte copies; errors before anything is enqueued
@@ -957,11 +998,11 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
 // table the CTAs index; the remaining layers are enqueued one after another on the same stream.
 // ---------------------------------------------------------------------------------------------
 namespace {
-// layers that share launches: one kernel variant, one cluster size
+// layers that share launches
 struct Variant {
-  int kind, R, cs, bf16;
-  explicit Variant(const asi_plan* p) : kind(p->fast_kind), R(p->fast_R), cs(p->fast_cs), bf16(p->bf16 ? 1 : 0) {}
-  bool operator==(const Variant& o) const { return kind == o.kind && R == o.R && cs == o.cs && bf16 == o.bf16; }
+  int kind, tile, R, bf16;
+  explicit Variant(const asi_plan* p) : kind(p->fast_kind), tile(p->tile_S), R(p->fast_R), bf16(p->bf16 ? 1 : 0) {}
+  bool operator==(const Variant& o) const { return kind == o.kind && tile == o.tile && R == o.R && bf16 == o.bf16; }
 };
 }  // namespace
 
@@ -1004,18 +1045,21 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (g == 1)
       return asi_compress(plans[i0], acts[i0], U_prev[i0], U_new[i0], cores[i0], ws[i0], ws_bytes[i0], st);
     const asi_plan* p0 = plans[i0];
-    std::vector<SmPass1Args> pa(g);
+    std::vector<SmPass1Args> pa(p0->tile_S ? 0 : g);
+    std::vector<SmTile1Args> ta(p0->tile_S ? g : 0);
     std::vector<SmReduceArgs> ra(g);
     std::vector<SmCoreArgs> ca(g);
     std::vector<int> mc(g);
     for (int k = 0; k < g; ++k) {
       const int j = grp[k];
       char* w = static_cast<char*>(ws[j]);
-      build_fused_pass1(plans[j], acts[j], U_prev[j], w, &pa[k]);
+      if (p0->tile_S) build_tile1(plans[j], acts[j], U_prev[j], w, &ta[k]);
+      else build_fused_pass1(plans[j], acts[j], U_prev[j], w, &pa[k]);
       mc[k] = build_fused_reduce(plans[j], w, U_prev[j], &ra[k]);
       build_fused_core(plans[j], acts[j], U_new[j], cores[j], w, true, &ca[k]);
     }
-    ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_kind, p0->fast_R, p0->bf16, st));
+    if (p0->tile_S) ASI_CUDA(launch_sm_tile1_batched(ta.data(), g, p0->tile_S, p0->fast_R, p0->bf16, st));
+    else ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_kind, p0->fast_R, p0->bf16, st));
     ASI_CUDA(launch_sm_reduce_batched(ra.data(), mc.data(), g, st));
     ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_R, p0->bf16, st));
     return ASI_OK;
@@ -1042,7 +1086,8 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     std::vector<int> grp(1, i);
     if (plans[i]->fast_wgrad)
       for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j)
-        if (!done[j] && plans[j]->fast_wgrad && plans[j]->fast_R == plans[i]->fast_R && plans[j]->bf16 == plans[i]->bf16)
+        if (!done[j] && plans[j]->fast_wgrad && plans[j]->fast_R == plans[i]->fast_R && plans[j]->bf16 == plans[i]->bf16 &&
+            plans[j]->wgrad_nt == plans[i]->wgrad_nt)
           grp.push_back(j);
     for (int j : grp) done[j] = 1;
     chains.push_back(std::move(grp));

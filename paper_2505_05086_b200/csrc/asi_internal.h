@@ -109,7 +109,18 @@ struct ConvTailArgs {
 
 // Fused small-map conv kernels (asi_smallmap_kernels.cu)
 constexpr int kRedRows = 8;          // rows of P per CTA in the partial-reduction kernel
-struct SmPass1Args {
+struct SmTile1Args {            // k_sm_tile1
+  const void* act;
+  const float* U_prev;
+  float* Pp[ASI_MAX_MODES];     // per-mode partials [nsplit][a_m][r_m]
+  int* status;                  // status word (int 0) and completion counters (ints 16..255) of the workspace
+  int64_t u_off[ASI_MAX_MODES];
+  int r[ASI_MAX_MODES];
+  int B, C, n_tiles_b;
+  unsigned long long wait_ns;   // limit of the bounded wait on the bulk-copy barrier
+  int stall_copy;               // test hook: the producer arms the barrier but issues no copy (the wait must expire)
+};
+struct SmPass1Args {            // k_sm_pass1
   const void* act;
   const float* U_prev;
   float* Pp[ASI_MAX_MODES];     // per-mode partials [nsplit][a_m][r_m]
@@ -118,6 +129,7 @@ struct SmPass1Args {
   int r[ASI_MAX_MODES];
   int B, C, H, W, n_tiles_b;    // n_tiles_b: role-B CTAs (column tiles of all samples)
   int cs, cc, pitch, off_u2;    // role C: CTAs per sample, channels per CTA, floats per channel, start of U_2 in shared memory
+  int cl;                       // cluster size of the launch, a multiple of cs
   int vec4;                     // columns may be read four at a time (C H W % 4 == 0, 16-byte aligned base)
   int bulk;                     // role C's tile comes by bulk copies (fp32, vec4)
   unsigned long long wait_ns;   // limit of the bounded wait on the bulk-copy barrier
@@ -169,12 +181,17 @@ struct SmWgradArgs {
   int r[ASI_MAX_MODES];
   int B, C, Cout, H, W, Ho, Wo, kh, kw, sh, sw, ph, pw, groups, cpb;
   int vec4;                     // columns of dY may be read four at a time
+  int nt;                       // threads per CTA: 256 or 512
   int ncl;                      // output channels expanded per round of term 5 (divides cpb)
   int bulk_store;               // 1: dW row blocks leave through the bulk-copy engine (16-byte sized and aligned)
 };
+size_t sm_tile1_smem(int S, int R, int B, int C);
+int sm_tile1_role_c_ctas(int S, int B);
+cudaError_t launch_sm_tile1(const SmTile1Args& p, int S, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_tile1_batched(const SmTile1Args* a, int n, int S, int R, bool bf16, cudaStream_t st);
 size_t sm_pass1_smem(const SmPass1Args& p, int kind, int R);
 int sm_pass1_pitch(int HW);
-void sm_pass1_split(int HW, int C, int* cs, int* cc);
+void sm_pass1_split(int HW, int C, int B, int* cs, int* cc);
 int sm_pass1_off_u2(int R, int cc, int pitch);
 int sm_pass1_tiles_b(int64_t chw, bool vec4);
 int sm_core_tile_c(int HW, int C);
@@ -455,5 +472,6 @@ struct asi_plan {
   bool fiber2[ASI_MAX_MODES];      // ... by its register-tiled successor (ranks <= 4, 16-byte aligned rows)
   bool plane2;                     // 28 x 28 and 56 x 56 planes, ranks <= 4
   int fast_kind;                   // 7, 14: modes 3 and 4 as Gram matrices of such square maps; 0: any map of at most 256 positions
-  int fast_R, n_tiles_b, fast_cs, fast_cc, core_tile_c, n_tiles_core, cpb, wgrad_ncl, fold_gs;
+  int tile_S;                      // != 0: the first pass is k_sm_tile1 for this map size, else k_sm_pass1
+  int fast_R, n_tiles_b, fast_cs, fast_cc, core_tile_c, n_tiles_core, cpb, wgrad_ncl, wgrad_nt, fold_gs;
 };

@@ -23,7 +23,6 @@ namespace asi {
 
 namespace {
 
-constexpr int kNT = 512;             // threads per CTA of k_sm_wgrad
 constexpr int kRedNT = 256;          // threads per CTA of the partial-reduction kernel
 
 
@@ -117,10 +116,10 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src, int byte
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
 }
 // dst[k*RD + j] = j < r ? src[k*r + j] : 0 for k < rows: a factor [rows x r] padded to RD columns
-template <int RD>
+template <int RD, int NT>
 __device__ __forceinline__ void fac_issue_padded(const float* __restrict__ src, float* dst, int rows, int r) {
 #pragma unroll 1
-  for (int idx = threadIdx.x; idx < rows * RD; idx += kNT) {
+  for (int idx = threadIdx.x; idx < rows * RD; idx += NT) {
     const int k = idx / RD, j = idx % RD;
     cp_async4(dst + idx, src + (j < r ? k * r + j : 0), j < r ? 4 : 0);
   }
@@ -128,6 +127,25 @@ __device__ __forceinline__ void fac_issue_padded(const float* __restrict__ src, 
 __device__ __forceinline__ void fac_wait() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
+// two packed fp32 values (fma.rn.f32x2): one instruction, two multiply-adds
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void ffma2(f2& d, f2 a, f2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+__device__ __forceinline__ f2 fmul2(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
 template <int R>
 __device__ __forceinline__ void fma_row(float (&acc)[R], float x, const float* __restrict__ u) {
 #pragma unroll
@@ -192,8 +210,9 @@ __host__ __device__ constexpr int tri_index(int S, int k, int k2) {   // k <= k2
 // A unit is a quarter of a plane (fibers == part mod 4), so the lanes of a warp hit 32 banks; this
 // thread takes units u0, u0 + ustride, ...  es = step between the elements of a fiber, cs = step
 // between neighbouring fibers (mode 3: 14, 1; mode 4: 1, 14).
+template <int es, int cs>
 __device__ __forceinline__ void gram14_accumulate(const float* __restrict__ Xs, int PJ, int nunits, int u0, int ustride,
-                                                  int role, int es, int cs, float (&acc)[32]) {
+                                                  int role, float (&acc)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) acc[i] = 0.f;
   for (int un = u0; un < nunits; un += ustride) {
@@ -251,8 +270,8 @@ __device__ __forceinline__ void gram14_slot(int o, int& rl, int& e) {
 //
 // Role B (mode 1), one CTA per 128 neighbouring columns (c, h, w): lane = four columns, warp w = the samples b == w
 // (mod 8).  The activation goes straight from memory to registers -- a warp reads 512 contiguous bytes per sample --
-// V_1 of the columns meets in shared memory, and at ranks <= 4 the same registers feed the expansion (no tile is
-// staged, so nothing but the registers limits how many CTAs share an SM).
+// V_1 of the columns meets in shared memory, and the expansion reads the 64 KB again (from L1 or L2).  Holding the
+// tile in registers instead cost half the CTAs per SM and was slower: 102 against .. us on the MobileNetV2 tail.
 //
 // Role C (modes 2, 3, 4), a cluster of `cs` CTAs per sample, each with cc channels of it in shared memory (one bulk
 // copy): V_2 is the sum of the CTAs' shares through distributed shared memory, P_2 of the CTA's own channels follows
@@ -289,57 +308,96 @@ template <> struct RawCol<__nv_bfloat16, 1> {
   __device__ __forceinline__ void get(float (&x)[1]) const { x[0] = __bfloat162float(v); }
 };
 
+// upper triangle of G = A_m A_m^T over the planes pl0, pl0 + 128, .. of a 7 x 7 map
+template <int es, int cs>
+__device__ __forceinline__ void gram7_accumulate(const float* __restrict__ Xs, int nc, int pl0, float (&acc)[32]) {
+#pragma unroll 1
+  for (int pl = pl0; pl < nc; pl += 128) {
+    const float* base = Xs + pl * 49;
+#pragma unroll 1
+    for (int col = 0; col < 7; ++col, base += cs) {
+      float x[7];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) x[k] = base[k * es];
+#pragma unroll
+      for (int k = 0; k < 7; ++k)
+#pragma unroll
+        for (int k2 = k; k2 < 7; ++k2) acc[tri_index(7, k, k2)] = fmaf(x[k], x[k2], acc[tri_index(7, k, k2)]);
+    }
+  }
+}
+
+// Y[col][:] += x[col] u[:] over a thread's VW columns with column pairs packed: acc[p][j] holds columns 2 p, 2 p + 1
+template <int R>
+__device__ __forceinline__ void fma_pairs(f2 (&acc)[2][R], float4 x, const f2* __restrict__ ud) {      // ud[j] = (u_j, u_j)
+  const f2 x01 = pack2(x.x, x.y), x23 = pack2(x.z, x.w);
+#pragma unroll
+  for (int j = 0; j < R; j += 2) {
+    const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(ud + j);
+    ffma2(acc[0][j], x01, u.x); ffma2(acc[1][j], x23, u.x);
+    ffma2(acc[0][j + 1], x01, u.y); ffma2(acc[1][j + 1], x23, u.y);
+  }
+}
+
 template <int R, int VW, typename TX>
 __device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, float* smem) {
-  constexpr int JT = 32 * VW, NBH = 16, BPG = 32 / R;         // samples per thread and chunk; samples per reduction
-  constexpr bool kHold = (R == 4);
+  constexpr int JT = 32 * VW, BPG = 32 / R;          // columns; samples per thread and butterfly of the expansion
+  constexpr int U = 8;                               // samples in flight per thread
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int B = p.B, r1 = p.r[0];
   const int64_t chw = (int64_t)p.C * p.H * p.W;
-  float* U1s = smem;                                 // [B][R]
-  float* part = U1s + ((B * R + 3) & ~3);            // [8][JT][R]
-  float* V1s = part + 8 * JT * R;                    // [JT][R]
+  f2* U1d = reinterpret_cast<f2*>(smem);             // [B][R]: (u, u)
+  float* part = smem + 2 * B * R;                    // [8][R][JT]
+  float* V1s = part + 8 * JT * R;                    // [R][JT]
   for (int idx = tid; idx < B * R; idx += kPT) {
     const int k = idx / R, j = idx % R;
-    cp_async4(U1s + idx, p.U_prev + p.u_off[0] + (j < r1 ? k * r1 + j : 0), j < r1 ? 4 : 0);
+    const float* src = p.U_prev + p.u_off[0] + (j < r1 ? k * r1 + j : 0);
+    cp_async4(reinterpret_cast<float*>(U1d + idx), src, j < r1 ? 4 : 0);
+    cp_async4(reinterpret_cast<float*>(U1d + idx) + 1, src, j < r1 ? 4 : 0);
   }
   const int64_t col = (int64_t)tile * JT + VW * lane;
   const bool con = col < chw;
-  const TX* A = reinterpret_cast<const TX*>(p.act) + (con ? col : 0);
-  RawCol<TX, VW> x[NBH];
-  float v[VW][R];
+  const int nb = B > warp ? (B - warp + 7) / 8 : 0;  // samples of this warp: warp, warp + 8, ..
+  const TX* A = reinterpret_cast<const TX*>(p.act) + (con ? col : 0) + (nb > 0 ? (int64_t)warp * chw : 0);
+  const int64_t step = 8 * chw;
+  f2 acc[2][R];                                      // VW == 1: the low half of acc[0]
 #pragma unroll
-  for (int c = 0; c < VW; ++c)
+  for (int c = 0; c < 2; ++c)
 #pragma unroll
-    for (int j = 0; j < R; ++j) v[c][j] = 0.f;
+    for (int j = 0; j < R; ++j) acc[c][j] = 0ull;
   bool waited = false;
-  for (int bb = 0; bb < B; bb += 8 * NBH) {
+#pragma unroll 1
+  for (int t0 = 0; t0 < nb || !waited; t0 += U) {
+    RawCol<TX, VW> x[U];
 #pragma unroll
-    for (int t = 0; t < NBH; ++t) {
-      const int b = bb + warp + 8 * t;
-      x[t].load(A + (int64_t)(b < B ? b : B - 1) * chw);
-    }
+    for (int t = 0; t < U; ++t) x[t].load(A + (int64_t)(t0 + t < nb ? t0 + t : 0) * step);
     if (!waited) {
       fac_wait();
       __syncthreads();
       waited = true;
     }
 #pragma unroll
-    for (int t = 0; t < NBH; ++t) {
-      const int b = bb + warp + 8 * t;
-      if (b < B) {                                   // warp-uniform
+    for (int t = 0; t < U; ++t) {
+      if (t0 + t < nb) {                             // warp-uniform
         float xs[VW];
         x[t].get(xs);
+        const f2* ud = U1d + (warp + 8 * (t0 + t)) * R;
+        if constexpr (VW == 4) {
+          fma_pairs<R>(acc, make_float4(xs[0], xs[1], xs[2], xs[3]), ud);
+        } else {
 #pragma unroll
-        for (int c = 0; c < VW; ++c) fma_row<R>(v[c], xs[c], U1s + b * R);
+          for (int j = 0; j < R; ++j) ffma2(acc[0][j], pack2(xs[0], 0.f), ud[j]);
+        }
       }
     }
   }
+  // V_1 of the tile, [j][column]: the eight warps' shares meet in warp order
 #pragma unroll
-  for (int c = 0; c < VW; ++c)
-#pragma unroll
-    for (int j = 0; j < R; j += 4)
-      *reinterpret_cast<float4*>(part + (warp * JT + VW * lane + c) * R + j) = make_float4(v[c][j], v[c][j + 1], v[c][j + 2], v[c][j + 3]);
+  for (int j = 0; j < R; ++j) {
+    float* dst = part + (warp * R + j) * JT + VW * lane;
+    if constexpr (VW == 4) *reinterpret_cast<ulonglong2*>(dst) = make_ulonglong2(acc[0][j], acc[1][j]);
+    else *dst = unpack2(acc[0][j]).x;
+  }
   __syncthreads();
   for (int idx = tid; idx < JT * R; idx += kPT) {
     float s = part[idx];
@@ -350,45 +408,45 @@ __device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, flo
   __syncthreads();
   pdl_launch_dependents();
 #pragma unroll
-  for (int c = 0; c < VW; ++c)
-#pragma unroll
-    for (int j = 0; j < R; j += 4) {
-      const float4 s = con ? *reinterpret_cast<const float4*>(V1s + (VW * lane + c) * R + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      v[c][j] = s.x; v[c][j + 1] = s.y; v[c][j + 2] = s.z; v[c][j + 3] = s.w;
+  for (int j = 0; j < R; ++j) {
+    if constexpr (VW == 4) {
+      const ulonglong2 s = *reinterpret_cast<const ulonglong2*>(V1s + j * JT + 4 * lane);
+      acc[0][j] = con ? s.x : 0ull;
+      acc[1][j] = con ? s.y : 0ull;
+    } else {
+      acc[0][j] = con ? pack2(V1s[j * JT + lane], 0.f) : 0ull;
     }
+  }
   // P1[b,:] = sum over the tile's columns of X[b][col] V1[col,:]: BPG samples meet in one butterfly of 32 values
   float* P1 = p.Pp[0] + (int64_t)tile * B * r1;
-  const bool held = kHold && B <= 8 * NBH;
+  const int e = scatter_base<32>(lane), eb = warp + 8 * (e / R), ej = e % R;
 #pragma unroll 1
-  for (int bb = 0; bb < B; bb += 8 * NBH) {
-    if (!held) {
+  for (int t0 = 0; t0 < nb; t0 += BPG) {
+    RawCol<TX, VW> x[BPG];
 #pragma unroll
-      for (int t = 0; t < NBH; ++t) {
-        const int b = bb + warp + 8 * t;
-        x[t].load(A + (int64_t)(b < B ? b : B - 1) * chw);
-      }
-    }
+    for (int q = 0; q < BPG; ++q) x[q].load(A + (int64_t)(t0 + q < nb ? t0 + q : nb - 1) * step);
+    float val[32];
 #pragma unroll
-    for (int t0 = 0; t0 < NBH; t0 += BPG) {
-      if (bb + warp + 8 * t0 < B) {                  // warp-uniform
-        float val[32];
+    for (int q = 0; q < BPG; ++q) {
+      float xs[VW];
+      x[q].get(xs);
+      if constexpr (VW == 4) {
+        const f2 x01 = pack2(xs[0], xs[1]), x23 = pack2(xs[2], xs[3]);
 #pragma unroll
-        for (int q = 0; q < BPG; ++q) {
-          float xs[VW];
-          x[t0 + q].get(xs);
-#pragma unroll
-          for (int j = 0; j < R; ++j) {
-            float s = 0.f;
-#pragma unroll
-            for (int c = 0; c < VW; ++c) s = fmaf(xs[c], v[c][j], s);
-            val[q * R + j] = s;
-          }
+        for (int j = 0; j < R; ++j) {
+          f2 s = fmul2(x01, acc[0][j]);
+          ffma2(s, x23, acc[1][j]);
+          const float2 h = unpack2(s);
+          val[q * R + j] = h.x + h.y;
         }
-        warp_reduce_scatter<32>(val, lane);
-        const int e = scatter_base<32>(lane), b = bb + warp + 8 * (t0 + e / R), j = e % R;
-        if (b < B && j < r1) P1[b * r1 + j] = val[0];
+      } else {
+#pragma unroll
+        for (int j = 0; j < R; ++j) val[q * R + j] = xs[0] * unpack2(acc[0][j]).x;
       }
     }
+    warp_reduce_scatter<32>(val, lane);
+    const int b = eb + 8 * t0;
+    if (b < B && ej < r1) P1[b * r1 + ej] = val[0];
   }
 }
 
@@ -464,8 +522,9 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ int s_flag;
   namespace cg = cooperative_groups;
-  const int C = p.C, H = KIND ? KIND : p.H, W = KIND ? KIND : p.W, HW = H * W, P = p.pitch, cs = p.cs;
-  const int b = bid / cs, rank = bid - b * cs;
+  const int C = p.C, H = KIND ? KIND : p.H, W = KIND ? KIND : p.W, HW = H * W, P = KIND ? KIND * KIND : p.pitch, cs = p.cs;
+  const bool synced = p.cl > 1;                      // CTAs of several samples may share a cluster; all take its barriers
+  const int b = bid / cs, rank = bid - b * cs, rank0 = (bid % p.cl) - rank;   // rank0: the sample's first CTA in the cluster
   const int c0 = rank * p.cc, nc = (C - c0 < p.cc) ? (C > c0 ? C - c0 : 0) : p.cc;
   const int r2 = p.r[1];
   float* Xs = smem;                                  // [cc][P]
@@ -538,7 +597,7 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
   if (bulk && nc > 0) ok = cta_wait_tile(&s_bar, &s_flag, p.status, p.wait_ns);
   else __syncthreads();
   // ---- this CTA's share of V_2: thread (g, hw) sums the channels c == g (mod G)
-  const int G = kPT / HW;                            // HW <= 256
+  const int G = kPT / HW;                            // HW <= 256; a constant on the Gram kinds
   {
     const FDiv dHW(HW);
     int g, hw;
@@ -562,33 +621,21 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
       }
     }
   }
-  if (cs > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  if (synced) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   else __syncthreads();
   // ---- modes 3 and 4 while the other CTAs of the cluster finish their shares
   if (KIND == 7 || KIND == 14) {
-    const int mode = 2 + (warp >> 2), wq = warp & 3;  // warps 0-3: mode 3, warps 4-7: mode 4
-    const int es = mode == 2 ? W : 1, st = mode == 2 ? 1 : W;
+    const int wq = warp & 3;                         // warps 0-3: mode 3, warps 4-7: mode 4
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+    const int n = ok ? nc : 0;
     if (KIND == 7) {
-      // upper triangle of G, one plane per thread at a time (odd pitch: 32 lanes, 32 banks)
-      if (ok)
-        for (int pl = wq * 32 + lane; pl < nc; pl += 128) {
-          const float* base = Xs + pl * P;
-#pragma unroll 1
-          for (int col = 0; col < 7; ++col) {
-            float xv[7];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) xv[k] = base[col * st + k * es];
-#pragma unroll
-            for (int k = 0; k < 7; ++k)
-#pragma unroll
-              for (int k2 = k; k2 < 7; ++k2) acc[tri_index(7, k, k2)] = fmaf(xv[k], xv[k2], acc[tri_index(7, k, k2)]);
-          }
-        }
-    } else if (ok) {
-      gram14_accumulate(Xs, P, nc * 4, lane, 32, wq, es, st, acc);
+      if (warp < 4) gram7_accumulate<7, 1>(Xs, n, wq * 32 + lane, acc);
+      else gram7_accumulate<1, 7>(Xs, n, wq * 32 + lane, acc);
+    } else {
+      if (warp < 4) gram14_accumulate<14, 1>(Xs, P, n * 4, lane, 32, wq, acc);
+      else gram14_accumulate<1, 14>(Xs, P, n * 4, lane, 32, wq, acc);
     }
     warp_reduce_scatter<32>(acc, lane);
     float* gr = Vp;                                  // [8][32] (Vp is at least that large; its sums are in V2l)
@@ -617,19 +664,19 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
   }
   pdl_launch_dependents();
   // ---- V_2 = the shares of the cluster, in rank order
+  if (synced) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
   if (cs > 1) {
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     cg::cluster_group cluster = cg::this_cluster();
     for (int idx = tid; idx < HW * R; idx += kPT) {
-      float s = cluster.map_shared_rank(V2l, 0)[idx];
-      for (int q = 1; q < cs; ++q) s += cluster.map_shared_rank(V2l, q)[idx];
+      float s = cluster.map_shared_rank(V2l, rank0)[idx];
+      for (int q = 1; q < cs; ++q) s += cluster.map_shared_rank(V2l, rank0 + q)[idx];
       V2s[idx] = s;
     }
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // the shares have been read
-    __syncthreads();
   } else {
     V2s = V2l;
   }
+  if (synced) asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // the shares have been read
+  __syncthreads();
   // ---- P_2 of the CTA's channels: thread = four channels q, q + Q, .. and a share of the positions
   const int Q = (nc + 3) >> 2;
   if (ok && nc > 0) {
@@ -699,7 +746,7 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
       }
     }
   }
-  if (cs > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (synced) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 template <int KIND, int R, typename TX>
@@ -707,13 +754,441 @@ __device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
   if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
-  if (bid >= p.B * p.cs) {
-    const int tile = bid - p.B * p.cs;
+  const int nc_ctas = (p.B * p.cs + p.cl - 1) / p.cl * p.cl;
+  if (bid >= nc_ctas) {
+    const int tile = bid - nc_ctas;
     if (tile >= p.n_tiles_b) return;                 // padding to whole clusters
     if (p.vec4) pass1_role_b<R, 4, TX>(p, tile, smem);
     else pass1_role_b<R, 1, TX>(p, tile, smem);
-  } else {
+  } else if (bid < p.B * p.cs) {
     pass1_role_c<KIND, R, TX>(p, bid, smem);
+  } else {                                           // padding: only the cluster's barriers
+    for (int i = 0; i < 2; ++i) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// k_sm_tile1: the first pass for S x S maps, S in {7, 14, 16}, and batches that are a multiple of 8, where the tiles of
+// two CTAs of 512 threads fit an SM (ResNet-18 tail: 19 against 28 us of k_sm_pass1, whose smaller CTAs repeat more
+// set-up; a 16 x 16 layer of eight samples: 6.4 against 13 us).  CTAs of role B hold a tile [all B x J contiguous
+// (c, h, w)] with whole mode-1/3/4 fibers (one half of the CTA iterates mode 1 while the other does modes 3 and 4);
+// CTAs of role C hold one sample [all C x HW] (larger maps: a quarter of its positions) for mode 2.
+// ---------------------------------------------------------------------------------------------
+constexpr int kTT = 512;             // threads per CTA
+constexpr int kNG = 256;             // threads of one half (warp-specialised phases)
+
+__host__ __device__ constexpr int pitch4(int J) {      // >= J, multiple of 4, == 4 (mod 32)
+  int p = (J + 3) / 4 * 4;
+  while (p % 32 != 4) p += 4;
+  return p;
+}
+
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+template <typename TX>
+__device__ __forceinline__ float4 ld4(const TX* p);
+template <>
+__device__ __forceinline__ float4 ld4<float>(const float* p) {
+  return *reinterpret_cast<const float4*>(p);
+}
+template <>
+__device__ __forceinline__ float4 ld4<__nv_bfloat16>(const __nv_bfloat16* p) {
+  const uint2 raw = *reinterpret_cast<const uint2*>(p);
+  const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
+  const __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
+  return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
+}
+
+// Starts the copy of `rows` fp32 rows of J values (J a multiple of 4, both sides 16-byte aligned): row i
+// from src + i*src_stride to dst + i*PJ, 16 bytes per cp.async, one row per warp at a time.  (One bulk
+// copy per row would leave the issuing warp busy for ~60 cycles per row: the tile of a 64-sample
+// batch would arrive ~2 us later.)
+__device__ __forceinline__ void stage_rows_async(float* dst, const float* __restrict__ src, int rows, int J,
+                                                 int64_t src_stride, int PJ) {
+  const int lane = threadIdx.x & 31, nv = J >> 2;
+  for (int i = threadIdx.x >> 5; i < rows; i += kTT / 32) {
+    const float* s = src + i * src_stride;
+    float* d = dst + i * PJ;
+    for (int v = lane; v < nv; v += 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(d + 4 * v)), "l"(s + 4 * v) : "memory");
+  }
+}
+
+__device__ __forceinline__ void bar_sync(int id, int nthreads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// Number of interleaved sample groups project_batch uses for a tile of J columns on nthr threads.
+__host__ __device__ constexpr int batch_groups(int nthr, int J) {
+  const int items = J / 2;
+  int nh = nthr / items;
+  return nh < 1 ? 1 : (nh > 4 ? 4 : nh);
+}
+
+// out[j][0..R) = sum_b Xs[b*PJ + j] * Us[b*R + ..] for j < J: the mode-1 contraction of a staged tile
+// [B x J].  Runs on `nthr` threads (t = 0..nthr-1) that synchronise on named barrier `bar`.  A thread
+// owns two neighbouring columns (one 8-byte shared load per sample) and the samples b == h (mod NH);
+// the NH partial sums meet in `part` ([NH][J][R]) in a fixed order.
+template <int R>
+__device__ __forceinline__ void project_batch(const float* __restrict__ Xs, int PJ,
+                                              const float* __restrict__ Us, int B, int J,
+                                              float* __restrict__ part, float* __restrict__ out, int t,
+                                              int nthr, int bar) {
+  const int NH = batch_groups(nthr, J);
+  const int J2 = J >> 1;                             // J is even
+  const FDiv dJ2(J2);
+#pragma unroll 1
+  for (int it = t; it < NH * J2; it += nthr) {
+    int h, jp;
+    dJ2.divmod(it, h, jp);
+    float a0[R], a1[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) a0[q] = a1[q] = 0.f;
+#pragma unroll 4
+    for (int b = h; b < B; b += NH) {
+      const float2 x = *reinterpret_cast<const float2*>(Xs + b * PJ + 2 * jp);
+      fma_row<R>(a0, x.x, Us + b * R);
+      fma_row<R>(a1, x.y, Us + b * R);
+    }
+    float* dst = (NH > 1 ? part + h * J * R : out) + 2 * jp * R;
+#pragma unroll
+    for (int q = 0; q < R; q += 4) {
+      *reinterpret_cast<float4*>(dst + q) = make_float4(a0[q], a0[q + 1], a0[q + 2], a0[q + 3]);
+      *reinterpret_cast<float4*>(dst + R + q) = make_float4(a1[q], a1[q + 1], a1[q + 2], a1[q + 3]);
+    }
+  }
+  if (NH > 1) {
+    bar_sync(bar, nthr);
+#pragma unroll 1
+    for (int idx = t; idx < J * R; idx += nthr) {
+      float s = 0.f;
+      for (int h = 0; h < NH; ++h) s += part[h * J * R + idx];
+      out[idx] = s;
+    }
+  }
+  bar_sync(bar, nthr);
+}
+
+// V[hw][:] = sum_c Xs[c*PC + hw] * Us[c][:] for a staged block Xs [C][HWC] of one sample (the mode-2
+// projection of HWC positions).  Thread (g, hw) sums the channels c = g (mod G); group 0 writes V
+// itself, groups 1..G-1 write Vp ([G-1][HWC][R]; may alias Us: it is written only after every thread
+// has finished reading Us) and the sums meet in a fixed order.  All kTT threads call it.
+template <int HWC, int PC, int R>
+__device__ __forceinline__ void project_channels(const float* __restrict__ Xs, const float* Us, float* Vp,
+                                                 float* V, int C) {
+  constexpr int G = kTT / HWC;
+  const int tid = threadIdx.x;
+  float acc[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) acc[j] = 0.f;
+  const int g = tid / HWC, hw = tid - g * HWC;
+  if (g < G) {
+#pragma unroll 4
+    for (int c = g; c < C; c += G) fma_row<R>(acc, Xs[c * PC + hw], Us + c * R);
+  }
+  if (G > 1) __syncthreads();
+  if (g < G) {
+    float* dst = (g == 0 ? V : Vp + (g - 1) * HWC * R) + hw * R;
+#pragma unroll
+    for (int j = 0; j < R; j += 4)
+      *reinterpret_cast<float4*>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+  }
+  __syncthreads();
+  if (G > 1) {
+    for (int idx = tid; idx < HWC * R; idx += kTT) {
+      float s = V[idx];
+#pragma unroll
+      for (int gg = 0; gg < G - 1; ++gg) s += Vp[gg * HWC * R + idx];
+      V[idx] = s;
+    }
+    __syncthreads();
+  }
+}
+
+// Stages one tile [B x J] (row b at src + b*sample_stride) as fp32 rows of pitch PJ.
+template <typename TX>
+__device__ __forceinline__ void stage_tile_begin(const TX* __restrict__ src, int64_t sample_stride, float* Xs,
+                                                 int B, int J, int PJ) {
+  if constexpr (std::is_same<TX, float>::value) {
+    stage_rows_async(Xs, src, B, J, sample_stride, PJ);
+  } else {
+    const int J4 = J / 4;
+    for (int idx = threadIdx.x; idx < B * J4; idx += kTT) {
+      const int b = idx / J4, v = idx - b * J4;
+      *reinterpret_cast<float4*>(Xs + b * PJ + 4 * v) = ld4<TX>(src + b * sample_stride + 4 * v);
+    }
+  }
+}
+
+// Role C of the first pass takes the positions of a sample in NQ parts.  S = 7: the whole map.  Larger
+// maps: four parts that start on 16-byte boundaries -- 14 x 14 splits its 49 float4 per channel as
+// 13 + 12 + 12 + 12 (parts 1..3 carry four zero columns), 16 x 16 as 4 x 16.
+__host__ __device__ constexpr int role_c_hwc(int S) { return S == 7 ? 49 : (S == 14 ? 52 : S * S / 4); }
+__host__ __device__ constexpr int role_c_pitch(int S) { return S == 7 ? 49 : pitch4(role_c_hwc(S)); }
+
+template <int S, int R, typename TX>
+__device__ __forceinline__ void sm_tile1_cta(const SmTile1Args& p, const int bid) {
+  constexpr bool kBulk = std::is_same<TX, float>::value;
+  constexpr bool kGram = (S == 7);                   // modes 3, 4 as Gram matrices A_m A_m^T (7 x 7)
+  constexpr bool kGram14 = (S == 14);                // ... as 14 x 14 Gram matrices in four 7 x 7 blocks
+  constexpr int HW = S * S;
+  constexpr int CC = (S == 7) ? 4 : 1;               // channels per role-B tile
+  constexpr int J = CC * HW;                         // contiguous elements per sample in a tile
+  constexpr int PJ = pitch4(J);                      // row pitch == 4 (mod 32): conflict-free (b, j) reads
+  constexpr int NH1 = batch_groups(kNG, J);
+  extern __shared__ __align__(128) float smem[];
+  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ int s_flag;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const TX* __restrict__ A = reinterpret_cast<const TX*>(p.act);
+  const int B = p.B, C = p.C;
+
+  if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
+
+  constexpr int kNQ = (S == 7) ? 1 : 4;             // role-C CTAs per sample
+  if (bid >= B * kNQ) {
+    // ---------------- role B: modes 1, 3, 4 on tile [B x J] ----------------
+    const int tile = bid - B * kNQ;
+    float* Xs = smem;                                // [B][PJ]
+    float* U1s = Xs + B * PJ;                        // [B][R]
+    float* U3s = U1s + B * R;                        // [S][R]
+    float* U4s = U3s + S * R;                        // [S][R]
+    float* V1s = U4s + S * R;                        // [J][R]
+    float* part = V1s + J * R;                       // [NH1][J][R] (NH1 > 1 only)
+    float* red = part + (NH1 > 1 ? NH1 : 0) * J * R; // [8][32], S = 14: [8 + 16][32]
+    fac_issue_padded<R, kTT>(p.U_prev + p.u_off[0], U1s, B, p.r[0]);
+    if constexpr (!kGram && !kGram14) {
+      fac_issue_padded<R, kTT>(p.U_prev + p.u_off[2], U3s, S, p.r[2]);
+      fac_issue_padded<R, kTT>(p.U_prev + p.u_off[3], U4s, S, p.r[3]);
+    }
+    stage_tile_begin<TX>(A + (int64_t)tile * J, (int64_t)C * HW, Xs, B, J, PJ);
+    fac_wait();
+    __syncthreads();
+    const int t = tid & (kNG - 1), wg = t >> 5;
+    if (tid < kNG) {
+      // ---- half 0: mode 1.  V[j,:] = sum_b X[b,j] U1[b,:], then P1[b,:] = sum_j X[b,j] V[j,:]
+      project_batch<R>(Xs, PJ, U1s, B, J, part, V1s, t, kNG, 1);
+      float* P1 = p.Pp[0] + (int64_t)tile * B * p.r[0];
+      const int bl = lane >> 2, jl = lane & 3;       // a warp covers 8 samples x 4 column phases
+      for (int b0 = wg * 8; b0 < B; b0 += 64) {
+        const int b = b0 + bl;
+        float acc[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[q] = 0.f;
+#pragma unroll 7
+        for (int jj = jl; jj < J; jj += 4) fma_row<R>(acc, Xs[b * PJ + jj], V1s + jj * R);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
+          acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 2);
+        }
+        if (jl == 0) {
+#pragma unroll
+          for (int q = 0; q < R; ++q)
+            if (q < p.r[0]) P1[b * p.r[0] + q] = acc[q];
+        }
+      }
+    } else if constexpr (kGram) {
+      // ---- half 1, S = 7: G_m = A_m A_m^T for m = 3, 4, one plane (b, c) per thread at a time; the
+      // 32 lanes of a warp touch 32 different banks.  P_m = G_m U_m^prev follows in k_sm_reduce.
+      constexpr int NACC = 32;
+      static_assert(S * (S + 1) / 2 <= NACC, "upper triangle of the Gram matrix");
+      const int nplanes = B * CC;
+#pragma unroll 1
+      for (int mode = 2; mode <= 3; ++mode) {
+        const int es = (mode == 2) ? S : 1;          // step between the elements of a fiber
+        const int cs = (mode == 2) ? 1 : S;          // step between neighbouring fibers
+        float* Gm = p.Pp[mode] + (int64_t)tile * HW;
+        float acc[NACC];
+#pragma unroll
+        for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
+        for (int pl = t; pl < nplanes; pl += kNG) {
+          const int b = pl / CC, cl = pl % CC;
+          const float* base = Xs + b * PJ + cl * HW;
+#pragma unroll 1
+          for (int col = 0; col < S; ++col) {
+            const float* colp = base + col * cs;
+            float x[S];
+#pragma unroll
+            for (int k = 0; k < S; ++k) x[k] = colp[k * es];
+#pragma unroll
+            for (int k = 0; k < S; ++k)
+#pragma unroll
+              for (int k2 = k; k2 < S; ++k2) acc[tri_index(S, k, k2)] = fmaf(x[k], x[k2], acc[tri_index(S, k, k2)]);
+          }
+        }
+        warp_reduce_scatter<NACC>(acc, lane);
+        red[wg * 32 + scatter_base<NACC>(lane)] = acc[0];
+        bar_sync(2, kNG);
+        for (int o = t; o < HW; o += kNG) {
+          const int k = o / S, k2 = o % S;
+          const int e = (k <= k2) ? tri_index(S, k, k2) : tri_index(S, k2, k);
+          float s = 0.f;
+#pragma unroll
+          for (int w = 0; w < 8; ++w) s += red[w * 32 + e];
+          Gm[o] = s;
+        }
+        bar_sync(2, kNG);
+      }
+    } else if constexpr (kGram14) {
+      // ---- half 1, S = 14: G_3 = A_3 A_3^T (see gram14_accumulate); G_4 follows on all sixteen warps
+      const int role = wg & 3;
+      float* Gm = p.Pp[2] + (int64_t)tile * HW;
+      float acc[32];
+      gram14_accumulate<S, 1>(Xs, PJ, B * 4, (wg >> 2) * 32 + lane, 64, role, acc);
+      warp_reduce_scatter<32>(acc, lane);
+      red[wg * 32 + scatter_base<32>(lane)] = acc[0];
+      bar_sync(2, kNG);
+      for (int o = t; o < HW; o += kNG) {
+        int rl, e;
+        gram14_slot(o, rl, e);
+        Gm[o] = red[rl * 32 + e] + red[(rl + 4) * 32 + e];
+      }
+    } else {
+      // ---- half 1, other sizes: P_m = A_m (A_m^T U_m^prev) for m = 3, 4.  A unit is a quarter of a plane
+      // (columns == part mod 4); unit -> thread so that the 32 lanes of a warp touch 32 different
+      // banks.  Each thread owns 2 columns of the factor; warp w serves column pair w mod JH.
+      constexpr int TPP = 4, JT = 2, JH = R / JT, NACC = 32;
+      static_assert(S * JT <= NACC, "accumulators of one thread");
+      const int jh = wg % JH;
+      const int u0 = (wg / JH) * 32 + lane;
+      const int nunits = B * CC * TPP;
+#pragma unroll 1
+      for (int mode = 2; mode <= 3; ++mode) {
+        const float* Us = ((mode == 2) ? U3s : U4s) + jh * JT;
+        const int es = (mode == 2) ? S : 1;
+        const int cs = (mode == 2) ? 1 : S;
+        const int rm = p.r[mode];
+        float* Pm = p.Pp[mode] + (int64_t)tile * S * rm;
+        float acc[NACC];
+#pragma unroll
+        for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
+        for (int un = u0; un < nunits; un += kNG / JH) {
+          const int pl = un / TPP, part_ = un % TPP;
+          const int b = pl / CC, cl = pl % CC;
+          const float* base = Xs + b * PJ + cl * HW;
+#pragma unroll 1
+          for (int col = part_; col < S; col += TPP) {
+            const float* colp = base + col * cs;
+            float x[S], v0 = 0.f, v1 = 0.f;
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+              x[k] = colp[k * es];
+              const float2 u = *reinterpret_cast<const float2*>(Us + k * R);
+              v0 = fmaf(x[k], u.x, v0);
+              v1 = fmaf(x[k], u.y, v1);
+            }
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+              acc[2 * k] = fmaf(x[k], v0, acc[2 * k]);
+              acc[2 * k + 1] = fmaf(x[k], v1, acc[2 * k + 1]);
+            }
+          }
+        }
+        warp_reduce_scatter<NACC>(acc, lane);
+        red[wg * 32 + scatter_base<NACC>(lane)] = acc[0];
+        bar_sync(2, kNG);
+        for (int o = t; o < S * R; o += kNG) {
+          const int k = o / R, j = o % R;
+          const int e = k * JT + (j % JT);
+          float s = 0.f;
+          for (int w = j / JT; w < 8; w += JH) s += red[w * 32 + e];
+          if (j < rm) Pm[k * rm + j] = s;
+        }
+        bar_sync(2, kNG);
+      }
+    }
+    if constexpr (kGram14) {
+      // ---- S = 14, G_4 = A_4 A_4^T: each half joins as it finishes its first job (mode 1 or G_3)
+      const int gw = tid >> 5, role = gw & 3;
+      float* red4 = red + 8 * 32;                    // [16][32]
+      float acc[32];
+      gram14_accumulate<1, S>(Xs, PJ, B * 4, (gw >> 2) * 32 + lane, 128, role, acc);
+      warp_reduce_scatter<32>(acc, lane);
+      red4[gw * 32 + scatter_base<32>(lane)] = acc[0];
+      __syncthreads();
+      float* Gm = p.Pp[3] + (int64_t)tile * HW;
+      for (int o = tid; o < HW; o += kTT) {
+        int rl, e;
+        gram14_slot(o, rl, e);
+        Gm[o] = ((red4[rl * 32 + e] + red4[(rl + 4) * 32 + e]) + red4[(rl + 8) * 32 + e]) + red4[(rl + 12) * 32 + e];
+      }
+    }
+  } else {
+    // ---------------- role C: mode 2 on block [C x HWC] of one sample ----------------
+    // S = 7: the whole sample (contiguous, staged by the bulk-copy engine, odd row pitch for the
+    // row-per-thread reads below); larger maps: one part of the positions, rows staged by 16-byte
+    // cp.async at a pitch == 4 (mod 32), read back as float4.
+    constexpr int NQ = (S == 7) ? 1 : 4;
+    constexpr int HWC = role_c_hwc(S);
+    constexpr int PC = role_c_pitch(S);
+    constexpr int G = kTT / HWC;
+    constexpr bool kBulkC = kBulk && NQ == 1;
+    const int b = bid / NQ, q = bid % NQ;
+    const int hw0 = (S == 14) ? (q == 0 ? 0 : 4 + 48 * q) : q * HWC;     // first position of this part
+    const int nval = (S == 14 && q > 0) ? 48 : HWC;                      // positions it holds
+    float* Xs = smem;                                // [C][PC]
+    float* U2s = Xs + ((C * PC + 3) & ~3);           // [C][R]
+    float* V2s = U2s + C * R;                        // [HWC][R]
+    float* Vp = (C >= (G - 1) * HWC) ? U2s : V2s + HWC * R;   // [G-1][HWC][R]: on top of U2s when it fits
+    const TX* Xb = A + (int64_t)b * C * HW + hw0;
+    if constexpr (kBulkC)
+      stage_block(&s_bar, reinterpret_cast<char*>(Xs), reinterpret_cast<const char*>(Xb), (uint32_t)C * HW * 4u,
+                  p.stall_copy != 0);
+    fac_issue_padded<R, kTT>(p.U_prev + p.u_off[1], U2s, C, p.r[1]);
+    if constexpr (kBulkC) {
+    } else if constexpr (NQ == 1) {
+      const int n4 = C * HW / 4;
+      for (int idx = tid; idx < n4; idx += kTT) *reinterpret_cast<float4*>(Xs + 4 * idx) = ld4<TX>(Xb + 4 * idx);
+    } else {
+      constexpr int NV = HWC / 4;
+      const int n = C * NV;
+#pragma unroll 1
+      for (int idx = tid; idx < n; idx += kTT) {
+        const int c = idx / NV, v = idx - c * NV;
+        float* dst = Xs + c * PC + 4 * v;
+        const TX* src = Xb + (int64_t)c * HW + 4 * v;
+        if (4 * v >= nval) {
+          *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+        } else if constexpr (kBulk) {
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+        } else {
+          *reinterpret_cast<float4*>(dst) = ld4<TX>(src);
+        }
+      }
+    }
+    fac_wait();
+    if constexpr (kBulkC) {
+      if (!cta_wait_tile(&s_bar, &s_flag, p.status, p.wait_ns)) return;
+    } else {
+      __syncthreads();
+    }
+    project_channels<HWC, PC, R>(Xs, U2s, Vp, V2s, C);
+    // expansion: P2[c,:] = sum_hw X[c,hw] V2[hw,:], one channel row per thread
+    float* P2 = p.Pp[1] + (int64_t)bid * C * p.r[1];
+    for (int c = tid; c < C; c += kTT) {
+      const float* row = Xs + c * PC;
+      float acc[R];
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[j] = 0.f;
+      if constexpr (NQ == 1) {
+#pragma unroll 7
+        for (int hw = 0; hw < HWC; ++hw) fma_row<R>(acc, row[hw], V2s + hw * R);
+      } else {
+#pragma unroll 2
+        for (int hw = 0; hw < HWC; hw += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(row + hw);
+          fma_row<R>(acc, x.x, V2s + hw * R);
+          fma_row<R>(acc, x.y, V2s + (hw + 1) * R);
+          fma_row<R>(acc, x.z, V2s + (hw + 2) * R);
+          fma_row<R>(acc, x.w, V2s + (hw + 3) * R);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (j < p.r[1]) P2[c * p.r[1] + j] = acc[j];
+    }
   }
 }
 
@@ -732,12 +1207,22 @@ __device__ __forceinline__ int batch_layer(const SmBatch<Args>& b, int bid) {
   return l;
 }
 
+template <int S, int R, typename TX>
+__global__ void __launch_bounds__(kTT, 2) k_sm_tile1(const __grid_constant__ SmTile1Args p) {
+  sm_tile1_cta<S, R, TX>(p, (int)blockIdx.x);
+}
+template <int S, int R, typename TX>
+__global__ void __launch_bounds__(kTT, 2) k_sm_tile1_b(const __grid_constant__ SmBatch<SmTile1Args> b) {
+  const int l = batch_layer(b, (int)blockIdx.x);
+  sm_tile1_cta<S, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+}
+
 template <int KIND, int R, typename TX>
-__global__ void __launch_bounds__(kPT, 2) k_sm_pass1(const __grid_constant__ SmPass1Args p) {
+__global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1(const __grid_constant__ SmPass1Args p) {
   sm_pass1_cta<KIND, R, TX>(p, (int)blockIdx.x);
 }
 template <int KIND, int R, typename TX>
-__global__ void __launch_bounds__(kPT, 2) k_sm_pass1_b(const __grid_constant__ SmBatch<SmPass1Args> b) {
+__global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1_b(const __grid_constant__ SmBatch<SmPass1Args> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
   sm_pass1_cta<KIND, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
@@ -929,10 +1414,13 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
 //   core[i,j,k,l] = sum_c U2[c,j] M[c][i,k,l] by the last CTA of every group of tiles, then over the groups by the last
 //     group, both in index order.
 // ---------------------------------------------------------------------------------------------
-template <int R, int VW, typename TX>
+// W[col][:] = sum_b X[b][col] U1[b][:] for the tile's J columns (jvalid of them exist): thread = VW neighbouring columns
+// and the samples b == h (mod NH), eight in flight, the NH shares meet in order.  The first eight are requested before
+// `factors` (the row solves, which end with a barrier) runs.
+template <int R, int VW, typename TX, typename F>
 __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t chw, int B, int J, int jvalid,
                                              const float* __restrict__ U1s, float* __restrict__ part, float* __restrict__ Ws,
-                                             bool wait_rows) {
+                                             F&& factors) {
   constexpr int U = 8;
   const int tid = threadIdx.x;
   const int JV = (J + VW - 1) / VW, NH = kPT / JV;
@@ -946,25 +1434,29 @@ __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t c
   for (int c = 0; c < VW; ++c)
 #pragma unroll
     for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
-  if (h >= NH) h = 0;
-  for (int b0 = h; (on && b0 < B) || wait_rows; b0 += U * NH) {
+  const int nb = on && B > h ? (B - h + NH - 1) / NH : 0;   // samples of this thread
+  if (!on) h = 0;
+  src += (int64_t)h * chw;
+  const int64_t step = (int64_t)NH * chw;
+  bool first = true;
+#pragma unroll 1
+  for (int t0 = 0; t0 < nb || first; t0 += U) {
     RawCol<TX, VW> x[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) x[u].load(src + (int64_t)(b0 + u * NH < B ? b0 + u * NH : B - 1) * chw);
-    if (wait_rows) {                                 // uniform: every thread's first batch
-      __syncthreads();                               // the factor rows are there
-      wait_rows = false;
+    for (int t = 0; t < U; ++t) x[t].load(src + (int64_t)(t0 + t < nb ? t0 + t : 0) * step);
+    if (first) {                                     // uniform: every thread's first batch
+      factors();
+      first = false;
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int b = b0 + u * NH;
-      if (b < B) {
+    for (int t = 0; t < U; ++t)
+      if (t0 + t < nb) {
         float xs[VW];
-        x[u].get(xs);
+        x[t].get(xs);
+        const float* u = U1s + (h + (t0 + t) * NH) * R;
 #pragma unroll
-        for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], U1s + b * R);
+        for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], u);
       }
-    }
   }
   if (on) {
     float* dst = part + (h * J + jq * VW) * R;
@@ -998,51 +1490,51 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   float* Ws = U4s + W * R;              // [J][R]
   float* part = Ws + J * R;             // [NH][J][R], at most 256 * 4 R
   float* T1 = part;                     // [ncl r1][r3][W] after part is free
-  pdl_wait();                           // P_m and the Cholesky factors come from the reduction kernel
-  // ---- the Cholesky factors of the four modes (computed once, by the reduction kernel)
-  for (int e = tid; e < 4 * kRfStride; e += kPT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
-  // ---- factor rows: [U1: B rows][the tile's rows of U2][U3: H][U4: W]
-  const int nrows = B + ncl + H + W;
-  double prow[R];
-  bool synced = false;
+  auto factors = [&]() {
+    pdl_wait();                         // P_m and the Cholesky factors come from the reduction kernel
+    // factor rows: [U1: B rows][the tile's rows of U2][U3: H][U4: W]
+    const int nrows = B + ncl + H + W;
+    bool synced = false;
 #pragma unroll 1
-  for (int row = tid; row < nrows || !synced; row += kPT) {
-    int m = 0, k = row;
-    float* rdst = U1s + k * R;
-    bool owner = tile == 0;
-    if (row >= B + ncl + H) { m = 3; k = row - B - ncl - H; rdst = U4s + k * R; }
-    else if (row >= B + ncl) { m = 2; k = row - B - ncl; rdst = U3s + k * R; }
-    else if (row >= B) { m = 1; k = c0 + row - B; rdst = nullptr; owner = true; }
-    const int rr = p.r[m];
-    const bool on = row < nrows;
+    for (int row = tid; row < nrows || !synced; row += kPT) {
+      int m = 0, k = row;
+      float* rdst = U1s + k * R;
+      bool owner = tile == 0;
+      if (row >= B + ncl + H) { m = 3; k = row - B - ncl - H; rdst = U4s + k * R; }
+      else if (row >= B + ncl) { m = 2; k = row - B - ncl; rdst = U3s + k * R; }
+      else if (row >= B) { m = 1; k = c0 + row - B; rdst = nullptr; owner = true; }
+      const int rr = p.r[m];
+      const bool on = row < nrows;
+      double q[R];
 #pragma unroll
-    for (int j = 0; j < R; ++j) prow[j] = (on && j < rr) ? __ldcg(p.Pred[m] + (int64_t)k * rr + j) : 0.0;
-    if (!synced) {
-      __syncthreads();
-      synced = true;
-    }
-    if (!on) break;
-    float* gdst = p.U_new + p.u_off[m] + (int64_t)k * rr;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      float out = 0.f;
-      if (j < rr) {
-        double v = prow[j];
-#pragma unroll
-        for (int i = 0; i < R; ++i)
-          if (i < j) v = fma(-prow[i], Rs[m][i * 8 + j], v);
-        v *= Rs[m][64 + j];
-        prow[j] = v;
-        out = (float)v;
-        if (owner) gdst[j] = out;
+      for (int j = 0; j < R; ++j) q[j] = (on && j < rr) ? __ldcg(p.Pred[m] + (int64_t)k * rr + j) : 0.0;
+      if (!synced) {                    // the Cholesky factors of the four modes travel with the first rows
+        for (int e = tid; e < 4 * kRfStride; e += kPT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
+        __syncthreads();
+        synced = true;
       }
-      if (rdst) rdst[j] = out;
+      if (!on) break;
+      float* gdst = p.U_new + p.u_off[m] + (int64_t)k * rr;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        float out = 0.f;
+        if (j < rr) {
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+            if (i < j) q[j] = fma(-q[i], Rs[m][i * 8 + j], q[j]);
+          q[j] *= Rs[m][64 + j];
+          out = (float)q[j];
+          if (owner) gdst[j] = out;
+        }
+        if (rdst) rdst[j] = out;
+      }
     }
-  }
+    __syncthreads();
+  };
   const TX* A = reinterpret_cast<const TX*>(p.act) + (int64_t)c0 * HW;
   const int64_t chw = (int64_t)C * HW;
-  if (p.vec4) core_project<R, 4, TX>(A, chw, B, J, jvalid, U1s, part, Ws, true);
-  else core_project<R, 1, TX>(A, chw, B, J, jvalid, U1s, part, Ws, true);
+  if (p.vec4) core_project<R, 4, TX>(A, chw, B, J, jvalid, U1s, part, Ws, factors);
+  else core_project<R, 1, TX>(A, chw, B, J, jvalid, U1s, part, Ws, factors);
   // T1[cl,i][k][w] = sum_h W[cl,h,w][i] U3[h][k]
   const FDiv dW(W), d_r1(r1), d_r3(r3), d_r4(r4);
   for (int idx = tid; idx < ncl * r1 * r3 * W; idx += kPT) {
@@ -1080,16 +1572,18 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   __threadfence();
   {
     const int ch0 = gfirst * CC, nch = ((gfirst + gsize) * CC < C ? (gfirst + gsize) * CC : C) - ch0;
-    float* u2 = part;                   // [nch][r2] (gs CC r2 floats: fits, checked by the host)
-    for (int e = tid; e < nch * r2; e += kPT) u2[e] = __ldcg(p.U_new + p.u_off[1] + (int64_t)ch0 * r2 + e);
+    float* u2 = part;                   // [nch][R] (gs CC R floats: fits, checked by the host)
+    for (int e = tid; e < nch * R; e += kPT) {
+      const int c = e / R, j = e % R;
+      u2[e] = j < r2 ? __ldcg(p.U_new + p.u_off[1] + (int64_t)(ch0 + c) * r2 + j) : 0.f;
+    }
     __syncthreads();
-    const FDiv d34(r3 * r4), d_r2(r2);
-    for (int idx = tid; idx < ce; idx += kPT) {
-      int ij, kl, i, j;
-      d34.divmod(idx, ij, kl);
-      d_r2.divmod(ij, i, j);
-      const float* src = p.Tp + (int64_t)ch0 * ce3 + i * r3 * r4 + kl;
-      float s = 0.f;
+    // thread = one (i, k, l), all j: the channels' numbers are read once, 16 in flight
+    for (int e = tid; e < ce3; e += kPT) {
+      float s[R];
+#pragma unroll
+      for (int j = 0; j < R; ++j) s[j] = 0.f;
+      const float* src = p.Tp + (int64_t)ch0 * ce3 + e;
 #pragma unroll 1
       for (int c = 0; c < nch; c += 16) {
         float v[16];
@@ -1097,9 +1591,13 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
         for (int q = 0; q < 16; ++q) v[q] = __ldcg(src + (int64_t)(c + q < nch ? c + q : c) * ce3);
 #pragma unroll
         for (int q = 0; q < 16; ++q)
-          if (c + q < nch) s = fmaf(v[q], u2[(c + q) * r2 + j], s);
+          if (c + q < nch) fma_row<R>(s, v[q], u2 + (c + q) * R);
       }
-      p.Tg[(int64_t)grp * ce + idx] = s;
+      const int i = e / (r3 * r4), kl = e - i * (r3 * r4);
+      float* dst = p.Tg + (int64_t)grp * ce + (int64_t)i * r2 * r3 * r4 + kl;
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (j < r2) dst[j * r3 * r4] = s[j];
     }
   }
   __threadfence();
@@ -1112,6 +1610,26 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   if (!s_last) return;
   __threadfence();
   // few core elements: thread (e, q) sums the groups == q (mod nq) of element e, the nq sums meet in index order
+  if (ce > kPT && ngroups <= 8) {       // a wide core from few groups: four elements x eight groups in flight
+#pragma unroll 1
+    for (int e0 = tid; e0 < ce; e0 += 4 * kPT) {
+      float v[4][8];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          v[u][k] = __ldcg(p.Tg + (int64_t)(k < ngroups ? k : 0) * ce + (e0 + u * kPT < ce ? e0 + u * kPT : e0));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        float s = v[u][0];
+#pragma unroll
+        for (int k = 1; k < 8; ++k) s += k < ngroups ? v[u][k] : 0.f;
+        if (e0 + u * kPT < ce) p.core[e0 + u * kPT] = s;
+      }
+    }
+    if (tid == 0) *p.counter = 0;
+    return;
+  }
   int nq = kPT / ce;
   nq = nq > 8 ? 8 : (nq < 1 ? 1 : nq);
   float* fold = part;                   // [nq][ce]
@@ -1142,11 +1660,11 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
 }
 
 template <int R, typename TX>
-__global__ void __launch_bounds__(kPT, 3) k_sm_core(const __grid_constant__ SmCoreArgs p) {
+__global__ void __launch_bounds__(kPT, R == 4 ? 4 : 3) k_sm_core(const __grid_constant__ SmCoreArgs p) {
   sm_core_cta<R, TX>(p, (int)blockIdx.x);
 }
 template <int R, typename TX>
-__global__ void __launch_bounds__(kPT, 3) k_sm_core_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
+__global__ void __launch_bounds__(kPT, R == 4 ? 4 : 3) k_sm_core_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
   sm_core_cta<R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
@@ -1168,7 +1686,7 @@ __global__ void __launch_bounds__(kPT, 3) k_sm_core_b(const __grid_constant__ Sm
 // (cp.async.bulk shared -> global) when a channel's block is 16-byte sized and aligned, else by
 // coalesced stores.  With more than one round there are two staging blocks, so that a round's stores
 // run under the next round's arithmetic: the write of dW by all CTAs at once is DRAM-bound.
-template <int R>
+template <int R, int kNT>
 __device__ __forceinline__ void wgrad_expand_rows(const SmWgradArgs& p, const float* __restrict__ Z4s,
                                                   const float* __restrict__ U2s, float* stage, int c0) {
   const int kk = p.kh * p.kw;
@@ -1248,17 +1766,17 @@ __device__ __forceinline__ void wgrad_expand_rows(const SmWgradArgs& p, const fl
 }
 
 // groups of samples a CTA of k_sm_wgrad splits the batch over (JV column items)
-__host__ __device__ inline int wgrad_groups(int JV) {
-  const int n = kNT / (JV < kNT ? JV : kNT);
+__host__ __device__ inline int wgrad_groups(int JV, int nt) {
+  const int n = nt / (JV < nt ? JV : nt);
   return n > 8 ? 8 : n;
 }
 // Z1[j][:] = sum_b dY[b][j] U1[b][:] for the CTA's J columns; thread = VW neighbouring columns and the samples
 // b == h (mod NH), eight of them in flight; the NH shares meet in order.  The factors' asynchronous copies of this
 // thread are waited for behind the first loads.
-template <int R, int VW, typename TX>
+template <int R, int VW, int kNT, typename TX>
 __device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t sstride, int B, int J, int NH,
                                               const float* __restrict__ U1s, float* __restrict__ part, float* __restrict__ Z1s) {
-  constexpr int U = R == 4 ? 8 : 4;                  // 64 registers a thread: two CTAs of 512
+  constexpr int U = 8;
   const int tid = threadIdx.x, JV = (J + VW - 1) / VW;
   const FDiv dJ(JV);
   bool waited = false;
@@ -1268,30 +1786,33 @@ __device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t
     const bool on = h < NH;
     const TX* src = dY + (on ? jq * VW : 0);
     if (!on) h = 0;
+    src += (int64_t)h * sstride;
+    const int nb = on && B > h ? (B - h + NH - 1) / NH : 0;     // samples of this thread
+    const int64_t step = (int64_t)NH * sstride;
     float acc[VW][R];
 #pragma unroll
     for (int c = 0; c < VW; ++c)
 #pragma unroll
       for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
-    for (int b0 = h; (on && b0 < B) || !waited; b0 += U * NH) {
+#pragma unroll 1
+    for (int t0 = 0; t0 < nb || !waited; t0 += U) {
       RawCol<TX, VW> x[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) x[u].load(src + (int64_t)(b0 + u * NH < B ? b0 + u * NH : B - 1) * sstride);
+      for (int u = 0; u < U; ++u) x[u].load(src + (int64_t)(t0 + u < nb ? t0 + u : 0) * step);
       if (!waited) {
         fac_wait();
         __syncthreads();
         waited = true;
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int b = b0 + u * NH;
-        if (b < B) {
+      for (int u = 0; u < U; ++u)
+        if (t0 + u < nb) {
           float xs[VW];
           x[u].get(xs);
+          const float* u1 = U1s + (h + (t0 + u) * NH) * R;
 #pragma unroll
-          for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], U1s + b * R);
+          for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], u1);
         }
-      }
     }
     if (on) {
       float* dst = part + (h * J + jq * VW) * R;
@@ -1310,7 +1831,7 @@ __device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t
   }
 }
 
-template <int R, typename TX>
+template <int R, int kNT, typename TX>
 __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
@@ -1320,7 +1841,7 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
   const int c0 = bid * p.cpb;
   // staging blocks of term 5 reuse the tile's space: ncl channels per round, doubled when rounds follow
   const int n_stage = (p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
-  const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV);
+  const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV, kNT);
   float* stage = smem;                               // term 5's blocks; before that the shares of Z1 [NH][J][R]
   float* part = smem;
   float* U1s = smem + ((NH * J * R > n_stage ? NH * J * R : n_stage) + 3) / 4 * 4;   // [B][R]
@@ -1344,12 +1865,12 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
       const bool in = k < r3 && l < r4;
       cp_async4(Ss + idx, p.core + (in ? (ij * r3 + k) * r4 + l : 0), in ? 4 : 0);
     }
-    fac_issue_padded<R>(p.U + p.u_off[2], U3s, H, r3);
-    fac_issue_padded<R>(p.U + p.u_off[3], U4s, W, r4);
-    fac_issue_padded<R>(p.U + p.u_off[0], U1s, p.B, r1);
-    fac_issue_padded<R>(p.U + p.u_off[1], U2s, p.C, r2);
-    if (p.vec4) wgrad_project<R, 4, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
-    else wgrad_project<R, 1, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
+    fac_issue_padded<R, kNT>(p.U + p.u_off[2], U3s, H, r3);
+    fac_issue_padded<R, kNT>(p.U + p.u_off[3], U4s, W, r4);
+    fac_issue_padded<R, kNT>(p.U + p.u_off[0], U1s, p.B, r1);
+    fac_issue_padded<R, kNT>(p.U + p.u_off[1], U2s, p.C, r2);
+    if (p.vec4) wgrad_project<R, 4, kNT, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
+    else wgrad_project<R, 1, kNT, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
   }
   // terms 2-3: Tm[ij][h][l] = sum_k S[ij][k][l] U3[h][k];  Z3[ij][h][w] = sum_l Tm[ij][h][l] U4[w][l]
   // (rank indices padded to R with zeros: every sum is a fixed-length dot product of 16-byte reads)
@@ -1429,30 +1950,45 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
   }
   __syncthreads();
   // term 5: dW[c0+cl, c, t] = sum_j Z4[cl][j][t] U2[(g cg + c), j]
-  wgrad_expand_rows<R>(p, Z4s, U2s, stage, c0);
+  wgrad_expand_rows<R, kNT>(p, Z4s, U2s, stage, c0);
 }
 
-template <int R, typename TX>
-__global__ void __launch_bounds__(kNT, 2) k_sm_wgrad(const __grid_constant__ SmWgradArgs p) {
-  sm_wgrad_cta<R, TX>(p, (int)blockIdx.x);
+template <int R, int NT, typename TX>
+__global__ void __launch_bounds__(NT, (R == 4 ? 1024 : 512) / NT) k_sm_wgrad(const __grid_constant__ SmWgradArgs p) {
+  sm_wgrad_cta<R, NT, TX>(p, (int)blockIdx.x);
 }
-template <int R, typename TX>
-__global__ void __launch_bounds__(kNT, 2) k_sm_wgrad_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
+template <int R, int NT, typename TX>
+__global__ void __launch_bounds__(NT, (R == 4 ? 1024 : 512) / NT) k_sm_wgrad_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_wgrad_cta<R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_wgrad_cta<R, NT, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------------------------
+int sm_tile1_role_c_ctas(int S, int B) { return (S == 7) ? B : 4 * B; }
+
+size_t sm_tile1_smem(int S, int R, int B, int C) {
+  const int HW = S * S, CC = (S == 7) ? 4 : 1, J = CC * HW, PJ = pitch4(J);
+  const int NH1 = batch_groups(kNG, J);
+  const size_t role_b = (size_t)B * PJ + (size_t)B * R + 2 * S * R + (size_t)J * R +
+                        (NH1 > 1 ? (size_t)NH1 * J * R : 0) + 24 * 32;
+  const int HWC = role_c_hwc(S), PC = role_c_pitch(S);
+  const int G = kTT / HWC;
+  const size_t vp = (C >= (G - 1) * HWC) ? 0 : (size_t)(G - 1) * HWC * R;
+  const size_t role_c = (size_t)((C * PC + 3) & ~3) + (size_t)C * R + (size_t)HWC * R + vp;
+  return 4 * (role_b > role_c ? role_b : role_c);
+}
+
 int sm_pass1_pitch(int HW) { return HW % 4 == 0 && (HW / 4) % 2 == 0 ? HW + 4 : HW; }
 
-// CTAs per sample (a cluster) and channels per CTA: a sample of 32 or more channels goes to four CTAs, to eight where
-// four would hold more than 56 KB each
-void sm_pass1_split(int HW, int C, int* cs, int* cc) {
-  int n = C >= 32 ? 4 : 1;
+// CTAs per sample (they share a cluster) and channels per CTA: about 48 KB of the sample each, so that four CTAs share
+// an SM; a CTA of a few KB pays more for its set-up and reductions than for its share (a 160-channel 7 x 7 layer split
+// over four was slower than whole), but a small batch is spread over at least one CTA per SM
+void sm_pass1_split(int HW, int C, int B, int* cs, int* cc) {
+  int n = 1;
   auto per = [&](int k) { return ((C + k - 1) / k + 3) / 4 * 4; };
-  while (n < 8 && (size_t)per(n) * sm_pass1_pitch(HW) * 4 > 56 * 1024) n *= 2;
+  while (n < 8 && ((size_t)per(n) * sm_pass1_pitch(HW) * 4 > 50 * 1024 || (B * n < 148 && per(n) >= 16))) n *= 2;
   *cs = n;
   *cc = per(n);
 }
@@ -1463,7 +1999,7 @@ int sm_pass1_off_u2(int R, int cc, int pitch) {
 
 size_t sm_pass1_smem(const SmPass1Args& p, int kind, int R) {
   const int HW = p.H * p.W, JT = p.vec4 ? 128 : 32;
-  const size_t role_b = (size_t)((p.B * R + 3) & ~3) + (size_t)9 * JT * R;
+  const size_t role_b = (size_t)2 * p.B * R + (size_t)9 * JT * R;
   const size_t role_c = (size_t)p.off_u2 + (size_t)p.cc * R + (size_t)2 * HW * R + (size_t)(kPT / HW) * HW * R +
                         (kind == 0 ? (size_t)(p.H + p.W + 3 * 8 * 32) * R : 0);
   return 4 * (role_b > role_c ? role_b : role_c);
@@ -1480,7 +2016,7 @@ int sm_core_tile_c(int HW, int C) {
 size_t sm_core_smem(const SmCoreArgs& p, int R) {
   const int HW = p.H * p.W, J = p.tile_c * HW, VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW;
   size_t part = (size_t)(kPT / JV) * J * R;
-  const size_t t1 = (size_t)p.tile_c * p.r[0] * p.r[2] * p.W, u2 = (size_t)p.gs * p.tile_c * p.r[1];
+  const size_t t1 = (size_t)p.tile_c * p.r[0] * p.r[2] * p.W, u2 = (size_t)p.gs * p.tile_c * R;
   if (t1 > part) part = t1;
   if (u2 > part) part = u2;
   if (part < 8 * kPT) part = 8 * kPT;                // the final fold
@@ -1491,12 +2027,12 @@ size_t sm_wgrad_smem(const SmWgradArgs& p, int R) {
   const int r1 = p.r[0], r2 = p.r[1];
   const int J = p.cpb * p.Ho * p.Wo, kk = p.kh * p.kw, JV = p.vec4 ? J / 4 : J;
   const int N4 = r2 * kk;
-  const size_t part = (size_t)wgrad_groups(JV) * J * R,
+  const size_t part = (size_t)wgrad_groups(JV, p.nt) * J * R,
                stage = (size_t)(p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
   size_t n = ((part > stage ? part : stage) + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
              (size_t)r1 * r2 * R * R + (size_t)p.H * R + (size_t)p.W * R +
              (size_t)r1 * r2 * p.H * R + ((size_t)r1 * r2 * (p.H + 2 * p.ph) * (p.W + 2 * p.pw) + 3) / 4 * 4 +
-             (size_t)p.cpb * kk * R + (size_t)p.cpb * (N4 > kNT ? N4 : kNT);
+             (size_t)p.cpb * kk * R + (size_t)p.cpb * (N4 > p.nt ? N4 : p.nt);
   return 4 * n + 64;
 }
 
@@ -1519,11 +2055,13 @@ static cudaError_t launch_clustered(void (*kernel)(Arg), int grid, int cs, size_
   cfg.numAttrs = cs > 1 ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
-static int pass1_grid(const SmPass1Args& p) { return p.B * p.cs + (p.n_tiles_b + p.cs - 1) / p.cs * p.cs; }
+static int pass1_grid(const SmPass1Args& p) {
+  return (p.B * p.cs + p.cl - 1) / p.cl * p.cl + (p.n_tiles_b + p.cl - 1) / p.cl * p.cl;
+}
 
 template <int KIND, int R, typename TX>
 static cudaError_t launch_pass1_t(const SmPass1Args& p, size_t smem, cudaStream_t st) {
-  return launch_clustered(k_sm_pass1<KIND, R, TX>, pass1_grid(p), p.cs, smem, st, p);
+  return launch_clustered(k_sm_pass1<KIND, R, TX>, pass1_grid(p), p.cl, smem, st, p);
 }
 template <int R, typename TX>
 static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t st) {
@@ -1535,9 +2073,26 @@ static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t 
 template <int R, typename TX>
 static cudaError_t launch_wgrad_t(const SmWgradArgs& p, cudaStream_t st) {
   const size_t smem = sm_wgrad_smem(p, R);
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_wgrad<R, TX>), smem);
+  auto kernel = p.nt == 512 ? k_sm_wgrad<R, 512, TX> : k_sm_wgrad<R, 256, TX>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  k_sm_wgrad<R, TX><<<p.Cout / p.cpb, kNT, smem, st>>>(p);
+  kernel<<<p.Cout / p.cpb, p.nt, smem, st>>>(p);
+  return cudaGetLastError();
+}
+
+template <int S, int R, typename TX>
+static cudaError_t launch_tile1_t(const SmTile1Args& p, cudaStream_t st) {
+  const size_t smem = sm_tile1_smem(S, R, p.B, p.C);
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_tile1<S, R, TX>), smem);
+  if (e != cudaSuccess) return e;
+  k_sm_tile1<S, R, TX><<<p.n_tiles_b + sm_tile1_role_c_ctas(S, p.B), kTT, smem, st>>>(p);
+  return cudaGetLastError();
+}
+template <int S, int R, typename TX>
+static cudaError_t launch_tile1_bt(const SmBatch<SmTile1Args>& b, size_t smem, cudaStream_t st) {
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_tile1_b<S, R, TX>), smem);
+  if (e != cudaSuccess) return e;
+  k_sm_tile1_b<S, R, TX><<<b.first[b.n], kTT, smem, st>>>(b);
   return cudaGetLastError();
 }
 
@@ -1560,6 +2115,25 @@ static cudaError_t launch_wgrad_t(const SmWgradArgs& p, cudaStream_t st) {
     if (R == 4) return bf16 ? FN<4, __nv_bfloat16>(__VA_ARGS__) : FN<4, float>(__VA_ARGS__);             \
     return bf16 ? FN<8, __nv_bfloat16>(__VA_ARGS__) : FN<8, float>(__VA_ARGS__);                         \
   } while (0)
+
+#define ASI_DISPATCH_SR(FN, ...)                                                                         \
+  do {                                                                                                   \
+    if (S == 7) {                                                                                        \
+      if (R == 4) return bf16 ? FN<7, 4, __nv_bfloat16>(__VA_ARGS__) : FN<7, 4, float>(__VA_ARGS__);     \
+      return bf16 ? FN<7, 8, __nv_bfloat16>(__VA_ARGS__) : FN<7, 8, float>(__VA_ARGS__);                 \
+    }                                                                                                    \
+    if (S == 14) {                                                                                       \
+      if (R == 4) return bf16 ? FN<14, 4, __nv_bfloat16>(__VA_ARGS__) : FN<14, 4, float>(__VA_ARGS__);   \
+      return bf16 ? FN<14, 8, __nv_bfloat16>(__VA_ARGS__) : FN<14, 8, float>(__VA_ARGS__);               \
+    }                                                                                                    \
+    if (R == 4) return bf16 ? FN<16, 4, __nv_bfloat16>(__VA_ARGS__) : FN<16, 4, float>(__VA_ARGS__);     \
+    return bf16 ? FN<16, 8, __nv_bfloat16>(__VA_ARGS__) : FN<16, 8, float>(__VA_ARGS__);                 \
+  } while (0)
+
+cudaError_t launch_sm_tile1(const SmTile1Args& p, int S, int R, bool bf16, cudaStream_t st) {
+  ProfScope prof(ASI_K_SM_PASS1, st, (double)p.B * p.C * S * S * (bf16 ? 2 : 4));      // the activation, read once
+  ASI_DISPATCH_SR(launch_tile1_t, p, st);
+}
 
 cudaError_t launch_sm_pass1(const SmPass1Args& p, int kind, int R, bool bf16, cudaStream_t st) {
   const size_t eb = bf16 ? 2 : 4;
@@ -1592,7 +2166,7 @@ int sm_max_batch() { return kMaxBatch; }
 
 template <int KIND, int R, typename TX>
 static cudaError_t launch_pass1_bt(const SmBatch<SmPass1Args>& b, size_t smem, cudaStream_t st) {
-  return launch_clustered(k_sm_pass1_b<KIND, R, TX>, b.first[b.n], b.a[0].cs, smem, st, b);
+  return launch_clustered(k_sm_pass1_b<KIND, R, TX>, b.first[b.n], b.a[0].cl, smem, st, b);
 }
 template <int R, typename TX>
 static cudaError_t launch_core_bt(const SmBatch<SmCoreArgs>& b, size_t smem, cudaStream_t st) {
@@ -1602,10 +2176,29 @@ static cudaError_t launch_core_bt(const SmBatch<SmCoreArgs>& b, size_t smem, cud
 }
 template <int R, typename TX>
 static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_wgrad_b<R, TX>), smem);
+  auto kernel = b.a[0].nt == 512 ? k_sm_wgrad_b<R, 512, TX> : k_sm_wgrad_b<R, 256, TX>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  k_sm_wgrad_b<R, TX><<<b.first[b.n], kNT, smem, st>>>(b);
+  kernel<<<b.first[b.n], b.a[0].nt, smem, st>>>(b);
   return cudaGetLastError();
+}
+
+cudaError_t launch_sm_tile1_batched(const SmTile1Args* a, int n, int S, int R, bool bf16, cudaStream_t st) {
+  if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
+  SmBatch<SmTile1Args> b;
+  size_t smem = 0;
+  double bytes = 0.0;
+  b.n = n;
+  b.first[0] = 0;
+  for (int l = 0; l < n; ++l) {
+    b.a[l] = a[l];
+    b.first[l + 1] = b.first[l] + a[l].n_tiles_b + sm_tile1_role_c_ctas(S, a[l].B);
+    const size_t need = sm_tile1_smem(S, R, a[l].B, a[l].C);
+    if (need > smem) smem = need;
+    bytes += (double)a[l].B * a[l].C * S * S * (bf16 ? 2 : 4);
+  }
+  ProfScope prof(ASI_K_SM_PASS1, st, bytes);
+  ASI_DISPATCH_SR(launch_tile1_bt, b, smem, st);
 }
 
 cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int kind, int R, bool bf16, cudaStream_t st) {
@@ -1615,9 +2208,12 @@ cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int kind, int R
   double bytes = 0.0;
   b.n = n;
   b.first[0] = 0;
+  int cl = 1;                                        // the launch's cluster size: a multiple of every layer's split
+  for (int l = 0; l < n; ++l) cl = a[l].cs > cl ? a[l].cs : cl;
   for (int l = 0; l < n; ++l) {
     b.a[l] = a[l];
-    b.first[l + 1] = b.first[l] + pass1_grid(a[l]);
+    b.a[l].cl = cl;
+    b.first[l + 1] = b.first[l] + pass1_grid(b.a[l]);
     const size_t need = sm_pass1_smem(a[l], kind, R);
     if (need > smem) smem = need;
     bytes += (double)a[l].B * a[l].C * a[l].H * a[l].W * (bf16 ? 2 : 4);
