@@ -86,11 +86,12 @@ void choose_kernels(asi_plan* pl) {
     // (one at a time, too, where two would keep the CTA from sharing its SM with three others)
     a.ncl = cpb >= 2 ? cpb / 2 : 1;
     if (sm_wgrad_smem(a, R) > 56 * 1024) a.ncl = 1;
-    // 256 threads where three such CTAs share an SM, else 512 where two do.  A CTA that needs an SM for itself pays on
+    // 256 threads where three such CTAs share an SM and the stream of dY is short (at 128 x 784 values a CTA 512
+    // threads take 28 us against 36; at 128 x 196, 256 take 39 us against 46), else 512.  A CTA that needs an SM for itself pays on
     // small maps only: larger ones recompute Z3 in every CTA, and four launches are faster (28 x 28, B = 128, seven
     // layers: 118 us here against 28 us a layer beside other work)
     const size_t need = sm_wgrad_smem(a, R);
-    if (need > 75 * 1024) a.nt = 512;
+    if (need > 75 * 1024 || B * cpb * HoWo > 32768) a.nt = 512;
     if (need <= 113 * 1024 || (need <= kSmemLimit && H * W <= 256)) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
@@ -109,22 +110,27 @@ void layout_compress(asi_plan* pl) {
   pl->small_rank = !pl->fast_compress && rmax <= 8 && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY);
   for (int m = 0; m < ASI_MAX_MODES; ++m) {
     pl->fiber[m] = false;
+    pl->wfiber[m] = false;
     pl->fiber_grid[m] = 0;
   }
   pl->plane = false;
   pl->plane_grid = 0;
-  if (pl->small_rank && pl->d.kind == ASI_CONV2D && pl->dims[2] == pl->dims[3] && pl->dims[2] % 4 == 0 &&
-      pl->dims[2] >= 8 && pl->dims[2] <= 64 && plane_smem((int)pl->dims[2]) <= kSmemLimit) {
+  if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && pl->d.kind == ASI_CONV2D &&
+      wplane_supported(pl->dims[0] * pl->dims[1], pl->dims[2], pl->dims[3], pl->r[2], pl->r[3])) {
     pl->plane = true;
-    const int64_t np = 256 / pl->dims[2], planes = pl->dims[0] * pl->dims[1];
-    pl->plane_grid = (int)std::min<int64_t>((planes + np - 1) / np, 296);
+    pl->plane_grid = wplane_grid(pl->dims[0] * pl->dims[1], (int)pl->dims[2], (int)pl->dims[3],
+                                 std::max(pl->r[2], pl->r[3]), pl->bf16);
   }
   // one-pass kernel for every mode with a rank <= 8 and a short fiber, whatever the other modes' ranks
   if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY))
     for (int m = 0; m < pl->nd; ++m) {
       if (pl->plane && m >= 2) continue;
       const ModeView& v = pl->mv[m];
-      if (pl->r[m] <= 8 && v.a <= 128 && fiber_smem((int)v.a) <= kSmemLimit) {
+      pl->wfiber[m] = wfiber_supported(v.O, v.a, v.I, pl->r[m]);
+      if (pl->wfiber[m]) {
+        pl->fiber[m] = true;
+        pl->fiber_grid[m] = wfiber_grid(v.O, v.a, v.I, pl->r[m], pl->bf16);
+      } else if (pl->r[m] <= 8 && v.a <= 128 && fiber_smem((int)v.a) <= kSmemLimit) {
         pl->fiber[m] = true;
         pl->fiber_grid[m] = (int)std::min<int64_t>(fiber_tiles(v.O, v.a, v.I), 296);
       }
@@ -132,7 +138,7 @@ void layout_compress(asi_plan* pl) {
   // register-tiled successors where the shape fits them (one partial per CTA, fewer and larger CTAs)
   pl->plane2 = false;
   for (int m = 0; m < ASI_MAX_MODES; ++m) pl->fiber2[m] = false;
-  if (pl->plane && plane2_supported((int)pl->dims[2], pl->dims[0] * pl->dims[1], pl->r[2], pl->r[3])) {
+  if (pl->plane && pl->dims[2] == pl->dims[3] && plane2_supported((int)pl->dims[2], pl->dims[0] * pl->dims[1], pl->r[2], pl->r[3])) {
     pl->plane2 = true;
     pl->plane_grid = plane2_grid((int)pl->dims[2], pl->dims[0] * pl->dims[1],
                                  (pl->d.flags & ASI_FLAG_SHARE_SM) ? 148 : 296);
@@ -140,6 +146,7 @@ void layout_compress(asi_plan* pl) {
   for (int m = 0; m < pl->nd; ++m)
     if (pl->fiber[m] && fiber2_supported(pl->mv[m].O, pl->mv[m].a, pl->mv[m].I, pl->r[m], pl->bf16)) {
       pl->fiber2[m] = true;
+      pl->wfiber[m] = false;
       pl->fiber_grid[m] = fiber2_grid(pl->mv[m].O, pl->mv[m].a, pl->mv[m].I, pl->r[m], pl->bf16,
                                       (pl->d.flags & ASI_FLAG_SHARE_SM) != 0);
     }
@@ -495,8 +502,9 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
 cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, bool dep, cudaStream_t st) {
   const bool fits = !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && a.si == 1 && a.sj == a.I &&
                     a.so == (int64_t)a.n_out * a.I && a.Q * a.a >= (1 << 20) &&
-                    fiber2_supported(a.O, a.a, a.I, a.n_out, x_bf16) &&
-                    (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0;
+                    a.I >= 32 && wfiber_supported(a.O, a.a, a.I, a.n_out);
+  const bool f2 = fits && fiber2_supported(a.O, a.a, a.I, a.n_out, x_bf16) &&
+                  (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15u) == 0;
   if (!fits) {
     GemmGroup g;
     g.np = 0;
@@ -516,6 +524,7 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
   f.n_tiles = fiber2_tiles(a.O, a.I);
   f.project_only = 1;
   f.plain = !dep;
+  if (!f2) return launch_wfiber(f, wfiber_grid(a.O, a.a, a.I, a.n_out, x_bf16), x_bf16, st);
   return launch_fiber2(f, fiber2_grid(a.O, a.a, a.I, a.n_out, x_bf16, (pl->d.flags & ASI_FLAG_SHARE_SM) != 0),
                        x_bf16, st);
 }
@@ -943,17 +952,18 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
     g.Pp4 = reinterpret_cast<float*>(w + pl->off_Pp[3]);
     g.n_planes = pl->dims[0] * pl->dims[1];
     g.S = (int)pl->dims[2];
+    g.H = (int)pl->dims[2];
+    g.W = (int)pl->dims[3];
     g.r3 = pl->r[2];
     g.r4 = pl->r[3];
-    g.vec4 = (!pl->bf16 && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) ? 1 : 0;
     g.status = status;
     g.clear = take_clear();
-    ASI_CUDA(pl->plane2 ? launch_plane2(g, pl->plane_grid, pl->bf16, st) : launch_plane(g, pl->plane_grid, pl->bf16, st));
+    ASI_CUDA(pl->plane2 ? launch_plane2(g, pl->plane_grid, pl->bf16, st) : launch_wplane(g, pl->plane_grid, pl->bf16, st));
   }
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
     if (!pl->fiber[m] || (pl->plane && m >= 2)) continue;
-    if (pl->fiber2[m]) {
+    if (pl->fiber2[m] || pl->wfiber[m]) {
       Fiber2Args f;
       std::memset(&f, 0, sizeof(f));
       f.X = act;
@@ -964,7 +974,8 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
       f.n_tiles = fiber2_tiles(v.O, v.I);
       f.plain = first;
       f.clear = take_clear();
-      ASI_CUDA(launch_fiber2(f, pl->fiber_grid[m], pl->bf16, st));
+      ASI_CUDA(pl->wfiber[m] ? launch_wfiber(f, pl->fiber_grid[m], pl->bf16, st)
+                             : launch_fiber2(f, pl->fiber_grid[m], pl->bf16, st));
     } else {
       FiberArgs f;
       f.X = act;

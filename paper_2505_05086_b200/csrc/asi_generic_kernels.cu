@@ -2,7 +2,7 @@
 // They are the correctness baseline every layer shape can fall back on; shape-specialised
 // kernels live in their own files.
 //
-//   k_fiber, k_plane : both products of a mode (of the two spatial modes) in one pass, ranks <= 8
+//   k_fiber    : both products of a mode in one pass, ranks <= 8
 //   k_qrb_*    : Orthogonalize(P) for ranks 65..128 as Cholesky-QR in fp64 (up to 64: asi_orth_kernels.cu)
 //   k_conv_tail: terms 4 and 5 of C_ASI (appendix "Speedup")
 #include <cuda_bf16.h>
@@ -203,176 +203,6 @@ __global__ void __launch_bounds__(256) k_fiber(FiberArgs p) {
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// k_plane: the two spatial modes of a conv activation in one pass.  A tile is NP = 256 / S whole
-// planes X[h][w] (S x S, S a multiple of 4); thread (plane, i) owns column w = i and row h = i:
-//   V3[w,:] = sum_h X[h][w] U3[h,:]   (column read)      V4[h,:] = sum_w X[h][w] U4[w,:]   (row read)
-//   P3[h,:] += sum_w X[h][w] V3[w,:]  (row read)         P4[w,:] += sum_h X[h][w] V4[h,:]  (column read)
-// i.e. P_m = A_m (A_m^T U_m) for m = 3, 4 (Algorithm 1).  Rows are read as float4 (conflict-free for the
-// unpadded pitch S), columns as scalars.  P3 / P4 accumulate in registers across the CTA's tiles.
-// ---------------------------------------------------------------------------------------------
-template <int R, typename TX>
-__global__ void __launch_bounds__(256) k_plane(PlaneArgs p) {
-  constexpr int NT = 256;
-  extern __shared__ __align__(16) float fsm[];
-  pass_begin(p.clear);
-  const int tid = threadIdx.x;
-  const int S = p.S, SS = S * S, NP = NT / S;
-  float* Xs0 = fsm;
-  float* Xs1 = Xs0 + NP * SS;
-  float* U3s = Xs1 + NP * SS;                       // [S][R]
-  float* U4s = U3s + S * R;                         // [S][R]
-  float* V3s = U4s + S * R;                         // [NP][S][R]
-  float* V4s = V3s + NP * S * R;                    // [NP][S][R]
-  for (int idx = tid; idx < S * R; idx += NT) {
-    const int k = idx / R, j = idx % R;
-    U3s[idx] = (j < p.r3) ? p.U3[k * p.r3 + j] : 0.f;
-    U4s[idx] = (j < p.r4) ? p.U4[k * p.r4 + j] : 0.f;
-  }
-  const TX* __restrict__ X = reinterpret_cast<const TX*>(p.X);
-  const int pl = tid / S, i = tid - pl * S;
-  const int64_t n_tiles = (p.n_planes + NP - 1) / NP;
-
-  auto stage = [&](float* dst, int64_t t, int& np) {
-    const int64_t p0 = t * NP;
-    np = (int)((p.n_planes - p0 < NP) ? (p.n_planes - p0) : NP);
-    const TX* src = X + p0 * SS;
-    if (sizeof(TX) == 4 && p.vec4) {
-      for (int idx = tid; idx < np * SS / 4; idx += NT)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst + 4 * idx)), "l"(src + 4 * idx) : "memory");
-    } else {
-      for (int idx = tid; idx < np * SS; idx += NT) dst[idx] = ld_as_float(src + idx);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-
-  float acc3[R], acc4[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) acc3[j] = acc4[j] = 0.f;
-  int n_cur = 0, n_next = 0, buf = 0;
-  int64_t t = blockIdx.x;
-  if (t < n_tiles) stage(Xs0, t, n_cur);
-  for (; t < n_tiles; t += gridDim.x) {
-    float* Xc = buf ? Xs1 : Xs0;
-    float* Xn = buf ? Xs0 : Xs1;
-    const int64_t tn = t + gridDim.x;
-    if (tn < n_tiles) {
-      stage(Xn, tn, n_next);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const bool on = pl < n_cur;                     // pl < NP follows
-    const float* Xp = Xc + pl * SS;
-    if (on) {
-      float v3[R], v4[R];
-#pragma unroll
-      for (int j = 0; j < R; ++j) v3[j] = v4[j] = 0.f;
-#pragma unroll 4
-      for (int h = 0; h < S; ++h) {                 // column i
-        const float x = Xp[h * S + i];
-#pragma unroll
-        for (int j = 0; j < R; j += 4) {
-          const float4 u = *reinterpret_cast<const float4*>(U3s + h * R + j);
-          v3[j] = fmaf(x, u.x, v3[j]); v3[j + 1] = fmaf(x, u.y, v3[j + 1]);
-          v3[j + 2] = fmaf(x, u.z, v3[j + 2]); v3[j + 3] = fmaf(x, u.w, v3[j + 3]);
-        }
-      }
-#pragma unroll 2
-      for (int w = 0; w < S; w += 4) {              // row i
-        const float4 x = *reinterpret_cast<const float4*>(Xp + i * S + w);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-          for (int j = 0; j < R; j += 4) {
-            const float4 u = *reinterpret_cast<const float4*>(U4s + (w + e) * R + j);
-            v4[j] = fmaf(xs[e], u.x, v4[j]); v4[j + 1] = fmaf(xs[e], u.y, v4[j + 1]);
-            v4[j + 2] = fmaf(xs[e], u.z, v4[j + 2]); v4[j + 3] = fmaf(xs[e], u.w, v4[j + 3]);
-          }
-      }
-#pragma unroll
-      for (int j = 0; j < R; j += 4) {
-        *reinterpret_cast<float4*>(V3s + (pl * S + i) * R + j) = make_float4(v3[j], v3[j + 1], v3[j + 2], v3[j + 3]);
-        *reinterpret_cast<float4*>(V4s + (pl * S + i) * R + j) = make_float4(v4[j], v4[j + 1], v4[j + 2], v4[j + 3]);
-      }
-    }
-    __syncthreads();
-    if (on) {
-      const float* V3p = V3s + pl * S * R;
-      const float* V4p = V4s + pl * S * R;
-#pragma unroll 2
-      for (int w = 0; w < S; w += 4) {              // row i: P3[i,:]
-        const float4 x = *reinterpret_cast<const float4*>(Xp + i * S + w);
-        const float xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-          for (int j = 0; j < R; j += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(V3p + (w + e) * R + j);
-            acc3[j] = fmaf(xs[e], v.x, acc3[j]); acc3[j + 1] = fmaf(xs[e], v.y, acc3[j + 1]);
-            acc3[j + 2] = fmaf(xs[e], v.z, acc3[j + 2]); acc3[j + 3] = fmaf(xs[e], v.w, acc3[j + 3]);
-          }
-      }
-#pragma unroll 4
-      for (int h = 0; h < S; ++h) {                 // column i: P4[i,:]
-        const float x = Xp[h * S + i];
-#pragma unroll
-        for (int j = 0; j < R; j += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(V4p + h * R + j);
-          acc4[j] = fmaf(x, v.x, acc4[j]); acc4[j + 1] = fmaf(x, v.y, acc4[j + 1]);
-          acc4[j + 2] = fmaf(x, v.z, acc4[j + 2]); acc4[j + 3] = fmaf(x, v.w, acc4[j + 3]);
-        }
-      }
-    }
-    __syncthreads();
-    n_cur = n_next;
-    buf ^= 1;
-  }
-  if (tid == 0) pdl_wait();
-  // the NP planes of the CTA meet in shared memory in plane order: one partial of P3 and P4 per CTA
-  if (pl < NP) {
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      V3s[(pl * S + i) * R + j] = acc3[j];
-      V4s[(pl * S + i) * R + j] = acc4[j];
-    }
-  }
-  __syncthreads();
-  for (int idx = tid; idx < S * R; idx += NT) {
-    const int k = idx / R, j = idx % R;
-    float s3 = 0.f, s4 = 0.f;
-    for (int q = 0; q < NP; ++q) {
-      s3 += V3s[q * S * R + idx];
-      s4 += V4s[q * S * R + idx];
-    }
-    if (j < p.r3) p.Pp3[((int64_t)blockIdx.x * S + k) * p.r3 + j] = s3;
-    if (j < p.r4) p.Pp4[((int64_t)blockIdx.x * S + k) * p.r4 + j] = s4;
-  }
-}
-
-size_t plane_smem(int S) {
-  const int NP = 256 / S;
-  return 4 * ((size_t)2 * NP * S * S + 2 * S * 8 + 2 * NP * S * 8) + 64;
-}
-
-template <int R, typename TX>
-static cudaError_t launch_plane_t(const PlaneArgs& p, int grid, cudaStream_t st) {
-  const size_t smem = plane_smem(p.S);   // the default limit counts static shared memory too: always opt in
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_plane<R, TX>), smem);
-  if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.clear, k_plane<R, TX>, dim3(grid), dim3(256), smem, st, p);
-}
-
-cudaError_t launch_plane(const PlaneArgs& p, int grid, bool x_bf16, cudaStream_t st) {
-  ProfScope prof(ASI_K_EXPAND, st,
-                 (double)p.n_planes * p.S * p.S * (x_bf16 ? 2 : 4) + 4.0 * p.S * (p.r3 + p.r4) * (grid + 1));
-  const int r = p.r3 > p.r4 ? p.r3 : p.r4;
-  if (r <= 4) return x_bf16 ? launch_plane_t<4, __nv_bfloat16>(p, grid, st) : launch_plane_t<4, float>(p, grid, st);
-  return x_bf16 ? launch_plane_t<8, __nv_bfloat16>(p, grid, st) : launch_plane_t<8, float>(p, grid, st);
-}
-
 size_t fiber_smem(int a) {
   const int TQ = kFiberTQ, PQ = TQ + 4, PA = a | 1;
   const size_t tile = (size_t)std::max(TQ * PA, a * PQ);
@@ -519,8 +349,18 @@ cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st) {
 // k_conv_tail: one CTA per output channel c'.  Thread (o, s): output o = (j, kh, kw) of Z4 and
 // split s of the reduction over (i, h'); partial sums meet in shared memory in a fixed order.
 // Then dW[c', :, :, :] = Z4[c'] x_2 U2 over the channels of c''s group.
+// A chain of dependent reads: 1024 threads and sixteen reads in flight each (27 x 27 maps, stride 2, Cout = 90,
+// ranks 5: 256 threads with one read at a time took 40 us).
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_conv_tail(ConvTailArgs p) {
+constexpr int kTailNT = 1024;
+
+// splits s of the reduction over (i, h'): as many as the CTA's threads hold
+__host__ __device__ static inline int conv_tail_split(int n_out, int n_items) {
+  const int n = n_out <= kTailNT ? kTailNT / n_out : 1;
+  return n < n_items ? n : n_items;
+}
+
+__global__ void __launch_bounds__(kTailNT) k_conv_tail(ConvTailArgs p) {
   extern __shared__ float sm[];
   pdl_launch_dependents();
   pdl_wait();
@@ -528,65 +368,57 @@ __global__ void __launch_bounds__(256) k_conv_tail(ConvTailArgs p) {
   const int co = blockIdx.x;
   const int kk = p.kh * p.kw;
   const int n_out = p.r2 * kk;
+  const int nsplit = conv_tail_split(n_out, p.r1 * p.Ho);
   float* Z4s = sm;                       // [n_out]
-  float* red = sm + ((n_out + 31) / 32) * 32;   // [nsplit][n_out] when nsplit > 1
-
-  int nsplit = (n_out <= 128) ? 256 / n_out : 1;
+  float* red = sm + n_out;               // [nsplit][n_out]
   const int n_items = p.r1 * p.Ho;
-  if (nsplit > n_items) nsplit = n_items;
-  if (nsplit < 1) nsplit = 1;
-
-  if (nsplit > 1) {
-    const int o = tid % n_out, s = tid / n_out;
-    if (s < nsplit) {
-      const int j = o / kk, t = o % kk, ky = t / p.kw, kx = t % p.kw;
-      float acc = 0.f;
-      for (int it = s; it < n_items; it += nsplit) {
-        const int i = it / p.Ho, ho = it % p.Ho;
-        const int h = ho * p.sh + ky - p.ph;
-        if (h < 0 || h >= p.H) continue;
-        const float* z1 = p.Z1 + (((int64_t)i * p.Cout + co) * p.Ho + ho) * p.Wo;
-        const float* z3 = p.Z3 + (((int64_t)i * p.r2 + j) * p.H + h) * p.W;
-        for (int wo = 0; wo < p.Wo; ++wo) {
-          const int w = wo * p.sw + kx - p.pw;
-          if (w >= 0 && w < p.W) acc = fmaf(z1[wo], z3[w], acc);
+  for (int t0 = tid; t0 < n_out * nsplit; t0 += kTailNT) {
+    const int s = t0 / n_out, o = t0 - s * n_out;
+    const int j = o / kk, t = o - j * kk, ky = t / p.kw, kx = t - ky * p.kw;
+    const int wo_lo = (p.pw - kx > 0) ? (p.pw - kx + p.sw - 1) / p.sw : 0;
+    int wo_hi = (p.W - 1 + p.pw - kx >= 0) ? (p.W - 1 + p.pw - kx) / p.sw + 1 : 0;
+    if (wo_hi > p.Wo) wo_hi = p.Wo;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int it = s; it < n_items; it += nsplit) {
+      const int i = it / p.Ho, ho = it - i * p.Ho;
+      const int h = ho * p.sh + ky - p.ph;
+      if (h < 0 || h >= p.H) continue;
+      const float* z1 = p.Z1 + (((int64_t)i * p.Cout + co) * p.Ho + ho) * p.Wo;
+      const float* z3 = p.Z3 + (((int64_t)i * p.r2 + j) * p.H + h) * p.W + kx - p.pw;
+      // sixteen products in flight, from clamped addresses
+#pragma unroll 1
+      for (int wo = wo_lo; wo < wo_hi; wo += 8) {
+        float x[8], y[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int w = wo + e < wo_hi ? wo + e : wo;
+          x[e] = __ldg(z1 + w);
+          y[e] = __ldg(z3 + w * p.sw);
         }
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (wo + e < wo_hi) acc[e & 3] = fmaf(x[e], y[e], acc[e & 3]);
       }
-      red[s * n_out + o] = acc;
     }
-    __syncthreads();
-    if (tid < n_out) {
-      float v = 0.f;
-      for (int s = 0; s < nsplit; ++s) v += red[s * n_out + tid];
-      Z4s[tid] = v;
-    }
-  } else {
-    for (int o = tid; o < n_out; o += 256) {
-      const int j = o / kk, t = o % kk, ky = t / p.kw, kx = t % p.kw;
-      float acc = 0.f;
-      for (int it = 0; it < n_items; ++it) {
-        const int i = it / p.Ho, ho = it % p.Ho;
-        const int h = ho * p.sh + ky - p.ph;
-        if (h < 0 || h >= p.H) continue;
-        const float* z1 = p.Z1 + (((int64_t)i * p.Cout + co) * p.Ho + ho) * p.Wo;
-        const float* z3 = p.Z3 + (((int64_t)i * p.r2 + j) * p.H + h) * p.W;
-        for (int wo = 0; wo < p.Wo; ++wo) {
-          const int w = wo * p.sw + kx - p.pw;
-          if (w >= 0 && w < p.W) acc = fmaf(z1[wo], z3[w], acc);
-        }
-      }
-      Z4s[o] = acc;
-    }
+    red[t0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  }
+  __syncthreads();
+  for (int o = tid; o < n_out; o += kTailNT) {
+    float v = 0.f;
+    for (int s = 0; s < nsplit; ++s) v += red[s * n_out + o];
+    Z4s[o] = v;
   }
   __syncthreads();
   const int cg = p.C / p.groups, og = p.Cout / p.groups;
   const int g = co / og;
   float* dw = p.dW + (int64_t)co * cg * kk;
-  for (int idx = tid; idx < cg * kk; idx += 256) {
-    const int cl = idx / kk, t = idx % kk;
+  for (int idx = tid; idx < cg * kk; idx += kTailNT) {
+    const int cl = idx / kk, t = idx - cl * kk;
     const float* u = p.U2 + (int64_t)(g * cg + cl) * p.r2;
     float v = 0.f;
-    for (int j = 0; j < p.r2; ++j) v = fmaf(Z4s[j * kk + t], u[j], v);
+#pragma unroll 4
+    for (int j = 0; j < p.r2; ++j) v = fmaf(Z4s[j * kk + t], __ldg(u + j), v);
     dw[idx] = v;
   }
 }
@@ -684,25 +516,20 @@ cudaError_t launch_conv_tail_split(const ConvTailArgs& p, float* Z4p, int nsp, c
   return launch_pdl(k_conv_dw, dim3(p.Cout), dim3(256), (size_t)n_out * sizeof(float), st, p, (const float*)Z4p, nsp);
 }
 
-size_t conv_tail_smem(int r2, int kh, int kw) {
-  const int n_out = r2 * kh * kw;
-  const int nsplit_max = (n_out <= 128) ? 256 / n_out : 1;
-  const int G = (n_out <= 256) ? 256 / n_out : 1;            // k_conv_z4
-  const size_t tail = (size_t)(((n_out + 31) / 32) * 32 + (size_t)nsplit_max * n_out) * sizeof(float);
-  const size_t z4 = (size_t)G * n_out * sizeof(float);
-  return tail > z4 ? tail : z4;
+static size_t conv_tail_smem(int r1, int r2, int Ho, int kh, int kw) {
+  const size_t n_out = (size_t)r2 * kh * kw;
+  return n_out * (1 + conv_tail_split((int)n_out, r1 * Ho)) * sizeof(float);
 }
-
 cudaError_t launch_conv_tail(const ConvTailArgs& p, cudaStream_t st) {
   ProfScope prof(ASI_K_CONV_TAIL, st,
                  4.0 * ((double)p.r1 * p.Cout * p.Ho * p.Wo + (double)p.r1 * p.r2 * p.H * p.W +
                         (double)p.C * p.r2 + (double)p.Cout * (p.C / p.groups) * p.kh * p.kw));
-  const size_t smem = conv_tail_smem(p.r2, p.kh, p.kw);
+  const size_t smem = conv_tail_smem(p.r1, p.r2, p.Ho, p.kh, p.kw);
   if (smem > 40 * 1024) {
     cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_conv_tail), smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_pdl(k_conv_tail, dim3(p.Cout), dim3(256), smem, st, p);
+  return launch_pdl(k_conv_tail, dim3(p.Cout), dim3(kTailNT), smem, st, p);
 }
 
 }  // namespace asi

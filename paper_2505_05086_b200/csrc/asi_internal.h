@@ -53,7 +53,8 @@ struct PlaneArgs {
   float* Pp3;          // [grid][S][r3]
   float* Pp4;          // [grid][S][r4]
   int64_t n_planes;
-  int S, r3, r4, vec4;
+  int S, H, W, r3, r4;
+  int np, pitch, nsc, nsr;   // planes per tile, row pitch, lanes per column pair and row (set by the launcher)
   int* clear = nullptr;    // not null: CTA 0 zeroes the 256 ints of the workspace's status block
   int* status = nullptr;   // status word of the workspace (k_plane2: an expired wait on the bulk copy)
 };
@@ -356,9 +357,13 @@ cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st);
 cudaError_t launch_row_solve(const RowSolveArgs& p, cudaStream_t st);
 cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t st);
 size_t fiber_smem(int a);
-size_t conv_tail_smem(int r2, int kh, int kw);
-cudaError_t launch_plane(const PlaneArgs& p, int grid, bool x_bf16, cudaStream_t st);
-size_t plane_smem(int S);
+bool wfiber_supported(int64_t O, int64_t a, int64_t I, int r);
+int64_t wfiber_tiles(int64_t O, int64_t a, int64_t I, bool bf16);
+int wfiber_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16);
+cudaError_t launch_wfiber(const Fiber2Args& p, int grid, bool bf16, cudaStream_t st);
+bool wplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4);
+int wplane_grid(int64_t n_planes, int H, int W, int r, bool bf16);
+cudaError_t launch_wplane(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st);
 bool fiber2_supported(int64_t O, int64_t a, int64_t I, int r, bool bf16);
 int64_t fiber2_tiles(int64_t O, int64_t I);
 int fiber2_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16, bool share_sm);
@@ -469,6 +474,7 @@ struct asi_plan {
   int fiber_grid[ASI_MAX_MODES];
   bool plane;                      // modes 3 and 4 together by the whole-plane kernel
   int plane_grid;
+  bool wfiber[ASI_MAX_MODES];      // ... by warps on their own (strided fibers)
   bool fiber2[ASI_MAX_MODES];      // ... by its register-tiled successor (ranks <= 4, 16-byte aligned rows)
   bool plane2;                     // 28 x 28 and 56 x 56 planes, ranks <= 4
   int fast_kind;                   // 7, 14: modes 3 and 4 as Gram matrices of such square maps; 0: any map of at most 256 positions

@@ -294,11 +294,12 @@ int fiber2_stages(int a, int nj, bool bf16) {
   return 2;
 }
 
-// ranks up to 4 for a <= 128, up to 8 for a <= 64 (the register budget of the row accumulators)
+// The tiles the CTA shares suit ranks up to 4 with 16-byte rows: 31 us for 128 x 64 x 56 x 56 fp32 along the batch, the
+// warps of k_wfiber level at best.  At ranks 5..8 k_wfiber is faster (50 x 116 x 27 x 27 along the batch, ranks 5:
+// 11 us against 15), and it takes any row length.  Short modes stream through registers (k_fiber_reg).
 bool fiber2_supported(int64_t O, int64_t a, int64_t I, int r, bool bf16) {
-  (void)O;
-  return r <= 8 && a >= 2 && a <= (r <= 4 ? 128 : 64) && I >= kF2TQ && I % (bf16 ? 8 : 4) == 0 &&
-         O * ((I + kF2TQ - 1) / kF2TQ) < (1ll << 30);
+  return a >= 2 && a <= 128 && I >= kF2TQ && I % (bf16 ? 8 : 4) == 0 && O * ((I + kF2TQ - 1) / kF2TQ) < (1ll << 30) &&
+         (r <= 4 || fiber_reg_supported(O, a, I, r, bf16));
 }
 
 int64_t fiber2_tiles(int64_t O, int64_t I) { return O * ((I + kF2TQ - 1) / kF2TQ); }
@@ -330,18 +331,11 @@ cudaError_t launch_fiber2(const Fiber2Args& p0, int grid, bool bf16, cudaStream_
   ProfScope prof(p.project_only ? ASI_K_MODEPROD : ASI_K_EXPAND, st, xbytes);
 #define ASI_F2(RW_, NJ_)                                                                        \
   return bf16 ? launch_fiber2_t<RW_, NJ_, __nv_bfloat16>(p, grid, smem, st) : launch_fiber2_t<RW_, NJ_, float>(p, grid, smem, st)
-  if (nj == 4) {
-    switch (rw) {
-      case 1: ASI_F2(1, 4);
-      case 2: ASI_F2(2, 4);
-      case 4: ASI_F2(4, 4);
-      default: ASI_F2(8, 4);
-    }
-  }
   switch (rw) {
-    case 1: ASI_F2(1, 8);
-    case 2: ASI_F2(2, 8);
-    default: ASI_F2(4, 8);
+    case 1: ASI_F2(1, 4);
+    case 2: ASI_F2(2, 4);
+    case 4: ASI_F2(4, 4);
+    default: ASI_F2(8, 4);
   }
 #undef ASI_F2
 }

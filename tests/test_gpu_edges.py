@@ -1,0 +1,89 @@
+"""The kernels of the warm step at the edges of their tiles, element by element against the fp64 oracle."""
+import pytest
+
+from asi_inputs.configs import LayerSpec
+from asi_inputs.generator import LayerStream
+from tests.gpu_util import TOL_F32, check, compare_step, make_runner
+
+pytestmark = pytest.mark.gpu
+
+
+def _rho(r):
+    return min(0.7, 0.25 ** (1.0 / max(r - 1, 1)))
+
+
+def _two_steps(L, bf16, fused=None, rho=None, tol=TOL_F32):
+    st = LayerStream(dims=L.dims, ranks=L.ranks, dy_shape=L.dy_shape, seed=sum(L.dims) + L.cout, bf16=bf16,
+                     rho=rho or tuple(_rho(r) for r in L.ranks),
+                     gen_ranks=tuple(min(d, max(2 * r, r + 2, 4)) for d, r in zip(L.dims, L.ranks)))
+    run = make_runner(L, bf16=bf16)
+    if fused is not None:
+        assert (run.plan.launch_count(0) == 3) == fused
+    U_prev = st.u_prev0()
+    for _ in range(2):
+        A, dY = st.next()
+        err, U_prev = compare_step(run, L, A, dY, U_prev)
+        check(err, tol, f"{L.dims} {L.ranks} bf16={bf16}")
+
+
+# Fused small maps of any shape and any batch: (dims, ranks, cout, k, stride, pad, groups)
+ANY_MAP = [
+    ((3, 9, 6, 11), (2, 4, 3, 4), 7, 3, 1, 1, 1),          # fewer samples than a CTA has warps
+    ((13, 33, 7, 7), (4, 4, 4, 3), 12, 3, 1, 1, 1),        # batch not a multiple of eight, C H W odd
+    ((17, 40, 16, 16), (3, 8, 5, 8), 8, 3, 1, 1, 2),       # 256 positions, several CTAs per sample
+    ((70, 21, 8, 32), (4, 5, 4, 6), 9, 1, 1, 0, 1),        # a row of 32 lanes, batch above one warp's share
+    ((10, 130, 6, 6), (4, 4, 4, 4), 20, 3, 2, 1, 1),       # channels beyond one tile
+    ((9, 6, 1, 5), (3, 4, 1, 2), 4, 1, 1, 0, 1),           # one row
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("case", ANY_MAP)
+def test_fused_maps_of_any_shape_and_batch(case, bf16):
+    dims, ranks, cout, k, s, p, g = case
+    _two_steps(LayerSpec("t", "conv", dims, cout, k, s, p, g, ranks=ranks), bf16, fused=True)
+
+
+# Planes and strided fibers streamed by warps: odd and even widths, one plane a tile and many, rows or columns shared
+# by 2..8 lanes, the largest map; channel modes around 32, 64 and 128 rows; rows that start at any element
+STREAMED = [
+    ((4, 33, 17, 19), (3, 4, 4, 4)),
+    ((3, 64, 9, 50), (3, 5, 5, 6)),                        # few rows: eight lanes a row
+    ((2, 65, 50, 9), (2, 6, 6, 5)),                        # few columns: lanes share a pair
+    ((2, 31, 33, 33), (2, 4, 4, 4)),                       # two rows a lane, one plane a tile
+    ((3, 128, 27, 27), (3, 8, 5, 5)),                      # the longest fiber; odd planes
+    ((2, 12, 64, 64), (2, 8, 8, 8)),                       # the largest map, ranks 8
+    ((40, 7, 20, 24), (8, 4, 4, 4)),                       # vector copies along the batch, rank 8
+    ((5, 12, 60, 36), (3, 3, 3, 3)),                       # planes of unequal sides, aligned rows
+    ((129, 5, 18, 18), (4, 3, 4, 4)),                      # a batch one past the fiber kernels
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,ranks", STREAMED)
+def test_streamed_planes_and_fibers(dims, ranks, bf16):
+    _two_steps(LayerSpec("t", "conv", dims, 10, 3, 2, 1, 1, ranks=ranks), bf16, fused=False)
+
+
+def test_a_stride_two_layer_with_a_large_product_on_the_streamed_fibers():
+    """The first core product and Z1 of a layer of a million values, rows of an odd length."""
+    _two_steps(LayerSpec("t", "conv", (50, 40, 27, 27), 45, 3, 1, 1, 1, ranks=(5, 4, 4, 4)), False, fused=False)
+
+
+# Grouped products and Orthogonalize of token layers: ranks on both sides of 8, 16, 32 and 64, ragged token counts and
+# features, two modes and three
+GROUPED = [
+    ((5, 33, 31), (1, 9, 17)),
+    ((9, 100, 70), (9, 16, 33)),
+    ((3, 129, 257), (2, 8, 32)),
+    ((130, 70), (65, 40)),
+    ((140, 127), (17, 24)),
+    ((300, 96), (32, 64)),
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,ranks", GROUPED)
+def test_grouped_products_at_the_edges(dims, ranks, bf16):
+    rho = tuple(0.25 ** (1.0 / max(r, 4)) for r in ranks)
+    _two_steps(LayerSpec("t", "linear", dims, 37, ranks=ranks), bf16, rho=rho, tol=dict(TOL_F32, proj=1e-3, dw=1e-3))
