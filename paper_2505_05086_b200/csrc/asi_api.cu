@@ -129,7 +129,7 @@ void layout_compress(asi_plan* pl) {
       pl->wfiber[m] = wfiber_supported(v.O, v.a, v.I, pl->r[m]);
       if (pl->wfiber[m]) {
         pl->fiber[m] = true;
-        pl->fiber_grid[m] = wfiber_grid(v.O, v.a, v.I, pl->r[m], pl->bf16);
+        pl->fiber_grid[m] = wfiber_grid(v.O, v.a, v.I, pl->r[m]);
       } else if (pl->r[m] <= 8 && v.a <= 128 && fiber_smem((int)v.a) <= kSmemLimit) {
         pl->fiber[m] = true;
         pl->fiber_grid[m] = (int)std::min<int64_t>(fiber_tiles(v.O, v.a, v.I), 296);
@@ -524,7 +524,7 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
   f.n_tiles = fiber2_tiles(a.O, a.I);
   f.project_only = 1;
   f.plain = !dep;
-  if (!f2) return launch_wfiber(f, wfiber_grid(a.O, a.a, a.I, a.n_out, x_bf16), x_bf16, st);
+  if (!f2) return launch_wfiber(f, wfiber_grid(a.O, a.a, a.I, a.n_out), x_bf16, st);
   return launch_fiber2(f, fiber2_grid(a.O, a.a, a.I, a.n_out, x_bf16, (pl->d.flags & ASI_FLAG_SHARE_SM) != 0),
                        x_bf16, st);
 }

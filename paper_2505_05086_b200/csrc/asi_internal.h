@@ -359,7 +359,7 @@ cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t
 size_t fiber_smem(int a);
 bool wfiber_supported(int64_t O, int64_t a, int64_t I, int r);
 int64_t wfiber_tiles(int64_t O, int64_t a, int64_t I, bool bf16);
-int wfiber_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16);
+int wfiber_grid(int64_t O, int64_t a, int64_t I, int r);
 cudaError_t launch_wfiber(const Fiber2Args& p, int grid, bool bf16, cudaStream_t st);
 bool wplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4);
 int wplane_grid(int64_t n_planes, int H, int W, int r, bool bf16);

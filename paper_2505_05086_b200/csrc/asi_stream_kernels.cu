@@ -603,9 +603,10 @@ int64_t wfiber_tiles(int64_t O, int64_t a, int64_t I, bool bf16) {
   const int rk = wf_rk((int)a), tc = bf16 ? wf_cols<__nv_bfloat16>(rk) : wf_cols<float>(rk);
   return O * ((I + tc - 1) / tc);
 }
-int wfiber_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16) {
-  const int64_t nw = wf_warps((int)a, r <= 4 ? 4 : 8, bf16);
-  return (int)std::min<int64_t>((wfiber_tiles(O, a, I, bf16) + nw - 1) / nw, 148);
+// the same count for both types (a bf16 plan without tensor-core products has the fp32 plan's workspace)
+int wfiber_grid(int64_t O, int64_t a, int64_t I, int r) {
+  const int64_t nw = wf_warps((int)a, r <= 4 ? 4 : 8, false);
+  return (int)std::min<int64_t>((wfiber_tiles(O, a, I, false) + nw - 1) / nw, 148);
 }
 cudaError_t launch_wfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
   Fiber2Args p = p0;
