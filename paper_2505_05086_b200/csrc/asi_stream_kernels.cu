@@ -66,6 +66,40 @@ __device__ __forceinline__ void cp_one(float* dst, const float* src, bool on) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s_addr(dst)), "l"(src), "r"(on ? 4 : 0) : "memory");
 }
 
+// a pair of columns against one factor row: v[c][j / 2] += (x_c, x_c) (u_j, u_{j+1}).  A uniform 16-byte read of shared
+// memory costs two cycles whatever it holds, so the factor row is read once and the column values are doubled
+template <int R>
+__device__ __forceinline__ void fma_cols(f2 (&v)[2][R / 2], f2 x, const float* __restrict__ u) {
+  const float2 xs = unpack2(x);
+  const f2 x0 = pack2(xs.x, xs.x), x1 = pack2(xs.y, xs.y);
+#pragma unroll
+  for (int j = 0; j < R / 2; j += 2) {
+    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(u + 2 * j);
+    ffma2(v[0][j], x0, w.x);
+    ffma2(v[1][j], x1, w.x);
+    ffma2(v[0][j + 1], x0, w.y);
+    ffma2(v[1][j + 1], x1, w.y);
+  }
+}
+// the lanes that share a pair of columns: neighbours s, 2 s, .. below 32
+template <int R>
+__device__ __forceinline__ void sum_cols(f2 (&v)[2][R / 2], int from, int to) {
+  for (int s = from; s < to; s *= 2)
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int j = 0; j < R / 2; ++j) {
+        const float2 w = unpack2(v[c][j]);
+        v[c][j] = pack2(w.x + __shfl_xor_sync(0xffffffffu, w.x, s), w.y + __shfl_xor_sync(0xffffffffu, w.y, s));
+      }
+}
+// column j of the pair
+template <int R>
+__device__ __forceinline__ float2 col_pair(const f2 (&v)[2][R / 2], int j) {
+  const float2 a = unpack2(v[0][j >> 1]), b = unpack2(v[1][j >> 1]);
+  return (j & 1) ? make_float2(a.y, b.y) : make_float2(a.x, b.x);
+}
+
 constexpr int kWMaxWarps = 16;
 constexpr size_t kWSmemBudget = 224 * 1024;
 
@@ -82,20 +116,20 @@ __host__ __device__ constexpr int wf_cols(int RK) {
 
 template <int R, int RK, bool VEC, typename TX>
 __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_constant__ Fiber2Args p) {
-  constexpr int TC = wf_cols<TX>(RK), PT = TC + 4, NP = TC / 2, KQ = 32 / NP, UP = 2 * R + 4;
+  constexpr int TC = wf_cols<TX>(RK), PT = TC + 4, NP = TC / 2, KQ = 32 / NP, UP = 12;
   constexpr int KB = 8, KS = KQ == 4 ? 2 : KQ;       // rows per step of the column pass, between a lane's rows
   extern __shared__ __align__(16) unsigned char ws_smem[];
   pass_begin(p.clear);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int a = p.a, r = p.r, a8 = (a + 7) & ~7;
-  float* Ud = reinterpret_cast<float*>(ws_smem);     // [a8][UP]: (u, u) pairs, rows >= a and columns >= r zero
+  float* Ud = reinterpret_cast<float*>(ws_smem);     // [a8][UP]: rows >= a and columns >= r zero; rows 1, 4 and 5 apart are bank-disjoint
   float* Vt = Ud + a8 * UP + warp * (R * TC);        // [R][TC]
   TX* T = reinterpret_cast<TX*>(Ud + a8 * UP + nw * (R * TC)) + (size_t)warp * (2 * a8 * PT);   // [2][a8][PT]
   if (p.project_only) pdl_wait();                    // its factor comes from the kernel before
   for (int e = tid; e < a8 * R; e += blockDim.x) {
     const int k = e / R, j = e % R;
     const float u = (k < a && j < r) ? p.U[(int64_t)k * p.ldu + j] : 0.f;
-    *reinterpret_cast<f2*>(Ud + k * UP + 2 * j) = pack2(u, u);
+    Ud[k * UP + j] = u;
   }
   for (int e = lane; e < (a8 - a) * PT; e += 32) {   // rows a .. a8 - 1 of both tiles are never written again
     T[a * PT + e] = TX(0.f);
@@ -181,42 +215,28 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
     stage(T + buf * (a8 * PT));
     cp_wait1();
     __syncwarp();
-    f2 v[R];
+    f2 v[2][R / 2];
 #pragma unroll
-    for (int j = 0; j < R; ++j) v[j] = 0ull;
+    for (int j = 0; j < R / 2; ++j) v[0][j] = v[1][j] = 0ull;
     {
       const TX* xs = Tc + kfirst * PT + 2 * cp;
       const float* us = Ud + kfirst * UP;
 #pragma unroll 1
       for (int k = 0; k < a8; k += KB) {
 #pragma unroll
-        for (int s = 0; s < KB / KQ; ++s) {
-          const f2 x = ld_pair(xs + KS * s * PT);
-#pragma unroll
-          for (int j = 0; j < R; j += 2) {
-            const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(us + KS * s * UP + 2 * j);
-            ffma2(v[j], x, u.x);
-            ffma2(v[j + 1], x, u.y);
-          }
-        }
+        for (int s = 0; s < KB / KQ; ++s) fma_cols<R>(v, ld_pair(xs + KS * s * PT), us + KS * s * UP);
         xs += KB * PT;
         us += KB * UP;
       }
     }
-#pragma unroll
-    for (int s = NP; s < 32; s *= 2)
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const float2 w = unpack2(v[j]);
-        v[j] = pack2(w.x + __shfl_xor_sync(0xffffffffu, w.x, s), w.y + __shfl_xor_sync(0xffffffffu, w.y, s));
-      }
+    sum_cols<R>(v, NP, 32);
     if (p.project_only) {
       const int64_t i = (int64_t)i_c * TC + 2 * cp;
       float* dst = p.Y + (int64_t)o_c * p.y_so + i;
 #pragma unroll
       for (int j = 0; j < R; ++j)
         if (j < r && j % KQ == kq) {
-          const float2 w = unpack2(v[j]);
+          const float2 w = col_pair<R>(v, j);
           if constexpr (VEC) {
             if (i < p.I) *reinterpret_cast<float2*>(dst + j * p.y_sj) = w;
           } else {
@@ -227,7 +247,7 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
     } else {
 #pragma unroll
       for (int j = 0; j < R; ++j)
-        if (j % KQ == kq) *reinterpret_cast<f2*>(Vt + j * TC + 2 * cp) = v[j];
+        if (j % KQ == kq) *reinterpret_cast<float2*>(Vt + j * TC + 2 * cp) = col_pair<R>(v, j);
       __syncwarp();
       const TX* xr[RK];
 #pragma unroll
@@ -256,7 +276,7 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
   if (tid == 0) pdl_wait();
   __syncthreads();
   // one partial of P per CTA: the warps' sums meet in warp order
-  float* red = Ud + a8 * UP;                         // [nw][a][R] over the (idle) tiles
+  float* red = Ud + a8 * UP;                         // [nw][R][a] over the (idle) tiles
 #pragma unroll
   for (int i = 0; i < RK; ++i) {
     const int k = lane + 32 * i;
@@ -264,15 +284,16 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         const float2 w = unpack2(acc[i][j]);
-        red[(warp * a + k) * R + j] = w.x + w.y;
+        red[(warp * R + j) * a + k] = w.x + w.y;
       }
     }
   }
   __syncthreads();
   for (int e = tid; e < a * R; e += blockDim.x) {
-    const int k = e / R, j = e % R;
-    float s = red[e];
-    for (int w = 1; w < nw; ++w) s += red[w * a * R + e];
+    const int j = e / a, k = e - j * a;
+    float s = 0.f;
+#pragma unroll 4
+    for (int w = 0; w < nw; ++w) s += red[w * a * R + e];
     if (j < r) p.Pp[((int64_t)blockIdx.x * a + k) * r + j] = s;
   }
 }
@@ -281,11 +302,15 @@ size_t wf_warp_bytes(int a, int R, int rk, bool bf16) {
   const int tc = bf16 ? wf_cols<__nv_bfloat16>(rk) : wf_cols<float>(rk), a8 = (a + 7) & ~7;
   return (size_t)R * tc * 4 + (size_t)2 * a8 * (tc + 4) * (bf16 ? 2 : 4);
 }
-size_t wf_fixed_bytes(int a, int R) { return (size_t)((a + 7) & ~7) * (2 * R + 4) * 4; }
+size_t wf_fixed_bytes(int a) { return (size_t)((a + 7) & ~7) * 12 * 4; }
 int wf_rk(int a) { return a <= 32 ? 1 : (a <= 64 ? 2 : 4); }
-int wf_warps(int a, int R, bool bf16) {
-  const size_t n = (kWSmemBudget - wf_fixed_bytes(a, R)) / wf_warp_bytes(a, R, wf_rk(a), bf16);
-  return (int)std::min<size_t>(n, kWMaxWarps);
+// warps of a CTA: as many as fit, or as few of them as take the same number of tiles each on 148 CTAs
+int ws_balance(size_t fit, int64_t tiles) {
+  const int64_t n = std::min<int64_t>((int64_t)fit, kWMaxWarps), rounds = (tiles + 148 * n - 1) / (148 * n);
+  return (int)((tiles + 148 * rounds - 1) / (148 * rounds));
+}
+int wf_warps(int64_t tiles, int a, int R, bool bf16) {
+  return ws_balance((kWSmemBudget - wf_fixed_bytes(a)) / wf_warp_bytes(a, R, wf_rk(a), bf16), tiles);
 }
 
 
@@ -294,27 +319,28 @@ int wf_warps(int a, int R, bool bf16) {
 //   rows     V4[h][j]  = sum_w X[h][w] U4[w][j]
 //   columns  V3[w][j]  = sum_h X[h][w] U3[h][j]   and   P4[w][j] += sum_h X[h][w] V4[h][j]
 //   rows     P3[h][j] += sum_w X[h][w] V3[w][j]
-// A lane owns one pair of columns and two rows of the tile (the same ones in every tile, so that P3 and P4 stay in
-// registers).  Where a tile has fewer columns or rows than that, 2, 4 or 8 neighbouring lanes share one (nsc, nsr) and
-// meet by shuffles; np is as large as the 32 pairs and the 64 rows allow.
+// A lane owns one pair of columns and two rows of one plane of the tile (the same ones in every tile, so that P3 and P4
+// stay in registers).  Where a tile has fewer columns or rows than that, 2, 4 or 8 neighbouring lanes share them (nsc,
+// nsr) and meet by shuffles; np is as large as 32 pairs of columns and 32 pairs of rows allow.  The reads of shared
+// memory bound the kernel: 606 cycles a warp for two planes of 27 x 27 at ranks 5..8.
 // ---------------------------------------------------------------------------------------------
 template <int R, bool VEC, typename TX>
 __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_constant__ PlaneArgs p) {
   extern __shared__ __align__(16) unsigned char ws_smem[];
   pass_begin(p.clear);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int H = p.H, W = p.W, np = p.np, PT = p.pitch, W2 = (W + 1) >> 1, W4 = (W + 3) >> 2;
+  const int H = p.H, W = p.W, np = p.np, PT = p.pitch, W2 = (W + 1) >> 1, W4 = (W + 3) >> 2, H2 = (H + 1) >> 1;
   const int nsc = p.nsc, nsr = p.nsr;
-  const int v4s = H * 2 * R + 4, v3s = R * PT + 4;   // one plane's V4 (u, u) and V3, padded off each other's banks
-  float* U3d = reinterpret_cast<float*>(ws_smem);    // [H][R] pairs (u, u)
-  float* U4t = U3d + 2 * H * R;                      // [R][PT], columns >= W zero
-  float* V4d = U4t + R * PT + warp * np * (v4s + v3s);   // [np][H][R] pairs
+  const int v4s = H * R + 4, v3s = R * PT + 4;       // one plane's V4 and V3, padded off each other's banks
+  float* U3d = reinterpret_cast<float*>(ws_smem);    // [H][R]
+  float* U4t = U3d + H * R;                          // [R][PT], columns >= W zero
+  float* V4d = U4t + R * PT + warp * np * (v4s + v3s);   // [np][H][R]
   float* V3t = V4d + np * v4s;                       // [np][R][PT]
   TX* T = reinterpret_cast<TX*>(U4t + R * PT + nw * np * (v4s + v3s)) + (size_t)warp * (2 * np * H * PT);
   for (int e = tid; e < H * R; e += blockDim.x) {
     const int k = e / R, j = e % R;
     const float u = j < p.r3 ? p.U3[k * p.r3 + j] : 0.f;
-    *reinterpret_cast<f2*>(U3d + 2 * e) = pack2(u, u);
+    U3d[e] = u;
   }
   for (int e = tid; e < R * PT; e += blockDim.x) {
     const int j = e / PT, k = e - j * PT;
@@ -365,23 +391,18 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
     }
     cp_commit();
   };
-  // column role: lane = ((plane, pair), share); row role: lane + 32 q = (row of the tile, share)
+  // column role: lane = ((plane, pair), share); row role: lane = ((plane, i), share), rows i and i + H2
   const int ci = lane / nsc, cs = lane - ci * nsc;
   const bool c_on = ci < np * W2;
   const int c_pl = c_on ? ci / W2 : 0, c_p = c_on ? ci - c_pl * W2 : 0;
-  const int r_s = lane % nsr;                        // the same for both rows: nsr divides 32
-  int r_row[2], r_pl[2];
-  bool r_on[2];
+  const int ri = lane / nsr, r_s = lane - ri * nsr;
+  const bool r_on = ri < np * H2;
+  const int r_pl = r_on ? ri / H2 : 0, r_i = r_on ? ri - r_pl * H2 : 0;
+  const bool r_two = r_i + H2 < H;                   // an odd height leaves the last lane one row
+  const int r_row0 = r_pl * H + r_i, r_row1 = r_two ? r_row0 + H2 : r_row0;
+  f2 acc3[2][R], acc4[2][R / 2];
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int it = lane + 32 * q, row = it / nsr;
-    r_on[q] = row < np * H;
-    r_row[q] = r_on[q] ? row : 0;
-    r_pl[q] = r_row[q] / H;
-  }
-  f2 acc3[2][R], acc4[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) acc3[0][j] = acc3[1][j] = acc4[j] = 0ull;
+  for (int j = 0; j < R; ++j) acc3[0][j] = acc3[1][j] = acc4[j & 1][j >> 1] = 0ull;
   int t = warp * (int)gridDim.x + (int)blockIdx.x, buf = 0;
   stage(T, t);
   for (; t < total; t += stride) {
@@ -394,8 +415,8 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
       f2 v[2][R];
 #pragma unroll
       for (int j = 0; j < R; ++j) v[0][j] = v[1][j] = 0ull;
-      const TX* x0 = Tc + r_row[0] * PT;
-      const TX* x1 = Tc + r_row[1] * PT;
+      const TX* x0 = Tc + r_row0 * PT;
+      const TX* x1 = Tc + r_row1 * PT;
       // all lanes take the same number of steps; a share past the row reads its last quad against zeros
 #pragma unroll 2
       for (int i = 0; i < W4; i += nsr) {
@@ -424,18 +445,18 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
         for (int o = 1; o < nsr; o *= 2)
 #pragma unroll
           for (int j = 0; j < R; ++j) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
-        if (r_on[q] && r_s == 0) {
-          float* d = V4d + r_pl[q] * v4s + (r_row[q] - r_pl[q] * H) * 2 * R;
+        if (r_on && r_s == 0 && (q == 0 || r_two)) {
+          float* d = V4d + r_pl * v4s + (r_i + q * H2) * R;
 #pragma unroll
-          for (int j = 0; j < R; j += 2) *reinterpret_cast<float4*>(d + 2 * j) = make_float4(s[j], s[j], s[j + 1], s[j + 1]);
+          for (int j = 0; j < R; j += 4) *reinterpret_cast<float4*>(d + j) = make_float4(s[j], s[j + 1], s[j + 2], s[j + 3]);
         }
       }
     }
     __syncwarp();
     {                                                // V3 and P4: columns
-      f2 v[R];
+      f2 v[2][R / 2];
 #pragma unroll
-      for (int j = 0; j < R; ++j) v[j] = 0ull;
+      for (int j = 0; j < R / 2; ++j) v[0][j] = v[1][j] = 0ull;
       const TX* x0 = Tc + c_pl * H * PT + 2 * c_p;
       const float* v4 = V4d + c_pl * v4s;
 #pragma unroll 2
@@ -443,37 +464,21 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
         const int h = i + cs < H ? i + cs : H - 1;
         f2 x = ld_pair(x0 + h * PT);
         if (i + cs >= H) x = 0ull;
-#pragma unroll
-        for (int j = 0; j < R; j += 2) {
-          const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(U3d + (h * R + j) * 2);
-          ffma2(v[j], x, u.x);
-          ffma2(v[j + 1], x, u.y);
-        }
-#pragma unroll
-        for (int j = 0; j < R; j += 2) {
-          const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(v4 + (h * R + j) * 2);
-          ffma2(acc4[j], x, u.x);
-          ffma2(acc4[j + 1], x, u.y);
-        }
+        fma_cols<R>(v, x, U3d + h * R);
+        fma_cols<R>(acc4, x, v4 + h * R);
       }
-      for (int o = 1; o < nsc; o *= 2)
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-          const float2 w = unpack2(v[j]);
-          v[j] = pack2(w.x + __shfl_xor_sync(0xffffffffu, w.x, o), w.y + __shfl_xor_sync(0xffffffffu, w.y, o));
-        }
+      sum_cols<R>(v, 1, nsc);
       if (c_on && cs == 0) {
         float* d = V3t + c_pl * v3s + 2 * c_p;
 #pragma unroll
-        for (int j = 0; j < R; ++j) *reinterpret_cast<f2*>(d + j * PT) = v[j];
+        for (int j = 0; j < R; ++j) *reinterpret_cast<float2*>(d + j * PT) = col_pair<R>(v, j);
       }
     }
     __syncwarp();
     {                                                // P3: rows
-      const TX* x0 = Tc + r_row[0] * PT;
-      const TX* x1 = Tc + r_row[1] * PT;
-      const float* va = V3t + r_pl[0] * v3s;
-      const float* vb = V3t + r_pl[1] * v3s;
+      const TX* x0 = Tc + r_row0 * PT;
+      const TX* x1 = Tc + r_row1 * PT;
+      const float* va = V3t + r_pl * v3s;
 #pragma unroll 1
       for (int i = 0; i < W4; i += nsr) {
         const int qa = i + r_s, wa = 4 * (qa < W4 ? qa : W4 - 1);
@@ -486,10 +491,6 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
           const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(va + j * PT + wa);
           ffma2(acc3[0][j], xa, u.x);
           ffma2(acc3[0][j], xb, u.y);
-        }
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
-          const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(vb + j * PT + wa);
           ffma2(acc3[1][j], ya, u.x);
           ffma2(acc3[1][j], yb, u.y);
         }
@@ -501,67 +502,65 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_cons
   if (tid == 0) pdl_wait();
   __syncthreads();
   // one partial of P3 and of P4 per CTA: warps, then planes, then shares, in index order
-  float* red = U4t + R * PT;                         // [nw][64][R], then [nw][32][2][R], over the idle tiles
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const float2 w = unpack2(acc3[q][j]);
-      red[(warp * 64 + lane + 32 * q) * R + j] = w.x + w.y;
-    }
-  __syncthreads();
-  for (int e = tid; e < H * R; e += blockDim.x) {
-    const int h = e / R, j = e % R;
-    float s = 0.f;
-    for (int w = 0; w < nw; ++w)
-      for (int i = 0; i < np; ++i)
-        for (int o = 0; o < nsr; ++o) s += red[(w * 64 + (i * H + h) * nsr + o) * R + j];
-    if (j < p.r3) p.Pp3[((int64_t)blockIdx.x * H + h) * p.r3 + j] = s;
-  }
-  __syncthreads();
+  float* red3 = U4t + R * PT;                        // [nw][R][2][32], over the idle tiles
+  float* red4 = red3 + nw * R * 64;                  // [nw][R][2][32]
 #pragma unroll
   for (int j = 0; j < R; ++j) {
-    const float2 w = unpack2(acc4[j]);
-    red[((warp * 32 + lane) * 2) * R + j] = w.x;
-    red[((warp * 32 + lane) * 2 + 1) * R + j] = w.y;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float2 w = unpack2(acc3[q][j]);
+      red3[((warp * R + j) * 2 + q) * 32 + lane] = w.x + w.y;
+    }
+    const float2 c = col_pair<R>(acc4, j);
+    red4[(warp * R + j) * 64 + lane] = c.x;
+    red4[(warp * R + j) * 64 + 32 + lane] = c.y;
   }
   __syncthreads();
-  for (int e = tid; e < W * R; e += blockDim.x) {
-    const int c = e / R, j = e % R;
+  for (int e = tid; e < (H + W) * R; e += blockDim.x) {
+    const bool rows = e < H * R;
+    const int n = rows ? H : W, f = rows ? e : e - H * R, j = f / n, k = f - j * n;
+    const int half = rows ? (k >= H2 ? 1 : 0) : (k & 1), i = rows ? k - half * H2 : k >> 1;
+    const int ns = rows ? nsr : nsc, per = (rows ? H2 : W2) * ns;
+    const float* src = (rows ? red3 : red4) + (j * 2 + half) * 32 + i * ns;
     float s = 0.f;
+#pragma unroll 2
     for (int w = 0; w < nw; ++w)
-      for (int i = 0; i < np; ++i)
-        for (int o = 0; o < nsc; ++o) s += red[((w * 32 + (i * W2 + (c >> 1)) * nsc + o) * 2 + (c & 1)) * R + j];
-    if (j < p.r4) p.Pp4[((int64_t)blockIdx.x * W + c) * p.r4 + j] = s;
+      for (int q = 0; q < np; ++q)
+        for (int o = 0; o < ns; ++o) s += src[w * R * 64 + q * per + o];
+    if (rows) {
+      if (j < p.r3) p.Pp3[((int64_t)blockIdx.x * H + k) * p.r3 + j] = s;
+    } else {
+      if (j < p.r4) p.Pp4[((int64_t)blockIdx.x * W + k) * p.r4 + j] = s;
+    }
   }
 }
 
 // planes per tile, row pitch, lanes per column pair and per row
 void wp_geometry(int H, int W, int* np, int* pitch, int* nsc, int* nsr) {
-  const int w2 = (W + 1) / 2, q = (W + 3) / 4;
+  const int w2 = (W + 1) / 2, h2 = (H + 1) / 2, q = (W + 3) / 4;
   *pitch = 4 * (q | 1);
-  *np = std::max(1, std::min(32 / w2, 64 / H));
+  *np = std::max(1, std::min(32 / w2, 32 / h2));
   *nsc = *nsr = 1;
   while (*nsc < 8 && 2 * *nsc <= H && *np * w2 * 2 * *nsc <= 32) *nsc *= 2;
-  while (*nsr < 8 && 2 * *nsr <= q && *np * H * 2 * *nsr <= 64) *nsr *= 2;
+  while (*nsr < 8 && 2 * *nsr <= q && *np * h2 * 2 * *nsr <= 32) *nsr *= 2;
 }
-size_t wp_fixed_bytes(int H, int pitch, int R) { return (size_t)(2 * H * R + R * pitch) * 4; }
+size_t wp_fixed_bytes(int H, int pitch, int R) { return (size_t)(H * R + R * pitch) * 4; }
 size_t wp_warp_bytes(int H, int np, int pitch, int R, bool bf16) {
-  const size_t b = (size_t)np * ((size_t)(H * 2 * R + 4 + R * pitch + 4) * 4 + (size_t)2 * H * pitch * (bf16 ? 2 : 4));
-  return std::max(b, (size_t)64 * R * 4);            // the final sums of a warp
+  const size_t b = (size_t)np * ((size_t)(H * R + 4 + R * pitch + 4) * 4 + (size_t)2 * H * pitch * (bf16 ? 2 : 4));
+  return std::max(b, (size_t)128 * R * 4);           // the final sums of a warp
 }
-int wp_warps(int H, int W, int R, bool bf16) {
+int wp_warps(int64_t n_planes, int H, int W, int R, bool bf16) {
   int np, pitch, nsc, nsr;
   wp_geometry(H, W, &np, &pitch, &nsc, &nsr);
-  const size_t n = (kWSmemBudget - wp_fixed_bytes(H, pitch, R)) / wp_warp_bytes(H, np, pitch, R, bf16);
-  return (int)std::min<size_t>(n, kWMaxWarps);
+  return ws_balance((kWSmemBudget - wp_fixed_bytes(H, pitch, R)) / wp_warp_bytes(H, np, pitch, R, bf16),
+                    (n_planes + np - 1) / np);
 }
 
 template <int R, int RK, bool VEC, typename TX>
 cudaError_t wfiber_t(const Fiber2Args& p, int grid, cudaStream_t st) {
   const bool bf16 = sizeof(TX) == 2;
-  const int nw = wf_warps(p.a, R, bf16);
-  const size_t smem = wf_fixed_bytes(p.a, R) + nw * wf_warp_bytes(p.a, R, RK, bf16);
+  const int nw = wf_warps(p.n_tiles, p.a, R, bf16);
+  const size_t smem = wf_fixed_bytes(p.a) + nw * wf_warp_bytes(p.a, R, RK, bf16);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_wfiber<R, RK, VEC, TX>), smem);
   if (e != cudaSuccess) return e;
   return launch_maybe_pdl(!p.plain, k_wfiber<R, RK, VEC, TX>, dim3(grid), dim3(32 * nw), smem, st, p);
@@ -582,7 +581,7 @@ cudaError_t wfiber_r(const Fiber2Args& p, int grid, bool bf16, bool vec, cudaStr
 template <int R, bool VEC, typename TX>
 cudaError_t wplane_t(const PlaneArgs& p, int grid, cudaStream_t st) {
   const bool bf16 = sizeof(TX) == 2;
-  const int nw = wp_warps(p.H, p.W, R, bf16);
+  const int nw = wp_warps(p.n_planes, p.H, p.W, R, bf16);
   const size_t smem = wp_fixed_bytes(p.H, p.pitch, R) + nw * wp_warp_bytes(p.H, p.np, p.pitch, R, bf16);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_wplane<R, VEC, TX>), smem);
   if (e != cudaSuccess) return e;
@@ -605,8 +604,8 @@ int64_t wfiber_tiles(int64_t O, int64_t a, int64_t I, bool bf16) {
 }
 // the same count for both types (a bf16 plan without tensor-core products has the fp32 plan's workspace)
 int wfiber_grid(int64_t O, int64_t a, int64_t I, int r) {
-  const int64_t nw = wf_warps((int)a, r <= 4 ? 4 : 8, false);
-  return (int)std::min<int64_t>((wfiber_tiles(O, a, I, false) + nw - 1) / nw, 148);
+  const int64_t tiles = wfiber_tiles(O, a, I, false), nw = wf_warps(tiles, (int)a, r <= 4 ? 4 : 8, false);
+  return (int)std::min<int64_t>((tiles + nw - 1) / nw, 148);
 }
 cudaError_t launch_wfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
   Fiber2Args p = p0;
@@ -625,7 +624,7 @@ bool wplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4) {
 int wplane_grid(int64_t n_planes, int H, int W, int r, bool bf16) {
   int np, pitch, nsc, nsr;
   wp_geometry(H, W, &np, &pitch, &nsc, &nsr);
-  const int64_t nw = wp_warps(H, W, r <= 4 ? 4 : 8, bf16), tiles = (n_planes + np - 1) / np;
+  const int64_t nw = wp_warps(n_planes, H, W, r <= 4 ? 4 : 8, bf16), tiles = (n_planes + np - 1) / np;
   return (int)std::min<int64_t>((tiles + nw - 1) / nw, 148);
 }
 cudaError_t launch_wplane(const PlaneArgs& p0, int grid, bool bf16, cudaStream_t st) {
