@@ -702,25 +702,36 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
                      pl->q_per_split[m], pl->bf16);
 }
 
-// cold start: P_m = A_m Omega_m for one mode
-asi_status_t expand_mode(const asi_plan* pl, int m, const void* act, const float* V, char* w, cudaStream_t st) {
-  if (pl->tc_mode[m] && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) {
-    const ModeView& v = pl->mv[m];
-    TcSplitArgs sp;
-    sp.n = 0;
-    sp.clear = nullptr;
-    tc_add_split(&sp, V, v.Q, v.r, w + pl->tcv_off[m]);
-    ASI_CUDA(launch_tc_split(sp, false, st));
-    const TcCall t = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
-                      pl->q_per_split[m], v.r, pl->nsplit[m], 1};
-    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
-    return ASI_OK;
-  }
+// cold start: P_m = A_m Omega_m of all modes, one launch of SIMT products and one of tensor-core products.
+// clear: the first launch here zeroes the status block (it is then not a dependent one)
+asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool clear,
+                          cudaStream_t st) {
+  int* const status = reinterpret_cast<int*>(w);
   GemmGroup g;
   g.np = 0;
-  g.clear = nullptr;
-  gemm_add(&g, simt_expand(pl, m, act, V, w));
-  ASI_CUDA(launch_gemm_group(g, pl->bf16, false, st));
+  TcSplitArgs sp;
+  sp.n = 0;
+  TcCall t[3];
+  for (int m = 0; m < pl->nd; ++m) {
+    const ModeView& v = pl->mv[m];
+    if (pl->tc_mode[m] && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) {
+      t[sp.n] = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
+                 pl->q_per_split[m], v.r, pl->nsplit[m], 1};
+      tc_add_split(&sp, omega[m], v.Q, v.r, w + pl->tcv_off[m]);
+    } else {
+      gemm_add(&g, simt_expand(pl, m, act, omega[m], w));
+    }
+  }
+  g.clear = clear ? status : nullptr;
+  if (g.np) {
+    ASI_CUDA(launch_gemm_group(g, pl->bf16, !clear, st));
+    clear = false;
+  }
+  if (sp.n) {
+    sp.clear = clear ? status : nullptr;
+    ASI_CUDA(launch_tc_split(sp, false, st));
+    ASI_CUDA(launch_tc_group(t, sp.n, status, true, st));
+  }
   return ASI_OK;
 }
 
@@ -1167,20 +1178,20 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
-  ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
-  int64_t off = 0;
+  const float* om[ASI_MAX_MODES];
   for (int m = 0; m < pl->nd; ++m) {
-    s = expand_mode(pl, m, act, omega + off, w, st);
-    if (s != ASI_OK) return s;
-    off += pl->mv[m].Q * pl->r[m];
+    om[m] = omega;
+    omega += pl->mv[m].Q * pl->r[m];
   }
+  s = expand_modes(pl, act, om, w, true, st);
+  if (s != ASI_OK) return s;
   return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
 }
 
 static size_t omega_scratch_bytes(const asi_plan* pl) {
-  int64_t mx = 0;
-  for (int m = 0; m < pl->nd; ++m) mx = std::max<int64_t>(mx, pl->mv[m].Q * pl->r[m]);
-  return align_up((size_t)mx * 4, 256);
+  size_t all = 0;
+  for (int m = 0; m < pl->nd; ++m) all += align_up((size_t)pl->mv[m].Q * pl->r[m] * 4, 256);
+  return all;
 }
 
 size_t asi_init_seeded_ws_bytes(const asi_plan_t* pl) {
@@ -1196,18 +1207,29 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
   char* w = static_cast<char*>(ws);
   float* omega = reinterpret_cast<float*>(w + align_up(pl->compress_ws, 256));
   if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
-  ASI_CUDA(cudaMemsetAsync(w, 0, kStatusBytes, st));
-  for (int m = 0; m < pl->nd; ++m) {               // one mode's Omega at a time, in the same scratch
-    ASI_CUDA(launch_fill_gaussian(seed, (uint32_t)m, pl->mv[m].Q * pl->r[m], omega, st));
-    s = expand_mode(pl, m, act, omega, w, st);
-    if (s != ASI_OK) return s;
+  FillArgs f;
+  size_t at = 0;
+  for (int m = 0; m < pl->nd; ++m) {
+    f.out[m] = reinterpret_cast<float*>(reinterpret_cast<char*>(omega) + at);
+    f.n[m] = pl->mv[m].Q * pl->r[m];
+    f.stream[m] = (uint32_t)m;
+    at += align_up((size_t)f.n[m] * 4, 256);
   }
+  f.clear = reinterpret_cast<int*>(w);
+  ASI_CUDA(launch_fill_gaussian(seed, f, pl->nd, st));
+  s = expand_modes(pl, act, f.out, w, false, st);
+  if (s != ASI_OK) return s;
   return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
 }
 
 asi_status_t asi_gaussian_stream(uint64_t seed, uint32_t stream_id, int64_t n, float* out, void* stream) {
   if (n < 0 || (n > 0 && !valid_ptr(out))) return ASI_ERR_INVALID_ARG;
-  ASI_CUDA(launch_fill_gaussian(seed, stream_id, n, out, static_cast<cudaStream_t>(stream)));
+  FillArgs f;
+  f.out[0] = out;
+  f.n[0] = n;
+  f.stream[0] = stream_id;
+  f.clear = nullptr;
+  ASI_CUDA(launch_fill_gaussian(seed, f, 1, static_cast<cudaStream_t>(stream)));
   return ASI_OK;
 }
 

@@ -47,7 +47,14 @@ __global__ void __launch_bounds__(256) k_philox_words(uint64_t seed, uint32_t st
   *reinterpret_cast<uint4*>(out + 4 * g) = make_uint4(r.w[0], r.w[1], r.w[2], r.w[3]);
 }
 
-__global__ void __launch_bounds__(256) k_fill_gaussian(uint64_t seed, uint32_t stream, int64_t n, float* out) {
+// One stream per row of the grid: the matrices of a layer's modes in one launch (28 x 28 x 128 x 64, ranks 4: four
+// launches and their gaps took 25 us, this one 6).
+__global__ void __launch_bounds__(256) k_fill_gaussian(uint64_t seed, const __grid_constant__ FillArgs p) {
+  pdl_launch_dependents();
+  if (p.clear && blockIdx.x == 0 && blockIdx.y == 0) p.clear[threadIdx.x] = 0;
+  const uint32_t stream = p.stream[blockIdx.y];
+  const int64_t n = p.n[blockIdx.y];
+  float* out = p.out[blockIdx.y];
   const int64_t ng = (n + 3) / 4;
   for (int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x; g < ng; g += (int64_t)gridDim.x * 256) {
     const Words r = philox4x32_10((uint32_t)g, (uint32_t)((uint64_t)g >> 32), stream, 0u, (uint32_t)seed,
@@ -73,11 +80,12 @@ cudaError_t launch_philox_words(uint64_t seed, uint32_t stream, int64_t n_groups
   return cudaGetLastError();
 }
 
-cudaError_t launch_fill_gaussian(uint64_t seed, uint32_t stream, int64_t n, float* out, cudaStream_t st) {
+cudaError_t launch_fill_gaussian(uint64_t seed, const FillArgs& p, int count, cudaStream_t st) {
+  int64_t n = 0;
+  for (int m = 0; m < count; ++m) n = std::max(n, p.n[m]);
   if (n <= 0) return cudaSuccess;
-  const int64_t ng = (n + 3) / 4;
-  const int64_t blocks = std::min<int64_t>((ng + 255) / 256, 148 * 8);
-  k_fill_gaussian<<<(unsigned)blocks, 256, 0, st>>>(seed, stream, n, out);
+  const int64_t blocks = std::min<int64_t>(((n + 3) / 4 + 255) / 256, 148 * 8);
+  k_fill_gaussian<<<dim3((unsigned)blocks, (unsigned)count), 256, 0, st>>>(seed, p);
   return cudaGetLastError();
 }
 
