@@ -1416,7 +1416,8 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
 // ---------------------------------------------------------------------------------------------
 // W[col][:] = sum_b X[b][col] U1[b][:] for the tile's J columns (jvalid of them exist): thread = VW neighbouring columns
 // and the samples b == h (mod NH), eight in flight, the NH shares meet in order.  The first eight are requested before
-// `factors` (the row solves, which end with a barrier) runs.
+// `factors` (the row solves, which end with a barrier) runs.  Shares are stored by rank, columns side by side: stored by
+// column they cost four times the shared-memory cycles (ResNet-18 tail at 64: 26.6 -> 24.5 us).
 template <int R, int VW, typename TX, typename F>
 __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t chw, int B, int J, int jvalid,
                                              const float* __restrict__ U1s, float* __restrict__ part, float* __restrict__ Ws,
@@ -1429,11 +1430,11 @@ __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t c
   dJ.divmod(tid, h, jq);
   const bool on = h < NH && jq * VW < jvalid;
   const TX* src = A + (on ? jq * VW : 0);
-  float acc[VW][R];
+  f2 acc[VW][R / 2];                                 // pairs of ranks
 #pragma unroll
   for (int c = 0; c < VW; ++c)
 #pragma unroll
-    for (int j = 0; j < R; ++j) acc[c][j] = 0.f;
+    for (int j = 0; j < R / 2; ++j) acc[c][j] = 0ull;
   const int nb = on && B > h ? (B - h + NH - 1) / NH : 0;   // samples of this thread
   if (!on) h = 0;
   src += (int64_t)h * chw;
@@ -1455,20 +1456,37 @@ __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t c
         x[t].get(xs);
         const float* u = U1s + (h + (t0 + t) * NH) * R;
 #pragma unroll
-        for (int c = 0; c < VW; ++c) fma_row<R>(acc[c], xs[c], u);
+        for (int j = 0; j < R / 2; j += 2) {
+          const ulonglong2 uj = *reinterpret_cast<const ulonglong2*>(u + 2 * j);
+#pragma unroll
+          for (int c = 0; c < VW; ++c) {
+            const f2 xc = pack2(xs[c], xs[c]);
+            ffma2(acc[c][j], xc, uj.x);
+            ffma2(acc[c][j + 1], xc, uj.y);
+          }
+        }
       }
   }
   if (on) {
-    float* dst = part + (h * J + jq * VW) * R;
+    float* dst = part + h * J * R + jq * VW;         // [h][j][J]: neighbours write neighbouring quads
 #pragma unroll
-    for (int c = 0; c < VW; ++c)
+    for (int j = 0; j < R; j += 2) {
+      float2 v[VW];
 #pragma unroll
-      for (int j = 0; j < R; j += 4)
-        *reinterpret_cast<float4*>(dst + c * R + j) = make_float4(acc[c][j], acc[c][j + 1], acc[c][j + 2], acc[c][j + 3]);
+      for (int c = 0; c < VW; ++c) v[c] = unpack2(acc[c][j / 2]);
+      if constexpr (VW == 4) {
+        *reinterpret_cast<float4*>(dst + j * J) = make_float4(v[0].x, v[1].x, v[2].x, v[3].x);
+        *reinterpret_cast<float4*>(dst + (j + 1) * J) = make_float4(v[0].y, v[1].y, v[2].y, v[3].y);
+      } else {
+        dst[j * J] = v[0].x;
+        dst[(j + 1) * J] = v[0].y;
+      }
+    }
   }
   __syncthreads();
-  for (int idx = tid; idx < jvalid * R; idx += kPT) {
+  for (int idx = tid; idx < J * R; idx += kPT) {
     float s = part[idx];
+#pragma unroll 4
     for (int q = 1; q < NH; ++q) s += part[q * J * R + idx];
     Ws[idx] = s;
   }
@@ -1487,8 +1505,8 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   float* U1s = smem;                    // [B][R]
   float* U3s = U1s + ((B * R + 3) & ~3);   // [H][R]
   float* U4s = U3s + H * R;             // [W][R]
-  float* Ws = U4s + W * R;              // [J][R]
-  float* part = Ws + J * R;             // [NH][J][R], at most 256 * 4 R
+  float* Ws = U4s + W * R;              // [R][J]
+  float* part = Ws + J * R;             // [NH][R][J], at most 256 * 4 R
   float* T1 = part;                     // [ncl r1][r3][W] after part is free
   auto factors = [&]() {
     pdl_wait();                         // P_m and the Cholesky factors come from the reduction kernel
@@ -1542,10 +1560,10 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
     dW.divmod(idx, t, w);
     d_r3.divmod(t, ci, k);
     d_r1.divmod(ci, cl, i);
-    const float* ws = Ws + (cl * HW + w) * R + i;
+    const float* ws = Ws + i * J + cl * HW + w;
     float s = 0.f;
 #pragma unroll 4
-    for (int h = 0; h < H; ++h) s = fmaf(ws[h * W * R], U3s[h * R + k], s);
+    for (int h = 0; h < H; ++h) s = fmaf(ws[h * W], U3s[h * R + k], s);
     T1[idx] = s;
   }
   __syncthreads();
