@@ -174,7 +174,7 @@ void layout_compress(asi_plan* pl) {
       qps = ((v.Q + ns - 1) / ns + 127) / 128 * 128;                     // expansion splits the columns over at most as many
     }
     if (pl->fiber[m] || (pl->plane && m >= 2)) {                         // one partial per CTA of k_fiber /
-      ns = pl->fiber[m] ? pl->fiber_grid[m] : pl->plane_grid;            // k_plane; the cold-start expansion
+      ns = pl->fiber[m] ? pl->fiber_grid[m] : pl->plane_grid;            // a plane kernel; the cold-start expansion
       qps = ((v.Q + ns - 1) / ns + 63) / 64 * 64;                        // uses the same count (empty splits
     }                                                                    // write 0)
     pl->nsplit[m] = (int)ns;

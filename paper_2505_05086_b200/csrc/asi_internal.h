@@ -45,7 +45,7 @@ struct FiberArgs {
   int* clear;          // as in PlaneArgs
 };
 
-// Modes 3 and 4 of a conv activation in one pass over whole planes (k_plane).
+// Modes 3 and 4 of a conv activation in one pass over whole planes (k_wplane; k_plane2 for S x S maps).
 struct PlaneArgs {
   const void* X;
   const float* U3;
