@@ -69,18 +69,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ uint64_t globaltimer_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// waits for the phase with the given parity; gives up after ~1 s
+// waits for the phase with the given parity; gives up after 2e9 cycles (a second or so).  The limit is on the SM's own
+// clock: a read of %globaltimer costs over 600 cycles, and every chunk that was not there yet paid one
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;       // the common case costs no timer read
-  const uint64_t t0 = globaltimer_ns();
+  if (mbar_try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
   for (uint32_t it = 0; it < (1u << 28); ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u && globaltimer_ns() - t0 > 1000000000ull) return false;
+    if ((it & 1023u) == 1023u && clock64() - t0 > 2000000000ll) return false;
   }
   return false;
 }
@@ -187,11 +183,12 @@ struct TcProb {
   int ksp;             // CTAs that share a tile (1 or the cluster size)
   int first;           // first CTA of the product in the launch (a multiple of the cluster size)
   int n_cta;
+  int nst;             // stages: as many as its operand width leaves room for beside a second CTA
 };
 struct TcGroup {
   TcProb p[3];
   int* status;         // status word of the caller's workspace (may be null): ASI_ERR_TIMEOUT when a wait expires
-  int np, nst, tmem_cols, cs;
+  int np, tmem_cols, cs;
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -232,7 +229,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   int q = 0;
   while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
   const TcProb& p = g.p[q];
-  const int nst = g.nst, N = p.N;
+  const int nst = p.nst, N = p.N;
   const uint32_t tile_b = (uint32_t)(3 * N) * 128u;     // operand tile: 3 N rows of 64 bf16
   const uint32_t stage = kTileA + tile_b;               // 1024-byte multiples: N is a multiple of 16
   // carve-up: stages, then barriers
@@ -379,24 +376,36 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   if (g.cs > 1) {
     // the shares of a tile meet: CTA `rank` adds the rows [rank * 128 / ksp, ..) in rank order
     cluster_sync_all();
-    if (p.ksp > 1 && live && !fail) {
-      const int rows = kTcM / p.ksp, r0 = rank * rows;
-      const int items = rows * (N / 4);
+    // at most four items a thread (128 N / (4 ksp) <= 1024); the CTA tells its peers that it is done with their tiles
+    // before it stores, so that the barrier does not wait for the stores as well
+    const int rows = kTcM / p.ksp, r0 = rank * rows, items = rows * (N / 4);
+    const bool meet = p.ksp > 1 && live && !fail;
+    float4 sum[4];
+    if (meet) {
       const uint32_t xa = smem_u32(xch);
-      for (int e = tid; e < items; e += kTcThreads) {
-        const int r = r0 + e % rows, c4 = e / rows;     // lanes = neighbouring rows: coalesced operand stores
-        const uint32_t a = xa + (uint32_t)(r * PN + 4 * c4) * 4u;
-        float4 v[4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) v[t] = ld_cluster4(a, (uint32_t)(t < p.ksp ? t : 0));
-        float4 sum = v[0];
+      for (int u = 0; u < 4; ++u) {
+        const int e = tid + u * kTcThreads, ec = e < items ? e : 0;
+        const int r = r0 + ec % rows, c4 = ec / rows;   // lanes = neighbouring rows: coalesced operand stores
+        const uint32_t a = xa + (uint32_t)(r * PN + 4 * c4) * 4u;
+        sum[u] = ld_cluster4(a, 0);
 #pragma unroll
         for (int t = 1; t < 4; ++t)
-          if (t < p.ksp) { sum.x += v[t].x; sum.y += v[t].y; sum.z += v[t].z; sum.w += v[t].w; }
-        tc_store4(p, s, row0 + r, 4 * c4, sum);
+          if (t < p.ksp) {
+            const float4 v = ld_cluster4(a, (uint32_t)t);
+            sum[u].x += v.x; sum[u].y += v.y; sum[u].z += v.z; sum[u].w += v.w;
+          }
       }
     }
-    cluster_sync_all();                                 // no CTA leaves while its tile is being read
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (meet) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = tid + u * kTcThreads;
+        if (e < items) tc_store4(p, s, row0 + r0 + e % rows, 4 * (e / rows), sum[u]);
+      }
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // no CTA leaves while its tile is being read
   }
 }
 
@@ -545,11 +554,15 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaS
   }
   g.cs = cs;
   g.tmem_cols = 3 * nmax <= 64 ? 64 : (3 * nmax <= 128 ? 128 : 256);
-  const int stage = (int)kTileA + 3 * nmax * 128;
-  g.nst = nmax <= 16 ? 4 : (nmax <= 48 ? 3 : 2);
-  size_t smem = 1024 + (size_t)g.nst * stage;
-  const size_t xch = 1024 + (size_t)kTcM * (nmax + 4) * 4;
-  if (xch > smem) smem = xch;
+  // every product its own stage count: with those of the widest one (two at 64 columns) the four chunks of a narrower
+  // product's tile took one round trip more
+  size_t smem = 0;
+  for (int q = 0; q < n; ++q) {
+    TcProb& p = g.p[q];
+    p.nst = p.N <= 16 ? 4 : (p.N <= 48 ? 3 : 2);
+    smem = std::max(smem, 1024 + (size_t)p.nst * (kTileA + 3 * p.N * 128));
+    smem = std::max(smem, 1024 + (size_t)kTcM * (p.N + 4) * 4);
+  }
   const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_tc_group), smem);
   if (e != cudaSuccess) return e;
   ProfScope prof(c[0].expand ? ASI_K_EXPAND : ASI_K_MODEPROD, st, bytes);
