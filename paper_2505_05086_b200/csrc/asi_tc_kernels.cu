@@ -19,7 +19,8 @@
 //     [3 n x 64] (cp.async.bulk.tensor, 128-byte swizzle);
 //   * an issuer thread launches 4 k-steps of tcgen05.mma (M = 128, N = 3 n, K = 16) per chunk and commits
 //     them to the mbarrier that frees the stage;
-//   * eight warps then read the three accumulator groups with tcgen05.ld (lane = row) and add them.
+//   * eight warps then read the three accumulator groups with tcgen05.ld (lane = row) and add them; a CTA of a product
+//     with many tiles takes several, and the stages fill with the next one's chunks meanwhile.
 // A launch uses clusters of 1, 2 or 4 CTAs: the CTAs of a cluster share one tile of a product whose contraction
 // is long (each takes a quarter of K, the partial tiles meet in distributed shared memory in rank order) or own
 // different tiles.  Stage count and TMEM columns follow n so that two CTAs share an SM: what bounds these products
@@ -53,6 +54,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
@@ -183,6 +187,8 @@ struct TcProb {
   int ksp;             // CTAs that share a tile (1 or the cluster size)
   int first;           // first CTA of the product in the launch (a multiple of the cluster size)
   int n_cta;
+  int tpc;             // tiles a CTA takes one after another (1 where CTAs share a tile)
+  int tiles;
   int nst;             // stages: as many as its operand width leaves room for beside a second CTA
 };
 struct TcGroup {
@@ -234,7 +240,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   const uint32_t stage = kTileA + tile_b;               // 1024-byte multiples: N is a multiple of 16
   // carve-up: stages, then barriers
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem) + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[1];
+  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[1], acc_free[1];
   __shared__ uint32_t tmem_slot[1];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -242,23 +248,31 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   const int cta = (int)blockIdx.x - p.first;
   const bool live = cta < p.n_cta;                      // padding CTAs of the last cluster only take the barriers
   const int rank = p.ksp > 1 ? (int)cluster_rank() : 0;
-  const int tile = live ? cta / p.ksp : 0;
-  const int row0 = (tile % p.mt) * kTcM, s = tile / p.mt;   // s: outer index (kTcToken) or split of K
-  int k_begin = p.mode == kTcToken ? 0 : s * p.k_per_split;
-  int k_end = (p.mode == kTcToken || p.K - k_begin < p.k_per_split) ? p.K : k_begin + p.k_per_split;
-  if (k_end < k_begin) k_end = k_begin;
-  int nchunk = (k_end - k_begin + kTcKC - 1) / kTcKC;   // a ragged last chunk is zero-filled by TMA
-  if (p.ksp > 1) {
-    const int per = (nchunk + p.ksp - 1) / p.ksp;
-    k_begin += rank * per * kTcKC;
-    nchunk = nchunk - rank * per < per ? nchunk - rank * per : per;
-    if (nchunk < 0) nchunk = 0;
-  }
-  if (!live) nchunk = 0;
+  // the tiles of this CTA: the first one and how many (one that is shared, or up to tpc neighbours)
+  const int tile0 = p.ksp > 1 ? cta / p.ksp : cta * p.tpc;
+  const int ntile = !live ? 0 : (p.ksp > 1 ? 1 : (p.tiles - tile0 < p.tpc ? p.tiles - tile0 : p.tpc));
+  struct Tile { int row0, s, k_begin, nchunk; };
+  auto tile_of = [&](int t) {
+    Tile x;
+    x.row0 = ((tile0 + t) % p.mt) * kTcM;
+    x.s = (tile0 + t) / p.mt;                           // outer index (kTcToken) or split of K
+    x.k_begin = p.mode == kTcToken ? 0 : x.s * p.k_per_split;
+    int k_end = (p.mode == kTcToken || p.K - x.k_begin < p.k_per_split) ? p.K : x.k_begin + p.k_per_split;
+    if (k_end < x.k_begin) k_end = x.k_begin;
+    x.nchunk = (k_end - x.k_begin + kTcKC - 1) / kTcKC; // a ragged last chunk is zero-filled by TMA
+    if (p.ksp > 1) {
+      const int per = (x.nchunk + p.ksp - 1) / p.ksp;
+      x.k_begin += rank * per * kTcKC;
+      x.nchunk = x.nchunk - rank * per < per ? x.nchunk - rank * per : per;
+      if (x.nchunk < 0) x.nchunk = 0;
+    }
+    return x;
+  };
 
   if (tid == 0) {
     for (int i = 0; i < nst; ++i) { mbar_init(full + i, 1); mbar_init(s_free + i, 1); }
     mbar_init(done, 1);
+    mbar_init(acc_free, kTcWorkers);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {                                      // TMEM: fp32 columns x 128 lanes (3 N are used)
@@ -276,15 +290,25 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   // The three bf16 terms of the factor are stacked along the operand's rows: one MMA of width 3 N per
   // k-step reads the X tile once and leaves the three partial products in three column groups of TMEM.
   bool ok = true;                                       // this thread's waits so far
-  if (nchunk > 0) {
-    if (warp == kTcWorkers) {
-      // ---- MMA issuer (one thread): 4 k-steps per chunk, then the commit that frees the stage
-      if (lane == 0) {
-        const uint32_t idesc = instr_desc_bf16(kTcM, 3 * N, a_mn);
-        const uint32_t a_base = smem_u32(base);
-        const uint64_t a_step = a_mn ? 128 : 2;         // a k-step is 16 bf16: 32 bytes inside the swizzle row of a
-        int st = 0;                                     // K-major tile, 16 rows (2048 bytes) of an MN-major tile
-        uint32_t ph = 0;                                // (start-address field in 16-byte units)
+  const int PN = N + 4;                                 // pitch of the exchanged tile: rows four banks apart
+  float* xch = reinterpret_cast<float*>(base);          // [128][PN], over the stages of a tile that is shared
+  if (warp == kTcWorkers) {
+    // ---- MMA issuer (one thread): 4 k-steps per chunk, then the commit that frees the stage
+    if (lane == 0) {
+      const uint32_t idesc = instr_desc_bf16(kTcM, 3 * N, a_mn);
+      const uint32_t a_base = smem_u32(base);
+      const uint64_t a_step = a_mn ? 128 : 2;           // a k-step is 16 bf16: 32 bytes inside the swizzle row of a
+      int st = 0, busy = 0;                             // K-major tile, 16 rows (2048 bytes) of an MN-major tile
+      uint32_t ph = 0;                                  // (start-address field in 16-byte units)
+#pragma unroll 1
+      for (int t = 0; t < ntile && ok; ++t) {
+        const int nchunk = tile_of(t).nchunk;
+        if (nchunk == 0) continue;
+        if (busy) {                                     // the workers have read the tile before
+          ok = mbar_wait(acc_free, (uint32_t)(busy + 1) & 1u);
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        ++busy;
 #pragma unroll 1
         for (int c = 0; c < nchunk && ok; ++c) {
           ok = mbar_wait(full + st, ph);
@@ -300,86 +324,103 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
         }
         umma_commit(done);
       }
-    } else if (warp == kTcWorkers + 1) {
-      // ---- TMA producer (one thread): keeps the stages full
-      if (lane == 0) {
-        int st = 0;
-        uint32_t ph = 1;
+    }
+  } else if (warp == kTcWorkers + 1) {
+    // ---- TMA producer (one thread): keeps the stages full, across tiles
+    if (lane == 0) {
+      int st = 0, n = 0;
+      uint32_t ph = 1;
 #pragma unroll 1
-        for (int c = 0; c < nchunk && ok; ++c) {
-          if (c >= nst) ok = mbar_wait(s_free + st, ph);
+      for (int t = 0; t < ntile && ok; ++t) {
+        const Tile x = tile_of(t);
+#pragma unroll 1
+        for (int c = 0; c < x.nchunk && ok; ++c, ++n) {
+          if (n >= nst) ok = mbar_wait(s_free + st, ph);
           if (!ok) break;
           uint8_t* As = base + st * stage;
           mbar_expect_tx(full + st, stage);
-          const int kc = k_begin + c * kTcKC;
+          const int kc = x.k_begin + c * kTcKC;
           if (p.mode == kTcLastExpand) {
-            tma_load_2d(As, &p.mapX, row0, kc, full + st);
-            tma_load_2d(As + kTileA / 2, &p.mapX, row0 + 64, kc, full + st);
+            tma_load_2d(As, &p.mapX, x.row0, kc, full + st);
+            tma_load_2d(As + kTileA / 2, &p.mapX, x.row0 + 64, kc, full + st);
           } else if (p.mode == kTcToken) {
-            tma_load_3d(As, &p.mapX, row0, kc, s, full + st);
-            tma_load_3d(As + kTileA / 2, &p.mapX, row0 + 64, kc, s, full + st);
+            tma_load_3d(As, &p.mapX, x.row0, kc, x.s, full + st);
+            tma_load_3d(As + kTileA / 2, &p.mapX, x.row0 + 64, kc, x.s, full + st);
           } else if (p.mode == kTcTokenExpand) {
             const int o = kc / p.inner;
-            tma_load_3d(As, &p.mapX, kc - o * p.inner, row0, o, full + st);
+            tma_load_3d(As, &p.mapX, kc - o * p.inner, x.row0, o, full + st);
           } else {
-            tma_load_2d(As, &p.mapX, kc, row0, full + st);
+            tma_load_2d(As, &p.mapX, kc, x.row0, full + st);
           }
           tma_load_2d(As + kTileA, &p.mapB, kc, 0, full + st);
           if (++st == nst) { st = 0; ph ^= 1u; }
         }
       }
-    } else {
-      ok = mbar_wait(done, 0);                          // every reader of TMEM observes the completed phase
     }
-  }
-  const bool fail = __syncthreads_or(ok ? 0 : 1) != 0;
-  pdl_launch_dependents();
-  const int PN = N + 4;                                 // pitch of the exchanged tile: rows four banks apart
-  float* xch = reinterpret_cast<float*>(base);          // [128][PN] (the stages are free now)
-  if (!fail && warp < kTcWorkers && live) {
-    // thread = row: warp w reads lanes 32 (w % 4) ..., warps 0-3 the columns [0, N/2), warps 4-7 the rest
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  } else {
+    // ---- workers: thread = row: warp w reads lanes 32 (w % 4) ..., warps 0-3 the columns [0, N/2), warps 4-7 the rest;
+    // the loads of the next tile are under way meanwhile
     const int half = N >> 1;                            // 8, 16, 24 or 32 columns per warp
     const int col0 = (warp >> 2) * half;
     const int r = (warp & 3) * 32 + lane;
     const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    for (int cc = 0; cc < half; cc += 8) {
-      float o[8];
-      if (nchunk > 0) {
-        uint32_t h[8], m[8], l[8];
-        tmem_ld8(taddr + (uint32_t)cc, h);
-        tmem_ld8(taddr + (uint32_t)(N + cc), m);
-        tmem_ld8(taddr + (uint32_t)(2 * N + cc), l);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int i = 0; i < 8; ++i)                     // small terms first
-          o[i] = (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = 0.f;         // an empty share of K
+    uint32_t ph = 0;
+#pragma unroll 1
+    for (int t = 0; t < ntile && ok; ++t) {
+      const Tile x = tile_of(t);
+      if (x.nchunk > 0) {
+        ok = mbar_wait(done, ph);                       // every reader of TMEM observes the completed phase
+        if (__any_sync(0xffffffffu, ok ? 0 : 1)) ok = false;
+        if (!ok) break;
+        ph ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      const float4 v0 = make_float4(o[0], o[1], o[2], o[3]), v1 = make_float4(o[4], o[5], o[6], o[7]);
-      if (p.ksp > 1) {
-        *reinterpret_cast<float4*>(xch + r * PN + col0 + cc) = v0;
-        *reinterpret_cast<float4*>(xch + r * PN + col0 + cc + 4) = v1;
-      } else {
-        tc_store4(p, s, row0 + r, col0 + cc, v0);
-        tc_store4(p, s, row0 + r, col0 + cc + 4, v1);
+      for (int cc = 0; cc < half; cc += 8) {
+        float o[8];
+        if (x.nchunk > 0) {
+          uint32_t h[8], m[8], l[8];
+          tmem_ld8(taddr + (uint32_t)cc, h);
+          tmem_ld8(taddr + (uint32_t)(N + cc), m);
+          tmem_ld8(taddr + (uint32_t)(2 * N + cc), l);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < 8; ++i)                   // small terms first
+            o[i] = (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) o[i] = 0.f;       // an empty share of K
+        }
+        if (x.nchunk > 0 && cc + 8 >= half && t + 1 < ntile) {   // all read: the accumulator is free
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_free);
+        }
+        const float4 v0 = make_float4(o[0], o[1], o[2], o[3]), v1 = make_float4(o[4], o[5], o[6], o[7]);
+        if (p.ksp > 1) {
+          *reinterpret_cast<float4*>(xch + r * PN + col0 + cc) = v0;
+          *reinterpret_cast<float4*>(xch + r * PN + col0 + cc + 4) = v1;
+        } else {
+          tc_store4(p, x.s, x.row0 + r, col0 + cc, v0);
+          tc_store4(p, x.s, x.row0 + r, col0 + cc + 4, v1);
+        }
       }
     }
   }
+  const bool fail = __syncthreads_or(ok ? 0 : 1) != 0;
+  pdl_launch_dependents();
   if (fail && tid == 0 && g.status) atomicMax(g.status, (int)ASI_ERR_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(g.tmem_cols) : "memory");
-  if (g.cs > 1) {
+  if (p.ksp > 1) {                                      // uniform in a cluster: its CTAs belong to one product
     // the shares of a tile meet: CTA `rank` adds the rows [rank * 128 / ksp, ..) in rank order
     cluster_sync_all();
     // at most four items a thread (128 N / (4 ksp) <= 1024); the CTA tells its peers that it is done with their tiles
     // before it stores, so that the barrier does not wait for the stores as well
     const int rows = kTcM / p.ksp, r0 = rank * rows, items = rows * (N / 4);
-    const bool meet = p.ksp > 1 && live && !fail;
+    const Tile x = tile_of(0);
+    const bool meet = live && !fail;
     float4 sum[4];
     if (meet) {
       const uint32_t xa = smem_u32(xch);
@@ -402,7 +443,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int e = tid + u * kTcThreads;
-        if (e < items) tc_store4(p, s, row0 + r0 + e % rows, 4 * (e / rows), sum[u]);
+        if (e < items) tc_store4(p, x.s, x.row0 + r0 + e % rows, 4 * (e / rows), sum[u]);
       }
     }
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // no CTA leaves while its tile is being read
@@ -549,7 +590,11 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaS
     TcProb& p = g.p[q];
     p.ksp = (cs > 1 && tiles[q] < 200 && chunks[q] >= 4 * cs) ? cs : 1;
     p.first = first;
-    p.n_cta = (int)tiles[q] * p.ksp;
+    // tiles in turn where there are more than the machine holds at a time (two CTAs an SM): the next tile's loads run
+    // under this one's epilogue, and the set-up (4 k of 12 k cycles) is paid once
+    p.tiles = (int)tiles[q];
+    p.tpc = p.ksp > 1 ? 1 : (int)std::min<int64_t>(8, (tiles[q] + 295) / 296);
+    p.n_cta = p.ksp > 1 ? (int)tiles[q] * p.ksp : (p.tiles + p.tpc - 1) / p.tpc;
     first += (p.n_cta + cs - 1) / cs * cs;
   }
   g.cs = cs;

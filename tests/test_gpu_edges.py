@@ -87,3 +87,11 @@ GROUPED = [
 def test_grouped_products_at_the_edges(dims, ranks, bf16):
     rho = tuple(0.25 ** (1.0 / max(r, 4)) for r in ranks)
     _two_steps(LayerSpec("t", "linear", dims, 37, ranks=ranks), bf16, rho=rho, tol=dict(TOL_F32, proj=1e-3, dw=1e-3))
+
+
+@pytest.mark.parametrize("dims", [(23, 40, 1664), (37, 72, 1088)])
+def test_tensor_core_products_with_several_tiles_a_cta(dims):
+    """299 and 333 tiles of the token products: two a CTA, the last CTA one; the second token count has a ragged chunk."""
+    ranks = (3, 16, 16)
+    _two_steps(LayerSpec("t", "linear", dims, 1600, ranks=ranks), True, rho=(0.6, 0.93, 0.93),
+               tol=dict(TOL_F32, proj=1e-3))
