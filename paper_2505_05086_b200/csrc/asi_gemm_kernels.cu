@@ -41,6 +41,23 @@ __device__ __forceinline__ float as_f(__nv_bfloat16 v) { return __bfloat162float
 template <typename TX, bool VEC> struct Regs { TX v[16]; };
 template <> struct Regs<__nv_bfloat16, true> { uint2 v[4]; };
 
+__device__ __forceinline__ int cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ float ld_cluster(const float* own, int rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(a)
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
 template <typename TX, bool KM, bool VEC, int BN>
 struct GemmTile {
   static constexpr bool kAsync = VEC && sizeof(TX) == 4;
@@ -159,13 +176,23 @@ struct GemmTile {
     }
   }
 
+  template <bool CL>
   static __device__ void run(const GemmProb& p, int cta, int nst, float* smem) {
     constexpr int TN = BN / 4;                         // columns per lane
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lm = lane & 7, ln = lane >> 3;
+    const bool shared = CL && p.ksp > 1;
+    const int rank = shared ? cluster_rank() : 0;
+    if (shared) cta /= p.ksp;
     const int mt = cta % p.tiles_m, rest = cta / p.tiles_m, o = rest % p.O, split = rest / p.O;
     const int m0 = mt * kGM;
-    const int kbeg = split * p.kps, kend = min(p.K, kbeg + p.kps);
-    const int nit = kend > kbeg ? (kend - kbeg + kGK - 1) / kGK : 0;
+    int kbeg = split * p.kps, kend = min(p.K, kbeg + p.kps);
+    int nit = kend > kbeg ? (kend - kbeg + kGK - 1) / kGK : 0;
+    if (shared) {                                      // this CTA's chunks of the tile it shares
+      const int per = (nit + p.ksp - 1) / p.ksp;
+      kbeg += rank * per * kGK;
+      kend = min(kend, kbeg + per * kGK);
+      nit = max(0, min(per, nit - rank * per));
+    }
     const TX* X = reinterpret_cast<const TX*>(p.X) + (KM ? 0 : (int64_t)o * p.sxo);
     const float* B = p.B;
     float* stage = smem;
@@ -274,6 +301,40 @@ struct GemmTile {
     }
     __syncthreads();
     float* Y = p.Y + (int64_t)split * p.ysplit + (int64_t)o * p.so;
+    if (shared) {
+      // the CTA's sum in place, then CTA `rank` adds its share of the tile over the cluster in rank order; it tells its
+      // peers that it is done with theirs before it stores
+      for (int e = tid; e < kGM * BN; e += kGT) {
+        float v = red[e];
+#pragma unroll
+        for (int w = 1; w < kGW; ++w) v += red[w * kGM * BN + e];
+        red[e] = v;
+      }
+      cluster_arrive();
+      cluster_wait();
+      const int per = kGM * BN / p.ksp;                // 32 values or more
+      constexpr int kItems = kGM * BN / 2 / kGT > 0 ? kGM * BN / 2 / kGT : 1;
+      float sum[kItems];
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) {
+        const int e = tid + u * kGT;
+        const float* src = red + rank * per + (e < per ? e : 0);
+        float v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = ld_cluster(src, t < p.ksp ? t : 0);
+        sum[u] = v[0];
+#pragma unroll
+        for (int t = 1; t < 8; ++t) sum[u] += t < p.ksp ? v[t] : 0.f;
+      }
+      cluster_arrive();
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) {
+        const int e = tid + u * kGT, m = (rank * per + e) / BN, j = (rank * per + e) % BN;
+        if (e < per && m0 + m < p.M && j < p.n) Y[(int64_t)j * p.sj + (int64_t)(m0 + m) * p.si] = sum[u];
+      }
+      cluster_wait();
+      return;
+    }
     if (BN >= 16 && p.sj == 1 && p.yvec) {              // rows of C are contiguous: four columns at a time
 #pragma unroll 1
       for (int e = tid; e < kGM * BN / 4; e += kGT) {
@@ -301,19 +362,20 @@ struct GemmTile {
   }
 };
 
-template <typename TX, bool KM, bool VEC>
+template <bool CL, typename TX, bool KM, bool VEC>
 __device__ __forceinline__ void gemm_dispatch(const GemmProb& p, int cta, int nst, float* smem) {
-  if (p.n <= 8) GemmTile<TX, KM, VEC, 8>::run(p, cta, nst, smem);
-  else if (p.n <= 16) GemmTile<TX, KM, VEC, 16>::run(p, cta, nst, smem);
-  else if (p.n <= 32) GemmTile<TX, KM, VEC, 32>::run(p, cta, nst, smem);
-  else GemmTile<TX, KM, VEC, 64>::run(p, cta, nst, smem);
+  if (p.n <= 8) GemmTile<TX, KM, VEC, 8>::template run<CL>(p, cta, nst, smem);
+  else if (p.n <= 16) GemmTile<TX, KM, VEC, 16>::template run<CL>(p, cta, nst, smem);
+  else if (p.n <= 32) GemmTile<TX, KM, VEC, 32>::template run<CL>(p, cta, nst, smem);
+  else GemmTile<TX, KM, VEC, 64>::template run<CL>(p, cta, nst, smem);
 }
 
 int bn_of(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : (n <= 32 ? 32 : 64)); }
 
 }  // namespace
 
-template <typename TX>
+// CL: a launch in clusters (kept apart: with the shares' code in one kernel every other launch was 1 to 2 % slower)
+template <typename TX, bool CL>
 __global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ GemmGroup g) {
   extern __shared__ __align__(16) float gemm_smem[];
   int q = 0;
@@ -321,13 +383,14 @@ __global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ G
   const GemmProb& p = g.p[q];
   const int cta = (int)blockIdx.x - p.first;
   pdl_wait();
+  if (CL && cta >= p.n_cta) return;                          // padding of the last cluster of a product without shared tiles
   if (blockIdx.x == 0 && g.clear) g.clear[threadIdx.x] = 0;   // status block of the workspace (256 ints)
   if (p.km) {
-    if (p.vec) gemm_dispatch<TX, true, true>(p, cta, g.nst, gemm_smem);
-    else gemm_dispatch<TX, true, false>(p, cta, g.nst, gemm_smem);
+    if (p.vec) gemm_dispatch<CL, TX, true, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<CL, TX, true, false>(p, cta, g.nst, gemm_smem);
   } else {
-    if (p.vec) gemm_dispatch<TX, false, true>(p, cta, g.nst, gemm_smem);
-    else gemm_dispatch<TX, false, false>(p, cta, g.nst, gemm_smem);
+    if (p.vec) gemm_dispatch<CL, TX, false, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<CL, TX, false, false>(p, cta, g.nst, gemm_smem);
   }
 }
 
@@ -404,12 +467,25 @@ cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st
   std::sort(g.p, g.p + g.np, [](const GemmProb& a, const GemmProb& b) {
     return (int64_t)std::min(a.K, a.kps) * bn_of(a.n) > (int64_t)std::min(b.K, b.kps) * bn_of(b.n);
   });
+  // a product of few tiles and a long contraction shares each tile between the CTAs of a cluster, as far as an
+  // SM still gets one CTA: 128 x 1280 by 16 columns on 4 CTAs took 12.9 us, ten chunks in turn, and takes 5.9 on 32 (99
+  // tiles of six chunks: 12.8 us as they are, 15.0 in pairs).  Up to three chunks the barriers cost what the split saves
+  int cs = 1;
+  for (int q = 0; q < g.np; ++q) {
+    const int64_t tiles = (int64_t)g.p[q].tiles_m * g.p[q].O * g.p[q].nsplit;
+    const int chunks = (std::min(g.p[q].K, g.p[q].kps) + kGK - 1) / kGK;
+    while (cs < 8 && tiles * 2 * cs <= 148 && chunks >= 4 && 2 * cs <= chunks) cs *= 2;
+  }
   int first = 0, bn = 8;
   double bytes = 0.0;
   for (int q = 0; q < g.np; ++q) {
     GemmProb& p = g.p[q];
+    const int64_t tiles = (int64_t)p.tiles_m * p.O * p.nsplit;
+    const int chunks = (std::min(p.K, p.kps) + kGK - 1) / kGK;
+    p.ksp = (cs > 1 && tiles * cs <= 148 && chunks >= 4 && cs <= chunks) ? cs : 1;
     p.first = first;
-    first += p.tiles_m * p.O * p.nsplit;
+    p.n_cta = (int)tiles * p.ksp;
+    first += (p.n_cta + cs - 1) / cs * cs;
     bn = std::max(bn, bn_of(p.n));
     bytes += (double)p.M * p.O * p.K * (bf16 ? 2 : 4);
   }
@@ -417,12 +493,32 @@ cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st
   const size_t stage = (size_t)(kGM * kPK + kGK * bn) * 4;
   const size_t smem = std::max<size_t>(stage * g.nst, (size_t)kGW * kGM * bn * 4);
   ProfScope prof(ASI_K_MODEPROD, st, bytes);
-  auto kernel = bf16 ? k_gemm_group<__nv_bfloat16> : k_gemm_group<float>;
+  auto kernel = cs > 1 ? (bf16 ? k_gemm_group<__nv_bfloat16, true> : k_gemm_group<float, true>)
+                       : (bf16 ? k_gemm_group<__nv_bfloat16, false> : k_gemm_group<float, false>);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  if (pdl) return launch_pdl(kernel, dim3((unsigned)first), dim3(kGT), smem, st, g);
-  kernel<<<(unsigned)first, kGT, smem, st>>>(g);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)first);
+  cfg.blockDim = dim3(kGT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (cs > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)cs;
+    at[na].val.clusterDim.y = 1;
+    at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  if (pdl) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, kernel, g);
 }
 
 }  // namespace asi

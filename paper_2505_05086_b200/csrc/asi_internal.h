@@ -331,6 +331,7 @@ struct GemmProb {
   int M, K, O, n;
   int nsplit, kps;         // K in nsplit parts of kps (a multiple of 128 unless nsplit == 1)
   int tiles_m, first;      // 32-row tiles; first CTA of the product in the launch
+  int ksp, n_cta;          // CTAs that share a tile (1 or the cluster size), CTAs of the product (set by the launcher)
   int km, vec, bvec, yvec; // k-major A; rows of A / of B readable, rows of C writable four values at a time
 };
 constexpr int kMaxGroup = 8;

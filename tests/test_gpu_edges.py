@@ -95,3 +95,11 @@ def test_tensor_core_products_with_several_tiles_a_cta(dims):
     ranks = (3, 16, 16)
     _two_steps(LayerSpec("t", "linear", dims, 1600, ranks=ranks), True, rho=(0.6, 0.93, 0.93),
                tol=dict(TOL_F32, proj=1e-3))
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims", [(128, 1280), (70, 1290), (33, 390)])
+def test_long_contractions_of_few_tiles(dims, bf16):
+    """Tiles shared by clusters of 8 and 2 CTAs, the last ones with an empty or a ragged share of the contraction."""
+    ranks = (12, 14)
+    _two_steps(LayerSpec("t", "linear", dims, 40, ranks=ranks), bf16, rho=(0.9, 0.9), tol=dict(TOL_F32, proj=1e-3))
