@@ -84,18 +84,27 @@ void choose_kernels(asi_plan* pl) {
     a.nt = 256;
     // term 5 expands the channels in two rounds when the staging blocks fit, else one at a time
     // (one at a time, too, where two would keep the CTA from sharing its SM with three others)
+    a.nbuf = 2;
     a.ncl = cpb >= 2 ? cpb / 2 : 1;
     if (sm_wgrad_smem(a, R) > 56 * 1024) a.ncl = 1;
+    // one staging block where two keep a fourth CTA off the SM (ResNet-18 tail at 64: 512 CTAs, three an SM took 29.8 us,
+    // four take 24.9)
+    if (sm_wgrad_smem(a, R) > 56 * 1024) {
+      a.nbuf = 1;
+      if (sm_wgrad_smem(a, R) > 56 * 1024) a.nbuf = 2;
+    }
     // 256 threads where three such CTAs share an SM and the stream of dY is short (at 128 x 784 values a CTA 512
     // threads take 28 us against 36; at 128 x 196, 256 take 39 us against 46), else 512.  A CTA that needs an SM for itself pays on
     // small maps only: larger ones recompute Z3 in every CTA, and four launches are faster (28 x 28, B = 128, seven
     // layers: 118 us here against 28 us a layer beside other work)
     const size_t need = sm_wgrad_smem(a, R);
     if (need > 75 * 1024 || B * cpb * HoWo > 32768) a.nt = 512;
+    if (a.nt == 512 && sm_wgrad_smem(a, R) > kSmemLimit) a.nt = 256;
     if (need <= 113 * 1024 || (need <= kSmemLimit && H * W <= 256)) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
       pl->wgrad_ncl = a.ncl;
+      pl->wgrad_nbuf = a.nbuf;
       pl->wgrad_nt = a.nt;
     }
   }
@@ -434,6 +443,7 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
   g->ncl = pl->wgrad_ncl;
   g->vec4 = pl->wgrad_vec4 ? 1 : 0;
   g->nt = pl->wgrad_nt;
+  g->nbuf = pl->wgrad_nbuf;
   if (g->vec4 && (reinterpret_cast<uintptr_t>(dY) & (pl->bf16 ? 7u : 15u))) return false;
   g->status = reinterpret_cast<int*>(w);
   g->bulk_store = (((pl->dims[1] / pl->d.groups) * pl->d.kh * pl->d.kw) % 4 == 0 &&

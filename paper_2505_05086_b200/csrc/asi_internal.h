@@ -183,7 +183,8 @@ struct SmWgradArgs {
   int B, C, Cout, H, W, Ho, Wo, kh, kw, sh, sw, ph, pw, groups, cpb;
   int vec4;                     // columns of dY may be read four at a time
   int nt;                       // threads per CTA: 256 or 512
-  int ncl;                      // output channels expanded per round of term 5 (divides cpb)
+  int ncl;
+  int nbuf;            // staging blocks of term 5: two, or one                      // output channels expanded per round of term 5 (divides cpb)
   int bulk_store;               // 1: dW row blocks leave through the bulk-copy engine (16-byte sized and aligned)
 };
 size_t sm_tile1_smem(int S, int R, int B, int C);
@@ -487,4 +488,5 @@ struct asi_plan {
   int fast_kind;                   // 7, 14: modes 3 and 4 as Gram matrices of such square maps; 0: any map of at most 256 positions
   int tile_S;                      // != 0: the first pass is k_sm_tile1 for this map size, else k_sm_pass1
   int fast_R, n_tiles_b, fast_cs, fast_cc, core_tile_c, n_tiles_core, cpb, wgrad_ncl, wgrad_nt, fold_gs;
+  int wgrad_nbuf;
 };

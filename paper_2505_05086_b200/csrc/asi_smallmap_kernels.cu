@@ -1719,9 +1719,12 @@ __device__ __forceinline__ void wgrad_expand_rows(const SmWgradArgs& p, const fl
     const int g = co / og;
     float* dw = p.dW + (int64_t)(c0 + rd * p.ncl) * nblk;
     const float* u2 = U2s + (int64_t)g * cg * R;
-    float* buf = stage + (rd & 1) * p.ncl * nblk;
-    if (p.bulk_store && rd >= 2) {
-      if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+    float* buf = stage + (p.nbuf == 2 ? (rd & 1) : 0) * p.ncl * nblk;
+    if (rd >= p.nbuf) {                              // the block's last round has left it
+      if (p.bulk_store && tid == 0) {
+        if (p.nbuf == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      }
       __syncthreads();
     }
     float* out = buf + grp * nblk;
@@ -1852,8 +1855,8 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
   const int H = p.H, W = p.W, HoWo = p.Ho * p.Wo, kk = p.kh * p.kw;
   const int J = p.cpb * HoWo;                        // dY columns of this CTA, contiguous per sample
   const int c0 = bid * p.cpb;
-  // staging blocks of term 5 reuse the tile's space: ncl channels per round, doubled when rounds follow
-  const int n_stage = (p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
+  // staging blocks of term 5 reuse the tile's space: ncl channels per round, nbuf of them when rounds follow
+  const int n_stage = (p.cpb > p.ncl ? p.nbuf : 1) * p.ncl * (p.C / p.groups) * kk;
   const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV, kNT);
   float* stage = smem;                               // term 5's blocks; before that the shares of Z1 [NH][J][R]
   float* part = smem;
@@ -2041,7 +2044,7 @@ size_t sm_wgrad_smem(const SmWgradArgs& p, int R) {
   const int J = p.cpb * p.Ho * p.Wo, kk = p.kh * p.kw, JV = p.vec4 ? J / 4 : J;
   const int N4 = r2 * kk;
   const size_t part = (size_t)wgrad_groups(JV, p.nt) * J * R,
-               stage = (size_t)(p.cpb > p.ncl ? 2 : 1) * p.ncl * (p.C / p.groups) * kk;
+               stage = (size_t)(p.cpb > p.ncl ? p.nbuf : 1) * p.ncl * (p.C / p.groups) * kk;
   size_t n = ((part > stage ? part : stage) + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
              (size_t)r1 * r2 * R * R + (size_t)p.H * R + (size_t)p.W * R +
              (size_t)r1 * r2 * p.H * R + ((size_t)r1 * r2 * (p.H + 2 * p.ph) * (p.W + 2 * p.pw) + 3) / 4 * 4 +

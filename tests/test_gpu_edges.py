@@ -34,6 +34,7 @@ ANY_MAP = [
     ((70, 21, 8, 32), (4, 5, 4, 6), 9, 1, 1, 0, 1),        # a row of 32 lanes, batch above one warp's share
     ((10, 130, 6, 6), (4, 4, 4, 4), 20, 3, 2, 1, 1),       # channels beyond one tile
     ((9, 6, 1, 5), (3, 4, 1, 2), 4, 1, 1, 0, 1),           # one row
+    ((64, 512, 7, 7), (4, 4, 4, 4), 8, 3, 1, 1, 1),        # one staging block for four rounds of output channels
 ]
 
 
