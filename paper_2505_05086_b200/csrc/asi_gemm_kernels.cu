@@ -65,7 +65,7 @@ struct GemmTile {
   static constexpr int kTileB = kGK * BN;
 
   // A chunk [k0, k0 + 128) x rows [m0, m0 + 32): position of element / vector t of this thread
-  static __device__ __forceinline__ void issue_async(float* As, const TX* X, const GemmProb& p, int m0, int k0, int kend) {
+  static __device__ __forceinline__ void issue_async(float* As, const TX* X, const GemmArg& p, int m0, int k0, int kend) {
     const int tid = threadIdx.x;
     if constexpr (KM) {
       const int v = tid & 31, k = k0 + 4 * v;
@@ -88,7 +88,7 @@ struct GemmTile {
       }
     }
   }
-  static __device__ __forceinline__ void load_regs(Regs<TX, VEC>& rg, const TX* X, const GemmProb& p, int m0, int k0, int kend) {
+  static __device__ __forceinline__ void load_regs(Regs<TX, VEC>& rg, const TX* X, const GemmArg& p, int m0, int k0, int kend) {
     const int tid = threadIdx.x;
     if constexpr (VEC) {
       static_assert(sizeof(TX) == 2, "fp32 vectors go through cp.async");
@@ -129,7 +129,7 @@ struct GemmTile {
       }
     }
   }
-  static __device__ __forceinline__ void store_regs(const Regs<TX, VEC>& rg, float* As, const GemmProb& p, int m0, int k0, int kend) {
+  static __device__ __forceinline__ void store_regs(const Regs<TX, VEC>& rg, float* As, const GemmArg& p, int m0, int k0, int kend) {
     const int tid = threadIdx.x;
     if constexpr (VEC) {
 #pragma unroll
@@ -155,7 +155,7 @@ struct GemmTile {
       }
     }
   }
-  static __device__ __forceinline__ void issue_b(float* Bs, const float* B, const GemmProb& p, int k0, int kend) {
+  static __device__ __forceinline__ void issue_b(float* Bs, const float* B, const GemmArg& p, int k0, int kend) {
     const int tid = threadIdx.x;
     if (p.bvec) {
       constexpr int VPR = BN / 4;
@@ -176,8 +176,9 @@ struct GemmTile {
     }
   }
 
-  template <bool CL>
-  static __device__ void run(const GemmProb& p, int cta, int nst, float* smem) {
+  // WIDE: p is one tile of one split, its first k is p.k0
+  template <bool CL, bool WIDE>
+  static __device__ void run(const GemmArg& p, int cta, int nst, float* smem) {
     constexpr int TN = BN / 4;                         // columns per lane
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lm = lane & 7, ln = lane >> 3;
     const bool shared = CL && p.ksp > 1;
@@ -185,7 +186,7 @@ struct GemmTile {
     if (shared) cta /= p.ksp;
     const int mt = cta % p.tiles_m, rest = cta / p.tiles_m, o = rest % p.O, split = rest / p.O;
     const int m0 = mt * kGM;
-    int kbeg = split * p.kps, kend = min(p.K, kbeg + p.kps);
+    int kbeg = WIDE ? p.k0 : split * p.kps, kend = WIDE ? p.K : min(p.K, kbeg + p.kps);
     int nit = kend > kbeg ? (kend - kbeg + kGK - 1) / kGK : 0;
     if (shared) {                                      // this CTA's chunks of the tile it shares
       const int per = (nit + p.ksp - 1) / p.ksp;
@@ -362,12 +363,12 @@ struct GemmTile {
   }
 };
 
-template <bool CL, typename TX, bool KM, bool VEC>
-__device__ __forceinline__ void gemm_dispatch(const GemmProb& p, int cta, int nst, float* smem) {
-  if (p.n <= 8) GemmTile<TX, KM, VEC, 8>::template run<CL>(p, cta, nst, smem);
-  else if (p.n <= 16) GemmTile<TX, KM, VEC, 16>::template run<CL>(p, cta, nst, smem);
-  else if (p.n <= 32) GemmTile<TX, KM, VEC, 32>::template run<CL>(p, cta, nst, smem);
-  else GemmTile<TX, KM, VEC, 64>::template run<CL>(p, cta, nst, smem);
+template <bool CL, bool WIDE, typename TX, bool KM, bool VEC>
+__device__ __forceinline__ void gemm_dispatch(const GemmArg& p, int cta, int nst, float* smem) {
+  if (p.n <= 8) GemmTile<TX, KM, VEC, 8>::template run<CL, WIDE>(p, cta, nst, smem);
+  else if (p.n <= 16) GemmTile<TX, KM, VEC, 16>::template run<CL, WIDE>(p, cta, nst, smem);
+  else if (p.n <= 32) GemmTile<TX, KM, VEC, 32>::template run<CL, WIDE>(p, cta, nst, smem);
+  else GemmTile<TX, KM, VEC, 64>::template run<CL, WIDE>(p, cta, nst, smem);
 }
 
 int bn_of(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : (n <= 32 ? 32 : 64)); }
@@ -376,21 +377,42 @@ int bn_of(int n) { return n <= 8 ? 8 : (n <= 16 ? 16 : (n <= 32 ? 32 : 64)); }
 
 // CL: a launch in clusters (kept apart: with the shares' code in one kernel every other launch was 1 to 2 % slower)
 template <typename TX, bool CL>
-__global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ GemmGroup g) {
+__global__ void __launch_bounds__(kGT, 2) k_gemm_group(const __grid_constant__ GemmArgs g) {
   extern __shared__ __align__(16) float gemm_smem[];
   int q = 0;
   while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
-  const GemmProb& p = g.p[q];
+  const GemmArg& p = g.p[q];
   const int cta = (int)blockIdx.x - p.first;
   pdl_wait();
   if (CL && cta >= p.n_cta) return;                          // padding of the last cluster of a product without shared tiles
   if (blockIdx.x == 0 && g.clear) g.clear[threadIdx.x] = 0;   // status block of the workspace (256 ints)
   if (p.km) {
-    if (p.vec) gemm_dispatch<CL, TX, true, true>(p, cta, g.nst, gemm_smem);
-    else gemm_dispatch<CL, TX, true, false>(p, cta, g.nst, gemm_smem);
+    if (p.vec) gemm_dispatch<CL, false, TX, true, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<CL, false, TX, true, false>(p, cta, g.nst, gemm_smem);
   } else {
-    if (p.vec) gemm_dispatch<CL, TX, false, true>(p, cta, g.nst, gemm_smem);
-    else gemm_dispatch<CL, TX, false, false>(p, cta, g.nst, gemm_smem);
+    if (p.vec) gemm_dispatch<CL, false, TX, false, true>(p, cta, g.nst, gemm_smem);
+    else gemm_dispatch<CL, false, TX, false, false>(p, cta, g.nst, gemm_smem);
+  }
+}
+
+// One product whose sizes 32 bits do not count (a batch mode has C H W columns): every CTA rebases the product to its own
+// tile and span in 64 bits and runs it as a narrow one.  Kept apart from k_gemm_group, which it would cost 2 to 3 % (the
+// cold start of a 64 x 128 x 28 x 28 layer takes 79.0 us, with 64-bit spans in the one kernel it took 80.5).
+template <typename TX>
+__global__ void __launch_bounds__(kGT, 2) k_gemm_wide(const __grid_constant__ GemmProb p, const int64_t first, const int nst,
+                                                      int* const clear) {
+  extern __shared__ __align__(16) float gemm_smem[];
+  __shared__ GemmArg w;
+  pdl_wait();
+  if (blockIdx.x == 0 && clear) clear[threadIdx.x] = 0;
+  if (threadIdx.x == 0) w = gemm_tile_arg(p, first + blockIdx.x, (int)sizeof(TX));
+  __syncthreads();
+  if (p.km) {
+    if (p.vec) gemm_dispatch<false, true, TX, true, true>(w, 0, nst, gemm_smem);
+    else gemm_dispatch<false, true, TX, true, false>(w, 0, nst, gemm_smem);
+  } else {
+    if (p.vec) gemm_dispatch<false, true, TX, false, true>(w, 0, nst, gemm_smem);
+    else gemm_dispatch<false, true, TX, false, false>(w, 0, nst, gemm_smem);
   }
 }
 
@@ -400,7 +422,7 @@ int gemm_expand_splits(int64_t a, int64_t Q) {
   const int64_t tiles = (a + kGM - 1) / kGM;
   int64_t ns = std::max<int64_t>(1, 296 / tiles);
   ns = std::min<int64_t>(ns, std::max<int64_t>(1, Q / (2 * kGK)));
-  return (int)std::min<int64_t>(ns, 296);
+  return (int)std::max<int64_t>(std::min<int64_t>(ns, 296), (Q + kGemmMaxSpan - 129) / (kGemmMaxSpan - 128));
 }
 
 GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_t a, int64_t I, int n, int64_t so, int64_t sj,
@@ -410,17 +432,16 @@ GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_
   p.X = X; p.B = B; p.Y = Y; p.n = n; p.ldb = n;
   p.km = I == 1;
   p.nsplit = 1;
-  p.K = (int)a; p.kps = p.K;
+  p.K = p.kps = p.kin = a;
   p.sj = sj;
   if (I == 1) {
-    p.M = (int)O; p.O = 1; p.ld = a; p.kin = p.K; p.si = so;
+    p.M = O; p.O = 1; p.ld = a; p.si = so;
   } else {
-    p.M = (int)I; p.O = (int)O; p.ld = I; p.sxo = a * I; p.kin = p.K; p.so = so; p.si = si;
+    p.M = I; p.O = O; p.ld = I; p.sxo = a * I; p.so = so; p.si = si;
   }
   const int64_t al = I == 1 ? a : I;
   p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
   p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(B) & 15u) == 0;
-  p.tiles_m = (p.M + kGM - 1) / kGM;
   p.yvec = p.sj == 1 && n % 4 == 0 && p.si % 4 == 0 && p.so % 4 == 0 && p.ysplit % 4 == 0 &&
            (reinterpret_cast<uintptr_t>(p.Y) & 15u) == 0;
   return p;
@@ -432,15 +453,14 @@ GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_
   std::memset(&p, 0, sizeof(p));
   p.X = X; p.B = V; p.Y = Pp; p.n = n; p.ldb = n;
   p.km = I != 1;
-  p.M = (int)a; p.O = 1; p.K = (int)(O * I);
-  p.nsplit = nsplit; p.kps = (int)kps;
+  p.M = a; p.O = 1; p.K = O * I;
+  p.nsplit = nsplit; p.kps = kps;
   p.ysplit = a * n; p.si = n; p.sj = 1;
   if (I == 1) { p.ld = a; p.kin = p.K; }
-  else { p.ld = I; p.kin = (int)I; p.sxo = a * I; }
+  else { p.ld = I; p.kin = I; p.sxo = a * I; }
   const int64_t al = I == 1 ? a : I;
   p.vec = al % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (bf16 ? 7u : 15u)) == 0;
   p.bvec = n % 4 == 0 && (reinterpret_cast<uintptr_t>(V) & 15u) == 0;
-  p.tiles_m = (p.M + kGM - 1) / kGM;
   p.yvec = p.sj == 1 && n % 4 == 0 && p.si % 4 == 0 && p.so % 4 == 0 && p.ysplit % 4 == 0 &&
            (reinterpret_cast<uintptr_t>(p.Y) & 15u) == 0;
   return p;
@@ -457,14 +477,53 @@ void gemm_add(GemmGroup* g, const GemmProb& p) {
   }
 }
 
-bool gemm_fits(int64_t O, int64_t a, int64_t I, int n) {
-  return n >= 1 && n <= ASI_MAX_RANK && O * I < (1ll << 30) && a < (1ll << 30) && ((I + kGM - 1) / kGM) * O < (1ll << 30);
+// 32 bits count every index of the product, up to the end of the last chunk of the last split
+bool gemm_narrow(const GemmProb& p) {
+  constexpr int64_t most = (1ll << 31) - 2 * kGM * kGK;
+  return p.M < most && p.K < most && p.kps < most && p.K + p.kps < most &&
+         (p.M + kGM - 1) / kGM * p.O < (1ll << 26) / p.nsplit;    // eight products, eight CTAs a tile
 }
 
-cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st) {
-  if (g.np < 1) return cudaSuccess;
+// a tile and a split of a wide product (t counts the row tiles, then the outer indices, then the splits) as a product of
+// its own
+__host__ __device__ GemmArg gemm_tile_arg(const GemmProb& p, int64_t t, int xbytes) {
+  const int64_t tiles_m = (p.M + kGM - 1) / kGM, m0 = t % tiles_m * kGM, o = t / tiles_m % p.O, split = t / tiles_m / p.O;
+  const int64_t k = split * p.kps, left = p.K - k, len = left < 0 ? 0 : (left < p.kps ? left : p.kps);
+  GemmArg w;
+  int64_t x = m0 * (p.km ? p.ld : 1) + o * p.sxo + (p.km ? k : k * p.ld);
+  w.k0 = 0;
+  w.sxo = p.sxo; w.ld = p.ld; w.ysplit = 0; w.so = 0; w.sj = p.sj; w.si = p.si;
+  w.kin = (int)len;                                  // one slab, unless the span reaches into a second one
+  if (p.km && p.kin < p.K && len > 0) {
+    const int64_t slab = k / p.kin, in = k - slab * p.kin;
+    x = m0 * p.ld + slab * p.sxo + in;
+    if (p.kin < kGemmMaxSpan) {                      // k counted from the start of the slab
+      w.k0 = (int)in;
+      w.kin = (int)p.kin;
+    } else if (p.kin - in < len) {                   // slabs longer than a span: the one end it holds comes to lie at 2^29
+      w.k0 = (int)(kGemmMaxSpan - (p.kin - in));
+      w.kin = (int)kGemmMaxSpan;
+      w.sxo = p.sxo - p.kin + kGemmMaxSpan;
+    }
+    x -= w.k0;
+  }
+  w.X = static_cast<const char*>(p.X) + (len > 0 ? x * xbytes : 0);
+  w.B = p.B + (len > 0 ? (k - w.k0) * p.ldb : 0);
+  w.Y = p.Y + split * p.ysplit + o * p.so + m0 * p.si;
+  w.ldb = p.ldb;
+  w.M = (int)(p.M - m0 < kGM ? p.M - m0 : kGM);
+  w.K = w.k0 + (int)len;
+  w.O = w.nsplit = w.tiles_m = w.ksp = w.n_cta = 1;
+  w.n = p.n;
+  w.kps = w.K;
+  w.first = 0;
+  w.km = p.km; w.vec = p.vec; w.bvec = p.bvec; w.yvec = p.yvec;
+  return w;
+}
+
+static cudaError_t launch_narrow(GemmArgs& g, bool bf16, bool pdl, cudaStream_t st) {
   // the longest contractions first: their CTAs would otherwise start last and run alone
-  std::sort(g.p, g.p + g.np, [](const GemmProb& a, const GemmProb& b) {
+  std::sort(g.p, g.p + g.np, [](const GemmArg& a, const GemmArg& b) {
     return (int64_t)std::min(a.K, a.kps) * bn_of(a.n) > (int64_t)std::min(b.K, b.kps) * bn_of(b.n);
   });
   // a product of few tiles and a long contraction shares each tile between the CTAs of a cluster, as far as an
@@ -477,9 +536,8 @@ cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st
     while (cs < 8 && tiles * 2 * cs <= 148 && chunks >= 4 && 2 * cs <= chunks) cs *= 2;
   }
   int first = 0, bn = 8;
-  double bytes = 0.0;
   for (int q = 0; q < g.np; ++q) {
-    GemmProb& p = g.p[q];
+    GemmArg& p = g.p[q];
     const int64_t tiles = (int64_t)p.tiles_m * p.O * p.nsplit;
     const int chunks = (std::min(p.K, p.kps) + kGK - 1) / kGK;
     p.ksp = (cs > 1 && tiles * cs <= 148 && chunks >= 4 && cs <= chunks) ? cs : 1;
@@ -487,12 +545,10 @@ cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st
     p.n_cta = (int)tiles * p.ksp;
     first += (p.n_cta + cs - 1) / cs * cs;
     bn = std::max(bn, bn_of(p.n));
-    bytes += (double)p.M * p.O * p.K * (bf16 ? 2 : 4);
   }
   g.nst = bn == 64 ? 2 : 3;
   const size_t stage = (size_t)(kGM * kPK + kGK * bn) * 4;
   const size_t smem = std::max<size_t>(stage * g.nst, (size_t)kGW * kGM * bn * 4);
-  ProfScope prof(ASI_K_MODEPROD, st, bytes);
   auto kernel = cs > 1 ? (bf16 ? k_gemm_group<__nv_bfloat16, true> : k_gemm_group<float, true>)
                        : (bf16 ? k_gemm_group<__nv_bfloat16, false> : k_gemm_group<float, false>);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
@@ -519,6 +575,61 @@ cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st
   cfg.attrs = at;
   cfg.numAttrs = na;
   return cudaLaunchKernelEx(&cfg, kernel, g);
+}
+
+template <typename TX>
+static cudaError_t launch_wide(const GemmProb& p, int* clear, bool pdl, cudaStream_t st) {
+  if (p.kps > (p.nsplit > 1 || p.kin < p.K ? kGemmMaxSpan : INT32_MAX - kGK)) return cudaErrorInvalidValue;
+  const int64_t ctas = (p.M + kGM - 1) / kGM * p.O * p.nsplit;
+  const int bn = bn_of(p.n), nst = bn == 64 ? 2 : 3;
+  const size_t stage = (size_t)(kGM * kPK + kGK * bn) * 4;
+  const size_t smem = std::max<size_t>(stage * nst, (size_t)kGW * kGM * bn * 4);
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_gemm_wide<TX>), smem);
+  for (int64_t t = 0; t < ctas && e == cudaSuccess; t += kGemmMaxGrid) {       // more tiles than a grid holds: in parts
+    e = launch_maybe_pdl(pdl, k_gemm_wide<TX>, dim3((unsigned)std::min(ctas - t, kGemmMaxGrid)), dim3(kGT), smem, st, p, t, nst,
+                         clear);
+    clear = nullptr;
+    pdl = true;
+  }
+  return e;
+}
+
+cudaError_t launch_gemm_group(const GemmGroup& group, bool bf16, bool pdl, cudaStream_t st) {
+  GemmArgs g;
+  g.np = 0;
+  g.clear = group.clear;
+  double bytes = 0.0;
+  for (int q = 0; q < group.np; ++q) {
+    const GemmProb& p = group.p[q];
+    bytes += (double)p.M * p.O * p.K * (bf16 ? 2 : 4);
+    if (!gemm_narrow(p)) continue;
+    GemmArg& a = g.p[g.np++];
+    a.X = p.X; a.B = p.B; a.Y = p.Y;
+    a.sxo = p.sxo; a.ld = p.ld; a.ysplit = p.ysplit; a.so = p.so; a.sj = p.sj; a.si = p.si;
+    a.ldb = p.ldb; a.kin = (int)p.kin;
+    a.M = (int)p.M; a.K = (int)p.K; a.O = (int)p.O; a.n = p.n;
+    a.nsplit = p.nsplit; a.kps = (int)p.kps;
+    a.tiles_m = (a.M + kGM - 1) / kGM;
+    a.k0 = 0;
+    a.km = p.km; a.vec = p.vec; a.bvec = p.bvec; a.yvec = p.yvec;
+  }
+  ProfScope prof(ASI_K_MODEPROD, st, bytes);
+  const bool any = g.np > 0;
+  if (any) {
+    const cudaError_t e = launch_narrow(g, bf16, pdl, st);
+    if (e != cudaSuccess) return e;
+  }
+  int* clear = any ? nullptr : group.clear;          // the first launch clears
+  pdl = pdl || any;
+  for (int q = 0; q < group.np; ++q) {
+    const GemmProb& p = group.p[q];
+    if (gemm_narrow(p)) continue;
+    const cudaError_t e = bf16 ? launch_wide<__nv_bfloat16>(p, clear, pdl, st) : launch_wide<float>(p, clear, pdl, st);
+    if (e != cudaSuccess) return e;
+    clear = nullptr;
+    pdl = true;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace asi

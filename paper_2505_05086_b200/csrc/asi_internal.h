@@ -327,22 +327,45 @@ struct GemmProb {
   const float* B;          // [K][ldb], columns 0 .. n - 1
   float* Y;                // C(o, m, j) of split s at s * ysplit + o * so + m * si + j * sj
   int64_t sxo, ld, ysplit, so, sj, si;
-  int ldb;                 // row pitch of B
-  int kin;                 // k-major A: k per outer slab of X (K when there is one)
-  int M, K, O, n;
-  int nsplit, kps;         // K in nsplit parts of kps (a multiple of 128 unless nsplit == 1)
-  int tiles_m, first;      // 32-row tiles; first CTA of the product in the launch
-  int ksp, n_cta;          // CTAs that share a tile (1 or the cluster size), CTAs of the product (set by the launcher)
+  int64_t M, K, O;
+  int64_t kin;             // k-major A: k per outer slab of X (K when there is one)
+  int64_t kps;             // K in nsplit parts of kps (a multiple of 128 unless nsplit == 1)
+  int ldb, n, nsplit;      // row pitch of B, columns
   int km, vec, bvec, yvec; // k-major A; rows of A / of B readable, rows of C writable four values at a time
 };
+// the same as the kernels take it, counted in 32 bits
+struct GemmArg {
+  const void* X;
+  const float* B;
+  float* Y;
+  int64_t sxo, ld, ysplit, so, sj, si;
+  int ldb, kin;
+  int M, K, O, n;
+  int nsplit, kps;
+  int tiles_m, first;      // 32-row tiles; first CTA of the product in the launch
+  int ksp, n_cta;          // CTAs that share a tile (1 or the cluster size), CTAs of the product (set by the launcher)
+  int km, vec, bvec, yvec;
+  int k0;                  // first k (a tile of a wide product)
+};
+constexpr int64_t kGemmMaxSpan = 1ll << 29;    // k of a split, where there are several
+constexpr int64_t kGemmMaxGrid = 1ll << 30;
 constexpr int kMaxGroup = 8;
 struct GemmGroup {
   GemmProb p[kMaxGroup];
-  int np, nst;
+  int np;
   int* clear;              // not null: the first CTA zeroes the 256 ints of the workspace's status block
 };
+struct GemmArgs {
+  GemmArg p[kMaxGroup];
+  int np, nst;
+  int* clear;
+};
+bool gemm_narrow(const GemmProb& p);
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+GemmArg gemm_tile_arg(const GemmProb& p, int64_t t, int xbytes);
 int gemm_expand_splits(int64_t a, int64_t Q);
-bool gemm_fits(int64_t O, int64_t a, int64_t I, int n);
 // Y(o, j, i) = sum_k X[o][k][i] B[k][j] at Y + o * so + j * sj + i * si
 void gemm_add(GemmGroup* g, const GemmProb& p);
 GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_t a, int64_t I, int n, int64_t so, int64_t sj,
@@ -350,7 +373,7 @@ GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_
 // Pp[s][k][j] = sum over the columns (o, i) of split s of X[o][k][i] V[(o, i)][j]
 GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_t a, int64_t I, int n, int nsplit, int64_t kps,
                      bool bf16);
-cudaError_t launch_gemm_group(GemmGroup& g, bool bf16, bool pdl, cudaStream_t st);
+cudaError_t launch_gemm_group(const GemmGroup& g, bool bf16, bool pdl, cudaStream_t st);
 
 int orth_rows(int64_t a, int r, int64_t nsplit);
 size_t orth_gp_elems(int64_t nchunk, int r);

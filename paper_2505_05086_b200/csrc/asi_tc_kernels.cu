@@ -496,7 +496,10 @@ int tc_operand_n(int n) { return pad16(n); }
 
 // Which products of mode (O, a, I) with n columns run here: 0 none, 1 the last mode, 2 a mode with inner extent
 int tc_kind(int64_t O, int64_t a, int64_t I, int n) {
-  if (n % 4 != 0 || n < 16 || n > kTcNMax || a >= (1ll << 31) || O * I >= (1ll << 31)) return 0;
+  // the kernel counts columns in 32 bits up to the end of the last split: 2^24 is more than a split of such a tensor that
+  // fits the device
+  constexpr int64_t most = (1ll << 31) - (1ll << 24);
+  if (n % 4 != 0 || n < 16 || n > kTcNMax || a >= most || O * I >= most) return 0;
   if (I == 1) return a % 64 == 0 && O >= kTcM ? 1 : 0;
   return I % 64 == 0 && O < 65536 ? 2 : 0;
 }
