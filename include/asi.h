@@ -153,7 +153,8 @@ asi_status_t asi_philox_words(uint64_t seed, uint32_t stream_id, int64_t n_group
  * fine-tuned layer at every step (Sec. 4 fine-tunes the last two to four layers), and the backward pass
  * needs every layer's weight gradient.  Arrays of n entries, entry i as in asi_compress / asi_*_wgrad;
  * every layer has its own workspace (distinct pointers).  Results are bit-identical to n separate
- * calls.  Layers on the fused small-map path that share a kernel variant (map size, rank bucket, input
+ * calls (layers of asi_wgrad_batched that share a workspace after all, or any two whose outputs or workspaces overlap,
+ * run one after another).  Layers on the fused small-map path that share a kernel variant (map size, rank bucket, input
  * type) share one launch per kernel stage -- a step of L such layers is 3 + 1 launches instead of
  * 3L + L --; such a group and every other layer run side by side on streams the library keeps (at most eight sets
  * of eight, destroyed with the last plan), forked from and joined to `stream` by events, or one after another when

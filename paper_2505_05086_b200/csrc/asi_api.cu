@@ -4,6 +4,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "asi_internal.h"
@@ -682,10 +683,27 @@ LaneSet* borrow_lanes(cudaStream_t st) {
   return l;
 }
 
-// Runs n_chains independent pieces of work, chain c on the caller's stream (c == 0) or on a lane.
+// What the layers of a batched call write, as address ranges.  Layers that write to the same memory (a workspace that
+// two of them share) run one after another, each with launches of its own.
+struct Written {
+  std::vector<std::pair<uintptr_t, uintptr_t>> r;
+  void add(const void* p, size_t bytes) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    if (bytes) r.emplace_back(at, at + bytes);
+  }
+  bool apart() {
+    std::sort(r.begin(), r.end());
+    for (size_t i = 1; i < r.size(); ++i)
+      if (r[i].first < r[i - 1].second) return false;
+    return true;
+  }
+};
+
+// Runs n_chains pieces of work, chain c on the caller's stream (c == 0, or all of them when they are not independent) or
+// on a lane.
 template <typename F>
-asi_status_t run_chains(int n_chains, cudaStream_t st, F&& chain) {
-  LaneSet* l = n_chains > 1 ? borrow_lanes(st) : nullptr;
+asi_status_t run_chains(int n_chains, bool independent, cudaStream_t st, F&& chain) {
+  LaneSet* l = n_chains > 1 && independent ? borrow_lanes(st) : nullptr;
   asi_status_t rc = ASI_OK;
   cudaError_t e = cudaSuccess;
   const int used = l ? std::min(n_chains - 1, kLanes) : 0;
@@ -1043,6 +1061,7 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
                                   void* const* ws, const size_t* ws_bytes, int32_t n, void* stream) {
   if (!plans || !acts || !U_prev || !U_new || !cores || !ws || !ws_bytes || n < 1 || n > 4096)
     return ASI_ERR_INVALID_ARG;
+  Written out;
   for (int i = 0; i < n; ++i) {
     const asi_plan* pl = plans[i];
     if (!pl || !valid_ptr(acts[i]) || !valid_ptr(U_prev[i]) || !valid_ptr(U_new[i]) || !valid_ptr(cores[i]))
@@ -1053,7 +1072,11 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (pl->fast_compress && fused_misaligned(pl, acts[i])) return ASI_ERR_INVALID_ARG;
     for (int j = 0; j < i; ++j)
       if (ws[j] == ws[i]) return ASI_ERR_INVALID_ARG;            // every layer needs a workspace of its own
+    out.add(ws[i], pl->compress_ws);
+    out.add(U_new[i], (size_t)pl->u_elems * 4);
+    out.add(cores[i], (size_t)pl->core_elems * 4);
   }
+  const bool apart = out.apart();
   // chains: one per group of fused layers of a variant, one per other layer
   std::vector<char> done(n, 0);
   std::vector<std::vector<int>> chains;
@@ -1061,7 +1084,7 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
   for (int i = 0; i < n; ++i) {
     if (done[i]) continue;
     std::vector<int> grp(1, i);
-    if (plans[i]->fast_compress) {
+    if (plans[i]->fast_compress && apart) {
       const Variant v(plans[i]);
       for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j) {
         const asi_plan* q = plans[j];
@@ -1071,7 +1094,7 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     for (int j : grp) done[j] = 1;
     chains.push_back(std::move(grp));
   }
-  return run_chains((int)chains.size(), static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
+  return run_chains((int)chains.size(), apart, static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
     const std::vector<int>& grp = chains[c];
     const int g = (int)grp.size(), i0 = grp[0];
     if (g == 1)
@@ -1102,6 +1125,7 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
                                const void* const* dY, float* const* dW, void* const* ws, const size_t* ws_bytes,
                                int32_t n, void* stream) {
   if (!plans || !cores || !U || !dY || !dW || !ws || !ws_bytes || n < 1 || n > 4096) return ASI_ERR_INVALID_ARG;
+  Written out;
   for (int i = 0; i < n; ++i) {
     const asi_plan* pl = plans[i];
     if (!pl || !valid_ptr(cores[i]) || !valid_ptr(U[i]) || !valid_ptr(dY[i]) || !valid_ptr(dW[i]))
@@ -1109,14 +1133,17 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     const asi_status_t s = check_ws(ws[i], ws_bytes[i], pl->wgrad_ws);
     if (s != ASI_OK) return s;
     if (pl->fast_wgrad && pl->wgrad_vec4 && (reinterpret_cast<uintptr_t>(dY[i]) & (pl->bf16 ? 7u : 15u))) return ASI_ERR_INVALID_ARG;
+    out.add(ws[i], pl->wgrad_ws);
+    out.add(dW[i], (size_t)pl->dw_elems * 4);
   }
+  const bool apart = out.apart();
   std::vector<char> done(n, 0);
   std::vector<std::vector<int>> chains;
   const int maxb = sm_max_batch();
   for (int i = 0; i < n; ++i) {
     if (done[i]) continue;
     std::vector<int> grp(1, i);
-    if (plans[i]->fast_wgrad)
+    if (plans[i]->fast_wgrad && apart)
       for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j)
         if (!done[j] && plans[j]->fast_wgrad && plans[j]->fast_R == plans[i]->fast_R && plans[j]->bf16 == plans[i]->bf16 &&
             plans[j]->wgrad_nt == plans[i]->wgrad_nt)
@@ -1124,7 +1151,7 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     for (int j : grp) done[j] = 1;
     chains.push_back(std::move(grp));
   }
-  return run_chains((int)chains.size(), static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
+  return run_chains((int)chains.size(), apart, static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
     const std::vector<int>& grp = chains[c];
     const int g = (int)grp.size(), i0 = grp[0];
     const asi_plan* p0 = plans[i0];

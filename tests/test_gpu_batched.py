@@ -71,3 +71,78 @@ def test_mixed_batch_fused_generic_and_linear_layers():
                            gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(L.dims, L.ranks)))
                for i, L in enumerate(specs)]
     _check_batch(specs, streams, oracle_layers=(0, 1, 2, 3, 4))
+
+
+def _random_layers(specs, seed):
+    """Runners with random orthonormal factors, and random inputs (no oracle: single calls are the reference)."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    runs, acts, dys = [], [], []
+    for L in specs:
+        r = make_runner(L)
+        r.set_factors([torch.linalg.qr(torch.randn(d, k, generator=gen, device="cuda"))[0].cpu().numpy()
+                       for d, k in zip(L.dims, L.ranks)])
+        runs.append(r)
+        acts.append(torch.randn(*L.dims, generator=gen, device="cuda"))
+        dys.append(torch.randn(*L.dy_shape, generator=gen, device="cuda"))
+    return runs, acts, dys
+
+
+SHARING = [LayerSpec("a", "conv", (8, 24, 28, 28), 40, 3, 1, 1, 1, ranks=(3, 4, 3, 4)),      # four launches, split Z4
+           LayerSpec("b", "conv", (8, 24, 30, 26), 24, 3, 1, 1, 1, ranks=(4, 5, 6, 4)),
+           LayerSpec("c", "linear", (6, 37, 50), 21, ranks=(3, 5, 7)),
+           LayerSpec("d", "conv", (8, 12, 7, 7), 10, 3, 1, 1, 1, ranks=(3, 4, 3, 2)),        # fused
+           LayerSpec("e", "conv", (8, 16, 7, 7), 16, 3, 1, 1, 1, ranks=(2, 3, 3, 3))]
+
+
+@pytest.mark.parametrize("which", ["workspace", "overlap", "gradient"])
+def test_wgrad_layers_that_share_memory_run_one_after_another(which):
+    """One workspace for all layers, workspaces that overlap in part, and layers of one shape with one dW: what separate
+    calls give, twenty times over."""
+    specs = SHARING if which != "gradient" else [SHARING[0]] * 3
+    runs, acts, dys = _random_layers(specs, 7)
+    want = []
+    for r, a, d in zip(runs, acts, dys):
+        r.compress(a)
+        r.wgrad(d)
+        want.append(r.dW.clone())
+    from paper_2505_05086_b200.runner import StepRunner
+    step = StepRunner(runs)
+    most = max(r.ws_w.numel() for r in runs)
+    arena = torch.zeros(most + 4096 * len(runs), dtype=torch.uint8, device="cuda")
+    if which == "gradient":
+        for r in runs[1:]:
+            r.dW = runs[0].dW
+    else:
+        for i, r in enumerate(runs):
+            at = 4096 * i if which == "overlap" else 0
+            r.ws_w = arena[at:at + most]
+    for _ in range(20):
+        for r in runs:
+            r.dW.fill_(float("nan"))
+        step.wgrad(dys)
+        torch.cuda.synchronize()
+        if which == "gradient":
+            assert torch.equal(runs[0].dW, want[-1])
+        else:
+            assert all(torch.equal(r.dW, w) for r, w in zip(runs, want))
+
+
+def test_compress_layers_whose_workspaces_overlap_run_one_after_another():
+    runs, acts, _ = _random_layers(SHARING, 8)
+    want = []
+    for r, a in zip(runs, acts):
+        r.compress(a)
+        want.append((r.U[r.cur].clone(), r.core.clone()))
+        r.cur = 1 - r.cur
+    from paper_2505_05086_b200.runner import StepRunner
+    most = max(r.ws_c.numel() for r in runs)
+    arena = torch.zeros(most + 4096 * len(runs), dtype=torch.uint8, device="cuda")
+    for i, r in enumerate(runs):
+        r.ws_c = arena[4096 * i:4096 * i + most]
+    step = StepRunner(runs)
+    for _ in range(20):
+        step.compress(acts)
+        torch.cuda.synchronize()
+        for r, (u, c) in zip(runs, want):
+            assert torch.equal(r.U[r.cur], u) and torch.equal(r.core, c)
+            r.cur = 1 - r.cur
