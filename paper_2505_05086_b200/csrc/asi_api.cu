@@ -316,6 +316,14 @@ bool fused_misaligned(const asi_plan* pl, const void* act) {
   return (pl->fast_vec4 || pl->tile_S) && (reinterpret_cast<uintptr_t>(act) & (pl->bf16 ? 7u : 15u)) != 0;
 }
 
+// asi_compress takes this address: the fused kernels' rule, or the 16-byte rows of the large-map kernels' bulk copies
+bool compress_takes(const asi_plan* pl, const void* act) {
+  if (pl->fast_compress) return !fused_misaligned(pl, act);
+  bool rows16 = pl->plane2;
+  for (int m = 0; m < pl->nd; ++m) rows16 = rows16 || pl->fiber2[m];
+  return !rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+}
+
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
   if (!valid_ptr(ws)) return ASI_ERR_INVALID_ARG;
   if (have < need || (reinterpret_cast<uintptr_t>(ws) & 255u)) return ASI_ERR_WORKSPACE;
@@ -924,10 +932,10 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
   if (U_prev == U_new) return ASI_ERR_INVALID_ARG;
   asi_status_t s = check_ws(ws, ws_bytes, pl->compress_ws);
   if (s != ASI_OK) return s;
+  if (!compress_takes(pl, act)) return ASI_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   if (pl->fast_compress) {
-    if (fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
     if (pl->tile_S) {
       SmTile1Args a;
       build_tile1(pl, act, U_prev, w, &a);
@@ -939,8 +947,6 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
     }
     return finish_compress(pl, act, U_new, core, w, U_prev, false, st);
   }
-  for (int m = 0; m < pl->nd; ++m)                   // bulk and 16-byte copies; errors before anything is enqueued
-    if ((pl->fiber2[m] || pl->plane2) && (reinterpret_cast<uintptr_t>(act) & 15u)) return ASI_ERR_INVALID_ARG;
   // The first kernel on the caller's stream clears the status block and starts only when the stream's earlier work
   // is done; the mode passes behind it do not depend on one another and are launched as programmatic dependents
   // (each waits for its predecessor before it ends, so that what follows the last one sees all of them).
@@ -1069,7 +1075,7 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (U_prev[i] == U_new[i]) return ASI_ERR_INVALID_ARG;
     const asi_status_t s = check_ws(ws[i], ws_bytes[i], pl->compress_ws);
     if (s != ASI_OK) return s;
-    if (pl->fast_compress && fused_misaligned(pl, acts[i])) return ASI_ERR_INVALID_ARG;
+    if (!compress_takes(pl, acts[i])) return ASI_ERR_INVALID_ARG;
     for (int j = 0; j < i; ++j)
       if (ws[j] == ws[i]) return ASI_ERR_INVALID_ARG;            // every layer needs a workspace of its own
     out.add(ws[i], pl->compress_ws);

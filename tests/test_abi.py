@@ -160,3 +160,18 @@ def test_batched_entry_points_validate_before_enqueuing(asi):
     assert L.asi_compress_batched(h, fake, fake, other, fake, fake, small, n, None) == ASI_ERR_WORKSPACE
     assert L.asi_wgrad_batched(h, fake, fake, None, fake, fake, big, n, None) == ASI_ERR_INVALID_ARG
     assert L.asi_wgrad_batched(h, fake, fake, fake, fake, fake, small, n, None) == ASI_ERR_WORKSPACE
+
+
+def test_a_misaligned_layer_of_a_batch_is_refused_before_the_others_start(asi):
+    """The 16-byte rule of the large-map kernels is checked for every layer of the batch first: without a GPU a call that
+    had begun to enqueue its first layer would report a CUDA error instead."""
+    from paper_2505_05086_b200.binding import ASI_ERR_INVALID_ARG
+    L = asi.lib()
+    plans = [asi.Plan("conv", (8, 12, 7, 7), (3, 4, 3, 2), cout=10, k=3, stride=1, pad=1),
+             asi.Plan("conv", (8, 64, 56, 56), (3, 4, 3, 3), cout=64, k=3, stride=1, pad=1)]
+    h = (C.c_void_p * 2)(*[p.handle.value for p in plans])
+    far = [(C.c_void_p * 2)((2 * i + 1) << 40, (2 * i + 2) << 40) for i in range(5)]
+    acts = (C.c_void_p * 2)(1 << 50, (1 << 51) + 8)
+    big = (C.c_size_t * 2)(1 << 36, 1 << 36)
+    assert L.asi_compress(h[1], acts[1], far[1][1], far[2][1], far[3][1], far[4][1], big[1], None) == ASI_ERR_INVALID_ARG
+    assert L.asi_compress_batched(h, acts, far[1], far[2], far[3], far[4], big, 2, None) == ASI_ERR_INVALID_ARG
