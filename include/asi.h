@@ -28,7 +28,12 @@
  *     returned immediately and nothing is enqueued.  Conditions only the
  *     device can see (a rank-deficient A_m A_m^T U_m) are written to a status
  *     word at the start of the workspace and read back by asi_poll_status.
- *   - Workspaces must be 256-byte aligned.
+ *   - Workspaces must be 256-byte aligned.  act and dY may start at any element
+ *     of their type (16-byte aligned ones are read faster), with one exception:
+ *     outside the fused small maps (conv layers of at most 256 positions, ranks
+ *     <= 8) asi_compress may use 16-byte copies where a mode's rows are whole
+ *     multiples of 16 bytes; it then needs act on 16 bytes and returns
+ *     ASI_ERR_INVALID_ARG otherwise.
  */
 #ifndef ASI_B200_H
 #define ASI_B200_H

@@ -311,17 +311,19 @@ void layout_wgrad(asi_plan* pl) {
   pl->wgrad_ws = off;
 }
 
-// the fused kernels read the activation four values at a time where its columns allow it
-bool fused_misaligned(const asi_plan* pl, const void* act) {
-  return (pl->fast_vec4 || pl->tile_S) && (reinterpret_cast<uintptr_t>(act) & (pl->bf16 ? 7u : 15u)) != 0;
+// act and dY are read four values at a time where they start on 16 bytes (bf16: 8), else one at a time
+bool four_aligned(const asi_plan* pl, const void* p) {
+  return (reinterpret_cast<uintptr_t>(p) & (pl->bf16 ? 7u : 15u)) == 0;
+}
+bool element_aligned(const asi_plan* pl, const void* p) {
+  return (reinterpret_cast<uintptr_t>(p) & (elem_bytes(pl) - 1)) == 0;
 }
 
-// asi_compress takes this address: the fused kernels' rule, or the 16-byte rows of the large-map kernels' bulk copies
+// asi_compress takes this address: any element's, but for the 16-byte rows of the large-map kernels' bulk copies
 bool compress_takes(const asi_plan* pl, const void* act) {
-  if (pl->fast_compress) return !fused_misaligned(pl, act);
   bool rows16 = pl->plane2;
   for (int m = 0; m < pl->nd; ++m) rows16 = rows16 || pl->fiber2[m];
-  return !rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+  return element_aligned(pl, act) && (!rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
 }
 
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
@@ -363,7 +365,8 @@ void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev,
   a->pitch = sm_pass1_pitch(a->H * a->W);
   a->off_u2 = sm_pass1_off_u2(pl->fast_R, a->cc, a->pitch);
   a->vec4 = pl->fast_vec4 ? 1 : 0;
-  a->bulk = (!pl->bf16 && pl->fast_vec4) ? 1 : 0;
+  a->aligned = four_aligned(pl, act) ? 1 : 0;
+  a->bulk = (!pl->bf16 && pl->fast_vec4 && a->aligned) ? 1 : 0;
   a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;      // 1 ms under the test hook, else 1 s
 }
@@ -380,6 +383,7 @@ void build_tile1(const asi_plan* pl, const void* act, const float* U_prev, char*
   a->B = (int)pl->dims[0];
   a->C = (int)pl->dims[1];
   a->n_tiles_b = pl->n_tiles_b;
+  a->aligned = four_aligned(pl, act) ? 1 : 0;
   a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;
 }
@@ -434,11 +438,10 @@ void build_fused_core(const asi_plan* pl, const void* act, float* U_new, float* 
   c->W = (int)pl->dims[3];
   c->tile_c = pl->core_tile_c;
   c->n_tiles = pl->n_tiles_core;
-  c->vec4 = (pl->fast_vec4 && (pl->core_tile_c * c->H * c->W) % 4 == 0) ? 1 : 0;
+  c->vec4 = (pl->fast_vec4 && (pl->core_tile_c * c->H * c->W) % 4 == 0 && four_aligned(pl, act)) ? 1 : 0;
 }
 
-// false: dY is not aligned as the staged copies of this plan need
-bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, char* w,
+void build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, char* w,
                        SmWgradArgs* g) {
   g->core = core; g->U = U; g->dY = dY; g->dW = dW;
   for (int m = 0; m < 4; ++m) {
@@ -450,14 +453,12 @@ bool build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, co
   g->kh = pl->d.kh; g->kw = pl->d.kw; g->sh = pl->d.stride_h; g->sw = pl->d.stride_w;
   g->ph = pl->d.pad_h; g->pw = pl->d.pad_w; g->groups = pl->d.groups; g->cpb = pl->cpb;
   g->ncl = pl->wgrad_ncl;
-  g->vec4 = pl->wgrad_vec4 ? 1 : 0;
+  g->vec4 = pl->wgrad_vec4 && four_aligned(pl, dY) ? 1 : 0;
   g->nt = pl->wgrad_nt;
   g->nbuf = pl->wgrad_nbuf;
-  if (g->vec4 && (reinterpret_cast<uintptr_t>(dY) & (pl->bf16 ? 7u : 15u))) return false;
   g->status = reinterpret_cast<int*>(w);
   g->bulk_store = (((pl->dims[1] / pl->d.groups) * pl->d.kh * pl->d.kw) % 4 == 0 &&
                    (reinterpret_cast<uintptr_t>(dW) & 15u) == 0) ? 1 : 0;
-  return true;
 }
 
 // U_m^{new} = Orthogonalize(P_m) for all modes given the split partials.
@@ -1090,11 +1091,12 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
   for (int i = 0; i < n; ++i) {
     if (done[i]) continue;
     std::vector<int> grp(1, i);
-    if (plans[i]->fast_compress && apart) {
+    // layers whose activations are read value by value have launches of their own
+    if (plans[i]->fast_compress && apart && four_aligned(plans[i], acts[i])) {
       const Variant v(plans[i]);
       for (int j = i + 1; j < n && (int)grp.size() < maxb; ++j) {
         const asi_plan* q = plans[j];
-        if (!done[j] && q->fast_compress && v == Variant(q)) grp.push_back(j);
+        if (!done[j] && q->fast_compress && v == Variant(q) && four_aligned(q, acts[j])) grp.push_back(j);
       }
     }
     for (int j : grp) done[j] = 1;
@@ -1138,7 +1140,7 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
       return ASI_ERR_INVALID_ARG;
     const asi_status_t s = check_ws(ws[i], ws_bytes[i], pl->wgrad_ws);
     if (s != ASI_OK) return s;
-    if (pl->fast_wgrad && pl->wgrad_vec4 && (reinterpret_cast<uintptr_t>(dY[i]) & (pl->bf16 ? 7u : 15u))) return ASI_ERR_INVALID_ARG;
+    if (!element_aligned(pl, dY[i])) return ASI_ERR_INVALID_ARG;
     out.add(ws[i], pl->wgrad_ws);
     out.add(dW[i], (size_t)pl->dw_elems * 4);
   }
@@ -1167,8 +1169,7 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     std::vector<SmWgradArgs> wa(g);
     for (int k = 0; k < g; ++k) {
       const int j = grp[k];
-      if (!build_fused_wgrad(plans[j], cores[j], U[j], dY[j], dW[j], static_cast<char*>(ws[j]), &wa[k]))
-        return ASI_ERR_INVALID_ARG;                  // alignment: refused above, before anything was enqueued
+      build_fused_wgrad(plans[j], cores[j], U[j], dY[j], dW[j], static_cast<char*>(ws[j]), &wa[k]);
     }
     ASI_CUDA(launch_sm_wgrad_batched(wa.data(), g, p0->fast_R, p0->bf16, st));
     return ASI_OK;
@@ -1220,7 +1221,7 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
   if (s != ASI_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
-  if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
+  if (!element_aligned(pl, act)) return ASI_ERR_INVALID_ARG;
   const float* om[ASI_MAX_MODES];
   for (int m = 0; m < pl->nd; ++m) {
     om[m] = omega;
@@ -1249,7 +1250,7 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   float* omega = reinterpret_cast<float*>(w + align_up(pl->compress_ws, 256));
-  if (pl->fast_compress && fused_misaligned(pl, act)) return ASI_ERR_INVALID_ARG;
+  if (!element_aligned(pl, act)) return ASI_ERR_INVALID_ARG;
   FillArgs f;
   size_t at = 0;
   for (int m = 0; m < pl->nd; ++m) {
@@ -1287,14 +1288,14 @@ asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float
                             float* dW, void* ws, size_t ws_bytes, void* stream) {
   if (!pl || !valid_ptr(core) || !valid_ptr(U) || !valid_ptr(dY) || !valid_ptr(dW))
     return ASI_ERR_INVALID_ARG;
-  if (pl->d.kind != ASI_CONV2D) return ASI_ERR_INVALID_ARG;
+  if (pl->d.kind != ASI_CONV2D || !element_aligned(pl, dY)) return ASI_ERR_INVALID_ARG;
   asi_status_t s = check_ws(ws, ws_bytes, pl->wgrad_ws);
   if (s != ASI_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* w = static_cast<char*>(ws);
   if (pl->fast_wgrad) {
     SmWgradArgs g;
-    if (!build_fused_wgrad(pl, core, U, dY, dW, w, &g)) return ASI_ERR_INVALID_ARG;
+    build_fused_wgrad(pl, core, U, dY, dW, w, &g);
     ASI_CUDA(launch_sm_wgrad(g, pl->fast_R, pl->bf16, st));
     return ASI_OK;
   }
@@ -1331,7 +1332,7 @@ asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const flo
                               float* dW, void* ws, size_t ws_bytes, void* stream) {
   if (!pl || !valid_ptr(core) || !valid_ptr(U) || !valid_ptr(dY) || !valid_ptr(dW))
     return ASI_ERR_INVALID_ARG;
-  if (pl->d.kind != ASI_LINEAR) return ASI_ERR_INVALID_ARG;
+  if (pl->d.kind != ASI_LINEAR || !element_aligned(pl, dY)) return ASI_ERR_INVALID_ARG;
   asi_status_t s = check_ws(ws, ws_bytes, pl->wgrad_ws);
   if (s != ASI_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -118,6 +118,7 @@ struct SmTile1Args {            // k_sm_tile1
   int64_t u_off[ASI_MAX_MODES];
   int r[ASI_MAX_MODES];
   int B, C, n_tiles_b;
+  int aligned;                  // act starts on 16 bytes (bf16: 8); else it is read one value at a time (never batched)
   unsigned long long wait_ns;   // limit of the bounded wait on the bulk-copy barrier
   int stall_copy;               // test hook: the producer arms the barrier but issues no copy (the wait must expire)
 };
@@ -131,8 +132,9 @@ struct SmPass1Args {            // k_sm_pass1
   int B, C, H, W, n_tiles_b;    // n_tiles_b: role-B CTAs (column tiles of all samples)
   int cs, cc, pitch, off_u2;    // role C: CTAs per sample, channels per CTA, floats per channel, start of U_2 in shared memory
   int cl;                       // cluster size of the launch, a multiple of cs
-  int vec4;                     // columns may be read four at a time (C H W % 4 == 0, 16-byte aligned base)
-  int bulk;                     // role C's tile comes by bulk copies (fp32, vec4)
+  int vec4;                     // columns come in whole groups of four (C H W % 4 == 0)
+  int aligned;                  // act starts on 16 bytes (bf16: 8); else a group is read value by value (never batched)
+  int bulk;                     // role C's tile comes by bulk copies (fp32, vec4, aligned)
   unsigned long long wait_ns;   // limit of the bounded wait on the bulk-copy barrier
   int stall_copy;               // test hook: the producer arms the barrier but issues no copy (the wait must expire)
 };
@@ -170,7 +172,7 @@ struct SmCoreArgs {
   int64_t u_off[ASI_MAX_MODES];
   int r[ASI_MAX_MODES];
   int B, C, H, W, tile_c, n_tiles;   // tile_c: channels per tile
-  int vec4;                     // as in SmPass1Args
+  int vec4;                     // columns may be read four at a time (whole groups, aligned)
 };
 struct SmWgradArgs {
   const float* core;

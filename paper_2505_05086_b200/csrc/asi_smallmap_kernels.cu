@@ -278,10 +278,12 @@ __device__ __forceinline__ void gram14_slot(int o, int& rl, int& e) {
 // ---------------------------------------------------------------------------------------------
 constexpr int kPT = 256;             // threads per CTA of k_sm_pass1 and k_sm_core
 
-template <typename TX, int VW> struct RawCol;                 // VW neighbouring values as they lie in memory
+// VW neighbouring values as they lie in memory: load() wants the address a multiple of all four, load_any() of one
+template <typename TX, int VW> struct RawCol;
 template <> struct RawCol<float, 4> {
   float4 v;
   __device__ __forceinline__ void load(const float* p) { v = __ldg(reinterpret_cast<const float4*>(p)); }
+  __device__ __forceinline__ void load_any(const float* p) { v = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3)); }
   __device__ __forceinline__ void get(float (&x)[4]) const { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
 };
 template <> struct RawCol<float, 1> {
@@ -292,6 +294,10 @@ template <> struct RawCol<float, 1> {
 template <> struct RawCol<__nv_bfloat16, 4> {
   uint2 v;
   __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint2*>(p)); }
+  __device__ __forceinline__ void load_any(const __nv_bfloat16* p) {
+    const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+    v = make_uint2(__ldg(q) | (uint32_t)__ldg(q + 1) << 16, __ldg(q + 2) | (uint32_t)__ldg(q + 3) << 16);
+  }
   __device__ __forceinline__ void get(float (&x)[4]) const {
     x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xffff0000u);
     x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xffff0000u);
@@ -334,7 +340,7 @@ __device__ __forceinline__ void fma_pairs(f2 (&acc)[2][R], float4 x, const f2* _
   }
 }
 
-template <int R, int VW, typename TX>
+template <int R, int VW, bool ANY, typename TX>
 __device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, float* smem) {
   constexpr int JT = 32 * VW, BPG = 32 / R;          // columns; samples per thread and butterfly of the expansion
   constexpr int U = 8;                               // samples in flight per thread
@@ -365,7 +371,11 @@ __device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, flo
   for (int t0 = 0; t0 < nb || !waited; t0 += U) {
     RawCol<TX, VW> x[U];
 #pragma unroll
-    for (int t = 0; t < U; ++t) x[t].load(A + (int64_t)(t0 + t < nb ? t0 + t : 0) * step);
+    for (int t = 0; t < U; ++t) {
+      const TX* at = A + (int64_t)(t0 + t < nb ? t0 + t : 0) * step;
+      if constexpr (ANY) x[t].load_any(at);
+      else x[t].load(at);
+    }
     if (!waited) {
       fac_wait();
       __syncthreads();
@@ -419,7 +429,11 @@ __device__ __forceinline__ void pass1_role_b(const SmPass1Args& p, int tile, flo
   for (int t0 = 0; t0 < nb; t0 += BPG) {
     RawCol<TX, VW> x[BPG];
 #pragma unroll
-    for (int q = 0; q < BPG; ++q) x[q].load(A + (int64_t)(t0 + q < nb ? t0 + q : nb - 1) * step);
+    for (int q = 0; q < BPG; ++q) {
+      const TX* at = A + (int64_t)(t0 + q < nb ? t0 + q : nb - 1) * step;
+      if constexpr (ANY) x[q].load_any(at);
+      else x[q].load(at);
+    }
     float val[32];
 #pragma unroll
     for (int q = 0; q < BPG; ++q) {
@@ -511,7 +525,7 @@ __device__ __forceinline__ void planes_modes34(const float* Xs, int P, int nc, i
   }
 }
 
-template <int KIND, int R, typename TX>
+template <int KIND, int R, bool ANY, typename TX>
 __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, float* smem) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ __align__(8) uint64_t s_bar;
@@ -530,7 +544,7 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
   float* U3s = Vp + (kPT / HW) * HW * R;             // KIND 0: [H][R], [W][R], [8][32][R]
   float* red = Xs;                                   // free once every thread is done with the tile
   const TX* A = reinterpret_cast<const TX*>(p.act) + ((int64_t)b * C + c0) * HW;
-  const bool bulk = std::is_same<TX, float>::value && p.bulk;
+  const bool bulk = !ANY && std::is_same<TX, float>::value && p.bulk;
   if (bulk) {
     const char* src = reinterpret_cast<const char*>(A);
     if (P == HW) {
@@ -561,7 +575,7 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
         dHW.divmod(idx, c, q);
         cp_async4(Xs + c * P + q, reinterpret_cast<const float*>(A) + idx, 4);
       }
-    } else if (p.vec4) {
+    } else if (!ANY && p.vec4) {
       const FDiv dV(HW % 4 == 0 ? HW / 4 : 1 << 20);
       for (int i0 = tid; i0 < nc * HW / 4; i0 += 4 * kPT) {
         uint2 raw[4];
@@ -744,7 +758,9 @@ __device__ __forceinline__ void pass1_role_c(const SmPass1Args& p, int bid, floa
   if (synced) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <int KIND, int R, typename TX>
+// ANY: the activation starts at any element (its columns still come in groups of four where they are whole groups, so
+// that the partials do not depend on the address)
+template <int KIND, int R, bool ANY, typename TX>
 __device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
@@ -753,10 +769,10 @@ __device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid
   if (bid >= nc_ctas) {
     const int tile = bid - nc_ctas;
     if (tile >= p.n_tiles_b) return;                 // padding to whole clusters
-    if (p.vec4) pass1_role_b<R, 4, TX>(p, tile, smem);
-    else pass1_role_b<R, 1, TX>(p, tile, smem);
+    if (p.vec4) pass1_role_b<R, 4, ANY, TX>(p, tile, smem);
+    else pass1_role_b<R, 1, false, TX>(p, tile, smem);
   } else if (bid < p.B * p.cs) {
-    pass1_role_c<KIND, R, TX>(p, bid, smem);
+    pass1_role_c<KIND, R, ANY, TX>(p, bid, smem);
   } else {                                           // padding: only the cluster's barriers
     for (int i = 0; i < 2; ++i) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
   }
@@ -902,10 +918,13 @@ __device__ __forceinline__ void project_channels(const float* __restrict__ Xs, c
 }
 
 // Stages one tile [B x J] (row b at src + b*sample_stride) as fp32 rows of pitch PJ.
-template <typename TX>
+template <bool ANY, typename TX>
 __device__ __forceinline__ void stage_tile_begin(const TX* __restrict__ src, int64_t sample_stride, float* Xs,
                                                  int B, int J, int PJ) {
-  if constexpr (std::is_same<TX, float>::value) {
+  if constexpr (ANY) {                               // one value at a time
+    for (int b = threadIdx.x >> 5; b < B; b += kTT / 32)
+      for (int j = threadIdx.x & 31; j < J; j += 32) Xs[b * PJ + j] = to_f(src[b * sample_stride + j]);
+  } else if constexpr (std::is_same<TX, float>::value) {
     stage_rows_async(Xs, src, B, J, sample_stride, PJ);
   } else {
     const int J4 = J / 4;
@@ -922,9 +941,9 @@ __device__ __forceinline__ void stage_tile_begin(const TX* __restrict__ src, int
 __host__ __device__ constexpr int role_c_hwc(int S) { return S == 7 ? 49 : (S == 14 ? 52 : S * S / 4); }
 __host__ __device__ constexpr int role_c_pitch(int S) { return S == 7 ? 49 : pitch4(role_c_hwc(S)); }
 
-template <int S, int R, typename TX>
+template <int S, int R, bool ANY, typename TX>
 __device__ __forceinline__ void sm_tile1_cta(const SmTile1Args& p, const int bid) {
-  constexpr bool kBulk = std::is_same<TX, float>::value;
+  constexpr bool kBulk = std::is_same<TX, float>::value && !ANY;
   constexpr bool kGram = (S == 7);                   // modes 3, 4 as Gram matrices A_m A_m^T (7 x 7)
   constexpr bool kGram14 = (S == 14);                // ... as 14 x 14 Gram matrices in four 7 x 7 blocks
   constexpr int HW = S * S;
@@ -957,7 +976,7 @@ __device__ __forceinline__ void sm_tile1_cta(const SmTile1Args& p, const int bid
       fac_issue_padded<R, kTT>(p.U_prev + p.u_off[2], U3s, S, p.r[2]);
       fac_issue_padded<R, kTT>(p.U_prev + p.u_off[3], U4s, S, p.r[3]);
     }
-    stage_tile_begin<TX>(A + (int64_t)tile * J, (int64_t)C * HW, Xs, B, J, PJ);
+    stage_tile_begin<ANY, TX>(A + (int64_t)tile * J, (int64_t)C * HW, Xs, B, J, PJ);
     fac_wait();
     __syncthreads();
     const int t = tid & (kNG - 1), wg = t >> 5;
@@ -1132,7 +1151,10 @@ __device__ __forceinline__ void sm_tile1_cta(const SmTile1Args& p, const int bid
       stage_block(&s_bar, reinterpret_cast<char*>(Xs), reinterpret_cast<const char*>(Xb), (uint32_t)C * HW * 4u,
                   p.stall_copy != 0);
     fac_issue_padded<R, kTT>(p.U_prev + p.u_off[1], U2s, C, p.r[1]);
-    if constexpr (kBulkC) {
+    if constexpr (ANY) {                             // one value at a time
+      for (int c = tid >> 5; c < C; c += kTT / 32)
+        for (int v = lane; v < HWC; v += 32) Xs[c * PC + v] = v < nval ? to_f(Xb[(int64_t)c * HW + v]) : 0.f;
+    } else if constexpr (kBulkC) {
     } else if constexpr (NQ == 1) {
       const int n4 = C * HW / 4;
       for (int idx = tid; idx < n4; idx += kTT) *reinterpret_cast<float4*>(Xs + 4 * idx) = ld4<TX>(Xb + 4 * idx);
@@ -1202,24 +1224,24 @@ __device__ __forceinline__ int batch_layer(const SmBatch<Args>& b, int bid) {
   return l;
 }
 
-template <int S, int R, typename TX>
+template <int S, int R, bool ANY, typename TX>
 __global__ void __launch_bounds__(kTT, 2) k_sm_tile1(const __grid_constant__ SmTile1Args p) {
-  sm_tile1_cta<S, R, TX>(p, (int)blockIdx.x);
+  sm_tile1_cta<S, R, ANY, TX>(p, (int)blockIdx.x);
 }
 template <int S, int R, typename TX>
 __global__ void __launch_bounds__(kTT, 2) k_sm_tile1_b(const __grid_constant__ SmBatch<SmTile1Args> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_tile1_cta<S, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_tile1_cta<S, R, false, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
-template <int KIND, int R, typename TX>
+template <int KIND, int R, bool ANY, typename TX>
 __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1(const __grid_constant__ SmPass1Args p) {
-  sm_pass1_cta<KIND, R, TX>(p, (int)blockIdx.x);
+  sm_pass1_cta<KIND, R, ANY, TX>(p, (int)blockIdx.x);
 }
 template <int KIND, int R, typename TX>
 __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1_b(const __grid_constant__ SmBatch<SmPass1Args> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_pass1_cta<KIND, R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_pass1_cta<KIND, R, false, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2077,7 +2099,8 @@ static int pass1_grid(const SmPass1Args& p) {
 
 template <int KIND, int R, typename TX>
 static cudaError_t launch_pass1_t(const SmPass1Args& p, size_t smem, cudaStream_t st) {
-  return launch_clustered(k_sm_pass1<KIND, R, TX>, pass1_grid(p), p.cl, smem, st, p);
+  return launch_clustered(p.aligned || !p.vec4 ? k_sm_pass1<KIND, R, false, TX> : k_sm_pass1<KIND, R, true, TX>, pass1_grid(p),
+                          p.cl, smem, st, p);
 }
 template <int R, typename TX>
 static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t st) {
@@ -2099,9 +2122,10 @@ static cudaError_t launch_wgrad_t(const SmWgradArgs& p, cudaStream_t st) {
 template <int S, int R, typename TX>
 static cudaError_t launch_tile1_t(const SmTile1Args& p, cudaStream_t st) {
   const size_t smem = sm_tile1_smem(S, R, p.B, p.C);
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_tile1<S, R, TX>), smem);
+  auto kernel = p.aligned ? k_sm_tile1<S, R, false, TX> : k_sm_tile1<S, R, true, TX>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  k_sm_tile1<S, R, TX><<<p.n_tiles_b + sm_tile1_role_c_ctas(S, p.B), kTT, smem, st>>>(p);
+  kernel<<<p.n_tiles_b + sm_tile1_role_c_ctas(S, p.B), kTT, smem, st>>>(p);
   return cudaGetLastError();
 }
 template <int S, int R, typename TX>

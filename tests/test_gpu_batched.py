@@ -146,3 +146,34 @@ def test_compress_layers_whose_workspaces_overlap_run_one_after_another():
         for r, (u, c) in zip(runs, want):
             assert torch.equal(r.U[r.cur], u) and torch.equal(r.core, c)
             r.cur = 1 - r.cur
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_layers_of_a_group_with_shifted_activations(bf16):
+    """Layers of one variant, two of which start at odd elements: they leave the shared launch, and every layer gives what
+    its separate call gives."""
+    from paper_2505_05086_b200.runner import StepRunner
+    specs = [LayerSpec("a", "conv", (8, 12 + 4 * i, 7, 7), 12, 3, 1, 1, 1, ranks=(3, 4, 3, 2)) for i in range(4)]
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    dtype = torch.bfloat16 if bf16 else torch.float32
+
+    def shifted(shape, k):
+        n = int(np.prod(shape))
+        return torch.randn(n + 8, generator=gen, device="cuda").to(dtype)[k:k + n].view(shape)
+
+    runs = [make_runner(L, bf16=bf16) for L in specs]
+    acts = [shifted(L.dims, k) for L, k in zip(specs, (0, 1, 0, 3))]
+    dys = [shifted(L.dy_shape, k) for L, k in zip(specs, (2, 0, 1, 0))]
+    want = []
+    for r, L, a, d in zip(runs, specs, acts, dys):
+        r.set_factors([np.linalg.qr(np.random.default_rng(3).standard_normal((n, k)))[0] for n, k in zip(L.dims, L.ranks)])
+        r.compress(a)
+        r.wgrad(d)
+        want.append((r.U[r.cur].clone(), r.core.clone(), r.dW.clone()))
+        r.cur = 1 - r.cur
+    step = StepRunner(runs)
+    step.compress(acts)
+    step.wgrad(dys)
+    torch.cuda.synchronize()
+    for r, w in zip(runs, want):
+        assert all(torch.equal(x, y) for x, y in zip((r.U[r.cur], r.core, r.dW), w))

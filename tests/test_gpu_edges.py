@@ -1,5 +1,6 @@
 """The kernels of the warm step at the edges of their tiles, element by element against the fp64 oracle."""
 import pytest
+import torch
 
 from asi_inputs.configs import LayerSpec
 from asi_inputs.generator import LayerStream
@@ -104,3 +105,51 @@ def test_long_contractions_of_few_tiles(dims, bf16):
     """Tiles shared by clusters of 8 and 2 CTAs, the last ones with an empty or a ragged share of the contraction."""
     ranks = (12, 14)
     _two_steps(LayerSpec("t", "linear", dims, 40, ranks=ranks), bf16, rho=(0.9, 0.9), tol=dict(TOL_F32, proj=1e-3))
+
+
+# Tensors that start at any element: (dims, ranks, cout, kernel, act shifted too).  Square maps with whole tiles, maps
+# with their samples over clusters, columns that come in whole groups of four and not, a weight gradient behind a large map
+SHIFTED = [
+    ((8, 32, 16, 16), (4, 8, 8, 8), 32, 3, True),
+    ((16, 16, 7, 7), (3, 4, 4, 4), 12, 3, True),
+    ((8, 12, 14, 14), (3, 4, 4, 4), 8, 1, True),
+    ((136, 20, 7, 7), (4, 4, 4, 4), 12, 3, True),
+    ((6, 3, 4, 5), (4, 3, 4, 4), 8, 3, True),
+    ((13, 33, 7, 7), (4, 4, 4, 3), 12, 3, True),
+    ((17, 40, 16, 16), (3, 8, 5, 8), 8, 3, True),
+    ((11, 64, 14, 14), (4, 4, 4, 4), 16, 3, True),
+    ((55, 9, 28, 28), (5, 2, 3, 4), 257, 3, False),
+    ((9, 12, 20, 24), (8, 5, 5, 5), 16, 3, False),
+    ((9, 13, 19, 23), (8, 5, 5, 5), 16, 3, True),
+]
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("case", SHIFTED)
+def test_tensors_that_start_at_any_element(case, bf16, shift):
+    dims, ranks, cout, k, act_too = case
+    L = LayerSpec("t", "conv", dims, cout, k, 1, k // 2, 1, ranks=ranks)
+    st = LayerStream(dims=L.dims, ranks=L.ranks, dy_shape=L.dy_shape, seed=sum(L.dims) + L.cout, bf16=bf16,
+                     rho=tuple(_rho(r) for r in L.ranks),
+                     gen_ranks=tuple(min(d, max(2 * r, r + 2, 4)) for d, r in zip(L.dims, L.ranks)))
+    run = make_runner(L, bf16=bf16)
+    to_device = run.to_device
+
+    def shifted(x):
+        t = to_device(x)
+        if x.shape == tuple(L.dims) and not act_too:
+            return t
+        buf = torch.full((t.numel() + 8,), float("nan"), dtype=t.dtype, device=t.device)
+        view = buf[shift:shift + t.numel()].view(t.shape)
+        view.copy_(t)
+        assert view.data_ptr() % 16 == shift * t.element_size()
+        return view
+
+    run.to_device = shifted
+    A, dY = st.next()
+    err, _ = compare_step(run, L, A, dY, st.u_prev0())
+    check(err, TOL_F32, f"{dims} {ranks} bf16={bf16} shift={shift}")
+    with pytest.raises(Exception, match="invalid argument"):      # half an element is refused, not read
+        run.plan.wgrad(run.core.data_ptr(), run.U[run.cur].data_ptr(), to_device(dY).data_ptr() + 1, run.dW.data_ptr(),
+                       run.ws_w.data_ptr(), run.ws_w.numel())
