@@ -65,7 +65,7 @@ void choose_kernels(asi_plan* pl) {
     SmCoreArgs c;
     build_fused_pass1(pl, nullptr, nullptr, nullptr, &a);
     build_fused_core(pl, nullptr, nullptr, nullptr, nullptr, true, &c);
-    pl->fast_compress = sm_pass1_smem(a, pl->fast_kind, R) <= kSmemLimit && sm_core_smem(c, R) <= kSmemLimit;
+    pl->fast_compress = sm_pass1_smem(a, pl->fast_kind, R) <= kSmemLimit && sm_core_smem(c, R, pl->bf16) <= kSmemLimit;
   }
   if (B <= 4096 && H <= 64 && W <= 64) {
     const int Cout = pl->d.cout;
@@ -87,20 +87,20 @@ void choose_kernels(asi_plan* pl) {
     // (one at a time, too, where two would keep the CTA from sharing its SM with three others)
     a.nbuf = 2;
     a.ncl = cpb >= 2 ? cpb / 2 : 1;
-    if (sm_wgrad_smem(a, R) > 56 * 1024) a.ncl = 1;
+    if (sm_wgrad_smem(a, R, false, pl->bf16) > 56 * 1024) a.ncl = 1;
     // one staging block where two keep a fourth CTA off the SM (ResNet-18 tail at 64: 512 CTAs, three an SM took 29.8 us,
     // four take 24.9)
-    if (sm_wgrad_smem(a, R) > 56 * 1024) {
+    if (sm_wgrad_smem(a, R, false, pl->bf16) > 56 * 1024) {
       a.nbuf = 1;
-      if (sm_wgrad_smem(a, R) > 56 * 1024) a.nbuf = 2;
+      if (sm_wgrad_smem(a, R, false, pl->bf16) > 56 * 1024) a.nbuf = 2;
     }
     // 256 threads where three such CTAs share an SM and the stream of dY is short (at 128 x 784 values a CTA 512
     // threads take 28 us against 36; at 128 x 196, 256 take 39 us against 46), else 512.  A CTA that needs an SM for itself pays on
     // small maps only: larger ones recompute Z3 in every CTA, and four launches are faster (28 x 28, B = 128, seven
     // layers: 118 us here against 28 us a layer beside other work)
-    const size_t need = sm_wgrad_smem(a, R);
+    const size_t need = sm_wgrad_smem(a, R, false, pl->bf16);
     if (need > 75 * 1024 || B * cpb * HoWo > 32768) a.nt = 512;
-    if (a.nt == 512 && sm_wgrad_smem(a, R) > kSmemLimit) a.nt = 256;
+    if (a.nt == 512 && sm_wgrad_smem(a, R, false, pl->bf16) > kSmemLimit) a.nt = 256;
     if (need <= 113 * 1024 || (need <= kSmemLimit && H * W <= 256)) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
@@ -439,6 +439,7 @@ void build_fused_core(const asi_plan* pl, const void* act, float* U_new, float* 
   c->tile_c = pl->core_tile_c;
   c->n_tiles = pl->n_tiles_core;
   c->vec4 = (pl->fast_vec4 && (pl->core_tile_c * c->H * c->W) % 4 == 0 && four_aligned(pl, act)) ? 1 : 0;
+  c->staged = 0;
 }
 
 void build_fused_wgrad(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, char* w,
@@ -551,7 +552,7 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
 
 // Orthogonalize, then core = A x_1 U_1^T ... x_n U_n^T (Algorithm 1, core update with U^T).
 asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, float* core,
-                             char* w, const float* gram_U_prev, bool tc_ready, cudaStream_t st) {
+                             char* w, const float* gram_U_prev, bool tc_ready, int beside, cudaStream_t st) {
   // the first core product runs on the tensor cores when its mode does: after a warm step the operand's zero columns
   // are there from the split of U_prev and Orthogonalize fills in the rest, a cold start splits U_new here
   const int m0 = pl->core_order[0];
@@ -568,7 +569,7 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
   if (pl->fast_compress) {
     SmCoreArgs c;
     build_fused_core(pl, act, U_new, core, w, gram_U_prev != nullptr, &c);
-    ASI_CUDA(launch_sm_core(c, pl->fast_R, pl->bf16, st));
+    ASI_CUDA(launch_sm_core(c, pl->fast_R, pl->bf16, beside, st));
     return ASI_OK;
   }
   int64_t cd[ASI_MAX_MODES];
@@ -926,8 +927,9 @@ int32_t asi_launch_count(const asi_plan_t* pl, int32_t which) {
   return which == 0 ? pl->launches_compress : pl->launches_wgrad;
 }
 
-asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_prev, float* U_new,
-                          float* core, void* ws, size_t ws_bytes, void* stream) {
+// beside: CTAs of the fused layers that a batched call runs next to this one (a choice of kernels, not of results)
+static asi_status_t compress_one(const asi_plan* pl, const void* act, const float* U_prev, float* U_new, float* core, void* ws,
+                                 size_t ws_bytes, int beside, void* stream) {
   if (!pl || !valid_ptr(act) || !valid_ptr(U_prev) || !valid_ptr(U_new) || !valid_ptr(core))
     return ASI_ERR_INVALID_ARG;
   if (U_prev == U_new) return ASI_ERR_INVALID_ARG;
@@ -946,7 +948,7 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
       build_fused_pass1(pl, act, U_prev, w, &a);
       ASI_CUDA(launch_sm_pass1(a, pl->fast_kind, pl->fast_R, pl->bf16, st));
     }
-    return finish_compress(pl, act, U_new, core, w, U_prev, false, st);
+    return finish_compress(pl, act, U_new, core, w, U_prev, false, beside, st);
   }
   // The first kernel on the caller's stream clears the status block and starts only when the stream's earlier work
   // is done; the mode passes behind it do not depend on one another and are launched as programmatic dependents
@@ -1045,7 +1047,12 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
     ASI_CUDA(launch_tc_group(proj, sp.n, status, true, st));
     ASI_CUDA(launch_tc_group(expd, sp.n, status, true, st));
   }
-  return finish_compress(pl, act, U_new, core, w, nullptr, sp.n > 0, st);
+  return finish_compress(pl, act, U_new, core, w, nullptr, sp.n > 0, beside, st);
+}
+
+asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_prev, float* U_new,
+                          float* core, void* ws, size_t ws_bytes, void* stream) {
+  return compress_one(pl, act, U_prev, U_new, core, ws, ws_bytes, 0, stream);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1102,11 +1109,18 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     for (int j : grp) done[j] = 1;
     chains.push_back(std::move(grp));
   }
+  auto of = [&](int c) {                             // CTAs of a chain's core kernel
+    int t = 0;
+    for (int j : chains[c]) t += plans[j]->fast_compress ? plans[j]->n_tiles_core : 0;
+    return t;
+  };
+  int all = 0;
+  for (int c = 0; c < (int)chains.size() && apart; ++c) all += of(c);
   return run_chains((int)chains.size(), apart, static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
     const std::vector<int>& grp = chains[c];
     const int g = (int)grp.size(), i0 = grp[0];
     if (g == 1)
-      return asi_compress(plans[i0], acts[i0], U_prev[i0], U_new[i0], cores[i0], ws[i0], ws_bytes[i0], st);
+      return compress_one(plans[i0], acts[i0], U_prev[i0], U_new[i0], cores[i0], ws[i0], ws_bytes[i0], all - of(c), st);
     const asi_plan* p0 = plans[i0];
     std::vector<SmPass1Args> pa(p0->tile_S ? 0 : g);
     std::vector<SmTile1Args> ta(p0->tile_S ? g : 0);
@@ -1124,10 +1138,13 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     if (p0->tile_S) ASI_CUDA(launch_sm_tile1_batched(ta.data(), g, p0->tile_S, p0->fast_R, p0->bf16, st));
     else ASI_CUDA(launch_sm_pass1_batched(pa.data(), g, p0->fast_kind, p0->fast_R, p0->bf16, st));
     ASI_CUDA(launch_sm_reduce_batched(ra.data(), mc.data(), g, st));
-    ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_R, p0->bf16, st));
+    ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_R, p0->bf16, all - of(c), st));
     return ASI_OK;
   });
 }
+
+static asi_status_t conv_wgrad_one(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, void* ws,
+                                   size_t ws_bytes, int beside, void* stream);
 
 asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* const* cores, const float* const* U,
                                const void* const* dY, float* const* dW, void* const* ws, const size_t* ws_bytes,
@@ -1159,19 +1176,26 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     for (int j : grp) done[j] = 1;
     chains.push_back(std::move(grp));
   }
+  auto of = [&](int c) {                             // CTAs of a chain's fused kernel
+    int t = 0;
+    for (int j : chains[c]) t += plans[j]->fast_wgrad ? plans[j]->d.cout / plans[j]->cpb : 0;
+    return t;
+  };
+  int all = 0;
+  for (int c = 0; c < (int)chains.size() && apart; ++c) all += of(c);
   return run_chains((int)chains.size(), apart, static_cast<cudaStream_t>(stream), [&](int c, cudaStream_t st) -> asi_status_t {
     const std::vector<int>& grp = chains[c];
     const int g = (int)grp.size(), i0 = grp[0];
     const asi_plan* p0 = plans[i0];
     if (g == 1)
-      return p0->d.kind == ASI_CONV2D ? asi_conv_wgrad(p0, cores[i0], U[i0], dY[i0], dW[i0], ws[i0], ws_bytes[i0], st)
+      return p0->d.kind == ASI_CONV2D ? conv_wgrad_one(p0, cores[i0], U[i0], dY[i0], dW[i0], ws[i0], ws_bytes[i0], all - of(c), st)
                                       : asi_linear_wgrad(p0, cores[i0], U[i0], dY[i0], dW[i0], ws[i0], ws_bytes[i0], st);
     std::vector<SmWgradArgs> wa(g);
     for (int k = 0; k < g; ++k) {
       const int j = grp[k];
       build_fused_wgrad(plans[j], cores[j], U[j], dY[j], dW[j], static_cast<char*>(ws[j]), &wa[k]);
     }
-    ASI_CUDA(launch_sm_wgrad_batched(wa.data(), g, p0->fast_R, p0->bf16, st));
+    ASI_CUDA(launch_sm_wgrad_batched(wa.data(), g, p0->fast_R, p0->bf16, all - of(c), st));
     return ASI_OK;
   });
 }
@@ -1229,7 +1253,7 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
   }
   s = expand_modes(pl, act, om, w, true, st);
   if (s != ASI_OK) return s;
-  return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
+  return finish_compress(pl, act, U_new, core, w, nullptr, false, 0, st);
 }
 
 static size_t omega_scratch_bytes(const asi_plan* pl) {
@@ -1263,7 +1287,7 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
   ASI_CUDA(launch_fill_gaussian(seed, f, pl->nd, st));
   s = expand_modes(pl, act, f.out, w, false, st);
   if (s != ASI_OK) return s;
-  return finish_compress(pl, act, U_new, core, w, nullptr, false, st);
+  return finish_compress(pl, act, U_new, core, w, nullptr, false, 0, st);
 }
 
 asi_status_t asi_gaussian_stream(uint64_t seed, uint32_t stream_id, int64_t n, float* out, void* stream) {
@@ -1284,8 +1308,8 @@ asi_status_t asi_philox_words(uint64_t seed, uint32_t stream_id, int64_t n_group
   return ASI_OK;
 }
 
-asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float* U, const void* dY,
-                            float* dW, void* ws, size_t ws_bytes, void* stream) {
+static asi_status_t conv_wgrad_one(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, void* ws,
+                                   size_t ws_bytes, int beside, void* stream) {
   if (!pl || !valid_ptr(core) || !valid_ptr(U) || !valid_ptr(dY) || !valid_ptr(dW))
     return ASI_ERR_INVALID_ARG;
   if (pl->d.kind != ASI_CONV2D || !element_aligned(pl, dY)) return ASI_ERR_INVALID_ARG;
@@ -1296,7 +1320,7 @@ asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float
   if (pl->fast_wgrad) {
     SmWgradArgs g;
     build_fused_wgrad(pl, core, U, dY, dW, w, &g);
-    ASI_CUDA(launch_sm_wgrad(g, pl->fast_R, pl->bf16, st));
+    ASI_CUDA(launch_sm_wgrad(g, pl->fast_R, pl->bf16, beside, st));
     return ASI_OK;
   }
   float* Z1 = reinterpret_cast<float*>(w + pl->off_Z[0]);
@@ -1326,6 +1350,11 @@ asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float
   else
     ASI_CUDA(launch_conv_tail(t, st));
   return ASI_OK;
+}
+
+asi_status_t asi_conv_wgrad(const asi_plan_t* pl, const float* core, const float* U, const void* dY,
+                            float* dW, void* ws, size_t ws_bytes, void* stream) {
+  return conv_wgrad_one(pl, core, U, dY, dW, ws, ws_bytes, 0, stream);
 }
 
 asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const float* U, const void* dY,

@@ -173,6 +173,7 @@ struct SmCoreArgs {
   int r[ASI_MAX_MODES];
   int B, C, H, W, tile_c, n_tiles;   // tile_c: channels per tile
   int vec4;                     // columns may be read four at a time (whole groups, aligned)
+  int staged;                   // the tile whole in shared memory (set by the launcher)
 };
 struct SmWgradArgs {
   const float* core;
@@ -199,8 +200,8 @@ void sm_pass1_split(int HW, int C, int B, int* cs, int* cc);
 int sm_pass1_off_u2(int R, int cc, int pitch);
 int sm_pass1_tiles_b(int64_t chw, bool vec4);
 int sm_core_tile_c(int HW, int C);
-size_t sm_core_smem(const SmCoreArgs& p, int R);
-size_t sm_wgrad_smem(const SmWgradArgs& p, int R);
+size_t sm_core_smem(const SmCoreArgs& p, int R, bool bf16);
+size_t sm_wgrad_smem(const SmWgradArgs& p, int R, bool staged, bool bf16);
 cudaError_t launch_sm_pass1(const SmPass1Args& p, int kind, int R, bool bf16, cudaStream_t st);
 // Tensor-core products of bf16 tensors (asi_tc_kernels.cu).  A factor enters as its stacked operand (three bf16 terms).
 size_t tc_operand_bytes(int64_t K, int n);
@@ -231,14 +232,14 @@ struct TcCall {
 };
 cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st);
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st);
-cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, cudaStream_t st);
-cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, int beside, cudaStream_t st);
+cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, int beside, cudaStream_t st);
 // the same kernels over several layers of one variant in one launch each (n <= sm_max_batch())
 int sm_max_batch();
 cudaError_t launch_sm_pass1_batched(const SmPass1Args* a, int n, int kind, int R, bool bf16, cudaStream_t st);
 cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunks, int n, cudaStream_t st);
-cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, cudaStream_t st);
-cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, cudaStream_t st);
+cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, int beside, cudaStream_t st);
+cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, int beside, cudaStream_t st);
 
 // Benchmark timing aid (asi_profile_begin / asi_profile_end).
 struct ProfState {

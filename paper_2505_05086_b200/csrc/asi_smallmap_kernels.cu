@@ -1425,12 +1425,68 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
 //     Cholesky factor the reduction kernel left -- all of U_1, the tile's own rows of U_2, all of U_3 and U_4 -- and
 //     the owners write them to U_new; the first samples of the tile are already on their way;
 //   W[c,h,w][i] = sum_b U1[b,i] X[b][c,h,w] straight from memory in registers (the activation is in L2 or streams
-//     from HBM; nothing is staged, so several CTAs share an SM);
+//     from HBM; nothing is staged, so several CTAs share an SM), or, in launches of few CTAs, from a tile in shared
+//     memory (choose_core);
 //   M[c][i,k,l] = W x_3 U3^T x_4 U4^T per channel -- the spatial modes before the channel mode: r1 r3 (W + r4) short
 //     sums per channel instead of r1 r2 HW, and r1 r3 r4 numbers leave a channel instead of a whole core;
 //   core[i,j,k,l] = sum_c U2[c,j] M[c][i,k,l] by the last CTA of every group of tiles, then over the groups by the last
 //     group, both in index order.
 // ---------------------------------------------------------------------------------------------
+// ---- A tile [B x J] (J a multiple of four) whole in shared memory: k_sm_core and k_sm_wgrad where a launch has few CTAs.
+// Every value is requested before there is anything to wait for, by 512 threads; the streamed forms of the same sums
+// hold eight samples a thread, so that four CTAs share an SM.  The bits are the same: sample b goes to share b mod NH, and
+// the shares meet in order.
+template <typename TX>
+__host__ __device__ constexpr int tile_pitch(int J) { return sizeof(TX) == 4 ? J + 4 : J + 8; }   // rows stay 16 (bf16: 8) byte aligned
+template <typename TX>
+__host__ __device__ constexpr size_t tile_floats(int B, int J) { return ((size_t)B * tile_pitch<TX>(J) * sizeof(TX) + 3) / 4; }
+template <typename TX>
+__device__ __forceinline__ void tile_issue(const TX* __restrict__ A, int64_t sstride, int B, int J, int jvalid, TX* __restrict__ Xs) {
+  const int JV = J / 4, PJ = tile_pitch<TX>(J);
+  const FDiv dJ(JV);
+  int b, q, sb, sq;
+  dJ.divmod((int)threadIdx.x, b, q);
+  dJ.divmod(kTT, sb, sq);
+  while (b < B) {
+    if (4 * q < jvalid) {
+      const TX* src = A + (int64_t)b * sstride + 4 * q;
+      if constexpr (sizeof(TX) == 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(Xs + b * PJ + 4 * q)), "l"(src) : "memory");
+      else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(Xs + b * PJ + 4 * q)), "l"(src) : "memory");
+    }
+    b += sb;
+    q += sq;
+    if (q >= JV) { q -= JV; ++b; }
+  }
+}
+// acc[c][j / 2] = sum over the samples b == h (mod NH) of X[b][4 jq + c] (U1[b][j], U1[b][j + 1])
+template <int R, typename TX>
+__device__ __forceinline__ void tile_project(const TX* Xs, int B, int PJ, int NH, int h, int jq, const float* __restrict__ U1s,
+                                             f2 (&acc)[4][R / 2]) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j) acc[c][j] = 0ull;
+  const TX* src = Xs + 4 * jq;
+#pragma unroll 4
+  for (int b = h; b < B; b += NH) {
+    const float4 x = ld4<TX>(src + b * PJ);
+    const float xs[4] = {x.x, x.y, x.z, x.w};
+    const float* u = U1s + b * R;
+#pragma unroll
+    for (int j = 0; j < R / 2; j += 2) {
+      const ulonglong2 uj = *reinterpret_cast<const ulonglong2*>(u + 2 * j);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const f2 xc = pack2(xs[c], xs[c]);
+        ffma2(acc[c][j], xc, uj.x);
+        ffma2(acc[c][j + 1], xc, uj.y);
+      }
+    }
+  }
+}
+
 // W[col][:] = sum_b X[b][col] U1[b][:] for the tile's J columns (jvalid of them exist): thread = VW neighbouring columns
 // and the samples b == h (mod NH), eight in flight, the NH shares meet in order.  The first eight are requested before
 // `factors` (the row solves, which end with a barrier) runs.  Shares are stored by rank, columns side by side: stored by
@@ -1511,7 +1567,40 @@ __device__ __forceinline__ void core_project(const TX* __restrict__ A, int64_t c
 }
 
 template <int R, typename TX>
+__device__ __forceinline__ void core_project_staged(const TX* Xs, int B, int J, int jvalid, const float* __restrict__ U1s,
+                                                    float* part, float* __restrict__ Ws) {
+  const int tid = threadIdx.x, JV = J / 4, NH = kPT / JV;
+  const FDiv dJ(JV);
+  int h, jq;
+  dJ.divmod(tid, h, jq);
+  const bool on = h < NH && 4 * jq < jvalid;
+  f2 acc[4][R / 2];
+  if (on) tile_project<R>(Xs, B, tile_pitch<TX>(J), NH, h, jq, U1s, acc);
+  __syncthreads();                                   // the tile has been read: the shares go over it
+  if (on) {
+    float* dst = part + h * J * R + 4 * jq;
+#pragma unroll
+    for (int j = 0; j < R; j += 2) {
+      float2 v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = unpack2(acc[c][j / 2]);
+      *reinterpret_cast<float4*>(dst + j * J) = make_float4(v[0].x, v[1].x, v[2].x, v[3].x);
+      *reinterpret_cast<float4*>(dst + (j + 1) * J) = make_float4(v[0].y, v[1].y, v[2].y, v[3].y);
+    }
+  }
+  __syncthreads();
+  for (int idx = tid; idx < J * R; idx += kTT) {
+    float s = part[idx];
+#pragma unroll 4
+    for (int q = 1; q < NH; ++q) s += part[q * J * R + idx];
+    Ws[idx] = s;
+  }
+  __syncthreads();
+}
+
+template <int R, bool STAGED, typename TX>
 __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) {
+  constexpr int NT = STAGED ? kTT : kPT;
   extern __shared__ __align__(128) float smem[];
   __shared__ int s_last;
   __shared__ double Rs[4][kRfStride];   // per mode: rows of R_m (pitch 8), then 1 / diag(R_m) at [64..]
@@ -1531,7 +1620,7 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
     const int nrows = B + ncl + H + W;
     bool synced = false;
 #pragma unroll 1
-    for (int row = tid; row < nrows || !synced; row += kPT) {
+    for (int row = tid; row < nrows || !synced; row += NT) {
       int m = 0, k = row;
       float* rdst = U1s + k * R;
       bool owner = tile == 0;
@@ -1544,7 +1633,7 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
 #pragma unroll
       for (int j = 0; j < R; ++j) q[j] = (on && j < rr) ? __ldcg(p.Pred[m] + (int64_t)k * rr + j) : 0.0;
       if (!synced) {                    // the Cholesky factors of the four modes travel with the first rows
-        for (int e = tid; e < 4 * kRfStride; e += kPT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
+        for (int e = tid; e < 4 * kRfStride; e += NT) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
         __syncthreads();
         synced = true;
       }
@@ -1568,11 +1657,18 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   };
   const TX* A = reinterpret_cast<const TX*>(p.act) + (int64_t)c0 * HW;
   const int64_t chw = (int64_t)C * HW;
-  if (p.vec4) core_project<R, 4, TX>(A, chw, B, J, jvalid, U1s, part, Ws, factors);
+  if constexpr (STAGED) {
+    TX* Xs = reinterpret_cast<TX*>(part);
+    tile_issue(A, chw, B, J, jvalid, Xs);
+    factors();
+    fac_wait();
+    __syncthreads();
+    core_project_staged<R>(Xs, B, J, jvalid, U1s, part, Ws);
+  } else if (p.vec4) core_project<R, 4, TX>(A, chw, B, J, jvalid, U1s, part, Ws, factors);
   else core_project<R, 1, TX>(A, chw, B, J, jvalid, U1s, part, Ws, factors);
   // T1[cl,i][k][w] = sum_h W[cl,h,w][i] U3[h][k]
   const FDiv dW(W), d_r1(r1), d_r3(r3), d_r4(r4);
-  for (int idx = tid; idx < ncl * r1 * r3 * W; idx += kPT) {
+  for (int idx = tid; idx < ncl * r1 * r3 * W; idx += NT) {
     int t, w, ci, k, cl, i;
     dW.divmod(idx, t, w);
     d_r3.divmod(t, ci, k);
@@ -1586,7 +1682,7 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   __syncthreads();
   // M[c][i,k,l] = sum_w T1[cl,i][k][w] U4[w][l]
   const int ce3 = r1 * r3 * r4;
-  for (int idx = tid; idx < ncl * ce3; idx += kPT) {
+  for (int idx = tid; idx < ncl * ce3; idx += NT) {
     int t, l;
     d_r4.divmod(idx, t, l);
     const float* ts = T1 + t * W;
@@ -1608,13 +1704,13 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   {
     const int ch0 = gfirst * CC, nch = ((gfirst + gsize) * CC < C ? (gfirst + gsize) * CC : C) - ch0;
     float* u2 = part;                   // [nch][R] (gs CC R floats: fits, checked by the host)
-    for (int e = tid; e < nch * R; e += kPT) {
+    for (int e = tid; e < nch * R; e += NT) {
       const int c = e / R, j = e % R;
       u2[e] = j < r2 ? __ldcg(p.U_new + p.u_off[1] + (int64_t)(ch0 + c) * r2 + j) : 0.f;
     }
     __syncthreads();
     // thread = one (i, k, l), all j: the channels' numbers are read once, 16 in flight
-    for (int e = tid; e < ce3; e += kPT) {
+    for (int e = tid; e < ce3; e += NT) {
       float s[R];
 #pragma unroll
       for (int j = 0; j < R; ++j) s[j] = 0.f;
@@ -1647,28 +1743,28 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
   // few core elements: thread (e, q) sums the groups == q (mod nq) of element e, the nq sums meet in index order
   if (ce > kPT && ngroups <= 8) {       // a wide core from few groups: four elements x eight groups in flight
 #pragma unroll 1
-    for (int e0 = tid; e0 < ce; e0 += 4 * kPT) {
+    for (int e0 = tid; e0 < ce; e0 += 4 * NT) {
       float v[4][8];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          v[u][k] = __ldcg(p.Tg + (int64_t)(k < ngroups ? k : 0) * ce + (e0 + u * kPT < ce ? e0 + u * kPT : e0));
+          v[u][k] = __ldcg(p.Tg + (int64_t)(k < ngroups ? k : 0) * ce + (e0 + u * NT < ce ? e0 + u * NT : e0));
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         float s = v[u][0];
 #pragma unroll
         for (int k = 1; k < 8; ++k) s += k < ngroups ? v[u][k] : 0.f;
-        if (e0 + u * kPT < ce) p.core[e0 + u * kPT] = s;
+        if (e0 + u * NT < ce) p.core[e0 + u * NT] = s;
       }
     }
     if (tid == 0) *p.counter = 0;
     return;
   }
-  int nq = kPT / ce;
+  int nq = kPT / ce;                   // (the order of these sums does not depend on NT)
   nq = nq > 8 ? 8 : (nq < 1 ? 1 : nq);
   float* fold = part;                   // [nq][ce]
-  for (int it = tid; it < nq * ce; it += kPT) {
+  for (int it = tid; it < nq * ce; it += NT) {
     const int q = it / ce, e = it - q * ce;
     const float* src = p.Tg + e;
     float s = 0.f;
@@ -1696,19 +1792,29 @@ __device__ __forceinline__ void sm_core_cta(const SmCoreArgs& p, const int bid) 
 
 template <int R, typename TX>
 __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 3) k_sm_core(const __grid_constant__ SmCoreArgs p) {
-  sm_core_cta<R, TX>(p, (int)blockIdx.x);
+  sm_core_cta<R, false, TX>(p, (int)blockIdx.x);
 }
 template <int R, typename TX>
 __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 3) k_sm_core_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_core_cta<R, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_core_cta<R, false, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+}
+template <int R, typename TX>
+__global__ void __launch_bounds__(kTT, 2) k_sm_core_staged(const __grid_constant__ SmCoreArgs p) {
+  sm_core_cta<R, true, TX>(p, (int)blockIdx.x);
+}
+template <int R, typename TX>
+__global__ void __launch_bounds__(kTT, 2) k_sm_core_staged_b(const __grid_constant__ SmBatch<SmCoreArgs> b) {
+  const int l = batch_layer(b, (int)blockIdx.x);
+  sm_core_cta<R, true, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
 // k_sm_wgrad: CTA owns cpb consecutive output channels, i.e. the dY tile [B x J], J = cpb*Ho*Wo
 // contiguous values per sample.
 //   Z1 = dY x_1 U1^T on the CTA's channels, straight from memory in registers (no staged tile: 100 KB less shared
-//     memory, so two CTAs share an SM and the set-up of one hides behind the stream of the other);
+//     memory, so two CTAs share an SM and the set-up of one hides behind the stream of the other), or, in launches of at
+//     most a CTA an SM, from a staged tile with Z3 formed while it is on its way (wgrad_staged);
 //   Z3 = core x_3 U3 x_4 U4 (recomputed per CTA);
 //   Z4[c',j,kh,kw] = sum_{i,h',w'} Z1[i,c',h',w'] Z3pad[i,j,h's+kh-p,w's+kw-p];  dW = Z4 x_2 U2.
 // ---------------------------------------------------------------------------------------------
@@ -1869,7 +1975,7 @@ __device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t
   }
 }
 
-template <int R, int kNT, typename TX>
+template <int R, int kNT, bool STAGED, typename TX>
 __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
@@ -1879,10 +1985,14 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
   const int c0 = bid * p.cpb;
   // staging blocks of term 5 reuse the tile's space: ncl channels per round, nbuf of them when rounds follow
   const int n_stage = (p.cpb > p.ncl ? p.nbuf : 1) * p.ncl * (p.C / p.groups) * kk;
-  const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV, kNT);
+  const int nt = STAGED ? p.nt : kNT;                // the thread count that the sums are split by
+  const int VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW, NH = wgrad_groups(JV, nt);
+  const int n_tile = STAGED ? (int)tile_floats<TX>(p.B, J) : 0;
   float* stage = smem;                               // term 5's blocks; before that the shares of Z1 [NH][J][R]
-  float* part = smem;
-  float* U1s = smem + ((NH * J * R > n_stage ? NH * J * R : n_stage) + 3) / 4 * 4;   // [B][R]
+  float* part = smem;                                // (and before these the tile of dY)
+  int n_head = NH * J * R > n_stage ? NH * J * R : n_stage;
+  if (n_tile > n_head) n_head = n_tile;
+  float* U1s = smem + (n_head + 3) / 4 * 4;          // [B][R]
   float* U2s = U1s + p.B * R;                        // [C][R]
   float* Z1s = U2s + p.C * R;                        // [J][R]
   float* Ss = Z1s + J * R;                           // [r1 r2][R (l)][R (k)]: core, modes 3 and 4 swapped, zero-padded
@@ -1907,7 +2017,12 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
     fac_issue_padded<R, kNT>(p.U + p.u_off[3], U4s, W, r4);
     fac_issue_padded<R, kNT>(p.U + p.u_off[0], U1s, p.B, r1);
     fac_issue_padded<R, kNT>(p.U + p.u_off[1], U2s, p.C, r2);
-    if (p.vec4) wgrad_project<R, 4, kNT, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
+    if constexpr (STAGED) {                          // Z3 is formed while the tile is on its way
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      tile_issue(dY, sstride, p.B, J, J, reinterpret_cast<TX*>(smem));
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+      __syncthreads();
+    } else if (p.vec4) wgrad_project<R, 4, kNT, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
     else wgrad_project<R, 1, kNT, TX>(dY, sstride, p.B, J, NH, U1s, part, Z1s);
   }
   // terms 2-3: Tm[ij][h][l] = sum_k S[ij][k][l] U3[h][k];  Z3[ij][h][w] = sum_l Tm[ij][h][l] U4[w][l]
@@ -1945,11 +2060,36 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
     }
     Z3s[idx] = s;
   }
+  if constexpr (STAGED) {
+    fac_wait();
+    __syncthreads();
+    const FDiv dJ(JV);
+    int h, jq;
+    dJ.divmod(tid, h, jq);
+    const bool on = h < NH;
+    f2 acc[4][R / 2];
+    if (on) tile_project<R>(reinterpret_cast<const TX*>(smem), p.B, tile_pitch<TX>(J), NH, h, jq, U1s, acc);
+    __syncthreads();                                 // the tile has been read: the shares go over it
+    if (on)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int j = 0; j < R; j += 4) {
+          const float2 a = unpack2(acc[c][j / 2]), b = unpack2(acc[c][j / 2 + 1]);
+          *reinterpret_cast<float4*>(part + (h * J + 4 * jq + c) * R + j) = make_float4(a.x, a.y, b.x, b.y);
+        }
+    __syncthreads();
+    for (int idx = tid; idx < J * R; idx += kNT) {
+      float s = part[idx];
+      for (int q = 1; q < NH; ++q) s += part[q * J * R + idx];
+      Z1s[idx] = s;
+    }
+  }
   __syncthreads();
   // term 4: thread (n, g): outputs n = (j, kh, kw) of all cpb channels and every G-th pair (i, h') of
   // the reduction; one Z3 operand feeds cpb FMAs.  The G partial sums meet in order.
   const int N4 = r2 * kk;
-  int G4 = (N4 <= kNT) ? kNT / N4 : 1;
+  int G4 = (N4 <= nt) ? nt / N4 : 1;
   if (G4 > r1 * p.Ho) G4 = r1 * p.Ho;
   const FDiv d_Ho(p.Ho), d_N4(N4);
   for (int it = tid; it < N4 * G4; it += kNT) {
@@ -1993,12 +2133,21 @@ __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid
 
 template <int R, int NT, typename TX>
 __global__ void __launch_bounds__(NT, (R == 4 ? 1024 : 512) / NT) k_sm_wgrad(const __grid_constant__ SmWgradArgs p) {
-  sm_wgrad_cta<R, NT, TX>(p, (int)blockIdx.x);
+  sm_wgrad_cta<R, NT, false, TX>(p, (int)blockIdx.x);
 }
 template <int R, int NT, typename TX>
 __global__ void __launch_bounds__(NT, (R == 4 ? 1024 : 512) / NT) k_sm_wgrad_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_wgrad_cta<R, NT, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+  sm_wgrad_cta<R, NT, false, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
+}
+template <int R, typename TX>
+__global__ void __launch_bounds__(kTT, R == 4 ? 2 : 1) k_sm_wgrad_staged(const __grid_constant__ SmWgradArgs p) {
+  sm_wgrad_cta<R, kTT, true, TX>(p, (int)blockIdx.x);
+}
+template <int R, typename TX>
+__global__ void __launch_bounds__(kTT, R == 4 ? 2 : 1) k_sm_wgrad_staged_b(const __grid_constant__ SmBatch<SmWgradArgs> b) {
+  const int l = batch_layer(b, (int)blockIdx.x);
+  sm_wgrad_cta<R, kTT, true, TX>(b.a[l], (int)blockIdx.x - b.first[l]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2051,23 +2200,28 @@ int sm_core_tile_c(int HW, int C) {
   if (HW % 4 != 0 && cc >= 4) cc = cc / 4 * 4;
   return cc < C ? cc : C;
 }
-size_t sm_core_smem(const SmCoreArgs& p, int R) {
+size_t sm_core_smem(const SmCoreArgs& p, int R, bool bf16) {
   const int HW = p.H * p.W, J = p.tile_c * HW, VW = p.vec4 ? 4 : 1, JV = (J + VW - 1) / VW;
   size_t part = (size_t)(kPT / JV) * J * R;
   const size_t t1 = (size_t)p.tile_c * p.r[0] * p.r[2] * p.W, u2 = (size_t)p.gs * p.tile_c * R;
+  const size_t tile = p.staged ? (bf16 ? tile_floats<__nv_bfloat16>(p.B, J) : tile_floats<float>(p.B, J)) : 0;
   if (t1 > part) part = t1;
   if (u2 > part) part = u2;
+  if (tile > part) part = tile;
   if (part < 8 * kPT) part = 8 * kPT;                // the final fold
   return 4 * ((size_t)((p.B * R + 3) & ~3) + (size_t)(p.H + p.W) * R + (size_t)J * R + part);
 }
 
-size_t sm_wgrad_smem(const SmWgradArgs& p, int R) {
+size_t sm_wgrad_smem(const SmWgradArgs& p, int R, bool staged, bool bf16) {
   const int r1 = p.r[0], r2 = p.r[1];
   const int J = p.cpb * p.Ho * p.Wo, kk = p.kh * p.kw, JV = p.vec4 ? J / 4 : J;
   const int N4 = r2 * kk;
   const size_t part = (size_t)wgrad_groups(JV, p.nt) * J * R,
                stage = (size_t)(p.cpb > p.ncl ? p.nbuf : 1) * p.ncl * (p.C / p.groups) * kk;
-  size_t n = ((part > stage ? part : stage) + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
+  const size_t tile = staged ? (bf16 ? tile_floats<__nv_bfloat16>(p.B, J) : tile_floats<float>(p.B, J)) : 0;
+  size_t head = part > stage ? part : stage;
+  if (tile > head) head = tile;
+  size_t n = (head + 3) / 4 * 4 + (size_t)p.B * R + (size_t)p.C * R + (size_t)J * R +
              (size_t)r1 * r2 * R * R + (size_t)p.H * R + (size_t)p.W * R +
              (size_t)r1 * r2 * p.H * R + ((size_t)r1 * r2 * (p.H + 2 * p.ph) * (p.W + 2 * p.pw) + 3) / 4 * 4 +
              (size_t)p.cpb * kk * R + (size_t)p.cpb * (N4 > p.nt ? N4 : p.nt);
@@ -2102,20 +2256,58 @@ static cudaError_t launch_pass1_t(const SmPass1Args& p, size_t smem, cudaStream_
   return launch_clustered(p.aligned || !p.vec4 ? k_sm_pass1<KIND, R, false, TX> : k_sm_pass1<KIND, R, true, TX>, pass1_grid(p),
                           p.cl, smem, st, p);
 }
-template <int R, typename TX>
-static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core<R, TX>), smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_sm_core<R, TX>, dim3(p.n_tiles), dim3(kPT), smem, st, p);
+// Which form a launch takes, by what it and the fused launches of the same call beside it (`beside` CTAs) bring to the
+// machine; results do not depend on it.  The staged forms need whole groups of four.
+//
+// Core: staged up to 296 CTAs (two an SM: one wave), and where a thread of the streamed form takes more than two rounds
+// of eight samples, each a round trip to memory.  One layer's step, streamed / staged: 64 x 512 x 7 x 7 (128 CTAs, two
+// rounds) 40.4 / 38.8 us, 128 x 960 x 7 x 7 (240, four) 63.9 / 57.7, 128 x 256 x 14 x 14 (256, four) 80.5 / 74.1; five
+// layers of 7 x 7 at 128 in a launch (840, four) 169.4 / 165.1; but the ResNet-18 tail at 64 (640 side by side, two rounds)
+// 91.0 / 95.2.  Up to 113 KB, two CTAs an SM (up to 208 KB: no difference on these).
+// All layers of a launch take one form.
+static void choose_core(SmCoreArgs* a, int n, int R, bool bf16, int beside) {
+  int ctas = beside, rounds = 0;
+  bool ok = true;
+  for (int l = 0; l < n; ++l) {
+    SmCoreArgs& p = a[l];
+    p.staged = 1;
+    ok = ok && p.vec4 && sm_core_smem(p, R, bf16) <= 113 * 1024;
+    if (!ok) break;
+    ctas += p.n_tiles;
+    const int per = 8 * (kPT / (p.tile_c * p.H * p.W / 4)), rd = (p.B + per - 1) / per;
+    if (rd > rounds) rounds = rd;
+  }
+  ok = ok && (ctas <= 296 || rounds > 2);
+  for (int l = 0; l < n; ++l) a[l].staged = ok ? 1 : 0;
+}
+// Weight gradient: staged up to one CTA an SM, where nothing else hides the stream of dY (64 x 512 x 7 x 7 layer, 128
+// CTAs, one layer's step: 38.8 / 37.5 us; 128 x 256 x 14 x 14 with stride two, 128 CTAs: 67.7 / 62.9; but 256 CTAs at 128 x
+// 14 x 14 74.1 / 75.0, and five layers at once 165 / 184).
+static bool wgrad_staged(const SmWgradArgs* a, int n, int R, bool bf16, int beside) {
+  int ctas = beside;
+  for (int l = 0; l < n; ++l) {
+    if (!a[l].vec4 || a[l].cpb * a[l].Ho * a[l].Wo / 4 > kTT || sm_wgrad_smem(a[l], R, true, bf16) > 208 * 1024) return false;
+    ctas += a[l].Cout / a[l].cpb;
+  }
+  return ctas <= 148;
 }
 
 template <int R, typename TX>
-static cudaError_t launch_wgrad_t(const SmWgradArgs& p, cudaStream_t st) {
-  const size_t smem = sm_wgrad_smem(p, R);
-  auto kernel = p.nt == 512 ? k_sm_wgrad<R, 512, TX> : k_sm_wgrad<R, 256, TX>;
+static cudaError_t launch_core_t(const SmCoreArgs& p, size_t smem, cudaStream_t st) {
+  auto kernel = p.staged ? k_sm_core_staged<R, TX> : k_sm_core<R, TX>;
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  kernel<<<p.Cout / p.cpb, p.nt, smem, st>>>(p);
+  return launch_pdl(kernel, dim3(p.n_tiles), dim3(p.staged ? kTT : kPT), smem, st, p);
+}
+
+template <int R, typename TX>
+static cudaError_t launch_wgrad_t(const SmWgradArgs& p, int beside, cudaStream_t st) {
+  const bool bf16 = sizeof(TX) == 2, staged = wgrad_staged(&p, 1, R, bf16, beside);
+  const size_t smem = sm_wgrad_smem(p, R, staged, bf16);
+  auto kernel = staged ? k_sm_wgrad_staged<R, TX> : (p.nt == 512 ? k_sm_wgrad<R, 512, TX> : k_sm_wgrad<R, 256, TX>);
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<p.Cout / p.cpb, staged ? kTT : p.nt, smem, st>>>(p);
   return cudaGetLastError();
 }
 
@@ -2182,19 +2374,21 @@ cudaError_t launch_sm_pass1(const SmPass1Args& p, int kind, int R, bool bf16, cu
   ASI_DISPATCH_KR(launch_pass1_t, p, sm_pass1_smem(p, kind, R), st);
 }
 
-cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_core(const SmCoreArgs& p0, int R, bool bf16, int beside, cudaStream_t st) {
+  SmCoreArgs p = p0;
+  choose_core(&p, 1, R, bf16, beside);
   const size_t eb = bf16 ? 2 : 4;
   ProfScope prof(ASI_K_SM_CORE, st, (double)p.B * p.C * p.H * p.W * eb);
-  ASI_DISPATCH_R(launch_core_t, p, sm_core_smem(p, R), st);
+  ASI_DISPATCH_R(launch_core_t, p, sm_core_smem(p, R, bf16), st);
 }
 
-cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, int beside, cudaStream_t st) {
   const size_t eb = bf16 ? 2 : 4;
   ProfScope prof(ASI_K_SM_WGRAD, st,
                  (double)p.B * p.Cout * p.Ho * p.Wo * eb +
                      4.0 * (double)p.Cout * (p.C / p.groups) * p.kh * p.kw);
-  if (R == 4) return bf16 ? launch_wgrad_t<4, __nv_bfloat16>(p, st) : launch_wgrad_t<4, float>(p, st);
-  return bf16 ? launch_wgrad_t<8, __nv_bfloat16>(p, st) : launch_wgrad_t<8, float>(p, st);
+  if (R == 4) return bf16 ? launch_wgrad_t<4, __nv_bfloat16>(p, beside, st) : launch_wgrad_t<4, float>(p, beside, st);
+  return bf16 ? launch_wgrad_t<8, __nv_bfloat16>(p, beside, st) : launch_wgrad_t<8, float>(p, beside, st);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2210,16 +2404,18 @@ static cudaError_t launch_pass1_bt(const SmBatch<SmPass1Args>& b, size_t smem, c
 }
 template <int R, typename TX>
 static cudaError_t launch_core_bt(const SmBatch<SmCoreArgs>& b, size_t smem, cudaStream_t st) {
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_core_b<R, TX>), smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_sm_core_b<R, TX>, dim3(b.first[b.n]), dim3(kPT), smem, st, b);
-}
-template <int R, typename TX>
-static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, cudaStream_t st) {
-  auto kernel = b.a[0].nt == 512 ? k_sm_wgrad_b<R, 512, TX> : k_sm_wgrad_b<R, 256, TX>;
+  const bool staged = b.a[0].staged != 0;            // all layers of a launch or none
+  auto kernel = staged ? k_sm_core_staged_b<R, TX> : k_sm_core_b<R, TX>;
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  kernel<<<b.first[b.n], b.a[0].nt, smem, st>>>(b);
+  return launch_pdl(kernel, dim3(b.first[b.n]), dim3(staged ? kTT : kPT), smem, st, b);
+}
+template <int R, typename TX>
+static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, bool staged, cudaStream_t st) {
+  auto kernel = staged ? k_sm_wgrad_staged_b<R, TX> : (b.a[0].nt == 512 ? k_sm_wgrad_b<R, 512, TX> : k_sm_wgrad_b<R, 256, TX>);
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<b.first[b.n], staged ? kTT : b.a[0].nt, smem, st>>>(b);
   return cudaGetLastError();
 }
 
@@ -2275,17 +2471,18 @@ cudaError_t launch_sm_reduce_batched(const SmReduceArgs* a, const int* max_chunk
   return launch_pdl(k_sm_reduce_b, dim3((unsigned)b.first[n], 4), dim3(kRedNT), 0, st, b);
 }
 
-cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16, int beside, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
   SmBatch<SmCoreArgs> b;
   size_t smem = 0;
   double bytes = 0.0;
   b.n = n;
   b.first[0] = 0;
+  for (int l = 0; l < n; ++l) b.a[l] = a[l];
+  choose_core(b.a, n, R, bf16, beside);
   for (int l = 0; l < n; ++l) {
-    b.a[l] = a[l];
     b.first[l + 1] = b.first[l] + a[l].n_tiles;
-    const size_t need = sm_core_smem(a[l], R);
+    const size_t need = sm_core_smem(b.a[l], R, bf16);
     if (need > smem) smem = need;
     bytes += (double)a[l].B * a[l].C * a[l].H * a[l].W * (bf16 ? 2 : 4);
   }
@@ -2293,8 +2490,9 @@ cudaError_t launch_sm_core_batched(const SmCoreArgs* a, int n, int R, bool bf16,
   ASI_DISPATCH_R(launch_core_bt, b, smem, st);
 }
 
-cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, cudaStream_t st) {
+cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf16, int beside, cudaStream_t st) {
   if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
+  const bool staged = wgrad_staged(a, n, R, bf16, beside);
   SmBatch<SmWgradArgs> b;
   size_t smem = 0;
   double bytes = 0.0;
@@ -2303,14 +2501,14 @@ cudaError_t launch_sm_wgrad_batched(const SmWgradArgs* a, int n, int R, bool bf1
   for (int l = 0; l < n; ++l) {
     b.a[l] = a[l];
     b.first[l + 1] = b.first[l] + a[l].Cout / a[l].cpb;
-    const size_t need = sm_wgrad_smem(a[l], R);
+    const size_t need = sm_wgrad_smem(a[l], R, staged, bf16);
     if (need > smem) smem = need;
     bytes += (double)a[l].B * a[l].Cout * a[l].Ho * a[l].Wo * (bf16 ? 2 : 4) +
              4.0 * (double)a[l].Cout * (a[l].C / a[l].groups) * a[l].kh * a[l].kw;
   }
   ProfScope prof(ASI_K_SM_WGRAD, st, bytes);
-  if (R == 4) return bf16 ? launch_wgrad_bt<4, __nv_bfloat16>(b, smem, st) : launch_wgrad_bt<4, float>(b, smem, st);
-  return bf16 ? launch_wgrad_bt<8, __nv_bfloat16>(b, smem, st) : launch_wgrad_bt<8, float>(b, smem, st);
+  if (R == 4) return bf16 ? launch_wgrad_bt<4, __nv_bfloat16>(b, smem, staged, st) : launch_wgrad_bt<4, float>(b, smem, staged, st);
+  return bf16 ? launch_wgrad_bt<8, __nv_bfloat16>(b, smem, staged, st) : launch_wgrad_bt<8, float>(b, smem, staged, st);
 }
 
 }  // namespace asi

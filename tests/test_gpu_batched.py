@@ -177,3 +177,42 @@ def test_layers_of_a_group_with_shifted_activations(bf16):
     torch.cuda.synchronize()
     for r, w in zip(runs, want):
         assert all(torch.equal(x, y) for x, y in zip((r.U[r.cur], r.core, r.dW), w))
+
+
+# Layers of few CTAs hold their tile in shared memory, steps of many CTAs stream it: the same bits.  Channels beyond the last
+# whole tile, few samples, a batch that is no multiple of the shares, ranks of both buckets, rows of odd length (not staged)
+FORMS = [
+    ((10, 130, 6, 6), (4, 4, 4, 4), 20, 3),
+    ((3, 84, 14, 14), (3, 3, 4, 4), 16, 3),
+    ((70, 100, 7, 8), (4, 5, 4, 6), 12, 1),
+    ((13, 133, 7, 7), (4, 4, 4, 3), 12, 3),
+    ((130, 96, 7, 7), (3, 4, 3, 4), 24, 3),
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("case", FORMS)
+def test_staged_and_streamed_tiles_give_the_same_bits(case, bf16):
+    from paper_2505_05086_b200.runner import StepRunner
+    dims, ranks, cout, k = case
+    L = LayerSpec("t", "conv", dims, cout, k, 1, k // 2, 1, ranks=ranks)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    dtype = torch.bfloat16 if bf16 else torch.float32
+    rng = np.random.default_rng(5)
+    runs = [make_runner(L, bf16=bf16) for _ in range(16)]
+    acts = [torch.randn(*dims, generator=gen, device="cuda").to(dtype) for _ in runs]
+    dys = [torch.randn(*L.dy_shape, generator=gen, device="cuda").to(dtype) for _ in runs]
+    want = []
+    for r, a, d in zip(runs, acts, dys):
+        r.set_factors([np.linalg.qr(rng.standard_normal((n, q)))[0] for n, q in zip(dims, ranks)])
+        r.compress(a)
+        r.wgrad(d)
+        want.append((r.U[r.cur].clone(), r.core.clone(), r.dW.clone()))
+        r.cur = 1 - r.cur
+    step = StepRunner(runs)
+    step.compress(acts)
+    step.wgrad(dys)
+    torch.cuda.synchronize()
+    for r, w in zip(runs, want):
+        assert r.ok()
+        assert all(torch.equal(x, y) for x, y in zip((r.U[r.cur], r.core, r.dW), w))
