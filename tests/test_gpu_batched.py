@@ -1,5 +1,7 @@
 """asi_compress_batched / asi_wgrad_batched: the layers of one training step in one call each way.
 The batched calls must give the bits that one call per layer gives, and match the fp64 oracle."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -216,3 +218,114 @@ def test_staged_and_streamed_tiles_give_the_same_bits(case, bf16):
     for r, w in zip(runs, want):
         assert r.ok()
         assert all(torch.equal(x, y) for x, y in zip((r.U[r.cur], r.core, r.dW), w))
+
+
+# twelve chains (no two layers share launches): more than a call has side streams
+MANY = [LayerSpec("c%d" % i, "conv", (6 + i, 9 + i, 18 + i, 21), 8 + i, 3, 1, 1, 1, ranks=(3, 4, 3, 4)) for i in range(6)] + \
+       [LayerSpec("l%d" % i, "linear", (5 + i, 33, 40 + 8 * i), 20 + i, ranks=(3, 5, 7)) for i in range(6)]
+
+
+def _singles(runs, acts, dys):
+    out = []
+    for r, a, d in zip(runs, acts, dys):
+        r.compress(a)
+        r.wgrad(d)
+        out.append((r.U[r.cur].clone(), r.core.clone(), r.dW.clone()))
+        r.cur = 1 - r.cur
+    torch.cuda.synchronize()
+    return out
+
+
+def _same(runs, want):
+    return all(torch.equal(x, y) for r, w in zip(runs, want) for x, y in zip((r.U[r.cur], r.core, r.dW), w))
+
+
+def test_more_chains_than_side_streams():
+    from paper_2505_05086_b200.runner import StepRunner
+    runs, acts, dys = _random_layers(MANY, 21)
+    want = _singles(runs, acts, dys)
+    step = StepRunner(runs)
+    for _ in range(5):
+        step.compress(acts)
+        step.wgrad(dys)
+        torch.cuda.synchronize()
+        assert _same(runs, want)
+        for r in runs:
+            r.cur = 1 - r.cur
+
+
+@pytest.mark.parametrize("specs", [SHARING, MANY])
+def test_batched_calls_in_a_captured_graph(specs):
+    """Captured on one stream: the layers follow one another there, the side streams stay out of the capture and serve
+    calls outside it while the graph exists."""
+    from paper_2505_05086_b200.runner import StepRunner
+    runs, acts, dys = _random_layers(specs, 22)
+    want = _singles(runs, acts, dys)
+    step = StepRunner(runs)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        step.compress(acts)                          # warm
+        step.wgrad(dys)
+        for r in runs:
+            r.cur = 1 - r.cur
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            step.compress(acts)
+            step.wgrad(dys)
+    for _ in range(3):
+        for r in runs:
+            r.dW.zero_()
+            r.core.zero_()
+            r.U[r.cur].zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert _same(runs, want)
+    for r in runs:
+        r.cur = 1 - r.cur
+    step.compress(acts)
+    step.wgrad(dys)
+    torch.cuda.synchronize()
+    assert _same(runs, want)
+    del graph
+
+
+def test_batched_calls_from_several_host_threads():
+    """Ten threads with layers and a stream of their own: more callers at a time than there are sets of side streams."""
+    from paper_2505_05086_b200.runner import StepRunner
+    specs = [MANY[0], MANY[7], SHARING[3], SHARING[4], SHARING[0]]
+    jobs = []
+    for i in range(10):
+        runs, acts, dys = _random_layers(specs, 30 + i)
+        jobs.append((runs, acts, dys, _singles(runs, acts, dys), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    errors = []
+    start = threading.Barrier(len(jobs))
+
+    def work(runs, acts, dys, want, stream):
+        try:
+            step = StepRunner(runs)
+            start.wait(timeout=60)
+            for _ in range(25):
+                step.compress(acts, stream)
+                step.wgrad(dys, stream)
+                stream.synchronize()
+                if not _same_on(stream, runs, want):
+                    raise AssertionError("results differ")
+                for r in runs:
+                    r.cur = 1 - r.cur
+        except BaseException as e:                   # handed to the test's own thread
+            errors.append(e)
+
+    def _same_on(stream, runs, want):
+        with torch.cuda.stream(stream):
+            return _same(runs, want)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join(timeout=120)
+    assert not errors, errors
+    assert not any(t.is_alive() for t in threads)
