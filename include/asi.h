@@ -86,7 +86,7 @@ typedef struct {
 /* The layer's kernels are expected to run beside kernels of other layers (one CUDA-graph branch or one stream
  * per layer; Algorithm 1 treats every fine-tuned layer of a step independently).  The streaming kernels of
  * large feature maps then launch one CTA per SM instead of two, which leaves registers and shared memory for
- * the neighbours: alone they run about 5 % slower, ten layers side by side about 4 % faster.  Results are the
+ * the neighbours: alone they run about 5 % slower, ten layers side by side 2 to 4 % faster.  Results are the
  * same up to the order of the per-CTA partial sums (a fixed order per plan). */
 #define ASI_FLAG_SHARE_SM 4
 
@@ -143,8 +143,8 @@ asi_status_t asi_init_factors(const asi_plan_t* plan, const void* act, const flo
  * the paper names no generator).  Omega_m is the first b_m r_m values of the counter-based stream
  * (seed, stream = m): Philox4x32-10 with key = seed and counter = (group index, stream, 0), a word x mapped to
  * u = ((x >> 9) + 0.5) 2^-23, pairs of words through Box-Muller in fp32; element e of a stream is value e mod 4
- * of group e div 4.  The matrices are drawn mode by mode into the workspace, so the caller holds no Omega and
- * the scratch grows by the largest b_m r_m floats only.  Same seed, same plan: same factors.
+ * of group e div 4.  The matrices of all modes are drawn in one launch into the workspace, so the caller holds no
+ * Omega and the scratch grows by the sum of b_m r_m floats over the modes.  Same seed, same plan: same factors.
  *   ws  device scratch of at least asi_init_seeded_ws_bytes(plan). */
 size_t asi_init_seeded_ws_bytes(const asi_plan_t* plan);
 asi_status_t asi_init_factors_seeded(const asi_plan_t* plan, const void* act, uint64_t seed, float* U_new,
@@ -163,7 +163,7 @@ asi_status_t asi_philox_words(uint64_t seed, uint32_t stream_id, int64_t n_group
  * type) share one launch per kernel stage -- a step of L such layers is 3 + 1 launches instead of
  * 3L + L --; such a group and every other layer run side by side on streams the library keeps (at most eight sets
  * of eight, destroyed with the last plan), forked from and joined to `stream` by events, or one after another when
- * `stream` is being captured.  Host-detectable errors are checked for all layers before anything is enqueued. */
+ * `stream` is being captured or when all sets are in use.  Host-detectable errors are checked for all layers before anything is enqueued. */
 asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* const* acts,
                                   const float* const* U_prev, float* const* U_new, float* const* cores,
                                   void* const* ws, const size_t* ws_bytes, int32_t n, void* stream);

@@ -1059,7 +1059,7 @@ asi_status_t asi_compress(const asi_plan_t* pl, const void* act, const float* U_
 // Batched entry points: the layers a training step compresses together (Algorithm 1 runs once per
 // fine-tuned layer and step; Sec. 4 fine-tunes the last 2..4 layers).  Layers on the fused small-map path
 // that share a kernel variant go through ONE launch of each kernel stage, their argument blocks in a
-// table the CTAs index; the remaining layers are enqueued one after another on the same stream.
+// table the CTAs index; these groups and the remaining layers are chains that run side by side (run_chains).
 // ---------------------------------------------------------------------------------------------
 namespace {
 // layers that share launches

@@ -185,9 +185,9 @@ struct SmWgradArgs {
   int r[ASI_MAX_MODES];
   int B, C, Cout, H, W, Ho, Wo, kh, kw, sh, sw, ph, pw, groups, cpb;
   int vec4;                     // columns of dY may be read four at a time
-  int nt;                       // threads per CTA: 256 or 512
-  int ncl;
-  int nbuf;            // staging blocks of term 5: two, or one                      // output channels expanded per round of term 5 (divides cpb)
+  int nt;                       // threads per CTA: 256 or 512 (the staged form has 512 and splits its sums as nt would)
+  int ncl;                      // output channels expanded per round of term 5 (divides cpb)
+  int nbuf;                     // staging blocks of term 5: two, or one
   int bulk_store;               // 1: dW row blocks leave through the bulk-copy engine (16-byte sized and aligned)
 };
 size_t sm_tile1_smem(int S, int R, int B, int C);
@@ -275,10 +275,6 @@ struct ProfScope {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// A mode pass of Algorithm 1 depends on nothing the passes before it on the stream write.  The first one (clear not
-// null) is launched normally and zeroes the workspace's status block; the others are programmatic dependents that
-// run beside their predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass
-// sees all of them finished.
 // Bt[(t N + j) ldb + k] = t-th bf16 term of v (hi, mid, lo: v = hi + mid + lo to 24 bits)
 __device__ __forceinline__ void tc_store_terms(__nv_bfloat16* Bt, int N, int64_t ldb, int j, int64_t k, float v) {
   const __nv_bfloat16 h = __float2bfloat16_rn(v);
@@ -289,6 +285,10 @@ __device__ __forceinline__ void tc_store_terms(__nv_bfloat16* Bt, int N, int64_t
   Bt[(int64_t)(2 * N + j) * ldb + k] = __float2bfloat16_rn(r1 - __bfloat162float(m));
 }
 
+// A mode pass of Algorithm 1 depends on nothing the passes before it on the stream write.  The first one (clear not
+// null) is launched normally and zeroes the workspace's status block; the others are programmatic dependents that
+// run beside their predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass
+// sees all of them finished.
 __device__ __forceinline__ void pass_begin(int* clear) {
   pdl_launch_dependents();
   if (clear && blockIdx.x == 0)
