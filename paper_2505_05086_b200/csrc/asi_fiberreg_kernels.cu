@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(NT, 1) k_fiber_reg(Fiber2Args p) {
   constexpr int NW = NT / 32;
   __shared__ __align__(16) float Us[R * KS * NJ];    // rows >= a and columns >= r are zero
   __shared__ float red[NW][R * KS * NJ];
-  if (!p.project_only) pass_begin(p.clear);          // a product alone: its successor starts when it ends (see k_fiber2)
+  if (!p.project_only || p.plain) pass_begin(p.clear);   // a product alone: its successor starts when it ends (see k_fiber2)
   if (p.project_only) pdl_wait();                    // its input comes from the kernel before
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ks = lane / QW, cq = lane - ks * QW;

@@ -96,9 +96,10 @@ __global__ void __launch_bounds__(kF2Threads, (RW <= 4 && NJ == 4) ? 3 : 2) k_fi
   constexpr int UPR = TQ / EPU;                      // units per staged row
   extern __shared__ __align__(128) unsigned char f2_smem[];
   // a product alone lets its successor start when it ends: the tail kernels that would wait beside a whole traversal take
-  // registers and shared memory from the other layers (ResNet-34 sweep, CUDA graph: 781 -> 774 us)
+  // registers and shared memory from the other layers (ResNet-34 sweep, CUDA graph: 781 -> 774 us).  Z1, the first kernel
+  // of a weight gradient, has k_z3 behind it, which does not wait for it
+  if (!p.project_only || p.plain) pass_begin(p.clear);
   if (p.project_only) pdl_wait();                    // its factor comes from the kernel before
-  else pass_begin(p.clear);
   const int tid = threadIdx.x, grp = tid >> 4, lane = tid & 15;
   const int a = p.a, r = p.r, nst = p.nstage;
   constexpr int AR = NG * RW;                        // staged rows: rows a..AR-1 stay zero, so no loop tests k < a
@@ -777,7 +778,6 @@ __global__ void __launch_bounds__(256) k_z3(const float* __restrict__ core, cons
                                             const float* __restrict__ U4, float* __restrict__ Z3, int r12, int r3,
                                             int r4, int H, int W) {
   extern __shared__ float z3_smem[];
-  pdl_launch_dependents();
   float* Ss = z3_smem;                 // [r3][r4] of this (i, j)
   float* U3s = Ss + r3 * r4;           // [H][r3]
   float* U4s = U3s + H * r3;           // [W][r4]

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
   constexpr int TC = wf_cols<TX>(RK), PT = TC + 4, NP = TC / 2, KQ = 32 / NP, UP = 12;
   constexpr int KB = 8, KS = KQ == 4 ? 2 : KQ;       // rows per step of the column pass, between a lane's rows
   extern __shared__ __align__(16) unsigned char ws_smem[];
-  if (!p.project_only) pass_begin(p.clear);          // a product alone: its successor starts when it ends (see k_fiber2)
+  if (!p.project_only || p.plain) pass_begin(p.clear);   // a product alone: its successor starts when it ends (see k_fiber2)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int a = p.a, r = p.r, a8 = (a + 7) & ~7;
   float* Ud = reinterpret_cast<float*>(ws_smem);     // [a8][UP]: rows >= a and columns >= r zero; rows 1, 4 and 5 apart are bank-disjoint
