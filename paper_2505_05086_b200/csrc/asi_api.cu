@@ -676,6 +676,7 @@ LaneSet* borrow_lanes(cudaStream_t st) {
       return l;
     }
   if (g_lane_sets >= kMaxSets) return nullptr;
+  g_lane_idle.reserve(kMaxSets);                     // handing a set back never allocates
   LaneSet* l = new (std::nothrow) LaneSet;
   if (!l) return nullptr;
   std::memset(l, 0, sizeof(*l));
@@ -691,6 +692,12 @@ LaneSet* borrow_lanes(cudaStream_t st) {
   }
   ++g_lane_sets;
   return l;
+}
+
+// the batched entry points keep lists on the host: a failed allocation is an error code like any other
+asi_status_t no_host_memory() {
+  snprintf(g_cuda_err, sizeof(g_cuda_err), "out of host memory");
+  return ASI_ERR_CUDA;
 }
 
 // What the layers of a batched call write, as address ranges.  Layers that write to the same memory (a workspace that
@@ -719,8 +726,13 @@ asi_status_t run_chains(int n_chains, bool independent, cudaStream_t st, F&& cha
   const int used = l ? std::min(n_chains - 1, kLanes) : 0;
   if (l) e = cudaEventRecord(l->fork, st);
   for (int i = 0; i < used && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(l->s[i], l->fork, 0);
-  for (int c = 0; c < n_chains && rc == ASI_OK && e == cudaSuccess; ++c)
-    rc = chain(c, (l && c > 0) ? l->s[(c - 1) % kLanes] : st);
+  for (int c = 0; c < n_chains && rc == ASI_OK && e == cudaSuccess; ++c) {
+    try {
+      rc = chain(c, (l && c > 0) ? l->s[(c - 1) % kLanes] : st);
+    } catch (const std::bad_alloc&) {
+      rc = no_host_memory();
+    }
+  }
   for (int i = 0; i < used; ++i) {                   // joined whatever happened: nothing of this call stays behind
     const cudaError_t e1 = cudaEventRecord(l->join[i], l->s[i]), e2 = cudaStreamWaitEvent(st, l->join[i], 0);
     if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
@@ -1072,7 +1084,7 @@ struct Variant {
 
 asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* const* acts,
                                   const float* const* U_prev, float* const* U_new, float* const* cores,
-                                  void* const* ws, const size_t* ws_bytes, int32_t n, void* stream) {
+                                  void* const* ws, const size_t* ws_bytes, int32_t n, void* stream) try {
   if (!plans || !acts || !U_prev || !U_new || !cores || !ws || !ws_bytes || n < 1 || n > 4096)
     return ASI_ERR_INVALID_ARG;
   Written out;
@@ -1141,6 +1153,8 @@ asi_status_t asi_compress_batched(const asi_plan_t* const* plans, const void* co
     ASI_CUDA(launch_sm_core_batched(ca.data(), g, p0->fast_R, p0->bf16, all - of(c), st));
     return ASI_OK;
   });
+} catch (const std::bad_alloc&) {
+  return no_host_memory();
 }
 
 static asi_status_t conv_wgrad_one(const asi_plan* pl, const float* core, const float* U, const void* dY, float* dW, void* ws,
@@ -1148,7 +1162,7 @@ static asi_status_t conv_wgrad_one(const asi_plan* pl, const float* core, const 
 
 asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* const* cores, const float* const* U,
                                const void* const* dY, float* const* dW, void* const* ws, const size_t* ws_bytes,
-                               int32_t n, void* stream) {
+                               int32_t n, void* stream) try {
   if (!plans || !cores || !U || !dY || !dW || !ws || !ws_bytes || n < 1 || n > 4096) return ASI_ERR_INVALID_ARG;
   Written out;
   for (int i = 0; i < n; ++i) {
@@ -1198,6 +1212,8 @@ asi_status_t asi_wgrad_batched(const asi_plan_t* const* plans, const float* cons
     ASI_CUDA(launch_sm_wgrad_batched(wa.data(), g, p0->fast_R, p0->bf16, all - of(c), st));
     return ASI_OK;
   });
+} catch (const std::bad_alloc&) {
+  return no_host_memory();
 }
 
 // ---------------------------------------------------------------------------------------------
