@@ -160,6 +160,26 @@ void layout_compress(asi_plan* pl) {
       pl->fiber_grid[m] = fiber2_grid(pl->mv[m].O, pl->mv[m].a, pl->mv[m].I, pl->r[m], pl->bf16,
                                       (pl->d.flags & ASI_FLAG_SHARE_SM) != 0);
     }
+  // these copy rows on 16 bytes, and so did the kernel that 28 x 28 planes had: such layers want the address on 16 bytes
+  const int64_t planes = pl->dims[0] * (pl->nd > 1 ? pl->dims[1] : 1);
+  pl->rows16 = pl->plane2 || (pl->plane && pl->dims[2] == 28 && pl->dims[3] == 28 && pl->r[2] <= 4 && pl->r[3] <= 4 && planes % 8 == 0);
+  for (int m = 0; m < pl->nd; ++m) pl->rows16 = pl->rows16 || pl->fiber2[m];
+  // the factor on the tensor cores, for conv layers (token layers have their own kernels)
+  pl->mplane = false;
+  for (int m = 0; m < ASI_MAX_MODES; ++m) pl->mfiber[m] = false;
+  const bool share = (pl->d.flags & ASI_FLAG_SHARE_SM) != 0;
+  if (pl->plane && mplane_supported(pl->dims[0] * pl->dims[1], pl->dims[2], pl->dims[3], pl->r[2], pl->r[3], pl->bf16)) {
+    pl->mplane = true;
+    pl->plane_grid = mplane_grid(pl->dims[0] * pl->dims[1], (int)pl->dims[2], (int)pl->dims[3], std::max(pl->r[2], pl->r[3]),
+                                 pl->bf16, share);
+  }
+  if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && pl->d.kind == ASI_CONV2D)
+    for (int m = 0; m < 2; ++m) {
+      const ModeView& v = pl->mv[m];
+      if (!mfiber_supported(v.O, v.a, v.I, v.r, pl->bf16) || (pl->bf16 && !pl->wfiber[m] && !pl->fiber2[m])) continue;
+      pl->mfiber[m] = pl->fiber[m] = true;
+      pl->fiber_grid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
+    }
   // V_m of the modes without a one-pass kernel, one region each (their products share launches); at least the
   // largest V of the layer
   if (!pl->fast_compress) {
@@ -321,9 +341,7 @@ bool element_aligned(const asi_plan* pl, const void* p) {
 
 // asi_compress takes this address: any element's, but for the 16-byte rows of the large-map kernels' bulk copies
 bool compress_takes(const asi_plan* pl, const void* act) {
-  bool rows16 = pl->plane2;
-  for (int m = 0; m < pl->nd; ++m) rows16 = rows16 || pl->fiber2[m];
-  return element_aligned(pl, act) && (!rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
+  return element_aligned(pl, act) && (!pl->rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
 }
 
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
@@ -1018,12 +1036,14 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     g.r4 = pl->r[3];
     g.status = status;
     g.clear = take_clear();
-    ASI_CUDA(pl->plane2 ? launch_plane2(g, pl->plane_grid, pl->bf16, st) : launch_wplane(g, pl->plane_grid, pl->bf16, st));
+    const bool mma = pl->mplane && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);   // else: odd bf16 addresses
+    if (mma) ASI_CUDA(launch_mplane(g, pl->plane_grid, pl->bf16, st));
+    else ASI_CUDA(pl->plane2 ? launch_plane2(g, pl->plane_grid, pl->bf16, st) : launch_wplane(g, pl->plane_grid, pl->bf16, st));
   }
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
     if (!pl->fiber[m] || (pl->plane && m >= 2)) continue;
-    if (pl->fiber2[m] || pl->wfiber[m]) {
+    if (pl->mfiber[m] || pl->fiber2[m] || pl->wfiber[m]) {
       Fiber2Args f;
       std::memset(&f, 0, sizeof(f));
       f.X = act;
@@ -1034,7 +1054,10 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
       f.n_tiles = fiber2_tiles(v.O, v.I);
       f.plain = first;
       f.clear = take_clear();
-      ASI_CUDA(pl->wfiber[m] ? launch_wfiber(f, pl->fiber_grid[m], pl->bf16, st)
+      f.status = status;
+      const bool mma = pl->mfiber[m] && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
+      if (mma) ASI_CUDA(launch_mfiber(f, pl->fiber_grid[m], pl->bf16, st));
+      else ASI_CUDA(pl->wfiber[m] ? launch_wfiber(f, pl->fiber_grid[m], pl->bf16, st)
                              : launch_fiber2(f, pl->fiber_grid[m], pl->bf16, st));
     } else {
       FiberArgs f;

@@ -69,6 +69,8 @@ struct Fiber2Args {
   int64_t y_so, y_sj;
   int64_t O, I, n_tiles;
   int ldu, a, r, project_only, nstage;
+  int team;            // k_mfiber: warps that share the rows of a tile (set by the launcher)
+  int* status;         // status word of the workspace (k_mfiber: an expired wait on a copy)
   int plain;           // launched after all earlier work of the stream (the first kernel of a call)
   int* clear;          // as in PlaneArgs (plain launches only)
 };
@@ -392,6 +394,12 @@ cudaError_t launch_wfiber(const Fiber2Args& p, int grid, bool bf16, cudaStream_t
 bool wplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4);
 int wplane_grid(int64_t n_planes, int H, int W, int r, bool bf16);
 cudaError_t launch_wplane(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st);
+bool mfiber_supported(int64_t O, int64_t a, int64_t I, int r, bool bf16);
+int mfiber_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16, bool share_sm);
+cudaError_t launch_mfiber(const Fiber2Args& p, int grid, bool bf16, cudaStream_t st);
+bool mplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4, bool bf16);
+int mplane_grid(int64_t n_planes, int H, int W, int r, bool bf16, bool share_sm);
+cudaError_t launch_mplane(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st);
 bool fiber2_supported(int64_t O, int64_t a, int64_t I, int r, bool bf16);
 int64_t fiber2_tiles(int64_t O, int64_t I);
 int fiber2_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16, bool share_sm);
@@ -510,7 +518,9 @@ struct asi_plan {
   int plane_grid;
   bool wfiber[ASI_MAX_MODES];      // ... by warps on their own (strided fibers)
   bool fiber2[ASI_MAX_MODES];      // ... by its register-tiled successor (ranks <= 4, 16-byte aligned rows)
-  bool plane2;                     // 28 x 28 and 56 x 56 planes, ranks <= 4
+  bool mfiber[ASI_MAX_MODES], mplane;   // ... with the factor on the tensor cores
+  bool plane2;                     // 56 x 56 planes, ranks <= 4
+  bool rows16;                     // act has to start on 16 bytes
   int fast_kind;                   // 7, 14: modes 3 and 4 as Gram matrices of such square maps; 0: any map of at most 256 positions
   int tile_S;                      // != 0: the first pass is k_sm_tile1 for this map size, else k_sm_pass1
   int fast_R, n_tiles_b, fast_cs, fast_cc, core_tile_c, n_tiles_core, cpb, wgrad_ncl, wgrad_nt, fold_gs;

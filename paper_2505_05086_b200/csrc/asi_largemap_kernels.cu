@@ -11,7 +11,7 @@
 //                                                                    registers across all tiles of the CTA
 //                With `project_only` the kernel stops after the projection and writes V: that is the mode
 //                product Y = X x_m U^T of the first core step and of Z1 = dY x_1 U_1^T (C_ASI term 1).
-//   k_plane2   : the two spatial modes of a conv activation with S x S planes, S = 28 or 56, in one pass over
+//   k_plane2   : the two spatial modes of a conv activation with 56 x 56 planes in one pass over
 //                whole planes: the column pass (contract h) gives V_3 and P_4, the row pass (contract w)
 //                gives V_4 and P_3.
 // Operand pairs are laid out so that no packing moves are needed: a 16-byte read of four neighbouring
@@ -344,7 +344,7 @@ cudaError_t launch_fiber2(const Fiber2Args& p0, int grid, bool bf16, cudaStream_
 }
 
 // ---------------------------------------------------------------------------------------------
-// k_plane2<S>: G = 224 * 28 / S^2 whole planes per tile (2 for S = 56, 8 for S = 28), 224 threads.
+// k_plane2<S>: G = 224 * 28 / S^2 whole planes per tile (2 for S = 56, the size that is built), 224 threads.
 //   column role  thread (quad, g, hs): columns 4 quad.. of plane g, rows 7 hs .. 7 hs + 6
 //       pass A   V3 partial [w][j] = sum_h X[h][w] U3[h][j]           (pairs along w, U3 duplicated)
 //       pass B   P4[w][j]        += sum_h X[h][w] V4[g,h][j]          (V4 duplicated)
@@ -604,7 +604,7 @@ size_t plane2_smem(int S, bool bf16) {
 int plane2_group(int S) { return kP2Threads / ((S / 4) * (S / 7)); }
 
 bool plane2_supported(int S, int64_t n_planes, int r3, int r4) {
-  return (S == 28 || S == 56) && r3 <= 4 && r4 <= 4 && n_planes % plane2_group(S) == 0;
+  return S == 56 && r3 <= 4 && r4 <= 4 && n_planes % plane2_group(S) == 0;
 }
 
 template <int S, typename TX>
@@ -617,8 +617,7 @@ static cudaError_t launch_plane2_t(const PlaneArgs& p, int grid, cudaStream_t st
 
 cudaError_t launch_plane2(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st) {
   ProfScope prof(ASI_K_EXPAND, st, (double)p.n_planes * p.S * p.S * (bf16 ? 2 : 4));
-  if (p.S == 56) return bf16 ? launch_plane2_t<56, __nv_bfloat16>(p, grid, st) : launch_plane2_t<56, float>(p, grid, st);
-  return bf16 ? launch_plane2_t<28, __nv_bfloat16>(p, grid, st) : launch_plane2_t<28, float>(p, grid, st);
+  return bf16 ? launch_plane2_t<56, __nv_bfloat16>(p, grid, st) : launch_plane2_t<56, float>(p, grid, st);
 }
 
 int plane2_grid(int S, int64_t n_planes, int max_ctas) {

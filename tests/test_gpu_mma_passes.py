@@ -1,0 +1,66 @@
+"""Mode passes with the factor on the tensor cores, at the sizes where their tiling can go wrong, against the fp64 oracle
+and the shape-generic kernels."""
+import numpy as np
+import pytest
+import torch
+
+from asi_inputs.configs import LayerSpec
+from asi_inputs.generator import LayerStream
+from tests.gpu_util import TOL_F32, check, compare_step, make_runner
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # (dims, ranks, bf16)
+    ((17, 33, 17, 20), (3, 4, 4, 4), False),       # two row tiles and one row more; columns in whole quads
+    ((65, 16, 18, 19), (4, 4, 3, 2), False),       # two warps a tile, the second nearly empty; odd rows
+    ((12, 130, 17, 17), (5, 8, 6, 7), False),      # three warps a tile, ranks above four, odd planes
+    ((6, 257, 16, 20), (2, 3, 4, 4), False),       # five warps a tile
+    ((3, 384, 17, 16), (3, 6, 5, 3), False),       # the longest mode, six warps
+    ((2, 48, 32, 32), (2, 4, 4, 4), False),        # the largest planes, a batch of two
+    ((16, 10, 12, 24), (4, 4, 4, 4), False),       # the smallest planes of their kernel, one row tile
+    ((9, 40, 31, 13), (4, 5, 8, 8), False),        # no square, no multiple of anything
+    ((128, 8, 28, 28), (3, 3, 3, 3), False),       # a full team; planes of 28
+    ((40, 48, 24, 24), (4, 4, 4, 4), True),        # bf16 rows and planes on 16 bytes
+    ((33, 128, 20, 20), (6, 5, 7, 5), True),       # bf16, ranks above four: 32 rows a warp
+    ((16, 24, 18, 26), (3, 4, 4, 4), True),        # bf16 rows off 16 bytes: the kernels of any address
+]
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", CASES)
+def test_mode_passes_against_the_oracle_and_the_generic_kernels(dims, ranks, bf16):
+    # decay that keeps sigma_r / sigma_1 >= 0.25, as the other small cases have it: fp32 sums then stay far below 1e-4
+    rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(dims, ranks)))
+    run, gen = make_runner(L, bf16=bf16), make_runner(L, bf16=bf16, generic_only=True)
+    U_prev = st.u_prev0()
+    for t in range(2):
+        A, dY = st.next()
+        err_g, _ = compare_step(gen, L, A, dY, U_prev)
+        err, U_prev = compare_step(run, L, A, dY, U_prev)
+        check(err_g, TOL_F32, f"generic {dims}")
+        check(err, TOL_F32, str(dims))
+
+
+@pytest.mark.parametrize("dims,ranks", [((50, 116, 27, 27), (5, 6, 5, 5)), ((40, 40, 18, 21), (5, 5, 6, 8))])
+def test_any_element_address(dims, ranks):
+    """Layers that take an fp32 activation at any element: off 16 bytes its rows and planes come by four-byte copies.  The sums
+    are the same up to the order of fp32 additions (1e-6 on well-conditioned random data, times ten)."""
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    run = make_runner(L)
+    rng = np.random.default_rng(3)
+    A = torch.from_numpy(rng.standard_normal(dims).astype(np.float32)).cuda()
+    run.U[0].copy_(torch.randn(run.plan.info.u_elems, generator=torch.Generator().manual_seed(1)))
+    big = torch.zeros(A.numel() + 8, device="cuda")
+    out = []
+    for shift in (0, 1, 3):
+        big[shift:shift + A.numel()].copy_(A.reshape(-1))
+        run.cur = 0
+        run.compress(big[shift:shift + A.numel()])
+        torch.cuda.synchronize()
+        assert run.ok()
+        out.append([run.U[1].clone(), run.core.clone()])
+    for o in out[1:]:
+        for x, y in zip(o, out[0]):
+            assert float((x - y).norm() / y.norm()) <= 1e-5
