@@ -283,9 +283,9 @@ void layout_compress(asi_plan* pl) {
   pl->launches_compress = 3;
   if (!pl->fast_compress) {
     pl->core_tok = pl->d.kind == ASI_LINEAR && (pl->nd == 2 || order[0] == 2);
-    // the two kernels of Orthogonalize, the core chain, one launch per one-pass mode (one for both spatial modes),
-    // one projection and one expansion launch for all SIMT modes together
-    pl->launches_compress = 2 + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
+    // the kernels of Orthogonalize (one for ranks up to eight), the core chain, one launch per one-pass mode (one for both
+    // spatial modes), one projection and one expansion launch for all SIMT modes together
+    pl->launches_compress = (pl->small_rank ? 1 : 2) + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
     bool simt = false, tc = false;
     for (int m = 0; m < pl->nd; ++m) {
       if (pl->plane && m >= 2) pl->launches_compress += (m == 2);
@@ -495,19 +495,8 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
   if (pl->small_rank) {
     SmReduceArgs ra;
     max_chunks = build_fused_reduce(pl, w, nullptr, &ra);
+    for (int m = 0; m < pl->nd; ++m) ra.m[m].U = U_new + pl->u_off[m];
     ASI_CUDA(launch_sm_reduce(ra, pl->nd, max_chunks, st));
-    RowSolveArgs rs;
-    std::memset(&rs, 0, sizeof(rs));
-    rs.Rf = ra.Rf;
-    rs.nd = pl->nd;
-    for (int m = 0; m < pl->nd; ++m) {
-      rs.Pred[m] = ra.m[m].Pred;
-      rs.U[m] = U_new + pl->u_off[m];
-      rs.a[m] = (int)pl->dims[m];
-      rs.r[m] = pl->r[m];
-      rs.total += rs.a[m];
-    }
-    ASI_CUDA(launch_row_solve(rs, st));
     return ASI_OK;
   }
   QRArgs qa;

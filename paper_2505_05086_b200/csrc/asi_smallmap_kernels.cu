@@ -23,7 +23,9 @@ namespace asi {
 
 namespace {
 
-constexpr int kRedNT = 256;          // threads per CTA of the partial-reduction kernel
+// threads per CTA of the partial-reduction kernel: fused layers (whose grids have many CTAs that end at once: MobileNetV2 tail 16.6 us,
+// 20.4 with 512 threads), and the layers of large maps
+constexpr int kRedNT = 256, kRedNTLarge = 512;
 
 
 // ---- bulk-copy engine (TMA, untiled form) and mbarrier ------------------------------------------
@@ -1251,15 +1253,19 @@ __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1_b(const __grid
 // Gram matrices A_m A_m^T (a <= 16) is summed the same way, a slice of the a x a elements per CTA.
 // With args.factor the last CTA of a mode to finish then factors the mode once for all CTAs of the
 // core kernel: it sums the shares of P_m^T P_m (a Gram mode: forms P_m = G_m U_m^prev first), and
-// leaves the Cholesky factor R_m and 1 / diag(R_m) in args.Rf.
+// leaves the Cholesky factor R_m and 1 / diag(R_m) in args.Rf; with M.U it also solves for the rows of U_m.
+// LARGE (the layers of large maps, 148 to 296 partials a mode): a chain of round trips to memory, so 512 threads with sixteen
+// partials each in flight, and the rows solved here: 10.7 us where 256 threads took 11.7 and a launch for the rows 3.5 more
+// (128 x 128 x 28 x 28 bf16, one layer's step 91.3 -> 89.2 us).  Fused layers lose by it (MobileNetV2 tail 165 -> 168 us).
 // ---------------------------------------------------------------------------------------------
+template <bool LARGE>
 __device__ __forceinline__ void sm_reduce_cta(const SmReduceArgs& args, const int c, const int mode) {
-  constexpr int RM = 8, RPC = kRedRows;
+  constexpr int RM = 8, RPC = kRedRows, NT = LARGE ? kRedNTLarge : kRedNT;
   const SmReduceMode M = args.m[mode];   // a copy in registers: reading the fields through the parameter each time cost 9 % of a step
   pdl_launch_dependents();
   if (c >= M.nchunk) return;
   pdl_wait();                                      // the partials come from the previous kernel
-  __shared__ double part[kRedNT];
+  __shared__ double part[NT];
   __shared__ double Ps[RPC][RM];
   const int tid = threadIdx.x;
   const int r = M.r, a = M.a;
@@ -1273,18 +1279,29 @@ __device__ __forceinline__ void sm_reduce_cta(const SmReduceArgs& args, const in
   const int64_t stride = M.gram ? (int64_t)a * a : (int64_t)a * r;
   int EP = 32;
   while (EP < E) EP <<= 1;
-  const int SG = kRedNT / EP;
+  const int SG = NT / EP;
   {
     const int e = tid & (EP - 1), sg = tid >> (31 - __clz(EP));
     double acc = 0.0;
     if (e < E) {
       const float* ptr = M.Pp + first + e;
+      if constexpr (LARGE) {                         // sixteen partials in flight, the last batch too
+#pragma unroll 1
+        for (int s = sg; s < M.nsplit; s += 16 * SG) {
+          float v[16];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) v[u] = s + u * SG < M.nsplit ? __ldcg(ptr + (s + u * SG) * stride) : 0.f;
+#pragma unroll
+          for (int u = 0; u < 16; ++u) acc += (double)v[u];
+        }
+      } else {
 #pragma unroll 8
-      for (int s = sg; s < M.nsplit; s += SG) acc += (double)__ldcg(ptr + s * stride);
+        for (int s = sg; s < M.nsplit; s += SG) acc += (double)__ldcg(ptr + s * stride);
+      }
     }
     part[tid] = acc;
   }
-  for (int idx = tid; idx < RPC * RM; idx += kRedNT) Ps[idx / RM][idx % RM] = 0.0;
+  for (int idx = tid; idx < RPC * RM; idx += NT) Ps[idx / RM][idx % RM] = 0.0;
   __syncthreads();
   if (tid < E) {
     double v = 0.0;
@@ -1347,8 +1364,8 @@ __device__ __forceinline__ void sm_reduce_cta(const SmReduceArgs& args, const in
   } else {
     // Gram mode (a <= 16): P_m = G_m U_m^prev (Algorithm 1: A_m (A_m^T U)), kept in fp64 for the row
     // solves of the core kernel, then its Gram matrix
-    for (int e = tid; e < a * a; e += kRedNT) Gfull[e] = __ldcg(M.Pred + e);
-    for (int e = tid; e < a * r; e += kRedNT) Ups[e] = __ldg(M.U_prev + e);
+    for (int e = tid; e < a * a; e += NT) Gfull[e] = __ldcg(M.Pred + e);
+    for (int e = tid; e < a * r; e += NT) Ups[e] = __ldg(M.U_prev + e);
     __syncthreads();
     if (tid < a * r) {
       const int k = tid / r, j = tid - k * r;
@@ -1400,14 +1417,41 @@ __device__ __forceinline__ void sm_reduce_cta(const SmReduceArgs& args, const in
     if (lane < r) Rf[RM * RM + lane] = Dinv[lane];
     if (lane == 0) args.counter[mode] = 0;
   }
+  if constexpr (!LARGE) return;
+  // ---- U_m = P_m R_m^{-1}, a row per thread (a launch of its own took 3.5 us of the chain)
+  __syncthreads();
+  double nx[RM];                                     // the next row is on its way while one is solved
+  auto fetch = [&](int row) {
+#pragma unroll
+    for (int j = 0; j < RM; ++j) nx[j] = (row < a && j < r) ? __ldcg(M.Pred + (int64_t)row * r + j) : 0.0;
+  };
+  fetch(tid);
+  for (int row = tid; row < a; row += NT) {
+    double q[RM];
+#pragma unroll
+    for (int j = 0; j < RM; ++j) q[j] = nx[j];
+    fetch(row + NT);
+#pragma unroll
+    for (int j = 0; j < RM; ++j)
+      if (j < r) {
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+          if (i < j) q[j] = fma(-q[i], Gs[i][j], q[j]);
+        q[j] *= Dinv[j];
+        M.U[(int64_t)row * r + j] = (float)q[j];
+      }
+  }
 }
 
 __global__ void __launch_bounds__(kRedNT) k_sm_reduce(const __grid_constant__ SmReduceArgs args) {
-  sm_reduce_cta(args, (int)blockIdx.x, (int)blockIdx.y);
+  sm_reduce_cta<false>(args, (int)blockIdx.x, (int)blockIdx.y);
+}
+__global__ void __launch_bounds__(kRedNTLarge) k_sm_reduce_large(const __grid_constant__ SmReduceArgs args) {
+  sm_reduce_cta<true>(args, (int)blockIdx.x, (int)blockIdx.y);
 }
 __global__ void __launch_bounds__(kRedNT) k_sm_reduce_b(const __grid_constant__ SmBatch<SmReduceArgs> b) {
   const int l = batch_layer(b, (int)blockIdx.x);
-  sm_reduce_cta(b.a[l], (int)blockIdx.x - b.first[l], (int)blockIdx.y);
+  sm_reduce_cta<false>(b.a[l], (int)blockIdx.x - b.first[l], (int)blockIdx.y);
 }
 
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st) {
@@ -1416,6 +1460,7 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
     bytes += 4.0 * p.m[m].nsplit * p.m[m].a * (p.m[m].gram ? p.m[m].a : p.m[m].r) + 8.0 * p.m[m].a * p.m[m].r;
   ProfScope prof(ASI_K_QR, st, bytes);
   dim3 grid((unsigned)max_chunks, (unsigned)nd);
+  if (p.m[0].U) return launch_pdl(k_sm_reduce_large, grid, dim3(kRedNTLarge), 0, st, p);
   return launch_pdl(k_sm_reduce, grid, dim3(kRedNT), 0, st, p);
 }
 
