@@ -250,6 +250,11 @@ void layout_compress(asi_plan* pl) {
     if ((double)pl->dims[m] / pl->r[m] > (double)pl->dims[best] / pl->r[best]) best = m;
   // linear layers: the feature mode first where that shrinks the tensor by four at least (k_core_tok does the rest)
   if (pl->d.kind == ASI_LINEAR && (pl->nd == 2 || pl->dims[pl->nd - 1] >= 4 * pl->r[pl->nd - 1])) best = pl->nd - 1;
+  // conv layers whose core k_core_tail finishes: the batch first where that shrinks the tensor by four at least (50 x 116 x 27 x 27,
+  // ranks 5: 91.0 -> 85.9 us a step; the channels first are three grouped products more)
+  const bool tail = pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
+                    core_tail_supported(pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[2], (int)pl->dims[3]);
+  if (tail && pl->dims[0] >= 4 * (int64_t)pl->r[0]) best = 0;
   std::swap(order[0], order[best]);
   std::sort(order + 1, order + pl->nd);
   std::memcpy(pl->core_order, order, sizeof(order));
@@ -272,9 +277,7 @@ void layout_compress(asi_plan* pl) {
   }
   pl->core_tail = pl->core_tok = false;
   pl->off_ctp = off;
-  if (pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
-      order[0] == 0 && order[1] == 1 && order[2] == 2 && order[3] == 3 &&
-      core_tail_supported(pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[2], (int)pl->dims[3])) {
+  if (tail && order[0] == 0) {                       // the others follow in order
     pl->core_tail = true;
     off = align_up(off + 4 * core_tail_part_elems(pl->r[0], pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[1],
                                                   (int)pl->dims[2], (int)pl->dims[3]), 256);

@@ -404,7 +404,7 @@ struct CoreTailArgs {
   const float *U2, *U3, *U4;
   float* part;         // [r1][chunks x splits][r2 r3 r4] partial cores
   float* core;
-  int* counter;        // zero on entry, zero again on exit
+  int* counter;        // one per i < r1, zero on entry, zero again on exit
   int r1, r2, r3, r4, C, H, W, RH, cper;
 };
 bool core_tail_supported(int r2, int r3, int r4, int H, int W);

@@ -630,7 +630,8 @@ int plane2_grid(int S, int64_t n_planes, int max_ctas) {
 // T = A x_1 U_1^T is [r1][C][H][W]; CTA (chunk, i, cs) takes RH whole rows of the planes T[i][c], c in
 // channel split cs:  Z[j][h,w] = sum_c U2[c][j] T[i][c][h][w]  (thread per position, coalesced),
 // Y[j][h][l] = sum_w Z[j][h][w] U4[w][l],  part[j][k][l] = sum_h U3[h][k] Y[j][h][l]  over the chunk's rows.
-// The last CTA to finish adds the partial cores in (chunk, split) order: core = T x_2 U_2^T x_3 U_3^T x_4 U_4^T.
+// The last CTA of each i to finish adds its partial cores in (chunk, split) order: core = T x_2 U_2^T x_3 U_3^T x_4 U_4^T
+// (one CTA for all i read six batches of shares one after another at ranks 5: 12.4 us, 8.4 now).
 // A chain of round trips to memory: a thread's sixteen channels are read at once, beside the factors, and the last CTA
 // reads sixteen shares at a time (128 x 128 x 28 x 28, ranks 3: 14.7 -> 11.8 us).
 // ---------------------------------------------------------------------------------------------
@@ -707,39 +708,39 @@ __global__ void __launch_bounds__(256) k_core_tail(CoreTailArgs p) {
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(p.counter, 1) == (int)(gridDim.x * gridDim.y * gridDim.z) - 1);
+  if (tid == 0) s_last = (atomicAdd(p.counter + i, 1) == nparts - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   // thread (element, q) adds the shares == q (mod nq) of its element, sixteen in flight; the nq sums meet in q order
-  const int n_el = p.r1 * ce;
-  int nq = 256 / n_el;
+  int nq = 256 / ce;
   nq = nq < 1 ? 1 : (nq > 8 ? 8 : nq);
-  __shared__ float fold[256];                // [nq][n_el] where nq > 1
-  for (int it = tid; it < nq * n_el; it += 256) {
-    const int q = it / n_el, idx = it - q * n_el, ii = idx / ce, e = idx - ii * ce;
-    const float* sp = p.part + (int64_t)ii * nparts * ce + e;
+  __shared__ float fold[256];                // [nq][ce] where nq > 1
+  const float* shares = p.part + (int64_t)i * nparts * ce;
+  float* core = p.core + (int64_t)i * ce;
+  for (int it = tid; it < nq * ce; it += 256) {
+    const int q = it / ce, e = it - q * ce;
     float s = 0.f;
 #pragma unroll 1
     for (int q0 = q; q0 < nparts; q0 += 16 * nq) {
       float v[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = __ldcg(sp + (int64_t)((q0 + u * nq < nparts) ? (q0 + u * nq) : q0) * ce);
+      for (int u = 0; u < 16; ++u) v[u] = __ldcg(shares + (int64_t)((q0 + u * nq < nparts) ? (q0 + u * nq) : q0) * ce + e);
 #pragma unroll
       for (int u = 0; u < 16; ++u) s += (q0 + u * nq < nparts) ? v[u] : 0.f;
     }
     if (nq > 1) fold[it] = s;
-    else p.core[idx] = s;
+    else core[e] = s;
   }
   if (nq > 1) {
     __syncthreads();
-    if (tid < n_el) {
+    if (tid < ce) {
       float s = fold[tid];
-      for (int q = 1; q < nq; ++q) s += fold[q * n_el + tid];
-      p.core[tid] = s;
+      for (int q = 1; q < nq; ++q) s += fold[q * ce + tid];
+      core[tid] = s;
     }
   }
-  if (tid == 0) *p.counter = 0;
+  if (tid == 0) p.counter[i] = 0;
 }
 
 bool core_tail_supported(int r2, int r3, int r4, int H, int W) {
