@@ -528,9 +528,8 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
 
 // A mode product: the register-tiled streaming kernel when a large tensor fits it (strided fibers, contiguous outputs
 // per (o, j)), else the grouped SIMT product.
-// dep: launched as a programmatic dependent (never the first kernel of a call: the kernels behind it may start
-// before it does, and must find everything older finished).
-cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, bool dep, cudaStream_t st) {
+// first: the first kernel of a call.
+cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf16, bool first, cudaStream_t st) {
   const bool fits = !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && a.si == 1 && a.sj == a.I &&
                     a.so == (int64_t)a.n_out * a.I && a.Q * a.a >= (1 << 20) &&
                     a.I >= 32 && wfiber_supported(a.O, a.a, a.I, a.n_out);
@@ -541,7 +540,7 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
     g.np = 0;
     g.clear = nullptr;
     gemm_add(&g, gemm_project(a.X, a.B, a.Y, a.O, a.a, a.I, a.n_out, a.so, a.sj, a.si, x_bf16));
-    return launch_gemm_group(g, x_bf16, dep, st);
+    return launch_gemm_group(g, x_bf16, st);
   }
   Fiber2Args f;
   std::memset(&f, 0, sizeof(f));
@@ -554,7 +553,7 @@ cudaError_t stream_modeprod(const asi_plan* pl, const ModeProdArgs& a, bool x_bf
   f.O = a.O; f.I = a.I; f.a = (int)a.a; f.r = a.n_out;
   f.n_tiles = fiber2_tiles(a.O, a.I);
   f.project_only = 1;
-  f.plain = !dep;
+  f.first = first;
   if (!f2) return launch_wfiber(f, wfiber_grid(a.O, a.a, a.I, a.n_out), x_bf16, st);
   return launch_fiber2(f, fiber2_grid(a.O, a.a, a.I, a.n_out, x_bf16, (pl->d.flags & ASI_FLAG_SHARE_SM) != 0),
                        x_bf16, st);
@@ -574,7 +573,7 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     sp.n = 0;
     sp.clear = nullptr;
     tc_add_split(&sp, U_new + pl->u_off[m0], pl->mv[m0].a, pl->r[m0], w + pl->tcu_off[m0]);
-    ASI_CUDA(launch_tc_split(sp, true, st));
+    ASI_CUDA(launch_tc_split(sp, st));
   }
   if (pl->fast_compress) {
     SmCoreArgs c;
@@ -606,9 +605,9 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     if (s == 0 && tc_core) {
       const ModeView& v = pl->mv[m];
       const TcCall t = {act, w + pl->tcu_off[m], dst, nullptr, 0, v.O, v.a, v.I, 0, v.r, 1, 0};
-      ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
+      ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), st));
     } else {
-      ASI_CUDA(stream_modeprod(pl, a, src_bf16, true, st));
+      ASI_CUDA(stream_modeprod(pl, a, src_bf16, false, st));
     }
     if (s == 0 && pl->core_tok) {
       CoreTokArgs t;
@@ -763,7 +762,7 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
 }
 
 // cold start: P_m = A_m Omega_m of all modes, one launch of SIMT products and one of tensor-core products.
-// clear: the first launch here zeroes the status block (it is then not a dependent one)
+// clear: the first launch here zeroes the status block
 asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool clear,
                           cudaStream_t st) {
   int* const status = reinterpret_cast<int*>(w);
@@ -784,13 +783,13 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
   }
   g.clear = clear ? status : nullptr;
   if (g.np) {
-    ASI_CUDA(launch_gemm_group(g, pl->bf16, !clear, st));
+    ASI_CUDA(launch_gemm_group(g, pl->bf16, st));
     clear = false;
   }
   if (sp.n) {
     sp.clear = clear ? status : nullptr;
-    ASI_CUDA(launch_tc_split(sp, false, st));
-    ASI_CUDA(launch_tc_group(t, sp.n, status, true, st));
+    ASI_CUDA(launch_tc_split(sp, st));
+    ASI_CUDA(launch_tc_group(t, sp.n, status, st));
   }
   return ASI_OK;
 }
@@ -972,9 +971,8 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     }
     return finish_compress(pl, act, U_new, core, w, U_prev, false, beside, st);
   }
-  // The first kernel on the caller's stream clears the status block and starts only when the stream's earlier work
-  // is done; the mode passes behind it do not depend on one another and are launched as programmatic dependents
-  // (each waits for its predecessor before it ends, so that what follows the last one sees all of them).
+  // The first kernel waits for the stream's earlier work and clears the status block; the mode passes behind it do not depend
+  // on one another (each waits for its predecessor before it ends, so that what follows the last one sees all of them).
   int* const status = reinterpret_cast<int*>(w);
   bool first = true;
   auto take_clear = [&]() {
@@ -1011,7 +1009,7 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
   }
   if (sp.n) {
     sp.clear = take_clear();
-    ASI_CUDA(launch_tc_split(sp, false, st));
+    ASI_CUDA(launch_tc_split(sp, st));
   }
   if (pl->plane) {
     PlaneArgs g;
@@ -1044,7 +1042,7 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
       f.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
       f.O = v.O; f.I = v.I; f.a = (int)v.a; f.r = v.r;
       f.n_tiles = fiber2_tiles(v.O, v.I);
-      f.plain = first;
+      f.first = first;
       f.clear = take_clear();
       f.status = status;
       const bool mma = pl->mfiber[m] && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
@@ -1065,14 +1063,13 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     }
   }
   if (gp.np) {
-    const bool dep = !first;
     gp.clear = take_clear();
-    ASI_CUDA(launch_gemm_group(gp, pl->bf16, dep, st));
-    ASI_CUDA(launch_gemm_group(ge, pl->bf16, true, st));
+    ASI_CUDA(launch_gemm_group(gp, pl->bf16, st));
+    ASI_CUDA(launch_gemm_group(ge, pl->bf16, st));
   }
   if (sp.n) {
-    ASI_CUDA(launch_tc_group(proj, sp.n, status, true, st));
-    ASI_CUDA(launch_tc_group(expd, sp.n, status, true, st));
+    ASI_CUDA(launch_tc_group(proj, sp.n, status, st));
+    ASI_CUDA(launch_tc_group(expd, sp.n, status, st));
   }
   return finish_compress(pl, act, U_new, core, w, nullptr, sp.n > 0, beside, st);
 }
@@ -1366,7 +1363,7 @@ static asi_status_t conv_wgrad_one(const asi_plan* pl, const float* core, const 
   a.O = 1; a.a = B; a.I = per_sample; a.Q = per_sample;
   a.n_out = r1;
   a.so = (int64_t)r1 * per_sample; a.sj = per_sample; a.si = 1;
-  ASI_CUDA(stream_modeprod(pl, a, pl->bf16, false, st));
+  ASI_CUDA(stream_modeprod(pl, a, pl->bf16, true, st));
   // terms 2-3 in one launch
   ASI_CUDA(launch_z3(core, U + pl->u_off[2], U + pl->u_off[3], Z3, r1 * r2, r3, r4, (int)H, (int)W, st));
   // terms 4 and 5
@@ -1412,15 +1409,15 @@ asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const flo
     sp.n = 0;
     sp.clear = reinterpret_cast<int*>(w);
     tc_add_split(&sp, a.B, N, a.n_out, w + pl->off_wtc);
-    ASI_CUDA(launch_tc_split(sp, false, st));
+    ASI_CUDA(launch_tc_split(sp, st));
     const TcCall t = {dY, w + pl->off_wtc, Y1, nullptr, 0, B, N, Dout, 0, a.n_out, 1, 0};
-    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), true, st));
+    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), st));
   } else {
     GemmGroup g;
     g.np = 0;
     g.clear = nullptr;
     gemm_add(&g, gemm_project(a.X, a.B, a.Y, a.O, a.a, a.I, a.n_out, a.so, a.sj, a.si, pl->bf16));
-    ASI_CUDA(launch_gemm_group(g, pl->bf16, false, st));
+    ASI_CUDA(launch_gemm_group(g, pl->bf16, st));
   }
   LinMidArgs mid;
   mid.Y1 = Y1; mid.core = core; mid.Z4 = Z4;

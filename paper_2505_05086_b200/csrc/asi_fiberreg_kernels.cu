@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(NT, 1) k_fiber_reg(Fiber2Args p) {
   constexpr int NW = NT / 32;
   __shared__ __align__(16) float Us[R * KS * NJ];    // rows >= a and columns >= r are zero
   __shared__ float red[NW][R * KS * NJ];
-  if (!p.project_only || p.plain) pass_begin(p.clear);   // a product alone: its successor starts when it ends (see k_fiber2)
+  if (!p.project_only || p.first) pass_begin(p.clear, p.first);   // a product alone: its successor starts when it ends (see k_fiber2)
   if (p.project_only) pdl_wait();                    // its input comes from the kernel before
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ks = lane / QW, cq = lane - ks * QW;
@@ -208,7 +208,7 @@ FrShape fiber_reg_shape(int64_t a, int rank, bool bf16) {
 
 template <int NJ, int KS, int R, int CW, int NT, typename TX>
 cudaError_t launch_fr(const Fiber2Args& p, int grid, cudaStream_t st) {
-  return launch_maybe_pdl(!p.plain, k_fiber_reg<NJ, KS, R, CW, NT, TX>, dim3(grid), dim3(NT), 0, st, p);
+  return launch_pdl(k_fiber_reg<NJ, KS, R, CW, NT, TX>, dim3(grid), dim3(NT), 0, st, p);
 }
 
 template <int NJ, int R, int CW, int NT, typename TX>

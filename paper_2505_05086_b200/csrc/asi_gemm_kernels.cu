@@ -521,7 +521,7 @@ __host__ __device__ GemmArg gemm_tile_arg(const GemmProb& p, int64_t t, int xbyt
   return w;
 }
 
-static cudaError_t launch_narrow(GemmArgs& g, bool bf16, bool pdl, cudaStream_t st) {
+static cudaError_t launch_narrow(GemmArgs& g, bool bf16, cudaStream_t st) {
   // the longest contractions first: their CTAs would otherwise start last and run alone
   std::sort(g.p, g.p + g.np, [](const GemmArg& a, const GemmArg& b) {
     return (int64_t)std::min(a.K, a.kps) * bn_of(a.n) > (int64_t)std::min(b.K, b.kps) * bn_of(b.n);
@@ -567,18 +567,16 @@ static cudaError_t launch_narrow(GemmArgs& g, bool bf16, bool pdl, cudaStream_t 
     at[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (pdl) {
-    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
+  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
   cfg.attrs = at;
   cfg.numAttrs = na;
   return cudaLaunchKernelEx(&cfg, kernel, g);
 }
 
 template <typename TX>
-static cudaError_t launch_wide(const GemmProb& p, int* clear, bool pdl, cudaStream_t st) {
+static cudaError_t launch_wide(const GemmProb& p, int* clear, cudaStream_t st) {
   if (p.kps > (p.nsplit > 1 || p.kin < p.K ? kGemmMaxSpan : INT32_MAX - kGK)) return cudaErrorInvalidValue;
   const int64_t ctas = (p.M + kGM - 1) / kGM * p.O * p.nsplit;
   const int bn = bn_of(p.n), nst = bn == 64 ? 2 : 3;
@@ -586,15 +584,14 @@ static cudaError_t launch_wide(const GemmProb& p, int* clear, bool pdl, cudaStre
   const size_t smem = std::max<size_t>(stage * nst, (size_t)kGW * kGM * bn * 4);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_gemm_wide<TX>), smem);
   for (int64_t t = 0; t < ctas && e == cudaSuccess; t += kGemmMaxGrid) {       // more tiles than a grid holds: in parts
-    e = launch_maybe_pdl(pdl, k_gemm_wide<TX>, dim3((unsigned)std::min(ctas - t, kGemmMaxGrid)), dim3(kGT), smem, st, p, t, nst,
+    e = launch_pdl(k_gemm_wide<TX>, dim3((unsigned)std::min(ctas - t, kGemmMaxGrid)), dim3(kGT), smem, st, p, t, nst,
                          clear);
     clear = nullptr;
-    pdl = true;
   }
   return e;
 }
 
-cudaError_t launch_gemm_group(const GemmGroup& group, bool bf16, bool pdl, cudaStream_t st) {
+cudaError_t launch_gemm_group(const GemmGroup& group, bool bf16, cudaStream_t st) {
   GemmArgs g;
   g.np = 0;
   g.clear = group.clear;
@@ -616,18 +613,16 @@ cudaError_t launch_gemm_group(const GemmGroup& group, bool bf16, bool pdl, cudaS
   ProfScope prof(ASI_K_MODEPROD, st, bytes);
   const bool any = g.np > 0;
   if (any) {
-    const cudaError_t e = launch_narrow(g, bf16, pdl, st);
+    const cudaError_t e = launch_narrow(g, bf16, st);
     if (e != cudaSuccess) return e;
   }
   int* clear = any ? nullptr : group.clear;          // the first launch clears
-  pdl = pdl || any;
   for (int q = 0; q < group.np; ++q) {
     const GemmProb& p = group.p[q];
     if (gemm_narrow(p)) continue;
-    const cudaError_t e = bf16 ? launch_wide<__nv_bfloat16>(p, clear, pdl, st) : launch_wide<float>(p, clear, pdl, st);
+    const cudaError_t e = bf16 ? launch_wide<__nv_bfloat16>(p, clear, st) : launch_wide<float>(p, clear, st);
     if (e != cudaSuccess) return e;
     clear = nullptr;
-    pdl = true;
   }
   return cudaSuccess;
 }

@@ -53,7 +53,7 @@ template <int R, typename TX>
 __global__ void __launch_bounds__(256) k_fiber(FiberArgs p) {
   constexpr int TQ = kFiberTQ, NT = 256, KS = NT / TQ;
   extern __shared__ __align__(16) float fsm[];
-  pass_begin(p.clear);
+  pass_begin(p.clear, p.clear != nullptr);
   const int tid = threadIdx.x, lane = tid & 31;
   const int a = (int)p.a, r = p.r;
   const bool last = p.I == 1;                       // fibers are contiguous
@@ -219,7 +219,7 @@ static cudaError_t launch_fiber_t(const FiberArgs& p, int grid, cudaStream_t st)
   const size_t smem = fiber_smem((int)p.a);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_fiber<R, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.clear, k_fiber<R, TX>, dim3(grid), dim3(256), smem, st, p);
+  return launch_pdl(k_fiber<R, TX>, dim3(grid), dim3(256), smem, st, p);
 }
 
 cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t st) {
@@ -362,7 +362,6 @@ __host__ __device__ static inline int conv_tail_split(int n_out, int n_items) {
 
 __global__ void __launch_bounds__(kTailNT) k_conv_tail(ConvTailArgs p) {
   extern __shared__ float sm[];
-  pdl_launch_dependents();
   pdl_wait();
   const int tid = threadIdx.x;
   const int co = blockIdx.x;
@@ -473,7 +472,6 @@ __global__ void __launch_bounds__(256) k_conv_z4(ConvTailArgs p, float* __restri
 
 __global__ void __launch_bounds__(256) k_conv_dw(ConvTailArgs p, const float* Z4p, int nsp) {
   extern __shared__ float sm[];
-  pdl_launch_dependents();
   pdl_wait();
   const int tid = threadIdx.x;
   const int co = blockIdx.x;

@@ -71,8 +71,8 @@ struct Fiber2Args {
   int ldu, a, r, project_only, nstage;
   int team;            // k_mfiber: warps that share the rows of a tile (set by the launcher)
   int* status;         // status word of the workspace (k_mfiber: an expired wait on a copy)
-  int plain;           // launched after all earlier work of the stream (the first kernel of a call)
-  int* clear;          // as in PlaneArgs (plain launches only)
+  int first;           // the first kernel of a call
+  int* clear;          // as in PlaneArgs (first kernels only)
 };
 
 struct QRMode {
@@ -214,7 +214,7 @@ struct TcSplitArgs {
   int n;
 };
 void tc_add_split(TcSplitArgs* p, const float* U, int64_t K, int n, void* Bt);
-cudaError_t launch_tc_split(TcSplitArgs& p, bool dep, cudaStream_t st);
+cudaError_t launch_tc_split(TcSplitArgs& p, cudaStream_t st);
 struct TcCall {
   const void* X;           // bf16 [O][a][I]
   const void* bt;          // stacked operand of U [a][n] (projection) or of V [O I][n] (expansion)
@@ -224,7 +224,7 @@ struct TcCall {
   int64_t O, a, I, q_per_split;
   int n, nsplit, expand;
 };
-cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st);
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st);
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st);
 cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, int beside, cudaStream_t st);
 cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, int beside, cudaStream_t st);
@@ -262,10 +262,11 @@ struct ProfScope {
 };
 
 #ifdef __CUDACC__
-// Programmatic dependent launch.  A kernel launched with launch_pdl may start (and do whatever does not depend on
-// its predecessor in the stream) once every CTA of the predecessor has passed pdl_launch_dependents() or has
-// exited; pdl_wait() then blocks until the predecessor has finished and its writes are visible.  Without the
-// launch attribute both are no-ops.
+// Programmatic dependent launch.  Every kernel of the path may start (and do whatever does not depend on its predecessor in the
+// stream) once every CTA of the predecessor has passed pdl_launch_dependents() or has exited; pdl_wait() then blocks until
+// the predecessor has finished and its writes are visible.  The first kernel of a call is one too, whatever the caller had
+// on the stream before: all its threads wait first, and only then does it let its dependents start, so that everything
+// behind it finds all older work of the stream finished (its launch hides behind the kernel before: 1 to 2 us a call).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -279,11 +280,11 @@ __device__ __forceinline__ void tc_store_terms(__nv_bfloat16* Bt, int N, int64_t
   Bt[(int64_t)(2 * N + j) * ldb + k] = __float2bfloat16_rn(r1 - __bfloat162float(m));
 }
 
-// A mode pass of Algorithm 1 depends on nothing the passes before it on the stream write.  The first one (clear not
-// null) is launched normally and zeroes the workspace's status block; the others are programmatic dependents that
-// run beside their predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass
-// sees all of them finished.
-__device__ __forceinline__ void pass_begin(int* clear) {
+// A mode pass of Algorithm 1 depends on nothing the passes before it on the stream write.  The first kernel of a call waits
+// for all that is older and (clear not null) zeroes the workspace's status block; the passes behind it run beside their
+// predecessor and call pdl_wait() only before they end, so that the kernel behind the last pass sees all of them finished.
+__device__ __forceinline__ void pass_begin(int* clear, bool first) {
+  if (first) pdl_wait();
   pdl_launch_dependents();
   if (clear && blockIdx.x == 0)
     for (int e = threadIdx.x; e < 256; e += blockDim.x) clear[e] = 0;
@@ -303,14 +304,6 @@ static inline cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
-}
-// a programmatic dependent when `dep`, else an ordinary launch
-template <typename... Params, typename... Args>
-static inline cudaError_t launch_maybe_pdl(bool dep, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
-                                           cudaStream_t st, const Args&... args) {
-  if (dep) return launch_pdl(kernel, grid, block, smem, st, args...);
-  kernel<<<grid, block, smem, st>>>(static_cast<Params>(args)...);
-  return cudaGetLastError();
 }
 #endif
 
@@ -370,7 +363,7 @@ GemmProb gemm_project(const void* X, const float* B, float* Y, int64_t O, int64_
 // Pp[s][k][j] = sum over the columns (o, i) of split s of X[o][k][i] V[(o, i)][j]
 GemmProb gemm_expand(const void* X, const float* V, float* Pp, int64_t O, int64_t a, int64_t I, int n, int nsplit, int64_t kps,
                      bool bf16);
-cudaError_t launch_gemm_group(const GemmGroup& g, bool bf16, bool pdl, cudaStream_t st);
+cudaError_t launch_gemm_group(const GemmGroup& g, bool bf16, cudaStream_t st);
 
 int orth_rows(int64_t a, int r, int64_t nsplit);
 size_t orth_gp_elems(int64_t nchunk, int r);

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kF2Threads, (RW <= 4 && NJ == 4) ? 3 : 2) k_fi
   // a product alone lets its successor start when it ends: the tail kernels that would wait beside a whole traversal take
   // registers and shared memory from the other layers (ResNet-34 sweep, CUDA graph: 781 -> 774 us).  Z1, the first kernel
   // of a weight gradient, has k_z3 behind it, which does not wait for it
-  if (!p.project_only || p.plain) pass_begin(p.clear);
+  if (!p.project_only || p.first) pass_begin(p.clear, p.first);
   if (p.project_only) pdl_wait();                    // its factor comes from the kernel before
   const int tid = threadIdx.x, grp = tid >> 4, lane = tid & 15;
   const int a = p.a, r = p.r, nst = p.nstage;
@@ -321,7 +321,7 @@ template <int RW, int NJ, typename TX>
 static cudaError_t launch_fiber2_t(const Fiber2Args& p, int grid, size_t smem, cudaStream_t st) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_fiber2<RW, NJ, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.plain, k_fiber2<RW, NJ, TX>, dim3(grid), dim3(kF2Threads), smem, st, p);
+  return launch_pdl(k_fiber2<RW, NJ, TX>, dim3(grid), dim3(kF2Threads), smem, st, p);
 }
 
 cudaError_t launch_fiber2(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
   extern __shared__ __align__(128) unsigned char p2_smem[];
   __shared__ __align__(8) uint64_t bars[NST];
   __shared__ int s_fail;
-  pass_begin(p.clear);
+  pass_begin(p.clear, p.clear != nullptr);
   TX* stages = reinterpret_cast<TX*>(p2_smem);                                   // [NST][G][S][S]
   f2* U3d = reinterpret_cast<f2*>(p2_smem + (size_t)NST * kTileBytes);           // [S][4]: (u, u)
   float* U4t = reinterpret_cast<float*>(U3d + S * 4);                            // [4][S]
@@ -612,7 +612,7 @@ static cudaError_t launch_plane2_t(const PlaneArgs& p, int grid, cudaStream_t st
   const size_t smem = plane2_smem(S, sizeof(TX) == 2);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_plane2<S, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.clear, k_plane2<S, TX>, dim3(grid), dim3(kP2Threads), smem, st, p);
+  return launch_pdl(k_plane2<S, TX>, dim3(grid), dim3(kP2Threads), smem, st, p);
 }
 
 cudaError_t launch_plane2(const PlaneArgs& p, int grid, bool bf16, cudaStream_t st) {
@@ -638,7 +638,8 @@ int plane2_grid(int S, int64_t n_planes, int max_ctas) {
 __global__ void __launch_bounds__(256) k_core_tail(CoreTailArgs p) {
   extern __shared__ __align__(16) float ct_smem[];
   __shared__ int s_last;
-  pdl_launch_dependents();
+  // the last kernel of a call lets its successor start when it ends: the CTAs of a weight gradient that came in beside this
+  // kernel's were packed two to an SM with others idle (128 x 128 x 28 x 28 bf16: 28 us became 40)
   pdl_wait();
   const int tid = threadIdx.x;
   const int chunk = blockIdx.x, i = blockIdx.y, cs = blockIdx.z;

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
   constexpr int NV = 4 * NB, VP = TC + 4;            // columns of a factor, row pitch of V
   constexpr uint32_t BLK = (uint32_t)ROWS * 128u, STAGE = CB * BLK;
   extern __shared__ __align__(1024) unsigned char mf_smem[];
-  pass_begin(p.clear);
+  pass_begin(p.clear, p.first);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int g = lane >> 2, c4 = lane & 3;
   const int T = p.team, G = nw / T, team = warp / T, tw = warp - team * T;
@@ -517,7 +517,7 @@ template <int RT, int NB, int CB, int LD, typename TX>
 static cudaError_t launch_mfiber_t(const Fiber2Args& p, const CUtensorMap& map, const MfShape& s, int grid, cudaStream_t st) {
   const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mfiber<RT, NB, CB, LD, TX>), s.smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.plain, k_mfiber<RT, NB, CB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p, map);
+  return launch_pdl(k_mfiber<RT, NB, CB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p, map);
 }
 
 cudaError_t launch_mfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
   constexpr bool EX = sizeof(TX) == 2;
   constexpr int NV = 4 * NB, VP = 36;                // row pitch of V3 and V4: 32 and four
   extern __shared__ __align__(128) unsigned char mp_smem[];
-  pass_begin(p.clear);
+  pass_begin(p.clear, p.clear != nullptr);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int g = lane >> 2, c4 = lane & 3, H = p.H, W = p.W, hw = H * W;
   const int jb = NB == 1 ? (g & 3) : g;
@@ -853,7 +853,7 @@ template <int NB, int LD, typename TX>
 static cudaError_t launch_mplane_t(const PlaneArgs& p, const MpShape& s, int grid, cudaStream_t st) {
   const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mplane<NB, LD, TX>), s.smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.clear, k_mplane<NB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p);
+  return launch_pdl(k_mplane<NB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p);
 }
 
 cudaError_t launch_mplane(const PlaneArgs& p0, int grid, bool bf16, cudaStream_t st) {

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256) k_philox_words(uint64_t seed, uint32_t st
 // One stream per row of the grid: the matrices of a layer's modes in one launch (28 x 28 x 128 x 64, ranks 4: four
 // launches and their gaps took 25 us, this one 6).
 __global__ void __launch_bounds__(256) k_fill_gaussian(uint64_t seed, const __grid_constant__ FillArgs p) {
+  pdl_wait();
   pdl_launch_dependents();
   if (p.clear && blockIdx.x == 0 && blockIdx.y == 0) p.clear[threadIdx.x] = 0;
   const uint32_t stream = p.stream[blockIdx.y];
@@ -85,8 +86,7 @@ cudaError_t launch_fill_gaussian(uint64_t seed, const FillArgs& p, int count, cu
   for (int m = 0; m < count; ++m) n = std::max(n, p.n[m]);
   if (n <= 0) return cudaSuccess;
   const int64_t blocks = std::min<int64_t>(((n + 3) / 4 + 255) / 256, 148 * 8);
-  k_fill_gaussian<<<dim3((unsigned)blocks, (unsigned)count), 256, 0, st>>>(seed, p);
-  return cudaGetLastError();
+  return launch_pdl(k_fill_gaussian, dim3((unsigned)blocks, (unsigned)count), dim3(256), 0, st, seed, p);
 }
 
 }  // namespace asi

@@ -766,6 +766,7 @@ template <int KIND, int R, bool ANY, typename TX>
 __device__ __forceinline__ void sm_pass1_cta(const SmPass1Args& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
   const int tid = threadIdx.x;
+  pdl_wait();                                        // the first kernel of a call
   if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
   const int nc_ctas = (p.B * p.cs + p.cl - 1) / p.cl * p.cl;
   if (bid >= nc_ctas) {
@@ -960,6 +961,7 @@ __device__ __forceinline__ void sm_tile1_cta(const SmTile1Args& p, const int bid
   const TX* __restrict__ A = reinterpret_cast<const TX*>(p.act);
   const int B = p.B, C = p.C;
 
+  pdl_wait();                                        // the first kernel of a call
   if (bid == 0 && tid < 241) p.status[tid == 0 ? 0 : 15 + tid] = 0;  // status word, counters 16..255
 
   constexpr int kNQ = (S == 7) ? 1 : 4;             // role-C CTAs per sample
@@ -2023,6 +2025,7 @@ __device__ __forceinline__ void wgrad_project(const TX* __restrict__ dY, int64_t
 template <int R, int kNT, bool STAGED, typename TX>
 __device__ __forceinline__ void sm_wgrad_cta(const SmWgradArgs& p, const int bid) {
   extern __shared__ __align__(128) float smem[];
+  pdl_wait();                                        // the only kernel of a call
   const int tid = threadIdx.x;
   const int r1 = p.r[0], r2 = p.r[1], r3 = p.r[2], r4 = p.r[3];
   const int H = p.H, W = p.W, HoWo = p.Ho * p.Wo, kk = p.kh * p.kw;
@@ -2273,7 +2276,7 @@ size_t sm_wgrad_smem(const SmWgradArgs& p, int R, bool staged, bool bf16) {
   return 4 * n + 64;
 }
 
-// an ordinary launch, in clusters of cs CTAs
+// a launch in clusters of cs CTAs
 template <typename Arg>
 static cudaError_t launch_clustered(void (*kernel)(Arg), int grid, int cs, size_t smem, cudaStream_t st, const Arg& arg) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
@@ -2283,13 +2286,15 @@ static cudaError_t launch_clustered(void (*kernel)(Arg), int grid, int cs, size_
   cfg.blockDim = dim3(kPT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cs;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cs;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = cs > 1 ? 1 : 0;
+  cfg.numAttrs = cs > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
 static int pass1_grid(const SmPass1Args& p) {
@@ -2352,8 +2357,7 @@ static cudaError_t launch_wgrad_t(const SmWgradArgs& p, int beside, cudaStream_t
   auto kernel = staged ? k_sm_wgrad_staged<R, TX> : (p.nt == 512 ? k_sm_wgrad<R, 512, TX> : k_sm_wgrad<R, 256, TX>);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  kernel<<<p.Cout / p.cpb, staged ? kTT : p.nt, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3(p.Cout / p.cpb), dim3(staged ? kTT : p.nt), smem, st, p);
 }
 
 template <int S, int R, typename TX>
@@ -2362,15 +2366,13 @@ static cudaError_t launch_tile1_t(const SmTile1Args& p, cudaStream_t st) {
   auto kernel = p.aligned ? k_sm_tile1<S, R, false, TX> : k_sm_tile1<S, R, true, TX>;
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  kernel<<<p.n_tiles_b + sm_tile1_role_c_ctas(S, p.B), kTT, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3(p.n_tiles_b + sm_tile1_role_c_ctas(S, p.B)), dim3(kTT), smem, st, p);
 }
 template <int S, int R, typename TX>
 static cudaError_t launch_tile1_bt(const SmBatch<SmTile1Args>& b, size_t smem, cudaStream_t st) {
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_sm_tile1_b<S, R, TX>), smem);
   if (e != cudaSuccess) return e;
-  k_sm_tile1_b<S, R, TX><<<b.first[b.n], kTT, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_pdl(k_sm_tile1_b<S, R, TX>, dim3(b.first[b.n]), dim3(kTT), smem, st, b);
 }
 
 // FN<kind, R, TX> and FN<R, TX> for the plan's variant
@@ -2460,8 +2462,7 @@ static cudaError_t launch_wgrad_bt(const SmBatch<SmWgradArgs>& b, size_t smem, b
   auto kernel = staged ? k_sm_wgrad_staged_b<R, TX> : (b.a[0].nt == 512 ? k_sm_wgrad_b<R, 512, TX> : k_sm_wgrad_b<R, 256, TX>);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  kernel<<<b.first[b.n], staged ? kTT : b.a[0].nt, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3(b.first[b.n]), dim3(staged ? kTT : b.a[0].nt), smem, st, b);
 }
 
 cudaError_t launch_sm_tile1_batched(const SmTile1Args* a, int n, int S, int R, bool bf16, cudaStream_t st) {

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wfiber(const __grid_cons
   constexpr int TC = wf_cols<TX>(RK), PT = TC + 4, NP = TC / 2, KQ = 32 / NP, UP = 12;
   constexpr int KB = 8, KS = KQ == 4 ? 2 : KQ;       // rows per step of the column pass, between a lane's rows
   extern __shared__ __align__(16) unsigned char ws_smem[];
-  if (!p.project_only || p.plain) pass_begin(p.clear);   // a product alone: its successor starts when it ends (see k_fiber2)
+  if (!p.project_only || p.first) pass_begin(p.clear, p.first);   // a product alone: its successor starts when it ends (see k_fiber2)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int a = p.a, r = p.r, a8 = (a + 7) & ~7;
   float* Ud = reinterpret_cast<float*>(ws_smem);     // [a8][UP]: rows >= a and columns >= r zero; rows 1, 4 and 5 apart are bank-disjoint
@@ -327,7 +327,7 @@ int wf_warps(int64_t tiles, int a, int R, bool bf16) {
 template <int R, bool VEC, typename TX>
 __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_constant__ PlaneArgs p) {
   extern __shared__ __align__(16) unsigned char ws_smem[];
-  pass_begin(p.clear);
+  pass_begin(p.clear, p.clear != nullptr);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int H = p.H, W = p.W, np = p.np, PT = p.pitch, W2 = (W + 1) >> 1, W4 = (W + 3) >> 2, H2 = (H + 1) >> 1;
   const int nsc = p.nsc, nsr = p.nsr;
@@ -563,7 +563,7 @@ cudaError_t wfiber_t(const Fiber2Args& p, int grid, cudaStream_t st) {
   const size_t smem = wf_fixed_bytes(p.a) + nw * wf_warp_bytes(p.a, R, RK, bf16);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_wfiber<R, RK, VEC, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(!p.plain, k_wfiber<R, RK, VEC, TX>, dim3(grid), dim3(32 * nw), smem, st, p);
+  return launch_pdl(k_wfiber<R, RK, VEC, TX>, dim3(grid), dim3(32 * nw), smem, st, p);
 }
 template <int R, int RK>
 cudaError_t wfiber_x(const Fiber2Args& p, int grid, bool bf16, bool vec, cudaStream_t st) {
@@ -585,7 +585,7 @@ cudaError_t wplane_t(const PlaneArgs& p, int grid, cudaStream_t st) {
   const size_t smem = wp_fixed_bytes(p.H, p.pitch, R) + nw * wp_warp_bytes(p.H, p.np, p.pitch, R, bf16);
   cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_wplane<R, VEC, TX>), smem);
   if (e != cudaSuccess) return e;
-  return launch_maybe_pdl(p.clear == nullptr, k_wplane<R, VEC, TX>, dim3(grid), dim3(32 * nw), smem, st, p);
+  return launch_pdl(k_wplane<R, VEC, TX>, dim3(grid), dim3(32 * nw), smem, st, p);
 }
 template <int R>
 cudaError_t wplane_r(const PlaneArgs& p, int grid, bool bf16, bool vec, cudaStream_t st) {

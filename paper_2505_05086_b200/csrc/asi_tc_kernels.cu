@@ -139,8 +139,8 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {   /
 // of the call in one launch
 __global__ void __launch_bounds__(256) k_tc_split(const __grid_constant__ TcSplitArgs p) {
   __shared__ float tile[32][33];
+  pdl_wait();                                        // often the first kernel of a call: its dependents start behind all older work
   pdl_launch_dependents();
-  pdl_wait();
   if (p.clear && blockIdx.x == 0) p.clear[threadIdx.x] = 0;
   int q = 0;
   while (q + 1 < p.n && (int)blockIdx.x >= p.m[q + 1].first) ++q;
@@ -514,18 +514,18 @@ void tc_add_split(TcSplitArgs* p, const float* U, int64_t K, int n, void* Bt) {
   m.ldb = pad64(K);
 }
 
-cudaError_t launch_tc_split(TcSplitArgs& p, bool dep, cudaStream_t st) {
+cudaError_t launch_tc_split(TcSplitArgs& p, cudaStream_t st) {
   int first = 0;
   for (int q = 0; q < p.n; ++q) {
     p.m[q].first = first;
     first += ((p.m[q].K + 31) / 32) * ((p.m[q].N + 31) / 32);
   }
-  return launch_maybe_pdl(dep, k_tc_split, dim3((unsigned)first), dim3(256), 0, st, p);
+  return launch_pdl(k_tc_split, dim3((unsigned)first), dim3(256), 0, st, p);
 }
 
 // One launch over the products of `c` (all with operands already split).  cudaErrorNotSupported: a tensor map could
 // not be made (nothing was launched).
-cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaStream_t st) {
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st) {
   if (n < 1 || n > 3) return cudaErrorInvalidValue;
   TcGroup g;
   g.np = n;
@@ -628,11 +628,9 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, bool dep, cudaS
     at[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (dep) {
-    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
+  at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[na].val.programmaticStreamSerializationAllowed = 1;
+  ++na;
   cfg.attrs = at;
   cfg.numAttrs = na;
   return cudaLaunchKernelEx(&cfg, k_tc_group, g);
