@@ -12,11 +12,13 @@
 // 25.7 M values, where the register form needs 5.5).
 //
 // fp32 on tf32: x = hi + lo, hi the upper 19 bits of x -- which is all the unit reads, so x itself is the operand -- and lo the
-// exact rest, of which the unit reads eleven bits.  A factor is split at its nearest tf32 value instead, both parts exact to 24
-// bits: the eight columns of the B operand are (hi | lo) of up to four factor columns, or with NB = 2 two operands of up to
-// eight.  The unit's own sums truncate, so it never adds more than two steps of the leading term (16 products) before the
-// sum goes to a register in round-to-nearest; the small terms go first.  bf16 values are exact in tf32.  Against 64 bits the
-// factors of 48 drawn and listed layers come out with the fp32 kernels' errors (3.5e-8, 2.5e-8 of it the rounding of the output).
+// exact rest, of which the unit reads eleven bits.  A factor is split at its nearest tf32 value instead and its rest rounded
+// to the nearest one, because its error is the same for every column of the activation and does not average out.  The eight
+// columns of the B operand are (hi | lo) of up to four factor columns, or with NB = 2 two operands of up to eight.  The
+// unit's own sums truncate, so it never adds more than two steps of the leading term (16 products) before the sum goes to a
+// register in round-to-nearest; the small terms go first.  bf16 values are exact in tf32.  Against 64 bits, 72 drawn and listed
+// conv layers (the fp32 pipe in parentheses): worst factor 3.76e-8 (3.78e-8), core 6.9e-8 (7.4e-8), gradient 2.38e-7 (2.38e-7); the
+// batch mode's factor alone 2.76e-8 (2.69e-8), 2.4e-8 of it the rounding of the output.
 //
 // The k order of an operand is free as long as both sides agree, and so is the order of rows: a lane takes four (bf16:
 // eight) neighbouring columns by one 16-byte read, as four m-tiles' rows in one product and four k-steps in the other.
@@ -148,7 +150,7 @@ struct Acc {
 // one entry of the B operand of the columns: lane group g is the column
 template <int NB>
 __device__ __forceinline__ void set_b(float* b, int half, int g, float x) {
-  const float hi = nearest(x), lo = x - hi;
+  const float hi = nearest(x), lo = nearest(x - hi);
   if constexpr (NB == 1) b[half] = g < 4 ? hi : lo;
   else {
     b[half] = hi;

@@ -64,3 +64,26 @@ def test_any_element_address(dims, ranks):
     for o in out[1:]:
         for x, y in zip(o, out[0]):
             assert float((x - y).norm() / y.norm()) <= 1e-5
+
+
+TOKENS = [  # (dims, ranks, cout, bf16): batches on both sides of the rule's line and of a tile
+    ((8, 40, 128), (4, 12, 16), 24, True),
+    ((9, 40, 128), (8, 12, 16), 24, True),
+    ((17, 33, 96), (4, 8, 12), 20, False),
+    ((33, 24, 130), (7, 8, 12), 20, False),        # rows off 16 bytes
+    ((130, 24, 64), (5, 8, 8), 20, False),         # three warps a tile
+]
+
+
+@pytest.mark.parametrize("dims,ranks,cout,bf16", TOKENS)
+def test_batch_mode_of_token_layers(dims, ranks, cout, bf16):
+    rho = tuple(min(0.95, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "linear", dims, cout, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, 2 * r) for d, r in zip(dims, ranks)))
+    run = make_runner(L, bf16=bf16)
+    U_prev = st.u_prev0()
+    for t in range(2):
+        A, dY = st.next()
+        err, U_prev = compare_step(run, L, A, dY, U_prev)
+        check(err, TOL_F32, str(dims))
