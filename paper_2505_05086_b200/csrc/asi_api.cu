@@ -766,11 +766,15 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
                      pl->q_per_split[m], pl->bf16);
 }
 
-// cold start: P_m = A_m Omega_m of all modes, one launch of SIMT products and one of tensor-core products.
-// clear: the first launch here zeroes the status block
-asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool clear,
+// cold start: P_m = A_m Omega_m of all modes: one launch of SIMT products, one of tensor-core products, and the passes of the
+// modes that a warm step has on k_mfiber and k_mplane, which take Omega as their V (64 x 128 x 28 x 28 fp32, ranks 4: 72.1 -> 55.7 us).
+// first: nothing of this call is enqueued yet; the first launch here zeroes the status block
+asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool first,
                           cudaStream_t st) {
   int* const status = reinterpret_cast<int*>(w);
+  bool clear = first;
+  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0, mma = !pl->bf16 || on16;
+  const bool planes = pl->mplane && mma;
   GemmGroup g;
   g.np = 0;
   TcSplitArgs sp;
@@ -778,7 +782,8 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
   TcCall t[3];
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
-    if (pl->tc_mode[m] && (reinterpret_cast<uintptr_t>(act) & 15u) == 0) {
+    if ((pl->mfiber[m] && mma) || (planes && m >= 2)) continue;
+    if (pl->tc_mode[m] && on16) {
       t[sp.n] = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
                  pl->q_per_split[m], v.r, pl->nsplit[m], 1};
       tc_add_split(&sp, omega[m], v.Q, v.r, w + pl->tcv_off[m]);
@@ -787,9 +792,45 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     }
   }
   g.clear = clear ? status : nullptr;
+  bool head = true;                                  // the first launch here waits for Omega; those behind it find it there
   if (g.np) {
     ASI_CUDA(launch_gemm_group(g, pl->bf16, st));
-    clear = false;
+    clear = head = false;
+  }
+  if (planes) {
+    PlaneArgs a{};
+    a.X = act;
+    a.U3 = omega[2];
+    a.U4 = omega[3];
+    a.Pp3 = reinterpret_cast<float*>(w + pl->off_Pp[2]);
+    a.Pp4 = reinterpret_cast<float*>(w + pl->off_Pp[3]);
+    a.n_planes = pl->dims[0] * pl->dims[1];
+    a.H = (int)pl->dims[2];
+    a.W = (int)pl->dims[3];
+    a.r3 = pl->r[2];
+    a.r4 = pl->r[3];
+    a.status = status;
+    a.given = 1;
+    a.first = head;
+    a.clear = clear ? status : nullptr;
+    ASI_CUDA(launch_mplane(a, pl->plane_grid, pl->bf16, st));
+    clear = head = false;
+  }
+  for (int m = 0; m < pl->nd; ++m) {
+    if (!pl->mfiber[m] || !mma) continue;
+    const ModeView& v = pl->mv[m];
+    Fiber2Args f;
+    std::memset(&f, 0, sizeof(f));
+    f.X = act;
+    f.U = omega[m];
+    f.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
+    f.O = v.O; f.I = v.I; f.a = (int)v.a; f.r = v.r;
+    f.status = status;
+    f.given = 1;
+    f.first = head;
+    f.clear = clear ? status : nullptr;
+    ASI_CUDA(launch_mfiber(f, pl->fiber_grid[m], pl->bf16, st));
+    clear = head = false;
   }
   if (sp.n) {
     sp.clear = clear ? status : nullptr;
@@ -1030,6 +1071,7 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     g.r3 = pl->r[2];
     g.r4 = pl->r[3];
     g.status = status;
+    g.first = first;
     g.clear = take_clear();
     const bool mma = pl->mplane && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);   // else: odd bf16 addresses
     if (mma) ASI_CUDA(launch_mplane(g, pl->plane_grid, pl->bf16, st));

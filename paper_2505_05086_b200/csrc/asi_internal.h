@@ -55,8 +55,10 @@ struct PlaneArgs {
   int64_t n_planes;
   int S, H, W, r3, r4;
   int np, pitch, nsc, nsr;   // planes per tile, row pitch, lanes per column pair and row (set by the launcher)
+  int first = 0;           // the first kernel of a call
+  int given = 0;           // k_mplane: U3 and U4 are Omega_3 [planes W][r3] and Omega_4 [planes H][r4], and P_m = A_m Omega_m
   int* clear = nullptr;    // not null: CTA 0 zeroes the 256 ints of the workspace's status block
-  int* status = nullptr;   // status word of the workspace (k_plane2: an expired wait on the bulk copy)
+  int* status = nullptr;   // status word of the workspace (an expired wait on a bulk copy)
 };
 
 // One mode with strided fibers, a <= 128, r <= 4 (k_fiber2): both products in one pass, or with
@@ -69,6 +71,7 @@ struct Fiber2Args {
   int64_t y_so, y_sj;
   int64_t O, I, n_tiles;
   int ldu, a, r, project_only, nstage;
+  int given;           // k_mfiber: U is Omega [O I][r], and P = A Omega
   int team;            // k_mfiber: warps that share the rows of a tile (set by the launcher)
   int* status;         // status word of the workspace (k_mfiber: an expired wait on a copy)
   int first;           // the first kernel of a call

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
   extern __shared__ __align__(128) unsigned char p2_smem[];
   __shared__ __align__(8) uint64_t bars[NST];
   __shared__ int s_fail;
-  pass_begin(p.clear, p.clear != nullptr);
+  pass_begin(p.clear, p.first);
   TX* stages = reinterpret_cast<TX*>(p2_smem);                                   // [NST][G][S][S]
   f2* U3d = reinterpret_cast<f2*>(p2_smem + (size_t)NST * kTileBytes);           // [S][4]: (u, u)
   float* U4t = reinterpret_cast<float*>(U3d + S * 4);                            // [4][S]

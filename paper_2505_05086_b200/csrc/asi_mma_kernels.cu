@@ -232,9 +232,9 @@ constexpr int kMfThreads = 192;
 // k_mfiber.  A team of T warps takes the same columns; warp w of it owns the rows [16 RT w, 16 RT (w + 1)) and fills and
 // empties its own two buffers of them, [CB blocks][16 RT rows][128 bytes], each block 8 EPL columns wide with its 16-byte
 // units swizzled by the row (TMA's 128-byte pattern).  The warps of a team meet once a tile, for the sum of their shares
-// of V.
+// of V.  GIVEN (a cold start, P = A_m Omega): V is Omega, [Q][r] in memory, and comes with the tile.
 // ---------------------------------------------------------------------------------------------
-template <int RT, int NB, int CB, int LD, typename TX>
+template <int RT, int NB, int CB, int LD, bool GIVEN, typename TX>
 __global__ void __launch_bounds__(kMfThreads, 2)
     k_mfiber(const __grid_constant__ Fiber2Args p, const __grid_constant__ CUtensorMap map) {
   constexpr bool EX = sizeof(TX) == 2;
@@ -284,19 +284,36 @@ __global__ void __launch_bounds__(kMfThreads, 2)
         }
       }
     }
-    if constexpr (LD == 1) cp_commit();
+    if constexpr (GIVEN) {                           // the team's warps share the copy of V
+      if (t_ld < total) {
+        const int64_t i0 = (int64_t)i_ld * TC;
+        const float* src = p.U + ((int64_t)o_ld * p.I + i0) * r;
+        const uint32_t d = s_addr(Vt + st * T * (NV * VP));
+        const int n = (int)(p.I - i0 < TC ? p.I - i0 : TC) * r;
+        for (int e = 32 * tw + lane; e < TC * r; e += 32 * T) {
+          const int q = e / r, j = e - q * r;
+          cp_one(d + 4 * (j * VP + q), src + (e < n ? e : 0), e < n);
+        }
+      }
+    }
+    if constexpr (LD == 1 || GIVEN) cp_commit();
     t_ld += stride;
     o_ld += d_o;
     i_ld += d_i;
     if (i_ld >= nti) { i_ld -= nti; ++o_ld; }
   };
   const int t_first = t_ld;
+  if constexpr (GIVEN) {
+    for (int e = lane; e < 2 * NV * VP; e += 32) Vt[tw * 2 * NV * VP + e] = 0.f;   // columns past r
+    if (T > 1) bar_team(1 + team, 32 * T);
+    else __syncwarp();
+  }
   fill(0);
   fill(1);
   // the factor: step s, slots c4 and c4 + 4 are rows 8 s + 2 c4 and the next one
   float ub[2 * RT][2 * NB];
 #pragma unroll
-  for (int s = 0; s < 2 * RT; ++s)
+  for (int s = 0; s < 2 * RT && !GIVEN; ++s)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = row0 + 8 * s + 2 * c4 + h, j = NB == 1 ? (g & 3) : g;
@@ -322,15 +339,14 @@ __global__ void __launch_bounds__(kMfThreads, 2)
         atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
       }
       phase ^= 1u << st;
-    } else {
-      cp_wait1();
     }
+    if constexpr (LD == 1 || GIVEN) cp_wait1();
     __syncwarp();
     const unsigned char* xs = buf + st * STAGE;
     float* Vw = Vt + (vb * T + tw) * (NV * VP);
     // ---- V of this warp's rows
 #pragma unroll
-    for (int cb = 0; cb < CB; ++cb) {
+    for (int cb = 0; cb < CB && !GIVEN; ++cb) {
       Acc<NB, EX> v2[NMT];
 #pragma unroll
       for (int m = 0; m < NMT; ++m) v2[m].zero();
@@ -397,7 +413,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
             const float* src = Vr + (NB == 1 ? (g & 3) : g) * VP + cb * TCB + h * (TCB / 2) + c4 * EPL + u;
             float x[4];
             ld_vals(src, x);
-            for (int w = 1; w < T; ++w) {
+            for (int w = 1; w < T && !GIVEN; ++w) {
               float y[4];
               ld_vals(src + w * (NV * VP), y);
 #pragma unroll
@@ -428,9 +444,11 @@ __global__ void __launch_bounds__(kMfThreads, 2)
         }
       }
     }
-    __syncwarp();                                    // the stage has been read by all lanes
+    // the stage has been read by all lanes (its V by the team)
+    if (GIVEN && T > 1) bar_team(1 + team, 32 * T);
+    else __syncwarp();
     if (!failed) fill(st);
-    else { t_ld += stride; if constexpr (LD == 1) cp_commit(); }
+    else { t_ld += stride; if constexpr (LD == 1 || GIVEN) cp_commit(); }
     st ^= 1;
     vb ^= 1;
     if (T == 1) __syncwarp();
@@ -515,11 +533,17 @@ int mfiber_grid(int64_t O, int64_t a, int64_t I, int r, bool bf16, bool share_sm
   return (int)std::min<int64_t>((tiles + g - 1) / g, 148 * per_sm);
 }
 
+template <int RT, int NB, int CB, int LD, bool GIVEN, typename TX>
+static cudaError_t launch_mfiber_tg(const Fiber2Args& p, const CUtensorMap& map, const MfShape& s, int grid, cudaStream_t st) {
+  const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mfiber<RT, NB, CB, LD, GIVEN, TX>), s.smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_mfiber<RT, NB, CB, LD, GIVEN, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p, map);
+}
+
 template <int RT, int NB, int CB, int LD, typename TX>
 static cudaError_t launch_mfiber_t(const Fiber2Args& p, const CUtensorMap& map, const MfShape& s, int grid, cudaStream_t st) {
-  const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mfiber<RT, NB, CB, LD, TX>), s.smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_mfiber<RT, NB, CB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p, map);
+  return p.given ? launch_mfiber_tg<RT, NB, CB, LD, true, TX>(p, map, s, grid, st)
+                 : launch_mfiber_tg<RT, NB, CB, LD, false, TX>(p, map, s, grid, st);
 }
 
 cudaError_t launch_mfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_t st) {
@@ -568,25 +592,27 @@ cudaError_t launch_mfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_
 //   2 rows     V4[h][j] = sum_w X[h][w] U4[w][j] and P3[h][j] += sum_w X[h][w] V3[w][j], on the same fragments
 //   3 columns  P4[w][j] += sum_h X[h][w] V4[h][j]
 // The factors and the sums P3, P4 stay in registers.  Rows beyond the plane are zeros of the buffer; columns beyond a row are
-// its neighbour's values and meet a zero of the factor, or make sums nobody reads.
+// its neighbour's values and meet a zero of the factor, or make sums nobody reads.  GIVEN (a cold start): V3 and V4 are the
+// planes' rows of Omega_3 and Omega_4 and come with the plane.
 // ---------------------------------------------------------------------------------------------
 constexpr int kMpThreads = 192;
 
-template <int NB, int LD, typename TX>
+template <int NB, int LD, bool GIVEN, typename TX>
 __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant__ PlaneArgs p) {
   constexpr bool EX = sizeof(TX) == 2;
   constexpr int NV = 4 * NB, VP = 36;                // row pitch of V3 and V4: 32 and four
   extern __shared__ __align__(128) unsigned char mp_smem[];
-  pass_begin(p.clear, p.clear != nullptr);
+  pass_begin(p.clear, p.first);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int g = lane >> 2, c4 = lane & 3, H = p.H, W = p.W, hw = H * W;
   const int jb = NB == 1 ? (g & 3) : g;
   const int pb = p.pitch;                            // bytes of a buffer
   unsigned char* buf = mp_smem + (size_t)warp * (2 * pb);
-  float* V3 = reinterpret_cast<float*>(mp_smem + (size_t)nw * 2 * pb) + warp * (2 * NV * VP);     // [NV][VP]
-  float* V4 = V3 + NV * VP;                                                                       // [NV][VP]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(mp_smem + (size_t)nw * 2 * pb + (size_t)nw * 2 * NV * VP * 4) + 2 * warp;
+  float* V3 = reinterpret_cast<float*>(mp_smem + (size_t)nw * 2 * pb) + warp * (4 * NV * VP);     // [2][NV][VP] (GIVEN: per buffer)
+  float* V4 = V3 + 2 * NV * VP;                                                                   // [2][NV][VP]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(mp_smem + (size_t)nw * 2 * pb + (size_t)nw * 4 * NV * VP * 4) + 2 * warp;
   for (int e = lane; e < 2 * pb / 16; e += 32) reinterpret_cast<uint4*>(buf)[e] = make_uint4(0, 0, 0, 0);
+  for (int e = lane; e < 4 * NV * VP; e += 32) V3[e] = 0.f;
   if (LD == 0 && lane < 2) {
     mbar_init(bars + lane);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -609,8 +635,14 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll 8
         for (int e = lane; e < hw; e += 32) cp_one(d + 4 * e, src + e, true);
       }
+      if constexpr (GIVEN) {
+        const uint32_t d3 = s_addr(V3 + st * NV * VP), d4 = s_addr(V4 + st * NV * VP);
+        const float *s3 = p.U3 + t_ld * W * p.r3, *s4 = p.U4 + t_ld * H * p.r4;
+        for (int e = lane; e < W * p.r3; e += 32) cp_one(d3 + 4 * ((e % p.r3) * VP + e / p.r3), s3 + e, true);
+        for (int e = lane; e < H * p.r4; e += 32) cp_one(d4 + 4 * ((e % p.r4) * VP + e / p.r4), s4 + e, true);
+      }
     }
-    if constexpr (LD == 1) cp_commit();
+    if constexpr (LD == 1 || GIVEN) cp_commit();
     t_ld += stride;
   };
   const int64_t t_first = t_ld;
@@ -626,7 +658,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
   auto wrow = [&](int h, int e) { return LD == 0 ? 16 * h + 4 * c4 + e : 8 * e + 4 * h + c4; };
   float u3[4][2 * NB], u4[4][2 * NB];
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+  for (int s = 0; s < 4 && !GIVEN; ++s)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = 8 * s + (h ? kr1 : kr0), w = wrow(h, s);
@@ -680,13 +712,13 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
         atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
       }
       phase ^= 1u << st;
-    } else {
-      cp_wait1();
     }
+    if constexpr (LD == 1 || GIVEN) cp_wait1();
     __syncwarp();
     const TX* xs = reinterpret_cast<const TX*>(buf + st * pb);
+    const float *W3 = V3 + (GIVEN ? st * NV * VP : 0), *W4 = V4 + (GIVEN ? st * NV * VP : 0);
     // ---- 1: V3
-    {
+    if constexpr (!GIVEN) {
       Acc<NB, EX> v2[2];
       v2[0].zero();
       v2[1].zero();
@@ -726,7 +758,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) set_b<NB>(b3[e], h, g, wrow(h, e) < W ? V3[jb * VP + wrow(h, e)] : 0.f);
+        for (int e = 0; e < 4; ++e) set_b<NB>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         if (m >= nkh) break;
@@ -746,23 +778,25 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
             x00.put(f[h], 0, e + h); x10.put(f[h], 1, e + h);
             x01.put(f[h], 2, e + h); x11.put(f[h], 3, e + h);
           }
-          v2.two(f[0], f[1], u4[e], u4[e + 1]);
+          if constexpr (!GIVEN) v2.two(f[0], f[1], u4[e], u4[e + 1]);
           P3[m].two(f[0], f[1], b3[e], b3[e + 1]);
         }
-        float v[4];
+        if constexpr (!GIVEN) {
+          float v[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          v[i] = v2.s[i];
-          if constexpr (NB == 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 2);
-        }
-        if constexpr (NB == 1) {
-          float* d = V4 + (2 * (c4 & 1) + (c4 >> 1)) * VP;
-          d[ra] = (c4 & 2) ? v[1] : v[0];
-          d[rb] = (c4 & 2) ? v[3] : v[2];
-        } else {
-          float* d = V4 + 2 * c4 * VP;
-          d[ra] = v[0]; d[VP + ra] = v[1];
-          d[rb] = v[2]; d[VP + rb] = v[3];
+          for (int i = 0; i < 4; ++i) {
+            v[i] = v2.s[i];
+            if constexpr (NB == 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 2);
+          }
+          if constexpr (NB == 1) {
+            float* d = V4 + (2 * (c4 & 1) + (c4 >> 1)) * VP;
+            d[ra] = (c4 & 2) ? v[1] : v[0];
+            d[rb] = (c4 & 2) ? v[3] : v[2];
+          } else {
+            float* d = V4 + 2 * c4 * VP;
+            d[ra] = v[0]; d[VP + ra] = v[1];
+            d[rb] = v[2]; d[VP + rb] = v[3];
+          }
         }
       }
     }
@@ -774,14 +808,14 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
       float b4[2][2 * NB];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        set_b<NB>(b4[h], 0, g, V4[jb * VP + 8 * (2 * s2 + h) + kr0]);
-        set_b<NB>(b4[h], 1, g, V4[jb * VP + 8 * (2 * s2 + h) + kr1]);
+        set_b<NB>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
+        set_b<NB>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
       }
       col_steps(xs, s2, b4[0], b4[1], P4);
     }
     __syncwarp();                                    // the buffer has been read by all lanes
     if (!failed) fill(st);
-    else { t_ld += stride; if constexpr (LD == 1) cp_commit(); }
+    else { t_ld += stride; if constexpr (LD == 1 || GIVEN) cp_commit(); }
     st ^= 1;
   }
   if (tid == 0) pdl_wait();
@@ -832,7 +866,7 @@ MpShape mp_shape(int H, int W, int r, bool bf16) {
   MpShape s;
   const int nv = r <= 4 ? 4 : 8;
   s.pb = ((((H + 15) / 16 * 16) * W + 32) * (bf16 ? 2 : 4) + 127) / 128 * 128;
-  const size_t warp = std::max((size_t)2 * s.pb + (size_t)2 * nv * 36 * 4 + 16, (size_t)2 * 32 * nv * 4);   // the epilogue reuses the buffers
+  const size_t warp = std::max((size_t)2 * s.pb + (size_t)4 * nv * 36 * 4 + 16, (size_t)2 * 32 * nv * 4);   // the epilogue reuses the buffers
   s.nw = std::min((int)((112 * 1024) / warp), kMpThreads / 32);
   s.smem = warp * s.nw;
   return s;
@@ -851,11 +885,16 @@ int mplane_grid(int64_t n_planes, int H, int W, int r, bool bf16, bool share_sm)
   return (int)std::min<int64_t>((n_planes + s.nw - 1) / s.nw, 148 * (share_sm ? 1 : 2));
 }
 
+template <int NB, int LD, bool GIVEN, typename TX>
+static cudaError_t launch_mplane_tg(const PlaneArgs& p, const MpShape& s, int grid, cudaStream_t st) {
+  const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mplane<NB, LD, GIVEN, TX>), s.smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_mplane<NB, LD, GIVEN, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p);
+}
+
 template <int NB, int LD, typename TX>
 static cudaError_t launch_mplane_t(const PlaneArgs& p, const MpShape& s, int grid, cudaStream_t st) {
-  const cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_mplane<NB, LD, TX>), s.smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_mplane<NB, LD, TX>, dim3(grid), dim3(32 * s.nw), s.smem, st, p);
+  return p.given ? launch_mplane_tg<NB, LD, true, TX>(p, s, grid, st) : launch_mplane_tg<NB, LD, false, TX>(p, s, grid, st);
 }
 
 cudaError_t launch_mplane(const PlaneArgs& p0, int grid, bool bf16, cudaStream_t st) {

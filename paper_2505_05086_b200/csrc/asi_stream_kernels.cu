@@ -327,7 +327,7 @@ int wf_warps(int64_t tiles, int a, int R, bool bf16) {
 template <int R, bool VEC, typename TX>
 __global__ void __launch_bounds__(32 * kWMaxWarps, 1) k_wplane(const __grid_constant__ PlaneArgs p) {
   extern __shared__ __align__(16) unsigned char ws_smem[];
-  pass_begin(p.clear, p.clear != nullptr);
+  pass_begin(p.clear, p.first);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int H = p.H, W = p.W, np = p.np, PT = p.pitch, W2 = (W + 1) >> 1, W4 = (W + 3) >> 2, H2 = (H + 1) >> 1;
   const int nsc = p.nsc, nsr = p.nsr;

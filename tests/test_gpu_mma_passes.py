@@ -6,6 +6,7 @@ import torch
 
 from asi_inputs.configs import LayerSpec
 from asi_inputs.generator import LayerStream
+from oracle import asi_oracle as O
 from tests.gpu_util import TOL_F32, check, compare_step, make_runner
 
 pytestmark = pytest.mark.gpu
@@ -87,3 +88,24 @@ def test_batch_mode_of_token_layers(dims, ranks, cout, bf16):
         A, dY = st.next()
         err, U_prev = compare_step(run, L, A, dY, U_prev)
         check(err, TOL_F32, str(dims))
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", [c for c in CASES if c[0][0] >= 6])
+def test_cold_start_passes(dims, ranks, bf16):
+    """P_m = A_m Omega_m by the same passes, Omega in place of V (1e-4 as everywhere; the spectra keep the iterate's condition
+    number below a hundred)."""
+    rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(dims, ranks)))
+    A, _ = st.next()
+    rng = np.random.default_rng(5)
+    n = int(np.prod(dims))
+    Omega = [rng.standard_normal((n // d, r)).astype(np.float32) for d, r in zip(dims, ranks)]
+    run = make_runner(L, bf16=bf16)
+    run.init_factors(run.to_device(A), torch.from_numpy(np.concatenate([o.ravel() for o in Omega])).cuda())
+    assert run.ok()
+    S_ref, U_ref = O.asi_cold_start(A.astype(np.float64), [o.astype(np.float64) for o in Omega])
+    U = run.factors()
+    assert max(O.rel_fro(O.projector(a), O.projector(b)) for a, b in zip(U, U_ref)) <= 1e-4
+    assert O.rel_fro(O.sign_align(run.core_np(), U, U_ref)[0], S_ref) <= 1e-4
