@@ -36,16 +36,17 @@ constexpr int kMaxPacked = 136 * 16;     // packed upper triangle of a 64 x 64 m
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void named_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
-// element (i, k), k >= i, of the packed 4 x 4 blocks of an upper triangle with nb block rows
+// element (i, k), k >= i, of an upper triangle in 4 x 4 blocks, nb block rows: the blocks' elements of one place lie side by side, so
+// that threads with neighbouring blocks write them without bank conflicts
 __device__ __forceinline__ int packed_at(int i, int k, int nb) {
   const int bi = i >> 2, bk = k >> 2;
-  return (bi * nb - bi * (bi - 1) / 2 + bk - bi) * 16 + (i & 3) * 4 + (k & 3);
+  return ((i & 3) * 4 + (k & 3)) * (nb * (nb + 1) / 2) + bi * nb - bi * (bi - 1) / 2 + bk - bi;
 }
 
 // G = R^T R and Y = R^{-T} by one elimination on an r x r array T (ranks up to 16 NX): entries k >= i start as G,
 // the rest as zero; row i of Y takes the place of the entries k <= i.  Update thread (ti, tj) keeps
 // T[ti + 16 x][tj + 16 y] in registers and hands the four pivot rows of the next step over in Prow [4][64]; pivot
-// thread k solves column k of them and hands rows of R and Y back in W[step & 1] [64][4].  Y goes to Yg (row-major,
+// thread k solves column k of them and hands rows of R and Y back in W[step & 1] [4][64].  Y goes to Yg (row-major,
 // zero above the diagonal).
 template <int NX>
 __device__ __forceinline__ void eliminate(const double* Gq, double* Prow, double* W, double floor_d, int r,
@@ -84,9 +85,9 @@ __device__ __forceinline__ void eliminate(const double* Gq, double* Prow, double
           for (int k = i; k < 4; ++k) D[i][k] = fma(-D[c][i], D[c][k], D[i][k]);
         }
       }
-      double* Wp = W + ((p0 >> 2) & 1) * (4 * kQRMaxRank) + tid * 4;
-      *reinterpret_cast<double2*>(Wp) = make_double2(w[0], w[1]);
-      *reinterpret_cast<double2*>(Wp + 2) = make_double2(w[2], w[3]);
+      double* Wp = W + ((p0 >> 2) & 1) * (4 * kQRMaxRank) + tid;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) Wp[c * kQRMaxRank] = w[c];
       named_arrive(2, kOT);                          // W of this step is there
       if (tid < r) {                                 // rows p0 .. p0 + 3 of Y are final
 #pragma unroll
@@ -120,6 +121,11 @@ __device__ __forceinline__ void eliminate(const double* Gq, double* Prow, double
       const double* Ws = W + ((p0 >> 2) & 1) * (4 * kQRMaxRank);
       const bool mine = ((b ^ ti) & 12) == 0;        // this thread owns one of the rows b .. b + 3
       const int bx = b >> 4;
+      double cw[NX][4];                              // read once for all of the thread's rows
+#pragma unroll
+      for (int y = 0; y < NX; ++y)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) cw[y][c] = Ws[c * kQRMaxRank + tj + 16 * y];
 #pragma unroll
       for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1 || mine) {
@@ -128,17 +134,15 @@ __device__ __forceinline__ void eliminate(const double* Gq, double* Prow, double
             const int i = ti + 16 * x;
             const bool next = mine && x == bx;
             if (i >= b && (pass == 0) == next) {
-              const double2 a0 = *reinterpret_cast<const double2*>(Ws + i * 4);
-              const double2 a1 = *reinterpret_cast<const double2*>(Ws + i * 4 + 2);
+              double a[4];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) a[c] = Ws[c * kQRMaxRank + i];
 #pragma unroll
               for (int y = 0; y < NX; ++y) {
                 const int k = tj + 16 * y;
-                const double2 c0 = *reinterpret_cast<const double2*>(Ws + k * 4);
-                const double2 c1 = *reinterpret_cast<const double2*>(Ws + k * 4 + 2);
-                double v = fma(-a0.x, c0.x, T[x][y]);
-                v = fma(-a0.y, c0.y, v);
-                v = fma(-a1.x, c1.x, v);
-                v = fma(-a1.y, c1.y, v);
+                double v = T[x][y];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v = fma(-a[c], cw[y][c], v);
                 T[x][y] = (k < b || k >= i) ? v : 0.0;
                 if (pass == 0) Prow[(i - b) * kQRMaxRank + k] = T[x][y];
               }
@@ -255,11 +259,11 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
 #pragma unroll
           for (int y = 0; y < 4; ++y) g[x][y] = fma(a[x], b[y], g[x][y]);
       }
-      double* dst = (RG > 1 ? red + rg * len : share) + t * 16;
+      double* dst = (RG > 1 ? red + rg * len : share) + t;
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; y += 2) *reinterpret_cast<double2*>(dst + x * 4 + y) = make_double2(g[x][y], g[x][y + 1]);
+        for (int y = 0; y < 4; ++y) dst[(x * 4 + y) * nblk] = g[x][y];
     }
     if (RG > 1) {
       __syncthreads();
@@ -298,16 +302,17 @@ __global__ void __launch_bounds__(kOT) k_orth_factor(const __grid_constant__ QRA
   __threadfence();
   double* Gq = Ps;                                   // [len]
   double* Prow = Gq + kMaxPacked;                    // [4][64]
-  double* W = Prow + 4 * kQRMaxRank;                 // [2][64][4]
-  sum_strided<3, 8>(M.Gp, nclu, len, len, tid, kOT, 0, 1, [&](int e, double v) { Gq[e] = v; });
+  double* W = Prow + 4 * kQRMaxRank;                 // [2][4][64]
+  sum_strided<7, 6>(M.Gp, nclu, len, len, tid, kOT, 0, 1, [&](int e, double v) { Gq[e] = v; });
   for (int e = tid; e < 2 * 4 * kQRMaxRank; e += kOT) W[e] = 0.0;
   for (int e = tid; e < 4 * kQRMaxRank; e += kOT) Prow[e] = 0.0;
   __syncthreads();
   double trace = 0.0;
   for (int b = 0, o = 0; b < nb; o += nb - b, ++b)   // entries past r are zero
-    trace += (Gq[o * 16] + Gq[o * 16 + 5]) + (Gq[o * 16 + 10] + Gq[o * 16 + 15]);
+    trace += (Gq[o] + Gq[5 * nblk + o]) + (Gq[10 * nblk + o] + Gq[15 * nblk + o]);
   double* Yg = M.Gp + (int64_t)nclu * len;           // R^{-T}, row-major
-  if (r <= 32) eliminate<2>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
+  if (r <= 16) eliminate<1>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
+  else if (r <= 32) eliminate<2>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
   else eliminate<4>(Gq, Prow, W, 1e-12 * trace, r, Yg, args.status);
 }
 
@@ -322,6 +327,7 @@ __global__ void __launch_bounds__(kAT) k_orth_apply(const __grid_constant__ QRAr
   const int PY = r | 1;                              // odd pitch: the lanes' rows of Y fall in distinct banks
   double* Ys = orth_smem;                            // [r][PY]
   double* Ps = Ys + r * PY;                          // [32][r]
+  float* Us = reinterpret_cast<float*>(Ps + 32 * r); // [r][33]: the new rows, for the stacked operand
   const int nrows = min(32, M.a - row0);
   const int nb = (r + 3) >> 2;
   const double* Yg = M.Gp + (int64_t)((M.nchunk + kOrthCluster - 1) / kOrthCluster) * (nb * (nb + 1) * 8);
@@ -361,14 +367,19 @@ __global__ void __launch_bounds__(kAT) k_orth_apply(const __grid_constant__ QRAr
       s1 = fma(Ps[(ti + 16) * r + i], y[i], s1);
     }
     const float u0 = (float)(s0 + t0), u1 = (float)(s1 + t1);
-    if (row0 + ti < M.a) {
-      M.Uout[(int64_t)(row0 + ti) * r + j] = u0;
-      if (M.bt) tc_store_terms(M.bt, M.bt_n, M.bt_ld, j, row0 + ti, u0);
+    if (row0 + ti < M.a) M.Uout[(int64_t)(row0 + ti) * r + j] = u0;
+    if (row0 + ti + 16 < M.a) M.Uout[(int64_t)(row0 + ti + 16) * r + j] = u1;
+    if (M.bt) {
+      Us[j * 33 + ti] = u0;
+      Us[j * 33 + ti + 16] = u1;
     }
-    if (row0 + ti + 16 < M.a) {
-      M.Uout[(int64_t)(row0 + ti + 16) * r + j] = u1;
-      if (M.bt) tc_store_terms(M.bt, M.bt_n, M.bt_ld, j, row0 + ti + 16, u1);
-    }
+  }
+  if (!M.bt) return;
+  // the stacked operand has k contiguous: lanes along k
+  __syncthreads();
+  for (int e = tid; e < 32 * r; e += kAT) {
+    const int k = e & 31, j = e >> 5;
+    if (row0 + k < M.a) tc_store_terms(M.bt, M.bt_n, M.bt_ld, j, row0 + k, Us[j * 33 + k]);
   }
 }
 
@@ -399,7 +410,7 @@ cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st) {
   }
   ProfScope prof(ASI_K_QR, st, bytes);
   if (any) {
-    const size_t s1 = (size_t)(kOrthMaxRows * kQRMaxRank + kMaxPacked + kOT * 16) * 8, s2 = ((size_t)rmax * (rmax | 1) + 32 * rmax) * 8;
+    const size_t s1 = (size_t)(kOrthMaxRows * kQRMaxRank + kMaxPacked + kOT * 16) * 8, s2 = ((size_t)rmax * (rmax | 1) + 32 * rmax) * 8 + 33 * 4 * (size_t)rmax;
     cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_orth_factor), s1);
     if (e == cudaSuccess) e = opt_in_smem(reinterpret_cast<const void*>(k_orth_apply), s2);
     if (e != cudaSuccess) return e;
