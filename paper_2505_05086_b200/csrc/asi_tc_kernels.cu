@@ -19,8 +19,10 @@
 //     [3 n x 64] (cp.async.bulk.tensor, 128-byte swizzle);
 //   * an issuer thread launches 4 k-steps of tcgen05.mma (M = 128, N = 3 n, K = 16) per chunk and commits
 //     them to the mbarrier that frees the stage;
-//   * eight warps then read the three accumulator groups with tcgen05.ld (lane = row) and add them; a CTA of a product
-//     with many tiles takes several, and the stages fill with the next one's chunks meanwhile.
+//   * eight warps read the three accumulator groups with tcgen05.ld (lane = row) and add them to registers after every
+//     four chunks, because the unit's own sums truncate (a contraction of 2400 left in TMEM had eight times the error: 1.0e-6
+//     against 1.2e-7); two accumulators where they fit, so that the next chunks do not wait.  A CTA of a product with
+//     many tiles takes several, and the stages fill with the next one's chunks meanwhile.
 // A launch uses clusters of 1, 2 or 4 CTAs: the CTAs of a cluster share one tile of a product whose contraction
 // is long (each takes a quarter of K, the partial tiles meet in distributed shared memory in rank order) or own
 // different tiles.  Stage count and TMEM columns follow n so that two CTAs share an SM: what bounds these products
@@ -46,6 +48,7 @@ constexpr int kTcThreads = (kTcWorkers + 2) * 32;   // + the MMA issuer warp and
 constexpr int kTcM = 128;          // rows of Y per CTA (= TMEM lanes)
 constexpr int kTcKC = 64;          // k per chunk: 64 bf16 = one 128-byte swizzle row
 constexpr int kTcMaxStages = 4;
+constexpr int kTcSeg = 4;          // chunks that add up in TMEM before their sum goes to registers
 constexpr int kTcNMax = 64;
 constexpr uint32_t kTileA = kTcM * kTcKC * 2;       // 16 KB
 
@@ -189,6 +192,7 @@ struct TcProb {
   int n_cta;
   int tpc;             // tiles a CTA takes one after another (1 where CTAs share a tile)
   int tiles;
+  int nbuf;            // accumulators in TMEM: two where two CTAs' pairs fit an SM
   int nst;             // stages: as many as its operand width leaves room for beside a second CTA
 };
 struct TcGroup {
@@ -235,12 +239,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   int q = 0;
   while (q + 1 < g.np && (int)blockIdx.x >= g.p[q + 1].first) ++q;
   const TcProb& p = g.p[q];
-  const int nst = p.nst, N = p.N;
+  const int nst = p.nst, N = p.N, nbuf = p.nbuf;
   const uint32_t tile_b = (uint32_t)(3 * N) * 128u;     // operand tile: 3 N rows of 64 bf16
   const uint32_t stage = kTileA + tile_b;               // 1024-byte multiples: N is a multiple of 16
   // carve-up: stages, then barriers
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem) + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[1], acc_free[1];
+  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[2], acc_free[2];
   __shared__ uint32_t tmem_slot[1];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -271,8 +275,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
 
   if (tid == 0) {
     for (int i = 0; i < nst; ++i) { mbar_init(full + i, 1); mbar_init(s_free + i, 1); }
-    mbar_init(done, 1);
-    mbar_init(acc_free, kTcWorkers);
+    for (int i = 0; i < 2; ++i) { mbar_init(done + i, 1); mbar_init(acc_free + i, kTcWorkers); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {                                      // TMEM: fp32 columns x 128 lanes (3 N are used)
@@ -298,31 +301,36 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
       const uint32_t idesc = instr_desc_bf16(kTcM, 3 * N, a_mn);
       const uint32_t a_base = smem_u32(base);
       const uint64_t a_step = a_mn ? 128 : 2;           // a k-step is 16 bf16: 32 bytes inside the swizzle row of a
-      int st = 0, busy = 0;                             // K-major tile, 16 rows (2048 bytes) of an MN-major tile
+      int st = 0, seg = 0;                              // K-major tile, 16 rows (2048 bytes) of an MN-major tile
       uint32_t ph = 0;                                  // (start-address field in 16-byte units)
 #pragma unroll 1
       for (int t = 0; t < ntile && ok; ++t) {
         const int nchunk = tile_of(t).nchunk;
-        if (nchunk == 0) continue;
-        if (busy) {                                     // the workers have read the tile before
-          ok = mbar_wait(acc_free, (uint32_t)(busy + 1) & 1u);
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-        ++busy;
 #pragma unroll 1
-        for (int c = 0; c < nchunk && ok; ++c) {
-          ok = mbar_wait(full + st, ph);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t da0 = smem_desc_sw128(a_base + st * stage, a_mn ? kTileA / 2 : 16);
-          const uint64_t db0 = smem_desc_sw128(a_base + st * stage + kTileA);
+        for (int c0 = 0; c0 < nchunk && ok; c0 += kTcSeg, ++seg) {
+          const int buf = nbuf == 2 ? seg & 1 : 0, turn = nbuf == 2 ? seg >> 1 : seg;
+          if (turn > 0) {                               // the workers have read what the buffer held
+            ok = mbar_wait(acc_free + buf, (uint32_t)(turn + 1) & 1u);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
+          const int c1 = c0 + kTcSeg < nchunk ? c0 + kTcSeg : nchunk;
+#pragma unroll 1
+          for (int c = c0; c < c1; ++c) {
+            ok = mbar_wait(full + st, ph);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t da0 = smem_desc_sw128(a_base + st * stage, a_mn ? kTileA / 2 : 16);
+            const uint64_t db0 = smem_desc_sw128(a_base + st * stage + kTileA);
 #pragma unroll
-          for (int ks = 0; ks < kTcKC / 16; ++ks)
-            umma_bf16(tmem_d, da0 + (uint64_t)ks * a_step, db0 + (uint64_t)(ks * 2), idesc, (c | ks) ? 1u : 0u);
-          umma_commit(s_free + st);
-          if (++st == nst) { st = 0; ph ^= 1u; }
+            for (int ks = 0; ks < kTcKC / 16; ++ks)
+              umma_bf16(tmem_d + (uint32_t)(buf * 3 * N), da0 + (uint64_t)ks * a_step, db0 + (uint64_t)(ks * 2), idesc,
+                        ((c - c0) | ks) ? 1u : 0u);
+            umma_commit(s_free + st);
+            if (++st == nst) { st = 0; ph ^= 1u; }
+          }
+          if (ok) umma_commit(done + buf);
         }
-        umma_commit(done);
       }
     }
   } else if (warp == kTcWorkers + 1) {
@@ -364,46 +372,51 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
     const int col0 = (warp >> 2) * half;
     const int r = (warp & 3) * 32 + lane;
     const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
-    uint32_t ph = 0;
+    int seg = 0;
 #pragma unroll 1
     for (int t = 0; t < ntile && ok; ++t) {
       const Tile x = tile_of(t);
-      if (x.nchunk > 0) {
-        ok = mbar_wait(done, ph);                       // every reader of TMEM observes the completed phase
+      float sum[kTcNMax / 2];                           // an empty share of K adds nothing
+#pragma unroll
+      for (int i = 0; i < kTcNMax / 2; ++i) sum[i] = 0.f;
+#pragma unroll 1
+      for (int c0 = 0; c0 < x.nchunk; c0 += kTcSeg, ++seg) {
+        const int buf = nbuf == 2 ? seg & 1 : 0, turn = nbuf == 2 ? seg >> 1 : seg;
+        ok = mbar_wait(done + buf, (uint32_t)turn & 1u);   // every reader of TMEM observes the completed phase
         if (__any_sync(0xffffffffu, ok ? 0 : 1)) ok = false;
         if (!ok) break;
-        ph ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      }
-      for (int cc = 0; cc < half; cc += 8) {
-        float o[8];
-        if (x.nchunk > 0) {
-          uint32_t h[8], m[8], l[8];
-          tmem_ld8(taddr + (uint32_t)cc, h);
-          tmem_ld8(taddr + (uint32_t)(N + cc), m);
-          tmem_ld8(taddr + (uint32_t)(2 * N + cc), l);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int i = 0; i < 8; ++i)                   // small terms first
-            o[i] = (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
-        } else {
+        for (int cc = 0; cc < kTcNMax / 2; cc += 8)
+          if (cc < half) {
+            uint32_t h[8], m[8], l[8];
+            const uint32_t at = taddr + (uint32_t)(buf * 3 * N + cc);
+            tmem_ld8(at, h);
+            tmem_ld8(at + (uint32_t)N, m);
+            tmem_ld8(at + (uint32_t)(2 * N), l);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int i = 0; i < 8; ++i) o[i] = 0.f;       // an empty share of K
-        }
-        if (x.nchunk > 0 && cc + 8 >= half && t + 1 < ntile) {   // all read: the accumulator is free
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_free);
-        }
-        const float4 v0 = make_float4(o[0], o[1], o[2], o[3]), v1 = make_float4(o[4], o[5], o[6], o[7]);
-        if (p.ksp > 1) {
-          *reinterpret_cast<float4*>(xch + r * PN + col0 + cc) = v0;
-          *reinterpret_cast<float4*>(xch + r * PN + col0 + cc + 4) = v1;
-        } else {
-          tc_store4(p, x.s, x.row0 + r, col0 + cc, v0);
-          tc_store4(p, x.s, x.row0 + r, col0 + cc + 4, v1);
-        }
+            for (int i = 0; i < 8; ++i)                 // small terms first
+              sum[cc + i] += (__uint_as_float(l[i]) + __uint_as_float(m[i])) + __uint_as_float(h[i]);
+          }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_free + buf);     // all read: the buffer is free
       }
+      if (!ok) break;
+#pragma unroll
+      for (int cc = 0; cc < kTcNMax / 2; cc += 8)
+        if (cc < half) {
+          const float4 v0 = make_float4(sum[cc], sum[cc + 1], sum[cc + 2], sum[cc + 3]);
+          const float4 v1 = make_float4(sum[cc + 4], sum[cc + 5], sum[cc + 6], sum[cc + 7]);
+          if (p.ksp > 1) {
+            *reinterpret_cast<float4*>(xch + r * PN + col0 + cc) = v0;
+            *reinterpret_cast<float4*>(xch + r * PN + col0 + cc + 4) = v1;
+          } else {
+            tc_store4(p, x.s, x.row0 + r, col0 + cc, v0);
+            tc_store4(p, x.s, x.row0 + r, col0 + cc + 4, v1);
+          }
+        }
     }
   }
   const bool fail = __syncthreads_or(ok ? 0 : 1) != 0;
@@ -530,7 +543,6 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st
   TcGroup g;
   g.np = n;
   g.status = status;
-  int nmax = 16;
   double bytes = 0.0;
   int64_t tiles[3];
   int chunks[3];
@@ -544,7 +556,6 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st
     p.Bt = static_cast<__nv_bfloat16*>(k.out_bt);
     p.Y = k.Y;
     p.ldy = k.n;
-    nmax = p.N > nmax ? p.N : nmax;
     const int64_t Q = k.O * k.I;
     bool ok;
     int64_t second = 1;
@@ -582,26 +593,38 @@ cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st
     tiles[q] = p.mt * second;
     bytes += 2.0 * (double)k.a * Q;
   }
-  // a product with few tiles and a long contraction shares each tile between the CTAs of a cluster
-  int64_t total = 0;
-  for (int q = 0; q < n; ++q) total += tiles[q];
+  // A product with few tiles and a long contraction shares each tile between the CTAs of a cluster.  Few: below 64, where it
+  // leaves most SMs idle.  (At 200 a step's expansions of 64 + 64 tiles ran as 512 CTAs of four chunks, two waves of set-up and
+  // exchange: ViT-Base MLP 245 us, LLM-shaped tokens 310; at 64, with sums of four chunks in registers, 227 and 283; without
+  // clusters single layers lose 4 %.)
+  constexpr int kFewTiles = 64;
   int cs = 1;
   for (int q = 0; q < n; ++q)
-    while (cs < 4 && tiles[q] * cs < 200 && chunks[q] >= 8 * cs) cs *= 2;
+    while (cs < 4 && tiles[q] * cs < kFewTiles && chunks[q] >= 8 * cs) cs *= 2;
+  auto shares = [&](int q) { return cs > 1 && tiles[q] < kFewTiles && chunks[q] >= 4 * cs; };
+  // Tiles in turn where the launch has more than the machine holds at a time (two CTAs an SM), what the shared tiles leave of
+  // it but 200 at least: the next tile's loads run under this one's epilogue, and the set-up (4 k of 12 k cycles) is paid
+  // once (ViT-Base MLP 3 % against a count per product)
+  int64_t shared = 0, plain = 0;
+  for (int q = 0; q < n; ++q) (shares(q) ? shared : plain) += tiles[q] * (shares(q) ? cs : 1);
+  const int64_t room = std::max<int64_t>(200, 296 - shared);
   int first = 0;
   for (int q = 0; q < n; ++q) {
     TcProb& p = g.p[q];
-    p.ksp = (cs > 1 && tiles[q] < 200 && chunks[q] >= 4 * cs) ? cs : 1;
+    p.ksp = shares(q) ? cs : 1;
     p.first = first;
-    // tiles in turn where there are more than the machine holds at a time (two CTAs an SM): the next tile's loads run
-    // under this one's epilogue, and the set-up (4 k of 12 k cycles) is paid once
     p.tiles = (int)tiles[q];
-    p.tpc = p.ksp > 1 ? 1 : (int)std::min<int64_t>(8, (tiles[q] + 295) / 296);
+    p.tpc = p.ksp > 1 ? 1 : (int)std::min<int64_t>(8, (plain + room - 1) / room);
     p.n_cta = p.ksp > 1 ? (int)tiles[q] * p.ksp : (p.tiles + p.tpc - 1) / p.tpc;
     first += (p.n_cta + cs - 1) / cs * cs;
   }
   g.cs = cs;
-  g.tmem_cols = 3 * nmax <= 64 ? 64 : (3 * nmax <= 128 ? 128 : 256);
+  int cols = 0;
+  for (int q = 0; q < n; ++q) {
+    g.p[q].nbuf = 6 * g.p[q].N <= 256 ? 2 : 1;
+    cols = std::max(cols, g.p[q].nbuf * 3 * g.p[q].N);
+  }
+  g.tmem_cols = cols <= 64 ? 64 : (cols <= 128 ? 128 : 256);
   // every product its own stage count: with those of the widest one (two at 64 columns) the four chunks of a narrower
   // product's tile took one round trip more
   size_t smem = 0;
