@@ -101,7 +101,11 @@ void choose_kernels(asi_plan* pl) {
     const size_t need = sm_wgrad_smem(a, R, false, pl->bf16);
     if (need > 75 * 1024 || B * cpb * HoWo > 32768) a.nt = 512;
     if (a.nt == 512 && sm_wgrad_smem(a, R, false, pl->bf16) > kSmemLimit) a.nt = 256;
-    if (need <= 113 * 1024 || (need <= kSmemLimit && H * W <= 256)) {
+    // A CTA a channel that streams long and leaves SMs idle gives way to the launches that split the reduction (one layer's weight
+    // gradient, 128 x 28 x 28 to 96 channels 30.7 -> 24.4 us, 16 x 28 x 28 to 32 22.9 -> 19.2; short streams, 1 x 1 kernels and
+    // more channels than SMs lose: 4 x 30 x 30 to 100 41.3 against 43.4, 64 x 24 x 24 1 x 1 11.6 against 14.5)
+    const bool idle = Cout / cpb <= 148 && pl->d.kh * pl->d.kw >= 9 && B * cpb * HoWo >= 8192;
+    if (H * W <= 256 ? need <= kSmemLimit : need <= 113 * 1024 && !idle) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
       pl->wgrad_ncl = a.ncl;
