@@ -109,3 +109,42 @@ def test_cold_start_passes(dims, ranks, bf16):
     U = run.factors()
     assert max(O.rel_fro(O.projector(a), O.projector(b)) for a, b in zip(U, U_ref)) <= 1e-4
     assert O.rel_fro(O.sign_align(run.core_np(), U, U_ref)[0], S_ref) <= 1e-4
+
+
+WGRADS = [  # (dims, cout, k, stride, groups, ranks, split launches): both sides of the rule's three lines
+    ((16, 24, 24, 24), 24, 3, 1, 1, (3, 4, 4, 4), True),       # 9216 values a CTA
+    ((14, 24, 24, 24), 24, 3, 1, 1, (3, 4, 4, 4), False),      # 8064: one CTA a channel
+    ((13, 30, 25, 27), 148, 3, 1, 1, (4, 4, 4, 4), True),      # as many channels as SMs; odd planes of dY
+    ((13, 30, 25, 27), 149, 3, 1, 1, (4, 4, 4, 4), False),
+    ((40, 24, 29, 29), 36, 3, 2, 12, (4, 4, 4, 4), True),      # grouped, strided
+    ((16, 20, 24, 24), 20, 5, 1, 20, (4, 8, 8, 8), True),      # depthwise
+    ((16, 24, 24, 24), 24, 1, 1, 1, (4, 4, 4, 4), False),      # 1 x 1
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,cout,k,stride,groups,ranks,split", WGRADS)
+def test_weight_gradient_routes_of_large_maps(dims, cout, k, stride, groups, ranks, split, bf16):
+    """dY at a sixteen-byte address and one element past it, on either side of the line between the launches."""
+    rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "conv", dims, cout, k, stride, k // 2, groups, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(dims, ranks)))
+    run = make_runner(L, bf16=bf16)
+    assert (run.plan.launch_count(1) > 1) == split
+    A, dY = st.next()
+    U_prev = st.u_prev0()
+    to_device = run.to_device
+    for shift in (0, 1):
+        def place(x):
+            t = to_device(x)
+            if x is A:
+                return t
+            buf = torch.full((t.numel() + 8,), float("nan"), dtype=t.dtype, device=t.device)
+            view = buf[shift:shift + t.numel()].view(t.shape)
+            view.copy_(t)
+            return view
+
+        run.to_device = place
+        err, _ = compare_step(run, L, A, dY, U_prev)
+        check(err, TOL_F32, f"{dims} {cout} bf16={bf16} shift={shift}")
