@@ -85,7 +85,7 @@ __device__ __forceinline__ void rest2(const float* x, float* lo) {
   lo[0] = l.x;
   lo[1] = l.y;
 }
-// a value as its nearest tf32 value and the rest
+// the nearest tf32 value of a finite one (the carry makes a zero of 0x7fffffff, the NaN that arithmetic leaves)
 __device__ __forceinline__ float nearest(float x) { return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u); }
 
 __device__ __forceinline__ void add_pair(float* s, float x, float y) {
@@ -147,10 +147,18 @@ struct Acc {
   }
 };
 
-// one entry of the B operand of the columns: lane group g is the column
-template <int NB>
+// One entry of the B operand of the columns: lane group g is the column.  A NaN is lost in both roundings, but not in the difference:
+// x - (x - hi) is hi again, or NaN where x is NaN or infinite.  TOP (values of the caller's): what would round to infinity
+// leaves more to the rest instead
+template <int NB, bool TOP>
 __device__ __forceinline__ void set_b(float* b, int half, int g, float x) {
-  const float hi = nearest(x), lo = nearest(x - hi);
+  float hi = nearest(x);
+  if constexpr (TOP) {
+    const float top = __uint_as_float(0x7f7fe000u);
+    hi = fmaxf(fminf(hi, top), -top);
+  }
+  const float rest = x - hi, lo = nearest(rest);
+  hi = x - rest;
   if constexpr (NB == 1) b[half] = g < 4 ? hi : lo;
   else {
     b[half] = hi;
@@ -317,7 +325,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = row0 + 8 * s + 2 * c4 + h, j = NB == 1 ? (g & 3) : g;
-      set_b<NB>(ub[s], h, g, (k < a && j < r) ? __ldg(p.U + (int64_t)k * p.ldu + j) : 0.f);
+      set_b<NB, true>(ub[s], h, g, (k < a && j < r) ? __ldg(p.U + (int64_t)k * p.ldu + j) : 0.f);
     }
   Acc<NB, EX> P[RT];
 #pragma unroll
@@ -420,7 +428,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
               for (int i = 0; i < 4; ++i) x[i] += y[i];
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) set_b<NB>(b[u + i], h, g, x[i]);
+            for (int i = 0; i < 4; ++i) set_b<NB, GIVEN>(b[u + i], h, g, x[i]);
           }
 #pragma unroll
         for (int m = 0; m < RT; ++m) {
@@ -662,8 +670,8 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = 8 * s + (h ? kr1 : kr0), w = wrow(h, s);
-      set_b<NB>(u3[s], h, g, (k < H && jb < p.r3) ? __ldg(p.U3 + k * p.r3 + jb) : 0.f);
-      set_b<NB>(u4[s], h, g, (w < W && jb < p.r4) ? __ldg(p.U4 + w * p.r4 + jb) : 0.f);
+      set_b<NB, true>(u3[s], h, g, (k < H && jb < p.r3) ? __ldg(p.U3 + k * p.r3 + jb) : 0.f);
+      set_b<NB, true>(u4[s], h, g, (w < W && jb < p.r4) ? __ldg(p.U4 + w * p.r4 + jb) : 0.f);
     }
   Acc<NB, EX> P3[2], P4[2];
 #pragma unroll
@@ -758,7 +766,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) set_b<NB>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
+        for (int e = 0; e < 4; ++e) set_b<NB, GIVEN>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         if (m >= nkh) break;
@@ -808,8 +816,8 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
       float b4[2][2 * NB];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        set_b<NB>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
-        set_b<NB>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
+        set_b<NB, GIVEN>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
+        set_b<NB, GIVEN>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
       }
       col_steps(xs, s2, b4[0], b4[1], P4);
     }

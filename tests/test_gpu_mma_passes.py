@@ -148,3 +148,98 @@ def test_weight_gradient_routes_of_large_maps(dims, cout, k, stride, groups, ran
         run.to_device = place
         err, _ = compare_step(run, L, A, dY, U_prev)
         check(err, TOL_F32, f"{dims} {cout} bf16={bf16} shift={shift}")
+
+
+NAN_BITS = 0x7fffffff                              # the NaN that arithmetic on the GPU makes
+NANS = [c for c in CASES if c[0] in ((17, 33, 17, 20), (12, 130, 17, 17), (40, 48, 24, 24), (33, 128, 20, 20))]
+
+
+def _put_nan(flat, at):
+    flat.view(torch.int32)[at] = NAN_BITS
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", NANS)
+def test_a_nan_in_a_factor_reaches_the_results(dims, ranks, bf16):
+    """One NaN in column 1 of U_m (or of Omega_m): that column of P_m and so every column of the new factor from there on, and with
+    the core all of the gradient."""
+    from paper_2505_05086_b200.binding import ASI_ERR_RANK_DEFICIENT
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    run = make_runner(L, bf16=bf16)
+    rng = np.random.default_rng(4)
+    act, dY = (run.to_device(rng.standard_normal(s)) for s in (dims, L.dy_shape))
+    U0 = np.concatenate([np.linalg.qr(rng.standard_normal((d, r)))[0].ravel() for d, r in zip(dims, ranks)])
+    n = int(np.prod(dims))
+    omega = torch.from_numpy(rng.standard_normal(sum(n // d * r for d, r in zip(dims, ranks))).astype(np.float32)).cuda()
+    at_u = at_o = 0
+    for m, (d, r) in enumerate(zip(dims, ranks)):
+        for cold in (False, True):
+            if cold:
+                om = omega.clone()
+                _put_nan(om, at_o + (n // d // 2) * r + 1)
+                run.init_factors(act, om)
+            else:
+                run.U[run.cur].copy_(torch.from_numpy(U0.astype(np.float32)))
+                _put_nan(run.U[run.cur], at_u + (d // 2) * r + 1)
+                run.compress(act)
+            run.wgrad(dY)
+            assert run.device_status() == ASI_ERR_RANK_DEFICIENT, (m, cold)
+            U = run.factors()
+            assert np.isnan(U[m][:, 1:]).all(), (m, cold)
+            assert all(np.isfinite(u).all() for q, u in enumerate(U) if q != m), (m, cold)
+            assert np.isnan(np.moveaxis(run.core_np(), m, 0)[1:]).all(), (m, cold)
+            assert np.isnan(run.dW.cpu().numpy()).all(), (m, cold)
+        at_u += d * r
+        at_o += n // d * r
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", NANS)
+def test_a_nan_in_the_activation_stays_in_the_factors_of_the_next_step(dims, ranks, bf16):
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    run = make_runner(L, bf16=bf16)
+    rng = np.random.default_rng(4)
+    act, dY = (run.to_device(rng.standard_normal(s)) for s in (dims, L.dy_shape))
+    run.set_factors([np.linalg.qr(rng.standard_normal((d, r)))[0] for d, r in zip(dims, ranks)])
+    bad = act.clone()
+    bad.view(-1)[act.numel() // 2] = float("nan")
+    for x in (bad, act):
+        run.compress(x)
+        run.wgrad(dY)
+        assert not run.ok()
+        assert all(np.isnan(u).all() for u in run.factors())
+        assert np.isnan(run.dW.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("dims,ranks,cout,bf16", TOKENS[1:])
+def test_a_nan_in_the_batch_factor_of_a_token_layer(dims, ranks, cout, bf16):
+    L = LayerSpec("t", "linear", dims, cout, ranks=ranks)
+    run = make_runner(L, bf16=bf16)
+    rng = np.random.default_rng(4)
+    run.set_factors([np.linalg.qr(rng.standard_normal((d, r)))[0] for d, r in zip(dims, ranks)])
+    _put_nan(run.U[run.cur], dims[0] // 2 * ranks[0] + 1)
+    run.compress(run.to_device(rng.standard_normal(dims)))
+    run.wgrad(run.to_device(rng.standard_normal(L.dy_shape)))
+    assert not run.ok()
+    assert np.isnan(run.factors()[0][:, 1:]).all()
+    assert np.isnan(run.dW.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", NANS)
+def test_a_factor_of_the_largest_values(dims, ranks, bf16):
+    """U_m scaled to the top of fp32 beside an activation scaled down: the same factor as without (1e-6 of rounding on
+    well-conditioned random data, times ten)."""
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    run = make_runner(L, bf16=bf16)
+    rng = np.random.default_rng(4)
+    act = run.to_device(rng.standard_normal(dims))
+    U0 = [np.linalg.qr(rng.standard_normal((d, r)))[0].astype(np.float32) for d, r in zip(dims, ranks)]
+    out = []
+    for scale in (1.0, 2.0 ** -60):
+        U = [u.copy() for u in U0]
+        for u in U:
+            u[:] = np.sign(u) * (1.0 if scale == 1.0 else np.finfo(np.float32).max)
+        run.set_factors(U)
+        run.compress(act * scale)
+        assert run.ok()
+        out.append(run.factors())
+    for a, b in zip(*out):
+        assert np.linalg.norm(a - b) / np.linalg.norm(b) <= 1e-5
