@@ -354,6 +354,8 @@ bool compress_takes(const asi_plan* pl, const void* act) {
   return element_aligned(pl, act) && (!pl->rows16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
 }
 
+int stalls(const asi_plan* pl) { return (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0; }
+
 asi_status_t check_ws(const void* ws, size_t have, size_t need) {
   if (!valid_ptr(ws)) return ASI_ERR_INVALID_ARG;
   if (have < need || (reinterpret_cast<uintptr_t>(ws) & 255u)) return ASI_ERR_WORKSPACE;
@@ -395,7 +397,7 @@ void build_fused_pass1(const asi_plan* pl, const void* act, const float* U_prev,
   a->vec4 = pl->fast_vec4 ? 1 : 0;
   a->aligned = four_aligned(pl, act) ? 1 : 0;
   a->bulk = (!pl->bf16 && pl->fast_vec4 && a->aligned) ? 1 : 0;
-  a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
+  a->stall_copy = stalls(pl);
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;      // 1 ms under the test hook, else 1 s
 }
 
@@ -412,7 +414,7 @@ void build_tile1(const asi_plan* pl, const void* act, const float* U_prev, char*
   a->C = (int)pl->dims[1];
   a->n_tiles_b = pl->n_tiles_b;
   a->aligned = four_aligned(pl, act) ? 1 : 0;
-  a->stall_copy = (pl->d.flags & ASI_FLAG_TEST_EXPIRE_WAIT) ? 1 : 0;
+  a->stall_copy = stalls(pl);
   a->wait_ns = a->stall_copy ? 1000000ull : 1000000000ull;
 }
 
@@ -814,6 +816,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     a.r3 = pl->r[2];
     a.r4 = pl->r[3];
     a.status = status;
+    a.stall = stalls(pl);
     a.given = 1;
     a.first = head;
     a.clear = clear ? status : nullptr;
@@ -830,6 +833,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     f.Pp = reinterpret_cast<float*>(w + pl->off_Pp[m]);
     f.O = v.O; f.I = v.I; f.a = (int)v.a; f.r = v.r;
     f.status = status;
+    f.stall = stalls(pl);
     f.given = 1;
     f.first = head;
     f.clear = clear ? status : nullptr;
@@ -1075,6 +1079,7 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     g.r3 = pl->r[2];
     g.r4 = pl->r[3];
     g.status = status;
+    g.stall = stalls(pl);
     g.first = first;
     g.clear = take_clear();
     const bool mma = pl->mplane && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);   // else: odd bf16 addresses
@@ -1096,6 +1101,7 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
       f.first = first;
       f.clear = take_clear();
       f.status = status;
+      f.stall = stalls(pl);
       const bool mma = pl->mfiber[m] && (!pl->bf16 || (reinterpret_cast<uintptr_t>(act) & 15u) == 0);
       if (mma) ASI_CUDA(launch_mfiber(f, pl->fiber_grid[m], pl->bf16, st));
       else ASI_CUDA(pl->wfiber[m] ? launch_wfiber(f, pl->fiber_grid[m], pl->bf16, st)

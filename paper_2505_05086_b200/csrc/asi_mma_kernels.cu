@@ -201,16 +201,18 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// gives up after about one second
-__device__ __forceinline__ bool mbar_wait_1s(uint64_t* bar, uint32_t parity) {
+// gives up after `limit` cycles
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit) {
   if (mbar_try(bar, parity)) return true;
   const long long t0 = clock64();
   for (uint32_t it = 0; it < (1u << 28); ++it) {
     if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 255u && clock64() - t0 > 2000000000ll) return false;
+    if ((it & 255u) == 255u && clock64() - t0 > limit) return false;
   }
   return false;
 }
+// about a second; with the test hook, whose producer arms its barrier and issues no copy, about a millisecond
+__device__ __forceinline__ long long wait_limit(int stall) { return stall ? 2000000ll : 2000000000ll; }
 __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
@@ -275,7 +277,8 @@ __global__ void __launch_bounds__(kMfThreads, 2)
         if (lane == 0) {
           mbar_expect(bars + st, STAGE);
 #pragma unroll
-          for (int cb = 0; cb < CB; ++cb) tma_box(dst + cb * BLK, &map, i_ld * TC + cb * TCB, row0, o_ld, bars + st);
+          for (int cb = 0; cb < CB; ++cb)
+            if (!p.stall) tma_box(dst + cb * BLK, &map, i_ld * TC + cb * TCB, row0, o_ld, bars + st);
         }
       } else {
 #pragma unroll 1
@@ -341,10 +344,12 @@ __global__ void __launch_bounds__(kMfThreads, 2)
 #pragma unroll 1
   for (int t = t_first; t < total; t += stride) {
     if constexpr (LD == 0) {
-      if (!failed && !mbar_wait_1s(bars + st, (phase >> st) & 1u)) {
+      const long long limit = wait_limit(p.stall);
+      if (!failed && !mbar_wait(bars + st, (phase >> st) & 1u, limit)) {
         failed = true;                               // the team's barriers go on; what follows is not used
-        if (t + stride < total) mbar_wait_1s(bars + (st ^ 1), (phase >> (st ^ 1)) & 1u);   // nothing stays in flight
         atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
+        mbar_wait(bars + st, (phase >> st) & 1u, limit);   // the copies in flight get the limit once more
+        if (t + stride < total) mbar_wait(bars + (st ^ 1), (phase >> (st ^ 1)) & 1u, limit);
       }
       phase ^= 1u << st;
     }
@@ -463,7 +468,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
   }
   if (tid == 0) pdl_wait();
   // ---- one partial of P per CTA: the teams' sums meet in team order
-  __syncthreads();                                   // every copy that was issued has been waited for
+  if (__syncthreads_or(failed)) return;              // else every copy has landed, and the buffers serve again
   float* red = reinterpret_cast<float*>(mf_smem) + (size_t)warp * (ROWS * NV);     // [nw][ROWS][NV]
 #pragma unroll
   for (int m = 0; m < RT; ++m) {
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
       if constexpr (LD == 0) {
         if (lane == 0) {
           mbar_expect(bars + st, (uint32_t)(hw * sizeof(TX)));
-          bulk_copy(buf + st * pb, X + t_ld * hw, (uint32_t)(hw * sizeof(TX)), bars + st);
+          if (!p.stall) bulk_copy(buf + st * pb, X + t_ld * hw, (uint32_t)(hw * sizeof(TX)), bars + st);
         }
       } else {
         const float* src = reinterpret_cast<const float*>(X) + t_ld * hw;
@@ -714,10 +719,12 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll 1
   for (int64_t t = t_first; t < p.n_planes; t += stride) {
     if constexpr (LD == 0) {
-      if (!failed && !mbar_wait_1s(bars + st, (phase >> st) & 1u)) {
+      const long long limit = wait_limit(p.stall);
+      if (!failed && !mbar_wait(bars + st, (phase >> st) & 1u, limit)) {
         failed = true;
-        if (t + stride < p.n_planes) mbar_wait_1s(bars + (st ^ 1), (phase >> (st ^ 1)) & 1u);   // nothing stays in flight
         atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
+        mbar_wait(bars + st, (phase >> st) & 1u, limit);   // the copies in flight get the limit once more
+        if (t + stride < p.n_planes) mbar_wait(bars + (st ^ 1), (phase >> (st ^ 1)) & 1u, limit);
       }
       phase ^= 1u << st;
     }
@@ -828,7 +835,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
   }
   if (tid == 0) pdl_wait();
   // ---- one partial of P3 and P4 per CTA: the warps' sums meet in warp order
-  __syncthreads();                                   // every copy that was issued has been waited for
+  if (__syncthreads_or(failed)) return;              // else every copy has landed, and the buffers serve again
   float* red = reinterpret_cast<float*>(mp_smem) + (size_t)warp * (2 * 32 * NV);   // [nw][2][32][NV]
 #pragma unroll
   for (int m = 0; m < 2; ++m) {

@@ -243,3 +243,39 @@ def test_a_factor_of_the_largest_values(dims, ranks, bf16):
         out.append(run.factors())
     for a, b in zip(*out):
         assert np.linalg.norm(a - b) / np.linalg.norm(b) <= 1e-5
+
+
+@pytest.mark.parametrize("cold", [False, True])
+@pytest.mark.parametrize("kind,dims,ranks,bf16", [
+    ("conv", (16, 130, 28, 28), (4, 4, 4, 4), False),          # planes, and teams of one and of three warps
+    ("conv", (16, 130, 40, 40), (5, 6, 5, 5), False),          # strided fibers alone
+    ("conv", (40, 48, 24, 24), (4, 4, 4, 4), True),
+    ("linear", (33, 24, 64), (7, 8, 12), True),
+])
+def test_expired_waits_are_reported_and_the_workspace_recovers(kind, dims, ranks, bf16, cold):
+    """The producer arms its barriers and copies nothing; every wait runs out (1 ms), and the next call on the same workspace is
+    healthy again."""
+    from paper_2505_05086_b200.binding import ASI_ERR_TIMEOUT, ASI_FLAG_TEST_EXPIRE_WAIT, Plan
+    L = LayerSpec("t", kind, dims, 10, 3, 1, 1, 1, ranks=ranks) if kind == "conv" else LayerSpec("t", kind, dims, 10, ranks=ranks)
+    rho = tuple(min(0.95, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=7, rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, 2 * r) for d, r in zip(dims, ranks)))
+    A, dY = st.next()
+    run = make_runner(L, bf16=bf16)
+    stalled = Plan(kind, dims, ranks, 10, L.k, L.stride, L.pad, L.groups, bf16, flags=ASI_FLAG_TEST_EXPIRE_WAIT)
+    assert stalled.info.compress_ws_bytes == run.plan.info.compress_ws_bytes
+    U_prev = st.u_prev0()
+    run.set_factors(U_prev)
+    act = run.to_device(A)
+    s = int(torch.cuda.current_stream().cuda_stream)
+    out = [run.U[1 - run.cur].data_ptr(), run.core.data_ptr(), run.ws_c.data_ptr(), run.ws_c.numel(), s]
+    if cold:
+        n = int(np.prod(dims))
+        omega = torch.randn(sum(n // d * r for d, r in zip(dims, ranks)), device="cuda")
+        stalled.init_factors(act.data_ptr(), omega.data_ptr(), *out)
+    else:
+        stalled.compress(act.data_ptr(), run.U[run.cur].data_ptr(), *out)
+    assert stalled.poll_status(run.ws_c.data_ptr(), s) == ASI_ERR_TIMEOUT
+    err, _ = compare_step(run, L, A, dY, U_prev)
+    check(err, TOL_F32, f"{dims} after an expired wait")
+    assert run.device_status() == 0
