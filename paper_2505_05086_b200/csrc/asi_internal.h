@@ -59,7 +59,7 @@ struct PlaneArgs {
   int given = 0;           // k_mplane: U3 and U4 are Omega_3 [planes W][r3] and Omega_4 [planes H][r4], and P_m = A_m Omega_m
   int* clear = nullptr;    // not null: CTA 0 zeroes the 256 ints of the workspace's status block
   int* status = nullptr;   // status word of the workspace (an expired wait on a bulk copy)
-  int stall = 0;           // test hook (k_mplane): the barriers are armed and no copy is issued, so the waits expire
+  int stall = 0;           // test hook (k_mplane, k_plane2): the barriers are armed and no copy is issued, so the waits expire
 };
 
 // One mode with strided fibers, a <= 128, r <= 4 (k_fiber2): both products in one pass, or with

@@ -380,13 +380,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// every thread waits for the phase; gives up after about one second
-__device__ __forceinline__ bool mbar_wait_1s(uint64_t* bar, uint32_t parity) {
+// every thread waits for the phase; gives up after `limit` cycles
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   for (uint32_t it = 0; it < (1u << 28); ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 255u && clock64() - t0 > 2000000000ll) return false;
+    if ((it & 255u) == 255u && clock64() - t0 > limit) return false;
   }
   return false;
 }
@@ -427,8 +427,9 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
   // thread 0 arms the stage's barrier and starts the copy (the plane count is a multiple of G: checked on the host)
   auto issue = [&](int64_t t, int st) {
     mbar_expect_tx(bars + st, kTileBytes);
-    bulk_g2s(stages + (size_t)st * G * SS, X + t * G * SS, kTileBytes, bars + st);
+    if (!p.stall) bulk_g2s(stages + (size_t)st * G * SS, X + t * G * SS, kTileBytes, bars + st);
   };
+  const long long limit = p.stall ? 2000000ll : 2000000000ll;     // about a second; a millisecond with the test hook
   int64_t t_issue = blockIdx.x;
   if (tid == 0) {
     for (int s = 0; s < NST - 1; ++s) {
@@ -447,12 +448,20 @@ __global__ void __launch_bounds__(kP2Threads, 2) k_plane2(PlaneArgs p) {
   int st = 0;
   uint32_t phase_bits = 0;
   for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const bool ok = mbar_wait_1s(bars + st, (phase_bits >> st) & 1u);
+    const bool ok = mbar_wait(bars + st, (phase_bits >> st) & 1u, limit);
     if (!ok) s_fail = 1;
     phase_bits ^= 1u << st;
     __syncthreads();                                 // everyone is past the previous tile: its stage is free
     if (s_fail) {
-      if (tid == 0) atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
+      if (tid == 0) {
+        atomicMax(p.status, (int)ASI_ERR_TIMEOUT);
+        for (int q = 0, sf = st; q < NST - 1; ++q) {   // the copies in flight get the limit once more: tile t and those behind it
+          const uint32_t parity = ((phase_bits >> sf) & 1u) ^ (q == 0 ? 1u : 0u);
+          if (t + (int64_t)q * gridDim.x < n_tiles) mbar_wait(bars + sf, parity, limit);
+          if (++sf == NST) sf = 0;
+        }
+        pdl_wait();                                  // as every pass before it ends
+      }
       return;
     }
     if (tid == 0) {

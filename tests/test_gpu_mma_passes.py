@@ -250,6 +250,7 @@ def test_a_factor_of_the_largest_values(dims, ranks, bf16):
     ("conv", (16, 130, 28, 28), (4, 4, 4, 4), False),          # planes, and teams of one and of three warps
     ("conv", (16, 130, 40, 40), (5, 6, 5, 5), False),          # strided fibers alone
     ("conv", (40, 48, 24, 24), (4, 4, 4, 4), True),
+    ("conv", (16, 40, 56, 56), (4, 4, 4, 4), False),           # the planes of their own kernel
     ("linear", (33, 24, 64), (7, 8, 12), True),
 ])
 def test_expired_waits_are_reported_and_the_workspace_recovers(kind, dims, ranks, bf16, cold):
