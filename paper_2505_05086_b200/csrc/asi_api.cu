@@ -117,7 +117,11 @@ void choose_kernels(asi_plan* pl) {
 
 // Workspace layouts.  Every region is 256-byte aligned; region 0 holds the status word (byte 0)
 // and the completion counter of the core kernel (byte 64).
-void layout_compress(asi_plan* pl) {
+//   kSeparate  regions side by side, a V as large as the largest mode's among them
+//   kShared    the core's intermediate tensors take the place of what the mode passes and Orthogonalize leave to one another
+//   kPlain     regions side by side as without k_mfiber, k_mplane and the batch-first core
+enum Layout { kSeparate, kShared, kPlain };
+void layout_compress(asi_plan* pl, Layout how) {
   size_t off = kStatusBytes;
   int rmax = 0;
   for (int m = 0; m < pl->nd; ++m) rmax = std::max(rmax, pl->r[m]);
@@ -166,7 +170,9 @@ void layout_compress(asi_plan* pl) {
     }
   // these copy rows on 16 bytes, and so did the kernel that 28 x 28 planes had: such layers want the address on 16 bytes
   const int64_t planes = pl->dims[0] * (pl->nd > 1 ? pl->dims[1] : 1);
-  pl->rows16 = pl->plane2 || (pl->plane && pl->dims[2] == 28 && pl->dims[3] == 28 && pl->r[2] <= 4 && pl->r[3] <= 4 && planes % 8 == 0);
+  const bool plane28 = pl->plane && pl->dims[2] == 28 && pl->dims[3] == 28 && pl->r[2] <= 4 && pl->r[3] <= 4 && planes % 8 == 0;
+  if (plane28 && how == kPlain) pl->plane_grid = plane2_grid(28, planes, (pl->d.flags & ASI_FLAG_SHARE_SM) ? 148 : 296);
+  pl->rows16 = pl->plane2 || plane28;
   for (int m = 0; m < pl->nd; ++m) pl->rows16 = pl->rows16 || pl->fiber2[m];
   // the factor on the tensor cores: the first two modes of conv layers, the batch of token layers where it fills the tiles (a batch
   // of 8 leaves half of each empty: 8 x 512 x 5632 bf16, ranks 8, 36 us against 29 of k_fiber_reg; 32 x 197 x 3072 16 against 28).
@@ -174,19 +180,21 @@ void layout_compress(asi_plan* pl) {
   pl->mplane = false;
   for (int m = 0; m < ASI_MAX_MODES; ++m) pl->mfiber[m] = false;
   const bool share = (pl->d.flags & ASI_FLAG_SHARE_SM) != 0;
-  if (pl->plane && mplane_supported(pl->dims[0] * pl->dims[1], pl->dims[2], pl->dims[3], pl->r[2], pl->r[3], pl->bf16)) {
+  if (pl->plane && how != kPlain && mplane_supported(pl->dims[0] * pl->dims[1], pl->dims[2], pl->dims[3], pl->r[2], pl->r[3], pl->bf16)) {
     pl->mplane = true;
     pl->plane_grid = mplane_grid(pl->dims[0] * pl->dims[1], (int)pl->dims[2], (int)pl->dims[3], std::max(pl->r[2], pl->r[3]),
                                  pl->bf16, share);
   }
-  if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY))
+  if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && how != kPlain)
     for (int m = 0; m < (pl->d.kind == ASI_CONV2D ? 2 : 1); ++m) {
       const ModeView& v = pl->mv[m];
       if (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m] || v.a <= 8)) continue;
       if (!mfiber_supported(v.O, v.a, v.I, v.r, pl->bf16) || (pl->bf16 && !pl->wfiber[m] && !pl->fiber2[m])) continue;
       pl->mfiber[m] = pl->fiber[m] = true;
       pl->fiber_grid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
+      if (v.a > 128) pl->fiber_grid[m] -= pl->fiber_grid[m] * pl->long_cut / 16;
     }
+  const size_t passes = off;                          // what the mode passes and Orthogonalize leave to one another: from here
   // V_m of the modes without a one-pass kernel, one region each (their products share launches); at least the
   // largest V of the layer
   if (!pl->fast_compress) {
@@ -197,7 +205,7 @@ void layout_compress(asi_plan* pl) {
       vmax = std::max(vmax, bytes);
       if (!pl->fiber[m] && !(pl->plane && m >= 2)) used += bytes;
     }
-    off += std::max(used, vmax);
+    off += how == kShared ? used : std::max(used, vmax);
   }
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
@@ -228,6 +236,41 @@ void layout_compress(asi_plan* pl) {
     const size_t shares = (pl->fast_compress || pl->small_rank) ? (size_t)pl->nchunk[m] * v.r * v.r : 0;   // k_sm_reduce's
     off = align_up(off + std::max(shares, orth_gp_elems(pl->nchunk[m], v.r)) * 8, 256);
   }
+  // core chain: contract the mode with the largest a_m / r_m first, then the rest in order
+  int order[ASI_MAX_MODES];
+  for (int m = 0; m < pl->nd; ++m) order[m] = m;
+  int best = 0;
+  for (int m = 1; m < pl->nd; ++m)
+    if ((double)pl->dims[m] / pl->r[m] > (double)pl->dims[best] / pl->r[best]) best = m;
+  // linear layers: the feature mode first where that shrinks the tensor by four at least (k_core_tok does the rest)
+  if (pl->d.kind == ASI_LINEAR && (pl->nd == 2 || pl->dims[pl->nd - 1] >= 4 * pl->r[pl->nd - 1])) best = pl->nd - 1;
+  // conv layers whose core k_core_tail finishes: the batch first where that shrinks the tensor by four at least (50 x 116 x 27 x 27,
+  // ranks 5: 91.0 -> 85.9 us a step; the channels first are three grouped products more)
+  const bool tail = pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
+                    core_tail_supported(pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[2], (int)pl->dims[3]);
+  if (tail && how != kPlain && pl->dims[0] >= 4 * (int64_t)pl->r[0]) best = 0;
+  std::swap(order[0], order[best]);
+  std::sort(order + 1, order + pl->nd);
+  std::memcpy(pl->core_order, order, sizeof(order));
+  int64_t cd[ASI_MAX_MODES];
+  for (int m = 0; m < pl->nd; ++m) cd[m] = pl->dims[m];
+  int64_t tmax[2] = {0, 0};
+  for (int s = 0; s + 1 < pl->nd; ++s) {
+    cd[order[s]] = pl->r[order[s]];
+    int64_t n = 1;
+    for (int m = 0; m < pl->nd; ++m) n *= cd[m];
+    tmax[s & 1] = std::max(tmax[s & 1], n);
+  }
+  if (pl->fast_compress) {
+    tmax[0] = pl->dims[1] * (pl->core_elems / pl->r[1]);        // per-channel shares
+    tmax[1] = (int64_t)((pl->n_tiles_core + pl->fold_gs - 1) / pl->fold_gs) * pl->core_elems;
+  }
+  size_t t_off = how == kShared && !pl->fast_compress ? passes : off;   // the first of them is written behind all of Orthogonalize
+  for (int t = 0; t < 2; ++t) {
+    pl->off_T[t] = t_off;
+    t_off = align_up(t_off + (size_t)tmax[t] * 4, 256);
+  }
+  off = std::max(off, t_off);
   // Tensor-core products of bf16 tensors: a factor of 16..64 columns (a multiple of 4) over the last mode (a_m a
   // multiple of 64, at least 128 fibers) or over a mode whose inner extent is a multiple of 64
   for (int m = 0; m < pl->nd; ++m) {
@@ -249,39 +292,6 @@ void layout_compress(asi_plan* pl) {
       pl->off_Pg[m] = off;
       off = align_up(off + (size_t)pl->dims[m] * pl->r[m] * 8, 256);
     }
-  // core chain: contract the mode with the largest a_m / r_m first, then the rest in order
-  int order[ASI_MAX_MODES];
-  for (int m = 0; m < pl->nd; ++m) order[m] = m;
-  int best = 0;
-  for (int m = 1; m < pl->nd; ++m)
-    if ((double)pl->dims[m] / pl->r[m] > (double)pl->dims[best] / pl->r[best]) best = m;
-  // linear layers: the feature mode first where that shrinks the tensor by four at least (k_core_tok does the rest)
-  if (pl->d.kind == ASI_LINEAR && (pl->nd == 2 || pl->dims[pl->nd - 1] >= 4 * pl->r[pl->nd - 1])) best = pl->nd - 1;
-  // conv layers whose core k_core_tail finishes: the batch first where that shrinks the tensor by four at least (50 x 116 x 27 x 27,
-  // ranks 5: 91.0 -> 85.9 us a step; the channels first are three grouped products more)
-  const bool tail = pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
-                    core_tail_supported(pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[2], (int)pl->dims[3]);
-  if (tail && pl->dims[0] >= 4 * (int64_t)pl->r[0]) best = 0;
-  std::swap(order[0], order[best]);
-  std::sort(order + 1, order + pl->nd);
-  std::memcpy(pl->core_order, order, sizeof(order));
-  int64_t cd[ASI_MAX_MODES];
-  for (int m = 0; m < pl->nd; ++m) cd[m] = pl->dims[m];
-  int64_t tmax[2] = {0, 0};
-  for (int s = 0; s + 1 < pl->nd; ++s) {
-    cd[order[s]] = pl->r[order[s]];
-    int64_t n = 1;
-    for (int m = 0; m < pl->nd; ++m) n *= cd[m];
-    tmax[s & 1] = std::max(tmax[s & 1], n);
-  }
-  if (pl->fast_compress) {
-    tmax[0] = pl->dims[1] * (pl->core_elems / pl->r[1]);        // per-channel shares
-    tmax[1] = (int64_t)((pl->n_tiles_core + pl->fold_gs - 1) / pl->fold_gs) * pl->core_elems;
-  }
-  for (int t = 0; t < 2; ++t) {
-    pl->off_T[t] = off;
-    off = align_up(off + (size_t)tmax[t] * 4, 256);
-  }
   pl->core_tail = pl->core_tok = false;
   pl->off_ctp = off;
   if (tail && order[0] == 0) {                       // the others follow in order
@@ -306,6 +316,25 @@ void layout_compress(asi_plan* pl) {
     if (tc) pl->launches_compress += 3;              // operand split, projections, expansions
     if (simt) pl->launches_compress += 2;
   }
+}
+
+// asi_compress_static_ws takes the layers whose workspace fits its 4 MiB with the mode passes of the fp32 pipe.  k_mfiber has a partial
+// of P for each of up to 296 CTAs also on modes of 129 to 384 entries, where the grouped products keep a few, and a batch-first
+// core larger intermediate tensors (three in a hundred of these layers grew past 4 MiB).  Such a layer shares its regions, and where that is
+// not enough (one in five thousand) up to half of the CTAs of its long modes go: 148 for 296 cost 8 x 364 x 28 x 56 4 of
+// 76 us, 9 x 230 x 36 x 36 2 of 63
+void fit_compress(asi_plan* pl) {
+  const auto fits = [&](Layout how) {
+    layout_compress(pl, how);
+    return pl->compress_ws <= (size_t)ASI_STATIC_WS_MAX_BYTES;
+  };
+  pl->long_cut = 0;
+  if (fits(kSeparate)) return;
+  if (fits(kPlain))
+    for (; pl->long_cut <= 8; ++pl->long_cut)
+      if (fits(kShared)) return;
+  pl->long_cut = 0;
+  layout_compress(pl, kSeparate);
 }
 
 void layout_wgrad(asi_plan* pl) {
@@ -928,7 +957,7 @@ asi_status_t asi_plan_create(const asi_layer_desc_t* desc, asi_plan_t** out) {
   }
   set_mode_views(pl);
   choose_kernels(pl);
-  layout_compress(pl);
+  fit_compress(pl);
   layout_wgrad(pl);
   {
     std::lock_guard<std::mutex> lock(g_lane_mu);

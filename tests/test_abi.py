@@ -91,6 +91,22 @@ def test_bf16_plans_pick_the_tensor_core_products_by_shape(asi, dims, ranks, on_
     assert tc.launch_count(1) == f32.launch_count(1) + (1 if token_mode_on_tc else 0)
 
 
+@pytest.mark.parametrize("dims,ranks,bf16,flags", [
+    ((28, 92, 28, 28), (6, 8, 5, 8), True, 0),          # batch-first core, two strided modes and planes
+    ((8, 364, 28, 56), (1, 7, 4, 2), False, 0),         # a long mode, a partial of P for each CTA
+    ((11, 300, 56, 28), (1, 7, 5, 4), False, 0),
+    ((38, 196, 20, 20), (8, 6, 3, 5), False, 0),
+    ((90, 7, 36, 36), (16, 7, 8, 2), True, 0),          # a mode of grouped products beside them
+    ((9, 274, 24, 24), (2, 8, 12, 8), False, 0),        # fits with fewer CTAs on the long mode
+    ((195, 15, 17, 17), (8, 8, 2, 16), False, 0),
+    ((215, 14, 17, 40), (4, 4, 4, 16), False, 4),
+])
+def test_layers_that_fit_the_built_in_workspace(asi, dims, ranks, bf16, flags):
+    """Layers near its 4 MiB: what the passes leave to one another and the core's intermediate tensors share memory."""
+    p = asi.Plan("conv", dims, ranks, cout=16, k=3, stride=1, pad=1, bf16=bf16, flags=flags)
+    assert p.info.compress_ws_bytes <= 4 << 20
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(dims=(8, 32, 16, 16), ranks=(9, 8, 8, 8)), 3),            # r_1 > a_1
     (dict(dims=(8, 32, 16, 16), ranks=(0, 8, 8, 8)), 3),

@@ -280,3 +280,23 @@ def test_expired_waits_are_reported_and_the_workspace_recovers(kind, dims, ranks
     err, _ = compare_step(run, L, A, dY, U_prev)
     check(err, TOL_F32, f"{dims} after an expired wait")
     assert run.device_status() == 0
+
+
+@pytest.mark.parametrize("dims,ranks,bf16", [((28, 92, 28, 28), (6, 8, 5, 8), True), ((11, 300, 56, 28), (1, 7, 5, 4), False),
+                                             ((9, 274, 24, 24), (2, 8, 12, 8), False)])
+def test_built_in_workspace(dims, ranks, bf16):
+    """Layers near its 4 MiB, whose scratch regions take one another's place: the same bits as with a workspace of the caller's,
+    whatever it held before."""
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    run = make_runner(L, bf16=bf16)
+    rng = np.random.default_rng(4)
+    run.set_factors([np.linalg.qr(rng.standard_normal((d, r)))[0] for d, r in zip(dims, ranks)])
+    act = run.to_device(rng.standard_normal(dims))
+    run.ws_c.fill_(0xff)
+    run.compress(act)
+    assert run.ok()
+    U, core = torch.empty_like(run.U[0]), torch.empty_like(run.core)
+    for _ in range(2):
+        run.plan.compress_static_ws(act.data_ptr(), run.U[0].data_ptr(), U.data_ptr(), core.data_ptr(),
+                                    int(torch.cuda.current_stream().cuda_stream))
+        assert torch.equal(U, run.U[1]) and torch.equal(core, run.core)
