@@ -303,9 +303,11 @@ void layout_compress(asi_plan* pl, Layout how) {
   pl->launches_compress = 3;
   if (!pl->fast_compress) {
     pl->core_tok = pl->d.kind == ASI_LINEAR && (pl->nd == 2 || order[0] == 2);
-    // the kernels of Orthogonalize (one for ranks up to eight), the core chain, one launch per one-pass mode (one for both
+    // the kernels of Orthogonalize (one for ranks up to eight and up to kSolveRows rows), the core chain, one launch per one-pass mode (one for both
     // spatial modes), one projection and one expansion launch for all SIMT modes together
-    pl->launches_compress = (pl->small_rank ? 1 : 2) + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
+    bool wide = false;
+    for (int m = 0; m < pl->nd; ++m) wide = wide || pl->dims[m] > kSolveRows;
+    pl->launches_compress = (pl->small_rank && !wide ? 1 : 2) + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
     bool simt = false, tc = false;
     for (int m = 0; m < pl->nd; ++m) {
       if (pl->plane && m >= 2) pl->launches_compress += (m == 2);
@@ -536,8 +538,27 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
   if (pl->small_rank) {
     SmReduceArgs ra;
     max_chunks = build_fused_reduce(pl, w, nullptr, &ra);
-    for (int m = 0; m < pl->nd; ++m) ra.m[m].U = U_new + pl->u_off[m];
+    // Up to kSolveRows rows a mode the CTA that factors it solves for them too.  Longer modes are products with few partials, which 512
+    // threads reduce no faster, and their rows take the machine: two launches (one layer's compress, one CTA against these:
+    // 512 x 384 rank 4 42.7 us, 41.0; 512 x 1024 rank 8 43.0, 38.9; 128 x 4096 rank 8 88.3, 62.5; 128 x 14336 rank 8 213, 118)
+    RowSolveArgs rs;
+    std::memset(&rs, 0, sizeof(rs));
+    bool wide = false;
+    for (int m = 0; m < pl->nd; ++m) wide = wide || pl->dims[m] > kSolveRows;
+    for (int m = 0; m < pl->nd; ++m) {
+      float* const U = U_new + pl->u_off[m];
+      if (!wide) ra.m[m].U = U;
+      rs.Pred[m] = ra.m[m].Pred;
+      rs.U[m] = U;
+      rs.a[m] = (int)pl->dims[m];
+      rs.r[m] = pl->r[m];
+      rs.total += rs.a[m];
+    }
+    rs.Rf = ra.Rf;
+    rs.nd = pl->nd;
+    ra.large = !wide;
     ASI_CUDA(launch_sm_reduce(ra, pl->nd, max_chunks, st));
+    if (wide) ASI_CUDA(launch_row_solve(rs, st));
     return ASI_OK;
   }
   QRArgs qa;

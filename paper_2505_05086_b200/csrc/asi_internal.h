@@ -96,6 +96,14 @@ struct QRArgs {
   QRMode m[ASI_MAX_MODES];
   int* status;
 };
+// U_m = P_m R_m^{-1} for ranks <= 8, one row per thread, from what k_sm_reduce left (P_m and the Cholesky factor)
+struct RowSolveArgs {
+  const double* Pred[ASI_MAX_MODES];   // [a][r]
+  const double* Rf;                    // [modes][kRfStride]
+  float* U[ASI_MAX_MODES];
+  int a[ASI_MAX_MODES], r[ASI_MAX_MODES];
+  int nd, total;                       // total = sum of a
+};
 // Z4[c', j, kh, kw] = sum_{i,h',w'} Z1[i,c',h',w'] Z3pad[i,j,h's+kh-p,w's+kw-p], then
 // dW[c', cl, kh, kw] = sum_j Z4[c', j, kh, kw] U2[(g*cg + cl), j].
 struct ConvTailArgs {
@@ -144,12 +152,14 @@ struct SmReduceMode {
   double* Gp;          // [nchunk][r][r]
   double* Pg;          // gram != 0 and factor != 0: [a][r], P_m = G_m U_m^prev
   const float* U_prev; // gram != 0 and factor != 0: U_m^prev [a][r]
-  float* U;            // not null (gram == 0, factor != 0): U_m [a][r] is written here
+  float* U;            // large: U_m [a][r] is written here
   int a, r, nsplit, nchunk, gram;
 };
+constexpr int kSolveRows = 384;  // rows a mode that the CTA which factors it solves for: what k_mfiber takes, whose partials are many
 constexpr int kRfStride = 80;   // doubles per mode in Rf: rows of R_m at pitch 8, then 1 / diag(R_m) at [64..72)
 struct SmReduceArgs {
   SmReduceMode m[ASI_MAX_MODES];
+  int large;           // != 0: k_sm_reduce_large (gram == 0, factor != 0, at most kSolveRows rows a mode)
   int factor;          // != 0: the last CTA of each mode factors G_m = R_m^T R_m into Rf (ranks <= 8)
   double* Rf;          // [modes][kRfStride]
   int* counter;        // one per mode, zero on entry, zero again on exit
@@ -374,6 +384,7 @@ int orth_rows(int64_t a, int r, int64_t nsplit);
 size_t orth_gp_elems(int64_t nchunk, int r);
 cudaError_t launch_orth(const QRArgs& p, int nd, cudaStream_t st);
 cudaError_t launch_qr_big(const QRArgs& p, int nd, cudaStream_t st);
+cudaError_t launch_row_solve(const RowSolveArgs& p, cudaStream_t st);
 cudaError_t launch_fiber(const FiberArgs& p, int grid, bool x_bf16, cudaStream_t st);
 size_t fiber_smem(int a);
 bool wfiber_supported(int64_t O, int64_t a, int64_t I, int r);

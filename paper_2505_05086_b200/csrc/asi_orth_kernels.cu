@@ -383,6 +383,38 @@ __global__ void __launch_bounds__(kAT) k_orth_apply(const __grid_constant__ QRAr
   }
 }
 
+// One row of one factor per thread: u = p R^{-1} with the Cholesky factor that k_sm_reduce left (ranks <= 8).
+__global__ void __launch_bounds__(128) k_row_solve(const __grid_constant__ RowSolveArgs p) {
+  pdl_launch_dependents();
+  pdl_wait();
+  __shared__ double Rs[ASI_MAX_MODES][kRfStride];
+  for (int e = threadIdx.x; e < p.nd * kRfStride; e += 128) (&Rs[0][0])[e] = __ldcg(p.Rf + e);
+  int row = blockIdx.x * 128 + threadIdx.x, m = 0;
+  while (m + 1 < p.nd && row >= p.a[m]) row -= p.a[m++];
+  const bool on = row < p.a[m];
+  const int r = p.r[m];
+  double q[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) q[j] = (on && j < r) ? __ldcg(p.Pred[m] + (int64_t)row * r + j) : 0.0;
+  __syncthreads();
+  if (!on) return;
+  const double* R = Rs[m];
+  float* dst = p.U[m] + (int64_t)row * r;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < r) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < j) q[j] = fma(-q[i], R[i * 8 + j], q[j]);
+      q[j] *= R[64 + j];
+      dst[j] = (float)q[j];
+    }
+}
+
+cudaError_t launch_row_solve(const RowSolveArgs& p, cudaStream_t st) {
+  return launch_pdl(k_row_solve, dim3((unsigned)((p.total + 127) / 128)), dim3(128), 0, st, p);
+}
+
 // rows of P per CTA of k_orth_factor: about 64 partial loads per thread, so that many splits (the token mode: 40)
 // mean short chunks and few splits (a long feature mode) few shares of G
 int orth_rows(int64_t a, int r, int64_t nsplit) {

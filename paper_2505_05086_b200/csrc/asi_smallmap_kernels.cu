@@ -26,6 +26,7 @@ namespace {
 // threads per CTA of the partial-reduction kernel: fused layers (whose grids have many CTAs that end at once: MobileNetV2 tail 16.6 us,
 // 20.4 with 512 threads), and the layers of large maps
 constexpr int kRedNT = 256, kRedNTLarge = 512;
+static_assert(kSolveRows <= kRedNTLarge, "a row a thread");
 
 
 // ---- bulk-copy engine (TMA, untiled form) and mbarrier ------------------------------------------
@@ -1255,8 +1256,8 @@ __global__ void __launch_bounds__(kPT, R == 4 ? 4 : 2) k_sm_pass1_b(const __grid
 // Gram matrices A_m A_m^T (a <= 16) is summed the same way, a slice of the a x a elements per CTA.
 // With args.factor the last CTA of a mode to finish then factors the mode once for all CTAs of the
 // core kernel: it sums the shares of P_m^T P_m (a Gram mode: forms P_m = G_m U_m^prev first), and
-// leaves the Cholesky factor R_m and 1 / diag(R_m) in args.Rf; with M.U it also solves for the rows of U_m.
-// LARGE (the layers of large maps, 148 to 296 partials a mode): a chain of round trips to memory, so 512 threads with sixteen
+// leaves the Cholesky factor R_m and 1 / diag(R_m) in args.Rf; LARGE also solves for the rows of U_m.
+// LARGE (the layers of large maps, 148 to 296 partials a mode, at most kSolveRows rows): a chain of round trips to memory, so 512 threads with sixteen
 // partials each in flight, and the rows solved here: 10.7 us where 256 threads took 11.7 and a launch for the rows 3.5 more
 // (128 x 128 x 28 x 28 bf16, one layer's step 91.3 -> 89.2 us).  Fused layers lose by it (MobileNetV2 tail 165 -> 168 us).
 // ---------------------------------------------------------------------------------------------
@@ -1422,27 +1423,19 @@ __device__ __forceinline__ void sm_reduce_cta(const SmReduceArgs& args, const in
   if constexpr (!LARGE) return;
   // ---- U_m = P_m R_m^{-1}, a row per thread (a launch of its own took 3.5 us of the chain)
   __syncthreads();
-  double nx[RM];                                     // the next row is on its way while one is solved
-  auto fetch = [&](int row) {
+  if (tid >= a) return;
+  double q[RM];
 #pragma unroll
-    for (int j = 0; j < RM; ++j) nx[j] = (row < a && j < r) ? __ldcg(M.Pred + (int64_t)row * r + j) : 0.0;
-  };
-  fetch(tid);
-  for (int row = tid; row < a; row += NT) {
-    double q[RM];
+  for (int j = 0; j < RM; ++j) q[j] = j < r ? __ldcg(M.Pred + (int64_t)tid * r + j) : 0.0;
 #pragma unroll
-    for (int j = 0; j < RM; ++j) q[j] = nx[j];
-    fetch(row + NT);
+  for (int j = 0; j < RM; ++j)
+    if (j < r) {
 #pragma unroll
-    for (int j = 0; j < RM; ++j)
-      if (j < r) {
-#pragma unroll
-        for (int i = 0; i < RM; ++i)
-          if (i < j) q[j] = fma(-q[i], Gs[i][j], q[j]);
-        q[j] *= Dinv[j];
-        M.U[(int64_t)row * r + j] = (float)q[j];
-      }
-  }
+      for (int i = 0; i < RM; ++i)
+        if (i < j) q[j] = fma(-q[i], Gs[i][j], q[j]);
+      q[j] *= Dinv[j];
+      M.U[(int64_t)tid * r + j] = (float)q[j];
+    }
 }
 
 __global__ void __launch_bounds__(kRedNT) k_sm_reduce(const __grid_constant__ SmReduceArgs args) {
@@ -1462,7 +1455,7 @@ cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cuda
     bytes += 4.0 * p.m[m].nsplit * p.m[m].a * (p.m[m].gram ? p.m[m].a : p.m[m].r) + 8.0 * p.m[m].a * p.m[m].r;
   ProfScope prof(ASI_K_QR, st, bytes);
   dim3 grid((unsigned)max_chunks, (unsigned)nd);
-  if (p.m[0].U) return launch_pdl(k_sm_reduce_large, grid, dim3(kRedNTLarge), 0, st, p);
+  if (p.large) return launch_pdl(k_sm_reduce_large, grid, dim3(kRedNTLarge), 0, st, p);
   return launch_pdl(k_sm_reduce, grid, dim3(kRedNT), 0, st, p);
 }
 

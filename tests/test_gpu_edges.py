@@ -153,3 +153,13 @@ def test_tensors_that_start_at_any_element(case, bf16, shift):
     with pytest.raises(Exception, match="invalid argument"):      # half an element is refused, not read
         run.plan.wgrad(run.core.data_ptr(), run.U[run.cur].data_ptr(), to_device(dY).data_ptr() + 1, run.dW.data_ptr(),
                        run.ws_w.data_ptr(), run.ws_w.numel())
+
+
+@pytest.mark.parametrize("dims,ranks,split", [((24, 384), (5, 5), False), ((24, 385), (5, 5), True), ((520, 40), (8, 8), True),
+                                              ((6, 20, 1300), (3, 8, 8), True)])
+def test_rows_of_the_factors_on_both_sides_of_the_factoring_cta(dims, ranks, split):
+    """Ranks up to eight: 384 rows are solved by the CTA that factors the mode, more in a launch of their own."""
+    L = LayerSpec("t", "linear", dims, 37, ranks=ranks)
+    run, short = make_runner(L), make_runner(LayerSpec("t", "linear", tuple(min(d, 384) for d in dims), 37, ranks=ranks))
+    assert run.plan.launch_count(0) == short.plan.launch_count(0) + split
+    _two_steps(L, False)
