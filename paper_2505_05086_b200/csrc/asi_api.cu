@@ -174,8 +174,9 @@ void layout_compress(asi_plan* pl, Layout how) {
   if (plane28 && how == kPlain) pl->plane_grid = plane2_grid(28, planes, (pl->d.flags & ASI_FLAG_SHARE_SM) ? 148 : 296);
   pl->rows16 = pl->plane2 || plane28;
   for (int m = 0; m < pl->nd; ++m) pl->rows16 = pl->rows16 || pl->fiber2[m];
-  // the factor on the tensor cores: the first two modes of conv layers, the batch of token layers where it fills the tiles (a batch
-  // of 8 leaves half of each empty: 8 x 512 x 5632 bf16, ranks 8, 36 us against 29 of k_fiber_reg; 32 x 197 x 3072 16 against 28).
+  // the factor on the tensor cores: the first two modes of conv layers and the batch of token layers, where they fill the tiles (a
+  // mode of 8 leaves half of each empty: 8 x 512 x 5632 bf16, ranks 8, 36 us against 29 of k_fiber_reg; 32 x 197 x 3072 16 against 28;
+  // compress of 8 x 700 x 56 x 56 161 us against 140, of 10 x 700 x 56 x 56 182 against 178, of 10 x 64 x 28 x 28 29 against 30).
   // Not the rows of a matrix: few columns average the operands' rounding less (82 x 958: 9.3e-8 against 5.1e-8)
   pl->mplane = false;
   for (int m = 0; m < ASI_MAX_MODES; ++m) pl->mfiber[m] = false;
@@ -188,7 +189,7 @@ void layout_compress(asi_plan* pl, Layout how) {
   if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && how != kPlain)
     for (int m = 0; m < (pl->d.kind == ASI_CONV2D ? 2 : 1); ++m) {
       const ModeView& v = pl->mv[m];
-      if (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m] || v.a <= 8)) continue;
+      if (v.a <= 8 || (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m]))) continue;
       if (!mfiber_supported(v.O, v.a, v.I, v.r, pl->bf16) || (pl->bf16 && !pl->wfiber[m] && !pl->fiber2[m])) continue;
       pl->mfiber[m] = pl->fiber[m] = true;
       pl->fiber_grid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
