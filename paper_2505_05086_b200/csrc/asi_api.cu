@@ -115,6 +115,20 @@ void choose_kernels(asi_plan* pl) {
   }
 }
 
+// The core of a conv layer, batch first: one streamed product that leaves t1 values, then k_core_tail, where the mode with the largest
+// a_m / r_m first leaves fewer and takes two grouped products more.  The other side of each line, one layer's compress in us:
+//   the batch product is streamed: 16 x 64 x 28 x 28 ranks 3 41.3 against 34.5, where it would be a grouped one
+//   up to 128 channels their product is streamed too, so t1 must be small (ranks 8 4: 32 x 128 x 56 x 56 95 against 89; 32 x 128 x 28 x 28
+//   51 against 54), and so must the rank of a long fp32 batch (128 x 128 x 28 x 28 ranks 8 4: 88.6 against 83.2; 64 x 128 x 28 x 28 65 against 67)
+//   beyond, the channels are a grouped product, and a large t1 costs only fp32 layers whose batch hardly shrinks (24 x 768 x 28 x 28
+//   ranks 6 6: 151 against 136; 64 x 512 x 28 x 28 ranks 8 4 200 against 204; 32 x 512 x 28 x 28 bf16 118 against 122)
+bool batch_first(const asi_plan* pl) {
+  const int64_t B = pl->dims[0], C = pl->dims[1], chw = C * pl->dims[2] * pl->dims[3], r1 = pl->r[0], t1 = r1 * chw;
+  if (B < 4 * r1 || pl->N < (1 << 20) || !wfiber_supported(1, B, chw, pl->r[0])) return false;
+  if (C <= 128) return t1 <= (2 << 20) && (pl->bf16 || B <= 64 || r1 <= 4 || pl->r[1] > 4);
+  return pl->bf16 || C < 512 || B >= 8 * r1 || t1 <= (int64_t)(r1 > 4 ? 7 : 9) << 18;
+}
+
 // Workspace layouts.  Every region is 256-byte aligned; region 0 holds the status word (byte 0)
 // and the completion counter of the core kernel (byte 64).
 //   kSeparate  regions side by side, a V as large as the largest mode's among them
@@ -245,11 +259,10 @@ void layout_compress(asi_plan* pl, Layout how) {
     if ((double)pl->dims[m] / pl->r[m] > (double)pl->dims[best] / pl->r[best]) best = m;
   // linear layers: the feature mode first where that shrinks the tensor by four at least (k_core_tok does the rest)
   if (pl->d.kind == ASI_LINEAR && (pl->nd == 2 || pl->dims[pl->nd - 1] >= 4 * pl->r[pl->nd - 1])) best = pl->nd - 1;
-  // conv layers whose core k_core_tail finishes: the batch first where that shrinks the tensor by four at least (50 x 116 x 27 x 27,
-  // ranks 5: 91.0 -> 85.9 us a step; the channels first are three grouped products more)
+  // conv layers whose core k_core_tail finishes: the batch first where that pays
   const bool tail = pl->d.kind == ASI_CONV2D && !pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) &&
                     core_tail_supported(pl->r[1], pl->r[2], pl->r[3], (int)pl->dims[2], (int)pl->dims[3]);
-  if (tail && how != kPlain && pl->dims[0] >= 4 * (int64_t)pl->r[0]) best = 0;
+  if (tail && how != kPlain && batch_first(pl)) best = 0;
   std::swap(order[0], order[best]);
   std::sort(order + 1, order + pl->nd);
   std::memcpy(pl->core_order, order, sizeof(order));

@@ -107,6 +107,26 @@ def test_layers_that_fit_the_built_in_workspace(asi, dims, ranks, bf16, flags):
     assert p.info.compress_ws_bytes <= 4 << 20
 
 
+@pytest.mark.parametrize("dims,ranks,bf16,first", [
+    ((16, 64, 28, 28), (3, 3, 3, 3), False, False),     # below a million values the batch product is a grouped one
+    ((24, 64, 28, 28), (3, 3, 3, 3), False, True),
+    ((24, 64, 28, 28), (7, 3, 3, 3), False, False),     # shrinks by less than four
+    ((32, 128, 56, 56), (4, 8, 4, 4), False, True),
+    ((32, 128, 56, 56), (8, 4, 4, 4), False, False),    # three million values left
+    ((128, 128, 28, 28), (5, 4, 4, 4), False, False),   # a long batch of rank above four
+    ((128, 128, 28, 28), (5, 4, 4, 4), True, True),
+    ((24, 768, 28, 28), (3, 3, 3, 3), False, True),
+    ((24, 768, 28, 28), (5, 3, 3, 3), False, False),    # three million values of four times that
+    ((24, 768, 28, 28), (5, 3, 3, 3), True, True),
+    ((160, 300, 20, 20), (3, 4, 4, 4), False, False),   # a batch that is not streamed
+])
+def test_core_contracts_the_batch_first_where_that_pays(asi, dims, ranks, bf16, first):
+    """Both sides of the lines: batch first the core is two launches, else a mode product each.  Before it: the planes, the batch, the
+    channels and one reduction; of more than 384 channels two grouped products and two reductions."""
+    p = asi.Plan("conv", dims, ranks, cout=16, k=3, stride=1, pad=1, bf16=bf16)
+    assert p.launch_count(0) == (6 if dims[1] > 384 else 4) + (2 if first else 4)
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(dims=(8, 32, 16, 16), ranks=(9, 8, 8, 8)), 3),            # r_1 > a_1
     (dict(dims=(8, 32, 16, 16), ranks=(0, 8, 8, 8)), 3),
