@@ -129,6 +129,13 @@ bool batch_first(const asi_plan* pl) {
   return pl->bf16 || C < 512 || B >= 8 * r1 || t1 <= (int64_t)(r1 > 4 ? 7 : 9) << 18;
 }
 
+// ranks up to eight: the rows of the factors are solved for in a launch of their own
+bool solves_wide(const asi_plan* pl) {
+  int64_t most = 0;
+  for (int m = 0; m < pl->nd; ++m) most = std::max(most, pl->dims[m]);
+  return most > (pl->d.kind == ASI_CONV2D ? kSolveRows : kSolveRowsTokens);
+}
+
 // Workspace layouts.  Every region is 256-byte aligned; region 0 holds the status word (byte 0)
 // and the completion counter of the core kernel (byte 64).
 //   kSeparate  regions side by side, a V as large as the largest mode's among them
@@ -317,11 +324,9 @@ void layout_compress(asi_plan* pl, Layout how) {
   pl->launches_compress = 3;
   if (!pl->fast_compress) {
     pl->core_tok = pl->d.kind == ASI_LINEAR && (pl->nd == 2 || order[0] == 2);
-    // the kernels of Orthogonalize (one for ranks up to eight and up to kSolveRows rows), the core chain, one launch per one-pass mode (one for both
+    // the kernels of Orthogonalize (one for ranks up to eight where solves_wide does not say two), the core chain, one launch per one-pass mode (one for both
     // spatial modes), one projection and one expansion launch for all SIMT modes together
-    bool wide = false;
-    for (int m = 0; m < pl->nd; ++m) wide = wide || pl->dims[m] > kSolveRows;
-    pl->launches_compress = (pl->small_rank && !wide ? 1 : 2) + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
+    pl->launches_compress = (pl->small_rank && !solves_wide(pl) ? 1 : 2) + ((pl->core_tail || pl->core_tok) ? 2 : pl->nd);
     bool simt = false, tc = false;
     for (int m = 0; m < pl->nd; ++m) {
       if (pl->plane && m >= 2) pl->launches_compress += (m == 2);
@@ -552,13 +557,13 @@ asi_status_t orthogonalize_all(const asi_plan* pl, float* U_new, char* w, const 
   if (pl->small_rank) {
     SmReduceArgs ra;
     max_chunks = build_fused_reduce(pl, w, nullptr, &ra);
-    // Up to kSolveRows rows a mode the CTA that factors it solves for them too.  Longer modes are products with few partials, which 512
-    // threads reduce no faster, and their rows take the machine: two launches (one layer's compress, one CTA against these:
-    // 512 x 384 rank 4 42.7 us, 41.0; 512 x 1024 rank 8 43.0, 38.9; 128 x 4096 rank 8 88.3, 62.5; 128 x 14336 rank 8 213, 118)
+    // Few rows: the CTA that factors a mode solves for them too.  Longer modes are products with few partials, which 512 threads
+    // reduce no faster, and their rows take the machine: two launches (one layer's compress, one CTA against these:
+    // 512 x 384 rank 4 42.7 us, 41.0; 512 x 1024 rank 8 43.0, 38.9; 128 x 4096 rank 8 88.3, 62.5; 128 x 14336 rank 8 213, 118).
+    // Conv layers have the partials of the other modes: 32 x 512 x 20 x 20 ranks 3 74.9, 77.5; 8 x 1024 x 20 x 20 ranks 8 89, 85
     RowSolveArgs rs;
     std::memset(&rs, 0, sizeof(rs));
-    bool wide = false;
-    for (int m = 0; m < pl->nd; ++m) wide = wide || pl->dims[m] > kSolveRows;
+    const bool wide = solves_wide(pl);
     for (int m = 0; m < pl->nd; ++m) {
       float* const U = U_new + pl->u_off[m];
       if (!wide) ra.m[m].U = U;

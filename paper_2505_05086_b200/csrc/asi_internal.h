@@ -155,7 +155,9 @@ struct SmReduceMode {
   float* U;            // large: U_m [a][r] is written here
   int a, r, nsplit, nchunk, gram;
 };
-constexpr int kSolveRows = 384;  // rows a mode that the CTA which factors it solves for: what k_mfiber takes, whose partials are many
+// Rows a mode up to which k_sm_reduce_large, which solves for them too, takes a layer.  A conv layer: a row a thread.  Token layers: what
+// k_mfiber takes, whose partials are many
+constexpr int kSolveRows = 512, kSolveRowsTokens = 384;
 constexpr int kRfStride = 80;   // doubles per mode in Rf: rows of R_m at pitch 8, then 1 / diag(R_m) at [64..72)
 struct SmReduceArgs {
   SmReduceMode m[ASI_MAX_MODES];

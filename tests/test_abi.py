@@ -122,9 +122,9 @@ def test_layers_that_fit_the_built_in_workspace(asi, dims, ranks, bf16, flags):
 ])
 def test_core_contracts_the_batch_first_where_that_pays(asi, dims, ranks, bf16, first):
     """Both sides of the lines: batch first the core is two launches, else a mode product each.  Before it: the planes, the batch, the
-    channels and one reduction; of more than 384 channels two grouped products and two reductions."""
+    channels and one reduction; of more than 512 channels two grouped products and two reductions."""
     p = asi.Plan("conv", dims, ranks, cout=16, k=3, stride=1, pad=1, bf16=bf16)
-    assert p.launch_count(0) == (6 if dims[1] > 384 else 4) + (2 if first else 4)
+    assert p.launch_count(0) == (6 if dims[1] > 512 else 4) + (2 if first else 4)
 
 
 @pytest.mark.parametrize("kw,code", [

@@ -156,10 +156,13 @@ def test_tensors_that_start_at_any_element(case, bf16, shift):
 
 
 @pytest.mark.parametrize("dims,ranks,split", [((24, 384), (5, 5), False), ((24, 385), (5, 5), True), ((520, 40), (8, 8), True),
-                                              ((6, 20, 1300), (3, 8, 8), True)])
+                                              ((6, 20, 1300), (3, 8, 8), True), ((3, 512, 18, 18), (3, 8, 4, 4), False),
+                                              ((3, 513, 18, 18), (3, 4, 4, 4), True)])
 def test_rows_of_the_factors_on_both_sides_of_the_factoring_cta(dims, ranks, split):
-    """Ranks up to eight: 384 rows are solved by the CTA that factors the mode, more in a launch of their own."""
-    L = LayerSpec("t", "linear", dims, 37, ranks=ranks)
-    run, short = make_runner(L), make_runner(LayerSpec("t", "linear", tuple(min(d, 384) for d in dims), 37, ranks=ranks))
+    """Ranks up to eight: 384 rows (conv layers: 512) are solved by the CTA that factors the mode, more in a launch of their own."""
+    def layer(d):
+        return LayerSpec("t", "conv", d, 6, 3, 1, 1, 1, ranks=ranks) if len(d) == 4 else LayerSpec("t", "linear", d, 37, ranks=ranks)
+
+    run, short = make_runner(layer(dims)), make_runner(layer(tuple(min(d, 512 if len(dims) == 4 else 384) for d in dims)))
     assert run.plan.launch_count(0) == short.plan.launch_count(0) + split
-    _two_steps(L, False)
+    _two_steps(layer(dims), False)
