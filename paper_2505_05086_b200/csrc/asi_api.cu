@@ -200,7 +200,7 @@ void layout_compress(asi_plan* pl, Layout how) {
   // compress of 8 x 700 x 56 x 56 161 us against 140, of 10 x 700 x 56 x 56 182 against 178, of 10 x 64 x 28 x 28 29 against 30).
   // Not the rows of a matrix: few columns average the operands' rounding less (82 x 958: 9.3e-8 against 5.1e-8)
   pl->mplane = false;
-  for (int m = 0; m < ASI_MAX_MODES; ++m) pl->mfiber[m] = false;
+  for (int m = 0; m < ASI_MAX_MODES; ++m) pl->mfiber[m] = pl->cfiber[m] = false;
   const bool share = (pl->d.flags & ASI_FLAG_SHARE_SM) != 0;
   if (pl->plane && how != kPlain && mplane_supported(pl->dims[0] * pl->dims[1], pl->dims[2], pl->dims[3], pl->r[2], pl->r[3], pl->bf16)) {
     pl->mplane = true;
@@ -210,8 +210,10 @@ void layout_compress(asi_plan* pl, Layout how) {
   if (!pl->fast_compress && !(pl->d.flags & ASI_FLAG_GENERIC_ONLY) && how != kPlain)
     for (int m = 0; m < (pl->d.kind == ASI_CONV2D ? 2 : 1); ++m) {
       const ModeView& v = pl->mv[m];
-      if (v.a <= 8 || (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m]))) continue;
+      if (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m] || v.a <= 8)) continue;
       if (!mfiber_supported(v.O, v.a, v.I, v.r, pl->bf16) || (pl->bf16 && !pl->wfiber[m] && !pl->fiber2[m])) continue;
+      pl->cfiber[m] = v.a > 8 || pl->fiber[m];
+      if (v.a <= 8) continue;
       pl->mfiber[m] = pl->fiber[m] = true;
       pl->fiber_grid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
       if (v.a > 128) pl->fiber_grid[m] -= pl->fiber_grid[m] * pl->long_cut / 16;
@@ -843,12 +845,20 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
 
 // cold start: P_m = A_m Omega_m of all modes: one launch of SIMT products, one of tensor-core products, and the passes of the
 // modes that a warm step has on k_mfiber and k_mplane, which take Omega as their V (64 x 128 x 28 x 28 fp32, ranks 4: 72.1 -> 55.7 us).
+// These passes are launches of their own, so small tensors stay with the SIMT products (8 x 32 x 24 x 24 ranks 6 33 us with the passes,
+// 26 without; 16 x 115 x 24 x 24, a million values, 31 and 35).  Where SIMT products remain for another mode all the same, the line
+// lies at two million (15 x 70 x 32 x 33 51 and 46, 24 x 98 x 512 tokens 50 and 44; 49 x 40 x 40 x 40 52 and 56), but for batches of up
+// to eight, which these products take badly (3 x 163 x 56 x 56 57 and 66)
 // first: nothing of this call is enqueued yet; the first launch here zeroes the status block
 asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool first,
                           cudaStream_t st) {
   int* const status = reinterpret_cast<int*>(w);
   bool clear = first;
-  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0, mma = !pl->bf16 || on16;
+  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+  bool all = true;
+  for (int m = 0; m < pl->nd; ++m) all = all && (pl->cfiber[m] || (pl->mplane && m >= 2));
+  const bool early = all || (pl->d.kind == ASI_CONV2D && pl->dims[0] <= 8);
+  const bool mma = (!pl->bf16 || on16) && pl->N >= (early ? 1 << 20 : 1 << 21);
   const bool planes = pl->mplane && mma;
   GemmGroup g;
   g.np = 0;
@@ -857,7 +867,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
   TcCall t[3];
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
-    if ((pl->mfiber[m] && mma) || (planes && m >= 2)) continue;
+    if ((pl->cfiber[m] && mma) || (planes && m >= 2)) continue;
     if (pl->tc_mode[m] && on16) {
       t[sp.n] = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
                  pl->q_per_split[m], v.r, pl->nsplit[m], 1};
@@ -893,7 +903,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     clear = head = false;
   }
   for (int m = 0; m < pl->nd; ++m) {
-    if (!pl->mfiber[m] || !mma) continue;
+    if (!pl->cfiber[m] || !mma) continue;
     const ModeView& v = pl->mv[m];
     Fiber2Args f;
     std::memset(&f, 0, sizeof(f));

@@ -250,8 +250,8 @@ def test_a_factor_of_the_largest_values(dims, ranks, bf16):
     ("conv", (16, 130, 28, 28), (4, 4, 4, 4), False),          # planes, and teams of one and of three warps
     ("conv", (16, 130, 40, 40), (5, 6, 5, 5), False),          # strided fibers alone
     ("conv", (40, 48, 24, 24), (4, 4, 4, 4), True),
-    ("conv", (16, 40, 56, 56), (4, 4, 4, 4), False),           # the planes of their own kernel
-    ("linear", (33, 24, 64), (7, 8, 12), True),
+    ("conv", (16, 48, 56, 56), (4, 4, 4, 4), False),           # the planes of their own kernel
+    ("linear", (33, 64, 1024), (7, 8, 12), True),
 ])
 def test_expired_waits_are_reported_and_the_workspace_recovers(kind, dims, ranks, bf16, cold):
     """The producer arms its barriers and copies nothing; every wait runs out (1 ms), and the next call on the same workspace is
@@ -300,3 +300,49 @@ def test_built_in_workspace(dims, ranks, bf16):
         run.plan.compress_static_ws(act.data_ptr(), run.U[0].data_ptr(), U.data_ptr(), core.data_ptr(),
                                     int(torch.cuda.current_stream().cuda_stream))
         assert torch.equal(U, run.U[1]) and torch.equal(core, run.core)
+
+
+COLD = [  # (dims, ranks, bf16, launches of the passes): a million values with a pass for every mode, two million without
+    ((65, 60, 18, 19), (4, 4, 3, 2), False, 3),    # two warps a tile along the batch; odd rows along the channels
+    ((40, 130, 17, 17), (5, 8, 6, 7), False, 3),   # three warps, ranks above four, odd planes
+    ((17, 200, 20, 20), (3, 4, 4, 4), False, 3),   # two row tiles and one row more
+    ((12, 384, 17, 16), (3, 6, 5, 3), False, 3),   # the longest mode
+    ((40, 48, 24, 24), (4, 4, 4, 4), True, 3),
+    ((33, 128, 20, 20), (6, 5, 7, 5), True, 3),
+    ((13, 25, 56, 60), (4, 4, 4, 4), False, 0),    # planes without a pass: below two million the SIMT products do it all
+    ((30, 25, 56, 60), (4, 4, 4, 4), False, 2),
+    ((11, 70, 36, 36), (4, 6, 4, 4), True, 0),
+    ((9, 100, 24, 24), (4, 5, 4, 4), False, 0),    # a pass for every mode, half a million
+    ((8, 260, 24, 24), (4, 5, 4, 4), False, 3),    # a batch of eight: half a row tile, and only here
+    ((3, 120, 56, 60), (3, 5, 4, 4), False, 2),    # planes without a pass, but a batch below eight
+]
+
+
+@pytest.mark.parametrize("dims,ranks,bf16,passes", COLD)
+def test_cold_start_on_both_sides_of_the_passes(dims, ranks, bf16, passes):
+    import ctypes
+    from paper_2505_05086_b200.binding import lib
+    rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
+                     gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(dims, ranks)))
+    A, _ = st.next()
+    rng = np.random.default_rng(5)
+    n = int(np.prod(dims))
+    Omega = [rng.standard_normal((n // d, r)).astype(np.float32) for d, r in zip(dims, ranks)]
+    run = make_runner(L, bf16=bf16)
+    act, omega = run.to_device(A), torch.from_numpy(np.concatenate([o.ravel() for o in Omega])).cuda()
+    events = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    for e in events:
+        e.record()
+    lib().asi_profile_begin(2, (ctypes.c_void_p * 2)(*(e.cuda_event for e in events)), 1)   # ASI_K_EXPAND
+    try:
+        run.init_factors(act, omega)
+    finally:
+        seen = lib().asi_profile_end(None)
+    assert seen == passes
+    assert run.ok()
+    S_ref, U_ref = O.asi_cold_start(A.astype(np.float64), [o.astype(np.float64) for o in Omega])
+    U = run.factors()
+    assert max(O.rel_fro(O.projector(a), O.projector(b)) for a, b in zip(U, U_ref)) <= 1e-4
+    assert O.rel_fro(O.sign_align(run.core_np(), U, U_ref)[0], S_ref) <= 1e-4
