@@ -148,7 +148,7 @@ struct Acc {
 };
 
 // One entry of the B operand of the columns: lane group g is the column.  A NaN is lost in both roundings, but not in the difference:
-// x - (x - hi) is hi again, or NaN where x is NaN or infinite.  TOP (values of the caller's): what would round to infinity
+// x - (x - hi) is hi again, or NaN where x is NaN or infinite.  TOP (the previous factors): what would round to infinity
 // leaves more to the rest instead
 template <int NB, bool TOP>
 __device__ __forceinline__ void set_b(float* b, int half, int g, float x) {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
               for (int i = 0; i < 4; ++i) x[i] += y[i];
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) set_b<NB, GIVEN>(b[u + i], h, g, x[i]);
+            for (int i = 0; i < 4; ++i) set_b<NB, false>(b[u + i], h, g, x[i]);
           }
 #pragma unroll
         for (int m = 0; m < RT; ++m) {
@@ -773,7 +773,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) set_b<NB, GIVEN>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
+        for (int e = 0; e < 4; ++e) set_b<NB, false>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         if (m >= nkh) break;
@@ -823,8 +823,8 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
       float b4[2][2 * NB];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        set_b<NB, GIVEN>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
-        set_b<NB, GIVEN>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
+        set_b<NB, false>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
+        set_b<NB, false>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
       }
       col_steps(xs, s2, b4[0], b4[1], P4);
     }
