@@ -101,11 +101,16 @@ void choose_kernels(asi_plan* pl) {
     const size_t need = sm_wgrad_smem(a, R, false, pl->bf16);
     if (need > 75 * 1024 || B * cpb * HoWo > 32768) a.nt = 512;
     if (a.nt == 512 && sm_wgrad_smem(a, R, false, pl->bf16) > kSmemLimit) a.nt = 256;
-    // A CTA a channel that streams long and leaves SMs idle gives way to the launches that split the reduction (one layer's weight
-    // gradient, 128 x 28 x 28 to 96 channels 30.7 -> 24.4 us, 16 x 28 x 28 to 32 22.9 -> 19.2; short streams, 1 x 1 kernels and
-    // more channels than SMs lose: 4 x 30 x 30 to 100 41.3 against 43.4, 64 x 24 x 24 1 x 1 11.6 against 14.5)
-    const bool idle = Cout / cpb <= 148 && pl->d.kh * pl->d.kw >= 9 && B * cpb * HoWo >= 8192;
-    if (H * W <= 256 ? need <= kSmemLimit : need <= 113 * 1024 && !idle) {
+    // A CTA with much to do gives way to the launches that split the reduction where there are few of these CTAs: Cout / cpb of at most
+    // 128, and fewer where dY is below a million values, so that Z1 is a grouped product.  Much: the multiply-adds of term 4 and
+    // 0.7 for each of dY's values, which told the two apart best over 159 layers (maps to 40 x 40); half as many
+    // with ranks above four, whose loops are twice as wide.  One layer's weight gradient in us, a CTA a channel against the
+    // split launches: 32 x 28 x 28 to 55 channels 5 x 5 52.7, 24.1; 128 x 28 x 28 to 64 28.9, 20.0; 64 x 28 x 28 to 128 23.9, 22.6;
+    // 16 x 28 x 28 to 15 12.7, 15.1; 32 x 20 x 20 to 64 bf16 13.2, 19.1; 32 x 28 x 28 to 147 20.0, 23.8; 1 x 1 kernels lose (64 x 24 x 24 11.6, 14.5)
+    const int64_t ctas = Cout / cpb, dy = B * Cout * HoWo, kk = pl->d.kh * pl->d.kw;
+    const int64_t work = cpb * HoWo * (10 * kk * pl->r[0] * pl->r[1] + 7 * B) / 10000;   // thousands
+    const bool split = kk >= 9 && work >= (R == 4 ? 68 : 30) && ctas <= 128 && (dy >= (1 << 20) || ctas <= (work >= 150 ? 64 : R == 4 ? 24 : 36));
+    if (H * W <= 256 ? need <= kSmemLimit : need <= 113 * 1024 && !split) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;
       pl->wgrad_ncl = a.ncl;

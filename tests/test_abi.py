@@ -127,6 +127,24 @@ def test_core_contracts_the_batch_first_where_that_pays(asi, dims, ranks, bf16, 
     assert p.launch_count(0) == (6 if dims[1] > 512 else 4) + (2 if first else 4)
 
 
+@pytest.mark.parametrize("dims,cout,k,ranks,split", [   # dY as large as the activation's maps
+    ((32, 64, 28, 28), 55, 5, (3, 4, 4, 4), True),      # much for each of few CTAs
+    ((16, 64, 28, 28), 15, 3, (3, 2, 4, 2), False),     # little
+    ((16, 64, 28, 28), 15, 3, (3, 8, 4, 2), True),      # ranks above four
+    ((32, 64, 20, 20), 64, 3, (3, 4, 4, 4), False),
+    ((64, 64, 28, 28), 128, 3, (3, 4, 4, 4), True),
+    ((64, 64, 28, 28), 129, 3, (3, 4, 4, 4), False),    # more CTAs
+    ((16, 64, 28, 28), 30, 3, (4, 4, 4, 4), False),     # few values, so a grouped Z1: few CTAs only,
+    ((16, 64, 28, 28), 24, 3, (4, 4, 4, 4), True),
+    ((16, 64, 28, 28), 30, 3, (4, 7, 4, 4), True),      # some more with ranks above four
+    ((16, 64, 28, 28), 64, 5, (3, 4, 4, 4), True),      # or where the work is very long
+    ((16, 64, 28, 28), 65, 5, (3, 4, 4, 4), False),
+])
+def test_weight_gradient_splits_where_few_ctas_would_do_much(asi, dims, cout, k, ranks, split):
+    p = asi.Plan("conv", dims, ranks, cout=cout, k=k, stride=1, pad=k // 2)
+    assert (p.launch_count(1) > 1) == split
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(dims=(8, 32, 16, 16), ranks=(9, 8, 8, 8)), 3),            # r_1 > a_1
     (dict(dims=(8, 32, 16, 16), ranks=(0, 8, 8, 8)), 3),
