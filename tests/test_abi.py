@@ -115,6 +115,9 @@ def test_layers_that_fit_the_built_in_workspace(asi, dims, ranks, bf16, flags):
     ((32, 128, 56, 56), (8, 4, 4, 4), False, False),    # three million values left
     ((128, 128, 28, 28), (5, 4, 4, 4), False, False),   # a long batch of rank above four
     ((128, 128, 28, 28), (5, 4, 4, 4), True, True),
+    ((128, 128, 28, 28), (5, 5, 4, 4), False, True),
+    ((80, 128, 20, 20), (5, 4, 4, 4), False, True),     # four million values
+    ((128, 118, 27, 27), (5, 4, 4, 4), False, True),    # channel rows off 16 bytes
     ((24, 768, 28, 28), (3, 3, 3, 3), False, True),
     ((24, 768, 28, 28), (5, 3, 3, 3), False, False),    # three million values of four times that
     ((24, 768, 28, 28), (5, 3, 3, 3), True, True),
