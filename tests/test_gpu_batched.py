@@ -329,3 +329,67 @@ def test_batched_calls_from_several_host_threads():
         t.join(timeout=120)
     assert not errors, errors
     assert not any(t.is_alive() for t in threads)
+
+
+@pytest.mark.parametrize("spec,bf16", [
+    (LayerSpec("fused", "conv", (16, 24, 14, 14), 20, 3, 1, 1, 1, ranks=(4, 4, 4, 4)), False),
+    (LayerSpec("clustered", "conv", (136, 20, 7, 7), 12, 3, 1, 1, 1, ranks=(4, 4, 4, 4)), False),
+    (LayerSpec("large", "conv", (32, 64, 28, 28), 40, 3, 1, 1, 1, ranks=(4, 4, 4, 4)), False),
+    (LayerSpec("planes", "conv", (16, 40, 56, 56), 40, 3, 1, 1, 1, ranks=(4, 4, 4, 4)), True),
+    (LayerSpec("tokens", "linear", (16, 40, 128), 64, ranks=(8, 12, 16)), True),
+    (LayerSpec("matrix", "linear", (64, 300), 64, ranks=(12, 12)), False),
+], ids=lambda p: getattr(p, "name", str(p)))
+def test_calls_captured_behind_a_join_of_two_streams(spec, bf16):
+    """The first kernel of a call depends on two nodes of the graph, one of them on another stream; it must wait for both: the
+    activation and the gradient are written by these, anew in each replay."""
+    run = make_runner(spec, bf16=bf16)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+
+    def normal(shape):
+        return torch.randn(*shape, generator=gen, device="cuda").to(run.in_dtype)
+
+    a_src, d_src = normal(spec.dims), normal(spec.dy_shape)
+    act, dy, prev = torch.zeros_like(a_src), torch.zeros_like(d_src), torch.zeros_like(run.U[0])
+    u_src = torch.cat([torch.linalg.qr(torch.randn(d, r, generator=gen, device="cuda"))[0].reshape(-1)
+                       for d, r in zip(spec.dims, spec.ranks)])
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def enqueue():
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            torch.mul(u_src, 1.0, out=run.U[0])
+        torch.mul(a_src, 0.5, out=act)
+        main.wait_stream(side)
+        run.cur = 0
+        run.compress(act, stream=main)
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            torch.mul(d_src, 0.5, out=dy)
+        torch.mul(prev, 0.5, out=prev)
+        main.wait_stream(side)
+        run.wgrad(dy, stream=main)
+
+    with torch.cuda.stream(main):
+        enqueue()                                    # loads the kernels
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        enqueue()
+    for _ in range(3):
+        a_src.copy_(normal(spec.dims))
+        d_src.copy_(normal(spec.dy_shape))
+        out = []
+        for replay in (True, False):
+            for x in (act, dy, run.U[0], run.U[1], run.core, run.dW):
+                x.zero_()
+            torch.cuda.synchronize()
+            if replay:
+                graph.replay()
+            else:
+                with torch.cuda.stream(main):
+                    enqueue()
+            torch.cuda.synchronize()
+            assert run.ok()
+            out.append([x.clone() for x in (run.U[1], run.core, run.dW)])
+        assert all(float(x.abs().sum()) > 0 for x in out[0])
+        assert all(torch.equal(x, y) for x, y in zip(*out))

@@ -346,3 +346,40 @@ def test_cold_start_on_both_sides_of_the_passes(dims, ranks, bf16, passes):
     U = run.factors()
     assert max(O.rel_fro(O.projector(a), O.projector(b)) for a, b in zip(U, U_ref)) <= 1e-4
     assert O.rel_fro(O.sign_align(run.core_np(), U, U_ref)[0], S_ref) <= 1e-4
+
+
+@pytest.mark.parametrize("dims,ranks", [((33, 128, 20, 20), (6, 5, 7, 5)), ((40, 100, 20, 28), (5, 5, 5, 8))])
+def test_bf16_activations_off_sixteen_bytes(dims, ranks):
+    """Plans with the tensor-core passes whose activation starts at any element: other kernels on the same number of partials, warm
+    and cold, against the oracle."""
+    rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
+    L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
+    st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=True,
+                     gen_ranks=tuple(min(d, max(r + 2, 4)) for d, r in zip(dims, ranks)))
+    run = make_runner(L, bf16=True)
+    to_device = run.to_device
+    U_prev = st.u_prev0()
+    A, dY = st.next()
+    rng = np.random.default_rng(5)
+    n = int(np.prod(dims))
+    Omega = [rng.standard_normal((n // d, r)).astype(np.float32) for d, r in zip(dims, ranks)]
+    omega = torch.from_numpy(np.concatenate([o.ravel() for o in Omega])).cuda()
+    S_ref, U_ref = O.asi_cold_start(A.astype(np.float64), [o.astype(np.float64) for o in Omega])
+    for shift in (1, 4):
+        def place(x):
+            t = to_device(x)
+            if x is not A:
+                return t
+            buf = torch.full((t.numel() + 8,), float("nan"), dtype=t.dtype, device=t.device)
+            view = buf[shift:shift + t.numel()].view(t.shape)
+            view.copy_(t)
+            return view
+
+        run.to_device = place
+        err, _ = compare_step(run, L, A, dY, U_prev)
+        check(err, TOL_F32, f"{dims} shift={shift}")
+        run.init_factors(place(A), omega)
+        assert run.ok()
+        U = run.factors()
+        assert max(O.rel_fro(O.projector(a), O.projector(b)) for a, b in zip(U, U_ref)) <= 1e-4
+        assert O.rel_fro(O.sign_align(run.core_np(), U, U_ref)[0], S_ref) <= 1e-4
