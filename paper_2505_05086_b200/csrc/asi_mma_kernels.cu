@@ -16,9 +16,14 @@
 // to the nearest one, because its error is the same for every column of the activation and does not average out.  The eight
 // columns of the B operand are (hi | lo) of up to four factor columns, or with NB = 2 two operands of up to eight.  The
 // unit's own sums truncate, so it never adds more than two steps of the leading term (16 products) before the sum goes to a
-// register in round-to-nearest; the small terms go first.  bf16 values are exact in tf32.  Against 64 bits, 72 drawn and listed
-// conv layers (the fp32 pipe in parentheses): worst factor 3.76e-8 (3.78e-8), core 6.9e-8 (7.4e-8), gradient 2.38e-7 (2.38e-7); the
-// batch mode's factor alone 2.76e-8 (2.69e-8), 2.4e-8 of it the rounding of the output.
+// register in round-to-nearest; the small terms go first.  bf16 values are exact in tf32.
+// Against 64 bits, mean error of the factors of the batch, the channels, the rows and the columns in 1e-8 (the fp32 pipe in
+// parentheses): 60 conv layers of ranks above four 3.10 3.34 3.13 3.24 (2.91 4.74 3.21 3.32), 60 of ranks up to four 2.66 2.78
+// 2.70 2.77 (2.58 3.00 2.71 2.77), 60 bf16 2.94 3.77 2.89 2.98 (2.78 3.69 2.95 3.10); the batch of 60 token layers 3.14 (2.87); 40
+// cold starts 44.5 44.8 42.6 48.5 (46.7 47.4 50.8 61.1).  2.4 of each warm figure is the rounding of the output; what the short modes have more is
+// the last bit of the previous factor, which two terms of eleven bits do not hold.  (Rounding x to its nearest tf32 value takes a
+// tenth off the excess of ranks above four, but makes infinities of the largest values; the product of the two rests for ranks above
+// four takes 3.5 % of a compress of 50 x 116 x 27 x 27 for 1 to 3 % of the error.)
 //
 // The k order of an operand is free as long as both sides agree, and so is the order of rows: a lane takes four (bf16:
 // eight) neighbouring columns by one 16-byte read, as four m-tiles' rows in one product and four k-steps in the other.
@@ -583,18 +588,19 @@ cudaError_t launch_mfiber(const Fiber2Args& p0, int grid, bool bf16, cudaStream_
     return cudaErrorInvalidValue;                    // the caller takes another kernel
   }
   ProfScope prof(ASI_K_EXPAND, st, (double)p.O * p.a * p.I * eb);
-#define ASI_MF(RT_, CB_)                                                                                              \
+#define ASI_MF(RT_, CB_, NB16_)  /* NB16: of bf16 above rank four, which has at most two row tiles a warp */                \
   if (bf16) return p.r <= 4 ? launch_mfiber_t<RT_, 1, CB_, 0, __nv_bfloat16>(p, map, s, grid, st)                      \
-                            : launch_mfiber_t<RT_, 2, CB_, 0, __nv_bfloat16>(p, map, s, grid, st);                     \
+                            : launch_mfiber_t<RT_, NB16_, CB_, 0, __nv_bfloat16>(p, map, s, grid, st);                 \
   if (rows16) return p.r <= 4 ? launch_mfiber_t<RT_, 1, CB_, 0, float>(p, map, s, grid, st)                            \
                               : launch_mfiber_t<RT_, 2, CB_, 0, float>(p, map, s, grid, st);                           \
   return p.r <= 4 ? launch_mfiber_t<RT_, 1, CB_, 1, float>(p, map, s, grid, st)                                        \
                   : launch_mfiber_t<RT_, 2, CB_, 1, float>(p, map, s, grid, st)
+  if (bf16 && p.r > 4 && s.rt > 2) return cudaErrorInvalidValue;   // not built: mf_shape
   switch (s.rt) {
-    case 1: ASI_MF(1, 4);
-    case 2: ASI_MF(2, 2);
-    case 3: ASI_MF(3, 1);
-    default: ASI_MF(4, 1);
+    case 1: ASI_MF(1, 4, 2);
+    case 2: ASI_MF(2, 2, 2);
+    case 3: ASI_MF(3, 1, 1);
+    default: ASI_MF(4, 1, 1);
   }
 #undef ASI_MF
 }
@@ -888,7 +894,7 @@ MpShape mp_shape(int H, int W, int r, bool bf16) {
 }
 }  // namespace
 
-// Maps of 16 to 32 rows and columns (smaller ones leave the tiles empty, larger ones keep too few warps on an SM: 56 x 56
+// Maps of 12 to 32 rows and columns (smaller ones leave the tiles empty, larger ones keep too few warps on an SM: 56 x 56
 // takes 51 us here, 43 with k_plane2).
 // bf16 needs rows of four and planes on 16 bytes; fp32 planes of any size come by four-byte copies
 bool mplane_supported(int64_t n_planes, int64_t H, int64_t W, int r3, int r4, bool bf16) {
