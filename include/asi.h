@@ -78,10 +78,11 @@ typedef struct {
 /* Use only the shape-generic kernels even where a fused kernel covers the layer
  * (same results up to fp32 rounding; for testing and comparison). */
 #define ASI_FLAG_GENERIC_ONLY 1
-/* Test hook for the bounded device waits: on the fused small-map path, and in the mode passes (large maps, the batch of token
- * layers) that bring their tiles by bulk copies, the producer arms its barrier but issues no copy, and the wait limit drops from
- * about one second to one millisecond, so the waiting CTAs run into the limit, record ASI_ERR_TIMEOUT in the status word and
- * return.  The outputs of such a call are undefined; nothing faults and the workspace can be used again afterwards. */
+/* Test hook for the bounded device waits: in the kernels that bring their tiles by bulk or tensor copies (the fused small-map
+ * path, the mode passes of large maps and of the batch of token layers, the tensor-core products of token layers) the producer arms
+ * its barrier but issues no copy, and the wait limit drops from about one second to one millisecond, so the waiting CTAs run into
+ * the limit, record ASI_ERR_TIMEOUT in the status word and return.  The outputs of such a call are undefined; nothing faults and the
+ * workspace can be used again afterwards. */
 #define ASI_FLAG_TEST_EXPIRE_WAIT 2
 /* The layer's kernels are expected to run beside kernels of other layers (one CUDA-graph branch or one stream
  * per layer; Algorithm 1 treats every fine-tuned layer of a step independently).  The streaming kernels of

@@ -694,7 +694,7 @@ asi_status_t finish_compress(const asi_plan* pl, const void* act, float* U_new, 
     if (s == 0 && tc_core) {
       const ModeView& v = pl->mv[m];
       const TcCall t = {act, w + pl->tcu_off[m], dst, nullptr, 0, v.O, v.a, v.I, 0, v.r, 1, 0};
-      ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), st));
+      ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), stalls(pl), st));
     } else {
       ASI_CUDA(stream_modeprod(pl, a, src_bf16, false, st));
     }
@@ -931,7 +931,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
   if (sp.n) {
     sp.clear = clear ? status : nullptr;
     ASI_CUDA(launch_tc_split(sp, st));
-    ASI_CUDA(launch_tc_group(t, sp.n, status, st));
+    ASI_CUDA(launch_tc_group(t, sp.n, status, stalls(pl), st));
   }
   return ASI_OK;
 }
@@ -1213,8 +1213,8 @@ static asi_status_t compress_one(const asi_plan* pl, const void* act, const floa
     ASI_CUDA(launch_gemm_group(ge, pl->bf16, st));
   }
   if (sp.n) {
-    ASI_CUDA(launch_tc_group(proj, sp.n, status, st));
-    ASI_CUDA(launch_tc_group(expd, sp.n, status, st));
+    ASI_CUDA(launch_tc_group(proj, sp.n, status, stalls(pl), st));
+    ASI_CUDA(launch_tc_group(expd, sp.n, status, stalls(pl), st));
   }
   return finish_compress(pl, act, U_new, core, w, nullptr, sp.n > 0, beside, st);
 }
@@ -1556,7 +1556,7 @@ asi_status_t asi_linear_wgrad(const asi_plan_t* pl, const float* core, const flo
     tc_add_split(&sp, a.B, N, a.n_out, w + pl->off_wtc);
     ASI_CUDA(launch_tc_split(sp, st));
     const TcCall t = {dY, w + pl->off_wtc, Y1, nullptr, 0, B, N, Dout, 0, a.n_out, 1, 0};
-    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), st));
+    ASI_CUDA(launch_tc_group(&t, 1, reinterpret_cast<int*>(w), stalls(pl), st));
   } else {
     GemmGroup g;
     g.np = 0;

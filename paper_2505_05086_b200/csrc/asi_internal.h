@@ -241,7 +241,7 @@ struct TcCall {
   int64_t O, a, I, q_per_split;
   int n, nsplit, expand;
 };
-cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st);
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, int stall, cudaStream_t st);
 cudaError_t launch_sm_reduce(const SmReduceArgs& p, int nd, int max_chunks, cudaStream_t st);
 cudaError_t launch_sm_core(const SmCoreArgs& p, int R, bool bf16, int beside, cudaStream_t st);
 cudaError_t launch_sm_wgrad(const SmWgradArgs& p, int R, bool bf16, int beside, cudaStream_t st);

@@ -27,8 +27,8 @@
 // is long (each takes a quarter of K, the partial tiles meet in distributed shared memory in rank order) or own
 // different tiles.  Stage count and TMEM columns follow n so that two CTAs share an SM: what bounds these products
 // is latency -- few tiles, a prologue and an epilogue per tile, bytes in flight -- not the tensor pipe.
-// Every wait has a time limit; on expiry the kernel records ASI_ERR_TIMEOUT in the workspace's status word,
-// frees its TMEM and returns.
+// Every wait has a time limit; on expiry the kernel records ASI_ERR_TIMEOUT in the workspace's status word, gives the copies and
+// products in flight the limit once more, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -76,14 +76,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// waits for the phase with the given parity; gives up after 2e9 cycles (a second or so).  The limit is on the SM's own
-// clock: a read of %globaltimer costs over 600 cycles, and every chunk that was not there yet paid one
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// waits for the phase with the given parity; gives up after 2e9 cycles (a second or so; a millisecond with the test hook, whose
+// producer arms its barriers and issues no copy).  The limit is on the SM's own clock: a read of %globaltimer costs over 600
+// cycles, and every chunk that was not there yet paid one
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int stall) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   for (uint32_t it = 0; it < (1u << 28); ++it) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u && clock64() - t0 > 2000000000ll) return false;
+    if ((it & 1023u) == 1023u && clock64() - t0 > (stall ? 2000000ll : 2000000000ll)) return false;
   }
   return false;
 }
@@ -199,6 +200,7 @@ struct TcGroup {
   TcProb p[3];
   int* status;         // status word of the caller's workspace (may be null): ASI_ERR_TIMEOUT when a wait expires
   int np, tmem_cols, cs;
+  int stall;           // test hook: no copies, short waits
 };
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   const uint32_t stage = kTileA + tile_b;               // 1024-byte multiples: N is a multiple of 16
   // carve-up: stages, then barriers
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tc_smem) + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[2], acc_free[2];
+  __shared__ __align__(8) uint64_t full[kTcMaxStages], s_free[kTcMaxStages], done[2], acc_free[2], drained[1];
   __shared__ uint32_t tmem_slot[1];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -276,6 +278,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   if (tid == 0) {
     for (int i = 0; i < nst; ++i) { mbar_init(full + i, 1); mbar_init(s_free + i, 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(done + i, 1); mbar_init(acc_free + i, kTcWorkers); }
+    mbar_init(drained, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {                                      // TMEM: fp32 columns x 128 lanes (3 N are used)
@@ -293,6 +296,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   // The three bf16 terms of the factor are stacked along the operand's rows: one MMA of width 3 N per
   // k-step reads the X tile once and leaves the three partial products in three column groups of TMEM.
   bool ok = true;                                       // this thread's waits so far
+  int loads = 0;                                        // chunks that this thread has brought (the producer)
   const int PN = N + 4;                                 // pitch of the exchanged tile: rows four banks apart
   float* xch = reinterpret_cast<float*>(base);          // [128][PN], over the stages of a tile that is shared
   if (warp == kTcWorkers) {
@@ -310,14 +314,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
         for (int c0 = 0; c0 < nchunk && ok; c0 += kTcSeg, ++seg) {
           const int buf = nbuf == 2 ? seg & 1 : 0, turn = nbuf == 2 ? seg >> 1 : seg;
           if (turn > 0) {                               // the workers have read what the buffer held
-            ok = mbar_wait(acc_free + buf, (uint32_t)(turn + 1) & 1u);
+            ok = mbar_wait(acc_free + buf, (uint32_t)(turn + 1) & 1u, g.stall);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
           const int c1 = c0 + kTcSeg < nchunk ? c0 + kTcSeg : nchunk;
 #pragma unroll 1
           for (int c = c0; c < c1; ++c) {
-            ok = mbar_wait(full + st, ph);
+            ok = mbar_wait(full + st, ph, g.stall);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t da0 = smem_desc_sw128(a_base + st * stage, a_mn ? kTileA / 2 : 16);
@@ -336,17 +340,21 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   } else if (warp == kTcWorkers + 1) {
     // ---- TMA producer (one thread): keeps the stages full, across tiles
     if (lane == 0) {
-      int st = 0, n = 0;
+      int st = 0;
       uint32_t ph = 1;
 #pragma unroll 1
       for (int t = 0; t < ntile && ok; ++t) {
         const Tile x = tile_of(t);
 #pragma unroll 1
-        for (int c = 0; c < x.nchunk && ok; ++c, ++n) {
-          if (n >= nst) ok = mbar_wait(s_free + st, ph);
+        for (int c = 0; c < x.nchunk && ok; ++c, ++loads) {
+          if (loads >= nst) ok = mbar_wait(s_free + st, ph, g.stall);
           if (!ok) break;
           uint8_t* As = base + st * stage;
           mbar_expect_tx(full + st, stage);
+          if (g.stall) {
+            if (++st == nst) { st = 0; ph ^= 1u; }
+            continue;
+          }
           const int kc = x.k_begin + c * kTcKC;
           if (p.mode == kTcLastExpand) {
             tma_load_2d(As, &p.mapX, x.row0, kc, full + st);
@@ -382,7 +390,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
 #pragma unroll 1
       for (int c0 = 0; c0 < x.nchunk; c0 += kTcSeg, ++seg) {
         const int buf = nbuf == 2 ? seg & 1 : 0, turn = nbuf == 2 ? seg >> 1 : seg;
-        ok = mbar_wait(done + buf, (uint32_t)turn & 1u);   // every reader of TMEM observes the completed phase
+        ok = mbar_wait(done + buf, (uint32_t)turn & 1u, g.stall);   // every reader of TMEM observes the completed phase
         if (__any_sync(0xffffffffu, ok ? 0 : 1)) ok = false;
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -421,7 +429,17 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_group(const __grid_constan
   }
   const bool fail = __syncthreads_or(ok ? 0 : 1) != 0;
   pdl_launch_dependents();
-  if (fail && tid == 0 && g.status) atomicMax(g.status, (int)ASI_ERR_TIMEOUT);
+  if (fail) {                                           // what is in flight gets the limit once more
+    if (tid == 0 && g.status) atomicMax(g.status, (int)ASI_ERR_TIMEOUT);
+    if (warp == kTcWorkers && lane == 0) {
+      umma_commit(drained);
+      mbar_wait(drained, 0, g.stall);
+    } else if (warp == kTcWorkers + 1 && lane == 0) {
+      for (int i = 0; i < nst; ++i)
+        if (loads > i) mbar_wait(full + i, (uint32_t)((loads - 1 - i) / nst) & 1u, g.stall);   // the stage's last chunk
+    }
+    __syncwarp();
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
@@ -538,11 +556,12 @@ cudaError_t launch_tc_split(TcSplitArgs& p, cudaStream_t st) {
 
 // One launch over the products of `c` (all with operands already split).  cudaErrorNotSupported: a tensor map could
 // not be made (nothing was launched).
-cudaError_t launch_tc_group(const TcCall* c, int n, int* status, cudaStream_t st) {
+cudaError_t launch_tc_group(const TcCall* c, int n, int* status, int stall, cudaStream_t st) {
   if (n < 1 || n > 3) return cudaErrorInvalidValue;
   TcGroup g;
   g.np = n;
   g.status = status;
+  g.stall = stall;
   double bytes = 0.0;
   int64_t tiles[3];
   int chunks[3];

@@ -252,6 +252,8 @@ def test_a_factor_of_the_largest_values(dims, ranks, bf16):
     ("conv", (40, 48, 24, 24), (4, 4, 4, 4), True),
     ("conv", (16, 48, 56, 56), (4, 4, 4, 4), False),           # the planes of their own kernel
     ("linear", (33, 64, 1024), (7, 8, 12), True),
+    ("linear", (8, 64, 256), (4, 16, 16), True),               # tcgen05 products: one tile a CTA, and tiles shared by a cluster
+    ("linear", (24, 128, 1664), (4, 16, 16), True),            # several tiles a CTA
 ])
 def test_expired_waits_are_reported_and_the_workspace_recovers(kind, dims, ranks, bf16, cold):
     """The producer arms its barriers and copies nothing; every wait runs out (1 ms), and the next call on the same workspace is
