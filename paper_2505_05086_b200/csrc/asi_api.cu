@@ -222,6 +222,7 @@ void layout_compress(asi_plan* pl, Layout how) {
       if (pl->d.kind == ASI_LINEAR && (pl->nd != 3 || !pl->fiber[m] || v.a <= 8)) continue;
       if (!mfiber_supported(v.O, v.a, v.I, v.r, pl->bf16) || (pl->bf16 && !pl->wfiber[m] && !pl->fiber2[m])) continue;
       pl->cfiber[m] = v.a > 8 || pl->fiber[m];
+      pl->cgrid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
       if (v.a <= 8) continue;
       pl->mfiber[m] = pl->fiber[m] = true;
       pl->fiber_grid[m] = mfiber_grid(v.O, v.a, v.I, v.r, pl->bf16, share);
@@ -260,7 +261,8 @@ void layout_compress(asi_plan* pl, Layout how) {
     pl->qr_rows[m] = (pl->fast_compress || pl->small_rank) ? kRedRows : orth_rows(v.a, v.r, ns);
     pl->nchunk[m] = (int)((v.a + pl->qr_rows[m] - 1) / pl->qr_rows[m]);
     pl->off_Pp[m] = off;
-    size_t pp_elems = (size_t)ns * v.a * v.r;
+    if (pl->mfiber[m]) pl->cgrid[m] = (int)ns;
+    size_t pp_elems = (size_t)(pl->cfiber[m] ? std::max<int64_t>(ns, pl->cgrid[m]) : ns) * v.a * v.r;
     if (pl->fast_compress && pl->fast_kind && m >= 2) pp_elems = std::max(pp_elems, (size_t)ns * v.a * v.a);
     off = align_up(off + pp_elems * 4, 256);
     pl->off_Pred[m] = off;
@@ -852,23 +854,39 @@ GemmProb simt_expand(const asi_plan* pl, int m, const void* act, const float* V,
                      pl->q_per_split[m], pl->bf16);
 }
 
-// cold start: P_m = A_m Omega_m of all modes: one launch of SIMT products, one of tensor-core products, and the passes of the
+// The plan of a cold start: P_m = A_m Omega_m by one launch of SIMT products, one of tensor-core products, and the passes of the
 // modes that a warm step has on k_mfiber and k_mplane, which take Omega as their V (64 x 128 x 28 x 28 fp32, ranks 4: 72.1 -> 55.7 us).
 // These passes are launches of their own, so small tensors stay with the SIMT products (8 x 32 x 24 x 24 ranks 6 33 us with the passes,
 // 26 without; 16 x 115 x 24 x 24, a million values, 31 and 35).  Where SIMT products remain for another mode all the same, the line
 // lies at two million (15 x 70 x 32 x 33 51 and 46, 24 x 98 x 512 tokens 50 and 44; 49 x 40 x 40 x 40 52 and 56), but for batches of up
-// to eight, which these products take badly (3 x 163 x 56 x 56 57 and 66)
-// first: nothing of this call is enqueued yet; the first launch here zeroes the status block
+// to eight, which these products take badly (3 x 163 x 56 x 56 57 and 66).  The partials of P follow the kernel
+asi_plan cold_plan(const asi_plan* pl, const void* act) {
+  asi_plan c = *pl;
+  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
+  bool all = true;
+  for (int m = 0; m < c.nd; ++m) all = all && (c.cfiber[m] || (c.mplane && m >= 2));
+  const bool early = all || (c.d.kind == ASI_CONV2D && c.dims[0] <= 8);
+  const bool passes = (!c.bf16 || on16) && c.N >= (early ? 1 << 20 : 1 << 21);
+  c.mplane = c.mplane && passes;
+  for (int m = 0; m < c.nd; ++m) {
+    c.cfiber[m] = c.cfiber[m] && passes;
+    if (c.cfiber[m]) {
+      c.nsplit[m] = c.cgrid[m];
+    } else if (c.mfiber[m] && c.dims[m] > 128) {     // the grouped product of a long mode is not cut as small
+      const int64_t Q = c.mv[m].Q, ns = std::min(gemm_expand_splits(c.dims[m], Q), c.nsplit[m]);
+      c.q_per_split[m] = ((Q + ns - 1) / ns + 127) / 128 * 128;
+      c.nsplit[m] = (int)((Q + c.q_per_split[m] - 1) / c.q_per_split[m]);
+    }
+  }
+  return c;
+}
+
+// pl: of cold_plan.  first: nothing of this call is enqueued yet; the first launch here zeroes the status block
 asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* const* omega, char* w, bool first,
                           cudaStream_t st) {
   int* const status = reinterpret_cast<int*>(w);
   bool clear = first;
-  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0;
-  bool all = true;
-  for (int m = 0; m < pl->nd; ++m) all = all && (pl->cfiber[m] || (pl->mplane && m >= 2));
-  const bool early = all || (pl->d.kind == ASI_CONV2D && pl->dims[0] <= 8);
-  const bool mma = (!pl->bf16 || on16) && pl->N >= (early ? 1 << 20 : 1 << 21);
-  const bool planes = pl->mplane && mma;
+  const bool on16 = (reinterpret_cast<uintptr_t>(act) & 15u) == 0, planes = pl->mplane;
   GemmGroup g;
   g.np = 0;
   TcSplitArgs sp;
@@ -876,7 +894,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
   TcCall t[3];
   for (int m = 0; m < pl->nd; ++m) {
     const ModeView& v = pl->mv[m];
-    if ((pl->cfiber[m] && mma) || (planes && m >= 2)) continue;
+    if (pl->cfiber[m] || (planes && m >= 2)) continue;
     if (pl->tc_mode[m] && on16) {
       t[sp.n] = {act, w + pl->tcv_off[m], reinterpret_cast<float*>(w + pl->off_Pp[m]), nullptr, 0, v.O, v.a, v.I,
                  pl->q_per_split[m], v.r, pl->nsplit[m], 1};
@@ -912,7 +930,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     clear = head = false;
   }
   for (int m = 0; m < pl->nd; ++m) {
-    if (!pl->cfiber[m] || !mma) continue;
+    if (!pl->cfiber[m]) continue;
     const ModeView& v = pl->mv[m];
     Fiber2Args f;
     std::memset(&f, 0, sizeof(f));
@@ -925,7 +943,7 @@ asi_status_t expand_modes(const asi_plan* pl, const void* act, const float* cons
     f.given = 1;
     f.first = head;
     f.clear = clear ? status : nullptr;
-    ASI_CUDA(launch_mfiber(f, pl->fiber_grid[m], pl->bf16, st));
+    ASI_CUDA(launch_mfiber(f, pl->nsplit[m], pl->bf16, st));
     clear = head = false;
   }
   if (sp.n) {
@@ -1424,9 +1442,10 @@ asi_status_t asi_init_factors(const asi_plan_t* pl, const void* act, const float
     om[m] = omega;
     omega += pl->mv[m].Q * pl->r[m];
   }
-  s = expand_modes(pl, act, om, w, true, st);
+  const asi_plan cold = cold_plan(pl, act);
+  s = expand_modes(&cold, act, om, w, true, st);
   if (s != ASI_OK) return s;
-  return finish_compress(pl, act, U_new, core, w, nullptr, false, 0, st);
+  return finish_compress(&cold, act, U_new, core, w, nullptr, false, 0, st);
 }
 
 static size_t omega_scratch_bytes(const asi_plan* pl) {
@@ -1458,9 +1477,10 @@ asi_status_t asi_init_factors_seeded(const asi_plan_t* pl, const void* act, uint
   }
   f.clear = reinterpret_cast<int*>(w);
   ASI_CUDA(launch_fill_gaussian(seed, f, pl->nd, st));
-  s = expand_modes(pl, act, f.out, w, false, st);
+  const asi_plan cold = cold_plan(pl, act);
+  s = expand_modes(&cold, act, f.out, w, false, st);
   if (s != ASI_OK) return s;
-  return finish_compress(pl, act, U_new, core, w, nullptr, false, 0, st);
+  return finish_compress(&cold, act, U_new, core, w, nullptr, false, 0, st);
 }
 
 asi_status_t asi_gaussian_stream(uint64_t seed, uint32_t stream_id, int64_t n, float* out, void* stream) {

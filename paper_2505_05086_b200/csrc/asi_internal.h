@@ -522,6 +522,7 @@ struct asi_plan {
   bool fiber2[ASI_MAX_MODES];      // ... by its register-tiled successor (ranks <= 4, 16-byte aligned rows)
   bool mfiber[ASI_MAX_MODES], mplane;   // ... with the factor on the tensor cores
   bool cfiber[ASI_MAX_MODES];      // ... in a cold start, where one product is all there is: modes of up to eight entries too
+  int cgrid[ASI_MAX_MODES];        // ... and its CTAs there
   int long_cut;                    // sixteenths of its CTAs that k_mfiber goes without on modes of more than 128 entries
   bool plane2;                     // 56 x 56 planes, ranks <= 4
   bool rows16;                     // act has to start on 16 bytes
