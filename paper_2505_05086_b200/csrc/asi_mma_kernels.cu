@@ -12,15 +12,15 @@
 // 25.7 M values, where the register form needs 5.5).
 //
 // fp32 on tf32: x = hi + lo, hi the upper 19 bits of x -- which is all the unit reads, so x itself is the operand -- and lo the
-// exact rest, of which the unit reads eleven bits.  A factor is split at its nearest tf32 value instead and its rest rounded
-// to the nearest one, because its error is the same for every column of the activation and does not average out.  The eight
+// exact rest, of which the unit reads eleven bits.  V is split at its nearest tf32 value instead, and a factor's rest is rounded to
+// the nearest one as well, because its error is the same for every column of the activation and does not average out.  The eight
 // columns of the B operand are (hi | lo) of up to four factor columns, or with NB = 2 two operands of up to eight.  The
 // unit's own sums truncate, so it never adds more than two steps of the leading term (16 products) before the sum goes to a
 // register in round-to-nearest; the small terms go first.  bf16 values are exact in tf32.
 // Against 64 bits, mean error of the factors of the batch, the channels, the rows and the columns in 1e-8 (the fp32 pipe in
-// parentheses): 60 conv layers of ranks above four 3.10 3.34 3.13 3.24 (2.91 4.74 3.21 3.32), 60 of ranks up to four 2.66 2.78
-// 2.70 2.77 (2.58 3.00 2.71 2.77), 60 bf16 2.94 3.77 2.89 2.98 (2.78 3.69 2.95 3.10); the batch of 60 token layers 3.14 (2.87); 40
-// cold starts 44.5 44.8 42.6 48.5 (46.7 47.4 50.8 61.1).  2.4 of each warm figure is the rounding of the output; what the short modes have more is
+// parentheses): 60 conv layers of ranks above four 3.10 3.34 3.14 3.23 (2.91 4.74 3.21 3.32), 60 of ranks up to four 2.66 2.78
+// 2.72 2.76 (2.58 3.00 2.71 2.77), 60 bf16 2.90 3.79 2.89 2.96 (2.78 3.69 2.95 3.10); the batch of 60 token layers 3.08 (2.87); 40
+// cold starts 44.1 45.5 42.6 48.5 (46.7 47.4 50.8 61.1).  2.4 of each warm figure is the rounding of the output; what the short modes have more is
 // the last bit of the previous factor, which two terms of eleven bits do not hold.  (Rounding x to its nearest tf32 value takes a
 // tenth off the excess of ranks above four, but makes infinities of the largest values; the product of the two rests for ranks above
 // four takes 3.5 % of a compress of 50 x 116 x 27 x 27 for 1 to 3 % of the error.)
@@ -152,18 +152,23 @@ struct Acc {
   }
 };
 
-// One entry of the B operand of the columns: lane group g is the column.  A NaN is lost in both roundings, but not in the difference:
-// x - (x - hi) is hi again, or NaN where x is NaN or infinite.  TOP (the previous factors): what would round to infinity
-// leaves more to the rest instead
-template <int NB, bool TOP>
+// One entry of the B operand of the columns: lane group g is the column.  The rounding of a leading term carries a NaN over into a
+// zero.  V keeps its rest as it is, a NaN with it: what the unit cuts off averages out over the columns.  Omega (few steps are as
+// ill-conditioned as the first) and U_prev have theirs rounded too, which loses a NaN as well, but not in the difference: x - (x - hi) is
+// hi again, or NaN where x is NaN or infinite.  What of U_prev would round to infinity leaves more to the rest instead
+enum Operand { kV, kOmega, kFactor };
+template <int NB, Operand WHAT>
 __device__ __forceinline__ void set_b(float* b, int half, int g, float x) {
   float hi = nearest(x);
-  if constexpr (TOP) {
+  if constexpr (WHAT == kFactor) {
     const float top = __uint_as_float(0x7f7fe000u);
     hi = fmaxf(fminf(hi, top), -top);
   }
-  const float rest = x - hi, lo = nearest(rest);
-  hi = x - rest;
+  float lo = x - hi;
+  if constexpr (WHAT != kV) {
+    hi = x - lo;
+    lo = nearest(lo);
+  }
   if constexpr (NB == 1) b[half] = g < 4 ? hi : lo;
   else {
     b[half] = hi;
@@ -333,7 +338,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = row0 + 8 * s + 2 * c4 + h, j = NB == 1 ? (g & 3) : g;
-      set_b<NB, true>(ub[s], h, g, (k < a && j < r) ? __ldg(p.U + (int64_t)k * p.ldu + j) : 0.f);
+      set_b<NB, kFactor>(ub[s], h, g, (k < a && j < r) ? __ldg(p.U + (int64_t)k * p.ldu + j) : 0.f);
     }
   Acc<NB, EX> P[RT];
 #pragma unroll
@@ -438,7 +443,7 @@ __global__ void __launch_bounds__(kMfThreads, 2)
               for (int i = 0; i < 4; ++i) x[i] += y[i];
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i) set_b<NB, false>(b[u + i], h, g, x[i]);
+            for (int i = 0; i < 4; ++i) set_b<NB, GIVEN ? kOmega : kV>(b[u + i], h, g, x[i]);
           }
 #pragma unroll
         for (int m = 0; m < RT; ++m) {
@@ -681,8 +686,8 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = 8 * s + (h ? kr1 : kr0), w = wrow(h, s);
-      set_b<NB, true>(u3[s], h, g, (k < H && jb < p.r3) ? __ldg(p.U3 + k * p.r3 + jb) : 0.f);
-      set_b<NB, true>(u4[s], h, g, (w < W && jb < p.r4) ? __ldg(p.U4 + w * p.r4 + jb) : 0.f);
+      set_b<NB, kFactor>(u3[s], h, g, (k < H && jb < p.r3) ? __ldg(p.U3 + k * p.r3 + jb) : 0.f);
+      set_b<NB, kFactor>(u4[s], h, g, (w < W && jb < p.r4) ? __ldg(p.U4 + w * p.r4 + jb) : 0.f);
     }
   Acc<NB, EX> P3[2], P4[2];
 #pragma unroll
@@ -779,7 +784,7 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) set_b<NB, false>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
+        for (int e = 0; e < 4; ++e) set_b<NB, GIVEN ? kOmega : kV>(b3[e], h, g, wrow(h, e) < W ? W3[jb * VP + wrow(h, e)] : 0.f);
 #pragma unroll
       for (int m = 0; m < 2; ++m) {
         if (m >= nkh) break;
@@ -829,8 +834,8 @@ __global__ void __launch_bounds__(kMpThreads, 2) k_mplane(const __grid_constant_
       float b4[2][2 * NB];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        set_b<NB, false>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
-        set_b<NB, false>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
+        set_b<NB, GIVEN ? kOmega : kV>(b4[h], 0, g, W4[jb * VP + 8 * (2 * s2 + h) + kr0]);
+        set_b<NB, GIVEN ? kOmega : kV>(b4[h], 1, g, W4[jb * VP + 8 * (2 * s2 + h) + kr1]);
       }
       col_steps(xs, s2, b4[0], b4[1], P4);
     }
