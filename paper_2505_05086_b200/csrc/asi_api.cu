@@ -122,7 +122,8 @@ void choose_kernels(asi_plan* pl) {
 
 // The core of a conv layer, batch first: one streamed product that leaves t1 values, then k_core_tail, where the mode with the largest
 // a_m / r_m first leaves fewer and takes two grouped products more.  The other side of each line, one layer's compress in us:
-//   the batch product is streamed: 16 x 64 x 28 x 28 ranks 3 41.3 against 34.5, where it would be a grouped one
+//   below a million values the batch product is a grouped one, good where it is short against the batch: ranks 3 or 4 16 x 64 x 28 x 28 41
+//   against 33, 16 x 40 x 28 x 28 33 against 29; 33 x 19 x 18 x 18 27 against 32, 36 x 30 x 27 x 27 36 against 39
 //   up to 128 channels their product is streamed too, so t1 must be small (ranks 8 4: 32 x 128 x 56 x 56 95 against 89; 32 x 128 x 28 x 28
 //   51 against 54), and a large fp32 tensor with a long batch whose rank is above four has the channels first where these suit the
 //   faster kernel (ranks 8 4: 128 x 128 x 28 x 28 88.6 against 83.2, 96 x 128 x 28 x 28 72.7 against 69.1; 96 x 64 x 28 x 28 52 and 52; 64 x 128 x 28 x 28 65
@@ -131,7 +132,9 @@ void choose_kernels(asi_plan* pl) {
 //   ranks 6 6: 151 against 136; 64 x 512 x 28 x 28 ranks 8 4 200 against 204; 32 x 512 x 28 x 28 bf16 118 against 122)
 bool batch_first(const asi_plan* pl) {
   const int64_t B = pl->dims[0], C = pl->dims[1], chw = C * pl->dims[2] * pl->dims[3], r1 = pl->r[0], t1 = r1 * chw;
-  if (B < 4 * r1 || pl->N < (1 << 20) || !wfiber_supported(1, B, chw, pl->r[0])) return false;
+  if (B < 4 * r1) return false;
+  if (pl->N < (1 << 20)) return chw <= 800 * B;
+  if (!wfiber_supported(1, B, chw, pl->r[0])) return false;
   const bool channels = !pl->bf16 && B > 64 && r1 > 4 && pl->r[1] <= 4 && pl->N >= (6 << 20) &&
                         fiber2_supported(B, C, chw / C, pl->r[1], pl->bf16);
   if (C <= 128) return t1 <= (2 << 20) && !channels;

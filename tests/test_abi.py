@@ -108,7 +108,9 @@ def test_layers_that_fit_the_built_in_workspace(asi, dims, ranks, bf16, flags):
 
 
 @pytest.mark.parametrize("dims,ranks,bf16,first", [
-    ((16, 64, 28, 28), (3, 3, 3, 3), False, False),     # below a million values the batch product is a grouped one
+    ((16, 64, 28, 28), (3, 3, 3, 3), False, False),     # below a million values the batch product is a grouped one,
+    ((36, 36, 28, 28), (3, 3, 3, 3), False, True),      # short against the batch
+    ((36, 37, 28, 28), (3, 3, 3, 3), False, False),
     ((24, 64, 28, 28), (3, 3, 3, 3), False, True),
     ((24, 64, 28, 28), (7, 3, 3, 3), False, False),     # shrinks by less than four
     ((32, 128, 56, 56), (4, 8, 4, 4), False, True),
