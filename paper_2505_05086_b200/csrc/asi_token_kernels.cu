@@ -298,7 +298,11 @@ cudaError_t launch_lin_mid(const LinMidArgs& p, cudaStream_t st) {
 // rows fall in distinct banks): 12 loads per 64 packed multiply-adds (fma.rn.f32x2: the even and the odd k of a sum).  Both
 // tiles travel by asynchronous copies, all at once (through registers they were six round trips):
 // 197 x 32 tokens, 3072 x 768 weights, rank 64 29 -> 20 us beside another layer, 768 x 768 rank 32 7.9 -> 5.9.
-__global__ void __launch_bounds__(256, 2) k_lin_tail(const __grid_constant__ LinTailArgs p, int PR) {
+// A short sum leaves little but the stores and wants CTAs: up to rank 12 plain multiply-adds, whose sums take half the
+// registers, three CTAs an SM (whole weight gradient of 128 tokens, 4096 x 4096 weights: rank 3 30.8 -> 25.9 us, rank 8 34.3 -> 28.8, rank 12
+// 37.4 -> 32.6; 67 MB of it take 10).
+template <bool PACKED>
+__global__ void __launch_bounds__(256, PACKED ? 2 : 3) k_lin_tail(const __grid_constant__ LinTailArgs p, int PR) {
   extern __shared__ __align__(16) float lt_smem[];
   const int r = p.r;
   float* Z4s = lt_smem;                              // [64][PR]
@@ -309,7 +313,7 @@ __global__ void __launch_bounds__(256, 2) k_lin_tail(const __grid_constant__ Lin
   const int nd = (p.Din - d0 < kLtD) ? p.Din - d0 : kLtD;
   pdl_wait();
   // entries of a row in turn: [rows][per] with per = r / 4 units or r values, zeros behind them
-  auto stage = [&](float* dst, const float* src, int rows, int valid) {
+  auto stage = [&](float* dst, const float* src, int valid) {
     if (r % 4 == 0 && p.vec) {
       const int per = r / 4;
       for (int e = tid; e < valid * per; e += 256) {
@@ -322,51 +326,67 @@ __global__ void __launch_bounds__(256, 2) k_lin_tail(const __grid_constant__ Lin
         cp_async4(dst + row * PR + v, src + (int64_t)row * r + v);
       }
     }
-    for (int e = tid; e < rows * (PR - r); e += 256) {
-      const int row = e / (PR - r);
-      dst[row * PR + r + e - row * (PR - r)] = 0.f;
-    }
-    for (int e = tid; e < (rows - valid) * r; e += 256) {
-      const int row = valid + e / r;
-      dst[row * PR + e % r] = 0.f;
+    const int pad = (r + 3) / 4 * 4 - r;             // what the loop reads beyond the row; sums of rows >= valid are not stored
+    for (int e = tid; e < valid * pad; e += 256) {
+      const int row = e / pad;
+      dst[row * PR + r + e - row * pad] = 0.f;
     }
   };
-  stage(Us, p.U + (int64_t)d0 * r, kLtD, nd);
-  stage(Z4s, p.Z4 + (int64_t)o0 * r, kLtO, no);
+  stage(Us, p.U + (int64_t)d0 * r, nd);
+  stage(Z4s, p.Z4 + (int64_t)o0 * r, no);
   cp_async_all();
   __syncthreads();
   // dW[o0 + o][d0 + d] for o = 8 to .. 8 to + 7, d = lane + 32 i
   const int to = tid >> 5;
-  unsigned long long acc[8][4];
-#pragma unroll
-  for (int x = 0; x < 8; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0ull;
+  float out[8][4];
   const float* zrow = Z4s + 8 * to * PR;
   const float* urow = Us + lane * PR;
-  for (int k = 0; k < r; k += 4) {
-    ulonglong2 uu[4];
+  if constexpr (PACKED) {
+    unsigned long long acc[8][4];
 #pragma unroll
-    for (int y = 0; y < 4; ++y) uu[y] = *reinterpret_cast<const ulonglong2*>(urow + 32 * y * PR + k);
+    for (int x = 0; x < 8; ++x)
 #pragma unroll
-    for (int x = 0; x < 8; ++x) {
-      const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(zrow + x * PR + k);
+      for (int y = 0; y < 4; ++y) acc[x][y] = 0ull;
+    for (int k = 0; k < r; k += 4) {
+      ulonglong2 uu[4];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) uu[y] = *reinterpret_cast<const ulonglong2*>(urow + 32 * y * PR + k);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const ulonglong2 zz = *reinterpret_cast<const ulonglong2*>(zrow + x * PR + k);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[x][y]) : "l"(zz.x), "l"(uu[y].x));
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[x][y]) : "l"(zz.y), "l"(uu[y].y));
+        }
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
 #pragma unroll
       for (int y = 0; y < 4; ++y) {
-        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[x][y]) : "l"(zz.x), "l"(uu[y].x));
-        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[x][y]) : "l"(zz.y), "l"(uu[y].y));
+        float lo, hi;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[x][y]));
+        out[x][y] = lo + hi;
+      }
+  } else {
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 4; ++y) out[x][y] = 0.f;
+    for (int k = 0; k < r; k += 4) {
+      float4 uu[4];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) uu[y] = *reinterpret_cast<const float4*>(urow + 32 * y * PR + k);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const float4 zz = *reinterpret_cast<const float4*>(zrow + x * PR + k);
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          out[x][y] = fmaf(zz.w, uu[y].w, fmaf(zz.z, uu[y].z, fmaf(zz.y, uu[y].y, fmaf(zz.x, uu[y].x, out[x][y]))));
       }
     }
   }
-  float out[8][4];
-#pragma unroll
-  for (int x = 0; x < 8; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      float lo, hi;
-      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[x][y]));
-      out[x][y] = lo + hi;
-    }
 #pragma unroll
   for (int x = 0; x < 8; ++x) {
     const int o = o0 + 8 * to + x;
@@ -387,9 +407,10 @@ cudaError_t launch_lin_tail(const LinTailArgs& p0, cudaStream_t st) {
   ProfScope prof(ASI_K_MODEPROD, st, 4.0 * ((double)p.Dout * p.Din + (double)p.Dout * p.r));
   const size_t smem = 4 * (size_t)(kLtO + kLtD) * PR;
   dim3 grid((unsigned)((p.Dout + kLtO - 1) / kLtO), (unsigned)((p.Din + kLtD - 1) / kLtD));
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(k_lin_tail), smem);
+  const auto kernel = p.r > 12 ? k_lin_tail<true> : k_lin_tail<false>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void*>(kernel), smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_lin_tail, grid, dim3(256), smem, st, p, PR);
+  return launch_pdl(kernel, grid, dim3(256), smem, st, p, PR);
 }
 
 }  // namespace asi

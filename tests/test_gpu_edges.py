@@ -166,3 +166,10 @@ def test_rows_of_the_factors_on_both_sides_of_the_factoring_cta(dims, ranks, spl
     run, short = make_runner(layer(dims)), make_runner(layer(tuple(min(d, 512 if len(dims) == 4 else 384) for d in dims)))
     assert run.plan.launch_count(0) == short.plan.launch_count(0) + split
     _two_steps(layer(dims), False)
+
+
+@pytest.mark.parametrize("rank", [1, 4, 11, 12, 13])
+@pytest.mark.parametrize("cout", [64, 67])
+def test_weight_gradients_of_short_sums(rank, cout):
+    """Both forms of the last product of a linear layer, whole tiles and ragged ones, ranks that are whole groups of four and not."""
+    _two_steps(LayerSpec("t", "linear", (48, 131), cout, ranks=(rank, rank)), False, rho=(0.9, 0.9), tol=dict(TOL_F32, proj=1e-3))
