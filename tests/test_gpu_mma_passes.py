@@ -92,8 +92,8 @@ def test_batch_mode_of_token_layers(dims, ranks, cout, bf16):
 
 @pytest.mark.parametrize("dims,ranks,bf16", [c for c in CASES if c[0][0] >= 6])
 def test_cold_start_passes(dims, ranks, bf16):
-    """P_m = A_m Omega_m by the same passes, Omega in place of V (1e-4 as everywhere; the spectra keep the iterate's condition
-    number below a hundred)."""
+    """P_m = A_m Omega_m of the same layers (1e-4 as everywhere; the spectra keep the iterate's condition number below a hundred).
+    They are below a million values, so SIMT products do it; the passes with Omega in place of V are tested on larger ones."""
     rho = tuple(min(0.7, 0.25 ** (1.0 / max(r - 1, 1))) for r in ranks)
     L = LayerSpec("t", "conv", dims, 6, 3, 1, 1, 1, ranks=ranks)
     st = LayerStream(dims=dims, ranks=ranks, dy_shape=L.dy_shape, seed=sum(dims), rho=rho, bf16=bf16,
