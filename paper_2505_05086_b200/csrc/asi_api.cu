@@ -107,9 +107,11 @@ void choose_kernels(asi_plan* pl) {
     // with ranks above four, whose loops are twice as wide.  One layer's weight gradient in us, a CTA a channel against the
     // split launches: 32 x 28 x 28 to 55 channels 5 x 5 52.7, 24.1; 128 x 28 x 28 to 64 28.9, 20.0; 64 x 28 x 28 to 128 23.9, 22.6;
     // 16 x 28 x 28 to 15 12.7, 15.1; 32 x 20 x 20 to 64 bf16 13.2, 19.1; 32 x 28 x 28 to 147 20.0, 23.8; 1 x 1 kernels lose (64 x 24 x 24 11.6, 14.5)
+    // Long rows of dW, which the last of these launches writes with one CTA each, stay with the CTAs too (681 channels, 31 x 20 x 20 to 8,
+    // 5 x 5 20.5, 32.8; 192 channels, 40 x 27 x 27 to 34, 5 x 5 48.5, 31.3)
     const int64_t ctas = Cout / cpb, dy = B * Cout * HoWo, kk = pl->d.kh * pl->d.kw;
     const int64_t work = cpb * HoWo * (10 * kk * pl->r[0] * pl->r[1] + 7 * B) / 10000;   // thousands
-    const bool split = kk >= 9 && work >= (R == 4 ? 68 : 30) && ctas <= 128 && (dy >= (1 << 20) || ctas <= (work >= 150 ? 64 : R == 4 ? 24 : 36));
+    const bool split = kk >= 9 && C / pl->d.groups * kk <= 6400 && work >= (R == 4 ? 68 : 30) && ctas <= 128 && (dy >= (1 << 20) || ctas <= (work >= 150 ? 64 : R == 4 ? 24 : 36));
     if (H * W <= 256 ? need <= kSmemLimit : need <= 113 * 1024 && !split) {
       pl->fast_wgrad = true;
       pl->cpb = cpb;

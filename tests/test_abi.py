@@ -144,6 +144,8 @@ def test_core_contracts_the_batch_first_where_that_pays(asi, dims, ranks, bf16, 
     ((16, 64, 28, 28), 30, 3, (4, 7, 4, 4), True),      # some more with ranks above four
     ((16, 64, 28, 28), 64, 5, (3, 4, 4, 4), True),      # or where the work is very long
     ((16, 64, 28, 28), 65, 5, (3, 4, 4, 4), False),
+    ((32, 256, 28, 28), 55, 5, (3, 4, 4, 4), True),     # 6400 values a row of dW
+    ((32, 257, 28, 28), 55, 5, (3, 4, 4, 4), False),
 ])
 def test_weight_gradient_splits_where_few_ctas_would_do_much(asi, dims, cout, k, ranks, split):
     p = asi.Plan("conv", dims, ranks, cout=cout, k=k, stride=1, pad=k // 2)
